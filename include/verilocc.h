@@ -114,9 +114,10 @@ int vl_program_set_option(vl_program *prog, int option, uint32_t value);
  * Liveness (what "overlapping life cycles" in Section 2 and "Safety" in Section 3.4
  * rest on): per-block read/write bitsets, backward dataflow to the least fixed point,
  * then the set of vregs live after every instruction as CSR lists (ascending ids),
- * plus the tables vl_verify consumes.  Stream order: the run is enqueued on an internal stream
- * of the device, behind everything `cuda_stream` (a cudaStream_t, may be NULL) holds at the call;
- * `cuda_stream` itself is NOT made to wait for it.  Every call of this library that reads the
+ * plus the tables vl_verify consumes.  Stream order: the run of a program of more than 4,096 instructions
+ * is enqueued on an internal stream of the device, behind everything `cuda_stream` (a cudaStream_t, may be
+ * NULL) holds at the call; `cuda_stream` itself is NOT made to wait for it.  A shorter program's run is
+ * enqueued on `cuda_stream`.  Every call of this library that reads the
  * results waits for the run where it needs them: vl_verify* on the device (its table kernel, which
  * reads the candidates and the program's operand tables only, runs beside the liveness kernels;
  * the kernels after it wait), vl_liveness_result, vl_verify_host, vl_diagnose and
@@ -127,9 +128,7 @@ int vl_program_set_option(vl_program *prog, int option, uint32_t value);
  * reports NOT_STRICT or NO_CONVERGE, and the one that makes the operand tables (they depend on
  * the program alone and are kept).  Later runs recompute the liveness results on the device but
  * allocate from the remembered lengths and return without waiting: their outcome is checked by
- * the next call that uses the results, which may then return the error.  From the third such run
- * on the sequence of kernels is replayed as a CUDA graph (a recording of the library's own: do not
- * call vl_liveness while `cuda_stream` is itself being captured).
+ * the next call that uses the results, which may then return the error.
  * Errors: NOT_STRICT, NO_CONVERGE, UNSUPPORTED, CUDA.
  */
 int vl_liveness(vl_program *prog, void *cuda_stream);

@@ -11,7 +11,7 @@ std::atomic<uint64_t> g_vl_launches{0};
 // Lane streams are per device and shared by every handle on it; they live until the process exits.
 #define VL_MAX_DEVICES 64
 static std::mutex g_lane_mutex;
-static cudaStream_t g_lanes[VL_MAX_DEVICES][VL_STREAMS];  // the lanes, two side streams of a liveness run, the liveness stream
+static cudaStream_t g_lanes[VL_MAX_DEVICES][VL_STREAMS];  // the lanes, the liveness stream
 static bool g_lanes_made[VL_MAX_DEVICES];
 
 int vl_lane_streams(vl_program *p, cudaStream_t **lanes)
@@ -20,7 +20,7 @@ int vl_lane_streams(vl_program *p, cudaStream_t **lanes)
     {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
         if (!g_lanes_made[p->device]) {
-            for (int l = 0; l < VL_LANES + 2; ++l)
+            for (int l = 0; l < VL_LANES; ++l)
                 VL_CUDA(p, cudaStreamCreateWithFlags(&g_lanes[p->device][l], cudaStreamNonBlocking));
             // the liveness stream: its small kernels go first wherever a multiprocessor has room
             int least = 0, greatest = 0;
@@ -31,13 +31,14 @@ int vl_lane_streams(vl_program *p, cudaStream_t **lanes)
     }
     if (!p->ev_fork) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     if (!p->ev_pre) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_pre, cudaEventDisableTiming));
-    for (int l = 0; l < 3; ++l)
-        if (!p->ev_side[l]) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_side[l], cudaEventDisableTiming));
     for (int l = 0; l < VL_LANES; ++l)
         if (!p->ev_join[l]) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_join[l], cudaEventDisableTiming));
     *lanes = g_lanes[p->device];
     return VL_OK;
 }
+
+// Programs of at most this many instructions run their liveness on the caller's stream (see vl_liveness).
+#define LIVE_INLINE_INSTRS 4096
 
 static int validate(const vl_program_desc *d)
 {
@@ -204,11 +205,12 @@ void vl_free_liveness(vl_program *p)
     p->live_arena.reset();
     p->tmp_arena.reset();
     p->d_blk_in = p->d_blk_out = p->d_lo_off = p->d_lo = nullptr;
-    p->d_opflags = nullptr; p->d_iflags = nullptr;  // (the operand tables live in the layout arena)
+    p->d_opflags = nullptr;  // (the operand tables live in the layout arena)
     p->d_th_off = p->d_th = p->d_cev_off = nullptr;
     p->d_ev = nullptr;
     p->d_el = nullptr; p->d_el_count = nullptr;
     p->d_ls = p->d_ls_adj = p->d_th_cnt = p->d_blk_th = nullptr;
+    p->d_sev_off = p->d_sev = nullptr;
     p->live_ok = false;
     p->lo_len = 0;
 }
@@ -218,7 +220,6 @@ extern "C" void vl_program_destroy(vl_program *p)
     if (!p) return;
     cudaSetDevice(p->device);
     vl_live_settle(p);
-    vl_drop_live_graph(p);
     vl_free_liveness(p);
     if (p->h_live) cudaFreeHost(p->h_live);
     if (p->h_out_pinned) cudaFreeHost(p->h_out_pinned);
@@ -246,8 +247,6 @@ extern "C" void vl_program_destroy(vl_program *p)
     for (cudaEvent_t ev : p->kt_ev) cudaEventDestroy(ev);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_pre) cudaEventDestroy(p->ev_pre);
-    for (cudaEvent_t ev : p->ev_side)
-        if (ev) cudaEventDestroy(ev);
     for (cudaEvent_t ev : p->ev_join)
         if (ev) cudaEventDestroy(ev);
     delete p;
@@ -371,6 +370,14 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
 {
     if (!p) return VL_ERR_INVALID_ARG;
     VL_CUDA(p, cudaSetDevice(p->device));
+    // A short program's run (tens of microseconds) goes to the caller's stream: leaving it and coming back costs
+    // about as much as the run could hide.
+    if (p->nI <= LIVE_INLINE_INSTRS) {
+        p->live_stream = (cudaStream_t)stream;
+        const int rc = vl_liveness_impl(p, (cudaStream_t)stream);
+        p->live_deferred = true;
+        return rc;
+    }
     // The run goes to an internal stream, behind everything the caller's stream holds now.  The
     // caller's stream does not wait for it: the calls that read the results do (vl_live_join), and
     // the table kernel of a following vl_verify, which needs none of them, runs beside it.
@@ -380,6 +387,7 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     cudaStream_t ls = lanes[VL_LIVE_STREAM];
     VL_CUDA(p, cudaEventRecord(p->ev_pre, (cudaStream_t)stream));
     VL_CUDA(p, cudaStreamWaitEvent(ls, p->ev_pre, 0));
+    p->live_stream = ls;
     rc = vl_liveness_impl(p, ls);
     p->live_deferred = true;
     return rc;
@@ -387,7 +395,7 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
 
 int vl_live_join(vl_program *p, cudaStream_t st)
 {
-    if (p->live_deferred && p->ev_live) VL_CUDA(p, cudaStreamWaitEvent(st, p->ev_live, 0));
+    if (p->live_deferred && p->ev_live && st != p->live_stream) VL_CUDA(p, cudaStreamWaitEvent(st, p->ev_live, 0));
     return VL_OK;
 }
 

@@ -33,8 +33,8 @@ enum : uint32_t {
 
 #define VL_MAX_GROUP 8
 #define VL_LANES 8  // internal streams that the passes of device-resident verify calls can be spread over
-#define VL_LIVE_STREAM (VL_LANES + 2)  // index of the internal stream a single vl_liveness call runs on
-#define VL_STREAMS (VL_LANES + 3)      // the lanes, two side streams of a liveness run, the liveness stream
+#define VL_LIVE_STREAM VL_LANES      // index of the internal stream a single vl_liveness call runs on
+#define VL_STREAMS (VL_LANES + 1)    // the lanes, the liveness stream
 
 // Device memory pool of a program handle: slabs are kept across calls, so that a repeated
 // vl_liveness on the same handle allocates nothing.
@@ -79,19 +79,21 @@ struct vl_program {
     uint32_t chunk_instrs = 160;
     uint32_t group_opt = 0;
 
-    // chunks: every chunk lies inside one block; pieces: every piece lies inside one chunk
-    uint32_t nC = 0, nP = 0;
+    // chunks: every chunk lies inside one block; pieces: every piece lies inside one chunk; short chunks: runs of
+    // pieces of one chunk; segments: runs of chunks of one block
+    uint32_t nC = 0, nP = 0, nS = 0, nSeg = 0;
     uint32_t layout_chunk_instrs = 0;  // chunk size the device copies of the layout were made for (0: none)
     std::vector<uint32_t> h_blk_off, h_op_off;
     // list lengths of the last liveness run with this layout: the next run allocates from them
     bool sizes_known = false;
-    uint64_t known_lo_len = 0, known_steps = 0, known_thn = 0, known_ls_len = 0;
+    unsigned long long known[5] = {0, 0, 0, 0, 0};  // list entries, walk events, through-set entries, short-list entries, short-chunk events
 
     // device copies of the program
     uint32_t *d_blk_off = nullptr, *d_succ_off = nullptr, *d_succ = nullptr, *d_op_off = nullptr, *d_op_vreg = nullptr;
     uint8_t *d_ndefs = nullptr, *d_width = nullptr;
     uint32_t *d_chunk_i0 = nullptr, *d_chunk_i1 = nullptr, *d_chunk_blk = nullptr, *d_blk_chunk_off = nullptr;
-    uint32_t *d_piece_i0 = nullptr, *d_piece_i1 = nullptr, *d_piece_chunk = nullptr, *d_chunk_piece_off = nullptr;
+    uint32_t *d_piece_i0 = nullptr, *d_piece_chunk = nullptr, *d_chunk_piece_off = nullptr;
+    uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr;
 
     // liveness results
     uint32_t *d_blk_in = nullptr, *d_blk_out = nullptr, *d_lo_off = nullptr, *d_lo = nullptr;
@@ -112,7 +114,6 @@ struct vl_program {
     uint4 *d_opoff = nullptr;               // [nOpT / 4] per 4 operands: byte offsets of their vregs' 16-byte table entries
     uint8_t *d_first4 = nullptr;            // [nOpT / 4] per 4 operands: first-occurrence bits
     uint8_t *d_opflags = nullptr;           // [nO]
-    uint8_t *d_iflags = nullptr;            // [nI] 1 if the instruction has a definition the walk skips
     uint32_t *d_first_def_instr = nullptr;  // [V] lowest instruction defining v, 0xFFFFFFFF if none
     uint32_t *d_vinfo = nullptr;            // [V] width | VINFO_OCCURS | VINFO_DEFINED
     // optional hardware rules of the Realizability check (vl_program_set_constraints)
@@ -124,13 +125,11 @@ struct vl_program {
     uint32_t *d_ls = nullptr, *d_ls_adj = nullptr, *d_th_cnt = nullptr, *d_blk_th = nullptr;
     uint4 *d_el = nullptr;          // definitions without a walk event: {instruction, chunk, vreg, block}, any order
     uint32_t *d_el_count = nullptr;
-    uint32_t th_len = 0;
     uint32_t *d_cev_off = nullptr;  // [nC+1] first walk event of each chunk (every chunk padded to 8 events)
     uint4 *d_ev = nullptr;          // walk events, 112 bytes per group of 8, chunk after chunk
-    uint32_t ev_total = 0;
-    // walk work items: a run of chunks of one block
-    uint32_t nItems = 0;
-    uint32_t *d_item_blk = nullptr, *d_item_c0 = nullptr, *d_item_c1 = nullptr;
+    // events of the short chunks, 4 bytes each, 32 short chunks side by side: steps [sev_off[g], sev_off[g + 1]) of
+    // group g, [step][32]
+    uint32_t *d_sev_off = nullptr, *d_sev = nullptr;
     int bank_fast = 0;  // B in {1,2,4} and every instruction reads <= 4 distinct vregs
     int bank_many = 0;  // some instruction reads more than 4 distinct vregs
     uint2 *d_bank_list = nullptr;   // instructions with 2, 3, 4 distinct sources: their vreg ids, 16 bits each
@@ -147,27 +146,23 @@ struct vl_program {
     uint32_t *d_status = nullptr;  // [16] device status words
     int last_cuda_error = 0;
     bool live_ok = false;
-    // A repeated liveness run (same layout, lengths remembered) does not wait for the GPU: its status
-    // word and list lengths are copied to pinned host memory behind the kernels, and the next call
-    // that needs the results on the host side (vl_live_settle) waits for the copy and checks them.
-    uint32_t *h_live = nullptr;      // pinned: [0] status, [2..9] four 64-bit totals
+    // A repeated liveness run (same layout, lengths remembered) does not wait for the GPU: its kernels write
+    // the status word and the list lengths to pinned host memory, and the next call that needs the results on
+    // the host side (vl_live_settle) waits for the run and checks them.
+    uint32_t *h_live = nullptr;      // pinned: [0] status, [2..11] five 64-bit totals, written by the run's kernels
     cudaEvent_t ev_live = nullptr;
     bool live_pending = false;
-    // vl_liveness runs on an internal stream behind what the caller's stream held when it was called;
-    // the caller's stream is not made to wait.  Calls that read the results make their stream wait
+    // vl_liveness of a long program runs on an internal stream (live_stream) behind what the caller's stream held
+    // when it was called; the caller's stream is not made to wait.  Calls that read the results make their stream wait
     // for ev_live (vl_live_join); the table kernel, which reads the program's operand tables only,
     // runs beside the liveness kernels.
     bool live_deferred = false;
+    cudaStream_t live_stream = nullptr;
     cudaEvent_t ev_pre = nullptr;
     // The operand tables of the verify kernels (vreg per operand, first-occurrence bits, table
     // offsets, vreg descriptors, first definitions) depend on the program alone: they are made by the
     // first liveness run and kept (layout arena).
     bool tables_built = false;
-    // the recorded form of a liveness run with settled layout and lengths (see vl_liveness_impl)
-    cudaGraphExec_t live_graph = nullptr;
-    uint64_t live_graph_launches = 0;
-    uint32_t settled_runs = 0;
-    int graph_opt = 1;
 
     // per-call working memory of vl_verify (one set per internal stream slot), grown on demand
     struct VScratch {
@@ -183,7 +178,6 @@ struct vl_program {
     uint32_t sub_batch = 5120;       // candidates per pass of the verify kernels
     uint32_t lanes_opt = 3;          // lanes in use (1 = everything in order on the caller's stream)
     cudaEvent_t ev_fork = nullptr, ev_join[VL_LANES] = {};
-    cudaEvent_t ev_side[3] = {};     // fork and two joins of the side streams of a liveness run
 
     // opt-in per-kernel timing of vl_verify: five events per pass (before each of the four kernels, after the last)
     int ktime = 0;
@@ -220,8 +214,8 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
                    cudaStream_t st, int slot, bool dict = false);
 int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K,
                     const uint64_t *pitch, vl_verdict *const *d_out, cudaStream_t st, bool dict = false);
-// The lane streams of the handle's device (created once per device; two side streams for liveness
-// follow the VL_LANES lanes in the array) and the handle's fork / join events.
+// The lane streams of the handle's device (created once per device; the liveness stream
+// follows the VL_LANES lanes in the array) and the handle's fork / join events.
 int vl_lane_streams(vl_program *p, cudaStream_t **lanes);
 void vl_free_liveness(vl_program *p);
 // Waits for a liveness run that is still in flight and checks its outcome; VL_OK if none is pending.
@@ -230,4 +224,3 @@ int vl_live_join(vl_program *p, cudaStream_t st);  // st waits for the liveness 
 // Multiprocessors of a device / of the handle's device (asked once).
 int vl_device_sm_count(int device);
 int vl_sm_count(vl_program *p);
-void vl_drop_live_graph(vl_program *p);

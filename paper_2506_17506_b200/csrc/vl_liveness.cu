@@ -1,52 +1,98 @@
 // Liveness on the GPU and the per-program tables the verify kernels consume.
 //
-// Pipeline (all kernels on the caller's stream).  Every block is cut into chunks (the unit of the
-// verify walk) and every chunk into pieces of at most PIECE_INSTRS instructions (the unit of the
-// backward instruction walk here, so that a few thousand warps share it):
-//   piece read/write sets -> chunk sets -> block sets -> fixed point over blocks (one thread per
-//   bitset word) -> live set at every chunk boundary -> at every piece boundary -> backward walk
-//   of every piece (count, then fill) giving the per-instruction live-after lists in CSR form and
-//   the per-operand flags -> operand metadata, walk events, through-sets.
+// Every block is cut into chunks (the unit of the verify walk), every chunk into pieces of at most
+// PIECE_INSTRS instructions (the unit of the instruction-level work here), and runs of pieces of one chunk
+// form short chunks (the unit of the one-candidate walk).  A run is five launches:
+//   k_sets     read/write bitsets of every piece, composed to its chunk's (one thread block per chunk)
+//   k_flow     per 32 words of the bitsets: block sets, fixed point over the blocks, live sets at the
+//              chunk boundaries (bitset words are independent of each other)
+//   k_count    live sets at the piece boundaries; live-after list lengths, operand flags, walk-event
+//              counts and the vregs whose occupancy changes (one thread block per chunk)
+//   k_offsets  through-sets, entry counts; the last thread block makes every offset and leaves the totals
+//              and the status word in pinned host memory
+//   k_fill     live-after lists in CSR form, walk events, through-set lists, side by side in one grid
+// What bounds a run is the chain of launches and of L2 round trips inside them, not the bytes (34 MB of
+// lists for 32,000 instructions).  The 17 launches (a recorded graph) that did the same before spent most of
+// their time on launch latency and on one-thread loops over an instruction's operands; here the lanes of a
+// warp take the operands of a piece, and a kernel's blocks start while the kernel before it drains.
+// Liveness + vl_verify of 100 rows: 98 -> 65 us for 64 instructions, 122 -> 96 us for 2,000.
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "vl_internal.cuh"
 
-#define NT 128  // threads per block in every kernel of this file
+#define NT 128  // threads per block of the operand-table kernels
 #define PIECE_INSTRS 8
-#ifndef VL_ITEM_CHUNKS
-#define VL_ITEM_CHUNKS 32  // chunks per walk work item
-#endif
+#define PC_WARPS 20            // warps per block of k_sets and k_count: the pieces of a chunk of the default size at once
+#define PC_NT (PC_WARPS * 32)
+#define LV_WARPS 8             // warps per block of k_fill
+#define LV_NT (LV_WARPS * 32)
+#define FLOW_WARPS 16          // warps per block of k_flow
+#define OFF_NT 256             // threads per block of k_offsets
+#define SEG_CHUNKS 8           // chunks that a warp of k_flow composes in one go (longer in very long programs)
+#define SHORT_CHUNKS 512       // short chunks per program aimed at: the threads of one block of the one-candidate walk
+
+// Everything the five kernels of a run read and write.
+struct LiveArgs {
+    uint32_t nB, nI, V, nE, Wv, nC, nP, nS, nSeg;
+    int use_th;
+    // program and layout
+    const uint32_t *op_off, *op_vreg, *succ_off, *succ, *blk_off;
+    const uint8_t *ndefs, *width;
+    const uint32_t *chunk_i0, *chunk_i1, *chunk_blk, *blk_chunk_off, *piece_i0, *piece_chunk, *chunk_piece_off;
+    const uint32_t *seg_c0, *blk_seg_off;         // segments of k_flow: runs of chunks of one block
+    const uint32_t *short_p0, *chunk_short_off;   // short chunks: first piece of each; short chunks of every chunk
+    // working sets
+    uint32_t *piece_use, *piece_def, *piece_end, *chunk_use, *chunk_def, *chunk_end, *chunk_entry, *blk_touch;
+    uint32_t *lo_rel, *ev_rel;                    // per instruction: list entries / events before it in its chunk
+    unsigned long long *chunk_lo;                 // per chunk: list entries of its instructions
+    uint32_t *chunk_ev, *chunk_lo0;               // events of its instructions; first list entry
+    uint32_t *centry_cnt, *short_cnt;             // entry events per chunk; events per short chunk
+    uint32_t *flow_scratch;                       // k_flow's working set when it does not fit shared memory
+    uint32_t *counters;                           // [0] blocks of k_offsets that have finished
+    // results
+    uint32_t *blk_in, *blk_out, *lo_off, *lo, *ls, *ls_adj, *blk_th, *th_cnt, *th_off, *th, *cev_off, *sev_off, *sev;
+    uint8_t *opflags;
+    uint4 *ev, *el;
+    uint32_t *el_count, *status;
+    uint32_t *host_out;                           // pinned: [0] status, [2..] totals (64 bit)
+};
+enum { LV_TOT_LO = 0, LV_TOT_EV = 1, LV_TOT_TH = 2, LV_TOT_LS = 3, LV_TOT_SEV = 4, LV_TOTALS = 5 };
 
 // ------------------------------------------------------------------ device helpers
 __device__ __forceinline__ bool bit_get(const uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; }
-__device__ __forceinline__ void bit_set(uint32_t *s, uint32_t v) { s[v >> 5] |= 1u << (v & 31); }
-__device__ __forceinline__ void bit_clr(uint32_t *s, uint32_t v) { s[v >> 5] &= ~(1u << (v & 31)); }
 
-// Exclusive scan over the NT threads of a block; *total gets the block sum.
-// s_scan needs 34 words.  Contains barriers: every thread of the block must call it.
-__device__ uint32_t block_excl_scan(uint32_t x, uint32_t *s_scan, uint32_t *total)
+// Programmatic dependent launch: a kernel's blocks may start while the kernel before it still runs; what they do
+// before pdl_wait reads the program and its layout only.  pdl_go lets the next kernel's blocks start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Exclusive scan over the threads of a block (a whole number of warps, at most 32), any integer type;
+// *total gets the block sum.  s_scan needs 34 elements.  Contains barriers.
+template <typename T>
+__device__ T block_excl_scan(T x, T *s_scan, T *total)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t inc = x;
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    T inc = x;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += y;
+        const T y = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= (uint32_t)d) inc += y;
     }
     __syncthreads();  // protects s_scan against readers of a previous call
     if (lane == 31) s_scan[w] = inc;
     __syncthreads();
     if (w == 0) {
-        uint32_t t = lane < NT / 32 ? s_scan[lane] : 0u;
-        uint32_t ti = t;
+        const T t = lane < nw ? s_scan[lane] : (T)0;
+        T ti = t;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, ti, d);
-            if (lane >= d) ti += y;
+            const T y = __shfl_up_sync(0xffffffffu, ti, d);
+            if (lane >= (uint32_t)d) ti += y;
         }
-        if (lane < NT / 32) s_scan[lane] = ti - t;
+        if (lane < nw) s_scan[lane] = ti - t;
         if (lane == 31) s_scan[33] = ti;
     }
     __syncthreads();
@@ -54,418 +100,436 @@ __device__ uint32_t block_excl_scan(uint32_t x, uint32_t *s_scan, uint32_t *tota
     return s_scan[w] + inc - x;
 }
 
-// Calls emit(rank, bit index) for every set bit of words[0..nwords), ranks ascending with
-// the bit index.  Contains barriers.
-template <class F>
-__device__ void compact_bits(const uint32_t *words, uint32_t nwords, uint32_t *s_scan, uint32_t *total, F emit)
-{
-    const uint32_t per = (nwords + NT - 1) / NT;
-    const uint32_t w0 = min(nwords, threadIdx.x * per), w1 = min(nwords, w0 + per);
-    uint32_t cnt = 0;
-    for (uint32_t w = w0; w < w1; ++w) cnt += __popc(words[w]);
-    uint32_t off = block_excl_scan(cnt, s_scan, total);
-    for (uint32_t w = w0; w < w1; ++w) {
-        uint32_t x = words[w];
-        while (x) {
-            uint32_t b = __ffs(x) - 1;
-            x &= x - 1;
-            emit(off++, w * 32 + b);
-        }
+// The operands of a piece, one per lane and round of 32: vreg (16 bits), instruction inside the piece
+// (4 bits at 16), definition (bit 20).  Lanes beyond the piece hold 0xFFFFFFFF.
+struct PieceOps {
+    uint32_t ob, n, off;  // first operand, operands; lane k <= instructions of the piece: operand offset of instruction k
+    uint32_t nd, ni;      // lane k: definitions of instruction k; instructions
+    __device__ __forceinline__ void init(const LiveArgs &q, uint32_t p, uint32_t c, uint32_t lane)
+    {
+        const uint32_t i0 = q.piece_i0[p], i1 = min(i0 + PIECE_INSTRS, q.chunk_i1[c]);
+        ni = i1 - i0;
+        off = lane <= ni ? q.op_off[i0 + lane] : 0xFFFFFFFFu;
+        nd = lane < ni ? q.ndefs[i0 + lane] : 0u;
+        ob = __shfl_sync(0xffffffffu, off, 0);
+        n = __shfl_sync(0xffffffffu, off, ni) - ob;
     }
-}
+    __device__ __forceinline__ uint32_t get(const LiveArgs &q, uint32_t j) const  // (every lane of the warp)
+    {
+        const uint32_t o = ob + j;
+        uint32_t k = 0, first = ob, nd_k = __shfl_sync(0xffffffffu, nd, 0);
+        for (uint32_t u = 1; u < ni; ++u) {
+            const uint32_t f = __shfl_sync(0xffffffffu, off, u), d = __shfl_sync(0xffffffffu, nd, u);
+            if (f <= o) { k = u; first = f; nd_k = d; }
+        }
+        return j < n ? (q.op_vreg[o] | (k << 16) | (o - first < nd_k ? 1u << 20 : 0u)) : 0xFFFFFFFFu;
+    }
+};
+__device__ __forceinline__ uint32_t po_vreg(uint32_t x) { return x & 0xFFFFu; }
+__device__ __forceinline__ uint32_t po_instr(uint32_t x) { return (x >> 16) & 15u; }
+__device__ __forceinline__ bool po_def(uint32_t x) { return (x >> 20) & 1u; }
 
-// ------------------------------------------------------------------------- kernels
-// Per span of instructions (a piece): use = vregs read before any write inside the span, def = vregs written.
-__global__ void k_chunk_sets(const uint32_t *__restrict__ chunk_i0, const uint32_t *__restrict__ chunk_i1,
-                             const uint32_t *__restrict__ op_off, const uint8_t *__restrict__ ndefs,
-                             const uint32_t *__restrict__ op_vreg, uint32_t Wv, uint32_t *chunk_use,
-                             uint32_t *chunk_def)
+// ============================================================================ k_sets
+// One thread block per chunk.  use = vregs read before any write inside the piece (the chunk), def = vregs
+// written.  A lane holds an operand and meets the piece's other operands by shuffles.
+__global__ void __launch_bounds__(PC_NT) k_sets(const LiveArgs q)
 {
     extern __shared__ uint32_t sm[];
-    uint32_t *s_use = sm, *s_def = sm + Wv;
-    const uint32_t c = blockIdx.x;
-    for (uint32_t w = threadIdx.x; w < 2 * Wv; w += NT) sm[w] = 0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (uint32_t i = chunk_i0[c]; i < chunk_i1[c]; ++i) {
-            const uint32_t o0 = op_off[i], o1 = op_off[i + 1], nd = ndefs[i];
-            for (uint32_t o = o0 + nd; o < o1; ++o) {  // reads first
-                uint32_t v = op_vreg[o];
-                if (!bit_get(s_def, v)) bit_set(s_use, v);
-            }
-            for (uint32_t o = o0; o < o0 + nd; ++o) bit_set(s_def, op_vreg[o]);
-        }
-    }
-    __syncthreads();
-    for (uint32_t w = threadIdx.x; w < Wv; w += NT) {
-        chunk_use[(size_t)c * Wv + w] = s_use[w];
-        chunk_def[(size_t)c * Wv + w] = s_def[w];
-    }
-}
-
-// Per parent (a block over its chunks, a chunk over its pieces): compose the children's sets in order.
-__global__ void k_block_sets(const uint32_t *__restrict__ blk_chunk_off, uint32_t Wv,
-                             const uint32_t *__restrict__ chunk_use, const uint32_t *__restrict__ chunk_def,
-                             uint32_t *blk_use, uint32_t *blk_def)
-{
-    const uint32_t b = blockIdx.y, w = blockIdx.x * NT + threadIdx.x;  // one bitset word per thread
-    if (w >= Wv) return;
-    const uint32_t c_lo = blk_chunk_off[b], c_hi = blk_chunk_off[b + 1];
-    uint32_t u = 0, d = 0;
+    const uint32_t c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_go();
+    // what later kernels of the run update with atomics starts at zero
+    for (size_t i = (size_t)c * blockDim.x + tid; i < (size_t)q.nB * q.Wv; i += (size_t)gridDim.x * blockDim.x) q.blk_touch[i] = 0;
+    if (c == 0 && tid == 0) { q.counters[0] = 0; *q.el_count = 0; *q.status = 0; }
+    if (c >= q.nC) return;
+    uint32_t *s_use = sm + (size_t)warp * 2 * q.Wv, *s_def = s_use + q.Wv;
+    const uint32_t p0 = q.chunk_piece_off[c], p1 = q.chunk_piece_off[c + 1];
+    for (uint32_t p = p0 + warp; p < p1; p += blockDim.x / 32) {
+        for (uint32_t w = lane; w < 2 * q.Wv; w += 32) s_use[w] = 0;
+        PieceOps po;
+        po.init(q, p, c, lane);
+        __syncwarp();
+        for (uint32_t r = 0; r < po.n; r += 32) {
+            const uint32_t x = po.get(q, r + lane);
+            bool written = false;  // an earlier instruction of the piece writes this operand's vreg
+            for (uint32_t j0 = 0; j0 <= r; j0 += 32) {
+                const uint32_t y = j0 == r ? x : po.get(q, j0 + lane);
 #pragma unroll 8
-    for (uint32_t c = c_lo; c < c_hi; ++c) {
-        u |= chunk_use[(size_t)c * Wv + w] & ~d;
-        d |= chunk_def[(size_t)c * Wv + w];
+                for (uint32_t j = 0; j < 32; ++j) {
+                    const uint32_t z = __shfl_sync(0xffffffffu, y, j);
+                    written |= po_def(z) && po_vreg(z) == po_vreg(x) && po_instr(z) < po_instr(x);
+                }
+            }
+            if (r + lane < po.n) {
+                uint32_t *s = po_def(x) ? s_def : s_use;
+                if (po_def(x) || !written) atomicOr(&s[po_vreg(x) >> 5], 1u << (x & 31));
+            }
+        }
+        __syncwarp();
+        for (uint32_t w = lane; w < q.Wv; w += 32) {
+            q.piece_use[(size_t)p * q.Wv + w] = s_use[w];
+            q.piece_def[(size_t)p * q.Wv + w] = s_def[w];
+        }
+        __syncwarp();
     }
-    blk_use[(size_t)b * Wv + w] = u;
-    blk_def[(size_t)b * Wv + w] = d;
+    __syncthreads();
+    for (uint32_t w = tid; w < q.Wv; w += blockDim.x) {
+        uint32_t u = 0, d = 0;
+#pragma unroll 4
+        for (uint32_t p = p0; p < p1; ++p) {
+            u |= q.piece_use[(size_t)p * q.Wv + w] & ~d;
+            d |= q.piece_def[(size_t)p * q.Wv + w];
+        }
+        q.chunk_use[(size_t)c * q.Wv + w] = u;
+        q.chunk_def[(size_t)c * q.Wv + w] = d;
+    }
 }
 
-// Backward dataflow to the least fixed point.  Bitset words are independent of each other,
-// so one thread iterates one word column over all blocks until nothing changes; no barrier.
-// SMEM: the four sets of this thread's word column and the successor lists sit in shared memory
-// ([4][nB][NT] words, then succ_off[nB + 1] and succ[nE]); otherwise everything stays in global memory.
-template <bool SMEM>
-__global__ void k_fixed_point(uint32_t nB, uint32_t nE, uint32_t Wv, const uint32_t *__restrict__ succ_off,
-                              const uint32_t *__restrict__ succ, const uint32_t *__restrict__ blk_use,
-                              const uint32_t *__restrict__ blk_def, uint32_t *live_in, uint32_t *live_out,
-                              uint32_t *status)
+// ============================================================================ k_flow
+// Backward dataflow to the least fixed point.  A thread block takes 32 words of every bitset (one per lane);
+// bitset words are independent of each other, so nothing is exchanged between thread blocks.  Warps compose
+// the chunk sets of segments (SEG_CHUNKS loads in flight instead of a chain over a block's chunks), one warp
+// iterates the blocks, and the warps walk the segments back to the live sets at the chunk boundaries.
+// Working set: [4][nB][32] + [2][nSeg][32] words and the successor lists, in shared memory or flow_scratch.
+__global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const LiveArgs q)
 {
-    const uint32_t w = blockIdx.x * NT + threadIdx.x;
-    if (SMEM) {
-        extern __shared__ uint32_t fsm[];
-        uint32_t *s_use = fsm, *s_def = fsm + nB * NT, *s_in = fsm + 2 * nB * NT, *s_out = fsm + 3 * nB * NT;
-        uint32_t *s_so = fsm + 4 * nB * NT, *s_su = s_so + nB + 1;
-        for (uint32_t i = threadIdx.x; i <= nB; i += NT) s_so[i] = succ_off[i];
-        for (uint32_t i = threadIdx.x; i < nE; i += NT) s_su[i] = succ[i];
-        const uint32_t t = threadIdx.x;
-        for (uint32_t b = 0; b < nB; ++b) {
-            s_use[b * NT + t] = w < Wv ? blk_use[(size_t)b * Wv + w] : 0u;
-            s_def[b * NT + t] = w < Wv ? blk_def[(size_t)b * Wv + w] : 0u;
-            s_in[b * NT + t] = 0;
-            s_out[b * NT + t] = 0;
+    extern __shared__ uint32_t sm[];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t w = blockIdx.x * 32 + lane;
+    const bool in = w < q.Wv;
+    const size_t words = ((size_t)4 * q.nB + 2 * (size_t)q.nSeg) * 32 + q.nB + 1 + q.nE;
+    uint32_t *base = q.flow_scratch ? q.flow_scratch + blockIdx.x * words : sm;
+    uint32_t *s_use = base, *s_def = s_use + (size_t)q.nB * 32, *s_in = s_def + (size_t)q.nB * 32,
+             *s_out = s_in + (size_t)q.nB * 32, *seg_u = s_out + (size_t)q.nB * 32, *seg_d = seg_u + (size_t)q.nSeg * 32,
+             *s_so = seg_d + (size_t)q.nSeg * 32, *s_su = s_so + q.nB + 1;
+    for (uint32_t i = tid; i <= q.nB; i += FLOW_WARPS * 32) s_so[i] = q.succ_off[i];
+    for (uint32_t i = tid; i < q.nE; i += FLOW_WARPS * 32) s_su[i] = q.succ[i];
+    pdl_go();
+    pdl_wait();
+    for (uint32_t s = warp; s < q.nSeg; s += FLOW_WARPS) {
+        const uint32_t c1 = q.seg_c0[s + 1];
+        uint32_t u = 0, d = 0;
+        for (uint32_t c0 = q.seg_c0[s]; c0 < c1; c0 += SEG_CHUNKS) {
+            uint32_t cu[SEG_CHUNKS], cd[SEG_CHUNKS];
+#pragma unroll
+            for (int j = 0; j < SEG_CHUNKS; ++j) {
+                const bool ok = in && c0 + j < c1;
+                cu[j] = ok ? q.chunk_use[(size_t)(c0 + j) * q.Wv + w] : 0u;
+                cd[j] = ok ? q.chunk_def[(size_t)(c0 + j) * q.Wv + w] : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < SEG_CHUNKS; ++j) { u |= cu[j] & ~d; d |= cd[j]; }
         }
-        __syncthreads();
-        if (w >= Wv) return;
+        seg_u[s * 32 + lane] = u;
+        seg_d[s * 32 + lane] = d;
+    }
+    __syncthreads();
+    for (uint32_t b = warp; b < q.nB; b += FLOW_WARPS) {
+        uint32_t u = 0, d = 0;
+        for (uint32_t s = q.blk_seg_off[b]; s < q.blk_seg_off[b + 1]; ++s) { u |= seg_u[s * 32 + lane] & ~d; d |= seg_d[s * 32 + lane]; }
+        s_use[b * 32 + lane] = u;
+        s_def[b * 32 + lane] = d;
+        s_in[b * 32 + lane] = 0;
+        s_out[b * 32 + lane] = 0;
+    }
+    __syncthreads();
+    if (warp == 0) {
         bool changed = true;
-        for (uint32_t sweep = 0; sweep < nB + 2 && changed; ++sweep) {
+        for (uint32_t sweep = 0; sweep < q.nB + 2 && __any_sync(0xffffffffu, changed); ++sweep) {
             changed = false;
-            for (uint32_t n = 0; n < nB; ++n) {
-                const uint32_t b = nB - 1 - n;
+            for (uint32_t b = q.nB; b-- > 0;) {
                 uint32_t o = 0;
-                for (uint32_t e = s_so[b]; e < s_so[b + 1]; ++e) o |= s_in[s_su[e] * NT + t];
-                const uint32_t in = s_use[b * NT + t] | (o & ~s_def[b * NT + t]);
-                if (o != s_out[b * NT + t] || in != s_in[b * NT + t]) changed = true;
-                s_out[b * NT + t] = o;
-                s_in[b * NT + t] = in;
+                for (uint32_t e = s_so[b]; e < s_so[b + 1]; ++e) o |= s_in[s_su[e] * 32 + lane];
+                const uint32_t i = s_use[b * 32 + lane] | (o & ~s_def[b * 32 + lane]);
+                if (o != s_out[b * 32 + lane] || i != s_in[b * 32 + lane]) changed = true;
+                s_out[b * 32 + lane] = o;
+                s_in[b * 32 + lane] = i;
             }
         }
-        for (uint32_t b = 0; b < nB; ++b) {
-            live_in[(size_t)b * Wv + w] = s_in[b * NT + t];
-            live_out[(size_t)b * Wv + w] = s_out[b * NT + t];
-        }
-        if (changed) atomicOr(status, ST_NO_CONVERGE);
-        if (s_in[t] != 0) atomicOr(status, ST_NOT_STRICT);  // block 0 is the entry
-        return;
+        uint32_t st = changed ? (uint32_t)ST_NO_CONVERGE : 0u;
+        if (s_in[lane] != 0) st |= ST_NOT_STRICT;  // block 0 is the entry
+        st = __reduce_or_sync(0xffffffffu, st);
+        if (st && lane == 0) atomicOr(q.status, st);
     }
-    if (w >= Wv) return;
-    bool changed = true;
-    for (uint32_t sweep = 0; sweep < nB + 2 && changed; ++sweep) {
-        changed = false;
-        for (uint32_t n = 0; n < nB; ++n) {
-            const uint32_t b = nB - 1 - n;
-            uint32_t o = 0;
-            for (uint32_t e = succ_off[b]; e < succ_off[b + 1]; ++e) o |= live_in[(size_t)succ[e] * Wv + w];
-            const uint32_t in = blk_use[(size_t)b * Wv + w] | (o & ~blk_def[(size_t)b * Wv + w]);
-            if (o != live_out[(size_t)b * Wv + w] || in != live_in[(size_t)b * Wv + w]) changed = true;
-            live_out[(size_t)b * Wv + w] = o;
-            live_in[(size_t)b * Wv + w] = in;
+    __syncthreads();
+    for (uint32_t b = warp; b < q.nB; b += FLOW_WARPS) {
+        uint32_t live = s_out[b * 32 + lane];
+        if (in) {
+            q.blk_in[(size_t)b * q.Wv + w] = s_in[b * 32 + lane];
+            q.blk_out[(size_t)b * q.Wv + w] = live;
+        }
+        for (uint32_t s = q.blk_seg_off[b + 1]; s-- > q.blk_seg_off[b];) {  // seg_u becomes the live set behind the segment
+            const uint32_t u = seg_u[s * 32 + lane], d = seg_d[s * 32 + lane];
+            seg_u[s * 32 + lane] = live;
+            live = u | (live & ~d);
         }
     }
-    if (changed) atomicOr(status, ST_NO_CONVERGE);
-    if (live_in[w] != 0) atomicOr(status, ST_NOT_STRICT);  // block 0 is the entry
+    __syncthreads();
+    for (uint32_t s = warp; s < q.nSeg; s += FLOW_WARPS) {
+        uint32_t live = seg_u[s * 32 + lane];
+        const uint32_t c_lo = q.seg_c0[s];
+        for (uint32_t c1 = q.seg_c0[s + 1]; c1 > c_lo;) {
+            uint32_t cu[SEG_CHUNKS], cd[SEG_CHUNKS];
+#pragma unroll
+            for (int j = 0; j < SEG_CHUNKS; ++j) {
+                const bool ok = in && c1 - c_lo > (uint32_t)j;
+                cu[j] = ok ? q.chunk_use[(size_t)(c1 - 1 - j) * q.Wv + w] : 0u;
+                cd[j] = ok ? q.chunk_def[(size_t)(c1 - 1 - j) * q.Wv + w] : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < SEG_CHUNKS; ++j)
+                if (in && c1 - c_lo > (uint32_t)j) {
+                    q.chunk_end[(size_t)(c1 - 1 - j) * q.Wv + w] = live;
+                    live = cu[j] | (live & ~cd[j]);
+                    q.chunk_entry[(size_t)(c1 - 1 - j) * q.Wv + w] = live;
+                }
+            c1 -= min(c1 - c_lo, (uint32_t)SEG_CHUNKS);
+        }
+    }
 }
 
-// Live set after the last instruction of every child (chunk_end) and before its first (chunk_entry,
-// may be null), walking a parent's children backwards from the parent's live-out set: chunks of a
-// block, or pieces of a chunk.
-__global__ void k_chunk_boundaries(const uint32_t *__restrict__ blk_chunk_off, uint32_t Wv,
-                                   const uint32_t *__restrict__ live_out, const uint32_t *__restrict__ chunk_use,
-                                   const uint32_t *__restrict__ chunk_def, uint32_t *chunk_end, uint32_t *chunk_entry)
+// ============================================================================ k_count
+// One thread block per chunk.  First the live set after the last instruction of every piece (one thread per
+// bitset word, backwards over the chunk's pieces).  Then one warp per piece, one lane per operand: an operand's
+// vreg is live after its instruction iff the next instruction of the piece that touches it reads it, or, if
+// none does, iff it is live after the piece.  From that the operand flags, the walk events and the change of
+// the live count of every instruction follow without a serial walk; and the set of vregs whose occupancy
+// changes inside the block.  Last, offsets inside the chunk.
+__global__ void __launch_bounds__(PC_NT) k_count(const LiveArgs q)
 {
-    const uint32_t b = blockIdx.y, w = blockIdx.x * NT + threadIdx.x;  // one bitset word per thread
-    if (w >= Wv) return;
-    const uint32_t c_lo = blk_chunk_off[b], c_hi = blk_chunk_off[b + 1];
-    uint32_t live = live_out[(size_t)b * Wv + w];
-    if (chunk_entry) {
-#pragma unroll 8
-        for (uint32_t c = c_hi; c-- > c_lo;) {
-            chunk_end[(size_t)c * Wv + w] = live;
-            live = chunk_use[(size_t)c * Wv + w] | (live & ~chunk_def[(size_t)c * Wv + w]);
-            chunk_entry[(size_t)c * Wv + w] = live;
+    __shared__ uint32_t s_scan[34], s_ev[PC_WARPS][PIECE_INSTRS];
+    __shared__ int s_d[PC_WARPS][PIECE_INSTRS];
+    const uint32_t c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t p0 = q.chunk_piece_off[c], p1 = q.chunk_piece_off[c + 1];
+    const uint32_t blk = q.chunk_blk[c];
+    uint32_t *touch = q.blk_touch + (size_t)blk * q.Wv;
+    PieceOps po;
+    uint32_t x0 = 0xFFFFFFFFu;  // the first 32 operands of the warp's (first) piece: all of them, as a rule
+    if (p0 + warp < p1) {
+        po.init(q, p0 + warp, c, lane);
+        x0 = po.get(q, lane);
+    }
+    pdl_go();
+    pdl_wait();
+    for (uint32_t w = tid; w < q.Wv; w += PC_NT) {
+        uint32_t live = q.chunk_end[(size_t)c * q.Wv + w];
+        for (uint32_t pe = p1; pe > p0;) {
+            uint32_t pu[8], pd[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bool ok = pe - p0 > (uint32_t)j;
+                pu[j] = ok ? q.piece_use[(size_t)(pe - 1 - j) * q.Wv + w] : 0u;
+                pd[j] = ok ? q.piece_def[(size_t)(pe - 1 - j) * q.Wv + w] : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (pe - p0 > (uint32_t)j) {
+                    q.piece_end[(size_t)(pe - 1 - j) * q.Wv + w] = live;
+                    live = pu[j] | (live & ~pd[j]);
+                }
+            pe -= min(pe - p0, 8u);
+        }
+    }
+    __syncthreads();
+    for (uint32_t p = p0 + warp; p < p1; p += PC_WARPS) {
+        const uint32_t *end = q.piece_end + (size_t)p * q.Wv;
+        if (p != p0 + warp) {
+            po.init(q, p, c, lane);
+            x0 = po.get(q, lane);
+        }
+        if (lane < PIECE_INSTRS) { s_ev[warp][lane] = 0; s_d[warp][lane] = 0; }
+        uint32_t cnt = 0;
+        for (uint32_t w = lane; w < q.Wv; w += 32) cnt += __popc(end[w]);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        __syncwarp();
+        for (uint32_t r = 0; r < po.n; r += 32) {
+            const uint32_t x = r == 0 ? x0 : po.get(q, r + lane), v = po_vreg(x), k = po_instr(x);
+            const bool mine = r + lane < po.n, def = po_def(x);
+            const uint32_t nd = __shfl_sync(0xffffffffu, po.nd, k < PIECE_INSTRS ? k : 0);
+            const uint32_t touched = mine ? __ldcg(&touch[v >> 5]) : 0u;
+            const uint32_t live_end = mine ? (end[v >> 5] >> (v & 31)) & 1u : 0u;
+            uint32_t next = 0xFFFFFFFFu;  // next touch: instruction * 2 + (1 if it only writes)
+            bool dup = false, other = false;  // an earlier read of the instruction has the vreg; its other side (reads / writes) has it
+            for (uint32_t j0 = 0; j0 < po.n; j0 += 32) {
+                const uint32_t y = j0 == r ? x : po.get(q, j0 + lane);
+                const uint32_t nj = (min(32u, po.n - j0) + 7u) & ~7u;  // (lanes beyond the piece hold no vreg)
+                for (uint32_t j8 = 0; j8 < nj; j8 += 8)
+#pragma unroll
+                    for (uint32_t u = 0; u < 8; ++u) {
+                        const uint32_t z = __shfl_sync(0xffffffffu, y, j8 + u);
+                        const bool same = po_vreg(z) == v, later = (z & 0xF0000u) > (x & 0xF0000u);
+                        const bool here = same && po_instr(z) == k;
+                        if (same && later) next = min(next, po_instr(z) * 2 + (po_def(z) ? 1u : 0u));
+                        other |= here && po_def(z) != def;
+                        dup |= here && po_def(z) == def && j0 + j8 + u < r + lane;
+                    }
+            }
+            if (mine) {
+                const bool lv = next == 0xFFFFFFFFu ? live_end != 0 : (next & 1u) == 0;
+                uint32_t flags, evs = 0;
+                if (!def) {
+                    const bool kill = !dup && !lv;  // a read of a vreg that stays live releases nothing
+                    flags = (kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0);
+                    if (kill) evs = 1;
+                    // live before the instruction, but not among what is live behind it and not written by it
+                    if (!dup && !(lv && !other)) atomicAdd(&s_d[warp][k], 1);
+                } else {
+                    const bool elide = other && lv, post = !lv && nd > 1;
+                    flags = OPF_DEF | (elide ? OPF_ELIDE : 0) | ((lv || nd > 1) ? OPF_SET : 0) | (post ? OPF_POST : 0) |
+                            (lv ? 0 : OPF_DEAD);
+                    if (!elide) evs = 1 + (post ? 1 : 0);
+                    if (lv) atomicSub(&s_d[warp][k], 1);
+                }
+                q.opflags[po.ob + r + lane] = (uint8_t)flags;
+                if (evs) {
+                    atomicAdd(&s_ev[warp][k], evs);
+                    const uint32_t bit = 1u << (v & 31);
+                    if (!(touched & bit)) atomicOr(&touch[v >> 5], bit);
+                }
+            }
+        }
+        __syncwarp();
+        // live after instruction k = live after the piece + what the later instructions add going backwards
+        if (lane < po.ni) {
+            const uint32_t i = q.piece_i0[p] + lane;
+            int live = (int)cnt;
+            for (uint32_t u = lane + 1; u < po.ni; ++u) live += s_d[warp][u];
+            q.lo_rel[i] = (uint32_t)live;
+            q.ev_rel[i] = s_ev[warp][lane];
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    const uint32_t i0 = q.chunk_i0[c], i1 = q.chunk_i1[c];
+    unsigned long long lo_sum = 0;
+    uint32_t ev_sum = 0;
+    for (uint32_t ib = i0; ib < i1; ib += PC_NT) {
+        const uint32_t i = ib + tid;
+        const uint32_t a = i < i1 ? q.lo_rel[i] : 0u, e = i < i1 ? q.ev_rel[i] : 0u;
+        uint32_t ta, te;  // (PC_NT lists of at most 65,535 entries: 32 bits hold the sum)
+        const uint32_t xa = block_excl_scan(a, s_scan, &ta), xe = block_excl_scan(e, s_scan, &te);
+        if (i < i1) { q.lo_rel[i] = (uint32_t)lo_sum + xa; q.ev_rel[i] = ev_sum + xe; }
+        lo_sum += ta;
+        ev_sum += te;
+    }
+    if (tid == 0) { q.chunk_lo[c] = lo_sum; q.chunk_ev[c] = ev_sum; }
+}
+
+// The live set before piece p of chunk c (p0 = the chunk's first piece), one word, without the block's through-set.
+__device__ __forceinline__ uint32_t entry_word(const LiveArgs &q, uint32_t c, uint32_t p, uint32_t p0, uint32_t b, uint32_t w)
+{
+    const uint32_t x = p == p0 ? q.chunk_entry[(size_t)c * q.Wv + w] : q.piece_end[(size_t)(p - 1) * q.Wv + w];
+    const uint32_t th = q.use_th ? q.blk_in[(size_t)b * q.Wv + w] & ~q.blk_touch[(size_t)b * q.Wv + w] : 0u;
+    return x & ~th;
+}
+
+// ============================================================================ k_offsets
+// Thread blocks [0, nC): entry events of a chunk and events of its short chunks; [nC, nC + nB): the through-set
+// of a block (live on entry and never touched by an event inside it).  The block that finishes last makes the
+// offsets: list entries per chunk, walk events per chunk (padded to groups of 8), through-sets per block, steps
+// per 32 short chunks; and writes the totals and the status word to pinned host memory.
+__global__ void __launch_bounds__(OFF_NT) k_offsets(const LiveArgs q)
+{
+    __shared__ uint32_t s_scan[34];
+    __shared__ unsigned long long s_tot[LV_TOTALS];
+    __shared__ uint32_t s_last;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_go();
+    pdl_wait();
+    if (blockIdx.x < q.nC) {
+        const uint32_t c = blockIdx.x, b = q.chunk_blk[c], p0 = q.chunk_piece_off[c];
+        const uint32_t s1 = q.chunk_short_off[c + 1];
+        for (uint32_t s = q.chunk_short_off[c] + warp; s < s1; s += OFF_NT / 32) {
+            const uint32_t p = q.short_p0[s];
+            uint32_t cnt = 0;
+            for (uint32_t w = lane; w < q.Wv; w += 32) cnt += __popc(entry_word(q, c, p, p0, b, w));
+            cnt = __reduce_add_sync(0xffffffffu, cnt);
+            if (lane == 0) {
+                if (p == p0) q.centry_cnt[c] = cnt;
+                const uint32_t ev1 = s + 1 < s1 ? q.ev_rel[q.piece_i0[q.short_p0[s + 1]]] : q.chunk_ev[c];
+                q.short_cnt[s] = cnt + ev1 - q.ev_rel[q.piece_i0[p]];
+            }
         }
     } else {
-#pragma unroll 8
-        for (uint32_t c = c_hi; c-- > c_lo;) {
-            chunk_end[(size_t)c * Wv + w] = live;
-            live = chunk_use[(size_t)c * Wv + w] | (live & ~chunk_def[(size_t)c * Wv + w]);
+        const uint32_t b = blockIdx.x - q.nC;
+        uint32_t cnt = 0, total;
+        for (uint32_t w = tid; w < q.Wv; w += OFF_NT) {
+            const uint32_t t = q.use_th ? q.blk_in[(size_t)b * q.Wv + w] & ~q.blk_touch[(size_t)b * q.Wv + w] : 0u;
+            q.blk_th[(size_t)b * q.Wv + w] = t;
+            cnt += __popc(t);
         }
+        block_excl_scan(cnt, s_scan, &total);
+        if (tid == 0) q.th_cnt[b] = total;
     }
-}
-
-// Backward walk of one piece by one warp.  FILL = false: list sizes, per-operand flags, walk-event
-// counts, and the set of vregs whose occupancy changes inside the chunk.  FILL = true: the lists.
-// The chunk's slice of the operand arrays is staged in shared memory when it fits (WALK_CAP_I
-// instructions, WALK_CAP_O operands); lane 0 does the per-instruction bookkeeping, all lanes the
-// population count / compaction of the live bitset.
-#define WALK_CAP_I 32
-#define WALK_CAP_O 256
-template <bool FILL>
-__global__ void __launch_bounds__(32) k_instr_walk(const uint32_t *__restrict__ chunk_i0,
-                                                   const uint32_t *__restrict__ chunk_i1,
-                                                   const uint32_t *__restrict__ op_off, const uint8_t *__restrict__ ndefs,
-                                                   const uint32_t *__restrict__ op_vreg, uint32_t Wv,
-                                                   const uint32_t *__restrict__ chunk_end, uint32_t *lo_cnt,
-                                                   uint32_t *ev_cnt, uint8_t *opflags,
-                                                   const uint32_t *__restrict__ piece_chunk, uint32_t *chunk_touch,
-                                                   const uint32_t *__restrict__ lo_off, uint32_t *lo,
-                                                   const uint32_t *__restrict__ chunk_blk,
-                                                   const uint32_t *__restrict__ blk_th,
-                                                   const uint32_t *__restrict__ ls_adj,
-                                                   const uint32_t *__restrict__ th_cnt, uint32_t *ls)
-{
-    extern __shared__ uint32_t sm[];
-    uint32_t *s_live = sm, *s_touch = sm + Wv;
-    uint32_t *s_off = sm + 2 * Wv;                 // [WALK_CAP_I + 1]
-    uint32_t *s_lo = s_off + WALK_CAP_I + 1;       // [WALK_CAP_I] list offsets (FILL)
-    uint32_t *s_ops = s_lo + WALK_CAP_I;           // [WALK_CAP_O]
-    uint8_t *s_nd = reinterpret_cast<uint8_t *>(s_ops + WALK_CAP_O);  // [WALK_CAP_I]
-    const uint32_t c = blockIdx.x, lane = threadIdx.x;
-    const uint32_t i0 = chunk_i0[c], i1 = chunk_i1[c];
-    // FILL: second list per instruction without the vregs that stay occupied through the whole block
-    // (s_touch then holds the block's through-set); every instruction of the block has all of them in
-    // its live-after set, so the short list of instruction i starts at lo_off[i] - ls_adj[b] - i * th_cnt[b]
-    uint32_t ls_sub = 0, ls_mul = 0;
-    if (FILL) {
-        const uint32_t b = chunk_blk[piece_chunk[c]];
-        ls_sub = ls_adj[b];
-        ls_mul = th_cnt[b];
-        for (uint32_t w = lane; w < Wv; w += 32) s_touch[w] = blk_th[(size_t)b * Wv + w];
-    }
-    for (uint32_t w = lane; w < Wv; w += 32) {
-        s_live[w] = chunk_end[(size_t)c * Wv + w];
-        if (!FILL) s_touch[w] = 0;
-    }
-    const uint32_t ob = i1 > i0 ? op_off[i0] : 0, oe = i1 > i0 ? op_off[i1] : 0;
-    const bool staged = (i1 - i0) <= WALK_CAP_I && (oe - ob) <= WALK_CAP_O;
-    if (staged) {
-        for (uint32_t i = i0 + lane; i <= i1; i += 32) s_off[i - i0] = op_off[i];
-        for (uint32_t i = i0 + lane; i < i1; i += 32) {
-            s_nd[i - i0] = ndefs[i];
-            if (FILL) s_lo[i - i0] = lo_off[i];
-        }
-        for (uint32_t o = ob + lane; o < oe; o += 32) s_ops[o - ob] = op_vreg[o];
-    }
-    __syncwarp();
-    auto OFF = [&](uint32_t i) { return staged ? s_off[i - i0] : op_off[i]; };
-    auto ND = [&](uint32_t i) -> uint32_t { return staged ? s_nd[i - i0] : ndefs[i]; };
-    auto OP = [&](uint32_t o) { return staged ? s_ops[o - ob] : op_vreg[o]; };
-    const uint32_t rounds = (Wv + 31) / 32;
-    for (uint32_t i = i1; i-- > i0;) {
-        uint32_t total = 0;
-        if (FILL) {
-            // ascending ids, 32 words per round; every non-empty word is broadcast and each lane whose
-            // bit is set writes its id at the rank of that bit: up to 32 consecutive stores per word
-            uint32_t at = staged ? s_lo[i - i0] : lo_off[i];
-            uint32_t at_s = at - ls_sub - i * ls_mul;
-            for (uint32_t r = 0; r < rounds; ++r) {
-                const uint32_t w = r * 32 + lane;
-                const uint32_t mine = w < Wv ? s_live[w] : 0u;
-                const uint32_t mine_th = w < Wv ? s_touch[w] : 0u;
-                uint32_t nz = __ballot_sync(0xffffffffu, mine != 0);
-                while (nz) {
-                    const uint32_t src = __ffs(nz) - 1;
-                    nz &= nz - 1;
-                    const uint32_t x = __shfl_sync(0xffffffffu, mine, src);
-                    const uint32_t y = x & ~__shfl_sync(0xffffffffu, mine_th, src);
-                    const uint32_t id = (r * 32 + src) * 32 + lane, below = (1u << lane) - 1u;
-                    if ((x >> lane) & 1u) lo[at + __popc(x & below)] = id;
-                    if ((y >> lane) & 1u) ls[at_s + __popc(y & below)] = id;
-                    at += __popc(x);
-                    at_s += __popc(y);
-                }
-            }
-        } else {
-            uint32_t cnt = 0;
-            for (uint32_t w = lane; w < Wv; w += 32) cnt += __popc(s_live[w]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&q.counters[0], 1u) == gridDim.x - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // Four warps, four scans side by side; a lane takes up to 8 consecutive values at a time, whose loads are in
+    // flight together.  Exclusive offsets of n values into dst[0..n) (null: none), dst[n] = total, clipped to
+    // 32 bits; the total is returned.
+    auto offsets = [&](uint32_t n, uint32_t *dst, auto value, auto store) -> unsigned long long {
+        unsigned long long carry = 0;
+        for (uint32_t j0 = 0; j0 < n; j0 += 256) {
+            const uint32_t j = j0 + lane * 8;
+            unsigned long long x[8], sum = 0;
 #pragma unroll
-            for (int d = 16; d; d >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, d);
-            total = cnt;
-        }
-        __syncwarp();
-        if (lane == 0) {
-            const uint32_t o0 = OFF(i), o1 = OFF(i + 1), nd = ND(i);
-            if (!FILL) {
-                lo_cnt[i] = total;
-                uint32_t evs = 0;
-                for (uint32_t o = o0 + nd; o < o1; ++o) {
-                    const uint32_t v = OP(o);
-                    bool dup = false;
-                    for (uint32_t q = o0 + nd; q < o; ++q) dup |= (OP(q) == v);
-                    const bool lv = bit_get(s_live, v);
-                    const bool kill = !dup && !lv;  // a read of a vreg that stays live releases nothing
-                    opflags[o] = (uint8_t)((kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0));
-                    if (kill) { ++evs; bit_set(s_touch, v); }
-                }
-                for (uint32_t o = o0; o < o0 + nd; ++o) {
-                    const uint32_t v = OP(o);
-                    bool selfuse = false;
-                    for (uint32_t q = o0 + nd; q < o1; ++q) selfuse |= (OP(q) == v);
-                    const bool lv = bit_get(s_live, v);
-                    const bool elide = selfuse && lv;
-                    const bool set = lv || nd > 1;
-                    const bool post = !lv && nd > 1;
-                    opflags[o] = (uint8_t)(OPF_DEF | (elide ? OPF_ELIDE : 0) | (set ? OPF_SET : 0) |
-                                           (post ? OPF_POST : 0) | (lv ? 0 : OPF_DEAD));
-                    if (!elide) { evs += 1 + (post ? 1 : 0); bit_set(s_touch, v); }
-                }
-                ev_cnt[i] = evs;
-            }
-            for (uint32_t o = o0; o < o0 + nd; ++o) bit_clr(s_live, OP(o));
-            for (uint32_t o = o0 + nd; o < o1; ++o) bit_set(s_live, OP(o));
-        }
-        __syncwarp();
-    }
-    if (!FILL) {  // the vregs whose occupancy changes somewhere in the chunk this piece belongs to
-        const size_t row = (size_t)piece_chunk[c] * Wv;
-        for (uint32_t w = lane; w < Wv; w += 32)
-            if (s_touch[w]) atomicOr(&chunk_touch[row + w], s_touch[w]);
-    }
-}
-
-// Exclusive scan of a u32 array (16-byte aligned) by one block of 1024 threads, 32 items per thread and round;
-// out[n] = total (saturated), total64 exact.
-// Block b of the grid scans in_b into out_b (two arrays per launch).
-__global__ void __launch_bounds__(1024) k_scan(const uint32_t *__restrict__ in0, uint32_t *out0,
-                                               const uint32_t *__restrict__ in1, uint32_t *out1, uint32_t n,
-                                               unsigned long long *totals, uint32_t *status)
-{
-    const uint32_t *__restrict__ in = blockIdx.x ? in1 : in0;
-    uint32_t *out = blockIdx.x ? out1 : out0;
-    unsigned long long *total64 = totals + blockIdx.x;
-    __shared__ uint32_t s_w[33];
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned long long carry = 0;
-    constexpr int IT = 32;
-    for (uint32_t base = 0; base < n; base += 1024 * IT) {
-        const uint32_t i = base + tid * IT;
-        uint32_t x[IT];
-        if (i + IT <= n) {
+            for (int u = 0; u < 8; ++u) x[u] = j + u < n ? value(j + u) : 0ull;
 #pragma unroll
-            for (int j = 0; j < IT; j += 4) {
-                const uint4 v = *reinterpret_cast<const uint4 *>(in + i + j);
-                x[j] = v.x; x[j + 1] = v.y; x[j + 2] = v.z; x[j + 3] = v.w;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < IT; ++j) x[j] = i + j < n ? in[i + j] : 0u;
-        }
-        uint32_t mine = 0;
-#pragma unroll
-        for (int j = 0; j < IT; ++j) mine += x[j];
-        uint32_t inc = mine;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
-            if (lane >= d) inc += y;
-        }
-        __syncthreads();
-        if (lane == 31) s_w[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t t = s_w[lane];
-            uint32_t ti = t;
+            for (int u = 0; u < 8; ++u) sum += x[u];
+            unsigned long long inc = sum;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, ti, d);
-                if (lane >= d) ti += y;
+                const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= (uint32_t)d) inc += y;
             }
-            s_w[lane] = ti - t;
-            if (lane == 31) s_w[32] = ti;
-        }
-        __syncthreads();
-        uint32_t ex = (uint32_t)carry + s_w[warp] + inc - mine;
-        if (i + IT <= n) {
+            unsigned long long at = carry + inc - sum;
 #pragma unroll
-            for (int j = 0; j < IT; j += 4) {
-                uint4 v;
-                v.x = ex; ex += x[j];
-                v.y = ex; ex += x[j + 1];
-                v.z = ex; ex += x[j + 2];
-                v.w = ex; ex += x[j + 3];
-                *reinterpret_cast<uint4 *>(out + i + j) = v;
+            for (int u = 0; u < 8; ++u) {
+                if (j + u < n) store(j + u, (uint32_t)at);
+                at += x[u];
             }
-        } else {
-#pragma unroll
-            for (int j = 0; j < IT; ++j) {
-                if (i + j < n) out[i + j] = ex;
-                ex += x[j];
-            }
+            carry += __shfl_sync(0xffffffffu, inc, 31);
         }
-        carry += s_w[32];
+        if (dst && lane == 0) dst[n] = carry > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)carry;
+        return carry;
+    };
+    auto into = [](uint32_t *dst) { return [dst](uint32_t j, uint32_t at) { dst[j] = at; }; };
+    unsigned long long tot = 0;
+    if (warp == LV_TOT_LO) {
+        tot = offsets(q.nC, q.chunk_lo0, [&](uint32_t c) { return __ldcg(q.chunk_lo + c); }, into(q.chunk_lo0));
+        if (lane == 0) q.lo_off[q.nI] = tot > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)tot;
+    } else if (warp == LV_TOT_EV) {
+        tot = offsets(q.nC, q.cev_off, [&](uint32_t c) -> unsigned long long {
+            return (__ldcg(q.centry_cnt + c) + __ldcg(q.chunk_ev + c) + 7u) / 8u * 8u;
+        }, into(q.cev_off));
+    } else if (warp == LV_TOT_TH) {
+        tot = offsets(q.nB, q.th_off, [&](uint32_t b) -> unsigned long long { return __ldcg(q.th_cnt + b); }, into(q.th_off));
+    } else if (warp == LV_TOT_LS) {
+        // short lists (see vl_program): what the through-sets take off the lists of the blocks before b
+        tot = offsets(q.nB, nullptr, [&](uint32_t b) -> unsigned long long {
+            return (unsigned long long)(q.blk_off[b + 1] - q.blk_off[b]) * __ldcg(q.th_cnt + b);
+        }, [&](uint32_t b, uint32_t pre) { q.ls_adj[b] = pre - q.blk_off[b] * __ldcg(q.th_cnt + b); });
+    } else if (warp == LV_TOT_SEV) {  // a group of 32 short chunks per round: its longest
+        for (uint32_t g = 0; g * 32 < q.nS; ++g) {
+            const uint32_t m = __reduce_max_sync(0xffffffffu, g * 32 + lane < q.nS ? __ldcg(q.short_cnt + g * 32 + lane) : 0u);
+            if (lane == 0) q.sev_off[g] = (uint32_t)tot;
+            tot += m;
+        }
+        if (lane == 0) q.sev_off[(q.nS + 31) / 32] = (uint32_t)tot;
+        tot *= 32;
     }
+    if (warp < LV_TOTALS && lane == 0) s_tot[warp] = tot;
+    __syncthreads();
     if (tid == 0) {
-        out[n] = carry > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)carry;
-        *total64 = carry;
-        if (carry > 0xFFFFFFF0ull) atomicOr(status, ST_SIZE_OVERFLOW);
+        s_tot[LV_TOT_LS] = s_tot[LV_TOT_LO] - s_tot[LV_TOT_LS];
+        uint32_t st = __ldcg(q.status);
+        if (s_tot[LV_TOT_LO] > 0xFFFFFFF0ull) st |= ST_SIZE_OVERFLOW;
+        q.host_out[0] = st;
+        unsigned long long *h = reinterpret_cast<unsigned long long *>(q.host_out + 2);
+        for (int j = 0; j < LV_TOTALS; ++j) h[j] = s_tot[j];
     }
-}
-
-// Through-set of a block: live on entry and never touched by a walk event inside it.
-__global__ void k_block_through(const uint32_t *__restrict__ blk_chunk_off, uint32_t Wv, int use_th,
-                                const uint32_t *__restrict__ live_in, const uint32_t *__restrict__ chunk_touch,
-                                uint32_t *blk_th)
-{
-    const uint32_t b = blockIdx.y, w = blockIdx.x * NT + threadIdx.x;  // one bitset word per thread
-    if (w >= Wv) return;
-    const uint32_t c_lo = blk_chunk_off[b], c_hi = blk_chunk_off[b + 1];
-    uint32_t t = 0;
-#pragma unroll 8
-    for (uint32_t c = c_lo; c < c_hi; ++c) t |= chunk_touch[(size_t)c * Wv + w];
-    blk_th[(size_t)b * Wv + w] = use_th ? (live_in[(size_t)b * Wv + w] & ~t) : 0u;
-}
-
-// chunk_entry &= ~through(block); entry count; events of the chunk = entries + instruction events.
-__global__ void k_chunk_entry(const uint32_t *__restrict__ chunk_blk, const uint32_t *__restrict__ chunk_i0,
-                              const uint32_t *__restrict__ chunk_i1, uint32_t Wv,
-                              const uint32_t *__restrict__ blk_th, uint32_t *chunk_entry,
-                              const uint32_t *__restrict__ ev_off, uint32_t *centry_cnt, uint32_t *cev)
-{
-    __shared__ uint32_t s_scan[34];
-    const uint32_t c = blockIdx.x, b = chunk_blk[c];
-    uint32_t cnt = 0;
-    for (uint32_t w = threadIdx.x; w < Wv; w += NT) {
-        const uint32_t x = chunk_entry[(size_t)c * Wv + w] & ~blk_th[(size_t)b * Wv + w];
-        chunk_entry[(size_t)c * Wv + w] = x;
-        cnt += __popc(x);
-    }
-    uint32_t total;
-    block_excl_scan(cnt, s_scan, &total);
-    if (threadIdx.x == 0) {
-        centry_cnt[c] = total;
-        cev[c] = total + (ev_off[chunk_i1[c]] - ev_off[chunk_i0[c]]);
-    }
-}
-
-__global__ void k_row_popc(uint32_t Wv, const uint32_t *__restrict__ rows, uint32_t *cnt)
-{
-    __shared__ uint32_t s_scan[34];
-    const uint32_t r = blockIdx.x;
-    uint32_t c = 0;
-    for (uint32_t w = threadIdx.x; w < Wv; w += NT) c += __popc(rows[(size_t)r * Wv + w]);
-    uint32_t total;
-    block_excl_scan(c, s_scan, &total);
-    if (threadIdx.x == 0) cnt[r] = total;
 }
 
 // Per instruction: vreg id per operand (16 bit), first occurrence / first definition of every
@@ -489,29 +553,6 @@ __global__ void k_vreg_info(uint32_t V, const uint8_t *__restrict__ width, const
     if (v >= V) return;
     vinfo[v] = width[v] | (first_occ[v] != 0xFFFFFFFFu ? VINFO_OCCURS : 0u) |
                (first_def_instr[v] != 0xFFFFFFFFu ? VINFO_DEFINED : 0u);
-}
-
-// Per instruction: 1 if it has a definition the walk skips (a vreg redefined from itself while it
-// stays occupied); the recount visits only those when a block's through-set collided.
-__global__ void k_instr_flags(uint32_t nI, const uint32_t *__restrict__ op_off, const uint8_t *__restrict__ ndefs,
-                              const uint8_t *__restrict__ opflags, uint8_t *iflags)
-{
-    const uint32_t i = blockIdx.x * NT + threadIdx.x;
-    if (i >= nI) return;
-    uint8_t f = 0;
-    for (uint32_t o = op_off[i]; o < op_off[i] + ndefs[i]; ++o)
-        if (opflags[o] & OPF_ELIDE) f = 1;
-    iflags[i] = f;
-}
-
-// Every event slot starts as a no-op (see put_event for the layout of a group of 8 events).
-__global__ void k_fill_noop(uint4 *dst, size_t n_groups, uint32_t spare_vreg)
-{
-    const uint32_t vv = spare_vreg * 128u, ww = 31u | (31u << 16);
-    for (size_t i = (size_t)blockIdx.x * NT + threadIdx.x; i < n_groups * 7; i += (size_t)gridDim.x * NT) {
-        const uint32_t part = (uint32_t)(i % 7);
-        dst[i] = part < 2 ? make_uint4(vv, vv, vv, vv) : (part == 6 ? make_uint4(ww, ww, ww, ww) : make_uint4(0, 0, 0, 0));
-    }
 }
 
 __global__ void k_operand_meta(uint32_t nI, const uint32_t *__restrict__ op_off, const uint8_t *__restrict__ ndefs,
@@ -591,101 +632,181 @@ __device__ __forceinline__ void put_event(uint4 *ev, size_t idx, uint32_t v, uin
     reinterpret_cast<uint16_t *>(g + 96)[slot] = (uint16_t)(w > 32 ? (0x8000u | w) : (32u - w));
 }
 
-// Walk events of one chunk: entry occupancy (ascending vreg id), then per instruction the
-// releases of dying reads, the definitions, and the releases of dead co-definitions.
-__global__ void k_fill_events(const uint32_t *__restrict__ chunk_i0, const uint32_t *__restrict__ chunk_i1,
-                              const uint32_t *__restrict__ op_off, const uint8_t *__restrict__ ndefs,
-                              const uint32_t *__restrict__ op_vreg, const uint8_t *__restrict__ width,
-                              const uint8_t *__restrict__ opflags, uint32_t Wv,
-                              const uint32_t *__restrict__ chunk_entry, const uint32_t *__restrict__ centry_cnt,
-                              const uint32_t *__restrict__ ev_off, const uint32_t *__restrict__ cev_off,
-                              uint4 *ev, const uint32_t *__restrict__ chunk_blk, uint4 *el, uint32_t *el_count)
+// ============================================================================ k_fill
+// Four kinds of thread blocks in one grid: [0, ceil(nP / LV_WARPS)) live-after lists, a warp per piece; then nC
+// blocks with the walk events of a chunk; then the blocks with the events of short chunks, a warp per
+// short chunk; then nB blocks with the through-set list of a block.
+
+// Appends the set bits of word(w), w = 0 .. Wv - 1, in ascending order: emit(rank, bit index).  One warp.
+// Returns the number of bits.
+template <class W, class F>
+__device__ __forceinline__ uint32_t warp_bits(uint32_t Wv, uint32_t lane, W word, F emit)
 {
-    __shared__ uint32_t s_scan[34];
-    const uint32_t c = blockIdx.x;
-    const size_t base = cev_off[c];
-    uint32_t total;
-    compact_bits(chunk_entry + (size_t)c * Wv, Wv, s_scan, &total, [&](uint32_t rank, uint32_t v) {
-        put_event(ev, base + rank, v, width[v], true, true);
-    });
-    const uint32_t i0 = chunk_i0[c], i1 = chunk_i1[c];
-    const uint32_t e_base = centry_cnt[c];
-    for (uint32_t i = i0 + threadIdx.x; i < i1; i += NT) {
-        uint32_t e = e_base + (ev_off[i] - ev_off[i0]);
-        const uint32_t o0 = op_off[i], o1 = op_off[i + 1], nd = ndefs[i];
-        for (uint32_t o = o0 + nd; o < o1; ++o)
-            if (opflags[o] & OPF_KILL) {
-                const uint32_t v = op_vreg[o];
-                put_event(ev, base + (e++), v, width[v], false, true);
-            }
-        for (uint32_t o = o0; o < o0 + nd; ++o)
-            if (!(opflags[o] & OPF_ELIDE)) {
-                const uint32_t v = op_vreg[o];
-                put_event(ev, base + (e++), v, width[v], true, (opflags[o] & OPF_SET) != 0);
-            } else {  // no event: listed (in any order) for the recount of through-set collisions
-                el[atomicAdd(el_count, 1u)] = make_uint4(i, c, op_vreg[o], chunk_blk[c]);
-            }
-        for (uint32_t o = o0; o < o0 + nd; ++o)
-            if ((opflags[o] & OPF_POST) && !(opflags[o] & OPF_ELIDE)) {
-                const uint32_t v = op_vreg[o];
-                put_event(ev, base + (e++), v, width[v], false, true);
-            }
+    uint32_t at = 0;
+    for (uint32_t w0 = 0; w0 < Wv; w0 += 32) {
+        uint32_t x = w0 + lane < Wv ? word(w0 + lane) : 0u;
+        const uint32_t n = __popc(x);
+        uint32_t inc = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= (uint32_t)d) inc += y;
+        }
+        uint32_t rank = at + inc - n;
+        while (x) {
+            emit(rank++, (w0 + lane) * 32 + __ffs(x) - 1);
+            x &= x - 1;
+        }
+        at += __shfl_sync(0xffffffffu, inc, 31);
     }
+    return at;
 }
 
-__global__ void k_fill_through(uint32_t Wv, const uint32_t *__restrict__ blk_th, const uint8_t *__restrict__ width,
-                               const uint32_t *__restrict__ th_off, uint32_t *th)
+// The walk events of instruction i in order: the releases of dying reads, the definitions, the releases of dead
+// co-definitions: put(index, vreg, test, toggle).  skip(operand) is called for definitions without an event.
+template <class F, class G>
+__device__ __forceinline__ void instr_events(const LiveArgs &q, uint32_t i, F put, G skip)
 {
-    __shared__ uint32_t s_scan[34];
-    const uint32_t b = blockIdx.x;
-    const uint32_t base = th_off[b];
-    uint32_t total;
-    compact_bits(blk_th + (size_t)b * Wv, Wv, s_scan, &total,
-                 [&](uint32_t rank, uint32_t v) { th[base + rank] = v | ((uint32_t)width[v] << 16); });
+    const uint32_t o0 = q.op_off[i], o1 = q.op_off[i + 1], nd = q.ndefs[i];
+    uint32_t e = 0;
+    for (uint32_t o = o0 + nd; o < o1; ++o)
+        if (q.opflags[o] & OPF_KILL) put(e++, q.op_vreg[o], false, true);
+    for (uint32_t o = o0; o < o0 + nd; ++o) {
+        const uint32_t f = q.opflags[o];
+        if (f & OPF_ELIDE) skip(o);
+        else put(e++, q.op_vreg[o], true, (f & OPF_SET) != 0);
+    }
+    if (nd > 1)
+        for (uint32_t o = o0; o < o0 + nd; ++o)
+            if ((q.opflags[o] & OPF_POST) && !(q.opflags[o] & OPF_ELIDE)) put(e++, q.op_vreg[o], false, true);
 }
 
-// First walk event of every chunk (each chunk padded to a multiple of 8 events), first through-set
-// entry of every block, and both totals: totals[2] = events with padding, totals[3] = through entries.
-// One thread block; the arrays are short (chunks, blocks).
-// Also ls_adj[b] (see k_instr_walk) and totals[4] = length of all short live-after lists.
-__global__ void k_offsets(uint32_t nC, uint32_t nB, const uint32_t *__restrict__ cev, const uint32_t *__restrict__ th_cnt,
-                          uint32_t *cev_off, uint32_t *th_off, unsigned long long *totals,
-                          const uint32_t *__restrict__ blk_off, uint32_t *ls_adj)
+__global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
 {
-    __shared__ uint32_t s_scan[34];
-    __shared__ unsigned long long s_carry;
-    if (threadIdx.x == 0) s_carry = 0;
-    __syncthreads();
-    for (int which = 0; which < 2; ++which) {
-        const uint32_t n = which == 0 ? nC : nB;
-        const uint32_t *src = which == 0 ? cev : th_cnt;
-        uint32_t *dst = which == 0 ? cev_off : th_off;
-        for (uint32_t base = 0; base < n; base += NT) {
-            const uint32_t i = base + threadIdx.x;
-            uint32_t x = i < n ? src[i] : 0u;
-            if (which == 0) x = (x + 7u) / 8u * 8u;
-            uint32_t total;
-            const uint32_t ex = block_excl_scan(x, s_scan, &total);
-            const unsigned long long carry = s_carry;
-            if (i < n) dst[i] = (uint32_t)(carry + ex);
-            __syncthreads();
-            if (threadIdx.x == 0) s_carry = carry + total;
-            __syncthreads();
+    extern __shared__ uint32_t sm[];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t role = blockIdx.x;
+    const uint32_t n_list = (q.nP + LV_WARPS - 1) / LV_WARPS, n_short = ((q.nS + 31) & ~31u) / LV_WARPS;
+    if (role < n_list) {
+        // Backward walk of one piece.  Two lists per instruction: the vregs live after it, ascending, and the same
+        // without the block's through-set (every instruction of the block has all of that in its live-after set, so
+        // the short list of instruction i starts at lo_off[i] - ls_adj[b] - i * th_cnt[b]).  Every non-empty word
+        // of the live set is broadcast and each lane whose bit is set writes its id at the rank of that bit.
+        const uint32_t p = role * LV_WARPS + warp;
+        const bool mine = p < q.nP;
+        const uint32_t c = mine ? q.piece_chunk[p] : 0u, b = mine ? q.chunk_blk[c] : 0u;
+        PieceOps po;
+        uint32_t x0 = 0xFFFFFFFFu;  // the first 32 operands (all of them, as a rule)
+        if (mine) {
+            po.init(q, p, c, lane);
+            x0 = po.get(q, lane);
         }
-        if (threadIdx.x == 0) {
-            dst[n] = s_carry > 0xFFFFFFF0ull ? 0xFFFFFFF0u : (uint32_t)s_carry;
-            totals[2 + which] = s_carry;
-            s_carry = 0;
+        pdl_wait();
+        if (!mine) return;
+        const uint32_t ls_sub = q.ls_adj[b], ls_mul = q.th_cnt[b];
+        uint32_t *s_live = sm + (size_t)warp * 2 * q.Wv, *s_th = s_live + q.Wv;
+        for (uint32_t w = lane; w < q.Wv; w += 32) {
+            s_live[w] = q.piece_end[(size_t)p * q.Wv + w];
+            s_th[w] = q.blk_th[(size_t)b * q.Wv + w];
         }
-        __syncthreads();
+        const uint32_t i0 = q.piece_i0[p];
+        uint32_t my_lo = 0;
+        if (lane < po.ni) {
+            my_lo = q.chunk_lo0[c] + q.lo_rel[i0 + lane];
+            q.lo_off[i0 + lane] = my_lo;
+        }
+        __syncwarp();
+        const uint32_t rounds = (q.Wv + 31) / 32, below = (1u << lane) - 1u;
+        for (uint32_t k = po.ni; k-- > 0;) {
+            const uint32_t i = i0 + k;
+            uint32_t at = __shfl_sync(0xffffffffu, my_lo, k), at_s = at - ls_sub - i * ls_mul;
+            for (uint32_t r = 0; r < rounds; ++r) {
+                const uint32_t w = r * 32 + lane;
+                const uint32_t mine = w < q.Wv ? s_live[w] : 0u;
+                const uint32_t mine_th = w < q.Wv ? s_th[w] : 0u;
+                uint32_t nz = __ballot_sync(0xffffffffu, mine != 0);
+                while (nz) {
+                    const uint32_t src = __ffs(nz) - 1;
+                    nz &= nz - 1;
+                    const uint32_t x = __shfl_sync(0xffffffffu, mine, src);
+                    const uint32_t y = x & ~__shfl_sync(0xffffffffu, mine_th, src);
+                    const uint32_t id = (r * 32 + src) * 32 + lane;
+                    if ((x >> lane) & 1u) q.lo[at + __popc(x & below)] = id;
+                    if ((y >> lane) & 1u) q.ls[at_s + __popc(y & below)] = id;
+                    at += __popc(x);
+                    at_s += __popc(y);
+                }
+            }
+            __syncwarp();
+            for (uint32_t r = 0; r < po.n; r += 32) {  // live before the instruction: without its definitions ...
+                const uint32_t x = r == 0 ? x0 : po.get(q, r + lane);
+                if (r + lane < po.n && po_instr(x) == k && po_def(x)) atomicAnd(&s_live[po_vreg(x) >> 5], ~(1u << (x & 31)));
+            }
+            __syncwarp();
+            for (uint32_t r = 0; r < po.n; r += 32) {  // ... with its reads
+                const uint32_t x = r == 0 ? x0 : po.get(q, r + lane);
+                if (r + lane < po.n && po_instr(x) == k && !po_def(x)) atomicOr(&s_live[po_vreg(x) >> 5], 1u << (x & 31));
+            }
+            __syncwarp();
+        }
+        return;
     }
-    if (threadIdx.x == 0) {
-        unsigned long long pre = 0;  // through-set entries of all instructions of the blocks before b
-        for (uint32_t b = 0; b < nB; ++b) {
-            ls_adj[b] = (uint32_t)pre - blk_off[b] * th_cnt[b];
-            pre += (unsigned long long)(blk_off[b + 1] - blk_off[b]) * th_cnt[b];
+    pdl_wait();
+    role -= n_list;
+    if (role < q.nC) {  // walk events of a chunk: entry occupancy (ascending vreg id), then instruction by instruction
+        const uint32_t c = role, b = q.chunk_blk[c], p0 = q.chunk_piece_off[c];
+        const size_t base = q.cev_off[c];
+        const uint32_t n_entry = q.centry_cnt[c], n_ev = n_entry + q.chunk_ev[c];
+        if (warp == 0)
+            warp_bits(q.Wv, lane, [&](uint32_t w) { return entry_word(q, c, p0, p0, b, w); },
+                      [&](uint32_t rank, uint32_t v) { put_event(q.ev, base + rank, v, q.width[v], true, true); });
+        const uint32_t i1 = q.chunk_i1[c];
+        for (uint32_t i = q.chunk_i0[c] + (tid + LV_NT - 32) % LV_NT; i < i1; i += LV_NT) {
+            const size_t at = base + n_entry + q.ev_rel[i];
+            instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) { put_event(q.ev, at + e, v, q.width[v], test, toggle); },
+                         [&](uint32_t o) {  // listed (in any order) for the recount of through-set collisions
+                             q.el[atomicAdd(q.el_count, 1u)] = make_uint4(i, c, q.op_vreg[o], b);
+                         });
         }
-        totals[4] = totals[0] - pre;
+        // no-ops up to a whole group, and two no-op groups behind the last chunk (the walk reads ahead)
+        const uint32_t n_pad = (8u - (n_ev & 7u)) % 8u + (c == q.nC - 1 ? 16u : 0u);
+        if (tid < n_pad) put_event(q.ev, base + n_ev + tid, q.V, 1u, false, false);
+        return;
+    }
+    role -= q.nC;
+    if (role < n_short) {
+        // events of a short chunk, 4 bytes each: vreg | width << 16 | test << 24 | toggle << 25; 32 short chunks side
+        // by side, step by step, padded with zeros to the longest of the 32
+        const uint32_t s = role * LV_WARPS + warp;
+        const uint32_t steps = q.sev_off[(s >> 5) + 1] - q.sev_off[s >> 5];
+        uint32_t *dst = q.sev + (size_t)q.sev_off[s >> 5] * 32 + (s & 31);
+        uint32_t n = 0;
+        if (s < q.nS) {
+            const uint32_t p = q.short_p0[s], c = q.piece_chunk[p], b = q.chunk_blk[c], p0 = q.chunk_piece_off[c];
+            const uint32_t n_entry = warp_bits(q.Wv, lane, [&](uint32_t w) { return entry_word(q, c, p, p0, b, w); },
+                                               [&](uint32_t rank, uint32_t v) {
+                                                   dst[(size_t)rank * 32] = v | ((uint32_t)q.width[v] << 16) | (3u << 24);
+                                               });
+            const uint32_t i0 = q.piece_i0[p];
+            const uint32_t i1 = s + 1 < q.chunk_short_off[c + 1] ? q.piece_i0[q.short_p0[s + 1]] : q.chunk_i1[c];
+            const uint32_t ev0 = q.ev_rel[i0];
+            for (uint32_t i = i0 + lane; i < i1; i += 32) {
+                const uint32_t at = n_entry + q.ev_rel[i] - ev0;
+                instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) {
+                    dst[(size_t)(at + e) * 32] = v | ((uint32_t)q.width[v] << 16) | (test ? 1u << 24 : 0u) | (toggle ? 1u << 25 : 0u);
+                }, [](uint32_t) {});
+            }
+            n = q.short_cnt[s];
+        }
+        for (uint32_t e = n + lane; e < steps; e += 32) dst[(size_t)e * 32] = 0;
+        return;
+    }
+    role -= n_short;
+    {   // through-set list of a block: vreg | width << 16
+        const uint32_t b = role;
+        if (warp == 0)
+            warp_bits(q.Wv, lane, [&](uint32_t w) { return q.blk_th[(size_t)b * q.Wv + w]; },
+                      [&](uint32_t rank, uint32_t v) { q.th[q.th_off[b] + rank] = v | ((uint32_t)q.width[v] << 16); });
     }
 }
 
@@ -696,23 +817,51 @@ cudaError_t pool_get(VlArena &arena, T **out, size_t n)
 {
     return arena.alloc((void **)out, std::max<size_t>(n, 1) * sizeof(T) + 64);
 }
+
+// once per device: the kernels with a bitset or two per warp may use the whole shared memory of an SM
+int live_attributes(vl_program *p)
+{
+    static std::mutex mtx;
+    static bool done[64];
+    if (p->device < 0 || p->device >= 64) return VL_OK;
+    std::lock_guard<std::mutex> lock(mtx);
+    if (done[p->device]) return VL_OK;
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_flow, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_fill, at, 227 * 1024));
+    done[p->device] = true;
+    return VL_OK;
+}
 }  // namespace
 #define KEEP(out, n) VL_CUDA(p, pool_get(p->live_arena, out, n))
 #define TMP(out, n) VL_CUDA(p, pool_get(p->tmp_arena, out, n))
 #define LAYOUT(out, n) VL_CUDA(p, pool_get(p->layout_arena, out, n))
 
-static inline bool grid_nonempty(uint32_t g) { return g > 0; }
-static inline bool grid_nonempty(dim3 g) { return g.x > 0 && g.y > 0 && g.z > 0; }
-#define LAUNCH(kernel, grid, smem, st, ...)                          \
-    do {                                                             \
-        if (grid_nonempty(grid)) {                                   \
-            kernel<<<(grid), NT, (smem), (st)>>>(__VA_ARGS__);       \
-            g_vl_launches.fetch_add(1);                              \
-        }                                                            \
+// A launch that may overlap the tail of the launch before it (see pdl_wait).
+template <typename K>
+static cudaError_t launch_pdl(K kernel, uint32_t grid, uint32_t nt, size_t smem, cudaStream_t st, const LiveArgs &q)
+{
+    if (!grid) return cudaSuccess;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = nt; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    g_vl_launches.fetch_add(1);
+    return cudaLaunchKernelEx(&cfg, kernel, q);
+}
+#define LAUNCH(kernel, grid, nt, smem, st, ...)                 \
+    do {                                                        \
+        if ((grid) > 0) {                                       \
+            kernel<<<(grid), (nt), (smem), (st)>>>(__VA_ARGS__); \
+            g_vl_launches.fetch_add(1);                         \
+        }                                                       \
     } while (0)
 
-// Chunks, pieces and walk items depend on the program and on the chunk size only: they are laid
-// out (and uploaded) when the chunk size changes, not on every call.
+// Chunks, pieces, short chunks and segments depend on the program and on the chunk size only: they are laid
+// out (and uploaded, in one copy) when the chunk size changes, not on every call.
 static int vl_layout(vl_program *p, cudaStream_t st)
 {
     if (p->layout_chunk_instrs == p->chunk_instrs) return VL_OK;
@@ -724,19 +873,18 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     p->tables_built = false;
     p->d_vreg16 = nullptr; p->d_slotmeta = nullptr; p->d_opoff = nullptr; p->d_first4 = nullptr;
     p->d_first_def_instr = nullptr; p->d_vinfo = nullptr;
-    std::vector<uint32_t> c_i0, c_i1, c_blk, blk_c_off(nB + 1, 0), p_i0, p_i1, p_chunk, c_p_off;
+    std::vector<uint32_t> c_i0, c_i1, c_blk, blk_c_off(nB + 1, 0), p_i0, p_chunk, c_p_off, seg_c0, blk_seg_off(nB + 1, 0);
     for (uint32_t b = 0; b < nB; ++b) {
         const uint64_t s = p->h_blk_off[b], n = p->h_blk_off[b + 1] - s;
         uint64_t nc = (n + p->chunk_instrs - 1) / p->chunk_instrs;
-        // a walk item is shared by 8 warps, one chunk each at a time: a chunk count that is a multiple
-        // of 8 keeps them equally busy (the chunks get a little shorter than asked for)
+        // a thread block of the walk takes 8 chunks, one per warp: a chunk count that is a multiple
+        // of 8 keeps the warps equally busy (the chunks get a little shorter than asked for)
         if (nc > 4 && n >= 8 * 16) nc = (nc + 7) / 8 * 8;
         for (uint64_t j = 0; j < nc; ++j) {
             const uint32_t i0 = (uint32_t)(s + j * n / nc), i1 = (uint32_t)(s + (j + 1) * n / nc);
             c_p_off.push_back((uint32_t)p_i0.size());
             for (uint32_t q0 = i0; q0 < i1; q0 += PIECE_INSTRS) {
                 p_i0.push_back(q0);
-                p_i1.push_back(std::min(i1, q0 + PIECE_INSTRS));
                 p_chunk.push_back((uint32_t)c_i0.size());
             }
             c_i0.push_back(i0);
@@ -748,43 +896,63 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     c_p_off.push_back((uint32_t)p_i0.size());
     const uint32_t nC = p->nC = (uint32_t)c_i0.size();
     p->nP = (uint32_t)p_i0.size();
-    // walk work items: runs of at most VL_ITEM_CHUNKS chunks of one block
-    std::vector<uint32_t> it_blk, it_c0, it_c1;
-    for (uint32_t b = 0; b < nB; ++b)
-        for (uint32_t c = blk_c_off[b]; c < blk_c_off[b + 1]; c += VL_ITEM_CHUNKS) {
-            it_blk.push_back(b);
-            it_c0.push_back(c);
-            it_c1.push_back(std::min(c + VL_ITEM_CHUNKS, blk_c_off[b + 1]));
+    // segments of k_flow: at most about 256 of them beside one per block
+    const uint32_t seg = std::max<uint32_t>(SEG_CHUNKS, (nC + 255) / 256);
+    for (uint32_t b = 0; b < nB; ++b) {
+        for (uint32_t c = blk_c_off[b]; c < blk_c_off[b + 1]; c += seg) seg_c0.push_back(c);
+        blk_seg_off[b + 1] = (uint32_t)seg_c0.size();
+    }
+    p->nSeg = (uint32_t)seg_c0.size();
+    seg_c0.push_back(nC);
+    // short chunks: as few pieces as keep their number within SHORT_CHUNKS, equally long inside a chunk
+    std::vector<uint32_t> s_p0, c_s_off(nC + 1, 0), s_blk;
+    for (uint32_t r = std::max(1u, (p->nP + SHORT_CHUNKS - 1) / SHORT_CHUNKS);; ++r) {
+        uint64_t total = 0;
+        for (uint32_t c = 0; c < nC; ++c) total += (c_p_off[c + 1] - c_p_off[c] + r - 1) / r;
+        if (total > SHORT_CHUNKS && total > nC) continue;  // (a chunk is the longest they can get)
+        for (uint32_t c = 0; c < nC; ++c) {
+            const uint32_t n = c_p_off[c + 1] - c_p_off[c], k = (n + r - 1) / r;
+            for (uint32_t j = 0; j < k; ++j) {
+                s_p0.push_back(c_p_off[c] + (uint32_t)((uint64_t)n * j / k));
+                s_blk.push_back(c_blk[c]);
+            }
+            c_s_off[c + 1] = (uint32_t)s_p0.size();
         }
-    p->nItems = (uint32_t)it_blk.size();
-    auto up = [&](uint32_t **dst, const std::vector<uint32_t> &v) -> int {
-        LAYOUT(dst, v.size());
-        if (!v.empty()) VL_CUDA(p, cudaMemcpy(*dst, v.data(), v.size() * 4, cudaMemcpyHostToDevice));
-        return VL_OK;
-    };
-    int rc;
-    if ((rc = up(&p->d_chunk_i0, c_i0)) || (rc = up(&p->d_chunk_i1, c_i1)) || (rc = up(&p->d_chunk_blk, c_blk)) ||
-        (rc = up(&p->d_blk_chunk_off, blk_c_off)) || (rc = up(&p->d_piece_i0, p_i0)) || (rc = up(&p->d_piece_i1, p_i1)) ||
-        (rc = up(&p->d_piece_chunk, p_chunk)) || (rc = up(&p->d_chunk_piece_off, c_p_off)) ||
-        (rc = up(&p->d_item_blk, it_blk)) || (rc = up(&p->d_item_c0, it_c0)) || (rc = up(&p->d_item_c1, it_c1)))
-        return rc;
+        break;
+    }
+    p->nS = (uint32_t)s_p0.size();
+    std::vector<uint32_t> all;
+    struct Part { uint32_t **dst; const std::vector<uint32_t> *v; };
+    const Part parts[] = {{&p->d_chunk_i0, &c_i0}, {&p->d_chunk_i1, &c_i1}, {&p->d_chunk_blk, &c_blk},
+                          {&p->d_blk_chunk_off, &blk_c_off}, {&p->d_piece_i0, &p_i0}, {&p->d_piece_chunk, &p_chunk},
+                          {&p->d_chunk_piece_off, &c_p_off}, {&p->d_seg_c0, &seg_c0}, {&p->d_blk_seg_off, &blk_seg_off},
+                          {&p->d_short_p0, &s_p0}, {&p->d_chunk_short_off, &c_s_off}, {&p->d_short_blk, &s_blk}};
+    for (const Part &x : parts) {
+        all.insert(all.end(), x.v->begin(), x.v->end());
+        all.resize((all.size() + 4) & ~(size_t)3);  // (at least one word behind every array)
+    }
+    uint32_t *dev = nullptr;
+    LAYOUT(&dev, all.size());
+    VL_CUDA(p, cudaMemcpy(dev, all.data(), all.size() * 4, cudaMemcpyHostToDevice));
+    size_t at = 0;
+    for (const Part &x : parts) {
+        *x.dst = dev + at;
+        at = (at + x.v->size() + 4) & ~(size_t)3;
+    }
     const uint32_t Wp = (p->P + p->wmax + 31) / 32 + 1;
     p->use_th = (nB <= 32 && (uint64_t)nB * VL_MAX_GROUP * Wp * 4 <= 24 * 1024) ? 1 : 0;
     p->layout_chunk_instrs = p->chunk_instrs;
-    (void)nC;
     return VL_OK;
 }
 
-// Enqueues one complete liveness run on st (every kernel, the clears before them, the copy of the
-// status word and the list lengths to pinned host memory behind them).  Without remembered list
-// lengths it waits once in the middle to read them.
+// Enqueues one complete liveness run on st.  Without remembered list lengths it waits once in the middle to
+// read them.
 static int live_enqueue(vl_program *p, cudaStream_t st)
 {
     vl_free_liveness(p);
-    int rc = VL_OK;
+    int rc = live_attributes(p);
+    if (rc != VL_OK) return rc;
     const uint32_t nB = p->nB, nI = p->nI, V = p->V, nO = p->nO, Wv = p->Wv, nC = p->nC, nP = p->nP;
-    const size_t smem2 = (size_t)2 * Wv * 4;
-    const size_t walk_smem = smem2 + (size_t)(2 * WALK_CAP_I + 1 + WALK_CAP_O) * 4 + WALK_CAP_I + 16;
 
     // ---- results and tables that do not depend on the list lengths
     KEEP(&p->d_blk_in, (size_t)2 * nB * Wv);  // live-in rows, then live-out rows
@@ -801,7 +969,6 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
         LAYOUT(&p->d_vinfo, (size_t)V);
         LAYOUT(&p->d_opoff, (size_t)p->nOpT / 4);
     }
-    KEEP(&p->d_iflags, (size_t)nI);
     KEEP(&p->d_cev_off, (size_t)nC + 1);
     KEEP(&p->d_th_off, (size_t)nB + 1);
     KEEP(&p->d_th_cnt, (size_t)nB);
@@ -809,215 +976,111 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     KEEP(&p->d_blk_th, (size_t)nB * Wv);
     KEEP(&p->d_el, (size_t)nO);  // at most one entry per definition
     KEEP(&p->d_el_count, 1);
+    KEEP(&p->d_sev_off, (size_t)(p->nS + 31) / 32 + 1);
 
-    uint32_t *piece_use, *piece_def, *piece_end, *chunk_use, *chunk_def, *chunk_touch, *chunk_end, *chunk_entry;
-    uint32_t *blk_use, *blk_def, *lo_cnt, *ev_cnt, *ev_off, *centry_cnt, *cev, *first_occ;
-    uint32_t *const blk_th = p->d_blk_th, *const th_cnt = p->d_th_cnt;
-    uint8_t *opmeta;
-    unsigned long long *totals;
-    TMP(&piece_use, (size_t)nP * Wv);
-    TMP(&piece_def, (size_t)nP * Wv);
-    TMP(&piece_end, (size_t)nP * Wv);
-    TMP(&chunk_use, (size_t)nC * Wv);
-    TMP(&chunk_def, (size_t)nC * Wv);
-    TMP(&chunk_end, (size_t)nC * Wv);
-    TMP(&chunk_entry, (size_t)nC * Wv);
-    TMP(&blk_use, (size_t)nB * Wv);
-    TMP(&blk_def, (size_t)nB * Wv);
-    TMP(&lo_cnt, (size_t)nI + 1);
-    TMP(&ev_cnt, (size_t)nI + 1);
-    TMP(&ev_off, (size_t)nI + 1);
-    TMP(&centry_cnt, (size_t)nC);
-    TMP(&cev, (size_t)nC);
-    first_occ = nullptr;
-    opmeta = nullptr;
+    LiveArgs q{};
+    q.nB = nB; q.nI = nI; q.V = V; q.nE = p->nE; q.Wv = Wv; q.nC = nC; q.nP = nP; q.nS = p->nS; q.nSeg = p->nSeg;
+    q.use_th = p->use_th;
+    q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg; q.succ_off = p->d_succ_off; q.succ = p->d_succ; q.blk_off = p->d_blk_off;
+    q.ndefs = p->d_ndefs; q.width = p->d_width;
+    q.chunk_i0 = p->d_chunk_i0; q.chunk_i1 = p->d_chunk_i1; q.chunk_blk = p->d_chunk_blk; q.blk_chunk_off = p->d_blk_chunk_off;
+    q.piece_i0 = p->d_piece_i0; q.piece_chunk = p->d_piece_chunk; q.chunk_piece_off = p->d_chunk_piece_off;
+    q.seg_c0 = p->d_seg_c0; q.blk_seg_off = p->d_blk_seg_off; q.short_p0 = p->d_short_p0; q.chunk_short_off = p->d_chunk_short_off;
+    TMP(&q.piece_use, (size_t)nP * Wv);
+    TMP(&q.piece_def, (size_t)nP * Wv);
+    TMP(&q.piece_end, (size_t)nP * Wv);
+    TMP(&q.chunk_use, (size_t)nC * Wv);
+    TMP(&q.chunk_def, (size_t)nC * Wv);
+    TMP(&q.chunk_end, (size_t)nC * Wv);
+    TMP(&q.chunk_entry, (size_t)nC * Wv);
+    TMP(&q.blk_touch, (size_t)nB * Wv);
+    TMP(&q.lo_rel, (size_t)nI);
+    TMP(&q.ev_rel, (size_t)nI);
+    TMP(&q.chunk_lo, (size_t)nC);
+    TMP(&q.chunk_ev, (size_t)nC);
+    TMP(&q.chunk_lo0, (size_t)nC + 1);
+    TMP(&q.centry_cnt, (size_t)nC);
+    TMP(&q.short_cnt, (size_t)p->nS);
+    TMP(&q.counters, 1);
+    const uint32_t fgrid = (Wv + 31) / 32;
+    size_t flow_smem = (((size_t)4 * nB + 2 * (size_t)p->nSeg) * 32 + nB + 1 + p->nE) * 4;
+    if (flow_smem > 200 * 1024) {
+        TMP(&q.flow_scratch, flow_smem / 4 * fgrid);
+        flow_smem = 0;
+    }
+    uint32_t *first_occ = nullptr;
+    uint8_t *opmeta = nullptr;
     if (make_tables) {
         TMP(&first_occ, (size_t)V);
         TMP(&opmeta, (size_t)nO);
-    }
-    TMP(&chunk_touch, (size_t)nC * Wv + 16);  // followed by the totals: one memset clears both
-    totals = reinterpret_cast<unsigned long long *>(chunk_touch + (((size_t)nC * Wv + 1) & ~(size_t)1));
-    // what has to start from a known value: the fixed point's sets, the touch sets (updated with
-    // atomics), the totals, the status word, and the two "lowest index so far" arrays
-    VL_CUDA(p, cudaMemsetAsync(p->d_blk_in, 0, (size_t)2 * nB * Wv * 4, st));
-    VL_CUDA(p, cudaMemsetAsync(chunk_touch, 0, ((size_t)nC * Wv + 16) * 4, st));
-    VL_CUDA(p, cudaMemsetAsync(p->d_status, 0, 4, st));
-    VL_CUDA(p, cudaMemsetAsync(p->d_el_count, 0, 4, st));
-    if (make_tables) {
         VL_CUDA(p, cudaMemsetAsync(first_occ, 0xFF, std::max<size_t>(V, 1) * 4, st));
         VL_CUDA(p, cudaMemsetAsync(p->d_first_def_instr, 0xFF, std::max<size_t>(V, 1) * 4, st));
     }
+    q.blk_in = p->d_blk_in; q.blk_out = p->d_blk_out; q.lo_off = p->d_lo_off; q.opflags = p->d_opflags;
+    q.cev_off = p->d_cev_off; q.th_off = p->d_th_off; q.th_cnt = p->d_th_cnt; q.ls_adj = p->d_ls_adj; q.blk_th = p->d_blk_th;
+    q.el = p->d_el; q.el_count = p->d_el_count; q.status = p->d_status; q.sev_off = p->d_sev_off;
+    q.host_out = p->h_live;
+    // a bitset pair per warp of k_sets: fewer warps for programs of very many vregs
+    const uint32_t set_warps = (uint32_t)std::max<size_t>(1, std::min<size_t>(PC_WARPS, (size_t)224 * 1024 / ((size_t)2 * Wv * 4)));
 
-    LAUNCH(k_chunk_sets, nP, smem2, st, p->d_piece_i0, p->d_piece_i1, p->d_op_off, p->d_ndefs, p->d_op_vreg, Wv,
-           piece_use, piece_def);
-    const uint32_t wgrid = (Wv + NT - 1) / NT;
-    if (nC) LAUNCH(k_block_sets, dim3(wgrid, nC), 0, st, p->d_chunk_piece_off, Wv, piece_use, piece_def, chunk_use, chunk_def);
-    LAUNCH(k_block_sets, dim3(wgrid, nB), 0, st, p->d_blk_chunk_off, Wv, chunk_use, chunk_def, blk_use, blk_def);
-    {
-        const size_t fp_smem = ((size_t)4 * nB * NT + nB + 1 + p->nE) * 4;
-        if (fp_smem <= 48 * 1024)
-            LAUNCH(k_fixed_point<true>, wgrid, fp_smem, st, nB, p->nE, Wv, p->d_succ_off, p->d_succ, blk_use, blk_def,
-                   p->d_blk_in, p->d_blk_out, p->d_status);
-        else
-            LAUNCH(k_fixed_point<false>, wgrid, 0, st, nB, p->nE, Wv, p->d_succ_off, p->d_succ, blk_use, blk_def,
-                   p->d_blk_in, p->d_blk_out, p->d_status);
-    }
-    LAUNCH(k_chunk_boundaries, dim3(wgrid, nB), 0, st, p->d_blk_chunk_off, Wv, p->d_blk_out, chunk_use, chunk_def,
-           chunk_end, chunk_entry);
-    if (nC) LAUNCH(k_chunk_boundaries, dim3(wgrid, nC), 0, st, p->d_chunk_piece_off, Wv, chunk_end, piece_use, piece_def,
-                   piece_end, (uint32_t *)nullptr);
-    if (nP) k_instr_walk<false><<<nP, 32, walk_smem, st>>>(p->d_piece_i0, p->d_piece_i1, p->d_op_off, p->d_ndefs,
-           p->d_op_vreg, Wv, piece_end, lo_cnt, ev_cnt, p->d_opflags, p->d_piece_chunk, chunk_touch,
-           (const uint32_t *)nullptr, (uint32_t *)nullptr, (const uint32_t *)nullptr, (const uint32_t *)nullptr,
-           (const uint32_t *)nullptr, (const uint32_t *)nullptr, (uint32_t *)nullptr);
-    k_scan<<<2, 1024, 0, st>>>(lo_cnt, p->d_lo_off, ev_cnt, ev_off, nI, totals, p->d_status);
-    g_vl_launches.fetch_add(nP ? 2 : 1);
-    LAUNCH(k_block_through, dim3(wgrid, nB), 0, st, p->d_blk_chunk_off, Wv, p->use_th, p->d_blk_in, chunk_touch, blk_th);
-    LAUNCH(k_chunk_entry, nC, 0, st, p->d_chunk_blk, p->d_chunk_i0, p->d_chunk_i1, Wv, blk_th, chunk_entry, ev_off,
-           centry_cnt, cev);
-    LAUNCH(k_row_popc, nB, 0, st, Wv, blk_th, th_cnt);
-    k_offsets<<<1, NT, 0, st>>>(nC, nB, cev, th_cnt, p->d_cev_off, p->d_th_off, totals, p->d_blk_off, p->d_ls_adj);
-    g_vl_launches.fetch_add(1);
+    LAUNCH(k_sets, std::max(1u, nC), set_warps * 32, (size_t)set_warps * 2 * Wv * 4, st, q);
+    VL_CUDA(p, launch_pdl(k_flow, fgrid, FLOW_WARPS * 32, flow_smem, st, q));
+    VL_CUDA(p, launch_pdl(k_count, nC, PC_NT, 0, st, q));
+    VL_CUDA(p, launch_pdl(k_offsets, nC + nB, OFF_NT, 0, st, q));
 
-    // ---- list lengths: read back on the first run with this layout; later runs allocate from the
+    // ---- list lengths: read on the first run with this layout; later runs allocate from the
     // lengths they remember (same program, same layout) and only compare at the end
-    uint32_t status = 0;
-    unsigned long long h_tot[5] = {0, 0, 0, 0, 0};
     if (!p->sizes_known) {
-        VL_CUDA(p, cudaMemcpyAsync(&status, p->d_status, 4, cudaMemcpyDeviceToHost, st));
-        VL_CUDA(p, cudaMemcpyAsync(h_tot, totals, 40, cudaMemcpyDeviceToHost, st));
         VL_CUDA(p, cudaStreamSynchronize(st));
+        const uint32_t status = p->h_live[0];
+        unsigned long long tot[LV_TOTALS];
+        memcpy(tot, p->h_live + 2, sizeof(tot));
         if (status & ST_NO_CONVERGE) return VL_ERR_NO_CONVERGE;
         if (status & ST_NOT_STRICT) return VL_ERR_NOT_STRICT;
         if (status & ST_SIZE_OVERFLOW) return VL_ERR_UNSUPPORTED;
-        if (h_tot[2] > 0xFFFFFFF0ull) return VL_ERR_UNSUPPORTED;
-        p->known_lo_len = h_tot[0];
-        p->known_steps = h_tot[2];
-        p->known_thn = h_tot[3];
-        p->known_ls_len = h_tot[4];
+        if (tot[LV_TOT_EV] > 0xFFFFFFF0ull || tot[LV_TOT_SEV] > 0xFFFFFFF0ull) return VL_ERR_UNSUPPORTED;
+        memcpy(p->known, tot, sizeof(tot));
     }
-    p->lo_len = p->known_lo_len;
-    const uint64_t steps = p->known_steps;  // walk events in total, every chunk padded to a multiple of 8 with no-ops
-    p->ev_total = (uint32_t)steps;
-    p->th_len = (uint32_t)p->known_thn;
-
+    p->lo_len = p->known[LV_TOT_LO];
     KEEP(&p->d_lo, (size_t)p->lo_len);
-    KEEP(&p->d_ls, (size_t)p->known_ls_len);
-    KEEP(&p->d_ev, (size_t)(steps / 8 + 2) * 7);  // two no-op groups behind the last chunk: the walk reads ahead
-    KEEP(&p->d_th, (size_t)p->known_thn);
-    LAUNCH(k_fill_noop, (uint32_t)std::min<uint64_t>(1024, (steps + NT - 1) / NT + 1), 0, st, p->d_ev,
-           (size_t)(steps / 8 + 2), V);  // every slot starts as a no-op event
-
-    // The list fill, the operand tables and the walk events do not depend on each other: the latter
-    // two run on side streams beside the fill (as parallel branches when the run is recorded).
-    cudaStream_t *lanes = nullptr;
-    rc = vl_lane_streams(p, &lanes);
-    if (rc != VL_OK) return rc;
-    cudaStream_t sa = lanes[VL_LANES], sb = lanes[VL_LANES + 1];
-    VL_CUDA(p, cudaEventRecord(p->ev_side[0], st));
-    VL_CUDA(p, cudaStreamWaitEvent(sa, p->ev_side[0], 0));
-    VL_CUDA(p, cudaStreamWaitEvent(sb, p->ev_side[0], 0));
-    if (nP) k_instr_walk<true><<<nP, 32, walk_smem, st>>>(p->d_piece_i0, p->d_piece_i1, p->d_op_off, p->d_ndefs,
-           p->d_op_vreg, Wv, piece_end, (uint32_t *)nullptr, (uint32_t *)nullptr, (uint8_t *)nullptr,
-           (const uint32_t *)p->d_piece_chunk, (uint32_t *)nullptr, (const uint32_t *)p->d_lo_off, p->d_lo,
-           (const uint32_t *)p->d_chunk_blk, (const uint32_t *)blk_th, (const uint32_t *)p->d_ls_adj,
-           (const uint32_t *)th_cnt, p->d_ls);
-    if (nP) g_vl_launches.fetch_add(1);
+    KEEP(&p->d_ls, (size_t)p->known[LV_TOT_LS]);
+    KEEP(&p->d_ev, (size_t)(p->known[LV_TOT_EV] / 8 + 2) * 7);  // two no-op groups behind the last chunk
+    KEEP(&p->d_th, (size_t)p->known[LV_TOT_TH]);
+    KEEP(&p->d_sev, (size_t)p->known[LV_TOT_SEV]);
+    q.lo = p->d_lo; q.ls = p->d_ls; q.ev = p->d_ev; q.th = p->d_th; q.sev = p->d_sev;
+    const uint32_t n_list = (nP + LV_WARPS - 1) / LV_WARPS, n_short = ((p->nS + 31) & ~31u) / LV_WARPS;
+    VL_CUDA(p, launch_pdl(k_fill, n_list + nC + n_short + nB, LV_NT, (size_t)LV_WARPS * 2 * Wv * 4, st, q));
     if (make_tables) {
-        LAUNCH(k_first_occ, (nI + NT - 1) / NT, 0, sa, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, first_occ,
+        LAUNCH(k_first_occ, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, first_occ,
                p->d_first_def_instr);
-        LAUNCH(k_vreg_info, (V + NT - 1) / NT, 0, sa, V, p->d_width, first_occ, p->d_first_def_instr, p->d_vinfo);
-        LAUNCH(k_operand_meta, (nI + NT - 1) / NT, 0, sa, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, first_occ,
+        LAUNCH(k_vreg_info, (V + NT - 1) / NT, NT, 0, st, V, p->d_width, first_occ, p->d_first_def_instr, p->d_vinfo);
+        LAUNCH(k_operand_meta, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, first_occ,
                p->d_opflags, p->d_vreg16, opmeta, p->d_status);
-        LAUNCH(k_pack_slots, (p->nOpT / 8 + NT - 1) / NT, 0, sa, nO, p->nOp8, p->nOpT / 8, V, opmeta, p->d_vreg16, p->d_slotmeta,
-               p->d_opoff, p->d_first4);
+        LAUNCH(k_pack_slots, (p->nOpT / 8 + NT - 1) / NT, NT, 0, st, nO, p->nOp8, p->nOpT / 8, V, opmeta, p->d_vreg16,
+               p->d_slotmeta, p->d_opoff, p->d_first4);
     }
-    LAUNCH(k_instr_flags, (nI + NT - 1) / NT, 0, sa, nI, p->d_op_off, p->d_ndefs, p->d_opflags, p->d_iflags);
-    LAUNCH(k_fill_events, nC, 0, sb, p->d_chunk_i0, p->d_chunk_i1, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_width,
-           p->d_opflags, Wv, chunk_entry, centry_cnt, ev_off, p->d_cev_off, p->d_ev, p->d_chunk_blk, p->d_el,
-           p->d_el_count);
-    LAUNCH(k_fill_through, nB, 0, sb, Wv, blk_th, p->d_width, p->d_th_off, p->d_th);
-    VL_CUDA(p, cudaEventRecord(p->ev_side[1], sa));
-    VL_CUDA(p, cudaEventRecord(p->ev_side[2], sb));
-    VL_CUDA(p, cudaStreamWaitEvent(st, p->ev_side[1], 0));
-    VL_CUDA(p, cudaStreamWaitEvent(st, p->ev_side[2], 0));
     p->bank_fast = ((p->B == 1 || p->B == 2 || p->B == 4) && !p->bank_many) ? 1 : 0;
-    VL_CUDA(p, cudaMemcpyAsync(p->h_live, p->d_status, 4, cudaMemcpyDeviceToHost, st));
-    VL_CUDA(p, cudaMemcpyAsync(p->h_live + 2, totals, 40, cudaMemcpyDeviceToHost, st));
     p->tables_built = true;
-    return rc;
+    return VL_OK;
 }
 
-// A run is the same sequence of launches with the same arguments every time once the layout and
-// the list lengths are settled (the pools hand out the same addresses after a rewind).  The third
-// run with settled lengths is therefore recorded as a CUDA graph while it is enqueued, and later
-// runs replay the graph: one launch call instead of about thirty, which is what small programs and
-// batches of programs spend their time on.  Everything is recomputed on the device on every run.
+// One run.  Everything is recomputed on the device every time.
 int vl_liveness_impl(vl_program *p, cudaStream_t st)
 {
     vl_live_settle(p);  // the pinned words of an earlier run are about to be reused
     int rc = vl_layout(p, st);
     if (rc != VL_OK) return rc;
-    if (!p->h_live) VL_CUDA(p, cudaHostAlloc((void **)&p->h_live, 64, cudaHostAllocDefault));
+    if (!p->h_live) VL_CUDA(p, cudaHostAlloc((void **)&p->h_live, 128, cudaHostAllocDefault));
     if (!p->ev_live) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_live, cudaEventDisableTiming));
-    if (!p->sizes_known) vl_drop_live_graph(p);
-    bool replayed = false;
-    if (p->sizes_known && p->live_graph) {
-        if (cudaGraphLaunch(p->live_graph, st) == cudaSuccess) {
-            g_vl_launches.fetch_add(p->live_graph_launches);
-            replayed = true;
-        } else {
-            cudaGetLastError();
-            vl_drop_live_graph(p);
-        }
-    }
-    if (!replayed) {
-        bool capturing = false;
-        cudaStream_t rec = st;
-        if (p->sizes_known && p->graph_opt && ++p->settled_runs >= 2) {
-            // recorded on an internal stream (the caller's may be the legacy default stream, which
-            // cannot record; nothing runs while recording), then launched on the caller's
-            cudaStream_t *lanes = nullptr;
-            if (vl_lane_streams(p, &lanes) == VL_OK) {
-                rec = lanes[0];
-                capturing = cudaStreamBeginCapture(rec, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-            }
-            if (!capturing) { cudaGetLastError(); p->graph_opt = 0; rec = st; }
-        }
-        const uint64_t launches0 = g_vl_launches.load();
-        rc = live_enqueue(p, rec);
-        if (capturing) {
-            cudaGraph_t graph = nullptr;
-            cudaError_t e = cudaStreamEndCapture(rec, &graph);
-            if (e == cudaSuccess && rc == VL_OK) e = cudaGraphInstantiate(&p->live_graph, graph, 0);
-            if (graph) cudaGraphDestroy(graph);
-            if (e != cudaSuccess || rc != VL_OK) {
-                cudaGetLastError();
-                vl_drop_live_graph(p);
-                p->graph_opt = 0;  // recording does not work here: enqueue directly from now on
-                if (rc == VL_OK) rc = live_enqueue(p, st);
-            } else {
-                p->live_graph_launches = g_vl_launches.load() - launches0;
-                VL_CUDA(p, cudaGraphLaunch(p->live_graph, st));  // what was recorded has not run yet
-            }
-        }
-        if (rc != VL_OK) return rc;
-    }
+    if ((rc = live_enqueue(p, st)) != VL_OK) return rc;
     VL_CUDA(p, cudaEventRecord(p->ev_live, st));
     VL_CUDA(p, cudaGetLastError());
     p->live_pending = true;
     p->live_ok = true;
     if (p->sizes_known) return VL_OK;  // lengths remembered from an earlier run: checked when the results are used
     rc = vl_live_settle(p);
-    if (rc == VL_OK) { p->sizes_known = true; p->settled_runs = 0; }
+    if (rc == VL_OK) p->sizes_known = true;
     return rc;
-}
-
-void vl_drop_live_graph(vl_program *p)
-{
-    if (p->live_graph) cudaGraphExecDestroy(p->live_graph);
-    p->live_graph = nullptr;
-    p->settled_runs = 0;
 }
 
 int vl_live_settle(vl_program *p)
@@ -1027,13 +1090,12 @@ int vl_live_settle(vl_program *p)
     p->live_ok = false;
     VL_CUDA(p, cudaEventSynchronize(p->ev_live));
     const uint32_t status = p->h_live[0];
-    unsigned long long h_tot[5];
-    memcpy(h_tot, p->h_live + 2, 40);
+    unsigned long long tot[LV_TOTALS];
+    memcpy(tot, p->h_live + 2, sizeof(tot));
     if (status & ST_NO_CONVERGE) return VL_ERR_NO_CONVERGE;
     if (status & ST_NOT_STRICT) return VL_ERR_NOT_STRICT;
     if (status & ST_SIZE_OVERFLOW) return VL_ERR_UNSUPPORTED;
-    if (h_tot[0] != p->known_lo_len || h_tot[2] != p->known_steps || h_tot[3] != p->known_thn ||
-        h_tot[4] != p->known_ls_len) {
+    if (memcmp(tot, p->known, sizeof(tot)) != 0) {
         // the lengths the run allocated from do not fit what it computed: the next run measures again
         p->sizes_known = false;
         return VL_ERR_CUDA;

@@ -109,7 +109,7 @@ struct RParams {
     int bank_fast;
     uint64_t K;
     const uint32_t *vinfo, *chunk_i0, *chunk_i1, *chunk_blk, *blk_chunk_off, *th_off, *th, *op_off, *op_vreg, *lo_off, *lo;
-    const uint8_t *ndefs, *width, *opflags, *iflags;
+    const uint8_t *ndefs, *width, *opflags;
     const uint16_t *tg;
     const uint32_t *cstate, *anom;
     uint32_t *racc;
@@ -2410,7 +2410,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     rq.ls = p->d_ls; rq.ls_adj = p->d_ls_adj; rq.th_cnt = p->d_th_cnt; rq.R = p->P + p->wmax + 2;
     rq.vinfo = p->d_vinfo; rq.chunk_i0 = p->d_chunk_i0; rq.chunk_i1 = p->d_chunk_i1; rq.chunk_blk = p->d_chunk_blk;
     rq.op_off = p->d_op_off; rq.op_vreg = p->d_op_vreg; rq.lo_off = p->d_lo_off; rq.lo = p->d_lo;
-    rq.ndefs = p->d_ndefs; rq.width = p->d_width; rq.opflags = p->d_opflags; rq.iflags = p->d_iflags;
+    rq.ndefs = p->d_ndefs; rq.width = p->d_width; rq.opflags = p->d_opflags;
     rq.racc = vs.racc; rq.status = p->d_status + 1;
     rq.tg = vs.tg; rq.cstate = vs.cstate; rq.anom = vs.anom; rq.work = vs.work; rq.out = d_out;
     rq.bank_list = p->d_bank_list;
