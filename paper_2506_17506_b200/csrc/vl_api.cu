@@ -171,12 +171,14 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
         std::vector<uint4> off((size_t)p->nDT / 4, make_uint4(p->V * 16u, p->V * 16u, p->V * 16u, p->V * 16u));
         std::vector<uint8_t> f4((size_t)p->nDT / 4, 0);
         dict_instr.resize(p->nD8, 0);
+        std::vector<uint32_t> first_entry(p->V ? p->V : 1, 0xFFFFFFFFu);
         for (uint32_t e2 = 0; e2 < p->nD8; ++e2) {
             if (e2 < p->nD) {
                 const uint32_t v = p->h_dict_vreg[e2];
                 v16[e2] = (uint16_t)v;
                 uint32_t *w = &off[e2 / 4].x;
                 w[e2 % 4] = v * 16u;
+                if (is_first[e2]) first_entry[v] = e2;
                 if (is_first[e2]) { slot[e2 / 8] |= 1ull << (e2 % 8); f4[e2 / 4] |= (uint8_t)(1u << (e2 % 4)); }
             } else {
                 slot[e2 / 8] |= 1ull << (e2 % 8);  // padding column: writes the spare table entry, never compared
@@ -186,6 +188,7 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
         if (e == cudaSuccess) e = upload(&p->d_dict_slotmeta, slot.data(), slot.size());
         if (e == cudaSuccess) e = upload(&p->d_dict_opoff, off.data(), off.size());
         if (e == cudaSuccess) e = upload(&p->d_dict_first4, f4.data(), f4.size());
+        if (e == cudaSuccess) e = upload(&p->d_dict_first_occ, first_entry.data(), first_entry.size());
         if (e == cudaSuccess) e = upload(&p->d_dict_instr, dict_instr.data(), dict_instr.size());
     }
     if (e == cudaSuccess) e = cudaMalloc((void **)&p->d_status, 64);
@@ -210,7 +213,8 @@ void vl_free_liveness(vl_program *p)
     p->d_ev = nullptr;
     p->d_el = nullptr; p->d_el_count = nullptr;
     p->d_ls = p->d_ls_adj = p->d_th_cnt = p->d_blk_th = nullptr;
-    p->d_sev_off = p->d_sev = nullptr;
+    p->d_irec = nullptr;
+    p->d_sev_off = p->d_sev = p->d_sen_off = p->d_sen = nullptr;
     p->live_ok = false;
     p->lo_len = 0;
 }
@@ -235,7 +239,7 @@ extern "C" void vl_program_destroy(vl_program *p)
     cudaFree(p->d_ndefs); cudaFree(p->d_op_vreg); cudaFree(p->d_width); cudaFree(p->d_status);
     cudaFree(p->d_bank_list);
     cudaFree(p->d_dict_vreg16); cudaFree(p->d_dict_slotmeta); cudaFree(p->d_dict_opoff); cudaFree(p->d_dict_first4);
-    cudaFree(p->d_dict_instr);
+    cudaFree(p->d_dict_instr); cudaFree(p->d_dict_first_occ);
     cudaFree(p->d_vcons); cudaFree(p->d_rs_prefix);
     for (auto &v : p->vs) { cudaFree(v.tg); cudaFree(v.cstate); cudaFree(v.anom); cudaFree(v.work); cudaFree(v.racc); cudaFree(v.grp_done); cudaFree(v.thm); }
     for (int j = 0; j < 2; ++j) {

@@ -1,0 +1,582 @@
+// The whole check of a candidate by one thread block: the verify path of short jobs.
+//
+// The batched kernels (vl_verify.cu) hand a candidate from kernel to kernel through global memory and want
+// thousands of rows; a job of up to a few hundred rows spends its time in their launches and in chains of
+// dependent L2 loads.  Here a thread block does everything for its candidate out of shared memory:
+//   1. the vreg -> register table T from the first occurrences, with Realizability (file and rules);
+//   2. Consistency: every column against T;
+//   3. the exact bank tally;
+//   4. Safety: one thread per short chunk of instructions toggles the occupancy bits of its chunk's events in
+//      a mask of its own (column `tid` of [word][thread]), starting from the block's through-set and what else is
+//      occupied on entry (which all threads enter together: it needs no order);
+//   5. only if a test found an occupied bit: the exact count of the overlaps in the chunks concerned.
+// A vreg at or beyond P takes part in step 4 as if it sat at P: two of them live together then collide, so
+// that a chunk is never missed, and step 5 compares the true registers.
+#include <algorithm>
+#include <mutex>
+
+#include "vl_internal.cuh"
+
+namespace {
+
+struct FMisc {
+    uint32_t flags, minop, minr, bank, pairs, mind, thcol, any;
+    uint32_t n_list;
+};
+
+// Where the parts of a block's shared memory start (bytes), and how much there is.
+struct FSmem {
+    uint32_t w, th, occ, coll, list, misc, total;
+};
+
+inline uint32_t up16(uint32_t x) { return (x + 15u) & ~15u; }
+
+inline FSmem fused_smem(const vl_program *p, uint32_t threads)
+{
+    const uint32_t Wp = (p->P + p->wmax + 31) / 32;
+    FSmem s;
+    s.w = up16((p->V + 1) * 2);
+    s.th = s.w + up16(p->V + 1);
+    s.occ = s.th + (p->use_th ? up16(p->nB * Wp * 4) : 0u);
+    s.coll = s.occ + up16(std::max(Wp * threads * 4, (p->P + p->wmax + 2) * 8));
+    s.list = s.coll + up16((p->nS + 31) / 32 * 4 + 4);
+    s.misc = s.list + up16(p->nS * 8);
+    s.total = s.misc + up16(sizeof(FMisc));
+    return s;
+}
+
+struct FParams {
+    uint32_t nI, V, nO, P, B, nB, nS, Wp, R, Wv, wmax, short_shift;
+    int bank_fast, use_th;
+    FSmem sm;
+    const uint32_t *first_occ, *vinfo, *first_def_instr, *op_off, *op_vreg, *entry_instr, *blk_off;
+    const uint16_t *vreg16;
+    const uint8_t *opflags;
+    const uint8_t *ndefs;
+    const uint4 *vcons;
+    const uint16_t *rs_prefix;
+    const uint2 *bank_list;
+    uint32_t bank_seg[4];
+    // liveness results
+    const uint32_t *th_off, *th, *blk_th, *sev_off, *sev, *sen_off, *sen, *short_blk, *short_i0, *blk_chunk_off, *chunk_short_off;
+    const uint32_t *ls, *el_count;
+    const uint4 *el, *irec;
+    const uint16_t *cand;
+    uint64_t pitch;
+    vl_verdict *out;
+};
+
+__device__ __forceinline__ bool overlap(uint32_t a, uint32_t wa, uint32_t b, uint32_t wb) { return a < b + wb && b < a + wa; }
+
+// Sources of one list entry that cost a cycle: the register is new among the entry's sources, its bank is not.
+template <int N>
+__device__ __forceinline__ uint32_t bank_extra(const uint32_t (&x)[4], uint32_t bmask)
+{
+    uint32_t n = 0;
+#pragma unroll
+    for (int a = 1; a < N; ++a) {
+        bool value = false, bank = false;
+#pragma unroll
+        for (int b = 0; b < a; ++b) {
+            value |= x[b] == x[a];
+            bank |= ((x[b] ^ x[a]) & bmask) == 0;
+        }
+        n += !value && bank;
+    }
+    return n;
+}
+// An entry with n = 2, 3 or 4 distinct source vregs.
+__device__ __forceinline__ uint32_t bank_entry(const uint2 &id, uint32_t n, const uint16_t *T, uint32_t bmask)
+{
+    const uint32_t x[4] = {T[id.x & 0xFFFFu], T[id.x >> 16], T[id.y & 0xFFFFu], T[id.y >> 16]};
+    return n == 2 ? bank_extra<2>(x, bmask) : (n == 3 ? bank_extra<3>(x, bmask) : bank_extra<4>(x, bmask));
+}
+
+template <int NTHR>
+__global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint16_t *T = reinterpret_cast<uint16_t *>(smem);                 // [V + 1] register of every vreg
+    uint8_t *W = smem + q.sm.w;                                       // [V] width
+    uint32_t *s_th = reinterpret_cast<uint32_t *>(smem + q.sm.th);    // [nB][Wp] through-set masks
+    uint32_t *occ = reinterpret_cast<uint32_t *>(smem + q.sm.occ);    // [Wp][NTHR] masks; later cover[R], start[R]
+    uint32_t *coll = reinterpret_cast<uint32_t *>(smem + q.sm.coll);  // short chunks that collided
+    uint2 *list = reinterpret_cast<uint2 *>(smem + q.sm.list);        // those of a program block: instructions [x, y)
+    FMisc *M = reinterpret_cast<FMisc *>(smem + q.sm.misc);
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t k = blockIdx.x;
+    const uint16_t *row = q.cand + k * q.pitch;
+
+    if (tid == 0) *M = FMisc{0u, 0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u, 0xFFFFFFFFu, 0u, 0u, 0u};
+    if (q.use_th)
+        for (uint32_t j = tid; j < q.nB * q.Wp; j += NTHR) s_th[j] = 0;
+    __syncthreads();
+
+    // Every phase keeps several loads per thread in flight and asks for its first ones before the phase in front of
+    // it computes: with one candidate per block the time is a chain of L2 round trips, not work.
+    constexpr int CU = 3;  // column loads (8 columns each) in flight
+    uint4 r_nx[CU], v_nx[CU];
+    auto fetch_columns = [&](uint32_t o0) {
+#pragma unroll
+        for (int u = 0; u < CU; ++u) {
+            const uint32_t o = o0 + u * NTHR * 8;
+            const bool ok = o < q.nO;
+            r_nx[u] = ok ? *reinterpret_cast<const uint4 *>(row + o) : make_uint4(0, 0, 0, 0);
+            v_nx[u] = ok ? *reinterpret_cast<const uint4 *>(q.vreg16 + o) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    // ---- 1. the table, eight vregs per thread in flight
+    for (uint32_t v0 = tid; v0 < q.V; v0 += 8 * NTHR) {
+        uint32_t pos[8], vi[8], t[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool ok = v0 + u * NTHR < q.V;
+            pos[u] = ok ? q.first_occ[v0 + u * NTHR] : 0xFFFFFFFFu;
+            vi[u] = ok ? q.vinfo[v0 + u * NTHR] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t[u] = pos[u] != 0xFFFFFFFFu ? row[pos[u]] : 0u;
+        if (v0 + 8 * NTHR >= q.V) fetch_columns(tid * 8);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t v = v0 + u * NTHR, w = vi[u] & 0xFFu;
+            if (v >= q.V) break;
+            T[v] = (uint16_t)t[u];
+            W[v] = (uint8_t)w;
+            if (!(vi[u] & VINFO_DEFINED)) continue;
+            bool bad = t[u] + w > q.P;
+            if (q.vcons) {
+                const uint4 vc = q.vcons[v];
+                const uint32_t clo = vc.x & 0xFFFFu, chi = vc.x >> 16, al = vc.y;
+                bad = bad || (al > 1 && t[u] != __umulhi(t[u], vc.z) * al) || t[u] < clo || t[u] + w > chi;
+                if (!bad && q.rs_prefix) bad = q.rs_prefix[min(t[u] + w, q.P)] != q.rs_prefix[min(t[u], q.P)];
+            }
+            if (bad) {
+                atomicOr(&M->flags, (uint32_t)VL_OUT_OF_RANGE);
+                atomicMin(&M->minr, q.first_def_instr[v]);
+            }
+        }
+    }
+    if (tid >= q.V) fetch_columns(tid * 8);  // (a thread without a vreg)
+    if (tid == 0) T[q.V] = 0;
+    __syncthreads();
+
+    // ---- 2. Consistency: 8 columns per load
+    constexpr int BU = 6;  // bank list entries in flight
+    uint2 id_nx[BU];
+    const uint32_t n_ent = q.bank_fast ? q.bank_seg[3] : 0u;
+    auto fetch_bank = [&](uint32_t e0) {
+#pragma unroll
+        for (int u = 0; u < BU; ++u) id_nx[u] = e0 + u * NTHR < n_ent ? q.bank_list[e0 + u * NTHR] : make_uint2(0, 0);
+    };
+    for (uint32_t o0 = tid * 8; o0 < q.nO; o0 += CU * NTHR * 8) {
+        uint4 r4[CU], v4[CU];
+#pragma unroll
+        for (int u = 0; u < CU; ++u) { r4[u] = r_nx[u]; v4[u] = v_nx[u]; }
+        if (o0 + CU * NTHR * 8 < q.nO) fetch_columns(o0 + CU * NTHR * 8);
+        else fetch_bank(tid);
+#pragma unroll
+        for (int u = 0; u < CU; ++u) {
+            const uint32_t o = o0 + u * NTHR * 8;
+            if (o >= q.nO) break;
+            const uint32_t r[4] = {r4[u].x, r4[u].y, r4[u].z, r4[u].w}, v[4] = {v4[u].x, v4[u].y, v4[u].z, v4[u].w};
+            uint32_t d[4], any = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                d[j] = r[j] ^ ((uint32_t)T[v[j] & 0xFFFFu] | ((uint32_t)T[v[j] >> 16] << 16));
+                any |= d[j];
+            }
+            if (any) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (((j & 1) ? d[j >> 1] >> 16 : d[j >> 1] & 0xFFFFu) && o + j < q.nO) {
+                        atomicOr(&M->flags, (uint32_t)VL_INCONSISTENT);
+                        atomicMin(&M->minop, o + j);
+                    }
+            }
+        }
+    }
+    if (tid * 8 >= q.nO) fetch_bank(tid);  // (a thread without a column)
+
+    // ---- 3. bank tally
+    {
+        uint32_t n = 0;
+        for (uint32_t e0 = tid; e0 < n_ent; e0 += BU * NTHR) {
+            uint2 id[BU];
+#pragma unroll
+            for (int u = 0; u < BU; ++u) id[u] = id_nx[u];
+            fetch_bank(e0 + BU * NTHR);
+#pragma unroll
+            for (int u = 0; u < BU; ++u) {
+                const uint32_t e = e0 + u * NTHR;
+                if (e >= n_ent) break;
+                n += bank_entry(id[u], e < q.bank_seg[1] ? 2u : (e < q.bank_seg[2] ? 3u : 4u), T, q.B - 1);
+            }
+        }
+        if (!q.bank_fast) {
+            for (uint32_t i = tid; i < q.nI; i += NTHR) {
+                const uint32_t u0 = q.op_off[i] + q.ndefs[i], u1 = q.op_off[i + 1];
+                for (uint32_t a = u0 + 1; a < u1; ++a) {
+                    const uint32_t xa = T[q.op_vreg[a]];
+                    bool value = false, bank = false;
+                    for (uint32_t b = u0; b < a; ++b) {
+                        const uint32_t xb = T[q.op_vreg[b]];
+                        value |= xb == xa;
+                        bank |= xb % q.B == xa % q.B;
+                    }
+                    n += !value && bank;
+                }
+            }
+        }
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0 && n) atomicAdd(&M->bank, n);
+    }
+
+    // ---- 4. Safety
+    if (q.use_th) {
+        const uint32_t n_th = q.th_off[q.nB];
+        for (uint32_t e = tid; e < n_th; e += NTHR) {
+            const uint32_t x = q.th[e];
+            uint32_t b = 0;
+            while (b + 1 < q.nB && q.th_off[b + 1] <= e) ++b;  // (at most 32 blocks, the offsets sit in L1)
+            uint32_t pos = min((uint32_t)T[x & 0xFFFFu], q.P), left = x >> 16;
+            bool hit = false;
+            while (left) {
+                const uint32_t s2 = pos & 31, n = min(left, 32 - s2);
+                const uint32_t m = (0xFFFFFFFFu >> (32 - n)) << s2;
+                hit |= (atomicOr(&s_th[b * q.Wp + (pos >> 5)], m) & m) != 0;
+                pos += n;
+                left -= n;
+            }
+            if (hit) atomicOr(&M->thcol, 1u << b);  // through-sets are used only if nB <= 32
+        }
+        __syncthreads();
+    }
+    const uint32_t nSr = (q.nS + 31u) & ~31u;
+    for (uint32_t s0 = 0; s0 < nSr; s0 += NTHR) {  // (a warp takes a whole group of 32 short chunks)
+        const uint32_t s = s0 + tid;
+        const bool mine = s < nSr;
+        const uint32_t st0 = mine ? q.sev_off[s >> 5] : 0u, steps = mine ? q.sev_off[(s >> 5) + 1] - st0 : 0u;
+        const uint32_t *ev = q.sev + (size_t)st0 * 32 + lane;
+        constexpr int EU = 8;  // events in flight: loaded ahead, and applied
+        uint32_t nx[EU];
+#pragma unroll
+        for (int u = 0; u < EU; ++u) nx[u] = u < steps ? ev[u * 32] : 0u;
+        uint32_t en[4];
+        const uint32_t e_hi = q.sen_off[min(q.nS, s0 + NTHR)], e_lo = q.sen_off[s0];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) en[u] = e_lo + tid + u * NTHR < e_hi ? q.sen[e_lo + tid + u * NTHR] : 0u;
+        const uint32_t b = s < q.nS && q.use_th ? q.short_blk[s] : 0u;
+        for (uint32_t wd = 0; wd < q.Wp; ++wd) occ[wd * NTHR + tid] = q.use_th ? s_th[b * q.Wp + wd] : 0u;
+        if (mine && lane == 0) coll[s >> 5] = 0;
+        __syncthreads();
+        for (uint32_t e0 = e_lo + tid; e0 < e_hi; e0 += 4 * NTHR) {
+            uint32_t x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                x[u] = en[u];
+                const uint32_t e = e0 + (4 + u) * NTHR;
+                en[u] = e < e_hi ? q.sen[e] : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (e0 + u * NTHR >= e_hi) break;
+                const uint32_t v = x[u] & 0xFFFFu, col = ((x[u] >> 16) - s0) & 0xFFFFu;
+                uint32_t pos = min((uint32_t)T[v], q.P), left = W[v];
+                bool hit = false;
+                while (left) {
+                    const uint32_t s2 = pos & 31, n = min(left, 32 - s2);
+                    const uint32_t m = (0xFFFFFFFFu >> (32 - n)) << s2;
+                    hit |= (atomicOr(&occ[(pos >> 5) * NTHR + col], m) & m) != 0;
+                    pos += n;
+                    left -= n;
+                }
+                if (hit) { atomicOr(&coll[(s0 + col) >> 5], 1u << (col & 31)); M->any = 1; }
+            }
+        }
+        __syncthreads();
+        uint32_t viol = 0;
+        for (uint32_t e0 = 0; e0 < steps; e0 += EU) {
+            uint32_t x[EU], t[EU], old[EU];
+            uint32_t far = 0;  // some range of the batch reaches into the next word
+#pragma unroll
+            for (int u = 0; u < EU; ++u) {
+                x[u] = nx[u];
+                t[u] = min((uint32_t)T[x[u] & 0xFFFFu], q.P);
+                far |= (t[u] & 31) + ((x[u] >> 16) & 0xFFu) > 32 ? 1u : 0u;
+                nx[u] = e0 + EU + u < steps ? ev[(size_t)(e0 + EU + u) * 32] : 0u;
+            }
+            // toggling returns the old word: occupied and released are both a toggle as long as no collision
+            // has been seen (after one, the chunk is counted exactly anyway)
+            if (!far) {
+#pragma unroll
+                for (int u = 0; u < EU; ++u) {
+                    const uint32_t w = (x[u] >> 16) & 0xFFu, m = w ? (0xFFFFFFFFu >> (32 - w)) << (t[u] & 31) : 0u;
+                    old[u] = atomicXor(&occ[(t[u] >> 5) * NTHR + tid], (x[u] >> 25) & 1u ? m : 0u);
+                    t[u] = (x[u] >> 24) & 1u ? m : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < EU; ++u) viol |= old[u] & t[u];
+            } else {
+#pragma unroll 1
+                for (int u = 0; u < EU; ++u) {
+                    uint32_t xu = x[0], pos = t[0];
+#pragma unroll
+                    for (int j = 1; j < EU; ++j)
+                        if (j == u) { xu = x[j]; pos = t[j]; }
+                    const uint32_t tog = 0u - ((xu >> 25) & 1u), test = 0u - ((xu >> 24) & 1u);
+                    uint32_t left = (xu >> 16) & 0xFFu;
+                    while (left) {
+                        const uint32_t s2 = pos & 31, n = min(left, 32 - s2);
+                        const uint32_t m = (0xFFFFFFFFu >> (32 - n)) << s2;
+                        viol |= atomicXor(&occ[(pos >> 5) * NTHR + tid], m & tog) & m & test;
+                        pos += n;
+                        left -= n;
+                    }
+                }
+            }
+        }
+        const uint32_t hits = __ballot_sync(0xffffffffu, viol != 0);
+        if (mine && lane == 0 && hits) {
+            atomicOr(&coll[s >> 5], hits);
+            M->any = 1;
+        }
+        __syncthreads();
+    }
+    __syncthreads();
+
+    // ---- 5. exact counts where something collided: program block by program block
+    if (M->any | M->thcol) {
+        uint32_t *cover = occ, *start = occ + q.R;
+        uint32_t pairs = 0, mind = 0xFFFFFFFFu;
+        for (uint32_t b = 0; b < q.nB; ++b) {
+            const uint32_t s_lo = q.chunk_short_off[q.blk_chunk_off[b]], s_hi = q.chunk_short_off[q.blk_chunk_off[b + 1]];
+            const bool thcol = q.use_th && ((M->thcol >> b) & 1u);
+            if (tid == 0) M->n_list = 0;
+            __syncthreads();
+            for (uint32_t s = s_lo + tid; s < s_hi; s += NTHR)
+                if ((coll[s >> 5] >> (s & 31)) & 1u) list[atomicAdd(&M->n_list, 1u)] = make_uint2(q.short_i0[s], q.short_i0[s + 1]);
+            __syncthreads();
+            const uint32_t n_list = M->n_list;
+            __syncthreads();
+            if (!n_list && !thcol) continue;
+            // The block's through-set, counted into two arrays over the registers (cover[r]: members whose range holds
+            // r, start[r]: members whose range starts at r): a range [s, s+w) overlaps cover[s] + start[s+1] + ... +
+            // start[s+w-1] of them.  Members that reach beyond the arrays lie beyond the file: they are compared
+            // one by one, with definitions that lie there too.
+            const uint32_t t0 = q.th_off[b], n_th = q.th_off[b + 1] - t0;
+            for (uint32_t r = tid; r < 2 * q.R; r += NTHR) occ[r] = 0;
+            __syncthreads();
+            for (uint32_t j = tid; j < n_th; j += NTHR) {
+                const uint32_t v = q.th[t0 + j] & 0xFFFFu, reg = T[v], w = W[v];
+                if (reg + w <= q.R) {
+                    atomicAdd(&start[reg], 1u);
+                    for (uint32_t r = reg; r < reg + w; ++r) atomicAdd(&cover[r], 1u);
+                }
+            }
+            __syncthreads();
+            // through-set members other than v (itself a member: `member`) that overlap v's range; part `sub` of `of`
+            auto through_overlaps = [&](uint32_t v, bool member, uint32_t sub, uint32_t of) {
+                const uint32_t s = T[v], w = W[v];
+                uint32_t n = 0;
+                if (s < q.R) {
+                    if (sub == 0) n = cover[s] - (member && s + w <= q.R ? 1u : 0u);
+                    for (uint32_t r = s + 1 + sub; r < min(s + w, q.R); r += of) n += start[r];
+                }
+                if (s + w > q.P)
+                    for (uint32_t j = sub; j < n_th; j += of) {
+                        const uint32_t u = q.th[t0 + j] & 0xFFFFu;
+                        if (u != v && T[u] + W[u] > q.R && overlap(s, w, T[u], W[u])) ++n;
+                    }
+                return n;
+            };
+            auto is_member = [&](uint32_t v) { return ((q.blk_th[(size_t)b * q.Wv + (v >> 5)] >> (v & 31)) & 1u) != 0; };
+            // Two lanes take an instruction: the entries of its live-after list that are not in the through-set, the
+            // through-set from the arrays.  The record of the instruction after the next and the list entries of
+            // the next are fetched meanwhile.  The width of an entry is read only if its register is near enough.
+            constexpr uint32_t NG = NTHR / 2;
+            constexpr int LU = 12;  // list entries per lane in flight
+            const uint32_t sub = tid & 1u, n_slots = n_list << q.short_shift, len_mask = (1u << q.short_shift) - 1u;
+            auto instr_of = [&](uint32_t f) -> uint32_t {  // 0xFFFFFFFF: beyond the short chunk, or beyond the list
+                if (f >= n_slots) return 0xFFFFFFFFu;
+                const uint2 span = list[f >> q.short_shift];
+                const uint32_t i = span.x + (f & len_mask);
+                return i < span.y ? i : 0xFFFFFFFFu;
+            };
+            auto fetch_rec = [&](uint32_t i) { return i != 0xFFFFFFFFu ? q.irec[i] : make_uint4(0, 0, 0, 0); };
+            uint32_t us_nx[LU];
+            auto fetch_list = [&](const uint4 &r) {
+                const uint32_t n = r.y & 0xFFFFu;
+#pragma unroll
+                for (int u = 0; u < LU; ++u) us_nx[u] = sub + 2 * u < n ? q.ls[r.x + sub + 2 * u] : 0xFFFFFFFFu;
+            };
+            uint32_t i_nx = instr_of(tid / 2), i_nx2 = instr_of(tid / 2 + NG);
+            uint4 rec_nx = fetch_rec(i_nx), rec_nx2 = fetch_rec(i_nx2);
+            fetch_list(rec_nx);
+            for (uint32_t f = tid / 2; f < n_slots; f += NG) {
+                const uint32_t i = i_nx;
+                const uint4 rec = rec_nx;
+                uint32_t us[LU], ts[LU];
+#pragma unroll
+                for (int u = 0; u < LU; ++u) us[u] = us_nx[u];
+                i_nx = i_nx2;
+                rec_nx = rec_nx2;
+                fetch_list(rec_nx);
+                i_nx2 = instr_of(f + 2 * NG);
+                rec_nx2 = fetch_rec(i_nx2);
+                const uint32_t n = rec.y & 0xFFFFu, nd = (rec.y >> 16) & 0xFFu;
+                if (!nd) continue;
+                uint32_t cnt = 0;
+#pragma unroll
+                for (int u = 0; u < LU; ++u) ts[u] = us[u] != 0xFFFFFFFFu ? T[us[u]] : 0x1000000u;  // (near nothing)
+                for (uint32_t d = 0; d < nd; ++d) {
+                    const uint32_t v = d ? q.op_vreg[rec.w + d] : rec.z, sv = T[v], wv = W[v];
+                    // [t, t + wt) overlaps [sv, sv + wv): t < sv + wv and t > sv - wt, wt at most wmax
+                    const uint32_t shift = q.wmax - 1 - sv, span = wv + q.wmax - 1;
+                    cnt += through_overlaps(v, d ? is_member(v) : rec.y >> 31, sub, 2);
+#pragma unroll
+                    for (int u = 0; u < LU; ++u)
+                        if (ts[u] + shift < span)
+                            if (us[u] != v && ts[u] + W[us[u]] > sv) ++cnt;
+                    for (uint32_t e0 = sub + 2 * LU; e0 < n; e0 += 8) {
+                        uint32_t x[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) x[u] = e0 + 2 * u < n ? q.ls[rec.x + e0 + 2 * u] : v;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (x[u] != v && overlap(sv, wv, T[x[u]], W[x[u]])) ++cnt;
+                    }
+                    if (nd > 1)  // co-defined vregs that are not live after the instruction
+                        for (uint32_t d2 = sub; d2 < nd; d2 += 2) {
+                            if (d2 == d || !(q.opflags[rec.w + d2] & OPF_DEAD)) continue;
+                            const uint32_t x = q.op_vreg[rec.w + d2];
+                            if (overlap(sv, wv, T[x], W[x])) ++cnt;
+                        }
+                }
+                if (cnt) { pairs += cnt; mind = min(mind, i); }
+            }
+            // In a chunk whose own walk was clean everything that is live is disjoint from the through-set; a
+            // definition without an event (a member redefined from itself) overlaps the members that overlap it.
+            if (thcol) {
+                const uint32_t n_el = q.el_count[b];
+                const uint4 *el = q.el + q.op_off[q.blk_off[b]];  // instruction, chunk, vreg | member << 31, short chunk
+                for (uint32_t e0 = tid; e0 < n_el; e0 += 4 * NTHR) {
+                    uint4 x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = e0 + u * NTHR < n_el ? el[e0 + u * NTHR] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (!(x[u].z >> 31) || ((coll[x[u].w >> 5] >> (x[u].w & 31)) & 1u)) continue;
+                        const uint32_t n = through_overlaps(x[u].z & 0xFFFFu, true, 0, 1);
+                        if (n) { pairs += n; mind = min(mind, x[u].x); }
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        pairs = __reduce_add_sync(0xffffffffu, pairs);
+        mind = __reduce_min_sync(0xffffffffu, mind);
+        if (lane == 0 && pairs) {
+            atomicAdd(&M->pairs, pairs);
+            atomicMin(&M->mind, mind);
+        }
+        __syncthreads();
+    }
+
+    // ---- the verdict
+    if (warp == 0) {
+        uint32_t first = min(M->minr, M->mind);
+        const uint32_t o = M->minop;
+        if (o != 0xFFFFFFFFu) {
+            uint32_t i;
+            if (q.entry_instr) {
+                // dictionary rows: entries are in block order and, inside a block, in order of first occurrence, so the
+                // lowest violating entry is also the lowest violating instruction
+                i = q.entry_instr[o];
+            } else {  // operand -> instruction: the last i with op_off[i] <= operand, 32 probes per round
+                uint32_t lo = 0, hi = q.nI;  // op_off[lo] <= o < op_off[hi]
+                while (hi - lo > 1) {
+                    const uint32_t step = (hi - lo + 31) / 32, at = min(lo + (lane + 1) * step, hi);
+                    const uint32_t below = __popc(__ballot_sync(0xffffffffu, q.op_off[at] <= o));  // (op_off ascends)
+                    const uint32_t nlo = min(lo + below * step, hi);
+                    hi = min(nlo + step, hi);
+                    lo = nlo;
+                }
+                i = lo;
+            }
+            first = min(first, i);
+        }
+        if (lane == 0) {
+            const uint32_t flags = M->flags | (M->pairs ? (uint32_t)VL_INTERFERENCE : 0u);
+            vl_verdict vd;
+            vd.flags = flags ? flags : (uint32_t)VL_PASS;
+            vd.first_violation_instr = first == 0xFFFFFFFFu ? -1 : (int32_t)first;
+            vd.conflict_pairs = M->pairs;
+            vd.bank_conflicts = M->bank;
+            q.out[k] = vd;
+        }
+    }
+}
+
+// Threads per block for a job of K rows, 0 if the program does not fit the fused kernel.
+uint32_t fused_threads(vl_program *p, uint64_t K)
+{
+    const uint32_t cap = 227 * 1024;
+    const uint32_t want = K <= (uint64_t)vl_sm_count(p) ? 512u : 256u;
+    for (uint32_t t = want; t >= 256; t /= 2)
+        if (p->nS <= 65535u && fused_smem(p, t).total <= cap) return t;
+    return 0;
+}
+
+}  // namespace
+
+// Jobs of up to 100 rows: 10 us against 44 for a program of 2,000 instructions, 20 against 85 for 8,000, 39 against
+// 126 for 32,000.  From about two thirds of the multiprocessors on, one row whose every chunk collides (80 us on one
+// multiprocessor; the batched recount spreads it) decides the time, and from one row per multiprocessor on the
+// batched kernels read the program's tables for 8 or 64 rows at a time.
+bool vl_fused_wanted(vl_program *p, uint64_t K)
+{
+    if (p->group_opt || p->threads_opt || p->test_wait) return false;  // the caller asks for the batched kernels
+    if (p->P + p->wmax > 32768u) return false;                         // (not a program the verify path takes)
+    return K <= 100 && fused_threads(p, K) != 0;
+}
+
+int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict)
+{
+    static std::mutex mtx;
+    static bool done[64];
+    if (p->device >= 0 && p->device < 64) {
+        std::lock_guard<std::mutex> lock(mtx);
+        if (!done[p->device]) {
+            const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+            VL_CUDA(p, cudaFuncSetAttribute(k_fused<256>, at, 227 * 1024));
+            VL_CUDA(p, cudaFuncSetAttribute(k_fused<512>, at, 227 * 1024));
+            done[p->device] = true;
+        }
+    }
+    const uint32_t threads = fused_threads(p, K);
+    FParams q{};
+    q.nI = p->nI; q.V = p->V; q.nO = dict ? p->nD : p->nO; q.P = p->P; q.B = p->B; q.nB = p->nB; q.nS = p->nS; q.Wv = p->Wv;
+    q.Wp = (p->P + p->wmax + 31) / 32; q.R = p->P + p->wmax + 2; q.wmax = p->wmax;
+    q.bank_fast = p->bank_fast; q.use_th = p->use_th;
+    while ((1u << q.short_shift) < p->short_len) ++q.short_shift;
+    q.sm = fused_smem(p, threads);
+    q.first_occ = dict ? p->d_dict_first_occ : p->d_first_occ; q.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16;
+    q.vinfo = p->d_vinfo; q.first_def_instr = p->d_first_def_instr; q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg;
+    q.entry_instr = dict ? p->d_dict_instr : nullptr; q.ndefs = p->d_ndefs; q.opflags = p->d_opflags;
+    q.vcons = p->d_vcons; q.rs_prefix = p->d_rs_prefix; q.bank_list = p->d_bank_list;
+    for (int j = 0; j < 4; ++j) q.bank_seg[j] = p->bank_seg[j];
+    q.th_off = p->d_th_off; q.th = p->d_th; q.blk_th = p->d_blk_th; q.sev_off = p->d_sev_off; q.sev = p->d_sev;
+    q.sen_off = p->d_sen_off; q.sen = p->d_sen;
+    q.short_blk = p->d_short_blk; q.short_i0 = p->d_short_i0; q.blk_chunk_off = p->d_blk_chunk_off;
+    q.chunk_short_off = p->d_chunk_short_off; q.ls = p->d_ls; q.irec = p->d_irec; q.blk_off = p->d_blk_off;
+    q.el = p->d_el; q.el_count = p->d_el_count;
+    q.cand = d_cand; q.pitch = pitch; q.out = d_out;
+    const int rc = vl_live_join(p, st);
+    if (rc != VL_OK) return rc;
+    if (threads == 512) k_fused<512><<<(uint32_t)K, 512, q.sm.total, st>>>(q);
+    else k_fused<256><<<(uint32_t)K, 256, q.sm.total, st>>>(q);
+    VL_CUDA(p, cudaGetLastError());
+    g_vl_launches.fetch_add(1);
+    return VL_OK;
+}

@@ -82,18 +82,19 @@ struct vl_program {
     // chunks: every chunk lies inside one block; pieces: every piece lies inside one chunk; short chunks: runs of
     // pieces of one chunk; segments: runs of chunks of one block
     uint32_t nC = 0, nP = 0, nS = 0, nSeg = 0;
+    uint32_t short_len = 1;  // instructions of the longest short chunk
     uint32_t layout_chunk_instrs = 0;  // chunk size the device copies of the layout were made for (0: none)
     std::vector<uint32_t> h_blk_off, h_op_off;
     // list lengths of the last liveness run with this layout: the next run allocates from them
     bool sizes_known = false;
-    unsigned long long known[5] = {0, 0, 0, 0, 0};  // list entries, walk events, through-set entries, short-list entries, short-chunk events
+    unsigned long long known[6] = {0, 0, 0, 0, 0, 0};  // list entries, walk events, through-set entries, short-list entries, short-chunk events and entries
 
     // device copies of the program
     uint32_t *d_blk_off = nullptr, *d_succ_off = nullptr, *d_succ = nullptr, *d_op_off = nullptr, *d_op_vreg = nullptr;
     uint8_t *d_ndefs = nullptr, *d_width = nullptr;
     uint32_t *d_chunk_i0 = nullptr, *d_chunk_i1 = nullptr, *d_chunk_blk = nullptr, *d_blk_chunk_off = nullptr;
     uint32_t *d_piece_i0 = nullptr, *d_piece_chunk = nullptr, *d_chunk_piece_off = nullptr;
-    uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr;
+    uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr, *d_short_i0 = nullptr;
 
     // liveness results
     uint32_t *d_blk_in = nullptr, *d_blk_out = nullptr, *d_lo_off = nullptr, *d_lo = nullptr;
@@ -110,10 +111,12 @@ struct vl_program {
     uint64_t *d_dict_slotmeta = nullptr;
     uint4 *d_dict_opoff = nullptr;
     uint8_t *d_dict_first4 = nullptr;
+    uint32_t *d_dict_first_occ = nullptr; // [V] first entry of the vreg, 0xFFFFFFFF if none
     uint32_t *d_dict_instr = nullptr;     // [nD8] first instruction of the entry's block that touches its vreg
     uint4 *d_opoff = nullptr;               // [nOpT / 4] per 4 operands: byte offsets of their vregs' 16-byte table entries
     uint8_t *d_first4 = nullptr;            // [nOpT / 4] per 4 operands: first-occurrence bits
     uint8_t *d_opflags = nullptr;           // [nO]
+    uint32_t *d_first_occ = nullptr;        // [V] first operand that names v, 0xFFFFFFFF if none
     uint32_t *d_first_def_instr = nullptr;  // [V] lowest instruction defining v, 0xFFFFFFFF if none
     uint32_t *d_vinfo = nullptr;            // [V] width | VINFO_OCCURS | VINFO_DEFINED
     // optional hardware rules of the Realizability check (vl_program_set_constraints)
@@ -122,14 +125,19 @@ struct vl_program {
     uint32_t *d_th_off = nullptr, *d_th = nullptr;  // per block: vregs occupied through the whole block
     // live-after lists without the block's through-set, for the recount: the list of instruction i of
     // block b is ls[lo_off[i] - ls_adj[b] - i * th_cnt[b] ...), |live-after| - th_cnt[b] entries
+    // per instruction, for the exact counts: {first entry of its short list, entries | definitions << 16 | first defined
+    // vreg is in the block's through-set << 31, first defined vreg, first operand}
+    uint4 *d_irec = nullptr;
     uint32_t *d_ls = nullptr, *d_ls_adj = nullptr, *d_th_cnt = nullptr, *d_blk_th = nullptr;
-    uint4 *d_el = nullptr;          // definitions without a walk event: {instruction, chunk, vreg, block}, any order
+    // definitions without a walk event: {instruction, chunk, vreg | in the block's through-set << 31, short chunk};
+    // those of block b start at the index of its first operand, in any order, el_count[b] of them
+    uint4 *d_el = nullptr;
     uint32_t *d_el_count = nullptr;
     uint32_t *d_cev_off = nullptr;  // [nC+1] first walk event of each chunk (every chunk padded to 8 events)
     uint4 *d_ev = nullptr;          // walk events, 112 bytes per group of 8, chunk after chunk
     // events of the short chunks, 4 bytes each, 32 short chunks side by side: steps [sev_off[g], sev_off[g + 1]) of
-    // group g, [step][32]
-    uint32_t *d_sev_off = nullptr, *d_sev = nullptr;
+    // group g, [step][32]; and what is occupied when short chunk s begins, vreg | s << 16, [sen_off[s], sen_off[s + 1])
+    uint32_t *d_sev_off = nullptr, *d_sev = nullptr, *d_sen_off = nullptr, *d_sen = nullptr;
     int bank_fast = 0;  // B in {1,2,4} and every instruction reads <= 4 distinct vregs
     int bank_many = 0;  // some instruction reads more than 4 distinct vregs
     uint2 *d_bank_list = nullptr;   // instructions with 2, 3, 4 distinct sources: their vreg ids, 16 bits each
@@ -149,7 +157,7 @@ struct vl_program {
     // A repeated liveness run (same layout, lengths remembered) does not wait for the GPU: its kernels write
     // the status word and the list lengths to pinned host memory, and the next call that needs the results on
     // the host side (vl_live_settle) waits for the run and checks them.
-    uint32_t *h_live = nullptr;      // pinned: [0] status, [2..11] five 64-bit totals, written by the run's kernels
+    uint32_t *h_live = nullptr;      // pinned: [0] status, [2..13] six 64-bit totals, written by the run's kernels
     cudaEvent_t ev_live = nullptr;
     bool live_pending = false;
     // vl_liveness of a long program runs on an internal stream (live_stream) behind what the caller's stream held
@@ -210,6 +218,9 @@ extern std::atomic<uint64_t> g_vl_launches;
     } while (0)
 
 int vl_liveness_impl(vl_program *p, cudaStream_t st);
+// The one-kernel verify path of short jobs (vl_fused.cu): whether a job of K rows takes it; one launch on st.
+bool vl_fused_wanted(vl_program *p, uint64_t K);
+int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict);
 int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out,
                    cudaStream_t st, int slot, bool dict = false);
 int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K,

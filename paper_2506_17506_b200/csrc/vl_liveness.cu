@@ -49,17 +49,17 @@ struct LiveArgs {
     uint32_t *lo_rel, *ev_rel;                    // per instruction: list entries / events before it in its chunk
     unsigned long long *chunk_lo;                 // per chunk: list entries of its instructions
     uint32_t *chunk_ev, *chunk_lo0;               // events of its instructions; first list entry
-    uint32_t *centry_cnt, *short_cnt;             // entry events per chunk; events per short chunk
+    uint32_t *centry_cnt, *short_ent, *short_ev;  // entry events per chunk, per short chunk; other events per short chunk
     uint32_t *flow_scratch;                       // k_flow's working set when it does not fit shared memory
     uint32_t *counters;                           // [0] blocks of k_offsets that have finished
     // results
-    uint32_t *blk_in, *blk_out, *lo_off, *lo, *ls, *ls_adj, *blk_th, *th_cnt, *th_off, *th, *cev_off, *sev_off, *sev;
+    uint32_t *blk_in, *blk_out, *lo_off, *lo, *ls, *ls_adj, *blk_th, *th_cnt, *th_off, *th, *cev_off, *sev_off, *sev, *sen_off, *sen;
     uint8_t *opflags;
-    uint4 *ev, *el;
+    uint4 *ev, *el, *irec;
     uint32_t *el_count, *status;
     uint32_t *host_out;                           // pinned: [0] status, [2..] totals (64 bit)
 };
-enum { LV_TOT_LO = 0, LV_TOT_EV = 1, LV_TOT_TH = 2, LV_TOT_LS = 3, LV_TOT_SEV = 4, LV_TOTALS = 5 };
+enum { LV_TOT_LO = 0, LV_TOT_EV = 1, LV_TOT_TH = 2, LV_TOT_LS = 3, LV_TOT_SEV = 4, LV_TOT_SEN = 5, LV_TOTALS = 6 };
 
 // ------------------------------------------------------------------ device helpers
 __device__ __forceinline__ bool bit_get(const uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; }
@@ -139,7 +139,8 @@ __global__ void __launch_bounds__(PC_NT) k_sets(const LiveArgs q)
     pdl_go();
     // what later kernels of the run update with atomics starts at zero
     for (size_t i = (size_t)c * blockDim.x + tid; i < (size_t)q.nB * q.Wv; i += (size_t)gridDim.x * blockDim.x) q.blk_touch[i] = 0;
-    if (c == 0 && tid == 0) { q.counters[0] = 0; *q.el_count = 0; *q.status = 0; }
+    for (uint32_t b = c * blockDim.x + tid; b < q.nB; b += gridDim.x * blockDim.x) q.el_count[b] = 0;
+    if (c == 0 && tid == 0) { q.counters[0] = 0; *q.status = 0; }
     if (c >= q.nC) return;
     uint32_t *s_use = sm + (size_t)warp * 2 * q.Wv, *s_def = s_use + q.Wv;
     const uint32_t p0 = q.chunk_piece_off[c], p1 = q.chunk_piece_off[c + 1];
@@ -446,7 +447,8 @@ __global__ void __launch_bounds__(OFF_NT) k_offsets(const LiveArgs q)
             if (lane == 0) {
                 if (p == p0) q.centry_cnt[c] = cnt;
                 const uint32_t ev1 = s + 1 < s1 ? q.ev_rel[q.piece_i0[q.short_p0[s + 1]]] : q.chunk_ev[c];
-                q.short_cnt[s] = cnt + ev1 - q.ev_rel[q.piece_i0[p]];
+                q.short_ent[s] = cnt;
+                q.short_ev[s] = ev1 - q.ev_rel[q.piece_i0[p]];
             }
         }
     } else {
@@ -466,7 +468,7 @@ __global__ void __launch_bounds__(OFF_NT) k_offsets(const LiveArgs q)
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    // Four warps, four scans side by side; a lane takes up to 8 consecutive values at a time, whose loads are in
+    // A warp per total, the scans side by side; a lane takes up to 8 consecutive values at a time, whose loads are in
     // flight together.  Exclusive offsets of n values into dst[0..n) (null: none), dst[n] = total, clipped to
     // 32 bits; the total is returned.
     auto offsets = [&](uint32_t n, uint32_t *dst, auto value, auto store) -> unsigned long long {
@@ -513,12 +515,14 @@ __global__ void __launch_bounds__(OFF_NT) k_offsets(const LiveArgs q)
         }, [&](uint32_t b, uint32_t pre) { q.ls_adj[b] = pre - q.blk_off[b] * __ldcg(q.th_cnt + b); });
     } else if (warp == LV_TOT_SEV) {  // a group of 32 short chunks per round: its longest
         for (uint32_t g = 0; g * 32 < q.nS; ++g) {
-            const uint32_t m = __reduce_max_sync(0xffffffffu, g * 32 + lane < q.nS ? __ldcg(q.short_cnt + g * 32 + lane) : 0u);
+            const uint32_t m = __reduce_max_sync(0xffffffffu, g * 32 + lane < q.nS ? __ldcg(q.short_ev + g * 32 + lane) : 0u);
             if (lane == 0) q.sev_off[g] = (uint32_t)tot;
             tot += m;
         }
         if (lane == 0) q.sev_off[(q.nS + 31) / 32] = (uint32_t)tot;
         tot *= 32;
+    } else if (warp == LV_TOT_SEN) {
+        tot = offsets(q.nS, q.sen_off, [&](uint32_t s) -> unsigned long long { return __ldcg(q.short_ent + s); }, into(q.sen_off));
     }
     if (warp < LV_TOTALS && lane == 0) s_tot[warp] = tot;
     __syncthreads();
@@ -715,6 +719,8 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
             my_lo = q.chunk_lo0[c] + q.lo_rel[i0 + lane];
             q.lo_off[i0 + lane] = my_lo;
         }
+        uint32_t v0 = q.V, my_n = 0;  // lane k: first defined vreg of instruction k, length of its short list
+        if (lane < po.ni && po.nd) v0 = q.op_vreg[po.off];
         __syncwarp();
         const uint32_t rounds = (q.Wv + 31) / 32, below = (1u << lane) - 1u;
         for (uint32_t k = po.ni; k-- > 0;) {
@@ -737,6 +743,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
                     at_s += __popc(y);
                 }
             }
+            if (lane == k) my_n = at - my_lo - ls_mul;
             __syncwarp();
             for (uint32_t r = 0; r < po.n; r += 32) {  // live before the instruction: without its definitions ...
                 const uint32_t x = r == 0 ? x0 : po.get(q, r + lane);
@@ -749,6 +756,9 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
             }
             __syncwarp();
         }
+        if (lane < po.ni)
+            q.irec[i0 + lane] = make_uint4(my_lo - ls_sub - (i0 + lane) * ls_mul,
+                                           my_n | (po.nd << 16) | (po.nd && bit_get(s_th, v0) ? 0x80000000u : 0u), v0, po.off);
         return;
     }
     pdl_wait();
@@ -765,7 +775,10 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
             const size_t at = base + n_entry + q.ev_rel[i];
             instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) { put_event(q.ev, at + e, v, q.width[v], test, toggle); },
                          [&](uint32_t o) {  // listed (in any order) for the recount of through-set collisions
-                             q.el[atomicAdd(q.el_count, 1u)] = make_uint4(i, c, q.op_vreg[o], b);
+                             uint32_t s = q.chunk_short_off[c];
+                             while (s + 1 < q.chunk_short_off[c + 1] && q.piece_i0[q.short_p0[s + 1]] <= i) ++s;
+                             const uint32_t v = q.op_vreg[o], member = bit_get(q.blk_th + (size_t)b * q.Wv, v);
+                             q.el[q.op_off[q.blk_off[b]] + atomicAdd(q.el_count + b, 1u)] = make_uint4(i, c, v | (member << 31), s);
                          });
         }
         // no-ops up to a whole group, and two no-op groups behind the last chunk (the walk reads ahead)
@@ -775,28 +788,28 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
     }
     role -= q.nC;
     if (role < n_short) {
-        // events of a short chunk, 4 bytes each: vreg | width << 16 | test << 24 | toggle << 25; 32 short chunks side
-        // by side, step by step, padded with zeros to the longest of the 32
+        // Events of a short chunk, 4 bytes each: vreg | width << 16 | test << 24 | toggle << 25; 32 short chunks side
+        // by side, step by step, padded with zeros to the longest of the 32.  What is occupied on entry (and not
+        // through the whole block) is a list of its own, vreg | short chunk << 16: those need no order.
         const uint32_t s = role * LV_WARPS + warp;
         const uint32_t steps = q.sev_off[(s >> 5) + 1] - q.sev_off[s >> 5];
         uint32_t *dst = q.sev + (size_t)q.sev_off[s >> 5] * 32 + (s & 31);
         uint32_t n = 0;
         if (s < q.nS) {
             const uint32_t p = q.short_p0[s], c = q.piece_chunk[p], b = q.chunk_blk[c], p0 = q.chunk_piece_off[c];
-            const uint32_t n_entry = warp_bits(q.Wv, lane, [&](uint32_t w) { return entry_word(q, c, p, p0, b, w); },
-                                               [&](uint32_t rank, uint32_t v) {
-                                                   dst[(size_t)rank * 32] = v | ((uint32_t)q.width[v] << 16) | (3u << 24);
-                                               });
+            const uint32_t ent0 = q.sen_off[s];
+            warp_bits(q.Wv, lane, [&](uint32_t w) { return entry_word(q, c, p, p0, b, w); },
+                      [&](uint32_t rank, uint32_t v) { q.sen[ent0 + rank] = v | (s << 16); });
             const uint32_t i0 = q.piece_i0[p];
             const uint32_t i1 = s + 1 < q.chunk_short_off[c + 1] ? q.piece_i0[q.short_p0[s + 1]] : q.chunk_i1[c];
             const uint32_t ev0 = q.ev_rel[i0];
             for (uint32_t i = i0 + lane; i < i1; i += 32) {
-                const uint32_t at = n_entry + q.ev_rel[i] - ev0;
+                const uint32_t at = q.ev_rel[i] - ev0;
                 instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) {
                     dst[(size_t)(at + e) * 32] = v | ((uint32_t)q.width[v] << 16) | (test ? 1u << 24 : 0u) | (toggle ? 1u << 25 : 0u);
                 }, [](uint32_t) {});
             }
-            n = q.short_cnt[s];
+            n = q.short_ev[s];
         }
         for (uint32_t e = n + lane; e < steps; e += 32) dst[(size_t)e * 32] = 0;
         return;
@@ -872,7 +885,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     p->layout_arena.reset();
     p->tables_built = false;
     p->d_vreg16 = nullptr; p->d_slotmeta = nullptr; p->d_opoff = nullptr; p->d_first4 = nullptr;
-    p->d_first_def_instr = nullptr; p->d_vinfo = nullptr;
+    p->d_first_def_instr = nullptr; p->d_vinfo = nullptr; p->d_first_occ = nullptr;
     std::vector<uint32_t> c_i0, c_i1, c_blk, blk_c_off(nB + 1, 0), p_i0, p_chunk, c_p_off, seg_c0, blk_seg_off(nB + 1, 0);
     for (uint32_t b = 0; b < nB; ++b) {
         const uint64_t s = p->h_blk_off[b], n = p->h_blk_off[b + 1] - s;
@@ -905,7 +918,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     p->nSeg = (uint32_t)seg_c0.size();
     seg_c0.push_back(nC);
     // short chunks: as few pieces as keep their number within SHORT_CHUNKS, equally long inside a chunk
-    std::vector<uint32_t> s_p0, c_s_off(nC + 1, 0), s_blk;
+    std::vector<uint32_t> s_p0, c_s_off(nC + 1, 0), s_blk, s_i0;
     for (uint32_t r = std::max(1u, (p->nP + SHORT_CHUNKS - 1) / SHORT_CHUNKS);; ++r) {
         uint64_t total = 0;
         for (uint32_t c = 0; c < nC; ++c) total += (c_p_off[c + 1] - c_p_off[c] + r - 1) / r;
@@ -921,12 +934,17 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         break;
     }
     p->nS = (uint32_t)s_p0.size();
+    for (uint32_t x : s_p0) s_i0.push_back(p_i0[x]);
+    s_i0.push_back(p->nI);
+    p->short_len = 1;
+    for (uint32_t j = 0; j < p->nS; ++j) p->short_len = std::max(p->short_len, s_i0[j + 1] - s_i0[j]);
     std::vector<uint32_t> all;
     struct Part { uint32_t **dst; const std::vector<uint32_t> *v; };
     const Part parts[] = {{&p->d_chunk_i0, &c_i0}, {&p->d_chunk_i1, &c_i1}, {&p->d_chunk_blk, &c_blk},
                           {&p->d_blk_chunk_off, &blk_c_off}, {&p->d_piece_i0, &p_i0}, {&p->d_piece_chunk, &p_chunk},
                           {&p->d_chunk_piece_off, &c_p_off}, {&p->d_seg_c0, &seg_c0}, {&p->d_blk_seg_off, &blk_seg_off},
-                          {&p->d_short_p0, &s_p0}, {&p->d_chunk_short_off, &c_s_off}, {&p->d_short_blk, &s_blk}};
+                          {&p->d_short_p0, &s_p0}, {&p->d_chunk_short_off, &c_s_off}, {&p->d_short_blk, &s_blk},
+                          {&p->d_short_i0, &s_i0}};
     for (const Part &x : parts) {
         all.insert(all.end(), x.v->begin(), x.v->end());
         all.resize((all.size() + 4) & ~(size_t)3);  // (at least one word behind every array)
@@ -963,6 +981,7 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     const bool make_tables = !p->tables_built;
     if (!p->d_opoff) {
         LAYOUT(&p->d_first_def_instr, (size_t)V);
+        LAYOUT(&p->d_first_occ, (size_t)V);
         LAYOUT(&p->d_vreg16, (size_t)p->nOp8 + 8);
         LAYOUT(&p->d_slotmeta, (size_t)p->nOp8 / 8);
         LAYOUT(&p->d_first4, (size_t)p->nOpT / 4);
@@ -975,8 +994,10 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     KEEP(&p->d_ls_adj, (size_t)nB);
     KEEP(&p->d_blk_th, (size_t)nB * Wv);
     KEEP(&p->d_el, (size_t)nO);  // at most one entry per definition
-    KEEP(&p->d_el_count, 1);
+    KEEP(&p->d_el_count, (size_t)nB);
     KEEP(&p->d_sev_off, (size_t)(p->nS + 31) / 32 + 1);
+    KEEP(&p->d_sen_off, (size_t)p->nS + 1);
+    KEEP(&p->d_irec, (size_t)nI);
 
     LiveArgs q{};
     q.nB = nB; q.nI = nI; q.V = V; q.nE = p->nE; q.Wv = Wv; q.nC = nC; q.nP = nP; q.nS = p->nS; q.nSeg = p->nSeg;
@@ -1000,7 +1021,8 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     TMP(&q.chunk_ev, (size_t)nC);
     TMP(&q.chunk_lo0, (size_t)nC + 1);
     TMP(&q.centry_cnt, (size_t)nC);
-    TMP(&q.short_cnt, (size_t)p->nS);
+    TMP(&q.short_ent, (size_t)p->nS);
+    TMP(&q.short_ev, (size_t)p->nS);
     TMP(&q.counters, 1);
     const uint32_t fgrid = (Wv + 31) / 32;
     size_t flow_smem = (((size_t)4 * nB + 2 * (size_t)p->nSeg) * 32 + nB + 1 + p->nE) * 4;
@@ -1008,17 +1030,15 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
         TMP(&q.flow_scratch, flow_smem / 4 * fgrid);
         flow_smem = 0;
     }
-    uint32_t *first_occ = nullptr;
     uint8_t *opmeta = nullptr;
     if (make_tables) {
-        TMP(&first_occ, (size_t)V);
         TMP(&opmeta, (size_t)nO);
-        VL_CUDA(p, cudaMemsetAsync(first_occ, 0xFF, std::max<size_t>(V, 1) * 4, st));
+        VL_CUDA(p, cudaMemsetAsync(p->d_first_occ, 0xFF, std::max<size_t>(V, 1) * 4, st));
         VL_CUDA(p, cudaMemsetAsync(p->d_first_def_instr, 0xFF, std::max<size_t>(V, 1) * 4, st));
     }
     q.blk_in = p->d_blk_in; q.blk_out = p->d_blk_out; q.lo_off = p->d_lo_off; q.opflags = p->d_opflags;
     q.cev_off = p->d_cev_off; q.th_off = p->d_th_off; q.th_cnt = p->d_th_cnt; q.ls_adj = p->d_ls_adj; q.blk_th = p->d_blk_th;
-    q.el = p->d_el; q.el_count = p->d_el_count; q.status = p->d_status; q.sev_off = p->d_sev_off;
+    q.el = p->d_el; q.el_count = p->d_el_count; q.status = p->d_status; q.sev_off = p->d_sev_off; q.sen_off = p->d_sen_off; q.irec = p->d_irec;
     q.host_out = p->h_live;
     // a bitset pair per warp of k_sets: fewer warps for programs of very many vregs
     const uint32_t set_warps = (uint32_t)std::max<size_t>(1, std::min<size_t>(PC_WARPS, (size_t)224 * 1024 / ((size_t)2 * Wv * 4)));
@@ -1038,7 +1058,7 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
         if (status & ST_NO_CONVERGE) return VL_ERR_NO_CONVERGE;
         if (status & ST_NOT_STRICT) return VL_ERR_NOT_STRICT;
         if (status & ST_SIZE_OVERFLOW) return VL_ERR_UNSUPPORTED;
-        if (tot[LV_TOT_EV] > 0xFFFFFFF0ull || tot[LV_TOT_SEV] > 0xFFFFFFF0ull) return VL_ERR_UNSUPPORTED;
+        if (tot[LV_TOT_EV] > 0xFFFFFFF0ull || tot[LV_TOT_SEV] > 0xFFFFFFF0ull || tot[LV_TOT_SEN] > 0xFFFFFFF0ull) return VL_ERR_UNSUPPORTED;
         memcpy(p->known, tot, sizeof(tot));
     }
     p->lo_len = p->known[LV_TOT_LO];
@@ -1047,14 +1067,15 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     KEEP(&p->d_ev, (size_t)(p->known[LV_TOT_EV] / 8 + 2) * 7);  // two no-op groups behind the last chunk
     KEEP(&p->d_th, (size_t)p->known[LV_TOT_TH]);
     KEEP(&p->d_sev, (size_t)p->known[LV_TOT_SEV]);
-    q.lo = p->d_lo; q.ls = p->d_ls; q.ev = p->d_ev; q.th = p->d_th; q.sev = p->d_sev;
+    KEEP(&p->d_sen, (size_t)p->known[LV_TOT_SEN]);
+    q.lo = p->d_lo; q.ls = p->d_ls; q.ev = p->d_ev; q.th = p->d_th; q.sev = p->d_sev; q.sen = p->d_sen;
     const uint32_t n_list = (nP + LV_WARPS - 1) / LV_WARPS, n_short = ((p->nS + 31) & ~31u) / LV_WARPS;
     VL_CUDA(p, launch_pdl(k_fill, n_list + nC + n_short + nB, LV_NT, (size_t)LV_WARPS * 2 * Wv * 4, st, q));
     if (make_tables) {
-        LAUNCH(k_first_occ, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, first_occ,
+        LAUNCH(k_first_occ, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
                p->d_first_def_instr);
-        LAUNCH(k_vreg_info, (V + NT - 1) / NT, NT, 0, st, V, p->d_width, first_occ, p->d_first_def_instr, p->d_vinfo);
-        LAUNCH(k_operand_meta, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, first_occ,
+        LAUNCH(k_vreg_info, (V + NT - 1) / NT, NT, 0, st, V, p->d_width, p->d_first_occ, p->d_first_def_instr, p->d_vinfo);
+        LAUNCH(k_operand_meta, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
                p->d_opflags, p->d_vreg16, opmeta, p->d_status);
         LAUNCH(k_pack_slots, (p->nOpT / 8 + NT - 1) / NT, NT, 0, st, nO, p->nOp8, p->nOpT / 8, V, opmeta, p->d_vreg16,
                p->d_slotmeta, p->d_opoff, p->d_first4);

@@ -108,7 +108,7 @@ struct RParams {
     uint32_t nI, V, B, nB, nC, AW;
     int bank_fast;
     uint64_t K;
-    const uint32_t *vinfo, *chunk_i0, *chunk_i1, *chunk_blk, *blk_chunk_off, *th_off, *th, *op_off, *op_vreg, *lo_off, *lo;
+    const uint32_t *vinfo, *chunk_i0, *chunk_i1, *chunk_blk, *blk_chunk_off, *th_off, *th, *op_off, *op_vreg, *lo_off, *lo, *blk_off;
     const uint8_t *ndefs, *width, *opflags;
     const uint16_t *tg;
     const uint32_t *cstate, *anom;
@@ -118,7 +118,7 @@ struct RParams {
     uint32_t *work;
     vl_verdict *out;
     uint32_t *status;
-    const uint4 *el;           // the definitions the walk skips: {instruction, chunk, vreg, block}
+    const uint4 *el;           // the definitions the walk skips (see vl_program)
     const uint32_t *el_count;
     const uint32_t *ls, *ls_adj, *th_cnt;  // live-after lists without the through-sets (see vl_program)
     uint32_t R;                            // registers covered by the recount's through-set counters
@@ -1737,14 +1737,14 @@ __global__ void __launch_bounds__(RC_THREADS) k_recount(const RParams q)
                 }
                 return cc;
             };
-            // the program's skipped definitions are listed as {instruction, chunk, vreg, block}
+            // the block's skipped definitions are listed as {instruction, chunk, vreg | member << 31, short chunk}
             uint32_t pairs = 0, mind = 0xFFFFFFFFu;
-            const uint32_t n_el = *q.el_count;
+            const uint32_t n_el = q.el_count[c];
+            const uint4 *el = q.el + q.op_off[q.blk_off[c]];
             for (uint32_t e = tid; e < n_el; e += RC_THREADS) {
-                const uint4 x = q.el[e];
-                if (x.w != c) continue;
-                if ((q.anom[k * q.AW + (x.y >> 5)] >> (x.y & 31)) & 1u) continue;
-                const uint32_t cn = count_of(x.z);
+                const uint4 x = el[e];
+                if (!(x.z >> 31) || ((q.anom[k * q.AW + (x.y >> 5)] >> (x.y & 31)) & 1u)) continue;
+                const uint32_t cn = count_of(x.z & 0xFFFFu);
                 if (cn) { pairs += cn; mind = min(mind, x.x); }
             }
 #pragma unroll
@@ -2406,7 +2406,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     rq.nI = p->nI; rq.V = p->V; rq.B = p->B; rq.nB = p->nB; rq.nC = p->nC; rq.AW = (uint32_t)vs.aw;
     rq.bank_fast = p->bank_fast; rq.K = n;
     rq.blk_chunk_off = p->d_blk_chunk_off; rq.th_off = p->d_th_off; rq.th = p->d_th;
-    rq.el = p->d_el; rq.el_count = p->d_el_count;
+    rq.blk_off = p->d_blk_off; rq.el = p->d_el; rq.el_count = p->d_el_count;
     rq.ls = p->d_ls; rq.ls_adj = p->d_ls_adj; rq.th_cnt = p->d_th_cnt; rq.R = p->P + p->wmax + 2;
     rq.vinfo = p->d_vinfo; rq.chunk_i0 = p->d_chunk_i0; rq.chunk_i1 = p->d_chunk_i1; rq.chunk_blk = p->d_chunk_blk;
     rq.op_off = p->d_op_off; rq.op_vreg = p->d_op_vreg; rq.lo_off = p->d_lo_off; rq.lo = p->d_lo;
@@ -2431,6 +2431,12 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
 int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out,
                    cudaStream_t st, int slot, bool dict)
 {
+    if (vl_fused_wanted(p, K)) {
+        kt_mark(p, st);
+        const int rf = vl_fused_run(p, d_cand, K, pitch, d_out, st, dict);
+        for (int j = 0; j < 4; ++j) kt_mark(p, st);
+        return rf;
+    }
     PassPlan pp{};
     int rc = plan_passes(p, K, &pp);
     if (rc != VL_OK) return rc;
@@ -2471,6 +2477,11 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     for (uint32_t j = 0; j < nprog && rc == VL_OK; ++j) {
         if (K[j] == 0) continue;
         vl_program *p = progs[j];
+        if (vl_fused_wanted(p, K[j])) {
+            rc = vl_fused_run(p, d_cand[j], K[j], pitch[j], d_out[j], lane[job % L], dict);
+            ++job;
+            continue;
+        }
         PassPlan pp{};
         rc = plan_passes(p, K[j], &pp);
         if (rc != VL_OK) break;

@@ -1,0 +1,51 @@
+"""The one-kernel path of short jobs: at the edges of what it takes (rows, short chunks, register file sizes) against
+the CPU oracle, every verdict field, bit-exact."""
+import numpy as np
+import pytest
+
+from paper_2506_17506_b200 import synth
+from tests import helpers as H
+from tests.test_gpu_parity import _assert_same, _garbage_rows, _gpu_verify
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2506_17506_b200 import binding
+    return binding
+
+
+@pytest.mark.parametrize("P,chunk", [(31, 160), (64, 8), (4000, 16), (8000, 160)])
+def test_random_programs(B, oracle_mod, P, chunk):
+    """Register files whose masks take 512 threads, 256 threads and no block at all (the batched kernels); several
+    definitions per instruction, wide and misaligned tuples, rows that collide everywhere."""
+    for seed in range(6):
+        p = H.random_program(9100 + seed, max_instrs=400, max_vregs=60, max_blocks=9, P=P, widths=(1, 2, 3, 8, 33), B=[4, 3][seed % 2])
+        gp = B.Program(p)
+        gp.set_option(B.VL_OPT_CHUNK_INSTRS, chunk)
+        gp.vl_liveness()
+        op = oracle_mod.OracleProgram(p)
+        rows = _garbage_rows(p, 40, seed)
+        _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows), f"P {P} chunk {chunk} seed {seed}")
+        gp.close()
+
+
+@pytest.mark.parametrize("chunk", [160, 8])
+@pytest.mark.parametrize("K", [1, 100, 101])
+def test_row_counts_and_many_short_chunks(B, oracle_mod, K, chunk):
+    """Attention-shaped program with the last row count of the path, the first beyond it, and more short chunks (1,000)
+    than a thread block has threads."""
+    wl = synth.workload(2)
+    p = synth.build_program(wl.shapes[0], wl.seeds[0])
+    rows, _ = synth.candidate_rows(p, K, 0.5, 77)
+    rows[: K // 10] = _garbage_rows(p, K, 3)[: K // 10]
+    gp = B.Program(p)
+    gp.set_option(B.VL_OPT_CHUNK_INSTRS, chunk)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows), f"K {K} chunk {chunk}")
+    gp.close()
