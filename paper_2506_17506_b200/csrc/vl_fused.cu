@@ -22,6 +22,7 @@ namespace {
 struct FMisc {
     uint32_t flags, minop, minr, bank, pairs, mind, thcol, any;
     uint32_t n_list;
+    uint32_t th_off[33];  // (through-sets are used only by programs of at most 32 blocks)
 };
 
 // Where the parts of a block's shared memory start (bytes), and how much there is.
@@ -46,7 +47,7 @@ inline FSmem fused_smem(const vl_program *p, uint32_t threads)
 }
 
 struct FParams {
-    uint32_t nI, V, nO, P, B, nB, nS, Wp, R, Wv, wmax, short_shift;
+    uint32_t nI, V, nO, P, B, nB, nS, Wp, R, Wv, wmax, short_len;
     int bank_fast, use_th;
     FSmem sm;
     const uint32_t *first_occ, *vinfo, *first_def_instr, *op_off, *op_vreg, *entry_instr, *blk_off;
@@ -58,7 +59,7 @@ struct FParams {
     const uint2 *bank_list;
     uint32_t bank_seg[4];
     // liveness results
-    const uint32_t *th_off, *th, *blk_th, *sev_off, *sev, *sen_off, *sen, *short_blk, *short_i0, *blk_chunk_off, *chunk_short_off;
+    const uint32_t *th_off, *th, *blk_th, *sev_off, *sev, *sen_off, *sen, *short_blk, *short_i0, *blk_short_off;
     const uint32_t *ls, *el_count;
     const uint4 *el, *irec;
     const uint16_t *cand;
@@ -107,22 +108,28 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
     const uint64_t k = blockIdx.x;
     const uint16_t *row = q.cand + k * q.pitch;
 
-    if (tid == 0) *M = FMisc{0u, 0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u, 0xFFFFFFFFu, 0u, 0u, 0u};
+    if (tid == 0) {
+        M->flags = M->bank = M->pairs = M->thcol = M->any = 0;
+        M->minop = M->minr = M->mind = 0xFFFFFFFFu;
+    }
+    if (tid <= 32) M->th_off[tid] = q.use_th ? q.th_off[min(tid, q.nB)] : 0u;
     if (q.use_th)
         for (uint32_t j = tid; j < q.nB * q.Wp; j += NTHR) s_th[j] = 0;
     __syncthreads();
 
     // Every phase keeps several loads per thread in flight and asks for its first ones before the phase in front of
-    // it computes: with one candidate per block the time is a chain of L2 round trips, not work.
+    // it computes: with one candidate per block the time is a chain of L2 round trips, not work.  Loads past the end
+    // of a list take a clamped index and are dropped afterwards: a load under a condition of its own per thread is
+    // waited for before the next one is issued.
     constexpr int CU = 3;  // column loads (8 columns each) in flight
     uint4 r_nx[CU], v_nx[CU];
+    const uint32_t o_last = q.nO ? (q.nO - 1) & ~7u : 0u;
     auto fetch_columns = [&](uint32_t o0) {
 #pragma unroll
         for (int u = 0; u < CU; ++u) {
-            const uint32_t o = o0 + u * NTHR * 8;
-            const bool ok = o < q.nO;
-            r_nx[u] = ok ? *reinterpret_cast<const uint4 *>(row + o) : make_uint4(0, 0, 0, 0);
-            v_nx[u] = ok ? *reinterpret_cast<const uint4 *>(q.vreg16 + o) : make_uint4(0, 0, 0, 0);
+            const uint32_t o = min(o0 + u * NTHR * 8, o_last);
+            r_nx[u] = *reinterpret_cast<const uint4 *>(row + o);
+            v_nx[u] = *reinterpret_cast<const uint4 *>(q.vreg16 + o);
         }
     };
     // ---- 1. the table, eight vregs per thread in flight
@@ -130,12 +137,15 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
         uint32_t pos[8], vi[8], t[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const bool ok = v0 + u * NTHR < q.V;
-            pos[u] = ok ? q.first_occ[v0 + u * NTHR] : 0xFFFFFFFFu;
-            vi[u] = ok ? q.vinfo[v0 + u * NTHR] : 0u;
+            const uint32_t v = min(v0 + u * NTHR, q.V - 1);
+            pos[u] = q.first_occ[v];
+            vi[u] = q.vinfo[v];
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) t[u] = pos[u] != 0xFFFFFFFFu ? row[pos[u]] : 0u;
+        for (int u = 0; u < 8; ++u) {
+            t[u] = row[pos[u] != 0xFFFFFFFFu ? pos[u] : 0u];
+            if (pos[u] == 0xFFFFFFFFu) t[u] = 0;
+        }
         if (v0 + 8 * NTHR >= q.V) fetch_columns(tid * 8);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -164,10 +174,10 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
     // ---- 2. Consistency: 8 columns per load
     constexpr int BU = 6;  // bank list entries in flight
     uint2 id_nx[BU];
-    const uint32_t n_ent = q.bank_fast ? q.bank_seg[3] : 0u;
+    const uint32_t n_ent = q.bank_fast ? q.bank_seg[3] : 0u, ent_last = n_ent ? n_ent - 1 : 0u;
     auto fetch_bank = [&](uint32_t e0) {
 #pragma unroll
-        for (int u = 0; u < BU; ++u) id_nx[u] = e0 + u * NTHR < n_ent ? q.bank_list[e0 + u * NTHR] : make_uint2(0, 0);
+        for (int u = 0; u < BU; ++u) id_nx[u] = q.bank_list[min(e0 + u * NTHR, ent_last)];
     };
     for (uint32_t o0 = tid * 8; o0 < q.nO; o0 += CU * NTHR * 8) {
         uint4 r4[CU], v4[CU];
@@ -234,11 +244,11 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
 
     // ---- 4. Safety
     if (q.use_th) {
-        const uint32_t n_th = q.th_off[q.nB];
+        const uint32_t n_th = M->th_off[q.nB];
         for (uint32_t e = tid; e < n_th; e += NTHR) {
             const uint32_t x = q.th[e];
             uint32_t b = 0;
-            while (b + 1 < q.nB && q.th_off[b + 1] <= e) ++b;  // (at most 32 blocks, the offsets sit in L1)
+            while (b + 1 < q.nB && M->th_off[b + 1] <= e) ++b;
             uint32_t pos = min((uint32_t)T[x & 0xFFFFu], q.P), left = x >> 16;
             bool hit = false;
             while (left) {
@@ -258,14 +268,15 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
         const bool mine = s < nSr;
         const uint32_t st0 = mine ? q.sev_off[s >> 5] : 0u, steps = mine ? q.sev_off[(s >> 5) + 1] - st0 : 0u;
         const uint32_t *ev = q.sev + (size_t)st0 * 32 + lane;
+        const uint32_t step_last = steps ? steps - 1 : 0u;
         constexpr int EU = 8;  // events in flight: loaded ahead, and applied
         uint32_t nx[EU];
 #pragma unroll
-        for (int u = 0; u < EU; ++u) nx[u] = u < steps ? ev[u * 32] : 0u;
+        for (int u = 0; u < EU; ++u) nx[u] = ev[(size_t)min((uint32_t)u, step_last) * 32];
         uint32_t en[4];
-        const uint32_t e_hi = q.sen_off[min(q.nS, s0 + NTHR)], e_lo = q.sen_off[s0];
+        const uint32_t e_hi = q.sen_off[min(q.nS, s0 + NTHR)], e_lo = q.sen_off[s0], e_end = max(e_hi, 1u) - 1;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) en[u] = e_lo + tid + u * NTHR < e_hi ? q.sen[e_lo + tid + u * NTHR] : 0u;
+        for (int u = 0; u < 4; ++u) en[u] = q.sen[min(e_lo + tid + u * NTHR, e_end)];
         const uint32_t b = s < q.nS && q.use_th ? q.short_blk[s] : 0u;
         for (uint32_t wd = 0; wd < q.Wp; ++wd) occ[wd * NTHR + tid] = q.use_th ? s_th[b * q.Wp + wd] : 0u;
         if (mine && lane == 0) coll[s >> 5] = 0;
@@ -275,8 +286,7 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 x[u] = en[u];
-                const uint32_t e = e0 + (4 + u) * NTHR;
-                en[u] = e < e_hi ? q.sen[e] : 0u;
+                en[u] = q.sen[min(e0 + (4 + u) * NTHR, e_end)];
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -301,10 +311,10 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
             uint32_t far = 0;  // some range of the batch reaches into the next word
 #pragma unroll
             for (int u = 0; u < EU; ++u) {
-                x[u] = nx[u];
+                x[u] = e0 + u < steps ? nx[u] : 0u;
                 t[u] = min((uint32_t)T[x[u] & 0xFFFFu], q.P);
                 far |= (t[u] & 31) + ((x[u] >> 16) & 0xFFu) > 32 ? 1u : 0u;
-                nx[u] = e0 + EU + u < steps ? ev[(size_t)(e0 + EU + u) * 32] : 0u;
+                nx[u] = ev[(size_t)min(e0 + EU + u, step_last) * 32];
             }
             // toggling returns the old word: occupied and released are both a toggle as long as no collision
             // has been seen (after one, the chunk is counted exactly anyway)
@@ -349,22 +359,24 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
     if (M->any | M->thcol) {
         uint32_t *cover = occ, *start = occ + q.R;
         uint32_t pairs = 0, mind = 0xFFFFFFFFu;
+        uint32_t s_hi = 0, s_next = q.blk_short_off[1];
         for (uint32_t b = 0; b < q.nB; ++b) {
-            const uint32_t s_lo = q.chunk_short_off[q.blk_chunk_off[b]], s_hi = q.chunk_short_off[q.blk_chunk_off[b + 1]];
+            const uint32_t s_lo = s_hi;
+            s_hi = s_next;
+            s_next = q.blk_short_off[min(b + 2, q.nB)];
             const bool thcol = q.use_th && ((M->thcol >> b) & 1u);
+            bool any = false;
+            for (uint32_t s = s_lo + tid; s < s_hi; s += NTHR) any |= (coll[s >> 5] >> (s & 31)) & 1u;
+            if (!__syncthreads_or(any) && !thcol) continue;
             if (tid == 0) M->n_list = 0;
             __syncthreads();
             for (uint32_t s = s_lo + tid; s < s_hi; s += NTHR)
                 if ((coll[s >> 5] >> (s & 31)) & 1u) list[atomicAdd(&M->n_list, 1u)] = make_uint2(q.short_i0[s], q.short_i0[s + 1]);
-            __syncthreads();
-            const uint32_t n_list = M->n_list;
-            __syncthreads();
-            if (!n_list && !thcol) continue;
             // The block's through-set, counted into two arrays over the registers (cover[r]: members whose range holds
             // r, start[r]: members whose range starts at r): a range [s, s+w) overlaps cover[s] + start[s+1] + ... +
             // start[s+w-1] of them.  Members that reach beyond the arrays lie beyond the file: they are compared
             // one by one, with definitions that lie there too.
-            const uint32_t t0 = q.th_off[b], n_th = q.th_off[b + 1] - t0;
+            const uint32_t t0 = q.use_th ? M->th_off[b] : 0u, n_th = q.use_th ? M->th_off[b + 1] - t0 : 0u;
             for (uint32_t r = tid; r < 2 * q.R; r += NTHR) occ[r] = 0;
             __syncthreads();
             for (uint32_t j = tid; j < n_th; j += NTHR) {
@@ -375,45 +387,53 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
                 }
             }
             __syncthreads();
-            // through-set members other than v (itself a member: `member`) that overlap v's range; part `sub` of `of`
-            auto through_overlaps = [&](uint32_t v, bool member, uint32_t sub, uint32_t of) {
+            const uint32_t n_list = M->n_list;
+            // through-set members other than v (itself a member: `member`) that overlap v's range
+            auto through_overlaps = [&](uint32_t v, bool member) {
                 const uint32_t s = T[v], w = W[v];
                 uint32_t n = 0;
                 if (s < q.R) {
-                    if (sub == 0) n = cover[s] - (member && s + w <= q.R ? 1u : 0u);
-                    for (uint32_t r = s + 1 + sub; r < min(s + w, q.R); r += of) n += start[r];
+                    n = cover[s] - (member && s + w <= q.R ? 1u : 0u);
+                    for (uint32_t r = s + 1; r < min(s + w, q.R); ++r) n += start[r];
                 }
                 if (s + w > q.P)
-                    for (uint32_t j = sub; j < n_th; j += of) {
+                    for (uint32_t j = 0; j < n_th; ++j) {
                         const uint32_t u = q.th[t0 + j] & 0xFFFFu;
                         if (u != v && T[u] + W[u] > q.R && overlap(s, w, T[u], W[u])) ++n;
                     }
                 return n;
             };
             auto is_member = [&](uint32_t v) { return ((q.blk_th[(size_t)b * q.Wv + (v >> 5)] >> (v & 31)) & 1u) != 0; };
-            // Two lanes take an instruction: the entries of its live-after list that are not in the through-set, the
-            // through-set from the arrays.  The record of the instruction after the next and the list entries of
-            // the next are fetched meanwhile.  The width of an entry is read only if its register is near enough.
-            constexpr uint32_t NG = NTHR / 2;
-            constexpr int LU = 12;  // list entries per lane in flight
-            const uint32_t sub = tid & 1u, n_slots = n_list << q.short_shift, len_mask = (1u << q.short_shift) - 1u;
-            auto instr_of = [&](uint32_t f) -> uint32_t {  // 0xFFFFFFFF: beyond the short chunk, or beyond the list
-                if (f >= n_slots) return 0xFFFFFFFFu;
-                const uint2 span = list[f >> q.short_shift];
-                const uint32_t i = span.x + (f & len_mask);
-                return i < span.y ? i : 0xFFFFFFFFu;
+            // A thread takes an instruction: the entries of its live-after list that are not in the through-set, the
+            // through-set from the arrays.  The record of the instruction after the next and the first list entries
+            // of the next are fetched meanwhile.  (Bound by instruction issue: the lists of loop bodies hold 4 to 10
+            // entries, and few of them sit near enough to be looked at more closely.)
+            constexpr int LU = 8;  // list entries in flight
+            const uint32_t step_unit = NTHR / q.short_len, step_at = NTHR % q.short_len;
+            uint32_t unit = tid / q.short_len, at = tid % q.short_len;  // (advances by NTHR instructions)
+            auto next_instr = [&]() -> uint32_t {  // 0xFFFFFFFF: beyond the short chunk, or beyond the list
+                uint32_t i = 0xFFFFFFFFu;
+                if (unit < n_list) {
+                    const uint2 span = list[unit];
+                    if (span.x + at < span.y) i = span.x + at;
+                }
+                unit += step_unit;
+                at += step_at;
+                if (at >= q.short_len) { at -= q.short_len; ++unit; }
+                return i;
             };
-            auto fetch_rec = [&](uint32_t i) { return i != 0xFFFFFFFFu ? q.irec[i] : make_uint4(0, 0, 0, 0); };
+            auto fetch_rec = [&](uint32_t i) { return q.irec[min(i, q.nI - 1)]; };  // (looked at only if i is one)
             uint32_t us_nx[LU];
             auto fetch_list = [&](const uint4 &r) {
-                const uint32_t n = r.y & 0xFFFFu;
+                const uint32_t n = r.y & 0xFFFFu, last = n ? n - 1 : 0u;
 #pragma unroll
-                for (int u = 0; u < LU; ++u) us_nx[u] = sub + 2 * u < n ? q.ls[r.x + sub + 2 * u] : 0xFFFFFFFFu;
+                for (int u = 0; u < LU; ++u) us_nx[u] = q.ls[r.x + min((uint32_t)u, last)];
             };
-            uint32_t i_nx = instr_of(tid / 2), i_nx2 = instr_of(tid / 2 + NG);
+            uint32_t i_nx = next_instr(), i_nx2 = next_instr();
             uint4 rec_nx = fetch_rec(i_nx), rec_nx2 = fetch_rec(i_nx2);
             fetch_list(rec_nx);
-            for (uint32_t f = tid / 2; f < n_slots; f += NG) {
+            const uint32_t n_slots = n_list * q.short_len;
+            for (uint32_t f = tid; f < n_slots; f += NTHR) {
                 const uint32_t i = i_nx;
                 const uint4 rec = rec_nx;
                 uint32_t us[LU], ts[LU];
@@ -422,32 +442,36 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
                 i_nx = i_nx2;
                 rec_nx = rec_nx2;
                 fetch_list(rec_nx);
-                i_nx2 = instr_of(f + 2 * NG);
+                i_nx2 = next_instr();
                 rec_nx2 = fetch_rec(i_nx2);
-                const uint32_t n = rec.y & 0xFFFFu, nd = (rec.y >> 16) & 0xFFu;
+                const uint32_t n = rec.y & 0xFFFFu, nd = i != 0xFFFFFFFFu ? (rec.y >> 16) & 0xFFu : 0u;
                 if (!nd) continue;
                 uint32_t cnt = 0;
 #pragma unroll
-                for (int u = 0; u < LU; ++u) ts[u] = us[u] != 0xFFFFFFFFu ? T[us[u]] : 0x1000000u;  // (near nothing)
+                for (int u = 0; u < LU; ++u) ts[u] = T[(uint32_t)u < n ? us[u] : q.V];
                 for (uint32_t d = 0; d < nd; ++d) {
                     const uint32_t v = d ? q.op_vreg[rec.w + d] : rec.z, sv = T[v], wv = W[v];
                     // [t, t + wt) overlaps [sv, sv + wv): t < sv + wv and t > sv - wt, wt at most wmax
                     const uint32_t shift = q.wmax - 1 - sv, span = wv + q.wmax - 1;
-                    cnt += through_overlaps(v, d ? is_member(v) : rec.y >> 31, sub, 2);
+                    cnt += through_overlaps(v, d ? is_member(v) : rec.y >> 31);
+                    bool near = false;
 #pragma unroll
-                    for (int u = 0; u < LU; ++u)
-                        if (ts[u] + shift < span)
-                            if (us[u] != v && ts[u] + W[us[u]] > sv) ++cnt;
-                    for (uint32_t e0 = sub + 2 * LU; e0 < n; e0 += 8) {
-                        uint32_t x[4];
+                    for (int u = 0; u < LU; ++u) near |= ts[u] + shift < span;
+                    if (near) {
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) x[u] = e0 + 2 * u < n ? q.ls[rec.x + e0 + 2 * u] : v;
+                        for (int u = 0; u < LU; ++u)
+                            if ((uint32_t)u < n && us[u] != v && overlap(sv, wv, ts[u], W[us[u]])) ++cnt;
+                    }
+                    for (uint32_t e0 = LU; e0 < n; e0 += LU) {
+                        uint32_t x[LU];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (x[u] != v && overlap(sv, wv, T[x[u]], W[x[u]])) ++cnt;
+                        for (int u = 0; u < LU; ++u) x[u] = q.ls[rec.x + min(e0 + u, n - 1)];
+#pragma unroll
+                        for (int u = 0; u < LU; ++u)
+                            if (e0 + u < n && x[u] != v && overlap(sv, wv, T[x[u]], W[x[u]])) ++cnt;
                     }
                     if (nd > 1)  // co-defined vregs that are not live after the instruction
-                        for (uint32_t d2 = sub; d2 < nd; d2 += 2) {
+                        for (uint32_t d2 = 0; d2 < nd; ++d2) {
                             if (d2 == d || !(q.opflags[rec.w + d2] & OPF_DEAD)) continue;
                             const uint32_t x = q.op_vreg[rec.w + d2];
                             if (overlap(sv, wv, T[x], W[x])) ++cnt;
@@ -463,11 +487,11 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
                 for (uint32_t e0 = tid; e0 < n_el; e0 += 4 * NTHR) {
                     uint4 x[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) x[u] = e0 + u * NTHR < n_el ? el[e0 + u * NTHR] : make_uint4(0, 0, 0, 0);
+                    for (int u = 0; u < 4; ++u) x[u] = el[min(e0 + u * NTHR, n_el - 1)];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        if (!(x[u].z >> 31) || ((coll[x[u].w >> 5] >> (x[u].w & 31)) & 1u)) continue;
-                        const uint32_t n = through_overlaps(x[u].z & 0xFFFFu, true, 0, 1);
+                        if (e0 + u * NTHR >= n_el || !(x[u].z >> 31) || ((coll[x[u].w >> 5] >> (x[u].w & 31)) & 1u)) continue;
+                        const uint32_t n = through_overlaps(x[u].z & 0xFFFFu, true);
                         if (n) { pairs += n; mind = min(mind, x[u].x); }
                     }
                 }
@@ -518,27 +542,35 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
     }
 }
 
-// Threads per block for a job of K rows, 0 if the program does not fit the fused kernel.
-uint32_t fused_threads(vl_program *p, uint64_t K)
+// Threads per block for a job of K rows (0 if the program does not fit the kernel) and how many such blocks the device
+// holds at a time.  Up to one row per multiprocessor a block takes a whole one; for more rows two blocks share one,
+// where their masks let them (a program of 8,000 instructions: 16.6 us for 148 rows, 38 us for 300).
+uint32_t fused_plan(vl_program *p, uint64_t K, uint64_t *resident)
 {
     const uint32_t cap = 227 * 1024;
-    const uint32_t want = K <= (uint64_t)vl_sm_count(p) ? 512u : 256u;
-    for (uint32_t t = want; t >= 256; t /= 2)
-        if (p->nS <= 65535u && fused_smem(p, t).total <= cap) return t;
-    return 0;
+    const uint64_t sms = (uint64_t)vl_sm_count(p);
+    if (p->nS > 65535u) return 0;
+    const uint32_t half = fused_smem(p, 256).total, full = fused_smem(p, 512).total;
+    if (K > sms && 2 * (half + 1024) <= cap) { *resident = 2 * sms; return 256; }
+    *resident = sms;
+    return full <= cap ? 512u : (half <= cap ? 256u : 0u);
 }
 
 }  // namespace
 
-// Jobs of up to 100 rows: 10 us against 44 for a program of 2,000 instructions, 20 against 85 for 8,000, 39 against
-// 126 for 32,000.  From about two thirds of the multiprocessors on, one row whose every chunk collides (80 us on one
-// multiprocessor; the batched recount spreads it) decides the time, and from one row per multiprocessor on the
-// batched kernels read the program's tables for 8 or 64 rows at a time.
+// Jobs whose rows the device holds at a time: 10 us against 45 for 100 rows of a program of 2,000 instructions, 60
+// against 86 for 148 rows of one of 8,000 (17 against 73 when no row fails), 54 against 146 for one of 32,000.  Beyond
+// that the batched kernels, which read the program's tables for 8 or 64 rows at a time, win as soon as the rounds of
+// this kernel (about 4 us and 3 ns per instruction) take longer than their launches: 600 rows of 2,000 instructions 31
+// against 42 us, 1,000 rows 41 against 42; 3,000 rows of 64 instructions 40 against 68, 10,000 rows 124 against 79.
 bool vl_fused_wanted(vl_program *p, uint64_t K)
 {
     if (p->group_opt || p->threads_opt || p->test_wait) return false;  // the caller asks for the batched kernels
     if (p->P + p->wmax > 32768u) return false;                         // (not a program the verify path takes)
-    return K <= 100 && fused_threads(p, K) != 0;
+    uint64_t resident = 0;
+    if (!fused_plan(p, K, &resident)) return false;
+    const uint64_t rounds = (K + resident - 1) / resident;
+    return rounds <= 1 || rounds * (4000 + 3ull * p->nI) <= 36000;
 }
 
 int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict)
@@ -554,12 +586,13 @@ int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pit
             done[p->device] = true;
         }
     }
-    const uint32_t threads = fused_threads(p, K);
+    uint64_t resident = 0;
+    const uint32_t threads = fused_plan(p, K, &resident);
     FParams q{};
     q.nI = p->nI; q.V = p->V; q.nO = dict ? p->nD : p->nO; q.P = p->P; q.B = p->B; q.nB = p->nB; q.nS = p->nS; q.Wv = p->Wv;
     q.Wp = (p->P + p->wmax + 31) / 32; q.R = p->P + p->wmax + 2; q.wmax = p->wmax;
     q.bank_fast = p->bank_fast; q.use_th = p->use_th;
-    while ((1u << q.short_shift) < p->short_len) ++q.short_shift;
+    q.short_len = p->short_len;
     q.sm = fused_smem(p, threads);
     q.first_occ = dict ? p->d_dict_first_occ : p->d_first_occ; q.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16;
     q.vinfo = p->d_vinfo; q.first_def_instr = p->d_first_def_instr; q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg;
@@ -568,8 +601,8 @@ int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pit
     for (int j = 0; j < 4; ++j) q.bank_seg[j] = p->bank_seg[j];
     q.th_off = p->d_th_off; q.th = p->d_th; q.blk_th = p->d_blk_th; q.sev_off = p->d_sev_off; q.sev = p->d_sev;
     q.sen_off = p->d_sen_off; q.sen = p->d_sen;
-    q.short_blk = p->d_short_blk; q.short_i0 = p->d_short_i0; q.blk_chunk_off = p->d_blk_chunk_off;
-    q.chunk_short_off = p->d_chunk_short_off; q.ls = p->d_ls; q.irec = p->d_irec; q.blk_off = p->d_blk_off;
+    q.short_blk = p->d_short_blk; q.short_i0 = p->d_short_i0; q.blk_short_off = p->d_blk_short_off;
+    q.ls = p->d_ls; q.irec = p->d_irec; q.blk_off = p->d_blk_off;
     q.el = p->d_el; q.el_count = p->d_el_count;
     q.cand = d_cand; q.pitch = pitch; q.out = d_out;
     const int rc = vl_live_join(p, st);

@@ -94,7 +94,7 @@ struct vl_program {
     uint8_t *d_ndefs = nullptr, *d_width = nullptr;
     uint32_t *d_chunk_i0 = nullptr, *d_chunk_i1 = nullptr, *d_chunk_blk = nullptr, *d_blk_chunk_off = nullptr;
     uint32_t *d_piece_i0 = nullptr, *d_piece_chunk = nullptr, *d_chunk_piece_off = nullptr;
-    uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr, *d_short_i0 = nullptr;
+    uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr, *d_short_i0 = nullptr, *d_blk_short_off = nullptr;
 
     // liveness results
     uint32_t *d_blk_in = nullptr, *d_blk_out = nullptr, *d_lo_off = nullptr, *d_lo = nullptr;

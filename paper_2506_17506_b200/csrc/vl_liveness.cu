@@ -918,7 +918,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     p->nSeg = (uint32_t)seg_c0.size();
     seg_c0.push_back(nC);
     // short chunks: as few pieces as keep their number within SHORT_CHUNKS, equally long inside a chunk
-    std::vector<uint32_t> s_p0, c_s_off(nC + 1, 0), s_blk, s_i0;
+    std::vector<uint32_t> s_p0, c_s_off(nC + 1, 0), s_blk, s_i0, b_s_off;
     for (uint32_t r = std::max(1u, (p->nP + SHORT_CHUNKS - 1) / SHORT_CHUNKS);; ++r) {
         uint64_t total = 0;
         for (uint32_t c = 0; c < nC; ++c) total += (c_p_off[c + 1] - c_p_off[c] + r - 1) / r;
@@ -936,6 +936,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     p->nS = (uint32_t)s_p0.size();
     for (uint32_t x : s_p0) s_i0.push_back(p_i0[x]);
     s_i0.push_back(p->nI);
+    for (uint32_t b = 0; b <= nB; ++b) b_s_off.push_back(c_s_off[blk_c_off[b]]);
     p->short_len = 1;
     for (uint32_t j = 0; j < p->nS; ++j) p->short_len = std::max(p->short_len, s_i0[j + 1] - s_i0[j]);
     std::vector<uint32_t> all;
@@ -944,7 +945,8 @@ static int vl_layout(vl_program *p, cudaStream_t st)
                           {&p->d_blk_chunk_off, &blk_c_off}, {&p->d_piece_i0, &p_i0}, {&p->d_piece_chunk, &p_chunk},
                           {&p->d_chunk_piece_off, &c_p_off}, {&p->d_seg_c0, &seg_c0}, {&p->d_blk_seg_off, &blk_seg_off},
                           {&p->d_short_p0, &s_p0}, {&p->d_chunk_short_off, &c_s_off}, {&p->d_short_blk, &s_blk},
-                          {&p->d_short_i0, &s_i0}};
+                          {&p->d_short_i0, &s_i0},
+                          {&p->d_blk_short_off, &b_s_off}};
     for (const Part &x : parts) {
         all.insert(all.end(), x.v->begin(), x.v->end());
         all.resize((all.size() + 4) & ~(size_t)3);  // (at least one word behind every array)

@@ -35,10 +35,10 @@ def test_random_programs(B, oracle_mod, P, chunk):
 
 
 @pytest.mark.parametrize("chunk", [160, 8])
-@pytest.mark.parametrize("K", [1, 100, 101])
+@pytest.mark.parametrize("K", [1, 148, 149, 297])
 def test_row_counts_and_many_short_chunks(B, oracle_mod, K, chunk):
-    """Attention-shaped program with the last row count of the path, the first beyond it, and more short chunks (1,000)
-    than a thread block has threads."""
+    """Attention-shaped program with one row per multiprocessor, two, and too many for the path; and with more short
+    chunks (1,000) than a thread block has threads."""
     wl = synth.workload(2)
     p = synth.build_program(wl.shapes[0], wl.seeds[0])
     rows, _ = synth.candidate_rows(p, K, 0.5, 77)
