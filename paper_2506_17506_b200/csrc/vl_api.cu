@@ -12,16 +12,19 @@ std::atomic<uint64_t> g_vl_launches{0};
 #define VL_MAX_DEVICES 64
 static std::mutex g_lane_mutex;
 static cudaStream_t g_lanes[VL_MAX_DEVICES][VL_STREAMS];  // the lanes, the liveness stream
+static cudaEvent_t g_lane_done[VL_MAX_DEVICES][VL_LANES];  // behind the last liveness batch of a lane
 static bool g_lanes_made[VL_MAX_DEVICES];
 
-int vl_lane_streams(vl_program *p, cudaStream_t **lanes)
+int vl_lane_streams(vl_program *p, cudaStream_t **lanes, cudaEvent_t **done)
 {
     if (p->device < 0 || p->device >= VL_MAX_DEVICES) return VL_ERR_UNSUPPORTED;
     {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
         if (!g_lanes_made[p->device]) {
-            for (int l = 0; l < VL_LANES; ++l)
+            for (int l = 0; l < VL_LANES; ++l) {
                 VL_CUDA(p, cudaStreamCreateWithFlags(&g_lanes[p->device][l], cudaStreamNonBlocking));
+                VL_CUDA(p, cudaEventCreateWithFlags(&g_lane_done[p->device][l], cudaEventDisableTiming));
+            }
             // the liveness stream: its small kernels go first wherever a multiprocessor has room
             int least = 0, greatest = 0;
             VL_CUDA(p, cudaDeviceGetStreamPriorityRange(&least, &greatest));
@@ -33,6 +36,7 @@ int vl_lane_streams(vl_program *p, cudaStream_t **lanes)
     if (!p->ev_pre) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_pre, cudaEventDisableTiming));
     for (int l = 0; l < VL_LANES; ++l)
         if (!p->ev_join[l]) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_join[l], cudaEventDisableTiming));
+    if (done) *done = g_lane_done[p->device];
     *lanes = g_lanes[p->device];
     return VL_OK;
 }
@@ -378,7 +382,8 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     // about as much as the run could hide.
     if (p->nI <= LIVE_INLINE_INSTRS) {
         p->live_stream = (cudaStream_t)stream;
-        const int rc = vl_liveness_impl(p, (cudaStream_t)stream);
+        const cudaStream_t st = (cudaStream_t)stream;
+        const int rc = vl_liveness_impl(&p, 1, &st, nullptr, 1);
         p->live_deferred = true;
         return rc;
     }
@@ -392,14 +397,14 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     VL_CUDA(p, cudaEventRecord(p->ev_pre, (cudaStream_t)stream));
     VL_CUDA(p, cudaStreamWaitEvent(ls, p->ev_pre, 0));
     p->live_stream = ls;
-    rc = vl_liveness_impl(p, ls);
+    rc = vl_liveness_impl(&p, 1, &ls, nullptr, 1);
     p->live_deferred = true;
     return rc;
 }
 
 int vl_live_join(vl_program *p, cudaStream_t st)
 {
-    if (p->live_deferred && p->ev_live && st != p->live_stream) VL_CUDA(p, cudaStreamWaitEvent(st, p->ev_live, 0));
+    if (p->live_deferred && p->live_done && st != p->live_stream) VL_CUDA(p, cudaStreamWaitEvent(st, p->live_done, 0));
     return VL_OK;
 }
 
@@ -413,17 +418,22 @@ extern "C" int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *str
     VL_CUDA(p0, cudaSetDevice(p0->device));
     cudaStream_t st = (cudaStream_t)stream;
     cudaStream_t *lane = nullptr;
-    int rc = vl_lane_streams(p0, &lane);
+    cudaEvent_t *done = nullptr;
+    int rc = vl_lane_streams(p0, &lane, &done);
     if (rc != VL_OK) return rc;
     for (uint32_t j = 0; j < n; ++j) {
         // an earlier single run of one of these programs may still sit on the liveness stream
         if ((rc = vl_live_join(progs[j], st)) != VL_OK) return rc;
         progs[j]->live_deferred = false;
     }
-    if (n == 1) return vl_liveness_impl(p0, st);
+    if (n == 1) return vl_liveness_impl(progs, 1, &st, nullptr, 1);
     VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
     for (uint32_t l = 0; l < VL_LANES; ++l) VL_CUDA(p0, cudaStreamWaitEvent(lane[l], p0->ev_fork, 0));
-    for (uint32_t j = 0; j < n && rc == VL_OK; ++j) rc = vl_liveness_impl(progs[j], lane[j % VL_LANES]);
+    std::vector<vl_program *> once(progs, progs + n);  // a handle given twice runs once
+    std::sort(once.begin(), once.end());
+    once.erase(std::unique(once.begin(), once.end()), once.end());
+    if (once.size() == n) once.assign(progs, progs + n);  // (in the caller's order)
+    rc = vl_liveness_impl(once.data(), (uint32_t)once.size(), lane, done, VL_LANES);
     // join even after an error, so that the caller's stream stays ordered after what was launched
     for (uint32_t l = 0; l < VL_LANES; ++l) {
         cudaError_t e = cudaEventRecord(p0->ev_join[l], lane[l]);

@@ -115,6 +115,7 @@ struct vl_program {
     uint32_t *d_dict_instr = nullptr;     // [nD8] first instruction of the entry's block that touches its vreg
     uint4 *d_opoff = nullptr;               // [nOpT / 4] per 4 operands: byte offsets of their vregs' 16-byte table entries
     uint8_t *d_first4 = nullptr;            // [nOpT / 4] per 4 operands: first-occurrence bits
+    uint8_t *d_opmeta = nullptr;            // [nO] scratch of the first run
     uint8_t *d_opflags = nullptr;           // [nO]
     uint32_t *d_first_occ = nullptr;        // [V] first operand that names v, 0xFFFFFFFF if none
     uint32_t *d_first_def_instr = nullptr;  // [V] lowest instruction defining v, 0xFFFFFFFF if none
@@ -159,6 +160,7 @@ struct vl_program {
     // the host side (vl_live_settle) waits for the run and checks them.
     uint32_t *h_live = nullptr;      // pinned: [0] status, [2..13] six 64-bit totals, written by the run's kernels
     cudaEvent_t ev_live = nullptr;
+    cudaEvent_t live_done = nullptr;  // the event behind the last run: ev_live, or the one of the lane a batch ran it on
     bool live_pending = false;
     // vl_liveness of a long program runs on an internal stream (live_stream) behind what the caller's stream held
     // when it was called; the caller's stream is not made to wait.  Calls that read the results make their stream wait
@@ -217,7 +219,7 @@ extern std::atomic<uint64_t> g_vl_launches;
         }                                       \
     } while (0)
 
-int vl_liveness_impl(vl_program *p, cudaStream_t st);
+int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, const cudaEvent_t *done, uint32_t n_streams);
 // The one-kernel verify path of short jobs (vl_fused.cu): whether a job of K rows takes it; one launch on st.
 bool vl_fused_wanted(vl_program *p, uint64_t K);
 int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict);
@@ -227,7 +229,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
                     const uint64_t *pitch, vl_verdict *const *d_out, cudaStream_t st, bool dict = false);
 // The lane streams of the handle's device (created once per device; the liveness stream
 // follows the VL_LANES lanes in the array) and the handle's fork / join events.
-int vl_lane_streams(vl_program *p, cudaStream_t **lanes);
+int vl_lane_streams(vl_program *p, cudaStream_t **lanes, cudaEvent_t **done = nullptr);
 void vl_free_liveness(vl_program *p);
 // Waits for a liveness run that is still in flight and checks its outcome; VL_OK if none is pending.
 int vl_live_settle(vl_program *p);

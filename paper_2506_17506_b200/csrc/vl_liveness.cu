@@ -59,6 +59,16 @@ struct LiveArgs {
     uint32_t *el_count, *status;
     uint32_t *host_out;                           // pinned: [0] status, [2..] totals (64 bit)
 };
+// The runs of up to N programs in one grid: blockIdx.y is the program.  (As kernel arguments: 64 programs of one call
+// would otherwise be 320 launches, or an upload in front of every run.)
+#define LV_MANY 48
+template <int N>
+struct LiveMany {
+    LiveArgs p[N];
+};
+static_assert(sizeof(LiveMany<LV_MANY>) <= 32764, "kernel arguments");
+#define LIVE_ARGS const LiveArgs &q = a.p[N == 1 ? 0 : blockIdx.y]
+
 enum { LV_TOT_LO = 0, LV_TOT_EV = 1, LV_TOT_TH = 2, LV_TOT_LS = 3, LV_TOT_SEV = 4, LV_TOT_SEN = 5, LV_TOTALS = 6 };
 
 // ------------------------------------------------------------------ device helpers
@@ -132,8 +142,10 @@ __device__ __forceinline__ bool po_def(uint32_t x) { return (x >> 20) & 1u; }
 // ============================================================================ k_sets
 // One thread block per chunk.  use = vregs read before any write inside the piece (the chunk), def = vregs
 // written.  A lane holds an operand and meets the piece's other operands by shuffles.
-__global__ void __launch_bounds__(PC_NT) k_sets(const LiveArgs q)
+template <int N>
+__global__ void __launch_bounds__(PC_NT) k_sets(const __grid_constant__ LiveMany<N> a)
 {
+    LIVE_ARGS;
     extern __shared__ uint32_t sm[];
     const uint32_t c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_go();
@@ -191,11 +203,14 @@ __global__ void __launch_bounds__(PC_NT) k_sets(const LiveArgs q)
 // the chunk sets of segments (SEG_CHUNKS loads in flight instead of a chain over a block's chunks), one warp
 // iterates the blocks, and the warps walk the segments back to the live sets at the chunk boundaries.
 // Working set: [4][nB][32] + [2][nSeg][32] words and the successor lists, in shared memory or flow_scratch.
-__global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const LiveArgs q)
+template <int N>
+__global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const __grid_constant__ LiveMany<N> a)
 {
+    LIVE_ARGS;
     extern __shared__ uint32_t sm[];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t w = blockIdx.x * 32 + lane;
+    if (blockIdx.x * 32 >= q.Wv) return;
     const bool in = w < q.Wv;
     const size_t words = ((size_t)4 * q.nB + 2 * (size_t)q.nSeg) * 32 + q.nB + 1 + q.nE;
     uint32_t *base = q.flow_scratch ? q.flow_scratch + blockIdx.x * words : sm;
@@ -295,11 +310,14 @@ __global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const LiveArgs q)
 // none does, iff it is live after the piece.  From that the operand flags, the walk events and the change of
 // the live count of every instruction follow without a serial walk; and the set of vregs whose occupancy
 // changes inside the block.  Last, offsets inside the chunk.
-__global__ void __launch_bounds__(PC_NT) k_count(const LiveArgs q)
+template <int N>
+__global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMany<N> a)
 {
+    LIVE_ARGS;
     __shared__ uint32_t s_scan[34], s_ev[PC_WARPS][PIECE_INSTRS];
     __shared__ int s_d[PC_WARPS][PIECE_INSTRS];
     const uint32_t c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (c >= q.nC) return;
     const uint32_t p0 = q.chunk_piece_off[c], p1 = q.chunk_piece_off[c + 1];
     const uint32_t blk = q.chunk_blk[c];
     uint32_t *touch = q.blk_touch + (size_t)blk * q.Wv;
@@ -428,12 +446,15 @@ __device__ __forceinline__ uint32_t entry_word(const LiveArgs &q, uint32_t c, ui
 // of a block (live on entry and never touched by an event inside it).  The block that finishes last makes the
 // offsets: list entries per chunk, walk events per chunk (padded to groups of 8), through-sets per block, steps
 // per 32 short chunks; and writes the totals and the status word to pinned host memory.
-__global__ void __launch_bounds__(OFF_NT) k_offsets(const LiveArgs q)
+template <int N>
+__global__ void __launch_bounds__(OFF_NT) k_offsets(const __grid_constant__ LiveMany<N> a)
 {
+    LIVE_ARGS;
     __shared__ uint32_t s_scan[34];
     __shared__ unsigned long long s_tot[LV_TOTALS];
     __shared__ uint32_t s_last;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (blockIdx.x >= q.nC + q.nB) return;
     pdl_go();
     pdl_wait();
     if (blockIdx.x < q.nC) {
@@ -464,7 +485,7 @@ __global__ void __launch_bounds__(OFF_NT) k_offsets(const LiveArgs q)
     }
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(&q.counters[0], 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (tid == 0) s_last = atomicAdd(&q.counters[0], 1u) == q.nC + q.nB - 1 ? 1u : 0u;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -685,8 +706,10 @@ __device__ __forceinline__ void instr_events(const LiveArgs &q, uint32_t i, F pu
             if ((q.opflags[o] & OPF_POST) && !(q.opflags[o] & OPF_ELIDE)) put(e++, q.op_vreg[o], false, true);
 }
 
-__global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
+template <int N>
+__global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany<N> a)
 {
+    LIVE_ARGS;
     extern __shared__ uint32_t sm[];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t role = blockIdx.x;
@@ -815,7 +838,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const LiveArgs q)
         return;
     }
     role -= n_short;
-    {   // through-set list of a block: vreg | width << 16
+    if (role < q.nB) {  // through-set list of a block: vreg | width << 16
         const uint32_t b = role;
         if (warp == 0)
             warp_bits(q.Wv, lane, [&](uint32_t w) { return q.blk_th[(size_t)b * q.Wv + w]; },
@@ -840,9 +863,12 @@ int live_attributes(vl_program *p)
     std::lock_guard<std::mutex> lock(mtx);
     if (done[p->device]) return VL_OK;
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_flow, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_fill, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_flow<1>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_fill<1>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_flow<LV_MANY>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_fill<LV_MANY>, at, 227 * 1024));
     done[p->device] = true;
     return VL_OK;
 }
@@ -851,20 +877,22 @@ int live_attributes(vl_program *p)
 #define TMP(out, n) VL_CUDA(p, pool_get(p->tmp_arena, out, n))
 #define LAYOUT(out, n) VL_CUDA(p, pool_get(p->layout_arena, out, n))
 
-// A launch that may overlap the tail of the launch before it (see pdl_wait).
-template <typename K>
-static cudaError_t launch_pdl(K kernel, uint32_t grid, uint32_t nt, size_t smem, cudaStream_t st, const LiveArgs &q)
+// One kernel of the runs of n programs; overlap: it may start while the launch before it drains (see pdl_wait).
+template <int N>
+static cudaError_t launch_live(void (*kernel)(const LiveMany<N>), uint32_t grid, uint32_t n, uint32_t nt, size_t smem,
+                               cudaStream_t st, const LiveMany<N> &args, bool overlap)
 {
     if (!grid) return cudaSuccess;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid; cfg.blockDim = nt; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cfg.attrs = &at; cfg.numAttrs = 1;
+    cfg.gridDim = dim3(grid, n); cfg.blockDim = nt; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &at; cfg.numAttrs = overlap ? 1 : 0;
     g_vl_launches.fetch_add(1);
-    return cudaLaunchKernelEx(&cfg, kernel, q);
+    return cudaLaunchKernelEx(&cfg, kernel, args);
 }
+
 #define LAUNCH(kernel, grid, nt, smem, st, ...)                 \
     do {                                                        \
         if ((grid) > 0) {                                       \
@@ -965,13 +993,24 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     return VL_OK;
 }
 
-// Enqueues one complete liveness run on st.  Without remembered list lengths it waits once in the middle to
-// read them.
-static int live_enqueue(vl_program *p, cudaStream_t st)
+// What a run's launches need besides the arguments.
+struct LiveShape {
+    uint32_t set_warps = PC_WARPS, sets = 0, flows = 0, counts = 0, offs = 0, fills = 0;
+    size_t sets_smem = 0, flow_smem = 0, fill_smem = 0;
+    void add(const LiveShape &o)
+    {
+        set_warps = std::min(set_warps, o.set_warps);
+        sets = std::max(sets, o.sets); flows = std::max(flows, o.flows); counts = std::max(counts, o.counts);
+        offs = std::max(offs, o.offs); fills = std::max(fills, o.fills);
+        sets_smem = std::max(sets_smem, o.sets_smem); flow_smem = std::max(flow_smem, o.flow_smem);
+        fill_smem = std::max(fill_smem, o.fill_smem);
+    }
+};
+
+// The memory of a run that does not depend on the list lengths, and its arguments.
+static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st)
 {
     vl_free_liveness(p);
-    int rc = live_attributes(p);
-    if (rc != VL_OK) return rc;
     const uint32_t nB = p->nB, nI = p->nI, V = p->V, nO = p->nO, Wv = p->Wv, nC = p->nC, nP = p->nP;
 
     // ---- results and tables that do not depend on the list lengths
@@ -980,7 +1019,6 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     KEEP(&p->d_lo_off, (size_t)nI + 1);
     KEEP(&p->d_opflags, (size_t)nO);
     // the operand tables of the verify kernels depend on the program alone: made by the first run, kept
-    const bool make_tables = !p->tables_built;
     if (!p->d_opoff) {
         LAYOUT(&p->d_first_def_instr, (size_t)V);
         LAYOUT(&p->d_first_occ, (size_t)V);
@@ -1001,7 +1039,7 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     KEEP(&p->d_sen_off, (size_t)p->nS + 1);
     KEEP(&p->d_irec, (size_t)nI);
 
-    LiveArgs q{};
+    q = LiveArgs{};
     q.nB = nB; q.nI = nI; q.V = V; q.nE = p->nE; q.Wv = Wv; q.nC = nC; q.nP = nP; q.nS = p->nS; q.nSeg = p->nSeg;
     q.use_th = p->use_th;
     q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg; q.succ_off = p->d_succ_off; q.succ = p->d_succ; q.blk_off = p->d_blk_off;
@@ -1032,9 +1070,8 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
         TMP(&q.flow_scratch, flow_smem / 4 * fgrid);
         flow_smem = 0;
     }
-    uint8_t *opmeta = nullptr;
-    if (make_tables) {
-        TMP(&opmeta, (size_t)nO);
+    if (!p->tables_built) {
+        TMP(&p->d_opmeta, (size_t)nO);
         VL_CUDA(p, cudaMemsetAsync(p->d_first_occ, 0xFF, std::max<size_t>(V, 1) * 4, st));
         VL_CUDA(p, cudaMemsetAsync(p->d_first_def_instr, 0xFF, std::max<size_t>(V, 1) * 4, st));
     }
@@ -1043,24 +1080,28 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     q.el = p->d_el; q.el_count = p->d_el_count; q.status = p->d_status; q.sev_off = p->d_sev_off; q.sen_off = p->d_sen_off; q.irec = p->d_irec;
     q.host_out = p->h_live;
     // a bitset pair per warp of k_sets: fewer warps for programs of very many vregs
-    const uint32_t set_warps = (uint32_t)std::max<size_t>(1, std::min<size_t>(PC_WARPS, (size_t)224 * 1024 / ((size_t)2 * Wv * 4)));
+    sh.set_warps = (uint32_t)std::max<size_t>(1, std::min<size_t>(PC_WARPS, (size_t)224 * 1024 / ((size_t)2 * Wv * 4)));
+    sh.sets = std::max(1u, nC); sh.flows = fgrid; sh.counts = nC; sh.offs = nC + nB;
+    sh.fills = (nP + LV_WARPS - 1) / LV_WARPS + nC + ((p->nS + 31) & ~31u) / LV_WARPS + nB;
+    sh.sets_smem = (size_t)sh.set_warps * 2 * Wv * 4;
+    sh.flow_smem = flow_smem;
+    sh.fill_smem = (size_t)LV_WARPS * 2 * Wv * 4;
+    return VL_OK;
+}
 
-    LAUNCH(k_sets, std::max(1u, nC), set_warps * 32, (size_t)set_warps * 2 * Wv * 4, st, q);
-    VL_CUDA(p, launch_pdl(k_flow, fgrid, FLOW_WARPS * 32, flow_smem, st, q));
-    VL_CUDA(p, launch_pdl(k_count, nC, PC_NT, 0, st, q));
-    VL_CUDA(p, launch_pdl(k_offsets, nC + nB, OFF_NT, 0, st, q));
-
-    // ---- list lengths: read on the first run with this layout; later runs allocate from the
-    // lengths they remember (same program, same layout) and only compare at the end
+// The list lengths: read on the first run with this layout (its first four kernels have finished); later runs
+// allocate from the lengths they remember (same program, same layout) and only compare at the end.
+static int live_lengths(vl_program *p, LiveArgs &q)
+{
     if (!p->sizes_known) {
-        VL_CUDA(p, cudaStreamSynchronize(st));
         const uint32_t status = p->h_live[0];
         unsigned long long tot[LV_TOTALS];
         memcpy(tot, p->h_live + 2, sizeof(tot));
         if (status & ST_NO_CONVERGE) return VL_ERR_NO_CONVERGE;
         if (status & ST_NOT_STRICT) return VL_ERR_NOT_STRICT;
         if (status & ST_SIZE_OVERFLOW) return VL_ERR_UNSUPPORTED;
-        if (tot[LV_TOT_EV] > 0xFFFFFFF0ull || tot[LV_TOT_SEV] > 0xFFFFFFF0ull || tot[LV_TOT_SEN] > 0xFFFFFFF0ull) return VL_ERR_UNSUPPORTED;
+        if (tot[LV_TOT_EV] > 0xFFFFFFF0ull || tot[LV_TOT_SEV] > 0xFFFFFFF0ull || tot[LV_TOT_SEN] > 0xFFFFFFF0ull)
+            return VL_ERR_UNSUPPORTED;
         memcpy(p->known, tot, sizeof(tot));
     }
     p->lo_len = p->known[LV_TOT_LO];
@@ -1071,39 +1112,104 @@ static int live_enqueue(vl_program *p, cudaStream_t st)
     KEEP(&p->d_sev, (size_t)p->known[LV_TOT_SEV]);
     KEEP(&p->d_sen, (size_t)p->known[LV_TOT_SEN]);
     q.lo = p->d_lo; q.ls = p->d_ls; q.ev = p->d_ev; q.th = p->d_th; q.sev = p->d_sev; q.sen = p->d_sen;
-    const uint32_t n_list = (nP + LV_WARPS - 1) / LV_WARPS, n_short = ((p->nS + 31) & ~31u) / LV_WARPS;
-    VL_CUDA(p, launch_pdl(k_fill, n_list + nC + n_short + nB, LV_NT, (size_t)LV_WARPS * 2 * Wv * 4, st, q));
-    if (make_tables) {
-        LAUNCH(k_first_occ, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
-               p->d_first_def_instr);
-        LAUNCH(k_vreg_info, (V + NT - 1) / NT, NT, 0, st, V, p->d_width, p->d_first_occ, p->d_first_def_instr, p->d_vinfo);
-        LAUNCH(k_operand_meta, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
-               p->d_opflags, p->d_vreg16, opmeta, p->d_status);
-        LAUNCH(k_pack_slots, (p->nOpT / 8 + NT - 1) / NT, NT, 0, st, nO, p->nOp8, p->nOpT / 8, V, opmeta, p->d_vreg16,
-               p->d_slotmeta, p->d_opoff, p->d_first4);
-    }
+    return VL_OK;
+}
+
+// The operand tables of the verify kernels (first run).
+static int live_tables(vl_program *p, cudaStream_t st)
+{
     p->bank_fast = ((p->B == 1 || p->B == 2 || p->B == 4) && !p->bank_many) ? 1 : 0;
+    if (p->tables_built) return VL_OK;
+    const uint32_t nI = p->nI, V = p->V;
+    LAUNCH(k_first_occ, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
+           p->d_first_def_instr);
+    LAUNCH(k_vreg_info, (V + NT - 1) / NT, NT, 0, st, V, p->d_width, p->d_first_occ, p->d_first_def_instr, p->d_vinfo);
+    LAUNCH(k_operand_meta, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
+           p->d_opflags, p->d_vreg16, p->d_opmeta, p->d_status);
+    LAUNCH(k_pack_slots, (p->nOpT / 8 + NT - 1) / NT, NT, 0, st, p->nO, p->nOp8, p->nOpT / 8, V, p->d_opmeta, p->d_vreg16,
+           p->d_slotmeta, p->d_opoff, p->d_first4);
+    VL_CUDA(p, cudaGetLastError());
     p->tables_built = true;
     return VL_OK;
 }
 
-// One run.  Everything is recomputed on the device every time.
-int vl_liveness_impl(vl_program *p, cudaStream_t st)
+// The first four kernels of the runs of n <= N programs, or the last one.
+template <int N>
+static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *args, const LiveShape *shapes, bool fill,
+                       cudaStream_t st)
 {
-    vl_live_settle(p);  // the pinned words of an earlier run are about to be reused
-    int rc = vl_layout(p, st);
+    vl_program *p = progs[0];
+    LiveShape sh;
+    LiveMany<N> many;
+    for (uint32_t j = 0; j < n; ++j) {
+        sh.add(shapes[j]);
+        many.p[j] = args[j];
+    }
+    if (fill) {
+        VL_CUDA(p, launch_live<N>(k_fill<N>, sh.fills, n, LV_NT, sh.fill_smem, st, many, true));
+        return VL_OK;
+    }
+    VL_CUDA(p, launch_live<N>(k_sets<N>, sh.sets, n, sh.set_warps * 32, sh.sets_smem, st, many, false));
+    VL_CUDA(p, launch_live<N>(k_flow<N>, sh.flows, n, FLOW_WARPS * 32, sh.flow_smem, st, many, true));
+    VL_CUDA(p, launch_live<N>(k_count<N>, sh.counts, n, PC_NT, 0, st, many, true));
+    VL_CUDA(p, launch_live<N>(k_offsets<N>, sh.offs, n, OFF_NT, 0, st, many, true));
+    return VL_OK;
+}
+
+// The runs of n programs, LV_MANY of them per launch, the launches spread over the n_streams streams.  Everything is
+// recomputed on the device every time.  done[s] is the event recorded behind the work of stream s (null: the
+// program's own; n == 1).  Programs behind the first one with an error are left without a run.
+int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, const cudaEvent_t *done, uint32_t n_streams)
+{
+    std::vector<LiveArgs> args(n);
+    std::vector<LiveShape> shapes(n);
+    bool lengths_known = true;
+    int rc = n ? live_attributes(progs[0]) : VL_OK;
     if (rc != VL_OK) return rc;
-    if (!p->h_live) VL_CUDA(p, cudaHostAlloc((void **)&p->h_live, 128, cudaHostAllocDefault));
-    if (!p->ev_live) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_live, cudaEventDisableTiming));
-    if ((rc = live_enqueue(p, st)) != VL_OK) return rc;
-    VL_CUDA(p, cudaEventRecord(p->ev_live, st));
-    VL_CUDA(p, cudaGetLastError());
-    p->live_pending = true;
-    p->live_ok = true;
-    if (p->sizes_known) return VL_OK;  // lengths remembered from an earlier run: checked when the results are used
-    rc = vl_live_settle(p);
-    if (rc == VL_OK) p->sizes_known = true;
-    return rc;
+    const uint32_t per = n == 1 ? 1 : LV_MANY;
+    auto stream_of = [&](uint32_t j) { return (j / per) % n_streams; };
+    for (uint32_t j = 0; j < n; ++j) {
+        vl_program *p = progs[j];
+        vl_live_settle(p);  // the pinned words of an earlier run are about to be reused
+        if ((rc = vl_layout(p, streams[stream_of(j)])) != VL_OK) return rc;
+        if (!p->h_live) VL_CUDA(p, cudaHostAlloc((void **)&p->h_live, 128, cudaHostAllocDefault));
+        if (!p->ev_live) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_live, cudaEventDisableTiming));
+        if ((rc = live_begin(p, args[j], shapes[j], streams[stream_of(j)])) != VL_OK) return rc;
+        lengths_known = lengths_known && p->sizes_known;
+    }
+    auto launch = [&](bool fill) -> int {
+        for (uint32_t j = 0; j < n; j += per) {
+            const cudaStream_t st = streams[stream_of(j)];
+            const uint32_t m = std::min(per, n - j);
+            const int r = m == 1 ? live_launch<1>(progs + j, 1, &args[j], &shapes[j], fill, st)
+                                 : live_launch<LV_MANY>(progs + j, m, &args[j], &shapes[j], fill, st);
+            if (r != VL_OK) return r;
+        }
+        return VL_OK;
+    };
+    if ((rc = launch(false)) != VL_OK) return rc;
+    if (!lengths_known)
+        for (uint32_t s = 0; s < n_streams; ++s) VL_CUDA(progs[0], cudaStreamSynchronize(streams[s]));
+    int err = VL_OK;
+    for (uint32_t j = 0; j < n; ++j)
+        if ((err = live_lengths(progs[j], args[j])) != VL_OK) { n = j; break; }
+    if ((rc = launch(true)) != VL_OK) return rc;
+    for (uint32_t j = 0; j < n; ++j)
+        if ((rc = live_tables(progs[j], streams[stream_of(j)])) != VL_OK) return rc;
+    for (uint32_t j = 0; j < n; ++j) {
+        vl_program *p = progs[j];
+        p->live_done = done ? done[stream_of(j)] : p->ev_live;
+        if (j % per == 0 && j / per < n_streams) VL_CUDA(p, cudaEventRecord(p->live_done, streams[stream_of(j)]));  // once per stream
+        p->live_pending = true;
+        p->live_ok = true;
+    }
+    if (n) VL_CUDA(progs[0], cudaGetLastError());
+    if (lengths_known) return err;  // lengths remembered from an earlier run: checked when the results are used
+    for (uint32_t j = 0; j < n; ++j) {
+        if ((rc = vl_live_settle(progs[j])) != VL_OK) return rc;
+        progs[j]->sizes_known = true;
+    }
+    return err;
 }
 
 int vl_live_settle(vl_program *p)
@@ -1111,7 +1217,7 @@ int vl_live_settle(vl_program *p)
     if (!p->live_pending) return VL_OK;
     p->live_pending = false;
     p->live_ok = false;
-    VL_CUDA(p, cudaEventSynchronize(p->ev_live));
+    VL_CUDA(p, cudaEventSynchronize(p->live_done));
     const uint32_t status = p->h_live[0];
     unsigned long long tot[LV_TOTALS];
     memcpy(tot, p->h_live + 2, sizeof(tot));
