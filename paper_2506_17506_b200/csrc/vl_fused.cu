@@ -63,9 +63,16 @@ struct FParams {
     const uint32_t *ls, *el_count;
     const uint4 *el, *irec;
     const uint16_t *cand;
-    uint64_t pitch;
+    uint64_t K, pitch;
     vl_verdict *out;
 };
+
+// The jobs of up to N programs in one grid: blockIdx.y is the program.
+template <int N>
+struct FMany {
+    FParams p[N];
+};
+static_assert(sizeof(FMany<VL_FUSED_MANY>) <= 32764, "kernel arguments");
 
 __device__ __forceinline__ bool overlap(uint32_t a, uint32_t wa, uint32_t b, uint32_t wb) { return a < b + wb && b < a + wa; }
 
@@ -93,9 +100,11 @@ __device__ __forceinline__ uint32_t bank_entry(const uint2 &id, uint32_t n, cons
     return n == 2 ? bank_extra<2>(x, bmask) : (n == 3 ? bank_extra<3>(x, bmask) : bank_extra<4>(x, bmask));
 }
 
-template <int NTHR>
-__global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const FParams q)
+template <int NTHR, int N>
+__global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const __grid_constant__ FMany<N> a)
 {
+    const FParams &q = a.p[N == 1 ? 0 : blockIdx.y];
+    if (N > 1 && blockIdx.x >= q.K) return;
     extern __shared__ __align__(16) unsigned char smem[];
     uint16_t *T = reinterpret_cast<uint16_t *>(smem);                 // [V + 1] register of every vreg
     uint8_t *W = smem + q.sm.w;                                       // [V] width
@@ -561,7 +570,7 @@ uint32_t fused_plan(vl_program *p, uint64_t K, uint64_t *resident)
 // Jobs whose rows the device holds at a time: 10 us against 45 for 100 rows of a program of 2,000 instructions, 60
 // against 86 for 148 rows of one of 8,000 (17 against 73 when no row fails), 54 against 146 for one of 32,000.  Beyond
 // that the batched kernels, which read the program's tables for 8 or 64 rows at a time, win as soon as the rounds of
-// this kernel (about 4 us and 3 ns per instruction) take longer than their launches: 600 rows of 2,000 instructions 31
+// this kernel (about 3 us and 3.5 ns per instruction) take longer than their launches: 600 rows of 2,000 instructions 31
 // against 42 us, 1,000 rows 41 against 42; 3,000 rows of 64 instructions 40 against 68, 10,000 rows 124 against 79.
 bool vl_fused_wanted(vl_program *p, uint64_t K)
 {
@@ -570,46 +579,71 @@ bool vl_fused_wanted(vl_program *p, uint64_t K)
     uint64_t resident = 0;
     if (!fused_plan(p, K, &resident)) return false;
     const uint64_t rounds = (K + resident - 1) / resident;
-    return rounds <= 1 || rounds * (4000 + 3ull * p->nI) <= 36000;
+    return rounds <= 1 || rounds * (6000 + 7ull * p->nI) <= 72000;
 }
 
-int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict)
+// Up to VL_FUSED_MANY jobs in one launch on st.
+int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
+                 vl_verdict *const *d_out, cudaStream_t st, bool dict)
 {
+    vl_program *p0 = progs[0];
     static std::mutex mtx;
     static bool done[64];
-    if (p->device >= 0 && p->device < 64) {
+    if (p0->device >= 0 && p0->device < 64) {
         std::lock_guard<std::mutex> lock(mtx);
-        if (!done[p->device]) {
+        if (!done[p0->device]) {
             const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-            VL_CUDA(p, cudaFuncSetAttribute(k_fused<256>, at, 227 * 1024));
-            VL_CUDA(p, cudaFuncSetAttribute(k_fused<512>, at, 227 * 1024));
-            done[p->device] = true;
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 1>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<512, 1>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, VL_FUSED_MANY>, at, 227 * 1024));
+            done[p0->device] = true;
         }
     }
-    uint64_t resident = 0;
-    const uint32_t threads = fused_plan(p, K, &resident);
-    FParams q{};
-    q.nI = p->nI; q.V = p->V; q.nO = dict ? p->nD : p->nO; q.P = p->P; q.B = p->B; q.nB = p->nB; q.nS = p->nS; q.Wv = p->Wv;
-    q.Wp = (p->P + p->wmax + 31) / 32; q.R = p->P + p->wmax + 2; q.wmax = p->wmax;
-    q.bank_fast = p->bank_fast; q.use_th = p->use_th;
-    q.short_len = p->short_len;
-    q.sm = fused_smem(p, threads);
-    q.first_occ = dict ? p->d_dict_first_occ : p->d_first_occ; q.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16;
-    q.vinfo = p->d_vinfo; q.first_def_instr = p->d_first_def_instr; q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg;
-    q.entry_instr = dict ? p->d_dict_instr : nullptr; q.ndefs = p->d_ndefs; q.opflags = p->d_opflags;
-    q.vcons = p->d_vcons; q.rs_prefix = p->d_rs_prefix; q.bank_list = p->d_bank_list;
-    for (int j = 0; j < 4; ++j) q.bank_seg[j] = p->bank_seg[j];
-    q.th_off = p->d_th_off; q.th = p->d_th; q.blk_th = p->d_blk_th; q.sev_off = p->d_sev_off; q.sev = p->d_sev;
-    q.sen_off = p->d_sen_off; q.sen = p->d_sen;
-    q.short_blk = p->d_short_blk; q.short_i0 = p->d_short_i0; q.blk_short_off = p->d_blk_short_off;
-    q.ls = p->d_ls; q.irec = p->d_irec; q.blk_off = p->d_blk_off;
-    q.el = p->d_el; q.el_count = p->d_el_count;
-    q.cand = d_cand; q.pitch = pitch; q.out = d_out;
-    const int rc = vl_live_join(p, st);
-    if (rc != VL_OK) return rc;
-    if (threads == 512) k_fused<512><<<(uint32_t)K, 512, q.sm.total, st>>>(q);
-    else k_fused<256><<<(uint32_t)K, 256, q.sm.total, st>>>(q);
-    VL_CUDA(p, cudaGetLastError());
+    uint64_t resident = 0, rows = 0;
+    uint32_t smem = 0;
+    const uint32_t threads = n > 1 ? 256u : fused_plan(p0, K[0], &resident);
+    FMany<VL_FUSED_MANY> many;
+    for (uint32_t j = 0; j < n; ++j) {
+        vl_program *p = progs[j];
+        FParams &q = many.p[j];
+        q = FParams{};
+        q.nI = p->nI; q.V = p->V; q.nO = dict ? p->nD : p->nO; q.P = p->P; q.B = p->B; q.nB = p->nB; q.nS = p->nS; q.Wv = p->Wv;
+        q.Wp = (p->P + p->wmax + 31) / 32; q.R = p->P + p->wmax + 2; q.wmax = p->wmax;
+        q.bank_fast = p->bank_fast; q.use_th = p->use_th;
+        q.short_len = p->short_len;
+        q.sm = fused_smem(p, threads);
+        smem = std::max(smem, q.sm.total);
+        q.first_occ = dict ? p->d_dict_first_occ : p->d_first_occ; q.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16;
+        q.vinfo = p->d_vinfo; q.first_def_instr = p->d_first_def_instr; q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg;
+        q.entry_instr = dict ? p->d_dict_instr : nullptr; q.ndefs = p->d_ndefs; q.opflags = p->d_opflags;
+        q.vcons = p->d_vcons; q.rs_prefix = p->d_rs_prefix; q.bank_list = p->d_bank_list;
+        for (int c = 0; c < 4; ++c) q.bank_seg[c] = p->bank_seg[c];
+        q.th_off = p->d_th_off; q.th = p->d_th; q.blk_th = p->d_blk_th; q.sev_off = p->d_sev_off; q.sev = p->d_sev;
+        q.sen_off = p->d_sen_off; q.sen = p->d_sen;
+        q.short_blk = p->d_short_blk; q.short_i0 = p->d_short_i0; q.blk_short_off = p->d_blk_short_off;
+        q.ls = p->d_ls; q.irec = p->d_irec; q.blk_off = p->d_blk_off;
+        q.el = p->d_el; q.el_count = p->d_el_count;
+        q.cand = d_cand[j]; q.K = K[j]; q.pitch = pitch[j]; q.out = d_out[j];
+        rows = std::max(rows, K[j]);
+        const int rc = vl_live_join(p, st);
+        if (rc != VL_OK) return rc;
+    }
+    if (n > 1) {
+        k_fused<256, VL_FUSED_MANY><<<dim3((uint32_t)rows, n), 256, smem, st>>>(many);
+    } else {
+        FMany<1> one;
+        one.p[0] = many.p[0];
+        if (threads == 512) k_fused<512, 1><<<(uint32_t)rows, 512, smem, st>>>(one);
+        else k_fused<256, 1><<<(uint32_t)rows, 256, smem, st>>>(one);
+    }
+    VL_CUDA(p0, cudaGetLastError());
     g_vl_launches.fetch_add(1);
     return VL_OK;
+}
+
+// Whether a job may share a launch with jobs of other programs: blocks of 256 threads, small enough that several
+// share a multiprocessor whatever the others need.
+bool vl_fused_shares(vl_program *p, uint64_t K)
+{
+    return vl_fused_wanted(p, K) && fused_smem(p, 256).total <= 48 * 1024;
 }

@@ -220,9 +220,13 @@ extern std::atomic<uint64_t> g_vl_launches;
     } while (0)
 
 int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, const cudaEvent_t *done, uint32_t n_streams);
-// The one-kernel verify path of short jobs (vl_fused.cu): whether a job of K rows takes it; one launch on st.
+// The one-kernel verify path of short jobs (vl_fused.cu): whether a job of K rows takes it, whether it may share a
+// launch with other programs' jobs, and one launch for n <= VL_FUSED_MANY jobs.
+#define VL_FUSED_MANY 48
 bool vl_fused_wanted(vl_program *p, uint64_t K);
-int vl_fused_run(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict);
+bool vl_fused_shares(vl_program *p, uint64_t K);
+int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
+                 vl_verdict *const *d_out, cudaStream_t st, bool dict);
 int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out,
                    cudaStream_t st, int slot, bool dict = false);
 int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K,

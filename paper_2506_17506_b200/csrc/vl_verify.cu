@@ -2433,7 +2433,7 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
 {
     if (vl_fused_wanted(p, K)) {
         kt_mark(p, st);
-        const int rf = vl_fused_run(p, d_cand, K, pitch, d_out, st, dict);
+        const int rf = vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, dict);
         for (int j = 0; j < 4; ++j) kt_mark(p, st);
         return rf;
     }
@@ -2447,6 +2447,28 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
     }
     return VL_OK;
 }
+
+namespace {
+// Short jobs collected for one launch.
+struct FusedGroup {
+    uint32_t n = 0;
+    vl_program *progs[VL_FUSED_MANY];
+    const uint16_t *cand[VL_FUSED_MANY];
+    uint64_t K[VL_FUSED_MANY], pitch[VL_FUSED_MANY];
+    vl_verdict *out[VL_FUSED_MANY];
+    bool add(vl_program *p, const uint16_t *c, uint64_t k, uint64_t pt, vl_verdict *o)  // true: full
+    {
+        progs[n] = p; cand[n] = c; K[n] = k; pitch[n] = pt; out[n] = o;
+        return ++n == VL_FUSED_MANY;
+    }
+    int run(cudaStream_t st, bool dict)
+    {
+        const uint32_t m = n;
+        n = 0;
+        return vl_fused_run(m, progs, cand, K, pitch, out, st, dict);
+    }
+};
+}  // namespace
 
 // Passes of one or several programs spread round-robin over the device's lane streams, so that
 // the table kernel of one pass (bound by the row stream) runs beside the walk of another (bound by
@@ -2464,21 +2486,36 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     uint64_t jobs = 0;
     for (uint32_t j = 0; j < nprog; ++j) jobs += (K[j] + progs[j]->sub_batch - 1) / progs[j]->sub_batch;
     if (L == 1 || jobs <= 1) {
+        FusedGroup g;
         for (uint32_t j = 0; j < nprog; ++j) {
             if (K[j] == 0) continue;
+            if (nprog > 1 && vl_fused_shares(progs[j], K[j])) {
+                if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j]) && (rc = g.run(st, dict)) != VL_OK) return rc;
+                continue;
+            }
             rc = vl_verify_impl(progs[j], d_cand[j], K[j], pitch[j], d_out[j], st, 0, dict);
             if (rc != VL_OK) return rc;
         }
-        return VL_OK;
+        return g.n ? g.run(st, dict) : VL_OK;
     }
     VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
     for (uint32_t l = 0; l < L; ++l) VL_CUDA(p0, cudaStreamWaitEvent(lane[l], p0->ev_fork, 0));
     uint64_t job = 0;
+    // short jobs of different programs share launches (64 programs of one call: 2 launches instead of 64)
+    std::vector<uint8_t> shared(nprog, 0);
+    FusedGroup g;
+    for (uint32_t j = 0; j < nprog && nprog > 1 && rc == VL_OK; ++j) {
+        if (K[j] == 0 || !vl_fused_shares(progs[j], K[j])) continue;
+        shared[j] = 1;
+        if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j])) rc = g.run(lane[job++ % L], dict);
+    }
+    if (rc == VL_OK && g.n) rc = g.run(lane[job++ % L], dict);
     for (uint32_t j = 0; j < nprog && rc == VL_OK; ++j) {
         if (K[j] == 0) continue;
         vl_program *p = progs[j];
+        if (shared[j]) continue;
         if (vl_fused_wanted(p, K[j])) {
-            rc = vl_fused_run(p, d_cand[j], K[j], pitch[j], d_out[j], lane[job % L], dict);
+            rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, lane[job % L], dict);
             ++job;
             continue;
         }
