@@ -100,8 +100,11 @@ __device__ __forceinline__ uint32_t bank_entry(const uint2 &id, uint32_t n, cons
     return n == 2 ? bank_extra<2>(x, bmask) : (n == 3 ? bank_extra<3>(x, bmask) : bank_extra<4>(x, bmask));
 }
 
-template <int NTHR, int N>
-__global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const __grid_constant__ FMany<N> a)
+// BPM: thread blocks per multiprocessor that the registers have to leave room for.  One or two rows per multiprocessor are
+// bound by latency (registers for loads in flight), more rows by how many warps there are to switch between: 6,400 rows of
+// 64 programs 345 us with two blocks of 256 threads, 281 with three, 274 with four (but spills: one row 20 % slower).
+template <int NTHR, int BPM, int N>
+__global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMany<N> a)
 {
     const FParams &q = a.p[N == 1 ? 0 : blockIdx.y];
     if (N > 1 && blockIdx.x >= q.K) return;
@@ -551,18 +554,21 @@ __global__ void __launch_bounds__(NTHR, 512 / NTHR) k_fused(const __grid_constan
     }
 }
 
-// Threads per block for a job of K rows (0 if the program does not fit the kernel) and how many such blocks the device
-// holds at a time.  Up to one row per multiprocessor a block takes a whole one; for more rows two blocks share one,
-// where their masks let them (a program of 8,000 instructions: 16.6 us for 148 rows, 38 us for 300).
-uint32_t fused_plan(vl_program *p, uint64_t K, uint64_t *resident)
+// How a job of K rows runs: threads per block (0: the program does not fit the kernel), blocks per multiprocessor.  Up to
+// one row per multiprocessor a block takes a whole one; for more rows two or three blocks share one, where their masks let
+// them (a program of 8,000 instructions: 16.6 us for 148 rows, 38 us for 300).
+struct FPlan {
+    uint32_t threads, bpm;
+};
+FPlan fused_plan(vl_program *p, uint64_t K)
 {
     const uint32_t cap = 227 * 1024;
     const uint64_t sms = (uint64_t)vl_sm_count(p);
-    if (p->nS > 65535u) return 0;
+    if (p->nS > 65535u) return {0, 0};
     const uint32_t half = fused_smem(p, 256).total, full = fused_smem(p, 512).total;
-    if (K > sms && 2 * (half + 1024) <= cap) { *resident = 2 * sms; return 256; }
-    *resident = sms;
-    return full <= cap ? 512u : (half <= cap ? 256u : 0u);
+    if (K > 2 * sms && 3 * (half + 1024) <= cap) return {256, 3};
+    if (K > sms && 2 * (half + 1024) <= cap) return {256, 2};
+    return {full <= cap ? 512u : (half <= cap ? 256u : 0u), 1};
 }
 
 }  // namespace
@@ -576,8 +582,9 @@ bool vl_fused_wanted(vl_program *p, uint64_t K)
 {
     if (p->group_opt || p->threads_opt || p->test_wait) return false;  // the caller asks for the batched kernels
     if (p->P + p->wmax > 32768u) return false;                         // (not a program the verify path takes)
-    uint64_t resident = 0;
-    if (!fused_plan(p, K, &resident)) return false;
+    const FPlan pl = fused_plan(p, K);
+    if (!pl.threads) return false;
+    const uint64_t resident = (uint64_t)pl.bpm * vl_sm_count(p);
     const uint64_t rounds = (K + resident - 1) / resident;
     return rounds <= 1 || rounds * (6000 + 7ull * p->nI) <= 72000;
 }
@@ -593,15 +600,16 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         std::lock_guard<std::mutex> lock(mtx);
         if (!done[p0->device]) {
             const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 1>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<512, 1>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, VL_FUSED_MANY>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<512, 1, 1>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 2, 1>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 3, 1>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 3, VL_FUSED_MANY>, at, 227 * 1024));
             done[p0->device] = true;
         }
     }
-    uint64_t resident = 0, rows = 0;
+    uint64_t rows = 0;
     uint32_t smem = 0;
-    const uint32_t threads = n > 1 ? 256u : fused_plan(p0, K[0], &resident);
+    const FPlan pl = n > 1 ? FPlan{256, 3} : fused_plan(p0, K[0]);
     FMany<VL_FUSED_MANY> many;
     for (uint32_t j = 0; j < n; ++j) {
         vl_program *p = progs[j];
@@ -611,7 +619,7 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         q.Wp = (p->P + p->wmax + 31) / 32; q.R = p->P + p->wmax + 2; q.wmax = p->wmax;
         q.bank_fast = p->bank_fast; q.use_th = p->use_th;
         q.short_len = p->short_len;
-        q.sm = fused_smem(p, threads);
+        q.sm = fused_smem(p, pl.threads);
         smem = std::max(smem, q.sm.total);
         q.first_occ = dict ? p->d_dict_first_occ : p->d_first_occ; q.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16;
         q.vinfo = p->d_vinfo; q.first_def_instr = p->d_first_def_instr; q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg;
@@ -629,12 +637,13 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         if (rc != VL_OK) return rc;
     }
     if (n > 1) {
-        k_fused<256, VL_FUSED_MANY><<<dim3((uint32_t)rows, n), 256, smem, st>>>(many);
+        k_fused<256, 3, VL_FUSED_MANY><<<dim3((uint32_t)rows, n), 256, smem, st>>>(many);
     } else {
         FMany<1> one;
         one.p[0] = many.p[0];
-        if (threads == 512) k_fused<512, 1><<<(uint32_t)rows, 512, smem, st>>>(one);
-        else k_fused<256, 1><<<(uint32_t)rows, 256, smem, st>>>(one);
+        if (pl.threads == 512) k_fused<512, 1, 1><<<(uint32_t)rows, 512, smem, st>>>(one);
+        else if (pl.bpm == 3) k_fused<256, 3, 1><<<(uint32_t)rows, 256, smem, st>>>(one);
+        else k_fused<256, 2, 1><<<(uint32_t)rows, 256, smem, st>>>(one);
     }
     VL_CUDA(p0, cudaGetLastError());
     g_vl_launches.fetch_add(1);
