@@ -245,7 +245,7 @@ extern "C" void vl_program_destroy(vl_program *p)
     cudaFree(p->d_dict_vreg16); cudaFree(p->d_dict_slotmeta); cudaFree(p->d_dict_opoff); cudaFree(p->d_dict_first4);
     cudaFree(p->d_dict_instr); cudaFree(p->d_dict_first_occ);
     cudaFree(p->d_vcons); cudaFree(p->d_rs_prefix);
-    for (auto &v : p->vs) { cudaFree(v.tg); cudaFree(v.cstate); cudaFree(v.anom); cudaFree(v.work); cudaFree(v.racc); cudaFree(v.grp_done); cudaFree(v.thm); }
+    for (auto &v : p->vs) { cudaFree(v.tg); cudaFree(v.cstate); cudaFree(v.anom); cudaFree(v.work); cudaFree(v.racc); cudaFree(v.grp_done); cudaFree(v.thm); cudaFree(v.exact); }
     for (int j = 0; j < 2; ++j) {
         cudaFree(p->d_stage[j]);
         cudaFree(p->d_stage_out[j]);

@@ -17,17 +17,20 @@
 
 #include "vl_internal.cuh"
 
+#define EXACT_NT 256
+
 namespace {
 
 struct FMisc {
     uint32_t flags, minop, minr, bank, pairs, mind, thcol, any;
-    uint32_t n_list;
+    uint32_t n_list, dups;
     uint32_t th_off[33];  // (through-sets are used only by programs of at most 32 blocks)
 };
 
 // Where the parts of a block's shared memory start (bytes), and how much there is.
 struct FSmem {
     uint32_t w, th, occ, coll, list, misc, total;
+    uint32_t cb;  // program blocks whose register counts fit the masks' place
 };
 
 inline uint32_t up16(uint32_t x) { return (x + 15u) & ~15u; }
@@ -39,15 +42,17 @@ inline FSmem fused_smem(const vl_program *p, uint32_t threads)
     s.w = up16((p->V + 1) * 2);
     s.th = s.w + up16(p->V + 1);
     s.occ = s.th + (p->use_th ? up16(p->nB * Wp * 4) : 0u);
-    s.coll = s.occ + up16(std::max(Wp * threads * 4, (p->P + p->wmax + 2) * 8));
+    const uint32_t counts = (p->P + p->wmax + 2) * 4;  // (of one program block, see exact_counts)
+    s.coll = s.occ + up16(std::max(Wp * threads * 4, counts));
+    s.cb = p->use_th ? (s.coll - s.occ) / counts : p->nB;
     s.list = s.coll + up16((p->nS + 31) / 32 * 4 + 4);
-    s.misc = s.list + up16(p->nS * 8);
+    s.misc = s.list + p->nS * 16;
     s.total = s.misc + up16(sizeof(FMisc));
     return s;
 }
 
 struct FParams {
-    uint32_t nI, V, nO, P, B, nB, nS, Wp, R, Wv, wmax, short_len;
+    uint32_t nI, V, nO, P, B, nB, nS, Wp, R, Wv, wmax, short_len, cb;
     int bank_fast, use_th;
     FSmem sm;
     const uint32_t *first_occ, *vinfo, *first_def_instr, *op_off, *op_vreg, *entry_instr, *blk_off;
@@ -65,6 +70,7 @@ struct FParams {
     const uint16_t *cand;
     uint64_t K, pitch;
     vl_verdict *out;
+    VlExactArgs ex;  // (k_exact)
 };
 
 // The jobs of up to N programs in one grid: blockIdx.y is the program.
@@ -100,6 +106,332 @@ __device__ __forceinline__ uint32_t bank_entry(const uint2 &id, uint32_t n, cons
     return n == 2 ? bank_extra<2>(x, bmask) : (n == 3 ? bank_extra<3>(x, bmask) : bank_extra<4>(x, bmask));
 }
 
+// The same for instruction i of a program without a list (banks not 1, 2 or 4, or more than four distinct sources).
+__device__ __forceinline__ uint32_t bank_instr(const FParams &q, const uint16_t *T, uint32_t i)
+{
+    uint32_t n = 0;
+    const uint32_t u0 = q.op_off[i] + q.ndefs[i], u1 = q.op_off[i + 1];
+    for (uint32_t a = u0 + 1; a < u1; ++a) {
+        const uint32_t xa = T[q.op_vreg[a]];
+        bool value = false, bank = false;
+        for (uint32_t b = u0; b < a; ++b) {
+            const uint32_t xb = T[q.op_vreg[b]];
+            value |= xb == xa;
+            bank |= xb % q.B == xa % q.B;
+        }
+        n += !value && bank;
+    }
+    return n;
+}
+
+// Sources (up to four reads, vreg ids; repeats of a vreg do not count) that hold the register of an earlier source.
+__device__ __forceinline__ uint32_t duplicates(const uint32_t (&rd)[4], const uint16_t *T)
+{
+    uint32_t t[4], n = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) t[a] = T[rd[a]];
+#pragma unroll
+    for (int a = 1; a < 4; ++a) {
+        bool again = false, same = false;
+#pragma unroll
+        for (int c = 0; c < a; ++c) {
+            again |= rd[c] == rd[a];
+            same |= t[c] == t[a];
+        }
+        n += !again && same;
+    }
+    return n;
+}
+// The same for the read at operand a of an instruction whose reads begin at r0.
+__device__ __forceinline__ uint32_t duplicate_of(const FParams &q, const uint16_t *T, uint32_t r0, uint32_t a)
+{
+    const uint32_t v = q.op_vreg[a], t = T[v];
+    bool again = false, same = false;
+    for (uint32_t c = r0; c < a; ++c) {
+        const uint32_t u = q.op_vreg[c];
+        again |= u == v;
+        same |= T[u] == t;
+    }
+    return !again && same;
+}
+
+// Sources of instruction i in the through-set of block b that hold the register of an earlier source, where an earlier
+// source in the through-set holds it too.
+__device__ __noinline__ uint32_t member_duplicates(const FParams &q, const uint16_t *T, uint32_t b, uint32_t i)
+{
+    uint32_t n = 0;
+    const uint32_t *th = q.blk_th + (size_t)b * q.Wv;
+    const uint32_t r0 = q.op_off[i] + q.ndefs[i], r1 = q.op_off[i + 1];
+    for (uint32_t a = r0 + 1; a < r1; ++a) {
+        const uint32_t v = q.op_vreg[a];
+        if (!((th[v >> 5] >> (v & 31)) & 1u)) continue;
+        bool again = false, same = false;
+        for (uint32_t c = r0; c < a; ++c) {
+            const uint32_t u = q.op_vreg[c];
+            again |= u == v;
+            same |= ((th[u >> 5] >> (u & 31)) & 1u) && T[u] == T[v];
+        }
+        n += !again && same;
+    }
+    return n;
+}
+
+// Step 5: the overlaps in the short chunks marked in coll and, for program blocks whose through-set collided, those of the
+// definitions without an event, counted exactly; added to M->pairs and M->mind.  With several parts, this block's share.
+// The program blocks are taken q.cb at a time (all at once, as a rule: going block by block, the chain of L2 round trips
+// in front of the first count took 2 us for each).  cv: [cb][R] words; list: room for nS spans.
+// LISTED (k_exact): the bank tally of the table kernel (sources minus banks touched, per instruction) counts a register
+// that two source vregs share twice; M->dups receives the number of such sources.  Two sources of an instruction are live
+// together in front of it: if they hold the same register, its chunk has collided, or they are both in a through-set that
+// has.  And T, W hold nothing yet: what the share needs is fetched here (a hundredth of the vregs, for a row with one
+// misplaced vreg; fetching all 10,000 took 30 us).
+template <int NTHR, bool LISTED>
+__device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint8_t *W, uint32_t *cv, const uint32_t *coll,
+                                             uint4 *list, FMisc *M, uint32_t part, uint32_t parts, const uint16_t *row)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    uint32_t pairs = 0, mind = 0xFFFFFFFFu, dups = 0;
+    for (uint32_t b0 = 0; b0 < q.nB; b0 += q.cb) {
+        const uint32_t b1 = min(b0 + q.cb, q.nB);
+        const uint32_t s_lo = b0 ? q.blk_short_off[b0] : 0u, s_hi = b1 < q.nB ? q.blk_short_off[b1] : q.nS;
+        const uint32_t thcol = q.use_th ? M->thcol : 0u;
+        if (tid == 0) M->n_list = 0;
+        // The through-sets, counted into arrays over the registers: cv[r] = members whose range holds r, plus 65536 for
+        // each member whose range starts at r; a range [s, s+w) overlaps (members that hold s) + (members that start at
+        // s+1 .. s+w-1).  Members that reach beyond the arrays lie beyond the file: they are compared one by one, with
+        // definitions that lie there too.
+        if (q.use_th)
+            for (uint32_t r = tid; r < (b1 - b0) * q.R; r += NTHR) cv[r] = 0;
+        __syncthreads();
+        for (uint32_t s = s_lo + tid; s < s_hi; s += NTHR)
+            if (((coll[s >> 5] >> (s & 31)) & 1u) && s % parts == part) {
+                const uint32_t i0 = q.short_i0[s], b = q.use_th ? q.short_blk[s] - b0 : 0u;
+                list[atomicAdd(&M->n_list, 1u)] = make_uint4(i0, (q.short_i0[s + 1] - i0) | (b << 20), s, 0u);
+            }
+        if (LISTED) {
+            __syncthreads();
+            const uint32_t n_list = M->n_list, n_th = q.use_th ? M->th_off[b1] - M->th_off[b0] : 0u, th0 = q.use_th ? M->th_off[b0] : 0u;
+            constexpr int FU = 6;
+            // T and W of the n vregs that of(0 .. n - 1) names, by threads first, first + step, ...
+            auto fetch = [&](uint32_t n, uint32_t first, uint32_t step, auto of) {
+                for (uint32_t j0 = first; j0 < n; j0 += FU * step) {
+                    uint32_t v[FU], pos[FU], w[FU], t[FU];
+#pragma unroll
+                    for (int u = 0; u < FU; ++u) v[u] = of(min(j0 + u * step, n - 1));
+#pragma unroll
+                    for (int u = 0; u < FU; ++u) { pos[u] = q.first_occ[v[u]]; w[u] = q.vinfo[v[u]]; }
+#pragma unroll
+                    for (int u = 0; u < FU; ++u) t[u] = row[pos[u] != 0xFFFFFFFFu ? pos[u] : 0u];
+#pragma unroll
+                    for (int u = 0; u < FU; ++u) {  // (several threads may store the same value)
+                        T[v[u]] = pos[u] != 0xFFFFFFFFu ? (uint16_t)t[u] : (uint16_t)0;
+                        W[v[u]] = (uint8_t)w[u];
+                    }
+                }
+            };
+            if (n_list * q.short_len * 4 >= q.V) {
+                fetch(q.V, tid, NTHR, [](uint32_t j) { return j; });
+            } else {
+                fetch(n_th, tid, NTHR, [&](uint32_t j) { return q.th[th0 + j] & 0xFFFFu; });
+                // what is occupied when the short chunk begins, and its operands: a warp takes a short chunk
+                for (uint32_t l = tid >> 5; l < n_list; l += NTHR / 32) {
+                    const uint4 x = list[l];
+                    const uint32_t e0 = q.sen_off[x.z], e1 = q.sen_off[x.z + 1], o0 = q.op_off[x.x], o1 = q.op_off[x.x + (x.y & 0xFFFFFu)];
+                    fetch(e1 - e0, lane, 32, [&](uint32_t j) { return q.sen[e0 + j] & 0xFFFFu; });
+                    fetch(o1 - o0, lane, 32, [&](uint32_t j) { return q.op_vreg[o0 + j]; });
+                }
+            }
+            if (tid == 0) { T[q.V] = 0; W[q.V] = 0; }
+            __syncthreads();
+        }
+        if (q.use_th)
+            for (uint32_t j = M->th_off[b0] + tid; j < M->th_off[b1]; j += NTHR) {
+                const uint32_t v = q.th[j] & 0xFFFFu, reg = T[v], w = W[v];
+                uint32_t b = b0;
+                while (b + 1 < b1 && M->th_off[b + 1] <= j) ++b;
+                if (reg + w <= q.R) {
+                    uint32_t *c = cv + (b - b0) * q.R + reg;
+                    atomicAdd(c, 0x10001u);
+                    for (uint32_t r = 1; r < w; ++r) atomicAdd(c + r, 1u);
+                }
+            }
+        __syncthreads();
+        const uint32_t n_list = M->n_list;
+        // through-set members of block b other than v (itself a member: `member`) that overlap v's range
+        auto through_overlaps = [&](uint32_t b, uint32_t v, bool member) {
+            const uint32_t s = T[v], w = W[v];
+            uint32_t n = 0;
+            if (!q.use_th) return n;
+            const uint32_t *c = cv + (b - b0) * q.R;
+            if (s < q.R) {
+                n = (c[s] & 0xFFFFu) - (member && s + w <= q.R ? 1u : 0u);
+                for (uint32_t r = s + 1; r < min(s + w, q.R); ++r) n += c[r] >> 16;
+            }
+            if (s + w > q.P)
+                for (uint32_t j = M->th_off[b]; j < M->th_off[b + 1]; ++j) {
+                    const uint32_t u = q.th[j] & 0xFFFFu;
+                    if (u != v && T[u] + W[u] > q.R && overlap(s, w, T[u], W[u])) ++n;
+                }
+            return n;
+        };
+        // A thread takes an instruction: the entries of its live-after list that are not in the through-set, the
+        // through-set from the arrays.  The record of the instruction after the next and the first list entries
+        // of the next are fetched meanwhile.  (Bound by instruction issue: the lists of loop bodies hold 4 to 10
+        // entries, and few of them sit near enough to be looked at more closely.)
+        constexpr int LU = 8, LT = 16;  // list entries in flight: the first of a list, the others
+        const uint32_t step_unit = NTHR / q.short_len, step_at = NTHR % q.short_len;
+        uint32_t unit = tid / q.short_len, at = tid % q.short_len;  // (advances by NTHR instructions)
+        auto next_instr = [&](uint32_t &b) -> uint32_t {  // 0xFFFFFFFF: beyond the short chunk, or beyond the list
+            uint32_t i = 0xFFFFFFFFu;
+            if (unit < n_list) {
+                const uint4 span = list[unit];
+                if (at < (span.y & 0xFFFFFu)) i = span.x + at;
+                b = b0 + (span.y >> 20);
+            }
+            unit += step_unit;
+            at += step_at;
+            if (at >= q.short_len) { at -= q.short_len; ++unit; }
+            return i;
+        };
+        auto fetch_rec = [&](uint32_t i) { return q.irec[min(i, q.nI - 1)]; };  // (looked at only if i is one)
+        uint32_t us_nx[LU], rd_nx[4];
+        auto fetch_list = [&](const uint4 &r) {
+            const uint32_t n = r.y & 0xFFFFu, last = n ? n - 1 : 0u;
+            if (LISTED) {
+                const uint32_t nr = (r.y >> 24) & 127u, o = r.w + ((r.y >> 16) & 0xFFu);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) rd_nx[u] = q.op_vreg[nr ? o + min((uint32_t)u, nr - 1) : 0u];
+            }
+#pragma unroll
+            for (int u = 0; u < LU; ++u) us_nx[u] = q.ls[r.x + min((uint32_t)u, last)];
+        };
+        const uint32_t n_slots = n_list * q.short_len;
+        if (n_slots) {
+            uint32_t b_nx = b0, b_nx2 = b0, i_nx = next_instr(b_nx), i_nx2 = next_instr(b_nx2);
+            uint4 rec_nx = fetch_rec(i_nx), rec_nx2 = fetch_rec(i_nx2);
+            fetch_list(rec_nx);
+            for (uint32_t f = tid; f < n_slots; f += NTHR) {
+                const uint32_t i = i_nx, b = b_nx;
+                const uint4 rec = rec_nx;
+                uint32_t us[LU], ts[LU], rd[4];
+#pragma unroll
+                for (int u = 0; u < LU; ++u) us[u] = us_nx[u];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) rd[u] = LISTED ? rd_nx[u] : 0u;
+                i_nx = i_nx2;
+                b_nx = b_nx2;
+                rec_nx = rec_nx2;
+                fetch_list(rec_nx);
+                i_nx2 = next_instr(b_nx2);
+                rec_nx2 = fetch_rec(i_nx2);
+                const uint32_t n = rec.y & 0xFFFFu, nd = i != 0xFFFFFFFFu ? (rec.y >> 16) & 0xFFu : 0u;
+                if (LISTED && i != 0xFFFFFFFFu) {
+                    const uint32_t nr = (rec.y >> 24) & 127u;
+                    uint32_t n_dup = 0;
+                    if (nr <= 4) {  // (missing reads repeat the last one)
+                        if (nr > 1) n_dup = duplicates(rd, T);
+                    } else {
+                        for (uint32_t a = rec.w + nd; a < q.op_off[i + 1]; ++a) n_dup += duplicate_of(q, T, rec.w + nd, a);
+                    }
+                    // (those of two through-set members are counted with the block's through-set, below)
+                    if (n_dup && ((thcol >> b) & 1u)) n_dup -= member_duplicates(q, T, b, i);
+                    dups += n_dup;
+                }
+                if (!nd) continue;
+                uint32_t cnt = 0;
+#pragma unroll
+                for (int u = 0; u < LU; ++u) ts[u] = T[(uint32_t)u < n ? us[u] : q.V];
+                for (uint32_t d = 0; d < nd; ++d) {
+                    const uint32_t v = d ? q.op_vreg[rec.w + d] : rec.z, sv = T[v], wv = W[v];
+                    // [t, t + wt) overlaps [sv, sv + wv): t < sv + wv and t > sv - wt, wt at most wmax
+                    const uint32_t shift = q.wmax - 1 - sv, span = wv + q.wmax - 1;
+                    cnt += through_overlaps(b, v, d ? (q.blk_th[(size_t)b * q.Wv + (v >> 5)] >> (v & 31)) & 1u : rec.y >> 31);
+                    bool near = false;
+#pragma unroll
+                    for (int u = 0; u < LU; ++u) near |= ts[u] + shift < span;
+                    if (near) {
+#pragma unroll
+                        for (int u = 0; u < LU; ++u)
+                            if ((uint32_t)u < n && us[u] != v && overlap(sv, wv, ts[u], W[us[u]])) ++cnt;
+                    }
+                    for (uint32_t e0 = LU; e0 < n; e0 += LT) {
+                        uint32_t x[LT];
+#pragma unroll
+                        for (int u = 0; u < LT; ++u) x[u] = q.ls[rec.x + min(e0 + u, n - 1)];
+#pragma unroll
+                        for (int u = 0; u < LT; ++u) {
+                            const uint32_t t = T[x[u]];
+                            if (t + shift < span && e0 + u < n && x[u] != v && t + W[x[u]] > sv) ++cnt;
+                        }
+                    }
+                    if (nd > 1)  // co-defined vregs that are not live after the instruction
+                        for (uint32_t d2 = 0; d2 < nd; ++d2) {
+                            if (d2 == d || !(q.opflags[rec.w + d2] & OPF_DEAD)) continue;
+                            const uint32_t x = q.op_vreg[rec.w + d2];
+                            if (overlap(sv, wv, T[x], W[x])) ++cnt;
+                        }
+                }
+                if (cnt) { pairs += cnt; mind = min(mind, i); }
+            }
+        }
+        // In a chunk whose own walk was clean everything that is live is disjoint from the through-set; a
+        // definition without an event (a member redefined from itself) overlaps the members that overlap it.
+        for (uint32_t b = b0; b < b1 && thcol; ++b) {
+            if (!((thcol >> b) & 1u)) continue;
+            const uint32_t n_el = q.el_count[b];
+            const uint4 *el = q.el + q.op_off[q.blk_off[b]];  // instruction, chunk, vreg | member << 31, short chunk
+            for (uint32_t e0 = part * 4 * NTHR + tid; e0 < n_el; e0 += parts * 4 * NTHR) {
+                uint4 x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = el[min(e0 + u * NTHR, n_el - 1)];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (e0 + u * NTHR >= n_el || !(x[u].z >> 31) || ((coll[x[u].w >> 5] >> (x[u].w & 31)) & 1u)) continue;
+                    const uint32_t n = through_overlaps(b, x[u].z & 0xFFFFu, true);
+                    if (n) { pairs += n; mind = min(mind, x[u].x); }
+                }
+            }
+            if (LISTED) {  // sources of its instructions that are both in the through-set
+                const uint32_t i1 = q.blk_off[b + 1];
+                for (uint32_t i0 = q.blk_off[b] + part * 4 * NTHR + tid; i0 < i1; i0 += parts * 4 * NTHR) {
+                    uint4 rec[4];
+                    uint32_t rd[4][4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) rec[u] = q.irec[min(i0 + u * NTHR, i1 - 1)];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t nr = (rec[u].y >> 24) & 127u, o = rec[u].w + ((rec[u].y >> 16) & 0xFFu);
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) rd[u][r] = q.op_vreg[nr ? o + min((uint32_t)r, nr - 1) : 0u];
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t i = i0 + u * NTHR, nr = (rec[u].y >> 24) & 127u;
+                        if (i >= i1 || nr < 2) continue;
+                        if (nr <= 4) {
+                            if (duplicates(rd[u], T)) dups += member_duplicates(q, T, b, i);
+                        } else {
+                            dups += member_duplicates(q, T, b, i);
+                        }
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    pairs = __reduce_add_sync(0xffffffffu, pairs);
+    mind = __reduce_min_sync(0xffffffffu, mind);
+    if (LISTED) {
+        dups = __reduce_add_sync(0xffffffffu, dups);
+        if (lane == 0 && dups) atomicAdd(&M->dups, dups);
+    }
+    if (lane == 0 && pairs) {
+        atomicAdd(&M->pairs, pairs);
+        atomicMin(&M->mind, mind);
+    }
+    __syncthreads();
+}
+
 // BPM: thread blocks per multiprocessor that the registers have to leave room for.  One or two rows per multiprocessor are
 // bound by latency (registers for loads in flight), more rows by how many warps there are to switch between: 6,400 rows of
 // 64 programs 345 us with two blocks of 256 threads, 281 with three, 274 with four (but spills: one row 20 % slower).
@@ -112,9 +444,9 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
     uint16_t *T = reinterpret_cast<uint16_t *>(smem);                 // [V + 1] register of every vreg
     uint8_t *W = smem + q.sm.w;                                       // [V] width
     uint32_t *s_th = reinterpret_cast<uint32_t *>(smem + q.sm.th);    // [nB][Wp] through-set masks
-    uint32_t *occ = reinterpret_cast<uint32_t *>(smem + q.sm.occ);    // [Wp][NTHR] masks; later cover[R], start[R]
+    uint32_t *occ = reinterpret_cast<uint32_t *>(smem + q.sm.occ);    // [Wp][NTHR] masks; counts in step 5
     uint32_t *coll = reinterpret_cast<uint32_t *>(smem + q.sm.coll);  // short chunks that collided
-    uint2 *list = reinterpret_cast<uint2 *>(smem + q.sm.list);        // those of a program block: instructions [x, y)
+    uint4 *list = reinterpret_cast<uint4 *>(smem + q.sm.list);        // the same as a list, in step 5
     FMisc *M = reinterpret_cast<FMisc *>(smem + q.sm.misc);
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t k = blockIdx.x;
@@ -236,19 +568,7 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
             }
         }
         if (!q.bank_fast) {
-            for (uint32_t i = tid; i < q.nI; i += NTHR) {
-                const uint32_t u0 = q.op_off[i] + q.ndefs[i], u1 = q.op_off[i + 1];
-                for (uint32_t a = u0 + 1; a < u1; ++a) {
-                    const uint32_t xa = T[q.op_vreg[a]];
-                    bool value = false, bank = false;
-                    for (uint32_t b = u0; b < a; ++b) {
-                        const uint32_t xb = T[q.op_vreg[b]];
-                        value |= xb == xa;
-                        bank |= xb % q.B == xa % q.B;
-                    }
-                    n += !value && bank;
-                }
-            }
+            for (uint32_t i = tid; i < q.nI; i += NTHR) n += bank_instr(q, T, i);
         }
         n = __reduce_add_sync(0xffffffffu, n);
         if (lane == 0 && n) atomicAdd(&M->bank, n);
@@ -367,157 +687,8 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
     }
     __syncthreads();
 
-    // ---- 5. exact counts where something collided: program block by program block
-    if (M->any | M->thcol) {
-        uint32_t *cover = occ, *start = occ + q.R;
-        uint32_t pairs = 0, mind = 0xFFFFFFFFu;
-        uint32_t s_hi = 0, s_next = q.blk_short_off[1];
-        for (uint32_t b = 0; b < q.nB; ++b) {
-            const uint32_t s_lo = s_hi;
-            s_hi = s_next;
-            s_next = q.blk_short_off[min(b + 2, q.nB)];
-            const bool thcol = q.use_th && ((M->thcol >> b) & 1u);
-            bool any = false;
-            for (uint32_t s = s_lo + tid; s < s_hi; s += NTHR) any |= (coll[s >> 5] >> (s & 31)) & 1u;
-            if (!__syncthreads_or(any) && !thcol) continue;
-            if (tid == 0) M->n_list = 0;
-            __syncthreads();
-            for (uint32_t s = s_lo + tid; s < s_hi; s += NTHR)
-                if ((coll[s >> 5] >> (s & 31)) & 1u) list[atomicAdd(&M->n_list, 1u)] = make_uint2(q.short_i0[s], q.short_i0[s + 1]);
-            // The block's through-set, counted into two arrays over the registers (cover[r]: members whose range holds
-            // r, start[r]: members whose range starts at r): a range [s, s+w) overlaps cover[s] + start[s+1] + ... +
-            // start[s+w-1] of them.  Members that reach beyond the arrays lie beyond the file: they are compared
-            // one by one, with definitions that lie there too.
-            const uint32_t t0 = q.use_th ? M->th_off[b] : 0u, n_th = q.use_th ? M->th_off[b + 1] - t0 : 0u;
-            for (uint32_t r = tid; r < 2 * q.R; r += NTHR) occ[r] = 0;
-            __syncthreads();
-            for (uint32_t j = tid; j < n_th; j += NTHR) {
-                const uint32_t v = q.th[t0 + j] & 0xFFFFu, reg = T[v], w = W[v];
-                if (reg + w <= q.R) {
-                    atomicAdd(&start[reg], 1u);
-                    for (uint32_t r = reg; r < reg + w; ++r) atomicAdd(&cover[r], 1u);
-                }
-            }
-            __syncthreads();
-            const uint32_t n_list = M->n_list;
-            // through-set members other than v (itself a member: `member`) that overlap v's range
-            auto through_overlaps = [&](uint32_t v, bool member) {
-                const uint32_t s = T[v], w = W[v];
-                uint32_t n = 0;
-                if (s < q.R) {
-                    n = cover[s] - (member && s + w <= q.R ? 1u : 0u);
-                    for (uint32_t r = s + 1; r < min(s + w, q.R); ++r) n += start[r];
-                }
-                if (s + w > q.P)
-                    for (uint32_t j = 0; j < n_th; ++j) {
-                        const uint32_t u = q.th[t0 + j] & 0xFFFFu;
-                        if (u != v && T[u] + W[u] > q.R && overlap(s, w, T[u], W[u])) ++n;
-                    }
-                return n;
-            };
-            auto is_member = [&](uint32_t v) { return ((q.blk_th[(size_t)b * q.Wv + (v >> 5)] >> (v & 31)) & 1u) != 0; };
-            // A thread takes an instruction: the entries of its live-after list that are not in the through-set, the
-            // through-set from the arrays.  The record of the instruction after the next and the first list entries
-            // of the next are fetched meanwhile.  (Bound by instruction issue: the lists of loop bodies hold 4 to 10
-            // entries, and few of them sit near enough to be looked at more closely.)
-            constexpr int LU = 8;  // list entries in flight
-            const uint32_t step_unit = NTHR / q.short_len, step_at = NTHR % q.short_len;
-            uint32_t unit = tid / q.short_len, at = tid % q.short_len;  // (advances by NTHR instructions)
-            auto next_instr = [&]() -> uint32_t {  // 0xFFFFFFFF: beyond the short chunk, or beyond the list
-                uint32_t i = 0xFFFFFFFFu;
-                if (unit < n_list) {
-                    const uint2 span = list[unit];
-                    if (span.x + at < span.y) i = span.x + at;
-                }
-                unit += step_unit;
-                at += step_at;
-                if (at >= q.short_len) { at -= q.short_len; ++unit; }
-                return i;
-            };
-            auto fetch_rec = [&](uint32_t i) { return q.irec[min(i, q.nI - 1)]; };  // (looked at only if i is one)
-            uint32_t us_nx[LU];
-            auto fetch_list = [&](const uint4 &r) {
-                const uint32_t n = r.y & 0xFFFFu, last = n ? n - 1 : 0u;
-#pragma unroll
-                for (int u = 0; u < LU; ++u) us_nx[u] = q.ls[r.x + min((uint32_t)u, last)];
-            };
-            uint32_t i_nx = next_instr(), i_nx2 = next_instr();
-            uint4 rec_nx = fetch_rec(i_nx), rec_nx2 = fetch_rec(i_nx2);
-            fetch_list(rec_nx);
-            const uint32_t n_slots = n_list * q.short_len;
-            for (uint32_t f = tid; f < n_slots; f += NTHR) {
-                const uint32_t i = i_nx;
-                const uint4 rec = rec_nx;
-                uint32_t us[LU], ts[LU];
-#pragma unroll
-                for (int u = 0; u < LU; ++u) us[u] = us_nx[u];
-                i_nx = i_nx2;
-                rec_nx = rec_nx2;
-                fetch_list(rec_nx);
-                i_nx2 = next_instr();
-                rec_nx2 = fetch_rec(i_nx2);
-                const uint32_t n = rec.y & 0xFFFFu, nd = i != 0xFFFFFFFFu ? (rec.y >> 16) & 0xFFu : 0u;
-                if (!nd) continue;
-                uint32_t cnt = 0;
-#pragma unroll
-                for (int u = 0; u < LU; ++u) ts[u] = T[(uint32_t)u < n ? us[u] : q.V];
-                for (uint32_t d = 0; d < nd; ++d) {
-                    const uint32_t v = d ? q.op_vreg[rec.w + d] : rec.z, sv = T[v], wv = W[v];
-                    // [t, t + wt) overlaps [sv, sv + wv): t < sv + wv and t > sv - wt, wt at most wmax
-                    const uint32_t shift = q.wmax - 1 - sv, span = wv + q.wmax - 1;
-                    cnt += through_overlaps(v, d ? is_member(v) : rec.y >> 31);
-                    bool near = false;
-#pragma unroll
-                    for (int u = 0; u < LU; ++u) near |= ts[u] + shift < span;
-                    if (near) {
-#pragma unroll
-                        for (int u = 0; u < LU; ++u)
-                            if ((uint32_t)u < n && us[u] != v && overlap(sv, wv, ts[u], W[us[u]])) ++cnt;
-                    }
-                    for (uint32_t e0 = LU; e0 < n; e0 += LU) {
-                        uint32_t x[LU];
-#pragma unroll
-                        for (int u = 0; u < LU; ++u) x[u] = q.ls[rec.x + min(e0 + u, n - 1)];
-#pragma unroll
-                        for (int u = 0; u < LU; ++u)
-                            if (e0 + u < n && x[u] != v && overlap(sv, wv, T[x[u]], W[x[u]])) ++cnt;
-                    }
-                    if (nd > 1)  // co-defined vregs that are not live after the instruction
-                        for (uint32_t d2 = 0; d2 < nd; ++d2) {
-                            if (d2 == d || !(q.opflags[rec.w + d2] & OPF_DEAD)) continue;
-                            const uint32_t x = q.op_vreg[rec.w + d2];
-                            if (overlap(sv, wv, T[x], W[x])) ++cnt;
-                        }
-                }
-                if (cnt) { pairs += cnt; mind = min(mind, i); }
-            }
-            // In a chunk whose own walk was clean everything that is live is disjoint from the through-set; a
-            // definition without an event (a member redefined from itself) overlaps the members that overlap it.
-            if (thcol) {
-                const uint32_t n_el = q.el_count[b];
-                const uint4 *el = q.el + q.op_off[q.blk_off[b]];  // instruction, chunk, vreg | member << 31, short chunk
-                for (uint32_t e0 = tid; e0 < n_el; e0 += 4 * NTHR) {
-                    uint4 x[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) x[u] = el[min(e0 + u * NTHR, n_el - 1)];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (e0 + u * NTHR >= n_el || !(x[u].z >> 31) || ((coll[x[u].w >> 5] >> (x[u].w & 31)) & 1u)) continue;
-                        const uint32_t n = through_overlaps(x[u].z & 0xFFFFu, true);
-                        if (n) { pairs += n; mind = min(mind, x[u].x); }
-                    }
-                }
-            }
-            __syncthreads();
-        }
-        pairs = __reduce_add_sync(0xffffffffu, pairs);
-        mind = __reduce_min_sync(0xffffffffu, mind);
-        if (lane == 0 && pairs) {
-            atomicAdd(&M->pairs, pairs);
-            atomicMin(&M->mind, mind);
-        }
-        __syncthreads();
-    }
+    // ---- 5. exact counts where something collided
+    if (M->any | M->thcol) exact_counts<NTHR, false>(q, T, W, occ, coll, list, M, 0, 1, row);
 
     // ---- the verdict
     if (warp == 0) {
@@ -554,6 +725,92 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
     }
 }
 
+// Candidates of the batched kernels that need an exact count (their walk collided, several of their vregs lie outside the
+// file, or the program has no fast bank tally), listed in work as items of one or several parts per candidate; a thread
+// block takes an item.  Consistency and Realizability are in cstate; a chunk of the walk that collided marks all of its
+// short chunks.  GLOBAL: the block's arrays lie in a slice of global memory (programs that do not fit a multiprocessor).
+template <bool GLOBAL>
+__global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ FParams q)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ FMisc misc;
+    FMisc *M = &misc;
+    unsigned char *base = GLOBAL ? q.ex.scratch + (size_t)blockIdx.x * q.sm.total : smem;
+    uint16_t *T = reinterpret_cast<uint16_t *>(base);
+    uint8_t *W = base + q.sm.w;
+    uint32_t *occ = reinterpret_cast<uint32_t *>(base + q.sm.occ), *coll = reinterpret_cast<uint32_t *>(base + q.sm.coll);
+    uint4 *list = reinterpret_cast<uint4 *>(base + q.sm.list);
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t n_items = q.ex.work[0];
+    for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
+        const uint64_t k = q.ex.work[EXACT_HDR + 2 * it];
+        const uint32_t part = q.ex.work[EXACT_HDR + 2 * it + 1] & 0xFFu, parts = q.ex.work[EXACT_HDR + 2 * it + 1] >> 8;
+        const uint16_t *row = q.cand + k * q.pitch;
+        const uint32_t *cs = q.ex.cstate + k * 8;
+        const uint32_t walk = cs[CS_WALK], thcol = cs[CS_THCOL];
+        const bool full = walk & WALK_FULL;
+        __syncthreads();
+        if (tid == 0) {
+            M->bank = M->pairs = M->dups = 0;
+            M->thcol = full ? 0u : thcol;  // (with every chunk counted in full, nothing is left of the through-sets)
+            M->mind = 0xFFFFFFFFu;
+        }
+        if (tid <= 32) M->th_off[tid] = q.use_th ? q.th_off[min(tid, q.nB)] : 0u;
+        const bool count = (walk | thcol) != 0;
+        if (count)
+            for (uint32_t s = tid; s < ((q.nS + 31u) & ~31u); s += EXACT_NT) {
+                const uint32_t c = q.ex.short_chunk[min(s, q.nS - 1)];
+                const bool hit = s < q.nS && (full || ((q.ex.anom[k * q.ex.AW + (c >> 5)] >> (c & 31)) & 1u));
+                const uint32_t bits = __ballot_sync(0xffffffffu, hit);
+                if (lane == 0) coll[s >> 5] = bits;
+            }
+        __syncthreads();
+        if (count) exact_counts<EXACT_NT, true>(q, T, W, occ, coll, list, M, part, parts, row);
+        __syncthreads();
+        if (q.bank_fast) {
+            if (tid == 0) M->bank = (part == 0 ? cs[CS_BANK] : 0u) - M->dups;
+        } else {  // the general tally: the whole table, this part's instructions
+            for (uint32_t v = tid; v < q.V; v += EXACT_NT) {
+                const uint32_t pos = q.first_occ[v];
+                T[v] = pos != 0xFFFFFFFFu ? row[pos] : (uint16_t)0;
+            }
+            __syncthreads();
+            uint32_t n = 0;
+            const uint32_t i1 = (uint32_t)((uint64_t)q.nI * (part + 1) / parts);
+            for (uint32_t i = (uint32_t)((uint64_t)q.nI * part / parts) + tid; i < i1; i += EXACT_NT) n += bank_instr(q, T, i);
+            n = __reduce_add_sync(0xffffffffu, n);
+            if (lane == 0 && n) atomicAdd(&M->bank, n);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t pairs = M->pairs, mind = M->mind, bank = M->bank;
+            bool last = true;
+            if (parts > 1) {  // accumulators start at 0: the complement of the lowest instruction
+                uint32_t *acc = q.ex.racc + k * 4;
+                if (pairs) { atomicAdd(&acc[0], pairs); atomicMax(&acc[1], ~mind); }
+                if (bank) atomicAdd(&acc[2], bank);
+                __threadfence();
+                last = atomicAdd(&acc[3], 1u) == parts - 1;
+                if (last) {
+                    __threadfence();
+                    pairs = atomicAdd(&acc[0], 0u);
+                    mind = ~atomicMax(&acc[1], 0u);
+                    bank = atomicAdd(&acc[2], 0u);
+                }
+            }
+            if (last) {
+                const uint32_t flags = cs[CS_FLAGS] | (pairs ? (uint32_t)VL_INTERFERENCE : 0u), first = min(cs[CS_FIRST], mind);
+                vl_verdict vd;
+                vd.flags = flags ? flags : (uint32_t)VL_PASS;
+                vd.first_violation_instr = first == 0xFFFFFFFFu ? -1 : (int32_t)first;
+                vd.conflict_pairs = pairs;
+                vd.bank_conflicts = bank;
+                q.out[k] = vd;
+            }
+        }
+    }
+}
+
 // How a job of K rows runs: threads per block (0: the program does not fit the kernel), blocks per multiprocessor.  Up to
 // one row per multiprocessor a block takes a whole one; for more rows two or three blocks share one, where their masks let
 // them (a program of 8,000 instructions: 16.6 us for 148 rows, 38 us for 300).
@@ -569,6 +826,27 @@ FPlan fused_plan(vl_program *p, uint64_t K)
     if (K > 2 * sms && 3 * (half + 1024) <= cap) return {256, 3};
     if (K > sms && 2 * (half + 1024) <= cap) return {256, 2};
     return {full <= cap ? 512u : (half <= cap ? 256u : 0u), 1};
+}
+
+// What the kernels of this file read of a program.
+FParams fused_params(const vl_program *p, bool dict)
+{
+    FParams q{};
+    q.nI = p->nI; q.V = p->V; q.nO = dict ? p->nD : p->nO; q.P = p->P; q.B = p->B; q.nB = p->nB; q.nS = p->nS; q.Wv = p->Wv;
+    q.Wp = (p->P + p->wmax + 31) / 32; q.R = p->P + p->wmax + 2; q.wmax = p->wmax;
+    q.bank_fast = p->bank_fast; q.use_th = p->use_th;
+    q.short_len = p->short_len;
+    q.first_occ = dict ? p->d_dict_first_occ : p->d_first_occ; q.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16;
+    q.vinfo = p->d_vinfo; q.first_def_instr = p->d_first_def_instr; q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg;
+    q.entry_instr = dict ? p->d_dict_instr : nullptr; q.ndefs = p->d_ndefs; q.opflags = p->d_opflags;
+    q.vcons = p->d_vcons; q.rs_prefix = p->d_rs_prefix; q.bank_list = p->d_bank_list;
+    for (int c = 0; c < 4; ++c) q.bank_seg[c] = p->bank_seg[c];
+    q.th_off = p->d_th_off; q.th = p->d_th; q.blk_th = p->d_blk_th; q.sev_off = p->d_sev_off; q.sev = p->d_sev;
+    q.sen_off = p->d_sen_off; q.sen = p->d_sen;
+    q.short_blk = p->d_short_blk; q.short_i0 = p->d_short_i0; q.blk_short_off = p->d_blk_short_off;
+    q.ls = p->d_ls; q.irec = p->d_irec; q.blk_off = p->d_blk_off;
+    q.el = p->d_el; q.el_count = p->d_el_count;
+    return q;
 }
 
 }  // namespace
@@ -614,23 +892,10 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
     for (uint32_t j = 0; j < n; ++j) {
         vl_program *p = progs[j];
         FParams &q = many.p[j];
-        q = FParams{};
-        q.nI = p->nI; q.V = p->V; q.nO = dict ? p->nD : p->nO; q.P = p->P; q.B = p->B; q.nB = p->nB; q.nS = p->nS; q.Wv = p->Wv;
-        q.Wp = (p->P + p->wmax + 31) / 32; q.R = p->P + p->wmax + 2; q.wmax = p->wmax;
-        q.bank_fast = p->bank_fast; q.use_th = p->use_th;
-        q.short_len = p->short_len;
+        q = fused_params(p, dict);
         q.sm = fused_smem(p, pl.threads);
+        q.cb = q.sm.cb;
         smem = std::max(smem, q.sm.total);
-        q.first_occ = dict ? p->d_dict_first_occ : p->d_first_occ; q.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16;
-        q.vinfo = p->d_vinfo; q.first_def_instr = p->d_first_def_instr; q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg;
-        q.entry_instr = dict ? p->d_dict_instr : nullptr; q.ndefs = p->d_ndefs; q.opflags = p->d_opflags;
-        q.vcons = p->d_vcons; q.rs_prefix = p->d_rs_prefix; q.bank_list = p->d_bank_list;
-        for (int c = 0; c < 4; ++c) q.bank_seg[c] = p->bank_seg[c];
-        q.th_off = p->d_th_off; q.th = p->d_th; q.blk_th = p->d_blk_th; q.sev_off = p->d_sev_off; q.sev = p->d_sev;
-        q.sen_off = p->d_sen_off; q.sen = p->d_sen;
-        q.short_blk = p->d_short_blk; q.short_i0 = p->d_short_i0; q.blk_short_off = p->d_blk_short_off;
-        q.ls = p->d_ls; q.irec = p->d_irec; q.blk_off = p->d_blk_off;
-        q.el = p->d_el; q.el_count = p->d_el_count;
         q.cand = d_cand[j]; q.K = K[j]; q.pitch = pitch[j]; q.out = d_out[j];
         rows = std::max(rows, K[j]);
         const int rc = vl_live_join(p, st);
@@ -655,4 +920,54 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
 bool vl_fused_shares(vl_program *p, uint64_t K)
 {
     return vl_fused_wanted(p, K) && fused_smem(p, 256).total <= 48 * 1024;
+}
+
+// Shared memory of a block of k_exact; beyond what a multiprocessor has, its arrays take global memory.
+static FSmem exact_smem(const vl_program *p)
+{
+    FSmem s{};
+    s.w = up16((p->V + 1) * 2);
+    s.occ = s.w + up16(p->V + 1);
+    const uint32_t counts = (p->P + p->wmax + 2) * 4;
+    s.cb = p->use_th ? std::max(1u, std::min(p->nB, 48u * 1024u / counts)) : p->nB;
+    s.coll = s.occ + (p->use_th ? up16(s.cb * counts) : 0u);
+    s.list = s.coll + up16((p->nS + 31) / 32 * 4 + 4);
+    s.total = s.list + p->nS * 16;
+    return s;
+}
+
+uint32_t vl_exact_blocks(vl_program *p)
+{
+    const uint32_t bytes = exact_smem(p).total;
+    return (uint32_t)vl_sm_count(p) * (bytes <= 110 * 1024 ? 2u : 1u);
+}
+
+uint64_t vl_exact_scratch(vl_program *p)
+{
+    const uint64_t bytes = exact_smem(p).total;
+    return bytes <= 224 * 1024 ? 0 : bytes * vl_exact_blocks(p);
+}
+
+int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict)
+{
+    static std::mutex mtx;
+    static bool done[64];
+    if (p->device >= 0 && p->device < 64) {
+        std::lock_guard<std::mutex> lock(mtx);
+        if (!done[p->device]) {
+            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024));
+            done[p->device] = true;
+        }
+    }
+    FParams q = fused_params(p, dict);
+    q.sm = exact_smem(p);
+    q.cb = q.sm.cb;
+    q.ex = ex;
+    q.cand = d_cand; q.pitch = pitch; q.out = d_out;
+    const uint32_t grid = vl_exact_blocks(p);
+    if (ex.scratch) k_exact<true><<<grid, EXACT_NT, 0, st>>>(q);
+    else k_exact<false><<<grid, EXACT_NT, q.sm.total, st>>>(q);
+    VL_CUDA(p, cudaGetLastError());
+    g_vl_launches.fetch_add(1);
+    return VL_OK;
 }

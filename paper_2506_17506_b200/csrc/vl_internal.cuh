@@ -94,7 +94,7 @@ struct vl_program {
     uint8_t *d_ndefs = nullptr, *d_width = nullptr;
     uint32_t *d_chunk_i0 = nullptr, *d_chunk_i1 = nullptr, *d_chunk_blk = nullptr, *d_blk_chunk_off = nullptr;
     uint32_t *d_piece_i0 = nullptr, *d_piece_chunk = nullptr, *d_chunk_piece_off = nullptr;
-    uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr, *d_short_i0 = nullptr, *d_blk_short_off = nullptr;
+    uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr, *d_short_i0 = nullptr, *d_blk_short_off = nullptr, *d_short_chunk = nullptr;
 
     // liveness results
     uint32_t *d_blk_in = nullptr, *d_blk_out = nullptr, *d_lo_off = nullptr, *d_lo = nullptr;
@@ -126,8 +126,8 @@ struct vl_program {
     uint32_t *d_th_off = nullptr, *d_th = nullptr;  // per block: vregs occupied through the whole block
     // live-after lists without the block's through-set, for the recount: the list of instruction i of
     // block b is ls[lo_off[i] - ls_adj[b] - i * th_cnt[b] ...), |live-after| - th_cnt[b] entries
-    // per instruction, for the exact counts: {first entry of its short list, entries | definitions << 16 | first defined
-    // vreg is in the block's through-set << 31, first defined vreg, first operand}
+    // per instruction, for the exact counts: {first entry of its short list, entries | definitions << 16 | reads (at most
+    // 127) << 24 | first defined vreg is in the block's through-set << 31, first defined vreg, first operand}
     uint4 *d_irec = nullptr;
     uint32_t *d_ls = nullptr, *d_ls_adj = nullptr, *d_th_cnt = nullptr, *d_blk_th = nullptr;
     // definitions without a walk event: {instruction, chunk, vreg | in the block's through-set << 31, short chunk};
@@ -179,8 +179,9 @@ struct vl_program {
         uint16_t *tg = nullptr;      // [groups][V+1][64] tables, 64 candidates side by side
         uint32_t *cstate = nullptr;  // [rows][8]
         uint32_t *anom = nullptr;    // [rows][AW] chunks whose walk collided
-        uint32_t *work = nullptr;    // [1 + rows] count, then candidates that need the exact recount
-        uint32_t *racc = nullptr;    // [rows][4] recount accumulators: pairs, lowest instruction, bank tally, slices done
+        uint32_t *work = nullptr;    // count, then items of the exact count: candidate, part | parts << 8
+        uint32_t *racc = nullptr;    // [rows][4] accumulators of the exact count
+        unsigned char *exact = nullptr;  // block arrays of the exact count that do not fit a multiprocessor
         uint32_t *grp_done = nullptr;  // walk thread blocks that have finished, per group of 64 candidates; then the groups' mark flags
         uint32_t *thm = nullptr;       // [groups][n_blocks][mask words][2][32] through-set masks
         uint64_t rows = 0, aw = 0, vregs = 0, chunks = 0;
@@ -227,6 +228,22 @@ bool vl_fused_wanted(vl_program *p, uint64_t K);
 bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
                  vl_verdict *const *d_out, cudaStream_t st, bool dict);
+// The exact counts of the batched kernels' listed candidates (k_exact, vl_fused.cu).
+#define EXACT_HDR 4        // words in front of the listed items: their number
+#define EXACT_MAX_PARTS 32 // items of one candidate, at most
+#define EXACT_PART_CHUNKS 6 // chunks of the walk that an item counts, about
+// per-candidate state between the kernels (8 words)
+enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_NOUT = 3, CS_OUTV = 4, CS_OUTRAW = 5, CS_WALK = 6, CS_THCOL = 7 };
+enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
+struct VlExactArgs {
+    const uint32_t *work, *cstate, *anom;
+    const uint32_t *short_chunk;  // [nS] chunk of every short chunk
+    uint32_t *racc;               // [rows][4] overlaps, complement of the lowest instruction, bank tally, parts done; all 0
+    uint32_t AW;
+    unsigned char *scratch;       // vl_exact_scratch bytes, null if 0
+};
+uint64_t vl_exact_scratch(vl_program *p);
+int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict);
 int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out,
                    cudaStream_t st, int slot, bool dict = false);
 int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K,

@@ -779,9 +779,10 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
             }
             __syncwarp();
         }
+        const uint32_t n_reads = __shfl_down_sync(0xffffffffu, po.off, 1) - po.off - po.nd;
         if (lane < po.ni)
             q.irec[i0 + lane] = make_uint4(my_lo - ls_sub - (i0 + lane) * ls_mul,
-                                           my_n | (po.nd << 16) | (po.nd && bit_get(s_th, v0) ? 0x80000000u : 0u), v0, po.off);
+                                           my_n | (po.nd << 16) | (min(n_reads, 127u) << 24) | (po.nd && bit_get(s_th, v0) ? 0x80000000u : 0u), v0, po.off);
         return;
     }
     pdl_wait();
@@ -946,7 +947,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     p->nSeg = (uint32_t)seg_c0.size();
     seg_c0.push_back(nC);
     // short chunks: as few pieces as keep their number within SHORT_CHUNKS, equally long inside a chunk
-    std::vector<uint32_t> s_p0, c_s_off(nC + 1, 0), s_blk, s_i0, b_s_off;
+    std::vector<uint32_t> s_p0, c_s_off(nC + 1, 0), s_blk, s_i0, b_s_off, s_chunk;
     for (uint32_t r = std::max(1u, (p->nP + SHORT_CHUNKS - 1) / SHORT_CHUNKS);; ++r) {
         uint64_t total = 0;
         for (uint32_t c = 0; c < nC; ++c) total += (c_p_off[c + 1] - c_p_off[c] + r - 1) / r;
@@ -956,6 +957,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
             for (uint32_t j = 0; j < k; ++j) {
                 s_p0.push_back(c_p_off[c] + (uint32_t)((uint64_t)n * j / k));
                 s_blk.push_back(c_blk[c]);
+                s_chunk.push_back(c);
             }
             c_s_off[c + 1] = (uint32_t)s_p0.size();
         }
@@ -974,7 +976,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
                           {&p->d_chunk_piece_off, &c_p_off}, {&p->d_seg_c0, &seg_c0}, {&p->d_blk_seg_off, &blk_seg_off},
                           {&p->d_short_p0, &s_p0}, {&p->d_chunk_short_off, &c_s_off}, {&p->d_short_blk, &s_blk},
                           {&p->d_short_i0, &s_i0},
-                          {&p->d_blk_short_off, &b_s_off}};
+                          {&p->d_blk_short_off, &b_s_off}, {&p->d_short_chunk, &s_chunk}};
     for (const Part &x : parts) {
         all.insert(all.end(), x.v->begin(), x.v->end());
         all.resize((all.size() + 4) & ~(size_t)3);  // (at least one word behind every array)

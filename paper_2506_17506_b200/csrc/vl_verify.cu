@@ -29,11 +29,6 @@
 #define MAX_STAGES 4
 #define TGW 64  // candidates side by side per vreg in the tables handed from the table kernel to the walk
 #define WALK_WARPS 8
-#define RC_THREADS 256
-
-// per-candidate state between the kernels (8 words)
-enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_NOUT = 3, CS_OUTV = 4, CS_OUTRAW = 5, CS_WALK = 6, CS_THCOL = 7 };
-enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
 
 struct TParams {
     uint32_t nI, V, nO, nOp8, P, Bmask, ntiles;
@@ -97,31 +92,11 @@ struct WParams {
     uint32_t ev_cap;  // events a warp stages at a time (multiple of 8)
     uint32_t *cstate, *anom;
     uint32_t *grp_flag;  // per group: set by the table kernel when a walked candidate has a marked entry
-    // hand-over to k_recount by the last thread block of each group of 64 candidates
+    // hand-over to k_exact by the last thread block of each group of 64 candidates
     int list_all;
     const uint32_t *chunk_blk;
-    uint32_t *grp_done, *work, *racc;
+    uint32_t *grp_done, *work;
     vl_verdict *out;
-};
-
-struct RParams {
-    uint32_t nI, V, B, nB, nC, AW;
-    int bank_fast;
-    uint64_t K;
-    const uint32_t *vinfo, *chunk_i0, *chunk_i1, *chunk_blk, *blk_chunk_off, *th_off, *th, *op_off, *op_vreg, *lo_off, *lo, *blk_off;
-    const uint8_t *ndefs, *width, *opflags;
-    const uint16_t *tg;
-    const uint32_t *cstate, *anom;
-    uint32_t *racc;
-    const uint2 *bank_list;
-    uint32_t bank_seg[4];
-    uint32_t *work;
-    vl_verdict *out;
-    uint32_t *status;
-    const uint4 *el;           // the definitions the walk skips (see vl_program)
-    const uint32_t *el_count;
-    const uint32_t *ls, *ls_adj, *th_cnt;  // live-after lists without the through-sets (see vl_program)
-    uint32_t R;                            // registers covered by the recount's through-set counters
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -294,7 +269,7 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
     for (uint32_t j = tid; j < G * q.AW; j += NT) q.anom[k0 * q.AW + j] = 0;
     if (tid < G * 4) q.racc[k0 * 4 + tid] = 0;
     if (tid == 0 && (k0 & (TGW - 1)) == 0) q.grp_done[k0 / TGW] = 0;
-    if (tid == 0 && blockIdx.x == 0) { q.work[0] = 0; q.work[1] = 0; q.work[2] = 0; }  // item count and the recount's two cursors
+    if (tid == 0 && blockIdx.x == 0) q.work[0] = 0;  // items listed for the exact count
     __syncthreads();
 
     // The ring stage and the barrier phase of the current tile are kept as running counters (stage
@@ -692,7 +667,7 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
     for (uint32_t j = tid; j < G * q.AW; j += NT) q.anom[k0 * q.AW + j] = 0;
     if (tid < G * 4) q.racc[k0 * 4 + tid] = 0;
     if (tid == 0 && (k0 & (TGW - 1)) == 0) q.grp_done[k0 / TGW] = 0;
-    if (tid == 0 && blockIdx.x == 0) { q.work[0] = 0; q.work[1] = 0; q.work[2] = 0; }  // item count and the recount's two cursors
+    if (tid == 0 && blockIdx.x == 0) q.work[0] = 0;  // items listed for the exact count
     __syncthreads();
 
     // A tile is one box of the row tensor: 8 candidates x CH chunks x 256 operands, one copy.  (Boxes
@@ -1165,9 +1140,36 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr)
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
 }
-__device__ void finish_candidate(uint64_t k, uint32_t nC, uint32_t AW, int list_all, const uint32_t *cstate,
-                                 const uint32_t *anom, const uint32_t *__restrict__ chunk_blk, uint32_t *work,
-                                 uint32_t *racc, vl_verdict *out);
+// The verdict of candidate k if the walk vouches for it, else its items in the list of the exact count: as many as its
+// colliding chunks make worth while (one row of the workloads in a hundred moves a loop-carried vreg onto a register that
+// short-lived ones cycle through: every chunk of the loop collides, and that row decides the time).  Words that other
+// thread blocks updated with atomics are read from L2.
+__device__ __forceinline__ void finish_candidate(uint64_t k, uint32_t nC, uint32_t AW, int list_all, const uint32_t *cstate,
+                                                 const uint32_t *anom, uint32_t *work, vl_verdict *out)
+{
+    const uint32_t *cs = cstate + k * 8;
+    const uint32_t walk = __ldcg(cs + CS_WALK), thcol = __ldcg(cs + CS_THCOL);
+    if (list_all || (walk | thcol)) {
+        uint32_t chunks = list_all ? nC / 4 : (thcol ? nC / 8 : 0u);  // (the general bank tally; the sources in the through-set)
+        if (walk & WALK_FULL) chunks += nC;
+        else if (walk)
+            for (uint32_t w = 0; w < AW; ++w) chunks += __popc(__ldcg(anom + k * AW + w));
+        const uint32_t parts = min(1u + chunks / EXACT_PART_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
+        const uint32_t at = atomicAdd(work, parts);
+        for (uint32_t j = 0; j < parts; ++j) {
+            work[EXACT_HDR + 2 * (at + j)] = (uint32_t)k;
+            work[EXACT_HDR + 2 * (at + j) + 1] = j | (parts << 8);
+        }
+        return;
+    }
+    const uint32_t fl = __ldcg(cs + CS_FLAGS), first = __ldcg(cs + CS_FIRST);
+    vl_verdict vd;
+    vd.flags = fl ? fl : (uint32_t)VL_PASS;
+    vd.first_violation_instr = first == 0xFFFFFFFFu ? -1 : (int32_t)first;
+    vd.conflict_pairs = 0;
+    vd.bank_conflicts = __ldcg(cs + CS_BANK);
+    out[k] = vd;
+}
 
 // An event group in shared memory is 112 bytes: off[8] (byte offset of the vreg's table row),
 // toggle[8], test[8] (32-bit masks), wl[8] (16 bit).  Constant offsets go into the instruction.
@@ -1497,555 +1499,17 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 3) k_walk(const WParams q)
     if (!s_last) return;
     __threadfence();
     if (threadIdx.x == 0) q.grp_flag[grp] = 0;  // every block of the group has read it: clear for the next pass
-    for (uint32_t j = warp; j < TGW; j += n_warps) {
+    for (uint32_t j = threadIdx.x; j < TGW; j += blockDim.x) {
         const uint64_t kk = (uint64_t)grp * TGW + j;
-        if (kk < q.K) finish_candidate(kk, q.nC, q.AW, q.list_all, q.cstate, q.anom, q.chunk_blk, q.work, q.racc, q.out);
+        if (kk < q.K) finish_candidate(kk, q.nC, q.AW, q.list_all, q.cstate, q.anom, q.work, q.out);
     }
 }
 
-// =========================================================================== verdicts / work list
-// Verdicts of the candidates the walk vouches for.  For the others, work items for k_recount:
-// every chunk that needs an exact recount is cut into RC_PARTS pieces, the general bank tally into
-// RC_BANK_PARTS slices, and every block whose through-set collided gets one item for the
-// definitions the walk skipped in its other chunks; racc[k][3] counts the items pending.  An item
-// is (candidate, code) with code = kind << 30 | piece << 24 | chunk (or block).
-#define RC_PARTS 2
-#define RC_HDR 4  // words in front of the work items: item count, cursor of the first round, cursor of the second
-#define RC_BANK_PARTS 4
-#define RC_KIND_ALL 0u     // every definition of the piece
-#define RC_KIND_THROUGH 1u // a block whose through-set collided: the definitions the walk skipped, chunk = block
-#define RC_KIND_BANK 2u
-__device__ __forceinline__ uint32_t rc_code(uint32_t kind, uint32_t piece, uint32_t chunk)
+// Stand-alone form for programs without chunks (no instructions): one thread per candidate.
+__global__ void k_finish(uint64_t K, int list_all, const uint32_t *cstate, const uint32_t *anom, uint32_t *work, vl_verdict *out)
 {
-    return (kind << 30) | (piece << 24) | chunk;
-}
-
-// One warp finishes candidate k: the verdict if nothing is left to recount, else its work items.
-// cstate / anom words that other thread blocks updated with atomics are read from L2.
-__device__ void finish_candidate(uint64_t k, uint32_t nC, uint32_t AW, int list_all, const uint32_t *cstate,
-                                 const uint32_t *anom, const uint32_t *__restrict__ chunk_blk, uint32_t *work,
-                                 uint32_t *racc, vl_verdict *out)
-{
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t *cs = cstate + k * 8;
-    const uint32_t walk = __ldcg(cs + CS_WALK), thcol = __ldcg(cs + CS_THCOL);
-    if (!list_all && !(walk | thcol)) {
-        if (lane == 0) {
-            const uint32_t fl = __ldcg(cs + CS_FLAGS), first = __ldcg(cs + CS_FIRST);
-            vl_verdict vd;
-            vd.flags = fl ? fl : (uint32_t)VL_PASS;
-            vd.first_violation_instr = first == 0xFFFFFFFFu ? -1 : (int32_t)first;
-            vd.conflict_pairs = 0;
-            vd.bank_conflicts = __ldcg(cs + CS_BANK);
-            out[k] = vd;
-        }
-        return;
-    }
-    // a chunk that collided (or a candidate with several out-of-file vregs): every definition;
-    // a block whose through-set collided: the definitions the walk skipped in its other chunks (a
-    // vreg redefined from itself while it stays occupied), since everything else in them was walked
-    // exactly
-    const bool full = walk & WALK_FULL;
-    auto all_defs = [&](uint32_t c) -> bool {
-        return c < nC && (full || ((__ldcg(anom + k * AW + (c >> 5)) >> (c & 31)) & 1u));
-    };
-    uint32_t n_chunks = 0;
-    for (uint32_t c0 = 0; c0 < nC; c0 += 32) n_chunks += __popc(__ballot_sync(0xffffffffu, all_defs(c0 + lane)));
-    const uint32_t n_blocks = full ? 0u : __popc(thcol);
-    // the fast-path tally is one item per candidate (its table column is fetched once); the general tally
-    // of the other programs, which every candidate takes, is sliced
-    const uint32_t n_bank = list_all ? (uint32_t)RC_BANK_PARTS : 1u;
-    const uint32_t n = n_bank + RC_PARTS * n_chunks + n_blocks;
-    uint32_t at = 0;
-    if (lane == 0) {
-        racc[k * 4 + 3] = n;
-        at = atomicAdd(work, n);
-    }
-    at = __shfl_sync(0xffffffffu, at, 0);
-    if (lane < n_bank) {
-        work[RC_HDR + 2 * (at + lane)] = (uint32_t)k;
-        work[RC_HDR + 1 + 2 * (at + lane)] = rc_code(RC_KIND_BANK, lane, 0);
-    }
-    at += n_bank;
-    if (!full && ((thcol >> lane) & 1u)) {  // through-sets are used only if the program has at most 32 blocks
-        const uint32_t slot = at + __popc(thcol & ((1u << lane) - 1u));
-        work[RC_HDR + 2 * slot] = (uint32_t)k;
-        work[RC_HDR + 1 + 2 * slot] = rc_code(RC_KIND_THROUGH, 0, lane);
-    }
-    at += n_blocks;
-    for (uint32_t c0 = 0; c0 < nC; c0 += 32) {
-        const bool kd = all_defs(c0 + lane);
-        const uint32_t m = __ballot_sync(0xffffffffu, kd);
-        if (kd) {
-            const uint32_t slot = at + RC_PARTS * __popc(m & ((1u << lane) - 1u));
-#pragma unroll
-            for (uint32_t part = 0; part < RC_PARTS; ++part) {
-                work[RC_HDR + 2 * (slot + part)] = (uint32_t)k;
-                work[RC_HDR + 1 + 2 * (slot + part)] = rc_code(RC_KIND_ALL, part, c0 + lane);
-            }
-        }
-        at += RC_PARTS * __popc(m);
-    }
-}
-
-// Stand-alone form for programs without walk items (no instructions): one warp per candidate.
-__global__ void k_finish(uint64_t K, uint32_t nC, uint32_t AW, int list_all, const uint32_t *cstate,
-                         const uint32_t *anom, const uint32_t *__restrict__ chunk_blk, uint32_t *work, uint32_t *racc,
-                         vl_verdict *out)
-{
-    const uint64_t k = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (k < K) finish_candidate(k, nC, AW, list_all, cstate, anom, chunk_blk, work, racc, out);
-}
-
-// Bank list entries [e_lo, e_hi) with N distinct source vregs each: how many sources hold the register
-// of an earlier source of the same entry.  regs[v] = register of vreg v (shared memory).  8 entries per
-// thread and round; the entries of the next round are fetched meanwhile.
-template <int N>
-__device__ __forceinline__ uint32_t bank_duplicates(const uint2 *__restrict__ list, uint32_t e_lo, uint32_t e_hi,
-                                                    const uint32_t *regs, uint32_t tid)
-{
-    uint32_t dups = 0;
-    uint2 id_next[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-        id_next[u] = e_lo + tid + u * RC_THREADS < e_hi ? list[e_lo + tid + u * RC_THREADS] : make_uint2(0, 0);
-    for (uint32_t e0 = e_lo + tid; e0 < e_hi; e0 += 8 * RC_THREADS) {
-        uint2 idv[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            idv[u] = id_next[u];
-            const uint32_t en = e0 + (8 + u) * RC_THREADS;
-            id_next[u] = en < e_hi ? list[en] : make_uint2(0, 0);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (e0 + u * RC_THREADS >= e_hi) break;
-            const uint32_t x0 = regs[idv[u].x & 0xFFFFu], x1 = regs[idv[u].x >> 16];
-            dups += (x1 == x0);
-            if (N >= 3) {
-                const uint32_t x2 = regs[idv[u].y & 0xFFFFu];
-                dups += (x2 == x0) | (x2 == x1);
-                if (N >= 4) {
-                    const uint32_t x3 = regs[idv[u].y >> 16];
-                    dups += (x3 == x0) | (x3 == x1) | (x3 == x2);
-                }
-            }
-        }
-    }
-    return dups;
-}
-
-// =========================================================================== k_recount
-// Exact answers for the listed work items; thread blocks loop over the list.  A chunk item recounts
-// the overlaps of one piece of a chunk from the live-after lists (the warps share the piece's
-// instructions; the lanes of a warp fetch the bookkeeping of 32 instructions at a time); a bank
-// item does a slice of the general bank tally (distinct registers rather than distinct vregs).
-// The candidate's register and the width of a vreg are fetched from global memory the first time
-// an item needs them and kept in a shared-memory cache (CACHE; one word per vreg, valid bit 31):
-// the live-after sets of neighbouring instructions are nearly the same, so a piece touches a few
-// hundred vregs, not the whole table column.  Results are added to the candidate's accumulators;
-// the item that finishes last writes the verdict.
-template <bool CACHE>
-__global__ void __launch_bounds__(RC_THREADS) k_recount(const RParams q)
-{
-    extern __shared__ __align__(16) uint32_t Cv[];  // [V] register | width << 16 | valid << 31
-    __shared__ uint32_t s_pairs, s_mind, s_bank, s_big;
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr uint32_t NW = RC_THREADS / 32;
-    const uint32_t nitems = q.work[0];
-    __shared__ uint32_t s_item;
-    // The items differ a lot in length: thread blocks take the next one from a shared cursor.  Two rounds
-    // over the list: the long items first (a bank tally sweeps the whole program, a through-set item is
-    // quadratic in the set), then the chunk pieces, so that no long item starts when the others end.
-    for (uint32_t round = 0; round < 2;) {
-        __syncthreads();
-        if (tid == 0) s_item = atomicAdd(q.work + 1 + round, 1u);
-        __syncthreads();
-        const uint32_t it = s_item;
-        if (it >= nitems) { ++round; continue; }
-        const uint64_t k = q.work[RC_HDR + 2 * it];
-        const uint32_t code = q.work[RC_HDR + 1 + 2 * it];
-        const uint32_t kind = code >> 30, part = (code >> 24) & 63u, c = code & 0xFFFFFFu;
-        if ((kind == RC_KIND_ALL) != (round == 1)) continue;
-        const uint32_t *cs = q.cstate + k * 8;
-        const uint16_t *tg = q.tg + (k / TGW) * (uint64_t)(q.V + 1) * TGW + (k & (TGW - 1));
-        // a single out-of-file vreg sits parked in the table: its true register is in the candidate's state
-        const uint32_t out_v = cs[CS_NOUT] == 1 ? cs[CS_OUTV] : 0xFFFFFFFFu, out_raw = cs[CS_OUTRAW];
-        // a candidate with several out-of-file vregs was not walked and keeps its table unmarked
-        const uint32_t tmask = (cs[CS_WALK] & WALK_FULL) ? 0xFFFFu : 0x7FFFu;
-        __syncthreads();
-        if (CACHE)
-            for (uint32_t v = tid; v < q.V; v += RC_THREADS) Cv[v] = 0;
-        if (tid == 0) { s_pairs = 0; s_mind = 0xFFFFFFFFu; s_bank = 0; }
-        __syncthreads();
-        // register (low 16 bits) and width (bits 16..23) of vreg v for this candidate
-        auto fetch = [&](uint32_t v) -> uint32_t {
-            const uint32_t r = v == out_v ? out_raw : ((uint32_t)tg[(size_t)v * TGW] & tmask);
-            return r | ((q.vinfo[v] & 0xFFu) << 16);
-        };
-        auto reg_w = [&](uint32_t v) -> uint32_t {
-            if (!CACHE) return fetch(v);
-            uint32_t x = Cv[v];
-            if (!(x >> 31)) {
-                x = fetch(v) | 0x80000000u;
-                Cv[v] = x;  // several threads may store the same word
-            }
-            return x;
-        };
-        if (kind == RC_KIND_THROUGH) {
-            // The through-set of block c collided.  In a chunk of the block whose own walk was clean,
-            // everything else that is live is disjoint from the through-set and from each other, so a
-            // skipped definition of a through-set vreg overlaps exactly the through-set members that
-            // overlap it, whatever the instruction: count those once per member, then add them up over
-            // the skipped definitions.  (Chunks that did collide are recounted in full by their own items.)
-            const uint32_t t0 = q.th_off[c], n_th = q.th_off[c + 1] - t0;
-            uint32_t *ids = Cv;  // [n_th] member vreg ids (ascending), [n_th] register | width << 16, [n_th] counts
-            uint32_t *mem = Cv + n_th, *cnt_th = Cv + 2 * n_th;
-            const bool fits = CACHE && 3 * n_th <= q.V;
-            if (fits) {
-                __syncthreads();
-                for (uint32_t j = tid; j < n_th; j += RC_THREADS) {
-                    const uint32_t v = q.th[t0 + j] & 0xFFFFu;
-                    ids[j] = v;
-                    mem[j] = fetch(v);
-                }
-                __syncthreads();
-                for (uint32_t j = tid; j < n_th; j += RC_THREADS) {
-                    const uint32_t s = mem[j] & 0xFFFFu, w = (mem[j] >> 16) & 0xFFu;
-                    uint32_t cc = 0;
-                    for (uint32_t u = 0; u < n_th; ++u)
-                        if (u != j && ranges_overlap(s, w, mem[u] & 0xFFFFu, (mem[u] >> 16) & 0xFFu)) ++cc;
-                    cnt_th[j] = cc;
-                }
-                __syncthreads();
-            }
-            // overlap count of through-set member v (0 if v is not a member): the list is ascending
-            auto count_of = [&](uint32_t v) -> uint32_t {
-                uint32_t lo_j = 0, hi_j = n_th;
-                while (lo_j < hi_j) {
-                    const uint32_t mid = (lo_j + hi_j) >> 1;
-                    if ((fits ? ids[mid] : (q.th[t0 + mid] & 0xFFFFu)) < v) lo_j = mid + 1; else hi_j = mid;
-                }
-                if (lo_j >= n_th || (fits ? ids[lo_j] : (q.th[t0 + lo_j] & 0xFFFFu)) != v) return 0u;
-                if (fits) return cnt_th[lo_j];
-                const uint32_t x = fetch(v);
-                uint32_t cc = 0;
-                for (uint32_t u = 0; u < n_th; ++u) {
-                    if (u == lo_j) continue;
-                    const uint32_t y = fetch(q.th[t0 + u] & 0xFFFFu);
-                    if (ranges_overlap(x & 0xFFFFu, (x >> 16) & 0xFFu, y & 0xFFFFu, (y >> 16) & 0xFFu)) ++cc;
-                }
-                return cc;
-            };
-            // the block's skipped definitions are listed as {instruction, chunk, vreg | member << 31, short chunk}
-            uint32_t pairs = 0, mind = 0xFFFFFFFFu;
-            const uint32_t n_el = q.el_count[c];
-            const uint4 *el = q.el + q.op_off[q.blk_off[c]];
-            for (uint32_t e = tid; e < n_el; e += RC_THREADS) {
-                const uint4 x = el[e];
-                if (!(x.z >> 31) || ((q.anom[k * q.AW + (x.y >> 5)] >> (x.y & 31)) & 1u)) continue;
-                const uint32_t cn = count_of(x.z & 0xFFFFu);
-                if (cn) { pairs += cn; mind = min(mind, x.x); }
-            }
-#pragma unroll
-            for (int dd = 16; dd; dd >>= 1) {
-                pairs += __shfl_xor_sync(0xffffffffu, pairs, dd);
-                mind = min(mind, __shfl_xor_sync(0xffffffffu, mind, dd));
-            }
-            if (lane == 0 && pairs) {
-                atomicAdd(&s_pairs, pairs);
-                atomicMin(&s_mind, mind);
-            }
-        } else if (kind != RC_KIND_BANK) {
-            const uint32_t ci0 = q.chunk_i0[c], cn = q.chunk_i1[c] - ci0;
-            const uint32_t i_lo = ci0 + (uint32_t)((uint64_t)cn * part / RC_PARTS);
-            const uint32_t i_hi = ci0 + (uint32_t)((uint64_t)cn * (part + 1) / RC_PARTS);
-            uint32_t pairs = 0, mind = 0xFFFFFFFFu;
-            // The vregs that stay occupied through the whole block (its through-set) are live after every
-            // instruction of it.  Rather than meeting them again in every live-after list, the block
-            // counts them once into two arrays over the registers (cover[r]: members whose range holds r,
-            // start[r]: members whose range starts at r); a definition with range [s, s+w) then overlaps
-            // cover[s] + start[s+1] + ... + start[s+w-1] of them, and only the short list (live after,
-            // not in the through-set) is scanned entry by entry.  Needs every member inside the arrays
-            // (R registers: the file plus the widest vreg); otherwise the full lists are scanned.
-            const uint32_t blk = q.chunk_blk[c];
-            const uint32_t t0 = q.th_off[blk], n_th = q.th_off[blk + 1] - t0;
-            const uint32_t ls_sub = q.ls_adj[blk], ls_mul = q.th_cnt[blk];
-            uint32_t *cover = Cv + q.V + 4, *start = cover + q.R;
-            bool use_short = CACHE && n_th > 0 && ls_mul == n_th;
-            if (use_short) {
-                for (uint32_t r = tid; r < 2 * q.R; r += RC_THREADS) cover[r] = 0;
-                if (tid == 0) s_big = 0;
-                __syncthreads();
-                for (uint32_t j = tid; j < n_th; j += RC_THREADS) {
-                    const uint32_t v = q.th[t0 + j] & 0xFFFFu;
-                    const uint32_t f = fetch(v), reg = f & 0xFFFFu, w = (f >> 16) & 0xFFu;
-                    Cv[v] = f | 0xC0000000u;  // valid, member of the through-set
-                    if (reg + w <= q.R) {
-                        atomicAdd(&start[reg], 1u);
-                        for (uint32_t r = reg; r < reg + w; ++r) atomicAdd(&cover[r], 1u);
-                    } else {
-                        s_big = 1;
-                    }
-                }
-                __syncthreads();
-                use_short = s_big == 0;
-            }
-            const uint32_t *lst = use_short ? q.ls : q.lo;
-            // first entry and length of instruction i's list, from its two live-after offsets
-            auto list_lo = [&](uint32_t i, uint32_t off_i) { return use_short ? off_i - ls_sub - i * ls_mul : off_i; };
-            auto list_n = [&](uint32_t off_i, uint32_t off_i1) { return off_i1 - off_i - (use_short ? ls_mul : 0u); };
-            if (CACHE && i_lo < i_hi) {
-                // Every vreg that is live after an instruction of the piece is live after its first
-                // instruction or defined inside the piece: the whole block fetches those into the cache in
-                // one go, so that the instruction-by-instruction recount below finds them there instead of
-                // waiting for global memory once per instruction.
-                const uint32_t f0 = q.lo_off[i_lo], f1 = q.lo_off[i_lo + 1];
-                const uint32_t l0 = list_lo(i_lo, f0), l1 = l0 + list_n(f0, f1);
-                for (uint32_t e = l0 + tid; e < l1; e += RC_THREADS) {
-                    const uint32_t v = lst[e];
-                    if (!(Cv[v] >> 31)) Cv[v] = fetch(v) | 0x80000000u;
-                }
-                for (uint32_t i = i_lo + tid; i < i_hi; i += RC_THREADS) {
-                    const uint32_t o0 = q.op_off[i], nd = q.ndefs[i];
-                    for (uint32_t d = o0; d < o0 + nd; ++d) {
-                        const uint32_t v = q.op_vreg[d];
-                        if (!(Cv[v] >> 31)) Cv[v] = fetch(v) | 0x80000000u;
-                    }
-                }
-                __syncthreads();
-            }
-            if (use_short) {
-                // Short lists (the through-set is counted from the arrays): two lanes per instruction, 128
-                // instructions per round, so that the loads of a whole round (bookkeeping, then defined vregs
-                // and list entries) are in flight together instead of instruction after instruction.
-                const uint32_t sub = lane & 1u, slot = tid >> 1;
-                for (uint32_t ib = i_lo; ib < i_hi; ib += RC_THREADS / 2) {
-                    const uint32_t i = ib + slot;
-                    uint32_t cnt_i = 0;
-                    if (i < i_hi) {
-                        const uint32_t o0 = q.op_off[i], nd = q.ndefs[i];
-                        const uint32_t f0 = q.lo_off[i], f1 = q.lo_off[i + 1];
-                        const uint32_t l0 = list_lo(i, f0), l1 = l0 + list_n(f0, f1);
-                        for (uint32_t d = o0; d < o0 + nd; ++d) {
-                            const uint32_t v = q.op_vreg[d];
-                            const uint32_t sw = reg_w(v);
-                            const uint32_t s = sw & 0xFFFFu, w = (sw >> 16) & 0xFFu;
-                            uint32_t cnt = 0;
-                            if (s < q.R) {  // the through-set members that overlap [s, s+w), v itself excepted
-                                if (sub == 0) cnt = cover[s] - ((sw >> 30) & 1u);
-                                for (uint32_t r = s + 1 + sub; r < min(s + w, q.R); r += 2) cnt += start[r];
-                            }
-                            for (uint32_t e0 = l0 + sub; e0 < l1; e0 += 16) {  // 8 list entries per lane in flight
-                                uint32_t us[8], xs[8];
-#pragma unroll
-                                for (int u = 0; u < 8; ++u) {
-                                    const uint32_t e = e0 + u * 2;
-                                    us[u] = e < l1 ? lst[e] : v;
-                                }
-#pragma unroll
-                                for (int u = 0; u < 8; ++u) xs[u] = reg_w(us[u]);
-#pragma unroll
-                                for (int u = 0; u < 8; ++u)
-                                    if (us[u] != v && ranges_overlap(s, w, xs[u] & 0xFFFFu, (xs[u] >> 16) & 0xFFu)) ++cnt;
-                            }
-                            // co-defined vregs that are not live after the instruction
-                            if (nd > 1)
-                                for (uint32_t d2 = o0 + sub; d2 < o0 + nd; d2 += 2) {
-                                    if (d2 == d || !(q.opflags[d2] & OPF_DEAD)) continue;
-                                    const uint32_t x = reg_w(q.op_vreg[d2]);
-                                    if (ranges_overlap(s, w, x & 0xFFFFu, (x >> 16) & 0xFFu)) ++cnt;
-                                }
-                            cnt_i += cnt;
-                        }
-                    }
-                    cnt_i += __shfl_xor_sync(0xffffffffu, cnt_i, 1);
-                    if (cnt_i && sub == 0) { pairs += cnt_i; mind = min(mind, i); }
-                }
-#pragma unroll
-                for (int dd = 16; dd; dd >>= 1) {  // (lane 0 reports for the warp)
-                    pairs += __shfl_xor_sync(0xffffffffu, pairs, dd);
-                    mind = min(mind, __shfl_xor_sync(0xffffffffu, mind, dd));
-                }
-            }
-            // full lists: this warp's instructions are i_lo + warp, i_lo + warp + NW, ...; 32 of them per round
-            for (uint32_t ib = i_lo + warp; !use_short && ib < i_hi; ib += 32 * NW) {
-                const uint32_t my_i = ib + lane * NW;
-                uint32_t m_o0 = 0, m_nd = 0, m_l0 = 0, m_l1 = 0;
-                if (my_i < i_hi) {
-                    m_o0 = q.op_off[my_i]; m_nd = q.ndefs[my_i];
-                    const uint32_t f0 = q.lo_off[my_i], f1 = q.lo_off[my_i + 1];
-                    m_l0 = list_lo(my_i, f0);
-                    m_l1 = m_l0 + list_n(f0, f1);
-                }
-                // first defined vreg of each instruction, fetched by the lane that holds its bookkeeping
-                uint32_t m_v0 = 0;
-                if (m_nd) m_v0 = q.op_vreg[m_o0];
-                uint32_t todo = __ballot_sync(0xffffffffu, m_nd != 0);
-                // the first 256 entries of the next instruction's list are fetched while the current
-                // instruction is recounted
-                uint32_t us_nx[8];
-                auto fetch_list = [&](int src) {
-                    const uint32_t l0 = __shfl_sync(0xffffffffu, m_l0, src), l1 = __shfl_sync(0xffffffffu, m_l1, src);
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const uint32_t e = l0 + u * 32 + lane;
-                        us_nx[u] = e < l1 ? lst[e] : 0xFFFFFFFFu;
-                    }
-                };
-                if (todo) fetch_list(__ffs(todo) - 1);
-                while (todo) {
-                    const int src = __ffs(todo) - 1;
-                    todo &= todo - 1;
-                    uint32_t us0[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) us0[u] = us_nx[u];
-                    if (todo) fetch_list(__ffs(todo) - 1);
-                    const uint32_t i = ib + (uint32_t)src * NW;
-                    const uint32_t o0 = __shfl_sync(0xffffffffu, m_o0, src), nd = __shfl_sync(0xffffffffu, m_nd, src);
-                    const uint32_t l0 = __shfl_sync(0xffffffffu, m_l0, src), l1 = __shfl_sync(0xffffffffu, m_l1, src);
-                    const uint32_t v0 = __shfl_sync(0xffffffffu, m_v0, src);
-                    for (uint32_t d = o0; d < o0 + nd; ++d) {
-                        const uint32_t v = d == o0 ? v0 : q.op_vreg[d];
-                        const uint32_t sw = reg_w(v);
-                        const uint32_t s = sw & 0xFFFFu, w = (sw >> 16) & 0xFFu;
-                        uint32_t cnt = 0;
-                        if (use_short && s < q.R) {  // the through-set members that overlap [s, s+w), v itself excepted
-                            if (lane == 0) cnt = cover[s] - ((sw >> 30) & 1u);
-                            for (uint32_t r = s + 1 + lane; r < min(s + w, q.R); r += 32) cnt += start[r];
-                        }
-                        for (uint32_t e0 = l0; e0 < l1; e0 += 256) {  // 8 list entries per lane in flight
-                            uint32_t us[8], xs[8];
-#pragma unroll
-                            for (int u = 0; u < 8; ++u) {
-                                const uint32_t e = e0 + u * 32 + lane;
-                                us[u] = e0 == l0 ? us0[u] : (e < l1 ? lst[e] : 0xFFFFFFFFu);
-                                if (us[u] == 0xFFFFFFFFu) us[u] = v;
-                            }
-                            // (with the cache, every entry of the list and v itself were fetched up front)
-#pragma unroll
-                            for (int u = 0; u < 8; ++u) xs[u] = CACHE ? Cv[us[u]] : fetch(us[u]);
-#pragma unroll
-                            for (int u = 0; u < 8; ++u)
-                                if (us[u] != v && ranges_overlap(s, w, xs[u] & 0xFFFFu, (xs[u] >> 16) & 0xFFu)) ++cnt;
-                        }
-                        // co-defined vregs that are not live after the instruction
-                        if (nd > 1)
-                            for (uint32_t d2 = o0 + lane; d2 < o0 + nd; d2 += 32) {
-                                if (d2 == d || !(q.opflags[d2] & OPF_DEAD)) continue;
-                                const uint32_t x = reg_w(q.op_vreg[d2]);
-                                if (ranges_overlap(s, w, x & 0xFFFFu, (x >> 16) & 0xFFu)) ++cnt;
-                            }
-#pragma unroll
-                        for (int dd = 16; dd; dd >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, dd);
-                        if (cnt) { pairs += cnt; mind = min(mind, i); }
-                    }
-                }
-            }
-            if (lane == 0 && pairs) {
-                atomicAdd(&s_pairs, pairs);
-                atomicMin(&s_mind, mind);
-            }
-        } else {
-            // a source counts when its register is new among the instruction's sources and its bank is not
-            uint32_t bt = 0;
-            if (CACHE && q.bank_fast) {
-                // The table kernel's tally (sources minus banks touched, per instruction) counts a register
-                // that two source vregs share twice: the exact tally is that figure minus the number of such
-                // duplicates.  The candidate's registers are fetched in one go (every load in flight at once),
-                // then the list is swept from shared memory, one segment per source count.
-#pragma unroll 8
-                for (uint32_t v = tid; v < q.V; v += RC_THREADS)
-                    Cv[v] = v == out_v ? out_raw : ((uint32_t)tg[(size_t)v * TGW] & tmask);
-                __syncthreads();
-                const uint32_t dups = bank_duplicates<2>(q.bank_list, q.bank_seg[0], q.bank_seg[1], Cv, tid) +
-                                      bank_duplicates<3>(q.bank_list, q.bank_seg[1], q.bank_seg[2], Cv, tid) +
-                                      bank_duplicates<4>(q.bank_list, q.bank_seg[2], q.bank_seg[3], Cv, tid);
-                if (tid == 0) atomicAdd(&s_bank, cs[CS_BANK]);
-                if (dups) atomicSub(&s_bank, dups);
-            } else
-            if (q.bank_fast) {
-                const uint32_t n_all = q.bank_seg[3];
-                const uint32_t e_lo = 0, e_hi = n_all;  // (one item per candidate: part is 0)
-                // 8 list entries per thread and round; the entries of the next round are fetched meanwhile
-                uint2 id_next[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    id_next[u] = e_lo + tid + u * RC_THREADS < e_hi ? q.bank_list[e_lo + tid + u * RC_THREADS] : make_uint2(0, 0);
-                for (uint32_t e0 = e_lo + tid; e0 < e_hi; e0 += 8 * RC_THREADS) {
-                    uint2 idv[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        idv[u] = id_next[u];
-                        const uint32_t en = e0 + (8 + u) * RC_THREADS;
-                        id_next[u] = en < e_hi ? q.bank_list[en] : make_uint2(0, 0);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const uint32_t e = e0 + u * RC_THREADS;
-                        if (e >= e_hi) break;
-                        const uint2 ids = idv[u];
-                        const uint32_t n = e < q.bank_seg[1] ? 2u : (e < q.bank_seg[2] ? 3u : 4u);
-                        uint32_t x[4];
-                        x[0] = reg_w(ids.x & 0xFFFFu) & 0xFFFFu; x[1] = reg_w(ids.x >> 16) & 0xFFFFu;
-                        x[2] = reg_w(ids.y & 0xFFFFu) & 0xFFFFu; x[3] = reg_w(ids.y >> 16) & 0xFFFFu;
-#pragma unroll
-                        for (uint32_t a = 1; a < 4; ++a) {
-                            if (a >= n) break;
-                            bool seen_value = false, seen_bank = false;
-#pragma unroll
-                            for (uint32_t bb = 0; bb < a; ++bb) {
-                                seen_value |= (x[bb] == x[a]);
-                                seen_bank |= ((x[bb] ^ x[a]) & (q.B - 1)) == 0;
-                            }
-                            if (!seen_value && seen_bank) ++bt;
-                        }
-                    }
-                }
-            } else {
-                const uint32_t i_lo = (uint32_t)((uint64_t)q.nI * part / RC_BANK_PARTS);
-                const uint32_t i_hi = (uint32_t)((uint64_t)q.nI * (part + 1) / RC_BANK_PARTS);
-                for (uint32_t i = i_lo + tid; i < i_hi; i += RC_THREADS) {
-                    const uint32_t u0 = q.op_off[i] + q.ndefs[i], u1 = q.op_off[i + 1];
-                    for (uint32_t a = u0 + 1; a < u1; ++a) {
-                        const uint32_t xa = reg_w(q.op_vreg[a]) & 0xFFFFu;
-                        bool seen_value = false, seen_bank = false;
-                        for (uint32_t bb = u0; bb < a; ++bb) {
-                            const uint32_t xb = reg_w(q.op_vreg[bb]) & 0xFFFFu;
-                            seen_value |= (xb == xa);
-                            seen_bank |= (xb % q.B == xa % q.B);
-                        }
-                        if (!seen_value && seen_bank) ++bt;
-                    }
-                }
-            }
-#pragma unroll
-            for (int d = 16; d; d >>= 1) bt += __shfl_xor_sync(0xffffffffu, bt, d);
-            if (lane == 0 && bt) atomicAdd(&s_bank, bt);
-        }
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t *acc = q.racc + k * 4;
-            if (s_pairs) atomicAdd(&acc[0], s_pairs);
-            if (s_mind != 0xFFFFFFFFu) atomicMax(&acc[1], ~s_mind);  // accumulators start at 0: keep the complement
-            if (s_bank) atomicAdd(&acc[2], s_bank);
-            __threadfence();
-            if (atomicSub(&acc[3], 1u) == 1u) {  // last item of this candidate
-                __threadfence();
-                const uint32_t pairs = atomicAdd(&acc[0], 0u), mind = ~atomicMax(&acc[1], 0u),
-                               bank = atomicAdd(&acc[2], 0u);
-                uint32_t flags = cs[CS_FLAGS] | (pairs ? (uint32_t)VL_INTERFERENCE : 0u);
-                if (!flags) flags = VL_PASS;
-                const uint32_t first = min(cs[CS_FIRST], mind);
-                vl_verdict vd;
-                vd.flags = flags;
-                vd.first_violation_instr = first == 0xFFFFFFFFu ? -1 : (int32_t)first;
-                vd.conflict_pairs = pairs;
-                vd.bank_conflicts = bank;
-                q.out[k] = vd;
-            }
-        }
-    }
+    const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < K) finish_candidate(k, 0, 0, list_all, cstate, anom, work, out);
 }
 
 // --------------------------------------------------------------------------- host
@@ -2163,21 +1627,14 @@ cudaError_t launch_tables(const TParams &q, uint32_t grid, uint32_t smem, cudaSt
     return cudaGetLastError();
 }
 
-// Most work items one candidate can list for the recount: every chunk in RC_PARTS pieces, the bank
-// tally in RC_BANK_PARTS slices, one item per block whose through-set collided (through-sets are
-// used only by programs of at most 32 blocks).
-uint64_t rc_items_per_row(const vl_program *p)
-{
-    return (uint64_t)RC_PARTS * p->nC + RC_BANK_PARTS + std::min<uint32_t>(p->nB, 32u);
-}
-
 int ensure_scratch(vl_program *p, int slot, uint64_t rows)
 {
     vl_program::VScratch &v = p->vs[slot];
     const uint64_t aw = std::max(1u, (p->nC + 31) / 32);
     const uint64_t groups = (rows + TGW - 1) / TGW;
     if (v.rows >= rows && v.aw == aw && v.vregs == p->V && v.chunks == p->nC) return VL_OK;
-    cudaFree(v.tg); cudaFree(v.cstate); cudaFree(v.anom); cudaFree(v.work); cudaFree(v.racc); cudaFree(v.grp_done); cudaFree(v.thm);
+    cudaFree(v.tg); cudaFree(v.cstate); cudaFree(v.anom); cudaFree(v.work); cudaFree(v.racc); cudaFree(v.grp_done); cudaFree(v.thm); cudaFree(v.exact);
+    v.exact = nullptr;
     v.tg = nullptr; v.cstate = nullptr; v.anom = nullptr; v.work = nullptr; v.racc = nullptr; v.grp_done = nullptr; v.thm = nullptr;
     v.rows = 0;
     VL_CUDA(p, cudaMalloc((void **)&v.tg, groups * (p->V + 1) * TGW * sizeof(uint16_t)));
@@ -2185,7 +1642,8 @@ int ensure_scratch(vl_program *p, int slot, uint64_t rows)
     VL_CUDA(p, cudaMalloc((void **)&v.cstate, groups * TGW * 8 * sizeof(uint32_t)));
     VL_CUDA(p, cudaMemset(v.cstate, 0, groups * TGW * 8 * sizeof(uint32_t)));
     VL_CUDA(p, cudaMalloc((void **)&v.anom, groups * TGW * aw * sizeof(uint32_t)));
-    VL_CUDA(p, cudaMalloc((void **)&v.work, (RC_HDR + 2 * groups * TGW * rc_items_per_row(p)) * sizeof(uint32_t)));
+    VL_CUDA(p, cudaMalloc((void **)&v.work, (EXACT_HDR + 2 * EXACT_MAX_PARTS * groups * TGW) * sizeof(uint32_t)));
+    if (vl_exact_scratch(p)) VL_CUDA(p, cudaMalloc((void **)&v.exact, vl_exact_scratch(p)));
     VL_CUDA(p, cudaMalloc((void **)&v.racc, groups * TGW * 4 * sizeof(uint32_t)));
     // walk blocks finished per group, then the groups' straddle-mark flags (reset by the walk)
     VL_CUDA(p, cudaMalloc((void **)&v.grp_done, 2 * (groups + 1) * sizeof(uint32_t)));
@@ -2215,7 +1673,7 @@ static void kt_mark(vl_program *p, cudaStream_t st)
 namespace {
 struct PassPlan {
     Plan pl;
-    uint32_t Wp, ev_cap, walk_smem, walk_warps, rc_smem;
+    uint32_t Wp, ev_cap, walk_smem, walk_warps;
     uint64_t sub;
 };
 
@@ -2250,16 +1708,10 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
         if (pp->walk_smem <= SM_BYTES - 1024) break;
         if (pp->walk_warps == 1) return VL_ERR_UNSUPPORTED;
     }
-    // the recount keeps one cache word per vreg in shared memory when that leaves room for several
-    // thread blocks per SM, else it fetches from global memory every time
-    pp->rc_smem = (uint64_t)p->V * 4 <= 72 * 1024
-                      ? (uint32_t)align16(((uint64_t)(p->V + 4) + 2ull * (p->P + p->wmax + 2)) * 4) : 0u;
     // the walk's table entries keep bit 15 for a mark: every in-file register number must be below 2^15
     // (the occupancy masks of a register file that large would not fit shared memory anyway)
     if (p->P + p->wmax > 32768u) return VL_ERR_UNSUPPORTED;
-    // the recount work list holds up to rc_items_per_row items per candidate: keep it within 8 Mi items
-    const uint64_t sub_cap = std::max<uint64_t>(32, ((8ull << 20) / rc_items_per_row(p)) / 32 * 32);
-    pp->sub = std::min<uint64_t>(K, std::min<uint64_t>(p->sub_batch, sub_cap));
+    pp->sub = std::min<uint64_t>(K, p->sub_batch);
     // passes of equal size (whole groups of the tables) rather than full ones and a short last one
     if (K > pp->sub) {
         const uint64_t n_pass = (K + pp->sub - 1) / pp->sub;
@@ -2274,10 +1726,9 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
         if (!attr_done[p->device]) {
             const int sm = (int)SM_BYTES;
             const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-            // (the walk and the recount also have a few bytes of static shared memory)
+            // (the walk also has a few bytes of static shared memory)
             cudaError_t e = cudaFuncSetAttribute(k_walk, at, sm - 1024);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k_through, at, sm - 1024);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(k_recount<true>, at, sm - 1024);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tables<4, 256>, at, sm);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tables<2, 256>, at, sm);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tables<1, 256>, at, sm);
@@ -2379,7 +1830,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
         wq.cstate = vs.cstate; wq.anom = vs.anom;
         wq.grp_flag = vs.grp_done + (vs.rows / TGW + 1);
         wq.list_all = p->bank_fast ? 0 : 1; wq.chunk_blk = p->d_chunk_blk;
-        wq.grp_done = vs.grp_done; wq.work = vs.work; wq.racc = vs.racc; wq.out = d_out;
+        wq.grp_done = vs.grp_done; wq.work = vs.work; wq.out = d_out;
         if (own_through) {
             k_through<<<dim3(p->nB, ngrp), 256, pp.Wp * 64 * 4, st>>>(wq);
             e = cudaGetLastError();
@@ -2394,35 +1845,18 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     }
 
     // programs whose bank tally cannot take the fast path (banks not 1, 2 or 4, or an instruction
-    // with more than 4 distinct sources) send every candidate through k_recount
+    // with more than 4 distinct sources) list every candidate for k_exact
     kt_mark(p, st);
     if (!p->nC) {  // nothing to walk: the verdict step runs on its own
-        k_finish<<<(uint32_t)((n * 32 + 127) / 128), 128, 0, st>>>(n, p->nC, (uint32_t)vs.aw, p->bank_fast ? 0 : 1,
-                                                                  vs.cstate, vs.anom, p->d_chunk_blk, vs.work, vs.racc,
-                                                                  d_out);
+        k_finish<<<(uint32_t)((n + 127) / 128), 128, 0, st>>>(n, p->bank_fast ? 0 : 1, vs.cstate, vs.anom, vs.work, d_out);
         g_vl_launches.fetch_add(1);
     }
-    RParams rq{};
-    rq.nI = p->nI; rq.V = p->V; rq.B = p->B; rq.nB = p->nB; rq.nC = p->nC; rq.AW = (uint32_t)vs.aw;
-    rq.bank_fast = p->bank_fast; rq.K = n;
-    rq.blk_chunk_off = p->d_blk_chunk_off; rq.th_off = p->d_th_off; rq.th = p->d_th;
-    rq.blk_off = p->d_blk_off; rq.el = p->d_el; rq.el_count = p->d_el_count;
-    rq.ls = p->d_ls; rq.ls_adj = p->d_ls_adj; rq.th_cnt = p->d_th_cnt; rq.R = p->P + p->wmax + 2;
-    rq.vinfo = p->d_vinfo; rq.chunk_i0 = p->d_chunk_i0; rq.chunk_i1 = p->d_chunk_i1; rq.chunk_blk = p->d_chunk_blk;
-    rq.op_off = p->d_op_off; rq.op_vreg = p->d_op_vreg; rq.lo_off = p->d_lo_off; rq.lo = p->d_lo;
-    rq.ndefs = p->d_ndefs; rq.width = p->d_width; rq.opflags = p->d_opflags;
-    rq.racc = vs.racc; rq.status = p->d_status + 1;
-    rq.tg = vs.tg; rq.cstate = vs.cstate; rq.anom = vs.anom; rq.work = vs.work; rq.out = d_out;
-    rq.bank_list = p->d_bank_list;
-    for (int j = 0; j < 4; ++j) rq.bank_seg[j] = p->bank_seg[j];
-    const uint32_t rgrid = (uint32_t)vl_sm_count(p) * 6;  // thread blocks of the recount: they take items from a shared cursor
     kt_mark(p, st);
-    if (pp.rc_smem) k_recount<true><<<rgrid, RC_THREADS, pp.rc_smem, st>>>(rq);
-    else k_recount<false><<<rgrid, RC_THREADS, 0, st>>>(rq);
+    VlExactArgs ex{};
+    ex.work = vs.work; ex.cstate = vs.cstate; ex.anom = vs.anom; ex.short_chunk = p->d_short_chunk; ex.racc = vs.racc;
+    ex.AW = (uint32_t)vs.aw; ex.scratch = vs.exact;
+    if ((rc = vl_exact_run(p, ex, d_cand, pitch, d_out, st, dict)) != VL_OK) return rc;
     kt_mark(p, st);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) { p->last_cuda_error = (int)e; return VL_ERR_CUDA; }
-    g_vl_launches.fetch_add(1);
     return VL_OK;
 }
 }  // namespace
