@@ -23,7 +23,8 @@ namespace {
 
 struct FMisc {
     uint32_t flags, minop, minr, bank, pairs, mind, thcol, any;
-    uint32_t n_list, dups;
+    uint32_t n_list, n_chunks, dups;
+    uint32_t blk_i[33], el_n[32], el_o[32];  // first instruction; definitions without an event: how many, first of the list
     uint32_t th_off[33];  // (through-sets are used only by programs of at most 32 blocks)
 };
 
@@ -46,7 +47,7 @@ inline FSmem fused_smem(const vl_program *p, uint32_t threads)
     s.coll = s.occ + up16(std::max(Wp * threads * 4, counts));
     s.cb = p->use_th ? (s.coll - s.occ) / counts : p->nB;
     s.list = s.coll + up16((p->nS + 31) / 32 * 4 + 4);
-    s.misc = s.list + p->nS * 16;
+    s.misc = s.list + up16(p->nS * 8);
     s.total = s.misc + up16(sizeof(FMisc));
     return s;
 }
@@ -155,6 +156,21 @@ __device__ __forceinline__ uint32_t duplicate_of(const FParams &q, const uint16_
     return !again && same;
 }
 
+// The numbers of the program blocks that the counts of the through-sets need.
+__device__ __forceinline__ void load_blocks(const FParams &q, FMisc *M)
+{
+    const uint32_t b = threadIdx.x;
+    if (b > 32) return;
+    M->th_off[b] = q.use_th ? q.th_off[min(b, q.nB)] : 0u;
+    if (!q.use_th) return;
+    const uint32_t i0 = q.blk_off[min(b, q.nB)];
+    M->blk_i[b] = i0;
+    if (b < q.nB) {
+        M->el_n[b] = q.el_count[b];
+        M->el_o[b] = q.op_off[i0];
+    }
+}
+
 // Sources of instruction i in the through-set of block b that hold the register of an earlier source, where an earlier
 // source in the through-set holds it too.
 __device__ __noinline__ uint32_t member_duplicates(const FParams &q, const uint16_t *T, uint32_t b, uint32_t i)
@@ -179,7 +195,8 @@ __device__ __noinline__ uint32_t member_duplicates(const FParams &q, const uint1
 // Step 5: the overlaps in the short chunks marked in coll and, for program blocks whose through-set collided, those of the
 // definitions without an event, counted exactly; added to M->pairs and M->mind.  With several parts, this block's share.
 // The program blocks are taken q.cb at a time (all at once, as a rule: going block by block, the chain of L2 round trips
-// in front of the first count took 2 us for each).  cv: [cb][R] words; list: room for nS spans.
+// in front of the first count took 2 us for each).  cv: [cb][R] words; list: room for nS spans
+// (and, LISTED, behind them for the ranges of nC chunks).
 // LISTED (k_exact): the bank tally of the table kernel (sources minus banks touched, per instruction) counts a register
 // that two source vregs share twice; M->dups receives the number of such sources.  Two sources of an instruction are live
 // together in front of it: if they hold the same register, its chunk has collided, or they are both in a through-set that
@@ -187,7 +204,7 @@ __device__ __noinline__ uint32_t member_duplicates(const FParams &q, const uint1
 // misplaced vreg; fetching all 10,000 took 30 us).
 template <int NTHR, bool LISTED>
 __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint8_t *W, uint32_t *cv, const uint32_t *coll,
-                                             uint4 *list, FMisc *M, uint32_t part, uint32_t parts, const uint16_t *row)
+                                             uint2 *list, FMisc *M, uint32_t part, uint32_t parts, const uint16_t *row)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     uint32_t pairs = 0, mind = 0xFFFFFFFFu, dups = 0;
@@ -195,66 +212,83 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
         const uint32_t b1 = min(b0 + q.cb, q.nB);
         const uint32_t s_lo = b0 ? q.blk_short_off[b0] : 0u, s_hi = b1 < q.nB ? q.blk_short_off[b1] : q.nS;
         const uint32_t thcol = q.use_th ? M->thcol : 0u;
-        if (tid == 0) M->n_list = 0;
+        if (tid == 0) M->n_list = M->n_chunks = 0;
         // The through-sets, counted into arrays over the registers: cv[r] = members whose range holds r, plus 65536 for
         // each member whose range starts at r; a range [s, s+w) overlaps (members that hold s) + (members that start at
         // s+1 .. s+w-1).  Members that reach beyond the arrays lie beyond the file: they are compared one by one, with
         // definitions that lie there too.
         if (q.use_th)
             for (uint32_t r = tid; r < (b1 - b0) * q.R; r += NTHR) cv[r] = 0;
+        uint4 *chunks = reinterpret_cast<uint4 *>(list + ((q.nS + 1) & ~1u));
         __syncthreads();
         for (uint32_t s = s_lo + tid; s < s_hi; s += NTHR)
-            if (((coll[s >> 5] >> (s & 31)) & 1u) && s % parts == part) {
+            if ((coll[s >> 5] >> (s & 31)) & 1u) {
+                uint32_t c = 0, c_s0 = 0, c_s1 = 0;
+                if (LISTED) {  // a part takes whole chunks
+                    c = q.ex.short_chunk[s];
+                    if (c % parts != part) continue;
+                    c_s0 = q.ex.chunk_short_off[c];
+                    c_s1 = q.ex.chunk_short_off[c + 1];
+                }
                 const uint32_t i0 = q.short_i0[s], b = q.use_th ? q.short_blk[s] - b0 : 0u;
-                list[atomicAdd(&M->n_list, 1u)] = make_uint4(i0, (q.short_i0[s + 1] - i0) | (b << 20), s, 0u);
+                list[atomicAdd(&M->n_list, 1u)] = make_uint2(i0, (q.short_i0[s + 1] - i0) | (b << 20));
+                if (LISTED && s == c_s0) {  // what is occupied when the chunk begins, its operands
+                    const uint32_t e0 = q.sen_off[s], o0 = q.op_off[i0];
+                    chunks[atomicAdd(&M->n_chunks, 1u)] = make_uint4(e0, q.sen_off[s + 1] - e0, o0, q.op_off[q.short_i0[c_s1]] - o0);
+                }
             }
+        auto count_member = [&](uint32_t j, uint32_t reg, uint32_t w) {
+            uint32_t b = b0;
+            while (b + 1 < b1 && M->th_off[b + 1] <= j) ++b;
+            if (reg + w <= q.R) {
+                uint32_t *c = cv + (b - b0) * q.R + reg;
+                atomicAdd(c, 0x10001u);
+                for (uint32_t r = 1; r < w; ++r) atomicAdd(c + r, 1u);
+            }
+        };
+        const uint32_t th0 = q.use_th ? M->th_off[b0] : 0u, th1 = q.use_th ? M->th_off[b1] : 0u;
         if (LISTED) {
-            __syncthreads();
-            const uint32_t n_list = M->n_list, n_th = q.use_th ? M->th_off[b1] - M->th_off[b0] : 0u, th0 = q.use_th ? M->th_off[b0] : 0u;
+            // T and W of the n vregs that of(0 .. n - 1) names, by threads first, first + step, ...; then(j, register, width)
             constexpr int FU = 6;
-            // T and W of the n vregs that of(0 .. n - 1) names, by threads first, first + step, ...
-            auto fetch = [&](uint32_t n, uint32_t first, uint32_t step, auto of) {
+            auto fetch = [&](uint32_t n, uint32_t first, uint32_t step, auto of, auto then) {
                 for (uint32_t j0 = first; j0 < n; j0 += FU * step) {
                     uint32_t v[FU], pos[FU], w[FU], t[FU];
 #pragma unroll
                     for (int u = 0; u < FU; ++u) v[u] = of(min(j0 + u * step, n - 1));
 #pragma unroll
-                    for (int u = 0; u < FU; ++u) { pos[u] = q.first_occ[v[u]]; w[u] = q.vinfo[v[u]]; }
+                    for (int u = 0; u < FU; ++u) { pos[u] = q.first_occ[v[u]]; w[u] = q.vinfo[v[u]] & 0xFFu; }
 #pragma unroll
                     for (int u = 0; u < FU; ++u) t[u] = row[pos[u] != 0xFFFFFFFFu ? pos[u] : 0u];
 #pragma unroll
                     for (int u = 0; u < FU; ++u) {  // (several threads may store the same value)
-                        T[v[u]] = pos[u] != 0xFFFFFFFFu ? (uint16_t)t[u] : (uint16_t)0;
+                        if (pos[u] == 0xFFFFFFFFu) t[u] = 0;
+                        T[v[u]] = (uint16_t)t[u];
                         W[v[u]] = (uint8_t)w[u];
+                        if (j0 + u * step < n) then(j0 + u * step, t[u], w[u]);
                     }
                 }
             };
-            if (n_list * q.short_len * 4 >= q.V) {
-                fetch(q.V, tid, NTHR, [](uint32_t j) { return j; });
-            } else {
-                fetch(n_th, tid, NTHR, [&](uint32_t j) { return q.th[th0 + j] & 0xFFFFu; });
-                // what is occupied when the short chunk begins, and its operands: a warp takes a short chunk
-                for (uint32_t l = tid >> 5; l < n_list; l += NTHR / 32) {
-                    const uint4 x = list[l];
-                    const uint32_t e0 = q.sen_off[x.z], e1 = q.sen_off[x.z + 1], o0 = q.op_off[x.x], o1 = q.op_off[x.x + (x.y & 0xFFFFFu)];
-                    fetch(e1 - e0, lane, 32, [&](uint32_t j) { return q.sen[e0 + j] & 0xFFFFu; });
-                    fetch(o1 - o0, lane, 32, [&](uint32_t j) { return q.op_vreg[o0 + j]; });
-                }
-            }
+            auto nothing = [](uint32_t, uint32_t, uint32_t) {};
+            fetch(th1 - th0, tid, NTHR, [&](uint32_t j) { return q.th[th0 + j] & 0xFFFFu; },
+                  [&](uint32_t j, uint32_t t, uint32_t w) { count_member(th0 + j, t, w); });
             if (tid == 0) { T[q.V] = 0; W[q.V] = 0; }
             __syncthreads();
-        }
-        if (q.use_th)
-            for (uint32_t j = M->th_off[b0] + tid; j < M->th_off[b1]; j += NTHR) {
-                const uint32_t v = q.th[j] & 0xFFFFu, reg = T[v], w = W[v];
-                uint32_t b = b0;
-                while (b + 1 < b1 && M->th_off[b + 1] <= j) ++b;
-                if (reg + w <= q.R) {
-                    uint32_t *c = cv + (b - b0) * q.R + reg;
-                    atomicAdd(c, 0x10001u);
-                    for (uint32_t r = 1; r < w; ++r) atomicAdd(c + r, 1u);
+            const uint32_t n_chunks = M->n_chunks;
+            if (n_chunks * 512 >= q.V) {
+                fetch(q.V, tid, NTHR, [](uint32_t j) { return j; }, nothing);
+            } else {  // everything live inside a chunk is occupied when it begins or an operand of it
+                for (uint32_t l = tid / (NTHR / 2); l < n_chunks; l += 2) {
+                    const uint4 x = chunks[l];
+                    fetch(x.y + x.w, tid % (NTHR / 2), NTHR / 2,
+                          [&](uint32_t j) { return j < x.y ? q.sen[x.x + j] & 0xFFFFu : q.op_vreg[x.z + j - x.y]; }, nothing);
                 }
             }
+        } else {
+            for (uint32_t j = th0 + tid; j < th1; j += NTHR) {
+                const uint32_t v = q.th[j] & 0xFFFFu;
+                count_member(j, T[v], W[v]);
+            }
+        }
         __syncthreads();
         const uint32_t n_list = M->n_list;
         // through-set members of block b other than v (itself a member: `member`) that overlap v's range
@@ -278,13 +312,15 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
         // through-set from the arrays.  The record of the instruction after the next and the first list entries
         // of the next are fetched meanwhile.  (Bound by instruction issue: the lists of loop bodies hold 4 to 10
         // entries, and few of them sit near enough to be looked at more closely.)
-        constexpr int LU = 8, LT = 16;  // list entries in flight: the first of a list, the others
+        // List entries come four at a time (one request for each entry and lane kept the L1 tags busy for longer than
+        // the comparisons take): LQ pieces of the next instruction's list in flight, then LT at a time.
+        constexpr int LQ = 3, LT = 4;
         const uint32_t step_unit = NTHR / q.short_len, step_at = NTHR % q.short_len;
         uint32_t unit = tid / q.short_len, at = tid % q.short_len;  // (advances by NTHR instructions)
         auto next_instr = [&](uint32_t &b) -> uint32_t {  // 0xFFFFFFFF: beyond the short chunk, or beyond the list
             uint32_t i = 0xFFFFFFFFu;
             if (unit < n_list) {
-                const uint4 span = list[unit];
+                const uint2 span = list[unit];
                 if (at < (span.y & 0xFFFFFu)) i = span.x + at;
                 b = b0 + (span.y >> 20);
             }
@@ -294,16 +330,18 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
             return i;
         };
         auto fetch_rec = [&](uint32_t i) { return q.irec[min(i, q.nI - 1)]; };  // (looked at only if i is one)
-        uint32_t us_nx[LU], rd_nx[4];
+        uint32_t rd_nx[4];
+        uint4 us_nx[LQ];
+        const uint4 *ls4 = reinterpret_cast<const uint4 *>(q.ls);
         auto fetch_list = [&](const uint4 &r) {
-            const uint32_t n = r.y & 0xFFFFu, last = n ? n - 1 : 0u;
+            const uint32_t n = r.y & 0xFFFFu, p0 = r.x >> 2, p1 = n ? (r.x + n - 1) >> 2 : p0;
             if (LISTED) {
                 const uint32_t nr = (r.y >> 24) & 127u, o = r.w + ((r.y >> 16) & 0xFFu);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) rd_nx[u] = q.op_vreg[nr ? o + min((uint32_t)u, nr - 1) : 0u];
             }
 #pragma unroll
-            for (int u = 0; u < LU; ++u) us_nx[u] = q.ls[r.x + min((uint32_t)u, last)];
+            for (int u = 0; u < LQ; ++u) us_nx[u] = ls4[min(p0 + u, p1)];
         };
         const uint32_t n_slots = n_list * q.short_len;
         if (n_slots) {
@@ -313,9 +351,9 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
             for (uint32_t f = tid; f < n_slots; f += NTHR) {
                 const uint32_t i = i_nx, b = b_nx;
                 const uint4 rec = rec_nx;
-                uint32_t us[LU], ts[LU], rd[4];
+                uint32_t us[4 * LQ], ts[4 * LQ], rd[4];
 #pragma unroll
-                for (int u = 0; u < LU; ++u) us[u] = us_nx[u];
+                for (int u = 0; u < LQ; ++u) { us[4 * u] = us_nx[u].x; us[4 * u + 1] = us_nx[u].y; us[4 * u + 2] = us_nx[u].z; us[4 * u + 3] = us_nx[u].w; }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) rd[u] = LISTED ? rd_nx[u] : 0u;
                 i_nx = i_nx2;
@@ -339,8 +377,13 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
                 }
                 if (!nd) continue;
                 uint32_t cnt = 0;
+                const uint32_t skip = rec.x & 3u;  // (the list begins inside its first piece)
 #pragma unroll
-                for (int u = 0; u < LU; ++u) ts[u] = T[(uint32_t)u < n ? us[u] : q.V];
+                for (int u = 0; u < 4 * LQ; ++u) {
+                    const bool entry = (uint32_t)u - skip < n;
+                    ts[u] = T[entry ? us[u] : q.V];
+                    if (!entry) ts[u] = 0x1000000u;  // (near nothing)
+                }
                 for (uint32_t d = 0; d < nd; ++d) {
                     const uint32_t v = d ? q.op_vreg[rec.w + d] : rec.z, sv = T[v], wv = W[v];
                     // [t, t + wt) overlaps [sv, sv + wv): t < sv + wv and t > sv - wt, wt at most wmax
@@ -348,20 +391,32 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
                     cnt += through_overlaps(b, v, d ? (q.blk_th[(size_t)b * q.Wv + (v >> 5)] >> (v & 31)) & 1u : rec.y >> 31);
                     bool near = false;
 #pragma unroll
-                    for (int u = 0; u < LU; ++u) near |= ts[u] + shift < span;
+                    for (int u = 0; u < 4 * LQ; ++u) near |= ts[u] + shift < span;
                     if (near) {
 #pragma unroll
-                        for (int u = 0; u < LU; ++u)
-                            if ((uint32_t)u < n && us[u] != v && overlap(sv, wv, ts[u], W[us[u]])) ++cnt;
+                        for (int u = 0; u < 4 * LQ; ++u)
+                            if (ts[u] + shift < span && us[u] != v && ts[u] + W[us[u]] > sv) ++cnt;
                     }
-                    for (uint32_t e0 = LU; e0 < n; e0 += LT) {
-                        uint32_t x[LT];
+                    for (uint32_t p = (rec.x >> 2) + LQ; p * 4 < rec.x + n; p += LT) {
+                        uint4 x4[LT];
 #pragma unroll
-                        for (int u = 0; u < LT; ++u) x[u] = q.ls[rec.x + min(e0 + u, n - 1)];
+                        for (int u = 0; u < LT; ++u) x4[u] = ls4[min(p + u, (rec.x + n - 1) >> 2)];
+                        uint32_t x[4 * LT], t[4 * LT];
 #pragma unroll
-                        for (int u = 0; u < LT; ++u) {
-                            const uint32_t t = T[x[u]];
-                            if (t + shift < span && e0 + u < n && x[u] != v && t + W[x[u]] > sv) ++cnt;
+                        for (int u = 0; u < LT; ++u) { x[4 * u] = x4[u].x; x[4 * u + 1] = x4[u].y; x[4 * u + 2] = x4[u].z; x[4 * u + 3] = x4[u].w; }
+                        bool hit = false;
+#pragma unroll
+                        for (int u = 0; u < 4 * LT; ++u) {
+                            const bool entry = p * 4 + u < rec.x + n;
+                            t[u] = T[entry ? x[u] : q.V];
+                            if (!entry) t[u] = 0x1000000u;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4 * LT; ++u) hit |= t[u] + shift < span;
+                        if (hit) {
+#pragma unroll
+                            for (int u = 0; u < 4 * LT; ++u)
+                                if (t[u] + shift < span && x[u] != v && t[u] + W[x[u]] > sv) ++cnt;
                         }
                     }
                     if (nd > 1)  // co-defined vregs that are not live after the instruction
@@ -376,11 +431,14 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
         }
         // In a chunk whose own walk was clean everything that is live is disjoint from the through-set; a
         // definition without an event (a member redefined from itself) overlaps the members that overlap it.
+        uint32_t unit_no = 0;  // 4 NTHR entries or instructions; a part takes every parts-th
         for (uint32_t b = b0; b < b1 && thcol; ++b) {
             if (!((thcol >> b) & 1u)) continue;
-            const uint32_t n_el = q.el_count[b];
-            const uint4 *el = q.el + q.op_off[q.blk_off[b]];  // instruction, chunk, vreg | member << 31, short chunk
-            for (uint32_t e0 = part * 4 * NTHR + tid; e0 < n_el; e0 += parts * 4 * NTHR) {
+            const uint32_t n_el = M->el_n[b];
+            const uint4 *el = q.el + M->el_o[b];  // instruction, chunk, vreg | member << 31, short chunk
+            for (uint32_t u0 = 0; u0 < n_el; u0 += 4 * NTHR) {
+                if (unit_no++ % parts != part) continue;
+                const uint32_t e0 = u0 + tid;
                 uint4 x[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) x[u] = el[min(e0 + u * NTHR, n_el - 1)];
@@ -391,29 +449,27 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
                     if (n) { pairs += n; mind = min(mind, x[u].x); }
                 }
             }
-            if (LISTED) {  // sources of its instructions that are both in the through-set
-                const uint32_t i1 = q.blk_off[b + 1];
-                for (uint32_t i0 = q.blk_off[b] + part * 4 * NTHR + tid; i0 < i1; i0 += parts * 4 * NTHR) {
-                    uint4 rec[4];
-                    uint32_t rd[4][4];
+            if (!LISTED) continue;
+            // sources of the block's instructions that are both in the through-set
+            const uint32_t i1 = M->blk_i[b + 1];
+            for (uint32_t u0 = M->blk_i[b]; u0 < i1; u0 += 4 * NTHR) {
+                if (unit_no++ % parts != part) continue;
+                const uint32_t i0 = u0 + tid;
+                uint4 rec[4];
+                uint32_t rd[4][4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) rec[u] = q.irec[min(i0 + u * NTHR, i1 - 1)];
+                for (int u = 0; u < 4; ++u) rec[u] = q.irec[min(i0 + u * NTHR, i1 - 1)];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const uint32_t nr = (rec[u].y >> 24) & 127u, o = rec[u].w + ((rec[u].y >> 16) & 0xFFu);
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t nr = (rec[u].y >> 24) & 127u, o = rec[u].w + ((rec[u].y >> 16) & 0xFFu);
 #pragma unroll
-                        for (int r = 0; r < 4; ++r) rd[u][r] = q.op_vreg[nr ? o + min((uint32_t)r, nr - 1) : 0u];
-                    }
+                    for (int r = 0; r < 4; ++r) rd[u][r] = q.op_vreg[nr ? o + min((uint32_t)r, nr - 1) : 0u];
+                }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const uint32_t i = i0 + u * NTHR, nr = (rec[u].y >> 24) & 127u;
-                        if (i >= i1 || nr < 2) continue;
-                        if (nr <= 4) {
-                            if (duplicates(rd[u], T)) dups += member_duplicates(q, T, b, i);
-                        } else {
-                            dups += member_duplicates(q, T, b, i);
-                        }
-                    }
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t i = i0 + u * NTHR, nr = (rec[u].y >> 24) & 127u;
+                    if (i >= i1 || nr < 2) continue;
+                    if (nr > 4 || duplicates(rd[u], T)) dups += member_duplicates(q, T, b, i);
                 }
             }
         }
@@ -446,7 +502,7 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
     uint32_t *s_th = reinterpret_cast<uint32_t *>(smem + q.sm.th);    // [nB][Wp] through-set masks
     uint32_t *occ = reinterpret_cast<uint32_t *>(smem + q.sm.occ);    // [Wp][NTHR] masks; counts in step 5
     uint32_t *coll = reinterpret_cast<uint32_t *>(smem + q.sm.coll);  // short chunks that collided
-    uint4 *list = reinterpret_cast<uint4 *>(smem + q.sm.list);        // the same as a list, in step 5
+    uint2 *list = reinterpret_cast<uint2 *>(smem + q.sm.list);        // the same as a list, in step 5
     FMisc *M = reinterpret_cast<FMisc *>(smem + q.sm.misc);
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t k = blockIdx.x;
@@ -456,7 +512,7 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
         M->flags = M->bank = M->pairs = M->thcol = M->any = 0;
         M->minop = M->minr = M->mind = 0xFFFFFFFFu;
     }
-    if (tid <= 32) M->th_off[tid] = q.use_th ? q.th_off[min(tid, q.nB)] : 0u;
+    load_blocks(q, M);
     if (q.use_th)
         for (uint32_t j = tid; j < q.nB * q.Wp; j += NTHR) s_th[j] = 0;
     __syncthreads();
@@ -739,7 +795,7 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
     uint16_t *T = reinterpret_cast<uint16_t *>(base);
     uint8_t *W = base + q.sm.w;
     uint32_t *occ = reinterpret_cast<uint32_t *>(base + q.sm.occ), *coll = reinterpret_cast<uint32_t *>(base + q.sm.coll);
-    uint4 *list = reinterpret_cast<uint4 *>(base + q.sm.list);
+    uint2 *list = reinterpret_cast<uint2 *>(base + q.sm.list);
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     const uint32_t n_items = q.ex.work[0];
     for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
@@ -755,7 +811,7 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
             M->thcol = full ? 0u : thcol;  // (with every chunk counted in full, nothing is left of the through-sets)
             M->mind = 0xFFFFFFFFu;
         }
-        if (tid <= 32) M->th_off[tid] = q.use_th ? q.th_off[min(tid, q.nB)] : 0u;
+        load_blocks(q, M);
         const bool count = (walk | thcol) != 0;
         if (count)
             for (uint32_t s = tid; s < ((q.nS + 31u) & ~31u); s += EXACT_NT) {
@@ -932,7 +988,7 @@ static FSmem exact_smem(const vl_program *p)
     s.cb = p->use_th ? std::max(1u, std::min(p->nB, 48u * 1024u / counts)) : p->nB;
     s.coll = s.occ + (p->use_th ? up16(s.cb * counts) : 0u);
     s.list = s.coll + up16((p->nS + 31) / 32 * 4 + 4);
-    s.total = s.list + p->nS * 16;
+    s.total = s.list + up16(p->nS * 8) + p->nC * 16;
     return s;
 }
 

@@ -237,7 +237,7 @@ enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_NOUT = 3, CS_OUTV = 4, CS_OUT
 enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
 struct VlExactArgs {
     const uint32_t *work, *cstate, *anom;
-    const uint32_t *short_chunk;  // [nS] chunk of every short chunk
+    const uint32_t *short_chunk, *chunk_short_off;  // [nS] chunk of every short chunk, [nC + 1] first short chunk of every chunk
     uint32_t *racc;               // [rows][4] overlaps, complement of the lowest instruction, bank tally, parts done; all 0
     uint32_t AW;
     unsigned char *scratch;       // vl_exact_scratch bytes, null if 0

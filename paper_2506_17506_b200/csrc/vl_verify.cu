@@ -1853,7 +1853,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     }
     kt_mark(p, st);
     VlExactArgs ex{};
-    ex.work = vs.work; ex.cstate = vs.cstate; ex.anom = vs.anom; ex.short_chunk = p->d_short_chunk; ex.racc = vs.racc;
+    ex.work = vs.work; ex.cstate = vs.cstate; ex.anom = vs.anom; ex.short_chunk = p->d_short_chunk; ex.chunk_short_off = p->d_chunk_short_off; ex.racc = vs.racc;
     ex.AW = (uint32_t)vs.aw; ex.scratch = vs.exact;
     if ((rc = vl_exact_run(p, ex, d_cand, pitch, d_out, st, dict)) != VL_OK) return rc;
     kt_mark(p, st);

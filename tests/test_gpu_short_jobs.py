@@ -49,3 +49,21 @@ def test_row_counts_and_many_short_chunks(B, oracle_mod, K, chunk):
     op = oracle_mod.OracleProgram(p)
     _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows), f"K {K} chunk {chunk}")
     gp.close()
+
+
+def test_exact_counts_in_global_memory(B, oracle_mod):
+    """52,000 vregs and 20,000 registers: the block arrays of the exact counts do not fit a multiprocessor."""
+    V = 52000
+    blocks = [[([i], [i - 1, i - 2, i - 40] if i >= 40 else []) for i in range(V)]]
+    p = synth.program_from_lists(blocks, [], V, [1 + (v % 3 == 0) for v in range(V)], 20000)
+    gp = B.Program(p)
+    gp.set_option(B.VL_OPT_GROUP, 1)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    rng = np.random.default_rng(5)
+    good = (np.arange(V) * 2) % 20000
+    tables = [good, np.where(rng.random(V) < 1e-3, 20005, good), np.where(rng.random(V) < 1e-2, 7, good), rng.integers(0, 20000, V)]
+    rows = np.stack([H.row_from_table(p, t) for t in tables])
+    _assert_same(_gpu_verify(B, gp, rows), op.verify(lv, rows), "global")
+    gp.close()
