@@ -1681,23 +1681,23 @@ struct PassPlan {
 int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
 {
     const uint32_t SM_BYTES = 227 * 1024;
-    // preference: eight candidates per block (two blocks of 256 threads per SM if the tables are small,
-    // else one block of 512 threads), then the largest group that still lets two blocks share an SM,
-    // then anything that fits
+    // Preference: eight candidates per block (two blocks of 256 threads per SM if the tables are small, else one block of
+    // 512 threads), then as many candidates per block as fit an SM, with 512 threads if the copy ring leaves room for
+    // theirs: a lookup serves every candidate of the block.  1,000 rows of 20,000 vregs: four candidates and 512 threads
+    // 158 us, 256 threads 209, two candidates 261 and 352, one 382 and 515; of 28,000 vregs (two fit) 293, 387, 455, 593.
     Plan pl{};
     const uint32_t groups[3] = {4, 2, 1};
-    const uint32_t NT = p->threads_opt ? p->threads_opt : 256;
     if (p->group_opt == 0 || p->group_opt == 8) {
         pl = make_plan8(p, p->threads_opt ? p->threads_opt : 256, SM_BYTES / 2 - 1024);
         if (!pl.ok) pl = make_plan8(p, p->threads_opt ? p->threads_opt : 512, SM_BYTES);
         if (!pl.ok && !p->threads_opt) pl = make_plan8(p, 256, SM_BYTES);
     }
-    for (int pass = 0; pass < 2 && !pl.ok; ++pass)
-        for (uint32_t G : groups) {
-            if (p->group_opt && G != p->group_opt) continue;
-            pl = make_plan(p, G, NT, pass == 0 ? (SM_BYTES / 2 - 1024) : SM_BYTES);
-            if (pl.ok) break;
-        }
+    for (uint32_t G : groups) {
+        if (pl.ok) break;
+        if (p->group_opt && G != p->group_opt) continue;
+        if (p->threads_opt != 256) pl = make_plan(p, G, 512, SM_BYTES);
+        if (!pl.ok && p->threads_opt != 512) pl = make_plan(p, G, 256, SM_BYTES);
+    }
     if (!pl.ok) return VL_ERR_UNSUPPORTED;
     pp->pl = pl;
     pp->Wp = (p->P + p->wmax + 31) / 32;
