@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <utility>
 #include <new>
 
 #include "vl_internal.cuh"
@@ -83,13 +84,70 @@ static int validate(const vl_program_desc *d)
     return VL_OK;
 }
 
-template <typename T>
-static cudaError_t upload(T **dst, const T *src, size_t n)
+namespace {
+// Host arrays that go to the device together: one allocation, one copy.
+struct Upload {
+    std::vector<char> bytes;
+    std::vector<std::pair<void **, size_t>> places;
+    template <typename T>
+    void add(T **dst, const T *src, size_t n)
+    {
+        places.push_back({(void **)dst, bytes.size()});
+        if (n) bytes.insert(bytes.end(), (const char *)src, (const char *)src + n * sizeof(T));
+        bytes.resize((bytes.size() + 64 + 255) & ~(size_t)255);  // (at least 64 bytes behind every array)
+    }
+    cudaError_t send(void **block)
+    {
+        cudaError_t e = cudaMalloc(block, bytes.size());
+        if (e == cudaSuccess) e = cudaMemcpy(*block, bytes.data(), bytes.size(), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return e;
+        for (auto &x : places) *x.first = (char *)*block + x.second;
+        return e;
+    }
+};
+
+// Pinned slots in slabs of 512; the last slab is kept until the process exits, others go when their slots are back.
+struct PinnedSlab {
+    char *ptr;
+    uint32_t used;
+    std::vector<uint16_t> free_slots;
+};
+std::mutex g_pinned_mutex;
+std::vector<PinnedSlab> g_pinned;
+constexpr uint32_t PINNED_SLOTS = 512, PINNED_BYTES = 128;
+}  // namespace
+
+void *vl_pinned_get()
 {
-    cudaError_t e = cudaMalloc((void **)dst, std::max<size_t>(n, 1) * sizeof(T) + 64);
-    if (e != cudaSuccess) return e;
-    if (n) e = cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice);
-    return e;
+    std::lock_guard<std::mutex> lock(g_pinned_mutex);
+    for (auto &s : g_pinned)
+        if (!s.free_slots.empty()) {
+            const uint32_t j = s.free_slots.back();
+            s.free_slots.pop_back();
+            ++s.used;
+            return s.ptr + (size_t)j * PINNED_BYTES;
+        }
+    PinnedSlab s{nullptr, 1, {}};
+    if (cudaHostAlloc((void **)&s.ptr, PINNED_SLOTS * PINNED_BYTES, cudaHostAllocPortable) != cudaSuccess) return nullptr;
+    for (uint32_t j = PINNED_SLOTS; j-- > 1;) s.free_slots.push_back((uint16_t)j);
+    g_pinned.push_back(std::move(s));
+    return g_pinned.back().ptr;
+}
+
+void vl_pinned_put(void *slot)
+{
+    if (!slot) return;
+    std::lock_guard<std::mutex> lock(g_pinned_mutex);
+    for (size_t i = 0; i < g_pinned.size(); ++i) {
+        PinnedSlab &s = g_pinned[i];
+        if ((char *)slot < s.ptr || (char *)slot >= s.ptr + PINNED_SLOTS * PINNED_BYTES) continue;
+        s.free_slots.push_back((uint16_t)(((char *)slot - s.ptr) / PINNED_BYTES));
+        if (--s.used == 0 && g_pinned.size() > 1) {
+            cudaFreeHost(s.ptr);
+            g_pinned.erase(g_pinned.begin() + i);
+        }
+        return;
+    }
 }
 
 extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_program **out)
@@ -110,14 +168,14 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
     p->h_blk_off.assign(d->block_instr_off, d->block_instr_off + p->nB + 1);
     p->h_op_off.assign(d->instr_op_off, d->instr_op_off + p->nI + 1);
 
-    cudaError_t e = cudaSetDevice(device);
-    if (e == cudaSuccess) e = upload(&p->d_blk_off, d->block_instr_off, (size_t)p->nB + 1);
-    if (e == cudaSuccess) e = upload(&p->d_succ_off, d->succ_off, (size_t)p->nB + 1);
-    if (e == cudaSuccess) e = upload(&p->d_succ, d->succ, (size_t)p->nE);
-    if (e == cudaSuccess) e = upload(&p->d_op_off, d->instr_op_off, (size_t)p->nI + 1);
-    if (e == cudaSuccess) e = upload(&p->d_ndefs, d->instr_n_defs, (size_t)p->nI);
-    if (e == cudaSuccess) e = upload(&p->d_op_vreg, d->op_vreg, (size_t)p->nO);
-    if (e == cudaSuccess) e = upload(&p->d_width, d->vreg_width, (size_t)p->V);
+    Upload up;
+    up.add(&p->d_blk_off, d->block_instr_off, (size_t)p->nB + 1);
+    up.add(&p->d_succ_off, d->succ_off, (size_t)p->nB + 1);
+    up.add(&p->d_succ, d->succ, (size_t)p->nE);
+    up.add(&p->d_op_off, d->instr_op_off, (size_t)p->nI + 1);
+    up.add(&p->d_ndefs, d->instr_n_defs, (size_t)p->nI);
+    up.add(&p->d_op_vreg, d->op_vreg, (size_t)p->nO);
+    up.add(&p->d_width, d->vreg_width, (size_t)p->V);
     {   // instructions grouped by their number of distinct sources (2, 3, 4), for the bank tally
         std::vector<uint2> cls[3];
         for (uint32_t i = 0; i < p->nI; ++i) {
@@ -142,7 +200,7 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
             all.insert(all.end(), cls[c].begin(), cls[c].end());
             p->bank_seg[c + 1] = (uint32_t)all.size();
         }
-        if (e == cudaSuccess) e = upload(&p->d_bank_list, all.data(), all.size());
+        up.add(&p->d_bank_list, all.data(), all.size());
     }
     {   // The dictionary form of a candidate row (Section 3.1: one vreg -> register dictionary per basic
         // block): one entry per (block, vreg occurring in the block), blocks in order, a block's vregs
@@ -188,15 +246,17 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
                 slot[e2 / 8] |= 1ull << (e2 % 8);  // padding column: writes the spare table entry, never compared
             }
         }
-        if (e == cudaSuccess) e = upload(&p->d_dict_vreg16, v16.data(), v16.size());
-        if (e == cudaSuccess) e = upload(&p->d_dict_slotmeta, slot.data(), slot.size());
-        if (e == cudaSuccess) e = upload(&p->d_dict_opoff, off.data(), off.size());
-        if (e == cudaSuccess) e = upload(&p->d_dict_first4, f4.data(), f4.size());
-        if (e == cudaSuccess) e = upload(&p->d_dict_first_occ, first_entry.data(), first_entry.size());
-        if (e == cudaSuccess) e = upload(&p->d_dict_instr, dict_instr.data(), dict_instr.size());
+        up.add(&p->d_dict_vreg16, v16.data(), v16.size());
+        up.add(&p->d_dict_slotmeta, slot.data(), slot.size());
+        up.add(&p->d_dict_opoff, off.data(), off.size());
+        up.add(&p->d_dict_first4, f4.data(), f4.size());
+        up.add(&p->d_dict_first_occ, first_entry.data(), first_entry.size());
+        up.add(&p->d_dict_instr, dict_instr.data(), dict_instr.size());
     }
-    if (e == cudaSuccess) e = cudaMalloc((void **)&p->d_status, 64);
-    if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, 64);
+    const uint32_t no_status[16] = {0};
+    up.add(&p->d_status, no_status, 16);
+    cudaError_t e = cudaSetDevice(device);
+    if (e == cudaSuccess) e = up.send(&p->d_blob);
     if (e != cudaSuccess) {
         p->last_cuda_error = (int)e;
         vl_program_destroy(p);
@@ -210,7 +270,6 @@ void vl_free_liveness(vl_program *p)
 {
     // everything below lives in the handle's pools, which are rewound, not freed
     p->live_arena.reset();
-    p->tmp_arena.reset();
     p->d_blk_in = p->d_blk_out = p->d_lo_off = p->d_lo = nullptr;
     p->d_opflags = nullptr;  // (the operand tables live in the layout arena)
     p->d_th_off = p->d_th = p->d_cev_off = nullptr;
@@ -229,23 +288,18 @@ extern "C" void vl_program_destroy(vl_program *p)
     cudaSetDevice(p->device);
     vl_live_settle(p);
     vl_free_liveness(p);
-    if (p->h_live) cudaFreeHost(p->h_live);
+    vl_pinned_put(p->h_live);
     if (p->h_out_pinned) cudaFreeHost(p->h_out_pinned);
-    if (p->h_rs) cudaFreeHost(p->h_rs);
+    vl_pinned_put(p->h_rs);
     cudaFree(p->d_rs);
     cudaFree(p->d_diag_T);
     cudaFree(p->d_diag_n);
     if (p->ev_live) cudaEventDestroy(p->ev_live);
     p->live_arena.release();
-    p->tmp_arena.release();
     p->layout_arena.release();
-    cudaFree(p->d_blk_off); cudaFree(p->d_succ_off); cudaFree(p->d_succ); cudaFree(p->d_op_off);
-    cudaFree(p->d_ndefs); cudaFree(p->d_op_vreg); cudaFree(p->d_width); cudaFree(p->d_status);
-    cudaFree(p->d_bank_list);
-    cudaFree(p->d_dict_vreg16); cudaFree(p->d_dict_slotmeta); cudaFree(p->d_dict_opoff); cudaFree(p->d_dict_first4);
-    cudaFree(p->d_dict_instr); cudaFree(p->d_dict_first_occ);
+    cudaFree(p->d_blob);
     cudaFree(p->d_vcons); cudaFree(p->d_rs_prefix);
-    for (auto &v : p->vs) { cudaFree(v.tg); cudaFree(v.cstate); cudaFree(v.anom); cudaFree(v.work); cudaFree(v.racc); cudaFree(v.grp_done); cudaFree(v.thm); cudaFree(v.exact); }
+    for (auto &v : p->vs) cudaFree(v.block);
     for (int j = 0; j < 2; ++j) {
         cudaFree(p->d_stage[j]);
         cudaFree(p->d_stage_out[j]);

@@ -42,6 +42,7 @@ struct VlArena {
     struct Slab { char *ptr; size_t size; };
     std::vector<Slab> slabs;
     size_t cur = 0, off = 0;
+    size_t hint = 0;  // what the next slab should hold (a slab costs 20 us up to 64 KB, 330 us from 1 MB on, however large)
     cudaError_t alloc(void **out, size_t bytes)
     {
         bytes = (bytes + 64 + 255) & ~(size_t)255;
@@ -51,7 +52,8 @@ struct VlArena {
                 off += bytes;
                 return cudaSuccess;
             }
-        Slab s{nullptr, bytes > ((size_t)4 << 20) ? bytes : ((size_t)4 << 20)};
+        Slab s{nullptr, bytes > hint ? bytes : hint};
+        hint = (size_t)64 << 10;
         cudaError_t e = cudaMalloc((void **)&s.ptr, s.size);
         if (e != cudaSuccess) return e;
         slabs.push_back(s);
@@ -89,7 +91,8 @@ struct vl_program {
     bool sizes_known = false;
     unsigned long long known[6] = {0, 0, 0, 0, 0, 0};  // list entries, walk events, through-set entries, short-list entries, short-chunk events and entries
 
-    // device copies of the program
+    // device copies of the program: one allocation
+    void *d_blob = nullptr;
     uint32_t *d_blk_off = nullptr, *d_succ_off = nullptr, *d_succ = nullptr, *d_op_off = nullptr, *d_op_vreg = nullptr;
     uint8_t *d_ndefs = nullptr, *d_width = nullptr;
     uint32_t *d_chunk_i0 = nullptr, *d_chunk_i1 = nullptr, *d_chunk_blk = nullptr, *d_blk_chunk_off = nullptr;
@@ -150,7 +153,7 @@ struct vl_program {
     uint32_t test_wait = 0;  // test hook of the table kernel's bounded wait (VL_OPT_TEST_WAIT)
     int use_th = 0;
 
-    VlArena live_arena, tmp_arena;  // liveness results and tables / liveness working sets
+    VlArena live_arena;             // liveness results, tables and working sets
     VlArena layout_arena;           // chunks, pieces, walk items
     uint32_t *d_status = nullptr;  // [16] device status words
     int last_cuda_error = 0;
@@ -176,6 +179,7 @@ struct vl_program {
 
     // per-call working memory of vl_verify (one set per internal stream slot), grown on demand
     struct VScratch {
+        void *block = nullptr;       // the allocation that holds the arrays below
         uint16_t *tg = nullptr;      // [groups][V+1][64] tables, 64 candidates side by side
         uint32_t *cstate = nullptr;  // [rows][8]
         uint32_t *anom = nullptr;    // [rows][AW] chunks whose walk collided
@@ -252,6 +256,9 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
 // follows the VL_LANES lanes in the array) and the handle's fork / join events.
 int vl_lane_streams(vl_program *p, cudaStream_t **lanes, cudaEvent_t **done = nullptr);
 void vl_free_liveness(vl_program *p);
+// 128 bytes of pinned host memory (a pinned allocation of its own takes 155 us); null if there is none.
+void *vl_pinned_get();
+void vl_pinned_put(void *slot);
 // Waits for a liveness run that is still in flight and checks its outcome; VL_OK if none is pending.
 int vl_live_settle(vl_program *p);
 int vl_live_join(vl_program *p, cudaStream_t st);  // st waits for the liveness run in flight, if any

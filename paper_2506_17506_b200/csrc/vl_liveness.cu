@@ -875,7 +875,6 @@ int live_attributes(vl_program *p)
 }
 }  // namespace
 #define KEEP(out, n) VL_CUDA(p, pool_get(p->live_arena, out, n))
-#define TMP(out, n) VL_CUDA(p, pool_get(p->tmp_arena, out, n))
 #define LAYOUT(out, n) VL_CUDA(p, pool_get(p->layout_arena, out, n))
 
 // One kernel of the runs of n programs; overlap: it may start while the launch before it drains (see pdl_wait).
@@ -982,6 +981,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         all.resize((all.size() + 4) & ~(size_t)3);  // (at least one word behind every array)
     }
     uint32_t *dev = nullptr;
+    p->layout_arena.hint = all.size() * 4 + (size_t)p->V * 12 + (size_t)p->nOp8 * 3 + (size_t)p->nOpT * 5 + 16384;
     LAYOUT(&dev, all.size());
     VL_CUDA(p, cudaMemcpy(dev, all.data(), all.size() * 4, cudaMemcpyHostToDevice));
     size_t at = 0;
@@ -1015,6 +1015,9 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     vl_free_liveness(p);
     const uint32_t nB = p->nB, nI = p->nI, V = p->V, nO = p->nO, Wv = p->Wv, nC = p->nC, nP = p->nP;
 
+    // about what follows, in one slab
+    p->live_arena.hint = 4 * ((size_t)3 * nP + 4 * (size_t)nC + 5 * (size_t)nB) * Wv + (size_t)nI * 28 + (size_t)nO * 18 +
+                         (size_t)nC * 40 + (size_t)p->nS * 16 + (size_t)nB * 24 + 40 * 512;
     // ---- results and tables that do not depend on the list lengths
     KEEP(&p->d_blk_in, (size_t)2 * nB * Wv);  // live-in rows, then live-out rows
     p->d_blk_out = p->d_blk_in + (size_t)nB * Wv;
@@ -1049,31 +1052,31 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     q.chunk_i0 = p->d_chunk_i0; q.chunk_i1 = p->d_chunk_i1; q.chunk_blk = p->d_chunk_blk; q.blk_chunk_off = p->d_blk_chunk_off;
     q.piece_i0 = p->d_piece_i0; q.piece_chunk = p->d_piece_chunk; q.chunk_piece_off = p->d_chunk_piece_off;
     q.seg_c0 = p->d_seg_c0; q.blk_seg_off = p->d_blk_seg_off; q.short_p0 = p->d_short_p0; q.chunk_short_off = p->d_chunk_short_off;
-    TMP(&q.piece_use, (size_t)nP * Wv);
-    TMP(&q.piece_def, (size_t)nP * Wv);
-    TMP(&q.piece_end, (size_t)nP * Wv);
-    TMP(&q.chunk_use, (size_t)nC * Wv);
-    TMP(&q.chunk_def, (size_t)nC * Wv);
-    TMP(&q.chunk_end, (size_t)nC * Wv);
-    TMP(&q.chunk_entry, (size_t)nC * Wv);
-    TMP(&q.blk_touch, (size_t)nB * Wv);
-    TMP(&q.lo_rel, (size_t)nI);
-    TMP(&q.ev_rel, (size_t)nI);
-    TMP(&q.chunk_lo, (size_t)nC);
-    TMP(&q.chunk_ev, (size_t)nC);
-    TMP(&q.chunk_lo0, (size_t)nC + 1);
-    TMP(&q.centry_cnt, (size_t)nC);
-    TMP(&q.short_ent, (size_t)p->nS);
-    TMP(&q.short_ev, (size_t)p->nS);
-    TMP(&q.counters, 1);
+    KEEP(&q.piece_use, (size_t)nP * Wv);
+    KEEP(&q.piece_def, (size_t)nP * Wv);
+    KEEP(&q.piece_end, (size_t)nP * Wv);
+    KEEP(&q.chunk_use, (size_t)nC * Wv);
+    KEEP(&q.chunk_def, (size_t)nC * Wv);
+    KEEP(&q.chunk_end, (size_t)nC * Wv);
+    KEEP(&q.chunk_entry, (size_t)nC * Wv);
+    KEEP(&q.blk_touch, (size_t)nB * Wv);
+    KEEP(&q.lo_rel, (size_t)nI);
+    KEEP(&q.ev_rel, (size_t)nI);
+    KEEP(&q.chunk_lo, (size_t)nC);
+    KEEP(&q.chunk_ev, (size_t)nC);
+    KEEP(&q.chunk_lo0, (size_t)nC + 1);
+    KEEP(&q.centry_cnt, (size_t)nC);
+    KEEP(&q.short_ent, (size_t)p->nS);
+    KEEP(&q.short_ev, (size_t)p->nS);
+    KEEP(&q.counters, 1);
     const uint32_t fgrid = (Wv + 31) / 32;
     size_t flow_smem = (((size_t)4 * nB + 2 * (size_t)p->nSeg) * 32 + nB + 1 + p->nE) * 4;
     if (flow_smem > 200 * 1024) {
-        TMP(&q.flow_scratch, flow_smem / 4 * fgrid);
+        KEEP(&q.flow_scratch, flow_smem / 4 * fgrid);
         flow_smem = 0;
     }
     if (!p->tables_built) {
-        TMP(&p->d_opmeta, (size_t)nO);
+        KEEP(&p->d_opmeta, (size_t)nO);
         VL_CUDA(p, cudaMemsetAsync(p->d_first_occ, 0xFF, std::max<size_t>(V, 1) * 4, st));
         VL_CUDA(p, cudaMemsetAsync(p->d_first_def_instr, 0xFF, std::max<size_t>(V, 1) * 4, st));
     }
@@ -1107,6 +1110,8 @@ static int live_lengths(vl_program *p, LiveArgs &q)
         memcpy(p->known, tot, sizeof(tot));
     }
     p->lo_len = p->known[LV_TOT_LO];
+    p->live_arena.hint = 4 * (p->known[LV_TOT_LO] + p->known[LV_TOT_LS] + p->known[LV_TOT_TH] + p->known[LV_TOT_SEV] + p->known[LV_TOT_SEN]) +
+                         14 * p->known[LV_TOT_EV] + 8 * 512;
     KEEP(&p->d_lo, (size_t)p->lo_len);
     KEEP(&p->d_ls, (size_t)p->known[LV_TOT_LS]);
     KEEP(&p->d_ev, (size_t)(p->known[LV_TOT_EV] / 8 + 2) * 7);  // two no-op groups behind the last chunk
@@ -1174,7 +1179,7 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
         vl_program *p = progs[j];
         vl_live_settle(p);  // the pinned words of an earlier run are about to be reused
         if ((rc = vl_layout(p, streams[stream_of(j)])) != VL_OK) return rc;
-        if (!p->h_live) VL_CUDA(p, cudaHostAlloc((void **)&p->h_live, 128, cudaHostAllocDefault));
+        if (!p->h_live && !(p->h_live = (uint32_t *)vl_pinned_get())) return VL_ERR_CUDA;
         if (!p->ev_live) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_live, cudaEventDisableTiming));
         if ((rc = live_begin(p, args[j], shapes[j], streams[stream_of(j)])) != VL_OK) return rc;
         lengths_known = lengths_known && p->sizes_known;

@@ -176,7 +176,7 @@ extern "C" int vl_verify_until_pass(vl_program *p, const uint16_t *d_cand, uint6
     if (!d_cand || !d_out || ((uintptr_t)d_out & 15)) return VL_ERR_INVALID_ARG;
     VL_CUDA(p, cudaSetDevice(p->device));
     if (!p->d_rs) VL_CUDA(p, cudaMalloc(&p->d_rs, sizeof(vl_sample_stats)));
-    if (!p->h_rs) VL_CUDA(p, cudaMallocHost(&p->h_rs, sizeof(vl_sample_stats)));
+    if (!p->h_rs && !(p->h_rs = (vl_sample_stats *)vl_pinned_get())) return VL_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
     for (uint64_t b0 = 0; b0 < K; b0 += batch_rows) {
         const uint64_t nb = K - b0 < batch_rows ? K - b0 : batch_rows;

@@ -1633,23 +1633,35 @@ int ensure_scratch(vl_program *p, int slot, uint64_t rows)
     const uint64_t aw = std::max(1u, (p->nC + 31) / 32);
     const uint64_t groups = (rows + TGW - 1) / TGW;
     if (v.rows >= rows && v.aw == aw && v.vregs == p->V && v.chunks == p->nC) return VL_OK;
-    cudaFree(v.tg); cudaFree(v.cstate); cudaFree(v.anom); cudaFree(v.work); cudaFree(v.racc); cudaFree(v.grp_done); cudaFree(v.thm); cudaFree(v.exact);
-    v.exact = nullptr;
-    v.tg = nullptr; v.cstate = nullptr; v.anom = nullptr; v.work = nullptr; v.racc = nullptr; v.grp_done = nullptr; v.thm = nullptr;
-    v.rows = 0;
-    VL_CUDA(p, cudaMalloc((void **)&v.tg, groups * (p->V + 1) * TGW * sizeof(uint16_t)));
-    VL_CUDA(p, cudaMemset(v.tg, 0, groups * (p->V + 1) * TGW * sizeof(uint16_t)));
-    VL_CUDA(p, cudaMalloc((void **)&v.cstate, groups * TGW * 8 * sizeof(uint32_t)));
-    VL_CUDA(p, cudaMemset(v.cstate, 0, groups * TGW * 8 * sizeof(uint32_t)));
-    VL_CUDA(p, cudaMalloc((void **)&v.anom, groups * TGW * aw * sizeof(uint32_t)));
-    VL_CUDA(p, cudaMalloc((void **)&v.work, (EXACT_HDR + 2 * EXACT_MAX_PARTS * groups * TGW) * sizeof(uint32_t)));
-    if (vl_exact_scratch(p)) VL_CUDA(p, cudaMalloc((void **)&v.exact, vl_exact_scratch(p)));
-    VL_CUDA(p, cudaMalloc((void **)&v.racc, groups * TGW * 4 * sizeof(uint32_t)));
-    // walk blocks finished per group, then the groups' straddle-mark flags (reset by the walk)
-    VL_CUDA(p, cudaMalloc((void **)&v.grp_done, 2 * (groups + 1) * sizeof(uint32_t)));
-    VL_CUDA(p, cudaMemset(v.grp_done, 0, 2 * (groups + 1) * sizeof(uint32_t)));
-    // through-set masks of every (group, program block), in the walk's layout
-    VL_CUDA(p, cudaMalloc((void **)&v.thm, std::max<uint64_t>(1, groups * p->nB * ((p->P + p->wmax + 31) / 32) * 64) * sizeof(uint32_t)));
+    cudaFree(v.block);
+    v = vl_program::VScratch{};
+    struct Part { void **dst; uint64_t bytes; };
+    const Part parts[] = {
+        // zero to begin with: the tables (no-op events look up the spare entry, rows beyond the last keep what they have),
+        // the candidates' state, and walk blocks finished per group, then the groups' straddle-mark flags (reset by the walk)
+        {(void **)&v.cstate, groups * TGW * 8 * sizeof(uint32_t)},
+        {(void **)&v.grp_done, 2 * (groups + 1) * sizeof(uint32_t)},
+        {(void **)&v.tg, groups * (p->V + 1) * TGW * sizeof(uint16_t)},
+        {(void **)&v.anom, groups * TGW * aw * sizeof(uint32_t)},
+        {(void **)&v.work, (EXACT_HDR + 2 * EXACT_MAX_PARTS * groups * TGW) * sizeof(uint32_t)},
+        {(void **)&v.racc, groups * TGW * 4 * sizeof(uint32_t)},
+        // through-set masks of every (group, program block), in the walk's layout
+        {(void **)&v.thm, groups * p->nB * ((p->P + p->wmax + 31) / 32) * 64 * sizeof(uint32_t)},
+        {(void **)&v.exact, vl_exact_scratch(p)},
+    };
+    uint64_t total = 0, zero = 0;
+    for (int j = 0; j < 8; ++j) {
+        total += (parts[j].bytes + 255) & ~255ull;
+        if (j == 2) zero = total;
+    }
+    VL_CUDA(p, cudaMalloc(&v.block, total));
+    VL_CUDA(p, cudaMemset(v.block, 0, zero));
+    VL_CUDA(p, cudaStreamSynchronize(cudaStreamLegacy));  // (the passes run on streams that do not wait for it)
+    uint64_t at = 0;
+    for (const Part &x : parts) {
+        if (x.bytes) *x.dst = (char *)v.block + at;
+        at += (x.bytes + 255) & ~255ull;
+    }
     v.rows = groups * TGW;
     v.aw = aw;
     v.vregs = p->V;
