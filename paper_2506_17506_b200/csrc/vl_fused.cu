@@ -512,6 +512,8 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
         M->flags = M->bank = M->pairs = M->thcol = M->any = 0;
         M->minop = M->minr = M->mind = 0xFFFFFFFFu;
     }
+    pdl_go();
+    pdl_wait();  // (the rows, and what liveness computed)
     load_blocks(q, M);
     if (q.use_th)
         for (uint32_t j = tid; j < q.nB * q.Wp; j += NTHR) s_th[j] = 0;
@@ -797,6 +799,7 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
     uint32_t *occ = reinterpret_cast<uint32_t *>(base + q.sm.occ), *coll = reinterpret_cast<uint32_t *>(base + q.sm.coll);
     uint2 *list = reinterpret_cast<uint2 *>(base + q.sm.list);
     const uint32_t tid = threadIdx.x, lane = tid & 31;
+    pdl_wait();
     const uint32_t n_items = q.ex.work[0];
     for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
         const uint64_t k = q.ex.work[EXACT_HDR + 2 * it];
@@ -958,16 +961,15 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         if (rc != VL_OK) return rc;
     }
     if (n > 1) {
-        k_fused<256, 3, VL_FUSED_MANY><<<dim3((uint32_t)rows, n), 256, smem, st>>>(many);
+        VL_CUDA(p0, launch_overlap(k_fused<256, 3, VL_FUSED_MANY>, dim3((uint32_t)rows, n), 256, smem, st, true, many));
     } else {
         FMany<1> one;
         one.p[0] = many.p[0];
-        if (pl.threads == 512) k_fused<512, 1, 1><<<(uint32_t)rows, 512, smem, st>>>(one);
-        else if (pl.bpm == 3) k_fused<256, 3, 1><<<(uint32_t)rows, 256, smem, st>>>(one);
-        else k_fused<256, 2, 1><<<(uint32_t)rows, 256, smem, st>>>(one);
+        const dim3 grid((uint32_t)rows);
+        if (pl.threads == 512) VL_CUDA(p0, launch_overlap(k_fused<512, 1, 1>, grid, 512, smem, st, true, one));
+        else if (pl.bpm == 3) VL_CUDA(p0, launch_overlap(k_fused<256, 3, 1>, grid, 256, smem, st, true, one));
+        else VL_CUDA(p0, launch_overlap(k_fused<256, 2, 1>, grid, 256, smem, st, true, one));
     }
-    VL_CUDA(p0, cudaGetLastError());
-    g_vl_launches.fetch_add(1);
     return VL_OK;
 }
 
@@ -1004,7 +1006,8 @@ uint64_t vl_exact_scratch(vl_program *p)
     return bytes <= 224 * 1024 ? 0 : bytes * vl_exact_blocks(p);
 }
 
-int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict)
+int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st,
+                 bool dict, bool overlap)
 {
     static std::mutex mtx;
     static bool done[64];
@@ -1021,9 +1024,7 @@ int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, u
     q.ex = ex;
     q.cand = d_cand; q.pitch = pitch; q.out = d_out;
     const uint32_t grid = vl_exact_blocks(p);
-    if (ex.scratch) k_exact<true><<<grid, EXACT_NT, 0, st>>>(q);
-    else k_exact<false><<<grid, EXACT_NT, q.sm.total, st>>>(q);
-    VL_CUDA(p, cudaGetLastError());
-    g_vl_launches.fetch_add(1);
+    if (ex.scratch) VL_CUDA(p, launch_overlap(k_exact<true>, grid, EXACT_NT, 0, st, overlap, q));
+    else VL_CUDA(p, launch_overlap(k_exact<false>, grid, EXACT_NT, q.sm.total, st, overlap, q));
     return VL_OK;
 }

@@ -215,6 +215,27 @@ struct vl_program {
 
 extern std::atomic<uint64_t> g_vl_launches;
 
+// Programmatic dependent launch: a kernel's blocks may start while the kernel before it in the stream still runs; what
+// they do before pdl_wait reads the program, its layout and operand tables only.  pdl_go lets the next kernel's blocks
+// start as soon as every block of this one has.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// A launch that may (overlap) start before the launch in front of it has finished.
+template <typename... P, typename... A>
+static inline cudaError_t launch_overlap(void (*kernel)(P...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t st, bool overlap,
+                                         const A &...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = threads; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &at; cfg.numAttrs = overlap ? 1 : 0;
+    g_vl_launches.fetch_add(1);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 #define VL_CUDA(prog, call)                     \
     do {                                        \
         cudaError_t e__ = (call);               \
@@ -247,7 +268,8 @@ struct VlExactArgs {
     unsigned char *scratch;       // vl_exact_scratch bytes, null if 0
 };
 uint64_t vl_exact_scratch(vl_program *p);
-int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st, bool dict);
+int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st,
+                 bool dict, bool overlap);
 int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out,
                    cudaStream_t st, int slot, bool dict = false);
 int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K,

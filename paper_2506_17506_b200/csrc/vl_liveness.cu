@@ -74,11 +74,6 @@ enum { LV_TOT_LO = 0, LV_TOT_EV = 1, LV_TOT_TH = 2, LV_TOT_LS = 3, LV_TOT_SEV = 
 // ------------------------------------------------------------------ device helpers
 __device__ __forceinline__ bool bit_get(const uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; }
 
-// Programmatic dependent launch: a kernel's blocks may start while the kernel before it still runs; what they do
-// before pdl_wait reads the program and its layout only.  pdl_go lets the next kernel's blocks start.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Exclusive scan over the threads of a block (a whole number of warps, at most 32), any integer type;
 // *total gets the block sum.  s_scan needs 34 elements.  Contains barriers.
 template <typename T>
@@ -148,6 +143,7 @@ __global__ void __launch_bounds__(PC_NT) k_sets(const __grid_constant__ LiveMany
     LIVE_ARGS;
     extern __shared__ uint32_t sm[];
     const uint32_t c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_wait();
     pdl_go();
     // what later kernels of the run update with atomics starts at zero
     for (size_t i = (size_t)c * blockDim.x + tid; i < (size_t)q.nB * q.Wv; i += (size_t)gridDim.x * blockDim.x) q.blk_touch[i] = 0;
@@ -713,6 +709,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
     extern __shared__ uint32_t sm[];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t role = blockIdx.x;
+    pdl_go();
     const uint32_t n_list = (q.nP + LV_WARPS - 1) / LV_WARPS, n_short = ((q.nS + 31) & ~31u) / LV_WARPS;
     if (role < n_list) {
         // Backward walk of one piece.  Two lists per instruction: the vregs live after it, ascending, and the same
@@ -876,22 +873,6 @@ int live_attributes(vl_program *p)
 }  // namespace
 #define KEEP(out, n) VL_CUDA(p, pool_get(p->live_arena, out, n))
 #define LAYOUT(out, n) VL_CUDA(p, pool_get(p->layout_arena, out, n))
-
-// One kernel of the runs of n programs; overlap: it may start while the launch before it drains (see pdl_wait).
-template <int N>
-static cudaError_t launch_live(void (*kernel)(const LiveMany<N>), uint32_t grid, uint32_t n, uint32_t nt, size_t smem,
-                               cudaStream_t st, const LiveMany<N> &args, bool overlap)
-{
-    if (!grid) return cudaSuccess;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid, n); cfg.blockDim = nt; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cfg.attrs = &at; cfg.numAttrs = overlap ? 1 : 0;
-    g_vl_launches.fetch_add(1);
-    return cudaLaunchKernelEx(&cfg, kernel, args);
-}
 
 #define LAUNCH(kernel, grid, nt, smem, st, ...)                 \
     do {                                                        \
@@ -1153,13 +1134,13 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
         many.p[j] = args[j];
     }
     if (fill) {
-        VL_CUDA(p, launch_live<N>(k_fill<N>, sh.fills, n, LV_NT, sh.fill_smem, st, many, true));
+        VL_CUDA(p, launch_overlap(k_fill<N>, dim3(sh.fills, n), LV_NT, sh.fill_smem, st, true, many));
         return VL_OK;
     }
-    VL_CUDA(p, launch_live<N>(k_sets<N>, sh.sets, n, sh.set_warps * 32, sh.sets_smem, st, many, false));
-    VL_CUDA(p, launch_live<N>(k_flow<N>, sh.flows, n, FLOW_WARPS * 32, sh.flow_smem, st, many, true));
-    VL_CUDA(p, launch_live<N>(k_count<N>, sh.counts, n, PC_NT, 0, st, many, true));
-    VL_CUDA(p, launch_live<N>(k_offsets<N>, sh.offs, n, OFF_NT, 0, st, many, true));
+    VL_CUDA(p, launch_overlap(k_sets<N>, dim3(sh.sets, n), sh.set_warps * 32, sh.sets_smem, st, true, many));
+    VL_CUDA(p, launch_overlap(k_flow<N>, dim3(sh.flows, n), FLOW_WARPS * 32, sh.flow_smem, st, true, many));
+    if (sh.counts) VL_CUDA(p, launch_overlap(k_count<N>, dim3(sh.counts, n), PC_NT, 0, st, true, many));
+    VL_CUDA(p, launch_overlap(k_offsets<N>, dim3(sh.offs, n), OFF_NT, 0, st, true, many));
     return VL_OK;
 }
 

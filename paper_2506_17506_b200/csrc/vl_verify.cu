@@ -62,6 +62,7 @@ struct TParams {
     const uint32_t *entry_instr;
     uint32_t tg_rows;     // k_tables8: vregs per bulk store of the table (rows of the box of the tg tensor)
     uint32_t *grp_flag;   // per group of 64 candidates: some table entry carries the straddle mark
+    uint32_t early;       // the kernels behind this one may start early (calls of one pass)
     uint32_t test_wait;   // test hook: the wait for tile 0 polls a barrier nothing completes, with a short limit
     uint32_t pf;          // tiles asked into L2 ahead of the copy ring
     uint32_t stagger_ns, stagger_blocks;  // k_tables8: start offset between the four classes of the first wave's blocks
@@ -83,7 +84,7 @@ struct TMisc {
 };
 
 struct WParams {
-    uint32_t V, P, nB, nC, Wp, AW, use_th, wmax;
+    uint32_t V, P, nB, nC, Wp, AW, use_th, wmax, early;
     uint64_t K;
     const uint32_t *th_off, *th, *cev_off;
     uint32_t *thm;  // [groups][nB][Wp][2][32] through-set masks (k_through -> k_walk)
@@ -265,7 +266,8 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
         for (uint32_t s = 0; s < q.NS; ++s) mbar_init(&M->bar[s], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // state of this pass that the walk and the recount update with atomics starts at zero
+    if (q.early) pdl_go();
+    // state of this pass that the walk and the exact count update with atomics starts at zero
     for (uint32_t j = tid; j < G * q.AW; j += NT) q.anom[k0 * q.AW + j] = 0;
     if (tid < G * 4) q.racc[k0 * 4 + tid] = 0;
     if (tid == 0 && (k0 & (TGW - 1)) == 0) q.grp_done[k0 / TGW] = 0;
@@ -663,7 +665,8 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         T[q.V] = make_uint4(0, 0, 0, 0);  // the spare entry: what padding operands are compared with
     }
-    // state of this pass that the walk and the recount update with atomics starts at zero
+    if (q.early) pdl_go();
+    // state of this pass that the walk and the exact count update with atomics starts at zero
     for (uint32_t j = tid; j < G * q.AW; j += NT) q.anom[k0 * q.AW + j] = 0;
     if (tid < G * 4) q.racc[k0 * 4 + tid] = 0;
     if (tid == 0 && (k0 & (TGW - 1)) == 0) q.grp_done[k0 / TGW] = 0;
@@ -1365,9 +1368,11 @@ __global__ void __launch_bounds__(256) k_through(const WParams q)
     const uint32_t b = blockIdx.x, grp = blockIdx.y;
     const uint64_t kA = (uint64_t)grp * TGW + 2 * lane, kB = kA + 1;
     uint32_t *csA = q.cstate + kA * 8, *csB = csA + 8;  // rows beyond K exist in the working buffers (whole groups)
+    if (q.early) pdl_go();
+    for (uint32_t i = threadIdx.x; i < q.Wp * 64; i += blockDim.x) s_th[i] = 0;
+    pdl_wait();
     const bool walkedA = kA < q.K && !(csA[CS_WALK] & WALK_FULL), walkedB = kB < q.K && !(csB[CS_WALK] & WALK_FULL);
     const unsigned char *tgb = reinterpret_cast<const unsigned char *>(q.tg + (uint64_t)grp * (q.V + 1) * TGW + 2 * lane);
-    for (uint32_t i = threadIdx.x; i < q.Wp * 64; i += blockDim.x) s_th[i] = 0;
     __syncthreads();
     bool thcolA = false, thcolB = false;
     const uint32_t e1 = q.th_off[b + 1];
@@ -1406,6 +1411,8 @@ __global__ void __launch_bounds__(256) k_through(const WParams q)
 // Shared memory per warp: [occupancy [Wp][2][32]][events of the chunk].
 __global__ void __launch_bounds__(WALK_WARPS * 32, 3) k_walk(const WParams q)
 {
+    if (q.early) pdl_go();
+    pdl_wait();
     extern __shared__ __align__(16) uint32_t wsm[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const uint32_t per_warp = q.Wp * 64 + ((q.ev_cap >> 3) + 2) * 28;  // words: 112 bytes per group of 8 events
@@ -1756,9 +1763,10 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
     return VL_OK;
 }
 
-// One pass: the four kernels over n <= sub candidates, in order on `st`, with working set `slot`.
+// One pass: the four kernels over n <= sub candidates, in order on `st`, with working set `slot`.  early: each kernel's
+// blocks may start, and wait, while the kernel before it drains (passes of other streams would miss the room they hold).
 int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t n, uint64_t pitch, vl_verdict *d_out,
-             cudaStream_t st, int slot, bool dict, bool stagger)
+             cudaStream_t st, int slot, bool dict, bool stagger, bool early)
 {
     // what the rows hold: one column per operand occurrence, or one per dictionary entry
     const uint32_t nO = dict ? p->nD : p->nO, nOp8 = dict ? p->nD8 : p->nOp8;
@@ -1788,7 +1796,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     tq.vcons = p->d_vcons; tq.rs_prefix = p->d_rs_prefix;
     tq.opoff = dict ? p->d_dict_opoff : p->d_opoff; tq.first4 = dict ? p->d_dict_first4 : p->d_first4;
     tq.grp_flag = vs.grp_done + (vs.rows / TGW + 1);
-    tq.test_wait = p->test_wait;
+    tq.test_wait = p->test_wait; tq.early = early;
     tq.pf = p->prefetch_tiles;
     tq.stagger_ns = stagger ? p->stagger_us * 1000u : 0u;
     tq.stagger_blocks = (uint32_t)vl_sm_count(p);
@@ -1833,7 +1841,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     if (p->nC) {
         WParams wq{};
         wq.V = p->V; wq.P = p->P; wq.nB = p->nB; wq.nC = p->nC; wq.Wp = pp.Wp; wq.AW = (uint32_t)vs.aw;
-        wq.use_th = (uint32_t)p->use_th; wq.K = n;
+        wq.use_th = (uint32_t)p->use_th; wq.K = n; wq.early = early;
         wq.th_off = p->d_th_off; wq.th = p->d_th; wq.cev_off = p->d_cev_off; wq.ev = p->d_ev;
         // the through-set masks come from a kernel of their own, except for small jobs
         const bool own_through = p->use_th && n >= 512;
@@ -1844,16 +1852,12 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
         wq.list_all = p->bank_fast ? 0 : 1; wq.chunk_blk = p->d_chunk_blk;
         wq.grp_done = vs.grp_done; wq.work = vs.work; wq.out = d_out;
         if (own_through) {
-            k_through<<<dim3(p->nB, ngrp), 256, pp.Wp * 64 * 4, st>>>(wq);
-            e = cudaGetLastError();
+            e = launch_overlap(k_through, dim3(p->nB, ngrp), 256, pp.Wp * 64 * 4, st, early, wq);
             if (e != cudaSuccess) { p->last_cuda_error = (int)e; return VL_ERR_CUDA; }
-            g_vl_launches.fetch_add(1);
         }
         const dim3 wgrid((p->nC + pp.walk_warps - 1) / pp.walk_warps, ngrp);
-        k_walk<<<wgrid, pp.walk_warps * 32, pp.walk_smem, st>>>(wq);
-        e = cudaGetLastError();
+        e = launch_overlap(k_walk, wgrid, pp.walk_warps * 32, pp.walk_smem, st, early, wq);
         if (e != cudaSuccess) { p->last_cuda_error = (int)e; return VL_ERR_CUDA; }
-        g_vl_launches.fetch_add(1);
     }
 
     // programs whose bank tally cannot take the fast path (banks not 1, 2 or 4, or an instruction
@@ -1867,7 +1871,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     VlExactArgs ex{};
     ex.work = vs.work; ex.cstate = vs.cstate; ex.anom = vs.anom; ex.short_chunk = p->d_short_chunk; ex.chunk_short_off = p->d_chunk_short_off; ex.racc = vs.racc;
     ex.AW = (uint32_t)vs.aw; ex.scratch = vs.exact;
-    if ((rc = vl_exact_run(p, ex, d_cand, pitch, d_out, st, dict)) != VL_OK) return rc;
+    if ((rc = vl_exact_run(p, ex, d_cand, pitch, d_out, st, dict, early && p->nC)) != VL_OK) return rc;
     kt_mark(p, st);
     return VL_OK;
 }
@@ -1888,7 +1892,7 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
     if (rc != VL_OK) return rc;
     for (uint64_t kb = 0; kb < K; kb += pp.sub) {
         rc = run_pass(p, pp, d_cand + kb * pitch, std::min(pp.sub, K - kb), pitch, d_out + kb, st, slot, dict,
-                      kb == 0 && K >= 8ull * 2 * (uint64_t)vl_sm_count(p));
+                      kb == 0 && K >= 8ull * 2 * (uint64_t)vl_sm_count(p), true);
         if (rc != VL_OK) return rc;
     }
     return VL_OK;
@@ -1973,7 +1977,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
         uint64_t s = 0;
         for (uint64_t kb = 0; kb < K[j] && rc == VL_OK; kb += pp.sub, ++s, ++job)
             rc = run_pass(p, pp, d_cand[j] + kb * pitch[j], std::min(pp.sub, K[j] - kb), pitch[j], d_out[j] + kb,
-                          lane[(base + s) % L], (int)(s % L), dict, job == 0 && K[j] >= 8ull * 2 * (uint64_t)vl_sm_count(p));
+                          lane[(base + s) % L], (int)(s % L), dict, job == 0 && K[j] >= 8ull * 2 * (uint64_t)vl_sm_count(p), false);
     }
     // join even after an error, so that the caller's stream stays ordered after what was launched
     for (uint32_t l = 0; l < L; ++l) {
