@@ -298,8 +298,8 @@ int vl_resample_stats(int device, uint32_t n, const vl_verdict *const *d_out, co
  * (HOST) receives the number of rows checked, a multiple of batch_rows or K; *first_pass (HOST) the
  * row of the first passing candidate, K if none passed.  Verdicts of the rows checked are in d_out
  * (16-byte aligned); those of later rows are not written.  The call waits for the stream after every
- * batch (the caller needs the answer to stop sampling); the first call allocates one record in
- * device and in pinned host memory.  Errors: as vl_verify.
+ * batch (the caller needs the answer to stop sampling); the first call takes one record of
+ * pinned host memory.  Errors: as vl_verify.
  */
 int vl_verify_until_pass(vl_program *prog, const uint16_t *d_cand, uint64_t K, uint64_t pitch_elems,
                          uint64_t batch_rows, vl_verdict *d_out, uint64_t *rows_checked, uint64_t *first_pass,
@@ -336,6 +336,12 @@ int vl_diagnose(vl_program *prog, const uint16_t *d_row, uint64_t cap, vl_confli
  * Errors: INVALID_ARG, LIVENESS_NOT_RUN, CUDA.
  */
 int vl_occupied_masks(vl_program *prog, const uint16_t *d_row, uint32_t *d_masks, void *cuda_stream);
+
+/*
+ * Host helper for readers that want one byte per register: out[i * P + r] = bit r of row i, for n_rows masks of
+ * ceil(P / 32) words each as vl_occupied_masks writes them.  Both arrays are HOST memory.  Errors: INVALID_ARG.
+ */
+int vl_expand_masks(const uint32_t *words, uint64_t n_rows, uint32_t P, uint8_t *out);
 
 /*
  * Block-level liveness without any allocation.  (The paper has no counterpart; this exists for

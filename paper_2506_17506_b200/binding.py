@@ -33,6 +33,7 @@ EXPORTS = ["vl_program_create", "vl_program_destroy", "vl_program_set_option", "
            "vl_liveness_result", "vl_verify", "vl_verify_batch", "vl_verify_host", "vl_verify_status",
            "vl_kernel_launches", "vl_kernel_times", "vl_last_cuda_error", "vl_strerror", "vl_block_liveness_static",
            "vl_resample_stats", "vl_verify_until_pass", "vl_program_set_constraints", "vl_diagnose", "vl_occupied_masks",
+           "vl_expand_masks",
            "vl_dict_layout", "vl_verify_dict"]
 
 VERDICT_DTYPE = np.dtype([("flags", "<u4"), ("first_violation_instr", "<i4"),
@@ -102,6 +103,8 @@ _lib.vl_diagnose.restype = C.c_int
 _lib.vl_diagnose.argtypes = [C.c_void_p, C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
 _lib.vl_occupied_masks.restype = C.c_int
 _lib.vl_occupied_masks.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
+_lib.vl_expand_masks.restype = C.c_int
+_lib.vl_expand_masks.argtypes = [C.c_void_p, C.c_uint64, C.c_uint32, C.c_void_p]
 _lib.vl_program_set_constraints.restype = C.c_int
 _lib.vl_program_set_constraints.argtypes = [C.c_void_p, C.c_void_p]
 SAMPLE_STATS_DTYPE = np.dtype([("first_pass", "<u8"), ("n_pass", "<u8")])
@@ -129,6 +132,18 @@ def _stream_ptr(stream) -> C.c_void_p:
         import torch
         stream = torch.cuda.current_stream()
     return C.c_void_p(int(getattr(stream, "cuda_stream", stream)))
+
+
+def _to_host(t, stream=None) -> np.ndarray:
+    """Bytes of a contiguous CUDA tensor that work on `stream` (default: the current one) has written, in a pinned
+    buffer of torch's host cache: read it, do not keep it."""
+    import torch
+    host = torch.empty(t.shape, dtype=t.dtype, pin_memory=True)
+    if stream is not None:
+        torch.cuda.synchronize(t.device)
+    host.copy_(t, non_blocking=True)
+    torch.cuda.current_stream(t.device).synchronize()
+    return host.numpy().reshape(-1).view(np.uint8)
 
 
 def make_desc(prog):
@@ -299,30 +314,34 @@ class Program:
         """Diagnostics of one candidate (CUDA uint16 tensor of n_operands entries or more): returns
         (conflict records [n, 3] as numpy, total count, kinds per instruction, bank histogram)."""
         import torch
-        dev = row.device
-        rec = torch.zeros((max(cap, 1), 3), dtype=torch.int32, device=dev)
-        cnt = torch.zeros(1, dtype=torch.int64, device=dev)
-        kinds = torch.zeros(max(self.n_instrs, 1), dtype=torch.uint8, device=dev)
-        hist = torch.zeros(n_banks, dtype=torch.int64, device=dev)
-        self._check(_lib.vl_diagnose(self._h, row.data_ptr(), cap, rec.data_ptr(), cnt.data_ptr(), kinds.data_ptr(),
-                                     hist.data_ptr(), _stream_ptr(stream)), "vl_diagnose")
-        torch.cuda.synchronize(dev)
-        n = int(cnt.item())
-        return (rec[: min(n, cap)].cpu().numpy().view(np.uint32), n, kinds[: self.n_instrs].cpu().numpy(),
-                hist.cpu().numpy().view(np.uint64))
+        # one buffer on the device, one copy back: count, histogram, kinds, conflict records
+        o_kinds = 8 + 8 * n_banks
+        o_rec = (o_kinds + self.n_instrs + 15) // 16 * 16
+        first = min(cap, 4096)                          # records that come with that copy; more than these are rare
+        buf = torch.empty(o_rec + 12 * max(cap, 1), dtype=torch.uint8, device=row.device)
+        ptr = buf.data_ptr()
+        self._check(_lib.vl_diagnose(self._h, row.data_ptr(), cap, ptr + o_rec, ptr, ptr + o_kinds, ptr + 8, _stream_ptr(stream)),
+                    "vl_diagnose")
+        host = _to_host(buf[: o_rec + 12 * first], stream)
+        n = int(host[:8].view(np.uint64)[0])
+        rec = host[o_rec: o_rec + 12 * min(n, first)]
+        if min(n, cap) > first:
+            rec = _to_host(buf[o_rec: o_rec + 12 * min(n, cap)], stream)
+        return (rec.copy().view(np.uint32).reshape(-1, 3), n, host[o_kinds: o_kinds + self.n_instrs].copy(),
+                host[8: o_kinds].copy().view(np.uint64))
 
     def vl_occupied_masks(self, row, P: int, stream=None):
         """uint8 numpy array [n_instrs, P]: registers the definitions of every instruction must keep off,
         for one candidate (CUDA uint16 tensor; entries >= P mean "no register yet")."""
         import torch
         W = (P + 31) // 32
-        masks = torch.zeros((max(self.n_instrs, 1), W), dtype=torch.int32, device=row.device)
+        masks = torch.empty((max(self.n_instrs, 1), W), dtype=torch.int32, device=row.device)
         self._check(_lib.vl_occupied_masks(self._h, row.data_ptr(), masks.data_ptr(), _stream_ptr(stream)),
                     "vl_occupied_masks")
-        torch.cuda.synchronize(row.device)
-        words = masks[: self.n_instrs].cpu().numpy().view(np.uint32)
-        bits = np.unpackbits(words.view(np.uint8).reshape(self.n_instrs, W * 4), axis=1, bitorder="little")
-        return bits[:, :P]
+        words = _to_host(masks, stream)
+        out = np.empty((self.n_instrs, P), dtype=np.uint8)
+        self._check(_lib.vl_expand_masks(words.ctypes.data, self.n_instrs, P, out.ctypes.data), "vl_expand_masks")
+        return out
 
     def vl_verify_status(self, stream=None):
         self._check(_lib.vl_verify_status(self._h, _stream_ptr(stream)), "vl_verify_status")
@@ -394,17 +413,18 @@ def vl_resample_stats(outs, ks=(1, 10, 100), device: int = 0, stream=None):
     Returns (records as a numpy array, summary as a dict); waits for the stream to read them back."""
     import torch
     n = len(outs)
-    stats = torch.zeros((max(n, 1), 2), dtype=torch.int64, device=f"cuda:{device}")
-    summ = torch.zeros(4 + VL_MAX_PASS_AT, dtype=torch.int64, device=f"cuda:{device}")
-    op = (C.c_void_p * max(n, 1))(*[o.data_ptr() if o.numel() else None for o in outs])
-    Ks = (C.c_uint64 * max(n, 1))(*[o.shape[0] for o in outs])
+    m = max(n, 1)
+    buf = torch.empty(2 * m + 4 + VL_MAX_PASS_AT, dtype=torch.int64, device=f"cuda:{device}")   # records, then the summary
+    op = (C.c_void_p * m)(*[o.data_ptr() or None for o in outs])
+    Ks = (C.c_uint64 * m)(*[o.shape[0] for o in outs])
     kk = (C.c_uint32 * max(len(ks), 1))(*ks)
-    rc = _lib.vl_resample_stats(device, n, op, Ks, len(ks), kk, stats.data_ptr(), summ.data_ptr(), _stream_ptr(stream))
+    ptr = buf.data_ptr()
+    rc = _lib.vl_resample_stats(device, n, op, Ks, len(ks), kk, ptr, ptr + 16 * m, _stream_ptr(stream))
     if rc != VL_OK:
         raise VlError(rc, "vl_resample_stats")
-    torch.cuda.synchronize(device)
-    rec = stats[:n].cpu().numpy().view(np.uint64).copy().view(SAMPLE_STATS_DTYPE).reshape(-1)
-    s = summ.cpu().numpy().view(np.uint64)
+    host = _to_host(buf, stream).view(np.uint64)
+    rec = host[: 2 * n].copy().view(SAMPLE_STATS_DTYPE).reshape(-1)
+    s = host[2 * m:].copy()
     return rec, dict(n_cases=int(s[0]), n_solved=int(s[1]), sum_tries=int(s[2]), max_tries=int(s[3]),
                      pass_at=[int(x) for x in s[4:4 + len(ks)]])
 

@@ -291,7 +291,6 @@ extern "C" void vl_program_destroy(vl_program *p)
     vl_pinned_put(p->h_live);
     if (p->h_out_pinned) cudaFreeHost(p->h_out_pinned);
     vl_pinned_put(p->h_rs);
-    cudaFree(p->d_rs);
     cudaFree(p->d_diag_T);
     cudaFree(p->d_diag_n);
     if (p->ev_live) cudaEventDestroy(p->ev_live);

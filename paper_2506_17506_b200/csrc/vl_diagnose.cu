@@ -154,12 +154,12 @@ extern "C" int vl_occupied_masks(vl_program *p, const uint16_t *d_row, uint32_t 
 {
     if (!p || !d_row || !d_masks) return VL_ERR_INVALID_ARG;
     if (((uintptr_t)d_row & 1) || ((uintptr_t)d_masks & 3)) return VL_ERR_INVALID_ARG;
-    if (p->live_pending) {
-        const int rc = vl_live_settle(p);
-        if (rc != VL_OK) return rc;
-    }
     if (!p->live_ok) return VL_ERR_LIVENESS_NOT_RUN;
     VL_CUDA(p, cudaSetDevice(p->device));
+    {   // a liveness run may still be in flight: the kernels below are ordered behind it
+        const int rc = vl_live_join(p, (cudaStream_t)stream);
+        if (rc != VL_OK) return rc;
+    }
     if (!p->d_diag_T) VL_CUDA(p, cudaMalloc(&p->d_diag_T, sizeof(unsigned long long) * (p->V ? p->V : 1)));
     if (!p->d_diag_n) VL_CUDA(p, cudaMalloc(&p->d_diag_n, sizeof(unsigned long long)));
     cudaStream_t st = (cudaStream_t)stream;
@@ -174,7 +174,7 @@ extern "C" int vl_occupied_masks(vl_program *p, const uint16_t *d_row, uint32_t 
     if (p->nI) k_occupied<<<(p->nI + OCC_WARPS - 1) / OCC_WARPS, OCC_WARPS * 32, OCC_WARPS * W * sizeof(uint32_t), st>>>(q, W, d_masks);
     g_vl_launches.fetch_add(1 + (p->nO ? 1 : 0) + (p->nI ? 1 : 0));
     VL_CUDA(p, cudaGetLastError());
-    return VL_OK;
+    return vl_live_settle(p);  // (its outcome, after they have been enqueued)
 }
 
 extern "C" int vl_diagnose(vl_program *p, const uint16_t *d_row, uint64_t cap, vl_conflict *d_conflicts,
@@ -184,12 +184,12 @@ extern "C" int vl_diagnose(vl_program *p, const uint16_t *d_row, uint64_t cap, v
     if (((uintptr_t)d_row & 1) || ((uintptr_t)d_conflicts & 3) || ((uintptr_t)d_n_conflicts & 7) ||
         ((uintptr_t)d_bank_hist & 7))
         return VL_ERR_INVALID_ARG;
-    if (p->live_pending) {
-        const int rc = vl_live_settle(p);
-        if (rc != VL_OK) return rc;
-    }
     if (!p->live_ok) return VL_ERR_LIVENESS_NOT_RUN;
     VL_CUDA(p, cudaSetDevice(p->device));
+    {   // a liveness run may still be in flight: the kernels below are ordered behind it
+        const int rc = vl_live_join(p, (cudaStream_t)stream);
+        if (rc != VL_OK) return rc;
+    }
     if (!p->d_diag_T) VL_CUDA(p, cudaMalloc(&p->d_diag_T, sizeof(unsigned long long) * (p->V ? p->V : 1)));
     cudaStream_t st = (cudaStream_t)stream;
     DParams q{};
@@ -205,5 +205,39 @@ extern "C" int vl_diagnose(vl_program *p, const uint16_t *d_row, uint64_t cap, v
     if (p->nI) k_diag_instr<<<(p->nI + DIAG_WARPS - 1) / DIAG_WARPS, DIAG_WARPS * 32, 0, st>>>(q);
     g_vl_launches.fetch_add(1 + (p->nO ? 1 : 0) + (p->nI ? 1 : 0));
     VL_CUDA(p, cudaGetLastError());
+    return vl_live_settle(p);  // (its outcome, after they have been enqueued)
+}
+
+// 32 registers -> 32 bytes.  What bounds it is the store of the bytes (4 MB for 8,000 instructions and 512 registers).
+__attribute__((target("avx2"))) static void expand_avx2(const uint32_t *words, uint64_t n_rows, uint32_t W, uint32_t P, uint8_t *out)
+{
+    typedef char v32 __attribute__((vector_size(32), aligned(1), may_alias));
+    const v32 pick = {0, 0, 0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 1, 1, 2, 2, 2, 2, 2, 2, 2, 2, 3, 3, 3, 3, 3, 3, 3, 3};
+    const v32 bit = {1, 2, 4, 8, 16, 32, 64, (char)128, 1, 2, 4, 8, 16, 32, 64, (char)128,
+                     1, 2, 4, 8, 16, 32, 64, (char)128, 1, 2, 4, 8, 16, 32, 64, (char)128};
+    for (uint64_t i = 0; i < n_rows; ++i) {
+        const uint32_t *w = words + i * W;
+        uint8_t *o = out + i * P;
+        for (uint32_t j = 0; j < P / 32; ++j) {
+            typedef int v8i __attribute__((vector_size(32)));
+            const int x = (int)w[j];
+            const v8i all = {x, x, x, x, x, x, x, x};
+            const v32 bytes = (v32)__builtin_ia32_pshufb256((v32)all, pick);
+            *(v32 *)(o + j * 32) = ((bytes & bit) == bit) & 1;
+        }
+        for (uint32_t r = P / 32 * 32; r < P; ++r) o[r] = (uint8_t)((w[r >> 5] >> (r & 31)) & 1u);
+    }
+}
+
+extern "C" int vl_expand_masks(const uint32_t *words, uint64_t n_rows, uint32_t P, uint8_t *out)
+{
+    if (!P || (n_rows && (!words || !out))) return VL_ERR_INVALID_ARG;
+    const uint32_t W = (P + 31) / 32;
+    if (__builtin_cpu_supports("avx2")) {
+        expand_avx2(words, n_rows, W, P, out);
+        return VL_OK;
+    }
+    for (uint64_t i = 0; i < n_rows; ++i)
+        for (uint32_t r = 0; r < P; ++r) out[i * P + r] = (uint8_t)((words[i * W + (r >> 5)] >> (r & 31)) & 1u);
     return VL_OK;
 }

@@ -207,8 +207,8 @@ struct vl_program {
     uint64_t h_out_cap = 0;
     cudaStream_t h_streams[2] = {nullptr, nullptr};
     cudaEvent_t h_events[2] = {nullptr, nullptr};
-    // one record for vl_verify_until_pass: device copy and its pinned landing place
-    vl_sample_stats *d_rs = nullptr, *h_rs = nullptr;
+    // the record that vl_verify_until_pass polls for, in pinned memory
+    unsigned long long *h_rs = nullptr, rs_seq = 0;
     unsigned long long *d_diag_T = nullptr;  // [V] scratch of vl_diagnose: (first occurrence << 16) | value
     unsigned long long *d_diag_n = nullptr;  // one counter: scratch of vl_occupied_masks
 };

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_sample_stats(const RsParams q)
     const uint32_t c = blockIdx.y, tid = threadIdx.x;
     const uint64_t K = q.K[c];
     const uint64_t start = (uint64_t)blockIdx.x * RS_THREADS;
-    if (start >= K) return;
+    if (start >= K && blockIdx.x) return;
     const uint4 *out = q.out[c];
     const uint64_t step = (uint64_t)gridDim.x * RS_THREADS;
     unsigned long long first = K, cnt = 0;
@@ -58,7 +58,10 @@ __global__ void __launch_bounds__(RS_THREADS) k_sample_stats(const RsParams q)
             first = s_first[w] < first ? s_first[w] : first;
             cnt += s_cnt[w];
         }
-        if (cnt) {
+        if (gridDim.x == 1) {  // one block per test case: nothing to combine with
+            q.stats[c].first_pass = first;
+            q.stats[c].n_pass = cnt;
+        } else if (cnt) {
             atomicMin(reinterpret_cast<unsigned long long *>(&q.stats[c].first_pass), first);
             atomicAdd(reinterpret_cast<unsigned long long *>(&q.stats[c].n_pass), cnt);
         }
@@ -75,37 +78,67 @@ struct RsSumParams {
 // one block: the records of all test cases -> the summary
 __global__ void __launch_bounds__(256) k_resample_summary(const RsSumParams q)
 {
-    __shared__ unsigned long long s[3 + VL_MAX_PASS_AT];  // solved, attempts summed, largest, pass@k
+    constexpr int N = 3 + VL_MAX_PASS_AT;  // solved, attempts summed, largest, pass@k
+    __shared__ unsigned long long s[8][N];
     const uint32_t tid = threadIdx.x;
-    if (tid < 3 + VL_MAX_PASS_AT) s[tid] = 0;
-    __syncthreads();
-    unsigned long long solved = 0, sum = 0, mx = 0, at[VL_MAX_PASS_AT];
+    unsigned long long v[N];
 #pragma unroll
-    for (int j = 0; j < VL_MAX_PASS_AT; ++j) at[j] = 0;
+    for (int j = 0; j < N; ++j) v[j] = 0;
+    pdl_wait();
     for (uint32_t c = tid; c < q.n; c += blockDim.x) {
-        if (q.stats[c].n_pass == 0) continue;
-        const unsigned long long attempts = q.stats[c].first_pass + 1;
-        ++solved;
-        sum += attempts;
-        mx = attempts > mx ? attempts : mx;
+        const vl_sample_stats r = q.stats[c];
+        if (r.n_pass == 0) continue;
+        const unsigned long long attempts = r.first_pass + 1;
+        ++v[0];
+        v[1] += attempts;
+        v[2] = attempts > v[2] ? attempts : v[2];
 #pragma unroll
         for (int j = 0; j < VL_MAX_PASS_AT; ++j)
-            if ((uint32_t)j < q.n_k && attempts <= q.k[j]) ++at[j];
+            if ((uint32_t)j < q.n_k && attempts <= q.k[j]) ++v[3 + j];
     }
-    if (solved) {
-        atomicAdd(&s[0], solved);
-        atomicAdd(&s[1], sum);
-        atomicMax(&s[2], mx);
 #pragma unroll
-        for (int j = 0; j < VL_MAX_PASS_AT; ++j)
-            if (at[j]) atomicAdd(&s[3 + j], at[j]);
+    for (int j = 0; j < N; ++j) {
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, v[j], d);
+            v[j] = j == 2 ? (o > v[j] ? o : v[j]) : v[j] + o;
+        }
+        if ((tid & 31) == 0) s[tid >> 5][j] = v[j];
     }
     __syncthreads();
-    if (tid == 0) {
-        vl_resample_summary r;
-        r.n_cases = q.n; r.n_solved = s[0]; r.sum_tries = s[1]; r.max_tries = s[2];
-        for (int j = 0; j < VL_MAX_PASS_AT; ++j) r.pass_at[j] = s[3 + j];
-        *q.summary = r;
+    if (tid < N) {
+        unsigned long long x = 0;
+        for (int w = 0; w < 8; ++w) x = tid == 2 ? (s[w][tid] > x ? s[w][tid] : x) : x + s[w][tid];
+        unsigned long long *out = tid < 3 ? (tid == 0 ? (unsigned long long *)&q.summary->n_solved
+                                                      : (tid == 1 ? (unsigned long long *)&q.summary->sum_tries
+                                                                  : (unsigned long long *)&q.summary->max_tries))
+                                          : (unsigned long long *)&q.summary->pass_at[tid - 3];
+        *out = x;
+    }
+    if (tid == 0) q.summary->n_cases = q.n;
+}
+
+// One block, up to a few thousand verdicts of one test case: its record goes straight to pinned host memory, then the
+// sequence number that the host polls for (a kernel less, a copy less and no stream wait in the early-exit loop).
+__global__ void __launch_bounds__(RS_THREADS) k_batch_record(const uint4 *out, uint32_t K, unsigned long long *record,
+                                                             unsigned long long seq)
+{
+    __shared__ uint32_t s_first, s_cnt;
+    if (threadIdx.x == 0) { s_first = K; s_cnt = 0; }
+    __syncthreads();
+    pdl_wait();
+    uint32_t first = K, cnt = 0;
+    for (uint32_t k = threadIdx.x; k < K; k += RS_THREADS)
+        if (out[k].x & VL_PASS) { first = min(first, k); ++cnt; }
+    first = __reduce_min_sync(0xffffffffu, first);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if ((threadIdx.x & 31) == 0 && cnt) { atomicMin(&s_first, first); atomicAdd(&s_cnt, cnt); }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        record[0] = s_first;
+        record[1] = s_cnt;
+        __threadfence_system();
+        *(volatile unsigned long long *)(record + 2) = seq;
     }
 }
 
@@ -122,11 +155,13 @@ cudaError_t launch_stats(uint32_t m, const vl_verdict *const *d_out, const uint6
     }
     q.stats = d_stats;
     q.n = m;
-    k_sample_init<<<1, RS_CASES, 0, st>>>(q);
-    g_vl_launches.fetch_add(1);
+    uint64_t parts = (kmax + RS_ROWS_PER_BLOCK - 1) / RS_ROWS_PER_BLOCK;
+    if (parts > max_parts) parts = max_parts;
+    if (parts != 1) {  // (one block per test case writes its record itself)
+        k_sample_init<<<1, RS_CASES, 0, st>>>(q);
+        g_vl_launches.fetch_add(1);
+    }
     if (kmax) {
-        uint64_t parts = (kmax + RS_ROWS_PER_BLOCK - 1) / RS_ROWS_PER_BLOCK;
-        if (parts > max_parts) parts = max_parts;
         k_sample_stats<<<dim3((uint32_t)parts, m), RS_THREADS, 0, st>>>(q);
         g_vl_launches.fetch_add(1);
     }
@@ -157,9 +192,7 @@ extern "C" int vl_resample_stats(int device, uint32_t n, const vl_verdict *const
         RsSumParams s;
         s.stats = d_stats; s.summary = d_summary; s.n = n; s.n_k = n_k;
         for (uint32_t j = 0; j < VL_MAX_PASS_AT; ++j) s.k[j] = j < n_k ? k[j] : 0;
-        k_resample_summary<<<1, 256, 0, st>>>(s);
-        g_vl_launches.fetch_add(1);
-        if (cudaGetLastError() != cudaSuccess) return VL_ERR_CUDA;
+        if (launch_overlap(k_resample_summary, dim3(1), 256, 0, st, true, s) != cudaSuccess) return VL_ERR_CUDA;
     }
     return VL_OK;
 }
@@ -175,20 +208,29 @@ extern "C" int vl_verify_until_pass(vl_program *p, const uint16_t *d_cand, uint6
     if (K == 0) return VL_OK;
     if (!d_cand || !d_out || ((uintptr_t)d_out & 15)) return VL_ERR_INVALID_ARG;
     VL_CUDA(p, cudaSetDevice(p->device));
-    if (!p->d_rs) VL_CUDA(p, cudaMalloc(&p->d_rs, sizeof(vl_sample_stats)));
-    if (!p->h_rs && !(p->h_rs = (vl_sample_stats *)vl_pinned_get())) return VL_ERR_CUDA;
+    if (!p->h_rs && !(p->h_rs = (unsigned long long *)vl_pinned_get())) return VL_ERR_CUDA;
+    volatile unsigned long long *rec = p->h_rs;  // first passing row, passing rows, sequence number
     cudaStream_t st = (cudaStream_t)stream;
     for (uint64_t b0 = 0; b0 < K; b0 += batch_rows) {
         const uint64_t nb = K - b0 < batch_rows ? K - b0 : batch_rows;
         const int rc = vl_verify(p, d_cand + b0 * pitch, nb, pitch, d_out + b0, stream);
         if (rc != VL_OK) return rc;
-        const vl_verdict *outs = d_out + b0;
-        VL_CUDA(p, launch_stats(1, &outs, &nb, p->d_rs, st, 4u * (uint32_t)vl_sm_count(p)));
-        VL_CUDA(p, cudaMemcpyAsync(p->h_rs, p->d_rs, sizeof(vl_sample_stats), cudaMemcpyDeviceToHost, st));
-        VL_CUDA(p, cudaStreamSynchronize(st));
+        const unsigned long long seq = ++p->rs_seq;
+        VL_CUDA(p, launch_overlap(k_batch_record, dim3(1), RS_THREADS, 0, st, true, (const uint4 *)(d_out + b0), (uint32_t)nb,
+                                  p->h_rs, seq));
+        for (uint32_t polls = 0; rec[2] != seq;) {
+            if (++polls < 4096) continue;
+            polls = 0;
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e == cudaErrorNotReady) continue;
+            VL_CUDA(p, e);
+            VL_CUDA(p, cudaStreamSynchronize(st));  // (finished: the record is there)
+            if (rec[2] != seq) return VL_ERR_CUDA;
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
         *rows_checked = b0 + nb;
-        if (p->h_rs->n_pass) {
-            *first_pass = b0 + p->h_rs->first_pass;
+        if (rec[1]) {
+            *first_pass = b0 + rec[0];
             break;
         }
     }

@@ -1707,7 +1707,11 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
     Plan pl{};
     const uint32_t groups[3] = {4, 2, 1};
     if (p->group_opt == 0 || p->group_opt == 8) {
-        pl = make_plan8(p, p->threads_opt ? p->threads_opt : 256, SM_BYTES / 2 - 1024);
+        // (hardware rules, and no more blocks than multiprocessors: the sweep over the rules takes 512 threads; 98 blocks
+        // 51 -> 44 us.  Without rules 256 are the better choice even then, 83 us against 88 for a call of 125 blocks: a
+        // block leaves room for the first ones of the walk)
+        const bool alone = p->d_vcons && (K + 7) / 8 <= (uint64_t)vl_sm_count(p);
+        if (!alone || p->threads_opt) pl = make_plan8(p, p->threads_opt ? p->threads_opt : 256, SM_BYTES / 2 - 1024);
         if (!pl.ok) pl = make_plan8(p, p->threads_opt ? p->threads_opt : 512, SM_BYTES);
         if (!pl.ok && !p->threads_opt) pl = make_plan8(p, 256, SM_BYTES);
     }
