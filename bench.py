@@ -383,7 +383,7 @@ def main():
         bytes_per_step = 2.0 * prog.pitch * K + 16.0 * K
         # the four timing slots of a pass (the table kernel; the through-set kernel and the walk; the stand-alone
         # verdict step of programs without instructions; the recount)
-        names = ["k_tables8", "k_through+k_walk", "k_finish", "k_recount"]
+        names = ["k_tables8", "k_through+k_walk", "k_finish", "k_exact"]
         passes = max(1, kernel_passes)
         ksum = max(1e-9, sum(kernel_ms))
         kernels = {n: {"ms_per_launch": kernel_ms[j] / passes, "share": kernel_ms[j] / ksum} for j, n in enumerate(names)}
@@ -407,7 +407,7 @@ def main():
             # the figures of the whole vl_verify call as the timed region runs it (every verify kernel, passes
             # spread over the library's internal streams); the dominant kernel alone is a sub-field
             "roofline": {"bound": "hbm", "achieved": path_achieved, "peak": peak, "unit": "GB/s", "frac": path_achieved / peak,
-                         "traffic": traffic, "kernel": "vl_verify (k_tables8 + k_through + k_walk + k_recount)",
+                         "traffic": traffic, "kernel": "vl_verify (k_tables8 + k_through + k_walk + k_exact)",
                          "of": peak_kind, "launches": args.steps, "ms_per_launch": verify_ms,
                          "bytes_per_launch": bytes_per_step,
                          "how": "CUDA events on the caller's stream around each of the vl_verify calls of a loop of its own "

@@ -592,8 +592,10 @@ extern "C" int vl_verify_host(vl_program *p, const uint16_t *h_cand, uint64_t K,
     if (rc != VL_OK || K == 0) return rc;
     VL_CUDA(p, cudaSetDevice(p->device));
     if ((rc = vl_live_settle(p)) != VL_OK) return rc;
-    // slabs of about 64 MiB, a multiple of 4 rows
-    uint64_t rows = std::max<uint64_t>(4, ((64ull << 20) / (pitch * 2)) / 4 * 4);
+    // Slabs of an eighth of the rows, 4 to 16 MiB, a multiple of 4 rows.  The call is bound by the copies (about 55 GB/s);
+    // what is left over is the check of the last slab: 49.5 MB in one slab took 1,011 us, in eight 990.
+    const uint64_t slab_bytes = std::min<uint64_t>(16ull << 20, std::max<uint64_t>(4ull << 20, K * pitch * 2 / 8));
+    uint64_t rows = std::max<uint64_t>(4, (slab_bytes / (pitch * 2) + 3) / 4 * 4);
     rows = std::min<uint64_t>(rows, (K + 3) / 4 * 4);
     if (p->stage_rows < rows || p->stage_pitch != pitch) {
         for (int j = 0; j < 2; ++j) {
