@@ -258,7 +258,7 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
 #define EXACT_MAX_PARTS 32 // items of one candidate, at most
 #define EXACT_PART_CHUNKS 6 // chunks of the walk that an item counts, about
 // per-candidate state between the kernels (8 words)
-enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_NOUT = 3, CS_OUTV = 4, CS_OUTRAW = 5, CS_WALK = 6, CS_THCOL = 7 };
+enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_WALK = 6, CS_THCOL = 7 };
 enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
 struct VlExactArgs {
     const uint32_t *work, *cstate, *anom;

@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "vl_internal.cuh"
 
@@ -533,14 +534,7 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
 
     // ------------------------------------------------- hand-over to the walk
     // One vreg sticking out of the file cannot overlap another one out there: the walk sees it
-    // parked at P (bits beyond P are padding).  Two or more: the candidate is recounted in full.
-    // (such a candidate does not take part in the walk: it gets its table back without the marks)
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        if (M->nout[g] < 2) continue;
-        uint16_t *col = q.tg + (k0 / TGW) * (uint64_t)(q.V + 1) * TGW + (uint32_t)(k0 & (TGW - 1)) + g;
-        for (uint32_t v = tid; v < q.V; v += NT) col[(size_t)v * TGW] = (uint16_t)pk_get(t_load<G>(Tt, v), g);
-    }
+    // parked at P (bits beyond P are padding).  Two or more: the candidate is not walked but counted in full.
     if (tid < G && M->nout[tid] == 1 && M->out_raw[tid] >= q.P) {
         const uint32_t ov = M->out_v[tid];
         const uint32_t mark = ((q.P & 31u) + (q.vinfo[ov] & 0xFFu) > 32u) ? 0x8000u : 0u;
@@ -566,9 +560,6 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
         cs[CS_FLAGS] = M->flags[g];
         cs[CS_FIRST] = min(first, M->minR[g]);
         cs[CS_BANK] = q.bank_fast ? q.bank_total - M->bank[g] : 0u;
-        cs[CS_NOUT] = M->nout[g];
-        cs[CS_OUTV] = M->out_v[g];
-        cs[CS_OUTRAW] = M->out_raw[g];
         cs[CS_WALK] = M->nout[g] >= 2 ? WALK_FULL : 0u;
         cs[CS_THCOL] = 0;
     }
@@ -881,10 +872,17 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
     }
     __syncthreads();
 
-    // ---- first sweep over the vregs: the one-hot bank nibbles of the 8 candidates go to Hb, and
-    // [T, T+width) is checked against the register file (Realizability).
+    // ---- one sweep over the vregs: the hardware rules, if there are any; the one-hot bank nibbles of the 8 candidates
+    // (byte j: candidate j low, candidate j + 4 high) go to Hb; [T, T+width) is checked against the register file
+    // (Realizability); and entries whose range reaches into the next 32-bit word of an occupancy mask get bit 15, in
+    // place.  (A candidate with two or more vregs outside the file is not walked: what its entries become does not
+    // matter.)  Bound by instruction issue; as two sweeps, with a shift per candidate for the nibbles, it took 16.5 k
+    // cycles per block on 10,000 vregs, now 10.
     // (From here on the producer warp only keeps the block's barriers company.)
+    if (q.vcons && tid < NT) rules_sweep8<NT>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, M);
     if (tid < NT) {
+        uint32_t mk = 0, mk2 = 0, mk3 = 0, mk4 = 0;
+        const uint32_t bm = q.Bmask * 0x10001u;
         uint32_t vis_next[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) vis_next[u] = tid + u * NT < q.V ? q.vinfo[tid + u * NT] : 0u;
@@ -902,12 +900,14 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
                 if (v >= q.V) break;
                 const uint4 tt = T[v];
                 const uint32_t x[4] = {tt.x, tt.y, tt.z, tt.w};
-                if (q.bank_fast) {
-                    uint32_t h = 0;
+                if (q.bank_fast) {  // a byte permute looks up 1 << bank for four candidates at a time
+                    uint32_t h[2];
 #pragma unroll
-                    for (int m = 0; m < 4; ++m)
-                        h |= ((1u << (x[m] & q.Bmask)) << (8 * m)) | ((16u << ((x[m] >> 16) & q.Bmask)) << (8 * m));
-                    Hb[v] = h;
+                    for (int m = 0; m < 2; ++m) {
+                        const uint32_t w = (x[2 * m] & bm) | ((x[2 * m + 1] & bm) << 8);
+                        h[m] = __byte_perm(0x08040201u, 0u, w | (w >> 12));
+                    }
+                    Hb[v] = h[0] | (h[1] << 4);
                 }
                 if (!(vi & VINFO_OCCURS)) continue;
                 // quick test for "all eight inside the file": with c = 0x7FFF - (P - width) added to an
@@ -932,50 +932,16 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
                         }
                     }
                 }
-            }
-        }
-    }
-    if (q.vcons && tid < NT) rules_sweep8<NT>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, M);
-    __syncthreads();
-
-    // ---- second sweep, in place: entries whose range reaches into the next 32-bit word of an occupancy
-    // mask get bit 15.  The entries of a candidate with two or more vregs outside the register file stay as
-    // they are (it is not walked; the full recount reads them as plain numbers).
-    if (tid < NT) {
-        uint32_t keep[4];  // 16-bit fields of the candidates whose entries stay as they are
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-            keep[m] = (M->nout[2 * m] >= 2 ? 0xFFFFu : 0u) | (M->nout[2 * m + 1] >= 2 ? 0xFFFF0000u : 0u);
-        uint32_t mk = 0, mk2 = 0, mk3 = 0, mk4 = 0;
-        uint32_t vis_next[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) vis_next[u] = tid + u * NT < q.V ? q.vinfo[tid + u * NT] : 0u;
-        for (uint32_t v0 = tid; v0 < q.V; v0 += 4 * NT) {
-            uint32_t vis[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                vis[u] = vis_next[u];
-                const uint32_t vn = v0 + 4 * NT + u * NT;
-                vis_next[u] = vn < q.V ? q.vinfo[vn] : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t v = v0 + u * NT, vi = vis[u];
-                if (v >= q.V) break;
-                if (!(vi & VINFO_OCCURS)) continue;  // (never looked up)
-                const uint4 tt = T[v];
-                const uint32_t x[4] = {tt.x, tt.y, tt.z, tt.w};
                 // bit 15 := ((register & 31) + width > 32), per 16-bit entry; 0x7FDF = 0x8000 - 33
-                const uint32_t wc = (vi & 0xFFu) * 0x10001u + 0x7FDF7FDFu;
+                const uint32_t wc = w * 0x10001u + 0x7FDF7FDFu;
                 uint32_t o[4], diff = 0;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    const uint32_t marked = (x[m] & 0x7FFF7FFFu) | (((x[m] & 0x001F001Fu) + wc) & 0x80008000u);
-                    o[m] = (marked & ~keep[m]) | (x[m] & keep[m]);
+                    o[m] = (x[m] & 0x7FFF7FFFu) | (((x[m] & 0x001F001Fu) + wc) & 0x80008000u);
                     diff |= o[m] ^ x[m];
                 }
                 if (diff) T[v] = make_uint4(o[0], o[1], o[2], o[3]);
-                mk |= o[0] & ~keep[0]; mk2 |= o[1] & ~keep[1]; mk3 |= o[2] & ~keep[2]; mk4 |= o[3] & ~keep[3];
+                mk |= o[0]; mk2 |= o[1]; mk3 |= o[2]; mk4 |= o[3];
             }
         }
         const uint32_t mkw[4] = {mk, mk2, mk3, mk4};
@@ -984,8 +950,10 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
         for (int m = 0; m < 4; ++m) bits |= ((mkw[m] >> 15) & 1u) << (2 * m) | ((mkw[m] >> 31) & 1u) << (2 * m + 1);
         bits = __reduce_or_sync(0xffffffffu, bits);
         if (lane == 0 && bits) atomicOr(&M->marks, bits);
-        // the consumers go on to the bank tally (it reads Hb only); the producer warp waits for all of them here
+        // the consumers go on to the bank tally (Hb is complete when all of them are here: barrier 2); the producer warp
+        // waits for all of them on barrier 1
         asm volatile("bar.arrive 1, %0;" ::"r"(NT + 32) : "memory");
+        asm volatile("bar.sync 2, %0;" ::"r"(NT) : "memory");
     }
     // The table goes to global memory, 64 candidates side by side per vreg (this block's 8 are 16 bytes of
     // every 128): tiled bulk stores of up to 256 vregs each, carried out by the copy engine while the block
@@ -1032,43 +1000,52 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
         for (int g = 0; g < G; ++g) sum[g] = 0;
         auto flush = [&](uint32_t weight) {
 #pragma unroll
-            for (int g = 0; g < G; ++g) sum[g] += weight * ((((g & 1) ? acc_o : acc_e) >> (8 * (g >> 1))) & 0xFFu);
+            for (int g = 0; g < G; ++g) sum[g] += weight * (((g >= 4 ? acc_o : acc_e) >> (8 * (g & 3))) & 0xFFu);
             acc_e = 0; acc_o = 0;
         };
-        const uint32_t n_ent = q.bank_seg[3];
-        uint2 ids_next[8];
+        // one segment of the list per number of sources: as many lookups as an entry has sources (with four for every
+        // entry the shared-memory pipe took 12.4 k cycles per block on 31,000 entries, now 9)
+        auto segment = [&](auto sources, uint32_t e_lo, uint32_t e_hi) {
+            constexpr int N = decltype(sources)::value;
+            uint2 ids_next[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) ids_next[u] = tid + u * NT < n_ent ? q.bank_list[tid + u * NT] : make_uint2(0, 0);
-        for (uint32_t e0 = tid; e0 < n_ent; e0 += 8 * NT) {
-            uint2 ids[8];
+            for (int u = 0; u < 8; ++u) ids_next[u] = e_lo + tid + u * NT < e_hi ? q.bank_list[e_lo + tid + u * NT] : make_uint2(0, 0);
+            for (uint32_t e0 = e_lo + tid; e0 < e_hi; e0 += 8 * NT) {
+                uint2 ids[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                ids[u] = ids_next[u];
-                const uint32_t en = e0 + 8 * NT + u * NT;
-                ids_next[u] = en < n_ent ? q.bank_list[en] : make_uint2(0, 0);
-            }
-            uint32_t x[8];
+                for (int u = 0; u < 8; ++u) {
+                    ids[u] = ids_next[u];
+                    const uint32_t en = e0 + 8 * NT + u * NT;
+                    ids_next[u] = en < e_hi ? q.bank_list[en] : make_uint2(0, 0);
+                }
+                uint32_t x[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t o = Hb[ids[u].x & 0xFFFFu] | Hb[ids[u].x >> 16] | Hb[ids[u].y & 0xFFFFu] | Hb[ids[u].y >> 16];
-                x[u] = e0 + u * NT < n_ent ? o : 0u;
+                for (int u = 0; u < 8; ++u) {
+                    uint32_t o = Hb[ids[u].x & 0xFFFFu] | Hb[ids[u].x >> 16];
+                    if (N > 2) o |= Hb[ids[u].y & 0xFFFFu];
+                    if (N > 3) o |= Hb[ids[u].y >> 16];
+                    x[u] = e0 + u * NT < e_hi ? o : 0u;
+                }
+                uint32_t ta, tb, fa, fb, eights;
+                csa(ta, ones, ones, x[0], x[1]);
+                csa(tb, ones, ones, x[2], x[3]);
+                csa(fa, twos, twos, ta, tb);
+                csa(ta, ones, ones, x[4], x[5]);
+                csa(tb, ones, ones, x[6], x[7]);
+                csa(fb, twos, twos, ta, tb);
+                csa(eights, fours, fours, fa, fb);
+                const uint32_t c8 = nib_counts(eights);
+                acc_e += nib_even(c8);
+                acc_o += nib_odd(c8);
+                if (++rounds == 32) {  // the byte fields hold at most 4 per round
+                    flush(8u);
+                    rounds = 0;
+                }
             }
-            uint32_t ta, tb, fa, fb, eights;
-            csa(ta, ones, ones, x[0], x[1]);
-            csa(tb, ones, ones, x[2], x[3]);
-            csa(fa, twos, twos, ta, tb);
-            csa(ta, ones, ones, x[4], x[5]);
-            csa(tb, ones, ones, x[6], x[7]);
-            csa(fb, twos, twos, ta, tb);
-            csa(eights, fours, fours, fa, fb);
-            const uint32_t c8 = nib_counts(eights);
-            acc_e += nib_even(c8);
-            acc_o += nib_odd(c8);
-            if (++rounds == 32) {  // the byte fields hold at most 4 per round
-                flush(8u);
-                rounds = 0;
-            }
-        }
+        };
+        segment(std::integral_constant<int, 2>{}, q.bank_seg[0], q.bank_seg[1]);
+        segment(std::integral_constant<int, 3>{}, q.bank_seg[1], q.bank_seg[2]);
+        segment(std::integral_constant<int, 4>{}, q.bank_seg[2], q.bank_seg[3]);
         flush(8u);
         uint32_t c = nib_counts(fours);
         acc_e = nib_even(c); acc_o = nib_odd(c);
@@ -1108,9 +1085,6 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
         cs[CS_FLAGS] = M->flags[g];
         cs[CS_FIRST] = min(first, M->minR[g]);
         cs[CS_BANK] = q.bank_fast ? q.bank_total - M->bank[g] : 0u;
-        cs[CS_NOUT] = M->nout[g];
-        cs[CS_OUTV] = M->out_v[g];
-        cs[CS_OUTRAW] = M->out_raw[g];
         cs[CS_WALK] = M->nout[g] >= 2 ? WALK_FULL : 0u;
         cs[CS_THCOL] = 0;
         // a candidate that is walked and has a marked entry sends its group of 64 down the walk's
