@@ -800,10 +800,12 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
     uint2 *list = reinterpret_cast<uint2 *>(base + q.sm.list);
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     pdl_wait();
-    const uint32_t n_items = q.ex.work[0];
+    const bool fine = q.ex.work[1] <= q.ex.fine_items;
+    const uint32_t n_items = q.ex.work[fine ? 1 : 0];
+    const uint32_t *items = q.ex.work + EXACT_HDR + (fine ? 0 : 2 * EXACT_FINE_ITEMS);
     for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const uint64_t k = q.ex.work[EXACT_HDR + 2 * it];
-        const uint32_t part = q.ex.work[EXACT_HDR + 2 * it + 1] & 0xFFu, parts = q.ex.work[EXACT_HDR + 2 * it + 1] >> 8;
+        const uint64_t k = items[2 * it];
+        const uint32_t part = items[2 * it + 1] & 0xFFu, parts = items[2 * it + 1] >> 8;
         const uint16_t *row = q.cand + k * q.pitch;
         const uint32_t *cs = q.ex.cstate + k * 8;
         const uint32_t walk = cs[CS_WALK], thcol = cs[CS_THCOL];

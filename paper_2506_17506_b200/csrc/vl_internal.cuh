@@ -254,9 +254,15 @@ bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
                  vl_verdict *const *d_out, cudaStream_t st, bool dict);
 // The exact counts of the batched kernels' listed candidates (k_exact, vl_fused.cu).
-#define EXACT_HDR 4        // words in front of the listed items: their number
-#define EXACT_MAX_PARTS 32 // items of one candidate, at most
-#define EXACT_PART_CHUNKS 6 // chunks of the walk that an item counts, about
+// A candidate is listed twice, in items of about EXACT_FINE_CHUNKS and of about EXACT_PART_CHUNKS chunks of the walk.  The
+// fine ones are taken if each has a thread block of its own: 1,000 rows of 8,000 instructions of which 100 fail 77 us
+// against 81 for the whole call, 777 of 11,317 with 39 failing 103.5 against 109.  Beyond that what an item costs before
+// its first count weighs more: 350 of the 1,000 failing 95 us in fine items, 85.5 in coarse ones.
+#define EXACT_HDR 4         // words in front of the fine items, then the coarse ones: numbers of coarse and of fine items
+#define EXACT_MAX_PARTS 32  // items of one candidate, at most
+#define EXACT_PART_CHUNKS 6
+#define EXACT_FINE_CHUNKS 2
+#define EXACT_FINE_ITEMS 512
 // per-candidate state between the kernels (8 words)
 enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_WALK = 6, CS_THCOL = 7 };
 enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
@@ -264,9 +270,10 @@ struct VlExactArgs {
     const uint32_t *work, *cstate, *anom;
     const uint32_t *short_chunk, *chunk_short_off;  // [nS] chunk of every short chunk, [nC + 1] first short chunk of every chunk
     uint32_t *racc;               // [rows][4] overlaps, complement of the lowest instruction, bank tally, parts done; all 0
-    uint32_t AW;
+    uint32_t AW, fine_items;      // fine_items: up to that many fine items are taken
     unsigned char *scratch;       // vl_exact_scratch bytes, null if 0
 };
+uint32_t vl_exact_blocks(vl_program *p);  // thread blocks of k_exact: one item each at a time
 uint64_t vl_exact_scratch(vl_program *p);
 int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st,
                  bool dict, bool overlap);

@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
     for (uint32_t j = tid; j < G * q.AW; j += NT) q.anom[k0 * q.AW + j] = 0;
     if (tid < G * 4) q.racc[k0 * 4 + tid] = 0;
     if (tid == 0 && (k0 & (TGW - 1)) == 0) q.grp_done[k0 / TGW] = 0;
-    if (tid == 0 && blockIdx.x == 0) q.work[0] = 0;  // items listed for the exact count
+    if (tid == 0 && blockIdx.x == 0) q.work[0] = q.work[1] = 0;  // items listed for the exact count
     __syncthreads();
 
     // The ring stage and the barrier phase of the current tile are kept as running counters (stage
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
     for (uint32_t j = tid; j < G * q.AW; j += NT) q.anom[k0 * q.AW + j] = 0;
     if (tid < G * 4) q.racc[k0 * 4 + tid] = 0;
     if (tid == 0 && (k0 & (TGW - 1)) == 0) q.grp_done[k0 / TGW] = 0;
-    if (tid == 0 && blockIdx.x == 0) q.work[0] = 0;  // items listed for the exact count
+    if (tid == 0 && blockIdx.x == 0) q.work[0] = q.work[1] = 0;  // items listed for the exact count
     __syncthreads();
 
     // A tile is one box of the row tensor: 8 candidates x CH chunks x 256 operands, one copy.  (Boxes
@@ -1132,10 +1132,15 @@ __device__ __forceinline__ void finish_candidate(uint64_t k, uint32_t nC, uint32
         else if (walk)
             for (uint32_t w = 0; w < AW; ++w) chunks += __popc(__ldcg(anom + k * AW + w));
         const uint32_t parts = min(1u + chunks / EXACT_PART_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
-        const uint32_t at = atomicAdd(work, parts);
+        const uint32_t fine = min(1u + chunks / EXACT_FINE_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
+        const uint32_t at = EXACT_FINE_ITEMS + atomicAdd(work, parts), fine_at = atomicAdd(work + 1, fine);
         for (uint32_t j = 0; j < parts; ++j) {
             work[EXACT_HDR + 2 * (at + j)] = (uint32_t)k;
             work[EXACT_HDR + 2 * (at + j) + 1] = j | (parts << 8);
+        }
+        for (uint32_t j = 0; j < fine && fine_at + j < EXACT_FINE_ITEMS; ++j) {
+            work[EXACT_HDR + 2 * (fine_at + j)] = (uint32_t)k;
+            work[EXACT_HDR + 2 * (fine_at + j) + 1] = j | (fine << 8);
         }
         return;
     }
@@ -1624,7 +1629,7 @@ int ensure_scratch(vl_program *p, int slot, uint64_t rows)
         {(void **)&v.grp_done, 2 * (groups + 1) * sizeof(uint32_t)},
         {(void **)&v.tg, groups * (p->V + 1) * TGW * sizeof(uint16_t)},
         {(void **)&v.anom, groups * TGW * aw * sizeof(uint32_t)},
-        {(void **)&v.work, (EXACT_HDR + 2 * EXACT_MAX_PARTS * groups * TGW) * sizeof(uint32_t)},
+        {(void **)&v.work, (EXACT_HDR + 2 * (EXACT_FINE_ITEMS + EXACT_MAX_PARTS * groups * TGW)) * sizeof(uint32_t)},
         {(void **)&v.racc, groups * TGW * 4 * sizeof(uint32_t)},
         // through-set masks of every (group, program block), in the walk's layout
         {(void **)&v.thm, groups * p->nB * ((p->P + p->wmax + 31) / 32) * 64 * sizeof(uint32_t)},
@@ -1848,7 +1853,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     kt_mark(p, st);
     VlExactArgs ex{};
     ex.work = vs.work; ex.cstate = vs.cstate; ex.anom = vs.anom; ex.short_chunk = p->d_short_chunk; ex.chunk_short_off = p->d_chunk_short_off; ex.racc = vs.racc;
-    ex.AW = (uint32_t)vs.aw; ex.scratch = vs.exact;
+    ex.fine_items = std::min<uint32_t>(vl_exact_blocks(p), EXACT_FINE_ITEMS); ex.AW = (uint32_t)vs.aw; ex.scratch = vs.exact;
     if ((rc = vl_exact_run(p, ex, d_cand, pitch, d_out, st, dict, early && p->nC)) != VL_OK) return rc;
     kt_mark(p, st);
     return VL_OK;

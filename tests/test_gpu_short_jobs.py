@@ -67,3 +67,21 @@ def test_exact_counts_in_global_memory(B, oracle_mod):
     rows = np.stack([H.row_from_table(p, t) for t in tables])
     _assert_same(_gpu_verify(B, gp, rows), op.verify(lv, rows), "global")
     gp.close()
+
+
+@pytest.mark.parametrize("failing", [1, 12, 60])
+def test_exact_count_items(B, oracle_mod, failing):
+    """Failing rows of the batched kernels few enough that each fine share of their counts gets a thread block, about
+    that many, and more."""
+    wl = synth.workload(2)
+    p = synth.build_program(wl.shapes[0], wl.seeds[0])
+    rows, _ = synth.candidate_rows(p, 70, 0.0, 78)
+    bad = (np.arange(failing) * 7) % 70
+    rows[bad] = _garbage_rows(p, failing, 5)
+    rows[bad[::2]] = synth.candidate_rows(p, failing, 1.0, 79)[0][: len(bad[::2])]
+    gp = B.Program(p)
+    gp.set_option(B.VL_OPT_GROUP, 8)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows), f"{failing} failing")
+    gp.close()
