@@ -382,7 +382,7 @@ def main():
         # verdict is written; the table kernel is the one that streams the rows
         bytes_per_step = 2.0 * prog.pitch * K + 16.0 * K
         # the four timing slots of a pass (the table kernel; the through-set kernel and the walk; the stand-alone
-        # verdict step of programs without instructions; the recount)
+        # verdict step of programs without instructions; the exact counts)
         names = ["k_tables8", "k_through+k_walk", "k_finish", "k_exact"]
         passes = max(1, kernel_passes)
         ksum = max(1e-9, sum(kernel_ms))

@@ -299,6 +299,7 @@ extern "C" void vl_program_destroy(vl_program *p)
     cudaFree(p->d_blob);
     cudaFree(p->d_vcons); cudaFree(p->d_rs_prefix);
     for (auto &v : p->vs) cudaFree(v.block);
+    for (auto &v : p->fs) cudaFree(v.block);
     for (int j = 0; j < 2; ++j) {
         cudaFree(p->d_stage[j]);
         cudaFree(p->d_stage_out[j]);

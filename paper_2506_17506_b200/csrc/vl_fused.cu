@@ -491,7 +491,8 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
 // BPM: thread blocks per multiprocessor that the registers have to leave room for.  One or two rows per multiprocessor are
 // bound by latency (registers for loads in flight), more rows by how many warps there are to switch between: 6,400 rows of
 // 64 programs 345 us with two blocks of 256 threads, 281 with three, 274 with four (but spills: one row 20 % slower).
-template <int NTHR, int BPM, int N>
+// HAND: candidates with a collision are listed for k_exact, which spreads their counts over all multiprocessors.
+template <int NTHR, int BPM, int N, bool HAND>
 __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMany<N> a)
 {
     const FParams &q = a.p[N == 1 ? 0 : blockIdx.y];
@@ -746,7 +747,8 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
     __syncthreads();
 
     // ---- 5. exact counts where something collided
-    if (M->any | M->thcol) exact_counts<NTHR, false>(q, T, W, occ, coll, list, M, 0, 1, row);
+    const bool collided = M->any | M->thcol;
+    if (!HAND && collided) exact_counts<NTHR, false>(q, T, W, occ, coll, list, M, 0, 1, row);
 
     // ---- the verdict
     if (warp == 0) {
@@ -771,7 +773,25 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
             }
             first = min(first, i);
         }
-        if (lane == 0) {
+        if (HAND && collided) {
+            uint32_t chunks = M->thcol ? q.ex.nC / 8 : 0u;  // (the sources in the through-set)
+            for (uint32_t w = 0; w < q.ex.AW; ++w) {
+                const uint32_t c = w * 32 + lane;
+                bool hit = false;
+                if (c < q.ex.nC)
+                    for (uint32_t s = q.ex.chunk_short_off[c]; s < q.ex.chunk_short_off[c + 1]; ++s) hit |= (coll[s >> 5] >> (s & 31)) & 1u;
+                const uint32_t bits = __ballot_sync(0xffffffffu, hit);
+                if (lane == 0) q.ex.anom[k * q.ex.AW + w] = bits;
+                chunks += __popc(bits);
+            }
+            if (lane < 4) q.ex.racc[k * 4 + lane] = 0;
+            if (lane == 0) {
+                uint32_t *cs = q.ex.cstate + k * 8;
+                cs[CS_FLAGS] = M->flags; cs[CS_FIRST] = first; cs[CS_BANK] = M->bank;
+                cs[CS_WALK] = M->any ? WALK_ANOM : 0u; cs[CS_THCOL] = M->thcol;
+                list_exact(q.ex.work, k, chunks);
+            }
+        } else if (lane == 0) {
             const uint32_t flags = M->flags | (M->pairs ? (uint32_t)VL_INTERFERENCE : 0u);
             vl_verdict vd;
             vd.flags = flags ? flags : (uint32_t)VL_PASS;
@@ -828,8 +848,8 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
         __syncthreads();
         if (count) exact_counts<EXACT_NT, true>(q, T, W, occ, coll, list, M, part, parts, row);
         __syncthreads();
-        if (q.bank_fast) {
-            if (tid == 0) M->bank = (part == 0 ? cs[CS_BANK] : 0u) - M->dups;
+        if (q.bank_fast || q.ex.after_fused) {
+            if (tid == 0) M->bank = (part == 0 ? cs[CS_BANK] : 0u) - (q.ex.after_fused ? 0u : M->dups);
         } else {  // the general tally: the whole table, this part's instructions
             for (uint32_t v = tid; v < q.V; v += EXACT_NT) {
                 const uint32_t pos = q.first_occ[v];
@@ -870,6 +890,9 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
             }
         }
     }
+    // the next call lists from the start: the block that is last to be done sees to it (every block has read the counts)
+    __syncthreads();
+    if (q.ex.after_fused && tid == 0 && atomicAdd(q.ex.work + 2, 1u) == gridDim.x - 1) q.ex.work[0] = q.ex.work[1] = q.ex.work[2] = 0;
 }
 
 // How a job of K rows runs: threads per block (0: the program does not fit the kernel), blocks per multiprocessor.  Up to
@@ -928,9 +951,42 @@ bool vl_fused_wanted(vl_program *p, uint64_t K)
     return rounds <= 1 || rounds * (6000 + 7ull * p->nI) <= 72000;
 }
 
+// Programs of at least that many instructions whose rows share multiprocessors hand the exact counts to k_exact: a row that
+// fails used to keep its few warps busy for longer than all the rest took, now every multiprocessor shares in it.  300 rows
+// of 8,000 instructions 45 us against 88 with 10 % of the rows failing, of 11,317 instructions 62 against 90; with none
+// failing the second launch costs 1 us (32.9, 46.0).  Of 5,000 instructions it gains nothing (46.4 against 43.1, 48.2 against
+// 48.5 with 30 % failing), nor do rows that have a multiprocessor to themselves (50 rows of 11,317 instructions 22 us).
+#define FUSED_HAND_INSTRS 7000u
+
+// What k_fused and k_exact share.
+static int hand_scratch(vl_program *p, int slot, uint64_t rows, VlExactArgs *ex)
+{
+    vl_program::VScratch &v = p->fs[slot];
+    const uint64_t aw = (p->nC + 31) / 32;
+    if (v.rows < rows || v.aw != aw) {
+        VL_CUDA(p, cudaFree(v.block));
+        v = vl_program::VScratch{};
+        rows = std::max<uint64_t>(rows, 3ull * vl_sm_count(p));
+        const uint64_t words[4] = {EXACT_HDR + 2 * (EXACT_FINE_ITEMS + EXACT_MAX_PARTS * rows), rows * 8, rows * 4, rows * aw};
+        VL_CUDA(p, cudaMalloc(&v.block, (words[0] + words[1] + words[2] + words[3]) * 4));
+        uint32_t *w = static_cast<uint32_t *>(v.block);
+        VL_CUDA(p, cudaMemset(w, 0, EXACT_HDR * 4));
+        VL_CUDA(p, cudaStreamSynchronize(cudaStreamLegacy));  // (the kernels run on streams that do not wait for it)
+        v.work = w; v.cstate = w + words[0]; v.racc = v.cstate + words[1]; v.anom = v.racc + words[2];
+        v.rows = rows; v.aw = aw;
+    }
+    ex->work = v.work; ex->cstate = v.cstate; ex->racc = v.racc; ex->anom = v.anom;
+    ex->AW = (uint32_t)aw; ex->nC = p->nC;
+    ex->short_chunk = p->d_short_chunk; ex->chunk_short_off = p->d_chunk_short_off;
+    ex->fine_items = std::min<uint32_t>(vl_exact_blocks(p), EXACT_FINE_ITEMS);
+    ex->after_fused = 1;
+    ex->scratch = nullptr;
+    return VL_OK;
+}
+
 // Up to VL_FUSED_MANY jobs in one launch on st.
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
-                 vl_verdict *const *d_out, cudaStream_t st, bool dict)
+                 vl_verdict *const *d_out, cudaStream_t st, bool dict, int slot)
 {
     vl_program *p0 = progs[0];
     static std::mutex mtx;
@@ -939,10 +995,12 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         std::lock_guard<std::mutex> lock(mtx);
         if (!done[p0->device]) {
             const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<512, 1, 1>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 2, 1>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 3, 1>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 3, VL_FUSED_MANY>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<512, 1, 1, false>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 2, 1, false>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 3, 1, false>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 3, VL_FUSED_MANY, false>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 2, 1, true>, at, 227 * 1024));
+            VL_CUDA(p0, cudaFuncSetAttribute(k_fused<256, 3, 1, true>, at, 227 * 1024));
             done[p0->device] = true;
         }
     }
@@ -963,14 +1021,22 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         if (rc != VL_OK) return rc;
     }
     if (n > 1) {
-        VL_CUDA(p0, launch_overlap(k_fused<256, 3, VL_FUSED_MANY>, dim3((uint32_t)rows, n), 256, smem, st, true, many));
+        VL_CUDA(p0, launch_overlap(k_fused<256, 3, VL_FUSED_MANY, false>, dim3((uint32_t)rows, n), 256, smem, st, true, many));
     } else {
         FMany<1> one;
         one.p[0] = many.p[0];
         const dim3 grid((uint32_t)rows);
-        if (pl.threads == 512) VL_CUDA(p0, launch_overlap(k_fused<512, 1, 1>, grid, 512, smem, st, true, one));
-        else if (pl.bpm == 3) VL_CUDA(p0, launch_overlap(k_fused<256, 3, 1>, grid, 256, smem, st, true, one));
-        else VL_CUDA(p0, launch_overlap(k_fused<256, 2, 1>, grid, 256, smem, st, true, one));
+        if (slot >= 0 && pl.bpm > 1 && p0->nI >= FUSED_HAND_INSTRS && !vl_exact_scratch(p0)) {
+            VlExactArgs &ex = one.p[0].ex;
+            const int rc = hand_scratch(p0, slot, rows, &ex);
+            if (rc != VL_OK) return rc;
+            VL_CUDA(p0, pl.bpm == 3 ? launch_overlap(k_fused<256, 3, 1, true>, grid, 256, smem, st, true, one)
+                                    : launch_overlap(k_fused<256, 2, 1, true>, grid, 256, smem, st, true, one));
+            return vl_exact_run(p0, ex, d_cand[0], pitch[0], d_out[0], st, dict, true);
+        }
+        if (pl.threads == 512) VL_CUDA(p0, launch_overlap(k_fused<512, 1, 1, false>, grid, 512, smem, st, true, one));
+        else if (pl.bpm == 3) VL_CUDA(p0, launch_overlap(k_fused<256, 3, 1, false>, grid, 256, smem, st, true, one));
+        else VL_CUDA(p0, launch_overlap(k_fused<256, 2, 1, false>, grid, 256, smem, st, true, one));
     }
     return VL_OK;
 }

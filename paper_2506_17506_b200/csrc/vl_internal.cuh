@@ -127,7 +127,7 @@ struct vl_program {
     uint4 *d_vcons = nullptr;               // [V] (class first | class end << 16, alignment, ceil(2^32 / alignment), 0); null = no rules
     uint16_t *d_rs_prefix = nullptr;        // [P+1] reserved registers below r; null = none reserved
     uint32_t *d_th_off = nullptr, *d_th = nullptr;  // per block: vregs occupied through the whole block
-    // live-after lists without the block's through-set, for the recount: the list of instruction i of
+    // live-after lists without the block's through-set, for the exact counts: the list of instruction i of
     // block b is ls[lo_off[i] - ls_adj[b] - i * th_cnt[b] ...), |live-after| - th_cnt[b] entries
     // per instruction, for the exact counts: {first entry of its short list, entries | definitions << 16 | reads (at most
     // 127) << 24 | first defined vreg is in the block's through-set << 31, first defined vreg, first operand}
@@ -190,6 +190,7 @@ struct vl_program {
         uint32_t *thm = nullptr;       // [groups][n_blocks][mask words][2][32] through-set masks
         uint64_t rows = 0, aw = 0, vregs = 0, chunks = 0;
     } vs[VL_LANES + 2];              // one per lane, then one per staging buffer of vl_verify_host
+    VScratch fs[VL_LANES + 2];       // the same for what k_fused hands to k_exact: cstate, anom, work and racc only
     uint32_t sub_batch = 5120;       // candidates per pass of the verify kernels
     uint32_t lanes_opt = 3;          // lanes in use (1 = everything in order on the caller's stream)
     cudaEvent_t ev_fork = nullptr, ev_join[VL_LANES] = {};
@@ -252,13 +253,13 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
 bool vl_fused_wanted(vl_program *p, uint64_t K);
 bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
-                 vl_verdict *const *d_out, cudaStream_t st, bool dict);
+                 vl_verdict *const *d_out, cudaStream_t st, bool dict, int slot);  // slot: working set, -1: none
 // The exact counts of the batched kernels' listed candidates (k_exact, vl_fused.cu).
 // A candidate is listed twice, in items of about EXACT_FINE_CHUNKS and of about EXACT_PART_CHUNKS chunks of the walk.  The
 // fine ones are taken if each has a thread block of its own: 1,000 rows of 8,000 instructions of which 100 fail 77 us
 // against 81 for the whole call, 777 of 11,317 with 39 failing 103.5 against 109.  Beyond that what an item costs before
 // its first count weighs more: 350 of the 1,000 failing 95 us in fine items, 85.5 in coarse ones.
-#define EXACT_HDR 4         // words in front of the fine items, then the coarse ones: numbers of coarse and of fine items
+#define EXACT_HDR 4         // words in front of the fine items, then the coarse ones: numbers of coarse and of fine items, blocks done
 #define EXACT_MAX_PARTS 32  // items of one candidate, at most
 #define EXACT_PART_CHUNKS 6
 #define EXACT_FINE_CHUNKS 2
@@ -266,11 +267,27 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
 // per-candidate state between the kernels (8 words)
 enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_WALK = 6, CS_THCOL = 7 };
 enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
+// Lists candidate k, with that many chunks to count.
+__device__ __forceinline__ void list_exact(uint32_t *work, uint64_t k, uint32_t chunks)
+{
+    const uint32_t parts = min(1u + chunks / EXACT_PART_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
+    const uint32_t fine = min(1u + chunks / EXACT_FINE_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
+    const uint32_t at = EXACT_FINE_ITEMS + atomicAdd(work, parts), fine_at = atomicAdd(work + 1, fine);
+    for (uint32_t j = 0; j < parts; ++j) {
+        work[EXACT_HDR + 2 * (at + j)] = (uint32_t)k;
+        work[EXACT_HDR + 2 * (at + j) + 1] = j | (parts << 8);
+    }
+    for (uint32_t j = 0; j < fine && fine_at + j < EXACT_FINE_ITEMS; ++j) {
+        work[EXACT_HDR + 2 * (fine_at + j)] = (uint32_t)k;
+        work[EXACT_HDR + 2 * (fine_at + j) + 1] = j | (fine << 8);
+    }
+}
 struct VlExactArgs {
-    const uint32_t *work, *cstate, *anom;
+    uint32_t *work, *cstate, *anom;
     const uint32_t *short_chunk, *chunk_short_off;  // [nS] chunk of every short chunk, [nC + 1] first short chunk of every chunk
     uint32_t *racc;               // [rows][4] overlaps, complement of the lowest instruction, bank tally, parts done; all 0
-    uint32_t AW, fine_items;      // fine_items: up to that many fine items are taken
+    uint32_t AW, nC, fine_items;      // fine_items: up to that many fine items are taken
+    uint32_t after_fused;         // the candidates come from k_fused: their bank tally is exact, and the counts are reset at the end
     unsigned char *scratch;       // vl_exact_scratch bytes, null if 0
 };
 uint32_t vl_exact_blocks(vl_program *p);  // thread blocks of k_exact: one item each at a time

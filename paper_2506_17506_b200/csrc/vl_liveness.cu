@@ -795,7 +795,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
         for (uint32_t i = q.chunk_i0[c] + (tid + LV_NT - 32) % LV_NT; i < i1; i += LV_NT) {
             const size_t at = base + n_entry + q.ev_rel[i];
             instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) { put_event(q.ev, at + e, v, q.width[v], test, toggle); },
-                         [&](uint32_t o) {  // listed (in any order) for the recount of through-set collisions
+                         [&](uint32_t o) {  // listed (in any order) for the exact counts of through-set collisions
                              uint32_t s = q.chunk_short_off[c];
                              while (s + 1 < q.chunk_short_off[c + 1] && q.piece_i0[q.short_p0[s + 1]] <= i) ++s;
                              const uint32_t v = q.op_vreg[o], member = bit_get(q.blk_th + (size_t)b * q.Wv, v);

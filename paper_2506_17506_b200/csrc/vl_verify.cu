@@ -14,10 +14,9 @@
 //            event stream is the same for all lanes, the occupancy bitmasks of a lane sit in shared
 //            memory at [word][slot][lane] (Safety).  A chunk whose walk sees no collision provably
 //            has no overlap.  The thread block that ends a group of 64 candidates writes the verdicts
-//            of its clean candidates and lists the others for the recount.
-// k_recount  candidates with a collision are recounted exactly from the per-instruction live-after
-//            lists: work items (a piece of a colliding chunk, a block whose through-set collided, the
-//            bank tally of a candidate) taken from a shared cursor, long items first.
+//            of its clean candidates and lists the others for k_exact
+//            (vl_fused.cu), which counts their overlaps from the per-instruction live-after lists.
+// Jobs of up to a few hundred rows take one kernel instead (k_fused, vl_fused.cu).
 #include <cuda.h>
 
 #include <algorithm>
@@ -468,7 +467,7 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
     // sources minus the number of banks they touch.  Hb[v] holds, per candidate, the bank of T[v]
     // as a one-hot nibble: the banks touched are the bits of the OR over the sources (list entries
     // repeat their first source in unused slots).  The bits are counted with carry-save adders, 8
-    // entries per round.  Candidates with a collision get the general tally in k_recount.
+    // entries per round.  Candidates with a collision are put right in k_exact.
     if (q.bank_fast) {
         auto csa = [](uint32_t &h, uint32_t &l, uint32_t a, uint32_t b, uint32_t c) {
             const uint32_t u = a ^ b;
@@ -1131,17 +1130,7 @@ __device__ __forceinline__ void finish_candidate(uint64_t k, uint32_t nC, uint32
         if (walk & WALK_FULL) chunks += nC;
         else if (walk)
             for (uint32_t w = 0; w < AW; ++w) chunks += __popc(__ldcg(anom + k * AW + w));
-        const uint32_t parts = min(1u + chunks / EXACT_PART_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
-        const uint32_t fine = min(1u + chunks / EXACT_FINE_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
-        const uint32_t at = EXACT_FINE_ITEMS + atomicAdd(work, parts), fine_at = atomicAdd(work + 1, fine);
-        for (uint32_t j = 0; j < parts; ++j) {
-            work[EXACT_HDR + 2 * (at + j)] = (uint32_t)k;
-            work[EXACT_HDR + 2 * (at + j) + 1] = j | (parts << 8);
-        }
-        for (uint32_t j = 0; j < fine && fine_at + j < EXACT_FINE_ITEMS; ++j) {
-            work[EXACT_HDR + 2 * (fine_at + j)] = (uint32_t)k;
-            work[EXACT_HDR + 2 * (fine_at + j) + 1] = j | (fine << 8);
-        }
+        list_exact(work, k, chunks);
         return;
     }
     const uint32_t fl = __ldcg(cs + CS_FLAGS), first = __ldcg(cs + CS_FIRST);
@@ -1195,7 +1184,7 @@ struct WalkSlot {
 // Applies the 8 events of the group at shared address ga to the occupancy masks of this lane's two
 // candidates; viol collects the occupied bits that a test found.  Toggling returns the old word:
 // occupied and released are both a toggle as long as no collision has been seen (after one, the
-// chunk is recounted exactly anyway).  The caller vouches that no range of the group reaches into
+// chunk is counted exactly anyway).  The caller vouches that no range of the group reaches into
 // the next 32-bit word for any walked candidate and that none is wider than 32 registers: every
 // event is one atomic per candidate.  Masks and addresses are computed with multiply-adds where
 // possible, to spare the integer ALU pipe.
@@ -1400,7 +1389,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 3) k_walk(const WParams q)
     const uint32_t grp = blockIdx.y, c = blockIdx.x * n_warps + warp;
     const uint64_t kA = (uint64_t)grp * TGW + 2 * lane, kB = kA + 1;
     uint32_t *csA = q.cstate + kA * 8, *csB = csA + 8;  // rows beyond K exist in the working buffers (whole groups)
-    // candidates beyond K, and candidates that are recounted in full anyway (their table may hold
+    // candidates beyond K, and candidates that are counted in full anyway (their table may hold
     // anything), are not walked
     const bool walkedA = kA < q.K && !(csA[CS_WALK] & WALK_FULL), walkedB = kB < q.K && !(csB[CS_WALK] & WALK_FULL);
     const unsigned char *tgb = reinterpret_cast<const unsigned char *>(q.tg + (uint64_t)grp * (q.V + 1) * TGW + 2 * lane);
@@ -1476,7 +1465,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 3) k_walk(const WParams q)
         }
     }
     // the thread block that finishes a group's last chunk writes the verdicts of the group's clean
-    // candidates and lists the others for the recount
+    // candidates and lists the others for k_exact
     __shared__ uint32_t s_last;
     __threadfence();
     __syncthreads();
@@ -1866,7 +1855,7 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
 {
     if (vl_fused_wanted(p, K)) {
         kt_mark(p, st);
-        const int rf = vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, dict);
+        const int rf = vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, dict, slot);
         for (int j = 0; j < 4; ++j) kt_mark(p, st);
         return rf;
     }
@@ -1898,7 +1887,7 @@ struct FusedGroup {
     {
         const uint32_t m = n;
         n = 0;
-        return vl_fused_run(m, progs, cand, K, pitch, out, st, dict);
+        return vl_fused_run(m, progs, cand, K, pitch, out, st, dict, -1);
     }
 };
 }  // namespace
@@ -1948,7 +1937,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
         vl_program *p = progs[j];
         if (shared[j]) continue;
         if (vl_fused_wanted(p, K[j])) {
-            rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, lane[job % L], dict);
+            rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, lane[job % L], dict, (int)(job % L));
             ++job;
             continue;
         }

@@ -85,3 +85,23 @@ def test_exact_count_items(B, oracle_mod, failing):
     op = oracle_mod.OracleProgram(p)
     _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows), f"{failing} failing")
     gp.close()
+
+
+@pytest.mark.parametrize("P,n_banks,K", [(64, 4, 149), (500, 3, 300), (250, 2, 444)])
+def test_counts_handed_over(B, oracle_mod, P, n_banks, K):
+    """Programs large enough that the rows of a short job leave their counts to the kernel for those: general and
+    fast bank tally, rows that collide everywhere and hardly, two calls in a row."""
+    V = 7200
+    blocks = [[([i], [i - 1, i - 2, i - 17] if i >= 17 else []) for i in range(b * 1800, (b + 1) * 1800)] for b in range(4)]
+    p = synth.program_from_lists(blocks, [(0, 1), (1, 1), (1, 2), (2, 3)], V, [1 + (v % 5 == 0) for v in range(V)], P, n_banks)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    rng = np.random.default_rng(K)
+    good = (np.arange(V) * 2) % (P - P % 2)
+    for call in range(2):
+        rows = np.stack([H.row_from_table(p, np.where(rng.random(V) < [0, 0, 3e-4, 0.05, 1][k % 5], rng.integers(0, P, V), good))
+                         for k in range(K)])
+        _assert_same(_gpu_verify(B, gp, rows), op.verify(lv, rows), f"P {P} call {call}")
+    gp.close()
