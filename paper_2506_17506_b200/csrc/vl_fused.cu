@@ -935,8 +935,8 @@ FParams fused_params(const vl_program *p, bool dict)
 
 }  // namespace
 
-// Jobs whose rows the device holds at a time: 10 us against 45 for 100 rows of a program of 2,000 instructions, 60
-// against 86 for 148 rows of one of 8,000 (17 against 73 when no row fails), 54 against 146 for one of 32,000.  Beyond
+// Jobs whose rows the device holds at a time: 10 us against 45 for 100 rows of a program of 2,000 instructions, 40
+// against 81 for 148 rows of one of 8,000 (14 against 66 when no row fails), 54 against 146 for one of 32,000.  Beyond
 // that the batched kernels, which read the program's tables for 8 or 64 rows at a time, win as soon as the rounds of
 // this kernel (about 3 us and 3.5 ns per instruction) take longer than their launches: 600 rows of 2,000 instructions 31
 // against 42 us, 1,000 rows 41 against 42; 3,000 rows of 64 instructions 40 against 68, 10,000 rows 124 against 79.
