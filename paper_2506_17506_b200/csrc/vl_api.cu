@@ -125,10 +125,13 @@ void *vl_pinned_get()
             const uint32_t j = s.free_slots.back();
             s.free_slots.pop_back();
             ++s.used;
-            return s.ptr + (size_t)j * PINNED_BYTES;
+            char *slot = s.ptr + (size_t)j * PINNED_BYTES;
+            memset(slot, 0, PINNED_BYTES);  // (what its last owner left must not read as an answer)
+            return slot;
         }
     PinnedSlab s{nullptr, 1, {}};
     if (cudaHostAlloc((void **)&s.ptr, PINNED_SLOTS * PINNED_BYTES, cudaHostAllocPortable) != cudaSuccess) return nullptr;
+    memset(s.ptr, 0, PINNED_SLOTS * PINNED_BYTES);
     for (uint32_t j = PINNED_SLOTS; j-- > 1;) s.free_slots.push_back((uint16_t)j);
     g_pinned.push_back(std::move(s));
     return g_pinned.back().ptr;
@@ -288,9 +291,7 @@ extern "C" void vl_program_destroy(vl_program *p)
     cudaSetDevice(p->device);
     vl_live_settle(p);
     vl_free_liveness(p);
-    vl_pinned_put(p->h_live);
     if (p->h_out_pinned) cudaFreeHost(p->h_out_pinned);
-    vl_pinned_put(p->h_rs);
     cudaFree(p->d_diag_T);
     cudaFree(p->d_diag_n);
     if (p->ev_live) cudaEventDestroy(p->ev_live);
@@ -311,6 +312,8 @@ extern "C" void vl_program_destroy(vl_program *p)
     if (p->ev_pre) cudaEventDestroy(p->ev_pre);
     for (cudaEvent_t ev : p->ev_join)
         if (ev) cudaEventDestroy(ev);
+    vl_pinned_put(p->h_live);  // (last: the frees above wait for kernels that may still write to them)
+    vl_pinned_put(p->h_rs);
     delete p;
 }
 

@@ -302,7 +302,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
 // follows the VL_LANES lanes in the array) and the handle's fork / join events.
 int vl_lane_streams(vl_program *p, cudaStream_t **lanes, cudaEvent_t **done = nullptr);
 void vl_free_liveness(vl_program *p);
-// 128 bytes of pinned host memory (a pinned allocation of its own takes 155 us); null if there is none.
+// 128 bytes of pinned host memory, all zero (a pinned allocation of its own takes 155 us); null if there is none.
 void *vl_pinned_get();
 void vl_pinned_put(void *slot);
 // Waits for a liveness run that is still in flight and checks its outcome; VL_OK if none is pending.

@@ -143,3 +143,32 @@ def test_loop_stops_at_the_first_batch_with_a_passing_row(B, oracle_mod, batch_r
     out, done, first = gp.vl_verify_until_pass(empty, batch_rows)
     assert (done, first) == (0, 0)
     gp.close()
+
+
+def test_loop_of_a_new_handle_does_not_read_the_record_of_a_destroyed_one(B, oracle_mod):
+    """Handles whose loops ended in their first batch are destroyed; the loops of new handles, which may be given the
+    same pinned records, check rows that fail, and rows that pass in a later batch only."""
+    wl = synth.workload(0)
+    p = synth.build_program(wl.shapes[0], wl.seeds[0])
+    rows, faults = synth.candidate_rows(p, 100, 0.5, wl.seeds[0])
+    good, bad = rows[faults[:, 0] == 0], rows[faults[:, 0] != 0]
+    assert len(good) >= 4 and len(bad) >= 20
+    old = [B.Program(p) for _ in range(3)]
+    for gp in old:
+        gp.vl_liveness()
+    for gp in old:
+        assert gp.vl_verify_until_pass(_to_dev(good[:4]), 4)[1:] == (4, 0)
+    for gp in old:
+        gp.close()
+    new = [B.Program(p) for _ in range(3)]
+    for gp in new:
+        gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    for j, gp in enumerate(new):
+        r = np.ascontiguousarray(np.concatenate([bad[:20], good[:1]])) if j else np.ascontiguousarray(bad[:20])
+        out, done, first = gp.vl_verify_until_pass(_to_dev(r), 4)
+        assert (done, first) == ((21, 20) if j else (20, 20)), f"loop {j}"
+        assert B.verdicts_to_numpy(out).tobytes() == op.verify(lv, r).tobytes()
+    for gp in new:
+        gp.close()
