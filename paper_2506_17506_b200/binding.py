@@ -186,6 +186,7 @@ class Program:
     def __init__(self, prog, device: int = 0):
         self.n_blocks, self.n_instrs, self.n_vregs = prog.n_blocks, prog.n_instrs, prog.n_vregs
         self.n_operands = prog.n_operands
+        self.n_banks = prog.B
         self.pitch = max(8, (prog.n_operands + 7) // 8 * 8)
         self.device = device
         desc, keep = make_desc(prog)
@@ -312,10 +313,12 @@ class Program:
 
     def vl_diagnose(self, row, cap: int = 1 << 16, n_banks: int = 4, stream=None):
         """Diagnostics of one candidate (CUDA uint16 tensor of n_operands entries or more): returns
-        (conflict records [n, 3] as numpy, total count, kinds per instruction, bank histogram)."""
+        (conflict records [n, 3] as numpy, total count, kinds per instruction, bank histogram of n_banks entries: 0 for
+        banks that the program does not have)."""
         import torch
-        # one buffer on the device, one copy back: count, histogram, kinds, conflict records
-        o_kinds = 8 + 8 * n_banks
+        # one buffer on the device, one copy back: count, histogram (the library writes the program's banks), kinds,
+        # conflict records
+        o_kinds = 8 + 8 * self.n_banks
         o_rec = (o_kinds + self.n_instrs + 15) // 16 * 16
         first = min(cap, 4096)                          # records that come with that copy; more than these are rare
         buf = torch.empty(o_rec + 12 * max(cap, 1), dtype=torch.uint8, device=row.device)
@@ -327,8 +330,9 @@ class Program:
         rec = host[o_rec: o_rec + 12 * min(n, first)]
         if min(n, cap) > first:
             rec = _to_host(buf[o_rec: o_rec + 12 * min(n, cap)], stream)
-        return (rec.copy().view(np.uint32).reshape(-1, 3), n, host[o_kinds: o_kinds + self.n_instrs].copy(),
-                host[8: o_kinds].copy().view(np.uint64))
+        hist = np.zeros(n_banks, dtype=np.uint64)
+        hist[: self.n_banks] = host[8: o_kinds].view(np.uint64)[:n_banks]
+        return rec.copy().view(np.uint32).reshape(-1, 3), n, host[o_kinds: o_kinds + self.n_instrs].copy(), hist
 
     def vl_occupied_masks(self, row, P: int, stream=None):
         """uint8 numpy array [n_instrs, P]: registers the definitions of every instruction must keep off,

@@ -148,3 +148,27 @@ def test_stress_program_rows(B, oracle_mod):
         assert np.array_equal(got, op.occupied(lv, rows[k]))
     assert len(kinds_seen) >= 2
     gp.close()
+
+
+@pytest.mark.parametrize("banks,asked", [(1, 4), (2, 4), (4, 4), (8, 4), (3, 16), (9, 1)])
+def test_histogram_of_more_or_fewer_banks_than_the_program_has(B, oracle_mod, banks, asked):
+    """n_banks is the caller's: banks that the program does not have count 0, and a shorter histogram leaves the violation
+    kinds alone.  (The memory that the call's buffer is cut from is filled with ones first.)"""
+    import torch
+    p = H.random_program(9200 + banks, max_instrs=80, max_vregs=24, P=8, B=banks)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    for row in _garbage_rows(p, 6, banks):
+        dev = _to_dev(row[None, :])[0]
+        for size in (1 << 10, 1 << 20):
+            junk = torch.full((size,), 0x01010101, dtype=torch.int32, device="cuda")
+            del junk
+        _, n, kinds, hist = gp.vl_diagnose(dev, cap=1 << 10, n_banks=asked)
+        want = np.zeros(asked, dtype=np.uint64)
+        have = np.asarray(op.bank_histogram(lv, row))
+        want[: min(banks, asked)] = have[:asked]
+        assert hist.dtype == np.uint64 and np.array_equal(hist, want)
+        assert n == len(op.conflicts(lv, row)) and np.array_equal(kinds, op.violations(lv, row))
+    gp.close()
