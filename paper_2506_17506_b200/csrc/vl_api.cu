@@ -438,10 +438,9 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     // A short program's run (tens of microseconds) goes to the caller's stream: leaving it and coming back costs
     // about as much as the run could hide.
     if (p->nI <= LIVE_INLINE_INSTRS) {
-        p->live_stream = (cudaStream_t)stream;
         const cudaStream_t st = (cudaStream_t)stream;
         const int rc = vl_liveness_impl(&p, 1, &st, nullptr, 1);
-        p->live_deferred = true;
+        p->live_stream = st;
         return rc;
     }
     // The run goes to an internal stream, behind everything the caller's stream holds now.  The
@@ -453,15 +452,18 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     cudaStream_t ls = lanes[VL_LIVE_STREAM];
     VL_CUDA(p, cudaEventRecord(p->ev_pre, (cudaStream_t)stream));
     VL_CUDA(p, cudaStreamWaitEvent(ls, p->ev_pre, 0));
-    p->live_stream = ls;
     rc = vl_liveness_impl(&p, 1, &ls, nullptr, 1);
-    p->live_deferred = true;
+    p->live_stream = ls;
     return rc;
 }
 
-int vl_live_join(vl_program *p, cudaStream_t st)
+int vl_live_join(vl_program *p, cudaStream_t from, cudaStream_t st)
 {
-    if (p->live_deferred && p->live_done && st != p->live_stream) VL_CUDA(p, cudaStreamWaitEvent(st, p->live_done, 0));
+    if (!p->live_pending || from == p->live_stream) return VL_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    VL_CUDA(p, cudaStreamIsCapturing(st, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return vl_live_settle(p);  // (a capture cannot wait for what is not part of it)
+    VL_CUDA(p, cudaStreamWaitEvent(st, p->live_done, 0));
     return VL_OK;
 }
 
@@ -478,12 +480,11 @@ extern "C" int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *str
     cudaEvent_t *done = nullptr;
     int rc = vl_lane_streams(p0, &lane, &done);
     if (rc != VL_OK) return rc;
-    for (uint32_t j = 0; j < n; ++j) {
-        // an earlier single run of one of these programs may still sit on the liveness stream
-        if ((rc = vl_live_join(progs[j], st)) != VL_OK) return rc;
-        progs[j]->live_deferred = false;
+    if (n == 1) {
+        rc = vl_liveness_impl(progs, 1, &st, nullptr, 1);
+        p0->live_stream = st;
+        return rc;
     }
-    if (n == 1) return vl_liveness_impl(progs, 1, &st, nullptr, 1);
     VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
     for (uint32_t l = 0; l < VL_LANES; ++l) VL_CUDA(p0, cudaStreamWaitEvent(lane[l], p0->ev_fork, 0));
     std::vector<vl_program *> once(progs, progs + n);  // a handle given twice runs once
@@ -491,6 +492,7 @@ extern "C" int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *str
     once.erase(std::unique(once.begin(), once.end()), once.end());
     if (once.size() == n) once.assign(progs, progs + n);  // (in the caller's order)
     rc = vl_liveness_impl(once.data(), (uint32_t)once.size(), lane, done, VL_LANES);
+    for (vl_program *p : once) p->live_stream = st;  // (the lanes join it below)
     // join even after an error, so that the caller's stream stays ordered after what was launched
     for (uint32_t l = 0; l < VL_LANES; ++l) {
         cudaError_t e = cudaEventRecord(p0->ev_join[l], lane[l]);

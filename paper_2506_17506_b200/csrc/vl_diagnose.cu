@@ -157,7 +157,7 @@ extern "C" int vl_occupied_masks(vl_program *p, const uint16_t *d_row, uint32_t 
     if (!p->live_ok) return VL_ERR_LIVENESS_NOT_RUN;
     VL_CUDA(p, cudaSetDevice(p->device));
     {   // a liveness run may still be in flight: the kernels below are ordered behind it
-        const int rc = vl_live_join(p, (cudaStream_t)stream);
+        const int rc = vl_live_join(p, (cudaStream_t)stream, (cudaStream_t)stream);
         if (rc != VL_OK) return rc;
     }
     if (!p->d_diag_T) VL_CUDA(p, cudaMalloc(&p->d_diag_T, sizeof(unsigned long long) * (p->V ? p->V : 1)));
@@ -187,7 +187,7 @@ extern "C" int vl_diagnose(vl_program *p, const uint16_t *d_row, uint64_t cap, v
     if (!p->live_ok) return VL_ERR_LIVENESS_NOT_RUN;
     VL_CUDA(p, cudaSetDevice(p->device));
     {   // a liveness run may still be in flight: the kernels below are ordered behind it
-        const int rc = vl_live_join(p, (cudaStream_t)stream);
+        const int rc = vl_live_join(p, (cudaStream_t)stream, (cudaStream_t)stream);
         if (rc != VL_OK) return rc;
     }
     if (!p->d_diag_T) VL_CUDA(p, cudaMalloc(&p->d_diag_T, sizeof(unsigned long long) * (p->V ? p->V : 1)));

@@ -986,7 +986,7 @@ static int hand_scratch(vl_program *p, int slot, uint64_t rows, VlExactArgs *ex)
 
 // Up to VL_FUSED_MANY jobs in one launch on st.
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
-                 vl_verdict *const *d_out, cudaStream_t st, bool dict, int slot)
+                 vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot)
 {
     vl_program *p0 = progs[0];
     static std::mutex mtx;
@@ -1017,7 +1017,7 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         smem = std::max(smem, q.sm.total);
         q.cand = d_cand[j]; q.K = K[j]; q.pitch = pitch[j]; q.out = d_out[j];
         rows = std::max(rows, K[j]);
-        const int rc = vl_live_join(p, st);
+        const int rc = vl_live_join(p, from, st);
         if (rc != VL_OK) return rc;
     }
     if (n > 1) {

@@ -165,11 +165,10 @@ struct vl_program {
     cudaEvent_t ev_live = nullptr;
     cudaEvent_t live_done = nullptr;  // the event behind the last run: ev_live, or the one of the lane a batch ran it on
     bool live_pending = false;
-    // vl_liveness of a long program runs on an internal stream (live_stream) behind what the caller's stream held
-    // when it was called; the caller's stream is not made to wait.  Calls that read the results make their stream wait
-    // for ev_live (vl_live_join); the table kernel, which reads the program's operand tables only,
-    // runs beside the liveness kernels.
-    bool live_deferred = false;
+    // The stream that the run in flight is ordered on: the caller's, or (a long program's vl_liveness) an internal one,
+    // behind what the caller's stream held when it was called.  Calls on other streams that read the results make theirs
+    // wait for live_done (vl_live_join); the table kernel, which reads the program's operand tables only, runs beside the
+    // liveness kernels.
     cudaStream_t live_stream = nullptr;
     cudaEvent_t ev_pre = nullptr;
     // The operand tables of the verify kernels (vreg per operand, first-occurrence bits, table
@@ -253,7 +252,7 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
 bool vl_fused_wanted(vl_program *p, uint64_t K);
 bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
-                 vl_verdict *const *d_out, cudaStream_t st, bool dict, int slot);  // slot: working set, -1: none
+                 vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot);  // slot: working set, -1: none
 // The exact counts of the batched kernels' listed candidates (k_exact, vl_fused.cu).
 // A candidate is listed twice, in items of about EXACT_FINE_CHUNKS and of about EXACT_PART_CHUNKS chunks of the walk.  The
 // fine ones are taken if each has a thread block of its own: 1,000 rows of 8,000 instructions of which 100 fail 77 us
@@ -307,7 +306,8 @@ void *vl_pinned_get();
 void vl_pinned_put(void *slot);
 // Waits for a liveness run that is still in flight and checks its outcome; VL_OK if none is pending.
 int vl_live_settle(vl_program *p);
-int vl_live_join(vl_program *p, cudaStream_t st);  // st waits for the liveness run in flight, if any
+// st waits for the liveness run in flight, if any; from: the stream that st's work of this call was forked from, or st.
+int vl_live_join(vl_program *p, cudaStream_t from, cudaStream_t st);
 // Multiprocessors of a device / of the handle's device (asked once).
 int vl_device_sm_count(int device);
 int vl_sm_count(vl_program *p);

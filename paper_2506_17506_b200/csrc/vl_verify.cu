@@ -1738,7 +1738,7 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
 // One pass: the four kernels over n <= sub candidates, in order on `st`, with working set `slot`.  early: each kernel's
 // blocks may start, and wait, while the kernel before it drains (passes of other streams would miss the room they hold).
 int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t n, uint64_t pitch, vl_verdict *d_out,
-             cudaStream_t st, int slot, bool dict, bool stagger, bool early)
+             cudaStream_t from, cudaStream_t st, int slot, bool dict, bool stagger, bool early)
 {
     // what the rows hold: one column per operand occurrence, or one per dictionary entry
     const uint32_t nO = dict ? p->nD : p->nO, nOp8 = dict ? p->nD8 : p->nOp8;
@@ -1809,7 +1809,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     // Everything from here on reads what vl_liveness computes (through-sets, walk events, live-after
     // lists); the table kernel above reads the program's operand tables only and may run beside a
     // liveness run that is still in flight.
-    if ((rc = vl_live_join(p, st)) != VL_OK) return rc;
+    if ((rc = vl_live_join(p, from, st)) != VL_OK) return rc;
     if (p->nC) {
         WParams wq{};
         wq.V = p->V; wq.P = p->P; wq.nB = p->nB; wq.nC = p->nC; wq.Wp = pp.Wp; wq.AW = (uint32_t)vs.aw;
@@ -1855,7 +1855,7 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
 {
     if (vl_fused_wanted(p, K)) {
         kt_mark(p, st);
-        const int rf = vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, dict, slot);
+        const int rf = vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, st, dict, slot);
         for (int j = 0; j < 4; ++j) kt_mark(p, st);
         return rf;
     }
@@ -1863,7 +1863,7 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
     int rc = plan_passes(p, K, &pp);
     if (rc != VL_OK) return rc;
     for (uint64_t kb = 0; kb < K; kb += pp.sub) {
-        rc = run_pass(p, pp, d_cand + kb * pitch, std::min(pp.sub, K - kb), pitch, d_out + kb, st, slot, dict,
+        rc = run_pass(p, pp, d_cand + kb * pitch, std::min(pp.sub, K - kb), pitch, d_out + kb, st, st, slot, dict,
                       kb == 0 && K >= 8ull * 2 * (uint64_t)vl_sm_count(p), true);
         if (rc != VL_OK) return rc;
     }
@@ -1883,11 +1883,11 @@ struct FusedGroup {
         progs[n] = p; cand[n] = c; K[n] = k; pitch[n] = pt; out[n] = o;
         return ++n == VL_FUSED_MANY;
     }
-    int run(cudaStream_t st, bool dict)
+    int run(cudaStream_t from, cudaStream_t st, bool dict)
     {
         const uint32_t m = n;
         n = 0;
-        return vl_fused_run(m, progs, cand, K, pitch, out, st, dict, -1);
+        return vl_fused_run(m, progs, cand, K, pitch, out, from, st, dict, -1);
     }
 };
 }  // namespace
@@ -1912,13 +1912,13 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
         for (uint32_t j = 0; j < nprog; ++j) {
             if (K[j] == 0) continue;
             if (nprog > 1 && vl_fused_shares(progs[j], K[j])) {
-                if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j]) && (rc = g.run(st, dict)) != VL_OK) return rc;
+                if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j]) && (rc = g.run(st, st, dict)) != VL_OK) return rc;
                 continue;
             }
             rc = vl_verify_impl(progs[j], d_cand[j], K[j], pitch[j], d_out[j], st, 0, dict);
             if (rc != VL_OK) return rc;
         }
-        return g.n ? g.run(st, dict) : VL_OK;
+        return g.n ? g.run(st, st, dict) : VL_OK;
     }
     VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
     for (uint32_t l = 0; l < L; ++l) VL_CUDA(p0, cudaStreamWaitEvent(lane[l], p0->ev_fork, 0));
@@ -1929,15 +1929,15 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     for (uint32_t j = 0; j < nprog && nprog > 1 && rc == VL_OK; ++j) {
         if (K[j] == 0 || !vl_fused_shares(progs[j], K[j])) continue;
         shared[j] = 1;
-        if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j])) rc = g.run(lane[job++ % L], dict);
+        if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j])) rc = g.run(st, lane[job++ % L], dict);
     }
-    if (rc == VL_OK && g.n) rc = g.run(lane[job++ % L], dict);
+    if (rc == VL_OK && g.n) rc = g.run(st, lane[job++ % L], dict);
     for (uint32_t j = 0; j < nprog && rc == VL_OK; ++j) {
         if (K[j] == 0) continue;
         vl_program *p = progs[j];
         if (shared[j]) continue;
         if (vl_fused_wanted(p, K[j])) {
-            rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, lane[job % L], dict, (int)(job % L));
+            rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, st, lane[job % L], dict, (int)(job % L));
             ++job;
             continue;
         }
@@ -1949,7 +1949,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
         uint64_t s = 0;
         for (uint64_t kb = 0; kb < K[j] && rc == VL_OK; kb += pp.sub, ++s, ++job)
             rc = run_pass(p, pp, d_cand[j] + kb * pitch[j], std::min(pp.sub, K[j] - kb), pitch[j], d_out[j] + kb,
-                          lane[(base + s) % L], (int)(s % L), dict, job == 0 && K[j] >= 8ull * 2 * (uint64_t)vl_sm_count(p), false);
+                          st, lane[(base + s) % L], (int)(s % L), dict, job == 0 && K[j] >= 8ull * 2 * (uint64_t)vl_sm_count(p), false);
     }
     // join even after an error, so that the caller's stream stays ordered after what was launched
     for (uint32_t l = 0; l < L; ++l) {

@@ -1,0 +1,101 @@
+"""Calls that read liveness results wait for a run that is still in flight, whatever stream it is ordered on.  The run is
+held back by a kernel that sleeps for half a second in front of it; the results go to pinned host memory, which the test
+looks at meanwhile: nothing may have been written."""
+import threading
+import time
+
+import numpy as np
+import pytest
+
+from paper_2506_17506_b200 import synth
+from tests import helpers as H
+from tests.test_gpu_parity import _garbage_rows, _to_dev
+
+pytestmark = pytest.mark.gpu
+
+SLEEP_CYCLES = 1_000_000_000   # about half a second
+
+
+@pytest.fixture(scope="module")
+def B():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2506_17506_b200 import binding
+    return binding
+
+
+def _program(kind):
+    if kind == "short":
+        wl = synth.workload(1)
+        return synth.build_program(wl.shapes[0], wl.seeds[0])
+    wl = synth.workload(2)                                   # 8,000 instructions: its liveness takes an internal stream
+    return synth.build_program(wl.shapes[0], wl.seeds[0])
+
+
+def _call(B, gp, p, call, dev, stream):
+    """Buffers for the call (allocating them may wait for the device), and a function that makes it."""
+    import torch
+    n = {"verify": dev.shape[0] * 16, "diagnose": p.n_instrs, "occupied": p.n_instrs * ((p.P + 31) // 32) * 4}[call]
+    host = torch.full((n,), 0xA5, dtype=torch.uint8, pin_memory=True)
+    scratch = torch.zeros(1 << 20, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+
+    def go():
+        s = B._stream_ptr(stream)
+        if call == "verify":
+            return B._lib.vl_verify(gp.handle, dev.data_ptr(), dev.shape[0], dev.shape[1], host.data_ptr(), s)
+        if call == "diagnose":
+            return B._lib.vl_diagnose(gp.handle, dev.data_ptr(), 1000, scratch.data_ptr() + 64, scratch.data_ptr(), host.data_ptr(), None, s)
+        return B._lib.vl_occupied_masks(gp.handle, dev.data_ptr(), host.data_ptr(), s)
+
+    go()                                     # the working sets of the handle are made now
+    torch.cuda.synchronize()
+    host.fill_(0xA5)
+    return go, host.numpy(), (host, scratch)
+
+
+def _check(B, oracle_mod, p, call, made, rows, held, what):
+    """Makes the call in a thread of its own (it may wait on the host) while `held` sleeps."""
+    import torch
+    go, host, keep = made
+    rc = []
+    t = threading.Thread(target=lambda: rc.append(go()))
+    t.start()
+    time.sleep(0.15)
+    early = bool((host != 0xA5).any())
+    assert not held.query(), f"{what}: the sleep ended too soon"
+    t.join()
+    torch.cuda.synchronize()
+    assert rc == [B.VL_OK], what
+    assert not early, f"{what}: results were written before the liveness run had finished"
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    if call == "verify":
+        assert host.tobytes() == op.verify(lv, rows).tobytes(), what
+    elif call == "diagnose":
+        assert np.array_equal(host, op.violations(lv, rows[0])), what
+    else:
+        bits = np.unpackbits(host.reshape(p.n_instrs, -1), axis=1, bitorder="little")[:, : p.P]
+        assert np.array_equal(bits, op.occupied(lv, rows[0])), what
+
+
+@pytest.mark.parametrize("call", ["verify", "diagnose", "occupied"])
+@pytest.mark.parametrize("n", [1, 2])
+def test_batch_in_flight_on_another_stream(B, oracle_mod, call, n):
+    import torch
+    p = _program("short")
+    gps = [B.Program(p) for _ in range(n)]
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    rows = _garbage_rows(p, 20, 4)
+    dev = _to_dev(rows)
+    for _ in range(2):                       # (from the second run on the lengths are known and the call returns at once)
+        B.vl_liveness_batch(gps, s1)
+        torch.cuda.synchronize()
+    made = _call(B, gps[-1], p, call, dev, s2)
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(SLEEP_CYCLES)
+    B.vl_liveness_batch(gps, s1)
+    _check(B, oracle_mod, p, call, made, rows, s1, f"{call} after a batch of {n}")
+    for gp in gps:
+        gp.close()
