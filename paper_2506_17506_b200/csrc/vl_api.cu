@@ -439,9 +439,8 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     // about as much as the run could hide.
     if (p->nI <= LIVE_INLINE_INSTRS) {
         const cudaStream_t st = (cudaStream_t)stream;
-        const int rc = vl_liveness_impl(&p, 1, &st, nullptr, 1);
-        p->live_stream = st;
-        return rc;
+        VL_CUDA(p, cudaStreamGetId(st, &p->live_stream));
+        return vl_liveness_impl(&p, 1, &st, nullptr, 1);
     }
     // The run goes to an internal stream, behind everything the caller's stream holds now.  The
     // caller's stream does not wait for it: the calls that read the results do (vl_live_join), and
@@ -452,14 +451,16 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     cudaStream_t ls = lanes[VL_LIVE_STREAM];
     VL_CUDA(p, cudaEventRecord(p->ev_pre, (cudaStream_t)stream));
     VL_CUDA(p, cudaStreamWaitEvent(ls, p->ev_pre, 0));
-    rc = vl_liveness_impl(&p, 1, &ls, nullptr, 1);
-    p->live_stream = ls;
-    return rc;
+    VL_CUDA(p, cudaStreamGetId(ls, &p->live_stream));
+    return vl_liveness_impl(&p, 1, &ls, nullptr, 1);
 }
 
 int vl_live_join(vl_program *p, cudaStream_t from, cudaStream_t st)
 {
-    if (!p->live_pending || from == p->live_stream) return VL_OK;
+    if (!p->live_pending) return VL_OK;
+    unsigned long long id = 0;
+    VL_CUDA(p, cudaStreamGetId(from, &id));
+    if (id == p->live_stream) return VL_OK;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     VL_CUDA(p, cudaStreamIsCapturing(st, &cs));
     if (cs != cudaStreamCaptureStatusNone) return vl_live_settle(p);  // (a capture cannot wait for what is not part of it)
@@ -481,9 +482,8 @@ extern "C" int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *str
     int rc = vl_lane_streams(p0, &lane, &done);
     if (rc != VL_OK) return rc;
     if (n == 1) {
-        rc = vl_liveness_impl(progs, 1, &st, nullptr, 1);
-        p0->live_stream = st;
-        return rc;
+        VL_CUDA(p0, cudaStreamGetId(st, &p0->live_stream));
+        return vl_liveness_impl(progs, 1, &st, nullptr, 1);
     }
     VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
     for (uint32_t l = 0; l < VL_LANES; ++l) VL_CUDA(p0, cudaStreamWaitEvent(lane[l], p0->ev_fork, 0));
@@ -491,8 +491,10 @@ extern "C" int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *str
     std::sort(once.begin(), once.end());
     once.erase(std::unique(once.begin(), once.end()), once.end());
     if (once.size() == n) once.assign(progs, progs + n);  // (in the caller's order)
+    unsigned long long id = 0;
+    VL_CUDA(p0, cudaStreamGetId(st, &id));
+    for (vl_program *p : once) p->live_stream = id;  // (the lanes join it below)
     rc = vl_liveness_impl(once.data(), (uint32_t)once.size(), lane, done, VL_LANES);
-    for (vl_program *p : once) p->live_stream = st;  // (the lanes join it below)
     // join even after an error, so that the caller's stream stays ordered after what was launched
     for (uint32_t l = 0; l < VL_LANES; ++l) {
         cudaError_t e = cudaEventRecord(p0->ev_join[l], lane[l]);

@@ -165,11 +165,12 @@ struct vl_program {
     cudaEvent_t ev_live = nullptr;
     cudaEvent_t live_done = nullptr;  // the event behind the last run: ev_live, or the one of the lane a batch ran it on
     bool live_pending = false;
-    // The stream that the run in flight is ordered on: the caller's, or (a long program's vl_liveness) an internal one,
+    // The id of the stream that the run in flight is ordered on (ids are never used again; a caller's handle is, once its
+    // stream is destroyed, and the handle of the per-thread default stream names one in every thread): the caller's, or (a long program's vl_liveness) an internal one,
     // behind what the caller's stream held when it was called.  Calls on other streams that read the results make theirs
     // wait for live_done (vl_live_join); the table kernel, which reads the program's operand tables only, runs beside the
     // liveness kernels.
-    cudaStream_t live_stream = nullptr;
+    unsigned long long live_stream = 0;
     cudaEvent_t ev_pre = nullptr;
     // The operand tables of the verify kernels (vreg per operand, first-occurrence bits, table
     // offsets, vreg descriptors, first definitions) depend on the program alone: they are made by the

@@ -99,3 +99,45 @@ def test_batch_in_flight_on_another_stream(B, oracle_mod, call, n):
     _check(B, oracle_mod, p, call, made, rows, s1, f"{call} after a batch of {n}")
     for gp in gps:
         gp.close()
+
+
+@pytest.mark.parametrize("call", ["verify", "diagnose", "occupied"])
+@pytest.mark.parametrize("kind", ["short", "long"])
+def test_run_in_flight_on_the_per_thread_stream_of_another_thread(B, oracle_mod, call, kind):
+    """The per-thread default stream has the same handle in every thread and is another stream in each."""
+    import torch
+    p = _program(kind)
+    gp = B.Program(p)
+    per_thread = torch.cuda.ExternalStream(2)
+    rows = _garbage_rows(p, 20, 5)
+    dev = _to_dev(rows)
+    for _ in range(2):
+        gp.vl_liveness(per_thread)
+        torch.cuda.synchronize()
+    made = _call(B, gp, p, call, dev, per_thread)
+    with torch.cuda.stream(per_thread):
+        torch.cuda._sleep(SLEEP_CYCLES)
+    gp.vl_liveness(per_thread)
+    _check(B, oracle_mod, p, call, made, rows, per_thread, f"{call}, {kind}")
+    gp.close()
+
+
+def test_run_and_call_on_one_stream(B, oracle_mod):
+    """Liveness and verify of a short program on one stream, over and over, no synchronisation by the caller in between."""
+    import torch
+    p = _program("short")
+    gp = B.Program(p)
+    s = torch.cuda.Stream()
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    outs = []
+    for step in range(5):
+        rows = _garbage_rows(p, 60, 40 + step)
+        dev = _to_dev(rows)
+        torch.cuda.synchronize()
+        gp.vl_liveness(s)
+        outs.append((gp.vl_verify(dev, None, s), dev, rows))
+    torch.cuda.synchronize()
+    for out, _, rows in outs:
+        assert B.verdicts_to_numpy(out).tobytes() == op.verify(lv, rows).tobytes()
+    gp.close()
