@@ -1146,23 +1146,30 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
 
 // The runs of n programs, LV_MANY of them per launch, the launches spread over the n_streams streams.  Everything is
 // recomputed on the device every time.  done[s] is the event recorded behind the work of stream s (null: the
-// program's own; n == 1).  Programs behind the first one with an error are left without a run.
+// program's own; n == 1).  The first program with an error ends the call: those behind it keep what an earlier run left
+// them (their results are computed once more, the same), or stay without a run.
 int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, const cudaEvent_t *done, uint32_t n_streams)
 {
     std::vector<LiveArgs> args(n);
     std::vector<LiveShape> shapes(n);
+    std::vector<uint8_t> had_run(n);
     bool lengths_known = true;
-    int rc = n ? live_attributes(progs[0]) : VL_OK;
+    int rc = n ? live_attributes(progs[0]) : VL_OK, err = VL_OK;
     if (rc != VL_OK) return rc;
     const uint32_t per = n == 1 ? 1 : LV_MANY;
     auto stream_of = [&](uint32_t j) { return (j / per) % n_streams; };
     for (uint32_t j = 0; j < n; ++j) {
         vl_program *p = progs[j];
         vl_live_settle(p);  // the pinned words of an earlier run are about to be reused
-        if ((rc = vl_layout(p, streams[stream_of(j)])) != VL_OK) return rc;
-        if (!p->h_live && !(p->h_live = (uint32_t *)vl_pinned_get())) return VL_ERR_CUDA;
-        if (!p->ev_live) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_live, cudaEventDisableTiming));
-        if ((rc = live_begin(p, args[j], shapes[j], streams[stream_of(j)])) != VL_OK) return rc;
+        had_run[j] = p->live_ok;
+        err = vl_layout(p, streams[stream_of(j)]);
+        if (err == VL_OK && !p->h_live && !(p->h_live = (uint32_t *)vl_pinned_get())) err = VL_ERR_CUDA;
+        if (err == VL_OK && !p->ev_live) {
+            const cudaError_t e = cudaEventCreateWithFlags(&p->ev_live, cudaEventDisableTiming);
+            if (e != cudaSuccess) { p->last_cuda_error = (int)e; err = VL_ERR_CUDA; }
+        }
+        if (err == VL_OK) err = live_begin(p, args[j], shapes[j], streams[stream_of(j)]);
+        if (err != VL_OK) { n = j; break; }  // (those behind it are untouched)
         lengths_known = lengths_known && p->sizes_known;
     }
     auto launch = [&](bool fill) -> int {
@@ -1178,9 +1185,22 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
     if ((rc = launch(false)) != VL_OK) return rc;
     if (!lengths_known)
         for (uint32_t s = 0; s < n_streams; ++s) VL_CUDA(progs[0], cudaStreamSynchronize(streams[s]));
-    int err = VL_OK;
-    for (uint32_t j = 0; j < n; ++j)
-        if ((err = live_lengths(progs[j], args[j])) != VL_OK) { n = j; break; }
+    std::vector<vl_program *> run;  // the programs that the last kernel is launched for
+    for (uint32_t j = 0; j < n; ++j) {
+        if (err != VL_OK && !had_run[j]) continue;
+        const int r = live_lengths(progs[j], args[j]);
+        if (r != VL_OK) {
+            if (err == VL_OK) err = r;
+            continue;
+        }
+        args[run.size()] = args[j];
+        shapes[run.size()] = shapes[j];
+        run.push_back(progs[j]);
+    }
+    if (run.size() < n && lengths_known)  // (a program may move to another stream)
+        for (uint32_t s = 0; s < n_streams; ++s) VL_CUDA(progs[0], cudaStreamSynchronize(streams[s]));
+    progs = run.data();
+    n = (uint32_t)run.size();
     if ((rc = launch(true)) != VL_OK) return rc;
     for (uint32_t j = 0; j < n; ++j)
         if ((rc = live_tables(progs[j], streams[stream_of(j)])) != VL_OK) return rc;

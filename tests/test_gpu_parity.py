@@ -396,3 +396,35 @@ def test_liveness_and_verify_on_different_streams(B, oracle_mod):
         _assert_same(B.verdicts_to_numpy(out), want, f"step {step}")
     _check_liveness_result(B, oracle_mod, gp, p)
     gp.close()
+
+
+@pytest.mark.parametrize("n_before,n_behind", [(1, 1), (0, 2), (50, 60)])
+def test_liveness_batch_with_a_program_that_fails(B, oracle_mod, n_before, n_behind):
+    """The first error ends the call.  Programs in front of it have their results, programs behind it what an earlier run
+    left them: results, or none."""
+    import torch
+    bad = B.Program(synth.program_from_lists([[([], [0]), ([0], [])]], [], 1, [1], 4))      # reads v0 before writing it
+    ps = [H.random_program(9300 + j, max_instrs=120, max_vregs=30, P=64) for j in range(n_before + n_behind)]
+    gps = [B.Program(p) for p in ps]
+    for gp in gps[n_before::2]:          # every second program behind the bad one has run before
+        gp.vl_liveness()
+    with pytest.raises(B.VlError) as e:
+        B.vl_liveness_batch(gps[:n_before] + [bad] + gps[n_before:])
+    assert e.value.code == B.VL_ERR_NOT_STRICT
+    for j, (p, gp) in enumerate(zip(ps, gps)):
+        rows = _garbage_rows(p, 6, j)
+        if j >= n_before and (j - n_before) % 2:
+            with pytest.raises(B.VlError) as e:
+                gp.vl_verify(_to_dev(rows))
+            assert e.value.code == B.VL_ERR_LIVENESS_NOT_RUN
+            continue
+        gp, lv = _check_liveness_result(B, oracle_mod, gp, p)
+        _assert_same(_gpu_verify(B, gp, rows), oracle_mod.OracleProgram(p).verify(lv, rows), f"program {j}")
+    with pytest.raises(B.VlError) as e:
+        bad.vl_verify(torch.zeros((1, 8), dtype=torch.int16, device="cuda").view(torch.uint16))
+    assert e.value.code == B.VL_ERR_LIVENESS_NOT_RUN
+    B.vl_liveness_batch(gps)             # without it every program has its results
+    for p, gp in zip(ps, gps):
+        _check_liveness_result(B, oracle_mod, gp, p)
+        gp.close()
+    bad.close()
