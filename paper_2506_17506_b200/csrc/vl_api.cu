@@ -13,19 +13,16 @@ std::atomic<uint64_t> g_vl_launches{0};
 #define VL_MAX_DEVICES 64
 static std::mutex g_lane_mutex;
 static cudaStream_t g_lanes[VL_MAX_DEVICES][VL_STREAMS];  // the lanes, the liveness stream
-static cudaEvent_t g_lane_done[VL_MAX_DEVICES][VL_LANES];  // behind the last liveness batch of a lane
 static bool g_lanes_made[VL_MAX_DEVICES];
 
-int vl_lane_streams(vl_program *p, cudaStream_t **lanes, cudaEvent_t **done)
+int vl_lane_streams(vl_program *p, cudaStream_t **lanes)
 {
     if (p->device < 0 || p->device >= VL_MAX_DEVICES) return VL_ERR_UNSUPPORTED;
     {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
         if (!g_lanes_made[p->device]) {
-            for (int l = 0; l < VL_LANES; ++l) {
+            for (int l = 0; l < VL_LANES; ++l)
                 VL_CUDA(p, cudaStreamCreateWithFlags(&g_lanes[p->device][l], cudaStreamNonBlocking));
-                VL_CUDA(p, cudaEventCreateWithFlags(&g_lane_done[p->device][l], cudaEventDisableTiming));
-            }
             // the liveness stream: its small kernels go first wherever a multiprocessor has room
             int least = 0, greatest = 0;
             VL_CUDA(p, cudaDeviceGetStreamPriorityRange(&least, &greatest));
@@ -37,7 +34,6 @@ int vl_lane_streams(vl_program *p, cudaStream_t **lanes, cudaEvent_t **done)
     if (!p->ev_pre) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_pre, cudaEventDisableTiming));
     for (int l = 0; l < VL_LANES; ++l)
         if (!p->ev_join[l]) VL_CUDA(p, cudaEventCreateWithFlags(&p->ev_join[l], cudaEventDisableTiming));
-    if (done) *done = g_lane_done[p->device];
     *lanes = g_lanes[p->device];
     return VL_OK;
 }
@@ -294,7 +290,6 @@ extern "C" void vl_program_destroy(vl_program *p)
     if (p->h_out_pinned) cudaFreeHost(p->h_out_pinned);
     cudaFree(p->d_diag_T);
     cudaFree(p->d_diag_n);
-    if (p->ev_live) cudaEventDestroy(p->ev_live);
     p->live_arena.release();
     p->layout_arena.release();
     cudaFree(p->d_blob);
@@ -440,7 +435,7 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     if (p->nI <= LIVE_INLINE_INSTRS) {
         const cudaStream_t st = (cudaStream_t)stream;
         VL_CUDA(p, cudaStreamGetId(st, &p->live_stream));
-        return vl_liveness_impl(&p, 1, &st, nullptr, 1);
+        return vl_liveness_impl(&p, 1, &st, 1);
     }
     // The run goes to an internal stream, behind everything the caller's stream holds now.  The
     // caller's stream does not wait for it: the calls that read the results do (vl_live_join), and
@@ -452,7 +447,7 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
     VL_CUDA(p, cudaEventRecord(p->ev_pre, (cudaStream_t)stream));
     VL_CUDA(p, cudaStreamWaitEvent(ls, p->ev_pre, 0));
     VL_CUDA(p, cudaStreamGetId(ls, &p->live_stream));
-    return vl_liveness_impl(&p, 1, &ls, nullptr, 1);
+    return vl_liveness_impl(&p, 1, &ls, 1);
 }
 
 int vl_live_join(vl_program *p, cudaStream_t from, cudaStream_t st)
@@ -464,7 +459,7 @@ int vl_live_join(vl_program *p, cudaStream_t from, cudaStream_t st)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     VL_CUDA(p, cudaStreamIsCapturing(st, &cs));
     if (cs != cudaStreamCaptureStatusNone) return vl_live_settle(p);  // (a capture cannot wait for what is not part of it)
-    VL_CUDA(p, cudaStreamWaitEvent(st, p->live_done, 0));
+    VL_CUDA(p, cudaStreamWaitEvent(st, p->live_done->ev, 0));
     return VL_OK;
 }
 
@@ -478,12 +473,11 @@ extern "C" int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *str
     VL_CUDA(p0, cudaSetDevice(p0->device));
     cudaStream_t st = (cudaStream_t)stream;
     cudaStream_t *lane = nullptr;
-    cudaEvent_t *done = nullptr;
-    int rc = vl_lane_streams(p0, &lane, &done);
+    int rc = vl_lane_streams(p0, &lane);
     if (rc != VL_OK) return rc;
     if (n == 1) {
         VL_CUDA(p0, cudaStreamGetId(st, &p0->live_stream));
-        return vl_liveness_impl(progs, 1, &st, nullptr, 1);
+        return vl_liveness_impl(progs, 1, &st, 1);
     }
     VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
     for (uint32_t l = 0; l < VL_LANES; ++l) VL_CUDA(p0, cudaStreamWaitEvent(lane[l], p0->ev_fork, 0));
@@ -494,7 +488,7 @@ extern "C" int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *str
     unsigned long long id = 0;
     VL_CUDA(p0, cudaStreamGetId(st, &id));
     for (vl_program *p : once) p->live_stream = id;  // (the lanes join it below)
-    rc = vl_liveness_impl(once.data(), (uint32_t)once.size(), lane, done, VL_LANES);
+    rc = vl_liveness_impl(once.data(), (uint32_t)once.size(), lane, VL_LANES);
     // join even after an error, so that the caller's stream stays ordered after what was launched
     for (uint32_t l = 0; l < VL_LANES; ++l) {
         cudaError_t e = cudaEventRecord(p0->ev_join[l], lane[l]);

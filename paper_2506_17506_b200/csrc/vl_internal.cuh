@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <memory>
 #include <vector>
 
 #include "verilocc.h"
@@ -69,6 +70,12 @@ struct VlArena {
         slabs.clear();
         reset();
     }
+};
+
+// An event that several handles may wait for: the programs of a liveness batch that run on one stream share one.
+struct VlEvent {
+    cudaEvent_t ev = nullptr;
+    ~VlEvent() { if (ev) cudaEventDestroy(ev); }
 };
 
 struct vl_program {
@@ -162,8 +169,8 @@ struct vl_program {
     // the status word and the list lengths to pinned host memory, and the next call that needs the results on
     // the host side (vl_live_settle) waits for the run and checks them.
     uint32_t *h_live = nullptr;      // pinned: [0] status, [2..13] six 64-bit totals, written by the run's kernels
-    cudaEvent_t ev_live = nullptr;
-    cudaEvent_t live_done = nullptr;  // the event behind the last run: ev_live, or the one of the lane a batch ran it on
+    std::shared_ptr<VlEvent> ev_live;    // made by this handle, used again when no other handle waits for it
+    std::shared_ptr<VlEvent> live_done;  // behind the run in flight: ev_live of this handle, or of another one of its batch
     bool live_pending = false;
     // The id of the stream that the run in flight is ordered on (ids are never used again; a caller's handle is, once its
     // stream is destroyed, and the handle of the per-thread default stream names one in every thread): the caller's, or (a long program's vl_liveness) an internal one,
@@ -246,7 +253,7 @@ static inline cudaError_t launch_overlap(void (*kernel)(P...), dim3 grid, uint32
         }                                       \
     } while (0)
 
-int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, const cudaEvent_t *done, uint32_t n_streams);
+int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, uint32_t n_streams);
 // The one-kernel verify path of short jobs (vl_fused.cu): whether a job of K rows takes it, whether it may share a
 // launch with other programs' jobs, and one launch for n <= VL_FUSED_MANY jobs.
 #define VL_FUSED_MANY 48
@@ -300,7 +307,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
                     const uint64_t *pitch, vl_verdict *const *d_out, cudaStream_t st, bool dict = false);
 // The lane streams of the handle's device (created once per device; the liveness stream
 // follows the VL_LANES lanes in the array) and the handle's fork / join events.
-int vl_lane_streams(vl_program *p, cudaStream_t **lanes, cudaEvent_t **done = nullptr);
+int vl_lane_streams(vl_program *p, cudaStream_t **lanes);
 void vl_free_liveness(vl_program *p);
 // 128 bytes of pinned host memory, all zero (a pinned allocation of its own takes 155 us); null if there is none.
 void *vl_pinned_get();

@@ -1145,10 +1145,10 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
 }
 
 // The runs of n programs, LV_MANY of them per launch, the launches spread over the n_streams streams.  Everything is
-// recomputed on the device every time.  done[s] is the event recorded behind the work of stream s (null: the
-// program's own; n == 1).  The first program with an error ends the call: those behind it keep what an earlier run left
-// them (their results are computed once more, the same), or stay without a run.
-int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, const cudaEvent_t *done, uint32_t n_streams)
+// recomputed on the device every time.  One event is recorded per stream; the programs that run on it share it (64
+// programs of one call: 2 events instead of 64).  The first program with an error ends the call: those behind it keep what
+// an earlier run left them (their results are computed once more, the same), or stay without a run.
+int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *streams, uint32_t n_streams)
 {
     std::vector<LiveArgs> args(n);
     std::vector<LiveShape> shapes(n);
@@ -1164,10 +1164,6 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
         had_run[j] = p->live_ok;
         err = vl_layout(p, streams[stream_of(j)]);
         if (err == VL_OK && !p->h_live && !(p->h_live = (uint32_t *)vl_pinned_get())) err = VL_ERR_CUDA;
-        if (err == VL_OK && !p->ev_live) {
-            const cudaError_t e = cudaEventCreateWithFlags(&p->ev_live, cudaEventDisableTiming);
-            if (e != cudaSuccess) { p->last_cuda_error = (int)e; err = VL_ERR_CUDA; }
-        }
         if (err == VL_OK) err = live_begin(p, args[j], shapes[j], streams[stream_of(j)]);
         if (err != VL_OK) { n = j; break; }  // (those behind it are untouched)
         lengths_known = lengths_known && p->sizes_known;
@@ -1206,8 +1202,15 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
         if ((rc = live_tables(progs[j], streams[stream_of(j)])) != VL_OK) return rc;
     for (uint32_t j = 0; j < n; ++j) {
         vl_program *p = progs[j];
-        p->live_done = done ? done[stream_of(j)] : p->ev_live;
-        if (j % per == 0 && j / per < n_streams) VL_CUDA(p, cudaEventRecord(p->live_done, streams[stream_of(j)]));  // once per stream
+        if (j % per == 0 && j / per < n_streams) {  // the first program of a stream
+            if (!p->ev_live || p->ev_live.use_count() > 1) {
+                auto e = std::make_shared<VlEvent>();
+                VL_CUDA(p, cudaEventCreateWithFlags(&e->ev, cudaEventDisableTiming));
+                p->ev_live = e;
+            }
+            VL_CUDA(p, cudaEventRecord(p->ev_live->ev, streams[stream_of(j)]));
+        }
+        p->live_done = progs[stream_of(j) * per]->ev_live;
         p->live_pending = true;
         p->live_ok = true;
     }
@@ -1225,7 +1228,8 @@ int vl_live_settle(vl_program *p)
     if (!p->live_pending) return VL_OK;
     p->live_pending = false;
     p->live_ok = false;
-    VL_CUDA(p, cudaEventSynchronize(p->live_done));
+    const std::shared_ptr<VlEvent> done = std::move(p->live_done);
+    VL_CUDA(p, cudaEventSynchronize(done->ev));
     const uint32_t status = p->h_live[0];
     unsigned long long tot[LV_TOTALS];
     memcpy(tot, p->h_live + 2, sizeof(tot));

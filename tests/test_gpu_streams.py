@@ -141,3 +141,39 @@ def test_run_and_call_on_one_stream(B, oracle_mod):
     for out, _, rows in outs:
         assert B.verdicts_to_numpy(out).tobytes() == op.verify(lv, rows).tobytes()
     gp.close()
+
+
+def test_a_later_batch_of_other_handles_is_not_waited_for(B, oracle_mod):
+    """Verdicts of a program whose liveness batch has finished do not wait for a later batch of other programs that is held
+    back on its caller's stream."""
+    import torch
+    p = _program("short")
+    mine, theirs = [B.Program(p) for _ in range(3)], [B.Program(p) for _ in range(3)]
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    rows = _garbage_rows(p, 20, 6)
+    dev = _to_dev(rows)
+    out = torch.zeros((len(rows), 4), dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        B.vl_liveness_batch(mine, s1)
+        B.vl_liveness_batch(theirs, s2)
+        mine[2].vl_verify(dev, out, s1)
+        torch.cuda.synchronize()
+    out.zero_()
+    torch.cuda.synchronize()
+    B.vl_liveness_batch(mine, s1)
+    with torch.cuda.stream(s2):
+        torch.cuda._sleep(SLEEP_CYCLES)
+    B.vl_liveness_batch(theirs, s2)
+    mine[2].vl_verify(dev, out, s1)
+    s1.synchronize()
+    assert not s2.query(), "the call waited for a batch of other programs"
+    torch.cuda.synchronize()
+    op = oracle_mod.OracleProgram(p)
+    assert B.verdicts_to_numpy(out).tobytes() == op.verify(op.liveness(), rows).tobytes()
+    # the handles of a batch do not depend on the one whose event they share
+    B.vl_liveness_batch(mine, s1)
+    mine[0].close()
+    mine[1].vl_liveness(s2)
+    for gp in mine[1:] + theirs:
+        assert B.verdicts_to_numpy(gp.vl_verify(dev)).tobytes() == op.verify(op.liveness(), rows).tobytes()
+        gp.close()
