@@ -200,6 +200,7 @@ struct vl_program {
     VScratch fs[VL_LANES + 2];       // the same for what k_fused hands to k_exact: cstate, anom, work and racc only
     uint32_t sub_batch = 5120;       // candidates per pass of the verify kernels
     uint32_t lanes_opt = 3;          // lanes in use (1 = everything in order on the caller's stream)
+    uint64_t lane_call = 0, lane_base = 0;  // the last vl_verify* call that spread passes over lanes, the lane of its first
     cudaEvent_t ev_fork = nullptr, ev_join[VL_LANES] = {};
 
     // opt-in per-kernel timing of vl_verify: five events per pass (before each of the four kernels, after the last)

@@ -1895,7 +1895,8 @@ struct FusedGroup {
 // Passes of one or several programs spread round-robin over the device's lane streams, so that
 // the table kernel of one pass (bound by the row stream) runs beside the walk of another (bound by
 // instruction issue).  Pass j of a program uses working set j mod lanes and runs on lane
-// (first_lane + j) mod lanes: two passes that share a working set are ordered by their stream.
+// (first_lane + j) mod lanes: two passes that share a working set are ordered by their stream (also those of a program
+// that is given several times in one call: it keeps its first lane).
 int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K,
                     const uint64_t *pitch, vl_verdict *const *d_out, cudaStream_t st, bool dict)
 {
@@ -1922,6 +1923,8 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     }
     VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
     for (uint32_t l = 0; l < L; ++l) VL_CUDA(p0, cudaStreamWaitEvent(lane[l], p0->ev_fork, 0));
+    static std::atomic<uint64_t> calls{0};
+    const uint64_t call = ++calls;
     uint64_t job = 0;
     // short jobs of different programs share launches (64 programs of one call: 2 launches instead of 64)
     std::vector<uint8_t> shared(nprog, 0);
@@ -1945,7 +1948,8 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
         rc = plan_passes(p, K[j], &pp);
         if (rc != VL_OK) break;
         // a program's passes keep to "working set s on lane (base + s) mod L"
-        const uint64_t base = job;
+        if (p->lane_call != call) { p->lane_call = call; p->lane_base = job; }
+        const uint64_t base = p->lane_base;
         uint64_t s = 0;
         for (uint64_t kb = 0; kb < K[j] && rc == VL_OK; kb += pp.sub, ++s, ++job)
             rc = run_pass(p, pp, d_cand[j] + kb * pitch[j], std::min(pp.sub, K[j] - kb), pitch[j], d_out[j] + kb,

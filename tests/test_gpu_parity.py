@@ -428,3 +428,25 @@ def test_liveness_batch_with_a_program_that_fails(B, oracle_mod, n_before, n_beh
         _check_liveness_result(B, oracle_mod, gp, p)
         gp.close()
     bad.close()
+
+
+@pytest.mark.parametrize("K", [(700, 700, 700), (1500, 300, 2000, 20)])
+def test_batch_with_a_program_given_several_times(B, oracle_mod, K):
+    """The passes of one handle share its working sets whichever entry of the call they belong to."""
+    import torch
+    wl = synth.workload(2)
+    p = synth.build_program(wl.shapes[0], wl.seeds[0])
+    gp, lv = _check_liveness(B, oracle_mod, p)
+    gp.set_option(B.VL_OPT_SUB_BATCH, 512)
+    other = B.Program(p)
+    other.vl_liveness()
+    rows = [synth.candidate_rows(p, k, 0.4, 500 + j)[0] for j, k in enumerate(K)]
+    handles = [gp, other] + [gp] * (len(K) - 1)
+    rows.insert(1, rows[0])
+    for call in range(3):
+        outs = B.vl_verify_batch(handles, [_to_dev(r) for r in rows])
+        torch.cuda.synchronize()
+        for j, (o, r) in enumerate(zip(outs, rows)):
+            _assert_same(B.verdicts_to_numpy(o), _oracle_rows_threaded(oracle_mod, p, lv, r), f"call {call} entry {j}")
+    gp.close()
+    other.close()
