@@ -18,6 +18,8 @@
 #include "vl_internal.cuh"
 
 #define EXACT_NT 256
+#define EXACT_SMEM (224u * 1024)  // shared memory of a block of k_exact, at most
+#define EXACT_ROWS 2000           // rows that k_fused leaves counts of, at most: their items fit 16 bits
 
 namespace {
 
@@ -491,7 +493,7 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
 // BPM: thread blocks per multiprocessor that the registers have to leave room for.  One or two rows per multiprocessor are
 // bound by latency (registers for loads in flight), more rows by how many warps there are to switch between: 6,400 rows of
 // 64 programs 345 us with two blocks of 256 threads, 281 with three, 274 with four (but spills: one row 20 % slower).
-// HAND: candidates with a collision are listed for k_exact, which spreads their counts over all multiprocessors.
+// HAND: candidates with a collision are left to k_exact, which spreads their counts over all multiprocessors.
 template <int NTHR, int BPM, int N, bool HAND>
 __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMany<N> a)
 {
@@ -789,9 +791,10 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
                 uint32_t *cs = q.ex.cstate + k * 8;
                 cs[CS_FLAGS] = M->flags; cs[CS_FIRST] = first; cs[CS_BANK] = M->bank;
                 cs[CS_WALK] = M->any ? WALK_ANOM : 0u; cs[CS_THCOL] = M->thcol;
-                list_exact(q.ex.work, k, chunks);
+                cs[CS_ITEMS] = exact_parts(chunks, EXACT_PART_CHUNKS) | exact_parts(chunks, EXACT_FINE_CHUNKS) << 16;
             }
         } else if (lane == 0) {
+            if (HAND) q.ex.cstate[k * 8 + CS_ITEMS] = 0;
             const uint32_t flags = M->flags | (M->pairs ? (uint32_t)VL_INTERFERENCE : 0u);
             vl_verdict vd;
             vd.flags = flags ? flags : (uint32_t)VL_PASS;
@@ -807,7 +810,10 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
 // file, or the program has no fast bank tally), listed in work as items of one or several parts per candidate; a thread
 // block takes an item.  Consistency and Realizability are in cstate; a chunk of the walk that collided marks all of its
 // short chunks.  GLOBAL: the block's arrays lie in a slice of global memory (programs that do not fit a multiprocessor).
-template <bool GLOBAL>
+// ROWS: the candidates are the rows of k_fused, which left the number of items of each in cstate; every block adds them up
+// for itself (a list with its counts would have to be cleared in front of every call: 3.3 us of 26 for 200 rows of 8,000
+// instructions by a memset; reset by the last block, it is left as it is by a call whose second launch fails).
+template <bool GLOBAL, bool ROWS>
 __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ FParams q)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -820,12 +826,64 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
     uint2 *list = reinterpret_cast<uint2 *>(base + q.sm.list);
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     pdl_wait();
-    const bool fine = q.ex.work[1] <= q.ex.fine_items;
-    const uint32_t n_items = q.ex.work[fine ? 1 : 0];
-    const uint32_t *items = q.ex.work + EXACT_HDR + (fine ? 0 : 2 * EXACT_FINE_ITEMS);
+    uint32_t n_items;
+    const uint32_t *items = nullptr;
+    uint32_t *first = reinterpret_cast<uint32_t *>(base + q.sm.total);  // ROWS: [rows + 1] first item of every row
+    if (ROWS) {
+        __shared__ uint32_t s_sum[EXACT_NT / 32];
+        const uint32_t per = (q.ex.rows + EXACT_NT - 1) / EXACT_NT, k0 = tid * per, k1 = min(k0 + per, q.ex.rows);
+        uint32_t n = 0;  // of this thread's rows, coarse | fine << 16 (at most EXACT_ROWS rows: neither half overflows)
+        for (uint32_t k = k0; k < k1; ++k) {
+            const uint32_t x = q.ex.cstate[(size_t)k * 8 + CS_ITEMS];
+            first[k] = x;
+            n += x;
+        }
+        uint32_t inc = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= (uint32_t)d) inc += y;
+        }
+        if (lane == 31) s_sum[tid >> 5] = inc;
+        __syncthreads();
+        uint32_t before = inc - n, all = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < EXACT_NT / 32; ++w) {
+            if (w < tid >> 5) before += s_sum[w];
+            all += s_sum[w];
+        }
+        const uint32_t shift = all >> 16 <= q.ex.fine_items ? 16u : 0u;
+        n_items = (all >> shift) & 0xFFFFu;
+        uint32_t at = (before >> shift) & 0xFFFFu;
+        for (uint32_t k = k0; k < k1; ++k) {
+            const uint32_t x = (first[k] >> shift) & 0xFFFFu;
+            first[k] = at;
+            at += x;
+        }
+        if (tid == 0) first[q.ex.rows] = n_items;
+        __syncthreads();
+    } else {
+        const bool fine = q.ex.work[1] <= q.ex.fine_items;
+        n_items = q.ex.work[fine ? 1 : 0];
+        items = q.ex.work + EXACT_HDR + (fine ? 0 : 2 * EXACT_FINE_ITEMS);
+    }
     for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const uint64_t k = items[2 * it];
-        const uint32_t part = items[2 * it + 1] & 0xFFu, parts = items[2 * it + 1] >> 8;
+        uint64_t k;
+        uint32_t part, parts;
+        if (ROWS) {
+            uint32_t lo = 0, hi = q.ex.rows;  // first[lo] <= it < first[hi]
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (first[mid] <= it) lo = mid; else hi = mid;
+            }
+            k = lo;
+            part = it - first[lo];
+            parts = first[lo + 1] - first[lo];
+        } else {
+            k = items[2 * it];
+            part = items[2 * it + 1] & 0xFFu;
+            parts = items[2 * it + 1] >> 8;
+        }
         const uint16_t *row = q.cand + k * q.pitch;
         const uint32_t *cs = q.ex.cstate + k * 8;
         const uint32_t walk = cs[CS_WALK], thcol = cs[CS_THCOL];
@@ -848,8 +906,8 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
         __syncthreads();
         if (count) exact_counts<EXACT_NT, true>(q, T, W, occ, coll, list, M, part, parts, row);
         __syncthreads();
-        if (q.bank_fast || q.ex.after_fused) {
-            if (tid == 0) M->bank = (part == 0 ? cs[CS_BANK] : 0u) - (q.ex.after_fused ? 0u : M->dups);
+        if (ROWS || q.bank_fast) {
+            if (tid == 0) M->bank = (part == 0 ? cs[CS_BANK] : 0u) - (ROWS ? 0u : M->dups);
         } else {  // the general tally: the whole table, this part's instructions
             for (uint32_t v = tid; v < q.V; v += EXACT_NT) {
                 const uint32_t pos = q.first_occ[v];
@@ -890,9 +948,6 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
             }
         }
     }
-    // the next call lists from the start: the block that is last to be done sees to it (every block has read the counts)
-    __syncthreads();
-    if (q.ex.after_fused && tid == 0 && atomicAdd(q.ex.work + 2, 1u) == gridDim.x - 1) q.ex.work[0] = q.ex.work[1] = q.ex.work[2] = 0;
 }
 
 // How a job of K rows runs: threads per block (0: the program does not fit the kernel), blocks per multiprocessor.  Up to
@@ -961,26 +1016,21 @@ bool vl_fused_wanted(vl_program *p, uint64_t K)
 // What k_fused and k_exact share.
 static int hand_scratch(vl_program *p, int slot, uint64_t rows, VlExactArgs *ex)
 {
+    ex->rows = (uint32_t)rows;
     vl_program::VScratch &v = p->fs[slot];
     const uint64_t aw = (p->nC + 31) / 32;
     if (v.rows < rows || v.aw != aw) {
         VL_CUDA(p, cudaFree(v.block));
         v = vl_program::VScratch{};
         rows = std::max<uint64_t>(rows, 3ull * vl_sm_count(p));
-        const uint64_t words[4] = {EXACT_HDR + 2 * (EXACT_FINE_ITEMS + EXACT_MAX_PARTS * rows), rows * 8, rows * 4, rows * aw};
-        VL_CUDA(p, cudaMalloc(&v.block, (words[0] + words[1] + words[2] + words[3]) * 4));
-        uint32_t *w = static_cast<uint32_t *>(v.block);
-        VL_CUDA(p, cudaMemset(w, 0, EXACT_HDR * 4));
-        VL_CUDA(p, cudaStreamSynchronize(cudaStreamLegacy));  // (the kernels run on streams that do not wait for it)
-        v.work = w; v.cstate = w + words[0]; v.racc = v.cstate + words[1]; v.anom = v.racc + words[2];
+        VL_CUDA(p, cudaMalloc(&v.block, rows * (8 + 4 + aw) * 4));
+        v.cstate = static_cast<uint32_t *>(v.block); v.racc = v.cstate + rows * 8; v.anom = v.racc + rows * 4;
         v.rows = rows; v.aw = aw;
     }
-    ex->work = v.work; ex->cstate = v.cstate; ex->racc = v.racc; ex->anom = v.anom;
+    ex->cstate = v.cstate; ex->racc = v.racc; ex->anom = v.anom;
     ex->AW = (uint32_t)aw; ex->nC = p->nC;
     ex->short_chunk = p->d_short_chunk; ex->chunk_short_off = p->d_chunk_short_off;
     ex->fine_items = std::min<uint32_t>(vl_exact_blocks(p), EXACT_FINE_ITEMS);
-    ex->after_fused = 1;
-    ex->scratch = nullptr;
     return VL_OK;
 }
 
@@ -1026,7 +1076,7 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         FMany<1> one;
         one.p[0] = many.p[0];
         const dim3 grid((uint32_t)rows);
-        if (slot >= 0 && pl.bpm > 1 && p0->nI >= FUSED_HAND_INSTRS && !vl_exact_scratch(p0)) {
+        if (slot >= 0 && pl.bpm > 1 && p0->nI >= FUSED_HAND_INSTRS && vl_exact_takes_rows(p0, rows)) {
             VlExactArgs &ex = one.p[0].ex;
             const int rc = hand_scratch(p0, slot, rows, &ex);
             if (rc != VL_OK) return rc;
@@ -1071,7 +1121,12 @@ uint32_t vl_exact_blocks(vl_program *p)
 uint64_t vl_exact_scratch(vl_program *p)
 {
     const uint64_t bytes = exact_smem(p).total;
-    return bytes <= 224 * 1024 ? 0 : bytes * vl_exact_blocks(p);
+    return bytes <= EXACT_SMEM ? 0 : bytes * vl_exact_blocks(p);
+}
+
+bool vl_exact_takes_rows(vl_program *p, uint64_t rows)
+{
+    return rows <= EXACT_ROWS && exact_smem(p).total + (rows + 1) * 4 <= EXACT_SMEM;
 }
 
 int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st,
@@ -1082,7 +1137,8 @@ int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, u
     if (p->device >= 0 && p->device < 64) {
         std::lock_guard<std::mutex> lock(mtx);
         if (!done[p->device]) {
-            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024));
+            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, EXACT_SMEM));
+            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, EXACT_SMEM));
             done[p->device] = true;
         }
     }
@@ -1092,7 +1148,8 @@ int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, u
     q.ex = ex;
     q.cand = d_cand; q.pitch = pitch; q.out = d_out;
     const uint32_t grid = vl_exact_blocks(p);
-    if (ex.scratch) VL_CUDA(p, launch_overlap(k_exact<true>, grid, EXACT_NT, 0, st, overlap, q));
-    else VL_CUDA(p, launch_overlap(k_exact<false>, grid, EXACT_NT, q.sm.total, st, overlap, q));
+    if (ex.rows) VL_CUDA(p, launch_overlap(k_exact<false, true>, grid, EXACT_NT, q.sm.total + (ex.rows + 1) * 4, st, overlap, q));
+    else if (ex.scratch) VL_CUDA(p, launch_overlap(k_exact<true, false>, grid, EXACT_NT, 0, st, overlap, q));
+    else VL_CUDA(p, launch_overlap(k_exact<false, false>, grid, EXACT_NT, q.sm.total, st, overlap, q));
     return VL_OK;
 }

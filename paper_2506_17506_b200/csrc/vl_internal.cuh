@@ -197,7 +197,7 @@ struct vl_program {
         uint32_t *thm = nullptr;       // [groups][n_blocks][mask words][2][32] through-set masks
         uint64_t rows = 0, aw = 0, vregs = 0, chunks = 0;
     } vs[VL_LANES + 2];              // one per lane, then one per staging buffer of vl_verify_host
-    VScratch fs[VL_LANES + 2];       // the same for what k_fused hands to k_exact: cstate, anom, work and racc only
+    VScratch fs[VL_LANES + 2];       // the same for what k_fused hands to k_exact: cstate, anom and racc only
     uint32_t sub_batch = 5120;       // candidates per pass of the verify kernels
     uint32_t lanes_opt = 3;          // lanes in use (1 = everything in order on the caller's stream)
     uint64_t lane_call = 0, lane_base = 0;  // the last vl_verify* call that spread passes over lanes, the lane of its first
@@ -267,19 +267,20 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
 // fine ones are taken if each has a thread block of its own: 1,000 rows of 8,000 instructions of which 100 fail 77 us
 // against 81 for the whole call, 777 of 11,317 with 39 failing 103.5 against 109.  Beyond that what an item costs before
 // its first count weighs more: 350 of the 1,000 failing 95 us in fine items, 85.5 in coarse ones.
-#define EXACT_HDR 4         // words in front of the fine items, then the coarse ones: numbers of coarse and of fine items, blocks done
+#define EXACT_HDR 4         // words in front of the fine items, then the coarse ones: numbers of coarse and of fine items
 #define EXACT_MAX_PARTS 32  // items of one candidate, at most
 #define EXACT_PART_CHUNKS 6
 #define EXACT_FINE_CHUNKS 2
 #define EXACT_FINE_ITEMS 512
-// per-candidate state between the kernels (8 words)
-enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_WALK = 6, CS_THCOL = 7 };
+// per-candidate state between the kernels (8 words); CS_ITEMS: what k_fused leaves for k_exact, coarse | fine items << 16
+enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_ITEMS = 3, CS_WALK = 6, CS_THCOL = 7 };
 enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
-// Lists candidate k, with that many chunks to count.
+// Items of a candidate with that many chunks to count.
+__device__ __forceinline__ uint32_t exact_parts(uint32_t chunks, uint32_t per_item) { return min(1u + chunks / per_item, (uint32_t)EXACT_MAX_PARTS); }
+// Lists candidate k.
 __device__ __forceinline__ void list_exact(uint32_t *work, uint64_t k, uint32_t chunks)
 {
-    const uint32_t parts = min(1u + chunks / EXACT_PART_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
-    const uint32_t fine = min(1u + chunks / EXACT_FINE_CHUNKS, (uint32_t)EXACT_MAX_PARTS);
+    const uint32_t parts = exact_parts(chunks, EXACT_PART_CHUNKS), fine = exact_parts(chunks, EXACT_FINE_CHUNKS);
     const uint32_t at = EXACT_FINE_ITEMS + atomicAdd(work, parts), fine_at = atomicAdd(work + 1, fine);
     for (uint32_t j = 0; j < parts; ++j) {
         work[EXACT_HDR + 2 * (at + j)] = (uint32_t)k;
@@ -295,11 +296,12 @@ struct VlExactArgs {
     const uint32_t *short_chunk, *chunk_short_off;  // [nS] chunk of every short chunk, [nC + 1] first short chunk of every chunk
     uint32_t *racc;               // [rows][4] overlaps, complement of the lowest instruction, bank tally, parts done; all 0
     uint32_t AW, nC, fine_items;      // fine_items: up to that many fine items are taken
-    uint32_t after_fused;         // the candidates come from k_fused: their bank tally is exact, and the counts are reset at the end
+    uint32_t rows;                // k_fused's rows, each of which left the number of its items (and an exact bank tally) in cstate; 0: listed in work
     unsigned char *scratch;       // vl_exact_scratch bytes, null if 0
 };
 uint32_t vl_exact_blocks(vl_program *p);  // thread blocks of k_exact: one item each at a time
 uint64_t vl_exact_scratch(vl_program *p);
+bool vl_exact_takes_rows(vl_program *p, uint64_t rows);  // whether k_exact can count for that many rows of k_fused
 int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st,
                  bool dict, bool overlap);
 int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out,

@@ -5,7 +5,7 @@ import pytest
 
 from paper_2506_17506_b200 import synth
 from tests import helpers as H
-from tests.test_gpu_parity import _assert_same, _garbage_rows, _gpu_verify
+from tests.test_gpu_parity import _assert_same, _garbage_rows, _gpu_verify, _to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -104,4 +104,58 @@ def test_counts_handed_over(B, oracle_mod, P, n_banks, K):
         rows = np.stack([H.row_from_table(p, np.where(rng.random(V) < [0, 0, 3e-4, 0.05, 1][k % 5], rng.integers(0, P, V), good))
                          for k in range(K)])
         _assert_same(_gpu_verify(B, gp, rows), op.verify(lv, rows), f"P {P} call {call}")
+    gp.close()
+
+
+def test_counts_handed_over_after_a_call_that_was_cut_short(B, oracle_mod):
+    """A call whose rows were listed for the exact counts, which then never ran (as if their launch had failed: a captured
+    call with that kernel switched off), leaves nothing behind for the next one."""
+    import torch
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    P, V, K = 250, 7200, 300
+    blocks = [[([i], [i - 1, i - 2, i - 17] if i >= 17 else []) for i in range(b * 1800, (b + 1) * 1800)] for b in range(4)]
+    p = synth.program_from_lists(blocks, [(0, 1), (1, 1), (1, 2), (2, 3)], V, [1 + (v % 5 == 0) for v in range(V)], P)
+    gp = B.Program(p)
+    B.vl_liveness_batch([gp])
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    rng = np.random.default_rng(9)
+    good = (np.arange(V) * 2) % P
+    def rows_of(share):
+        return np.stack([H.row_from_table(p, np.where(rng.random(V) < share[k % len(share)], rng.integers(0, P, V), good)) for k in range(K)])
+    rows = rows_of([0, 3e-4, 0.05, 1])
+    _assert_same(_gpu_verify(B, gp, rows), op.verify(lv, rows), "before")
+    dev, s = _to_dev(rows), torch.cuda.Stream()
+    out = torch.full((K, 4), -9, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+
+    def ok(r):
+        assert int(r[0]) == 0, r
+        return r[1] if len(r) == 2 else r[1:]
+
+    ok(rt.cudaStreamBeginCapture(s.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed))
+    gp.vl_verify(dev, out, s)
+    graph = ok(rt.cudaStreamEndCapture(s.cuda_stream))
+    nodes, n = ok(rt.cudaGraphGetNodes(graph, 16))
+    nodes = nodes[:n]
+    kernels = [n for n in nodes if ok(rt.cudaGraphNodeGetType(n)) == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel]
+    assert len(kernels) == 2
+    whole = ok(rt.cudaGraphInstantiate(graph, 0))
+    cut = ok(rt.cudaGraphInstantiate(graph, 0))
+    ok(rt.cudaGraphNodeSetEnabled(cut, kernels[1], 0))
+    ok(rt.cudaGraphLaunch(cut, s.cuda_stream))
+    s.synchronize()
+    got, want = B.verdicts_to_numpy(out), op.verify(lv, rows)
+    unfinished = got["conflict_pairs"] == np.uint32(2**32 - 9)
+    assert (want["conflict_pairs"][unfinished] > 0).any()     # rows that collided were not counted
+    rows2 = rows_of([1, 0.05, 0, 3e-4])
+    _assert_same(_gpu_verify(B, gp, rows2), op.verify(lv, rows2), "after")
+    ok(rt.cudaGraphLaunch(cut, s.cuda_stream))
+    for _ in range(2):                                        # and a captured call can be replayed
+        ok(rt.cudaGraphLaunch(whole, s.cuda_stream))
+        s.synchronize()
+        _assert_same(B.verdicts_to_numpy(out), want, "replay")
+    for g in (whole, cut):
+        rt.cudaGraphExecDestroy(g)
+    rt.cudaGraphDestroy(graph)
     gp.close()
