@@ -998,7 +998,7 @@ FParams fused_params(const vl_program *p, bool dict)
 bool vl_fused_wanted(vl_program *p, uint64_t K)
 {
     if (p->group_opt || p->threads_opt || p->test_wait) return false;  // the caller asks for the batched kernels
-    if (p->P + p->wmax > 32768u) return false;                         // (not a program the verify path takes)
+    if (!vl_verify_takes(p)) return false;                             // (refused, however few the rows)
     const FPlan pl = fused_plan(p, K);
     if (!pl.threads) return false;
     const uint64_t resident = (uint64_t)pl.bpm * vl_sm_count(p);

@@ -259,6 +259,7 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
 // launch with other programs' jobs, and one launch for n <= VL_FUSED_MANY jobs.
 #define VL_FUSED_MANY 48
 bool vl_fused_wanted(vl_program *p, uint64_t K);
+bool vl_verify_takes(const vl_program *p);  // whether the verify path takes the program (vl_verify.cu)
 bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
                  vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot);  // slot: working set, -1: none

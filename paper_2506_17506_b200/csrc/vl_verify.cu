@@ -29,6 +29,8 @@
 #define MAX_STAGES 4
 #define TGW 64  // candidates side by side per vreg in the tables handed from the table kernel to the walk
 #define WALK_WARPS 8
+#define WALK_EV_CAP 256  // events that a warp of the walk stages at a time
+#define SM_BYTES (227u * 1024)  // shared memory of a multiprocessor, for one block
 
 struct TParams {
     uint32_t nI, V, nO, nOp8, P, Bmask, ntiles;
@@ -1512,6 +1514,18 @@ Plan make_plan(const vl_program *p, uint32_t G, uint32_t NT, uint32_t budget)
     return pl;
 }
 
+}  // namespace
+
+// Whether the verify path takes a program at all (whatever the number of rows): the table of one candidate, with its bank
+// nibbles and a copy ring of two stages, and the occupancy masks of one warp of the walk fit a multiprocessor; and every
+// register number in the file is below 2^15 (the walk's table entries keep bit 15 for a mark).
+bool vl_verify_takes(const vl_program *p)
+{
+    const uint64_t walk = ((p->P + p->wmax + 31) / 32 * 64ull + (WALK_EV_CAP / 8 + 2) * 28) * 4;
+    return p->P + p->wmax <= 32768u && walk <= SM_BYTES - 1024 && make_plan(p, 1, 256, SM_BYTES).ok;
+}
+
+namespace {
 // Shared memory of one k_tables8 block: [T, 16 bytes per vreg][copy ring][tail buffer][misc]; the
 // bank nibbles (4 bytes per vreg) reuse the copy ring.
 Plan make_plan8(const vl_program *p, uint32_t NT, uint32_t budget)
@@ -1667,7 +1681,7 @@ struct PassPlan {
 // Launch geometry of a program's passes and the shared-memory opt-ins of its kernels.
 int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
 {
-    const uint32_t SM_BYTES = 227 * 1024;
+    if (!vl_verify_takes(p)) return VL_ERR_UNSUPPORTED;
     // Preference: eight candidates per block (two blocks of 256 threads per SM if the tables are small, else one block of
     // 512 threads), then as many candidates per block as fit an SM, with 512 threads if the copy ring leaves room for
     // theirs: a lookup serves every candidate of the block.  1,000 rows of 20,000 vregs: four candidates and 512 threads
@@ -1692,16 +1706,12 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
     if (!pl.ok) return VL_ERR_UNSUPPORTED;
     pp->pl = pl;
     pp->Wp = (p->P + p->wmax + 31) / 32;
-    pp->ev_cap = 256;
+    pp->ev_cap = WALK_EV_CAP;
     // the walk's warps each keep the occupancy masks of 64 candidates: fewer warps for large register files
     for (pp->walk_warps = WALK_WARPS;; pp->walk_warps >>= 1) {
         pp->walk_smem = pp->walk_warps * (pp->Wp * 64 + ((pp->ev_cap >> 3) + 2) * 28) * 4;
         if (pp->walk_smem <= SM_BYTES - 1024) break;
-        if (pp->walk_warps == 1) return VL_ERR_UNSUPPORTED;
     }
-    // the walk's table entries keep bit 15 for a mark: every in-file register number must be below 2^15
-    // (the occupancy masks of a register file that large would not fit shared memory anyway)
-    if (p->P + p->wmax > 32768u) return VL_ERR_UNSUPPORTED;
     pp->sub = std::min<uint64_t>(K, p->sub_batch);
     // passes of equal size (whole groups of the tables) rather than full ones and a short last one
     if (K > pp->sub) {

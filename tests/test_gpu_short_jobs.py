@@ -159,3 +159,31 @@ def test_counts_handed_over_after_a_call_that_was_cut_short(B, oracle_mod):
         rt.cudaGraphExecDestroy(g)
     rt.cudaGraphDestroy(graph)
     gp.close()
+
+
+@pytest.mark.parametrize("V,takes", [(57000, True), (60000, False)])
+def test_a_refused_program_is_refused_for_every_number_of_rows(B, oracle_mod, V, takes):
+    """The table of one candidate with its bank nibbles does not fit a multiprocessor, whatever the short jobs' kernel needs."""
+    import torch
+    blocks = [[([i], [i - 1] if i else []) for i in range(V)]]
+    p = synth.program_from_lists(blocks, [], V, [1] * V, 64)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    rows = np.stack([H.row_from_table(p, (np.arange(V) * (k + 1)) % 64) for k in range(3)])
+    dev = _to_dev(rows)
+    n, off, vreg = 600, *gp.vl_dict_layout()
+    many = torch.zeros((n, gp.pitch), dtype=torch.int16, device="cuda").view(torch.uint16)
+    calls = [lambda: gp.vl_verify(dev), lambda: gp.vl_verify_dict(torch.zeros((1, (len(vreg) + 7) // 8 * 8), dtype=torch.int16, device="cuda").view(torch.uint16)),
+             lambda: gp.vl_verify_host(rows), lambda: gp.vl_verify_until_pass(dev, 1), lambda: B.vl_verify_batch([gp, gp], [dev, dev]),
+             lambda: gp.vl_verify(many)]
+    for j, call in enumerate(calls):
+        if takes:
+            call()
+            continue
+        with pytest.raises(B.VlError) as e:
+            call()
+        assert e.value.code == B.VL_ERR_UNSUPPORTED, j
+    if takes:
+        op = oracle_mod.OracleProgram(p)
+        _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows))
+    gp.close()
