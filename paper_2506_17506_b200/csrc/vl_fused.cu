@@ -204,7 +204,8 @@ __device__ __noinline__ uint32_t member_duplicates(const FParams &q, const uint1
 // together in front of it: if they hold the same register, its chunk has collided, or they are both in a through-set that
 // has.  And T, W hold nothing yet: what the share needs is fetched here (a hundredth of the vregs, for a row with one
 // misplaced vreg; fetching all 10,000 took 30 us).
-template <int NTHR, bool LISTED>
+// LONG: the program's lists are long (EXACT_LONG entries and more on average).
+template <int NTHR, bool LISTED, bool LONG = false>
 __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint8_t *W, uint32_t *cv, const uint32_t *coll,
                                              uint2 *list, FMisc *M, uint32_t part, uint32_t parts, const uint16_t *row)
 {
@@ -346,7 +347,70 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
             for (int u = 0; u < LQ; ++u) us_nx[u] = ls4[min(p0 + u, p1)];
         };
         const uint32_t n_slots = n_list * q.short_len;
-        if (n_slots) {
+        if constexpr (LONG) {
+            // A warp takes an instruction, its lanes the entries.  (A thread per instruction reads 32 lists at a time, 16 bytes
+            // of each.)
+            constexpr uint32_t NW = NTHR / 32, LU = 4;
+            const uint4 *ls4 = reinterpret_cast<const uint4 *>(q.ls);
+            uint32_t unit = (tid >> 5) / q.short_len, at = (tid >> 5) % q.short_len;
+            auto next = [&](uint32_t &b) -> uint32_t {
+                uint32_t i = 0xFFFFFFFFu;
+                if (unit < n_list) {
+                    const uint2 span = list[unit];
+                    if (at < (span.y & 0xFFFFFu)) i = span.x + at;
+                    b = b0 + (span.y >> 20);
+                }
+                at += NW;
+                while (at >= q.short_len) { at -= q.short_len; ++unit; }
+                return i;
+            };
+            uint32_t b_nx = b0, i_nx = next(b_nx);
+            uint4 rec_nx = q.irec[min(i_nx, q.nI - 1)];
+            for (uint32_t f = tid >> 5; f < n_slots; f += NW) {
+                const uint32_t i = i_nx, b = b_nx;
+                const uint4 rec = rec_nx;
+                i_nx = next(b_nx);
+                rec_nx = q.irec[min(i_nx, q.nI - 1)];
+                if (i == 0xFFFFFFFFu) continue;
+                const uint32_t n = rec.y & 0xFFFFu, nd = (rec.y >> 16) & 0xFFu, p0 = rec.x >> 2, p1 = n ? (rec.x + n - 1) >> 2 : p0;
+                uint32_t n_dup = 0;
+                for (uint32_t a = rec.w + nd + lane; a < q.op_off[i + 1]; a += 32) n_dup += duplicate_of(q, T, rec.w + nd, a);
+                n_dup = __reduce_add_sync(0xffffffffu, n_dup);
+                if (lane == 0 && n_dup) dups += n_dup - ((thcol >> b) & 1u ? member_duplicates(q, T, b, i) : 0u);
+                for (uint32_t d = 0; d < nd; ++d) {
+                    const uint32_t v = d ? q.op_vreg[rec.w + d] : rec.z, sv = T[v], wv = W[v];
+                    const uint32_t shift = q.wmax - 1 - sv, span = wv + q.wmax - 1;  // (as below)
+                    uint32_t cnt = lane ? 0u : through_overlaps(b, v, d ? (q.blk_th[(size_t)b * q.Wv + (v >> 5)] >> (v & 31)) & 1u : rec.y >> 31);
+                    for (uint32_t p = p0 + lane; n && p <= p1; p += 32 * LU) {
+                        uint4 x4[LU];
+#pragma unroll
+                        for (uint32_t u = 0; u < LU; ++u) x4[u] = ls4[min(p + u * 32, p1)];
+                        uint32_t x[4 * LU], t[4 * LU];
+#pragma unroll
+                        for (uint32_t u = 0; u < LU; ++u) { x[4 * u] = x4[u].x; x[4 * u + 1] = x4[u].y; x[4 * u + 2] = x4[u].z; x[4 * u + 3] = x4[u].w; }
+                        bool near = false;
+#pragma unroll
+                        for (uint32_t u = 0; u < 4 * LU; ++u) {
+                            const bool entry = (p + (u >> 2) * 32) * 4 + (u & 3) - rec.x < n;
+                            t[u] = T[entry ? x[u] : q.V];
+                            if (!entry) t[u] = 0x1000000u;  // (near nothing)
+                            near |= t[u] + shift < span;
+                        }
+                        if (near) {
+#pragma unroll
+                            for (uint32_t u = 0; u < 4 * LU; ++u)
+                                if (t[u] + shift < span && x[u] != v && t[u] + W[x[u]] > sv) ++cnt;
+                        }
+                    }
+                    for (uint32_t d2 = lane; nd > 1 && d2 < nd; d2 += 32) {  // co-defined vregs that are not live afterwards
+                        if (d2 == d || !(q.opflags[rec.w + d2] & OPF_DEAD)) continue;
+                        const uint32_t x = q.op_vreg[rec.w + d2];
+                        if (overlap(sv, wv, T[x], W[x])) ++cnt;
+                    }
+                    if (cnt) { pairs += cnt; mind = min(mind, i); }
+                }
+            }
+        } else if (n_slots) {
             uint32_t b_nx = b0, b_nx2 = b0, i_nx = next_instr(b_nx), i_nx2 = next_instr(b_nx2);
             uint4 rec_nx = fetch_rec(i_nx), rec_nx2 = fetch_rec(i_nx2);
             fetch_list(rec_nx);
@@ -813,7 +877,7 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
 // ROWS: the candidates are the rows of k_fused, which left the number of items of each in cstate; every block adds them up
 // for itself (a list with its counts would have to be cleared in front of every call: 3.3 us of 26 for 200 rows of 8,000
 // instructions by a memset; reset by the last block, it is left as it is by a call whose second launch fails).
-template <bool GLOBAL, bool ROWS>
+template <bool GLOBAL, bool ROWS, bool LONG>
 __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ FParams q)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -904,7 +968,7 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
                 if (lane == 0) coll[s >> 5] = bits;
             }
         __syncthreads();
-        if (count) exact_counts<EXACT_NT, true>(q, T, W, occ, coll, list, M, part, parts, row);
+        if (count) exact_counts<EXACT_NT, true, LONG>(q, T, W, occ, coll, list, M, part, parts, row);
         __syncthreads();
         if (ROWS || q.bank_fast) {
             if (tid == 0) M->bank = (part == 0 ? cs[CS_BANK] : 0u) - (ROWS ? 0u : M->dups);
@@ -995,10 +1059,22 @@ FParams fused_params(const vl_program *p, bool dict)
 // that the batched kernels, which read the program's tables for 8 or 64 rows at a time, win as soon as the rounds of
 // this kernel (about 3 us and 3.5 ns per instruction) take longer than their launches: 600 rows of 2,000 instructions 31
 // against 42 us, 1,000 rows 41 against 42; 3,000 rows of 64 instructions 40 against 68, 10,000 rows 124 against 79.
+// A program whose short chunks begin with many vregs occupied is something else: a row enters them all by itself and counts
+// its collisions in lists as long, which the batched kernels spread over the multiprocessors.  3,500 instructions with 500
+// vregs live everywhere, rows that collide everywhere: 1 row 101 us against 410, 100 rows 320 against 416, 148 rows 424
+// against 418, 300 rows 690 against 1,211; 24,300 instructions with 300 such vregs: 1 row 0.56 ms against 13, 127 rows 29.8
+// against 13, 148 rows 34.7 against 13.  (The line, 32,768 entries: 860 instructions with 200 vregs, 22,000 entries, take 60
+// us here and 65 there, 1,620 with 300, 60,000 entries, 115 and 74.  Programs whose values live shortly have below 10,000.)
+#define FUSED_FEW_ROWS 128u
+// 100 rows that collide everywhere, a warp per instruction against a thread: lists of 2,330 entries on average 5,916 us against
+// 8,602, of 1,013 1,441 against 1,261, of 557 640 against 454.
+static bool long_lists(const vl_program *p) { return p->known[VL_KNOWN_LS] >= (uint64_t)EXACT_LONG * p->nI; }
+
 bool vl_fused_wanted(vl_program *p, uint64_t K)
 {
     if (p->group_opt || p->threads_opt || p->test_wait) return false;  // the caller asks for the batched kernels
     if (!vl_verify_takes(p)) return false;                             // (refused, however few the rows)
+    if (p->known[VL_KNOWN_SEN] >= FUSED_MANY_ENTRIES && (K < FUSED_FEW_ROWS || K > (uint64_t)vl_sm_count(p) || long_lists(p))) return false;
     const FPlan pl = fused_plan(p, K);
     if (!pl.threads) return false;
     const uint64_t resident = (uint64_t)pl.bpm * vl_sm_count(p);
@@ -1137,8 +1213,9 @@ int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, u
     if (p->device >= 0 && p->device < 64) {
         std::lock_guard<std::mutex> lock(mtx);
         if (!done[p->device]) {
-            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, EXACT_SMEM));
-            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, EXACT_SMEM));
+            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, EXACT_SMEM));
+            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, EXACT_SMEM));
+            VL_CUDA(p, cudaFuncSetAttribute(k_exact<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, EXACT_SMEM));
             done[p->device] = true;
         }
     }
@@ -1148,8 +1225,9 @@ int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, u
     q.ex = ex;
     q.cand = d_cand; q.pitch = pitch; q.out = d_out;
     const uint32_t grid = vl_exact_blocks(p);
-    if (ex.rows) VL_CUDA(p, launch_overlap(k_exact<false, true>, grid, EXACT_NT, q.sm.total + (ex.rows + 1) * 4, st, overlap, q));
-    else if (ex.scratch) VL_CUDA(p, launch_overlap(k_exact<true, false>, grid, EXACT_NT, 0, st, overlap, q));
-    else VL_CUDA(p, launch_overlap(k_exact<false, false>, grid, EXACT_NT, q.sm.total, st, overlap, q));
+    if (ex.rows) VL_CUDA(p, launch_overlap(k_exact<false, true, false>, grid, EXACT_NT, q.sm.total + (ex.rows + 1) * 4, st, overlap, q));
+    else if (ex.scratch) VL_CUDA(p, launch_overlap(k_exact<true, false, false>, grid, EXACT_NT, 0, st, overlap, q));
+    else if (long_lists(p)) VL_CUDA(p, launch_overlap(k_exact<false, false, true>, grid, EXACT_NT, q.sm.total, st, overlap, q));
+    else VL_CUDA(p, launch_overlap(k_exact<false, false, false>, grid, EXACT_NT, q.sm.total, st, overlap, q));
     return VL_OK;
 }

@@ -33,6 +33,8 @@ enum : uint32_t {
 };
 
 #define VL_MAX_GROUP 8
+#define VL_KNOWN_LS 3   // vl_program::known: short-list entries
+#define VL_KNOWN_SEN 5  // and entries of the short chunks
 #define VL_LANES 8  // internal streams that the passes of device-resident verify calls can be spread over
 #define VL_LIVE_STREAM VL_LANES      // index of the internal stream a single vl_liveness call runs on
 #define VL_STREAMS (VL_LANES + 1)    // the lanes, the liveness stream
@@ -259,6 +261,9 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
 // launch with other programs' jobs, and one launch for n <= VL_FUSED_MANY jobs.
 #define VL_FUSED_MANY 48
 bool vl_fused_wanted(vl_program *p, uint64_t K);
+// Entries of the short chunks (vreg and short chunk at whose beginning it is occupied) from which a program counts as one
+// that occupies many.
+#define FUSED_MANY_ENTRIES 32768u  // (measured at vl_fused_wanted)
 bool vl_verify_takes(const vl_program *p);  // whether the verify path takes the program (vl_verify.cu)
 bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
@@ -270,18 +275,24 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
 // its first count weighs more: 350 of the 1,000 failing 95 us in fine items, 85.5 in coarse ones.
 #define EXACT_HDR 4         // words in front of the fine items, then the coarse ones: numbers of coarse and of fine items
 #define EXACT_MAX_PARTS 32  // items of one candidate, at most
+#define EXACT_MANY_PARTS 128  // the same of fine items, for programs that occupy many vregs (FUSED_MANY_ENTRIES): one row of 24,300
+                              // instructions with 300 vregs live everywhere 0.56 ms, 1.23 with 32 items
 #define EXACT_PART_CHUNKS 6
 #define EXACT_FINE_CHUNKS 2
 #define EXACT_FINE_ITEMS 512
+#define EXACT_LONG 1024      // entries of an instruction's short list, on average, from which a warp counts them together
 // per-candidate state between the kernels (8 words); CS_ITEMS: what k_fused leaves for k_exact, coarse | fine items << 16
 enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_ITEMS = 3, CS_WALK = 6, CS_THCOL = 7 };
 enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
 // Items of a candidate with that many chunks to count.
-__device__ __forceinline__ uint32_t exact_parts(uint32_t chunks, uint32_t per_item) { return min(1u + chunks / per_item, (uint32_t)EXACT_MAX_PARTS); }
-// Lists candidate k.
-__device__ __forceinline__ void list_exact(uint32_t *work, uint64_t k, uint32_t chunks)
+__device__ __forceinline__ uint32_t exact_parts(uint32_t chunks, uint32_t per_item, uint32_t most = EXACT_MAX_PARTS)
 {
-    const uint32_t parts = exact_parts(chunks, EXACT_PART_CHUNKS), fine = exact_parts(chunks, EXACT_FINE_CHUNKS);
+    return min(1u + chunks / per_item, most);
+}
+// Lists candidate k; fine_most: fine items of one candidate, at most.
+__device__ __forceinline__ void list_exact(uint32_t *work, uint64_t k, uint32_t chunks, uint32_t fine_most)
+{
+    const uint32_t parts = exact_parts(chunks, EXACT_PART_CHUNKS), fine = exact_parts(chunks, EXACT_FINE_CHUNKS, fine_most);
     const uint32_t at = EXACT_FINE_ITEMS + atomicAdd(work, parts), fine_at = atomicAdd(work + 1, fine);
     for (uint32_t j = 0; j < parts; ++j) {
         work[EXACT_HDR + 2 * (at + j)] = (uint32_t)k;

@@ -69,7 +69,7 @@ struct LiveMany {
 static_assert(sizeof(LiveMany<LV_MANY>) <= 32764, "kernel arguments");
 #define LIVE_ARGS const LiveArgs &q = a.p[N == 1 ? 0 : blockIdx.y]
 
-enum { LV_TOT_LO = 0, LV_TOT_EV = 1, LV_TOT_TH = 2, LV_TOT_LS = 3, LV_TOT_SEV = 4, LV_TOT_SEN = 5, LV_TOTALS = 6 };
+enum { LV_TOT_LO = 0, LV_TOT_EV = 1, LV_TOT_TH = 2, LV_TOT_LS = VL_KNOWN_LS, LV_TOT_SEV = 4, LV_TOT_SEN = VL_KNOWN_SEN, LV_TOTALS = 6 };
 
 // ------------------------------------------------------------------ device helpers
 __device__ __forceinline__ bool bit_get(const uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; }

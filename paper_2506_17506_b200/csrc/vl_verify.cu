@@ -86,7 +86,7 @@ struct TMisc {
 };
 
 struct WParams {
-    uint32_t V, P, nB, nC, Wp, AW, use_th, wmax, early;
+    uint32_t V, P, nB, nC, Wp, AW, use_th, wmax, early, fine_most;
     uint64_t K;
     const uint32_t *th_off, *th, *cev_off;
     uint32_t *thm;  // [groups][nB][Wp][2][32] through-set masks (k_through -> k_walk)
@@ -1123,7 +1123,7 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr)
 // short-lived ones cycle through: every chunk of the loop collides, and that row decides the time).  Words that other
 // thread blocks updated with atomics are read from L2.
 __device__ __forceinline__ void finish_candidate(uint64_t k, uint32_t nC, uint32_t AW, int list_all, const uint32_t *cstate,
-                                                 const uint32_t *anom, uint32_t *work, vl_verdict *out)
+                                                 const uint32_t *anom, uint32_t *work, vl_verdict *out, uint32_t fine_most)
 {
     const uint32_t *cs = cstate + k * 8;
     const uint32_t walk = __ldcg(cs + CS_WALK), thcol = __ldcg(cs + CS_THCOL);
@@ -1132,7 +1132,7 @@ __device__ __forceinline__ void finish_candidate(uint64_t k, uint32_t nC, uint32
         if (walk & WALK_FULL) chunks += nC;
         else if (walk)
             for (uint32_t w = 0; w < AW; ++w) chunks += __popc(__ldcg(anom + k * AW + w));
-        list_exact(work, k, chunks);
+        list_exact(work, k, chunks, fine_most);
         return;
     }
     const uint32_t fl = __ldcg(cs + CS_FLAGS), first = __ldcg(cs + CS_FIRST);
@@ -1478,7 +1478,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 3) k_walk(const WParams q)
     if (threadIdx.x == 0) q.grp_flag[grp] = 0;  // every block of the group has read it: clear for the next pass
     for (uint32_t j = threadIdx.x; j < TGW; j += blockDim.x) {
         const uint64_t kk = (uint64_t)grp * TGW + j;
-        if (kk < q.K) finish_candidate(kk, q.nC, q.AW, q.list_all, q.cstate, q.anom, q.work, q.out);
+        if (kk < q.K) finish_candidate(kk, q.nC, q.AW, q.list_all, q.cstate, q.anom, q.work, q.out, q.fine_most);
     }
 }
 
@@ -1486,7 +1486,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 3) k_walk(const WParams q)
 __global__ void k_finish(uint64_t K, int list_all, const uint32_t *cstate, const uint32_t *anom, uint32_t *work, vl_verdict *out)
 {
     const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < K) finish_candidate(k, 0, 0, list_all, cstate, anom, work, out);
+    if (k < K) finish_candidate(k, 0, 0, list_all, cstate, anom, work, out, EXACT_MAX_PARTS);
 }
 
 // --------------------------------------------------------------------------- host
@@ -1824,6 +1824,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
         WParams wq{};
         wq.V = p->V; wq.P = p->P; wq.nB = p->nB; wq.nC = p->nC; wq.Wp = pp.Wp; wq.AW = (uint32_t)vs.aw;
         wq.use_th = (uint32_t)p->use_th; wq.K = n; wq.early = early;
+        wq.fine_most = p->known[VL_KNOWN_SEN] >= FUSED_MANY_ENTRIES ? EXACT_MANY_PARTS : EXACT_MAX_PARTS;
         wq.th_off = p->d_th_off; wq.th = p->d_th; wq.cev_off = p->d_cev_off; wq.ev = p->d_ev;
         // the through-set masks come from a kernel of their own, except for small jobs
         const bool own_through = p->use_th && n >= 512;

@@ -187,3 +187,63 @@ def test_a_refused_program_is_refused_for_every_number_of_rows(B, oracle_mod, V,
         op = oracle_mod.OracleProgram(p)
         _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows))
     gp.close()
+
+
+def _crowded(n_blocks, per_block, V, P, seed):
+    """Every vreg is read again and again in every block: nearly all of them are live everywhere."""
+    rng = np.random.default_rng(seed)
+    blocks = [[([v], []) for v in range(V)] if b == 0 else [] for b in range(n_blocks)]
+    for b in range(n_blocks):
+        for _ in range(per_block):
+            blocks[b].append(([int(rng.integers(V))], [int(x) for x in rng.integers(0, V, 2)]))
+    edges = sorted({(b, b + 1) for b in range(n_blocks - 1)} | {(int(b), int(b) // 2) for b in rng.integers(1, n_blocks, n_blocks)})
+    return synth.program_from_lists(blocks, edges, V, [1 + int(x) for x in rng.integers(0, 3, V)], P)
+
+
+def _sm_count():
+    import torch
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("per_block,V,K", [(10, 200, 127), (40, 300, 1), (40, 300, 127), (40, 300, 128), (40, 300, "sms"), (40, 300, "sms+1")])
+def test_programs_that_occupy_many_vregs(B, oracle_mod, per_block, V, K):
+    """Fewer and more entries of the short chunks than the line between the kernels, at the edges of its row counts."""
+    K = {"sms": _sm_count(), "sms+1": _sm_count() + 1}.get(K, K)
+    p = _crowded(35, per_block, V, 700, per_block)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    rows = _garbage_rows(p, K, 3)
+    rows[::2] = np.stack([H.row_from_table(p, (np.arange(V) * 3 + 7 * (k % 4 == 0) * (np.arange(V) == 5)) % 690) for k in range(len(rows[::2]))])
+    _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows), f"K {K}")
+    gp.close()
+
+
+@pytest.mark.parametrize("with_through", [False, True])
+@pytest.mark.parametrize("n_banks", [4, 3])
+def test_long_lists(B, oracle_mod, with_through, n_banks):
+    """More than 1,024 entries per list on average (a warp counts an instruction), with and without a through-set;
+    instructions with many definitions and many reads, sources on one register."""
+    rng = np.random.default_rng(3)
+    A, N = 300, 1300
+    body = []
+    for i in range(900):
+        nd, nr = [(1, 2), (1, 4), (2, 3), (0, 2), (5, 9), (1, 0)][i % 6]
+        defs = [A + int(x) for x in rng.choice(N, nd, replace=False)]
+        body.append((defs, [int(x) for x in rng.integers(0, A + N, nr)]))
+    ends = [([], [A + v for v in range(j, min(j + 4, N))]) for j in range(0, N, 4)]
+    if with_through:   # vregs 0 .. A-1 are live through the loop; most of them are not touched in it
+        body = [(d, [v for v in r if v >= A or v < 20]) for d, r in body]
+    blocks = [[([v], []) for v in range(A)], [([A + v], []) for v in range(N)] + body + ends, [([], list(range(j, j + 4))) for j in range(0, A, 4)]]
+    p = synth.program_from_lists(blocks, [(0, 1), (1, 1), (1, 2)], A + N, [1 + (v % 7 == 0) + 2 * (v % 50 == 0) for v in range(A + N)], 3000, n_banks)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    good = np.cumsum(np.concatenate([[0], p.vreg_width[:-1]]))
+    assert good[-1] < 2900
+    tables = [good, good, np.where(np.arange(A + N) == 700, good[701], good), np.where(rng.random(A + N) < 0.01, good[::-1], good),
+              np.where(np.arange(A + N) < 2, 2999, good), np.where(np.arange(A + N) == 40, 3100, good), rng.integers(0, 3000, A + N)]
+    rows = np.stack([H.row_from_table(p, t) for t in tables] + list(_garbage_rows(p, 12, 4)))
+    rows[1, p.n_operands // 2] += 1
+    _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows))
+    gp.close()
