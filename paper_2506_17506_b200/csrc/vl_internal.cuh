@@ -94,6 +94,7 @@ struct vl_program {
     // pieces of one chunk; segments: runs of chunks of one block
     uint32_t nC = 0, nP = 0, nS = 0, nSeg = 0;
     uint32_t short_len = 1;  // instructions of the longest short chunk
+    bool wide_pieces = false;  // some piece has many operands (WIDE_OPERANDS, vl_liveness.cu)
     uint32_t layout_chunk_instrs = 0;  // chunk size the device copies of the layout were made for (0: none)
     std::vector<uint32_t> h_blk_off, h_op_off;
     // list lengths of the last liveness run with this layout: the next run allocates from them

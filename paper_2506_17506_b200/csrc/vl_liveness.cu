@@ -27,6 +27,8 @@
 #define PIECE_INSTRS 8
 #define PC_WARPS 20            // warps per block of k_sets and k_count: the pieces of a chunk of the default size at once
 #define PC_NT (PC_WARPS * 32)
+#define WIDE_OPERANDS 96       // operands of a piece from which k_count takes it instruction by instruction: 200
+                               // instructions of 60 reads 172 us for the run against 976, 100 of 100 definitions 202 against 2,133
 #define LV_WARPS 8             // warps per block of k_fill
 #define LV_NT (LV_WARPS * 32)
 #define FLOW_WARPS 16          // warps per block of k_flow
@@ -37,7 +39,7 @@
 // Everything the five kernels of a run read and write.
 struct LiveArgs {
     uint32_t nB, nI, V, nE, Wv, nC, nP, nS, nSeg;
-    int use_th;
+    int use_th, wide_smem;
     // program and layout
     const uint32_t *op_off, *op_vreg, *succ_off, *succ, *blk_off;
     const uint8_t *ndefs, *width;
@@ -136,8 +138,9 @@ __device__ __forceinline__ bool po_def(uint32_t x) { return (x >> 20) & 1u; }
 
 // ============================================================================ k_sets
 // One thread block per chunk.  use = vregs read before any write inside the piece (the chunk), def = vregs
-// written.  A lane holds an operand and meets the piece's other operands by shuffles.
-template <int N>
+// written.  A lane holds an operand and meets the piece's other operands by shuffles; WIDE (some piece of the launch has
+// many operands): a piece of more than 32 is taken instruction by instruction.
+template <int N, bool WIDE>
 __global__ void __launch_bounds__(PC_NT) k_sets(const __grid_constant__ LiveMany<N> a)
 {
     LIVE_ARGS;
@@ -157,7 +160,20 @@ __global__ void __launch_bounds__(PC_NT) k_sets(const __grid_constant__ LiveMany
         PieceOps po;
         po.init(q, p, c, lane);
         __syncwarp();
-        for (uint32_t r = 0; r < po.n; r += 32) {
+        if (WIDE && po.n > 32) {
+            for (uint32_t k = 0; k < po.ni; ++k) {
+                const uint32_t o0 = __shfl_sync(0xffffffffu, po.off, k), o1 = __shfl_sync(0xffffffffu, po.off, k + 1);
+                const uint32_t r0 = o0 + __shfl_sync(0xffffffffu, po.nd, k);
+                for (uint32_t o = r0 + lane; o < o1; o += 32) {
+                    const uint32_t v = q.op_vreg[o];
+                    if (!bit_get(s_def, v)) atomicOr(&s_use[v >> 5], 1u << (v & 31));
+                }
+                __syncwarp();
+                for (uint32_t o = o0 + lane; o < r0; o += 32) atomicOr(&s_def[q.op_vreg[o] >> 5], 1u << (q.op_vreg[o] & 31));
+                __syncwarp();
+            }
+        }
+        for (uint32_t r = 0; !(WIDE && po.n > 32) && r < po.n; r += 32) {
             const uint32_t x = po.get(q, r + lane);
             bool written = false;  // an earlier instruction of the piece writes this operand's vreg
             for (uint32_t j0 = 0; j0 <= r; j0 += 32) {
@@ -299,6 +315,56 @@ __global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const __grid_constant_
     }
 }
 
+// The operands of a wide piece (see k_count), instruction by instruction from the last: live (the vregs live after the
+// instruction) and reads (those it reads; empty between instructions) are bitsets of this warp's own.
+__device__ __noinline__ void count_wide(const LiveArgs &q, const PieceOps &po, volatile uint32_t *live, volatile uint32_t *reads,
+                                        uint32_t *touch, int *s_d, uint32_t *s_ev)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    auto has = [](volatile uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; };
+    auto word = [](volatile uint32_t *s, uint32_t v) { return const_cast<uint32_t *>(s) + (v >> 5); };
+    auto event = [&](uint32_t v, uint32_t k, uint32_t n) {
+        const uint32_t bit = 1u << (v & 31);
+        atomicAdd(&s_ev[k], n);
+        if (!(__ldcg(&touch[v >> 5]) & bit)) atomicOr(&touch[v >> 5], bit);
+    };
+    for (uint32_t k = po.ni; k-- > 0;) {
+        const uint32_t o0 = __shfl_sync(0xffffffffu, po.off, k), o1 = __shfl_sync(0xffffffffu, po.off, k + 1);
+        const uint32_t nd = __shfl_sync(0xffffffffu, po.nd, k), r0 = o0 + nd;
+        for (uint32_t o = r0; o < o1; o += 32) {  // which reads are the first of their vreg
+            const bool mine = o + lane < o1;
+            const uint32_t v = mine ? q.op_vreg[o + lane] : 0x10000u + lane;
+            const uint32_t same = __match_any_sync(0xffffffffu, v);
+            const bool dup = mine && ((same & ((1u << lane) - 1u)) || has(reads, v));
+            __syncwarp();
+            if (mine) {
+                if (!dup) atomicOr(word(reads, v), 1u << (v & 31));
+                const bool kill = !dup && !has(live, v);
+                q.opflags[o + lane] = (uint8_t)((kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0));
+                if (kill) event(v, k, 1);
+            }
+            __syncwarp();
+        }
+        for (uint32_t o = o0 + lane; o < r0; o += 32) {
+            const uint32_t v = q.op_vreg[o];
+            const bool lv = has(live, v), elide = has(reads, v) && lv, post = !lv && nd > 1;
+            q.opflags[o] = (uint8_t)(OPF_DEF | (elide ? OPF_ELIDE : 0) | ((lv || nd > 1) ? OPF_SET : 0) | (post ? OPF_POST : 0) | (lv ? 0 : OPF_DEAD));
+            if (!elide) event(v, k, 1 + (post ? 1 : 0));
+            if (lv) {  // (an instruction defines a vreg once)
+                atomicSub(&s_d[k], 1);
+                atomicAnd(word(live, v), ~(1u << (v & 31)));
+            }
+        }
+        __syncwarp();
+        for (uint32_t o = r0 + lane; o < o1; o += 32) {
+            const uint32_t v = q.op_vreg[o], bit = 1u << (v & 31);
+            if (!(atomicOr(word(live, v), bit) & bit)) atomicAdd(&s_d[k], 1);
+            atomicAnd(word(reads, v), ~bit);
+        }
+        __syncwarp();
+    }
+}
+
 // ============================================================================ k_count
 // One thread block per chunk.  First the live set after the last instruction of every piece (one thread per
 // bitset word, backwards over the chunk's pieces).  Then one warp per piece, one lane per operand: an operand's
@@ -306,7 +372,9 @@ __global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const __grid_constant_
 // none does, iff it is live after the piece.  From that the operand flags, the walk events and the change of
 // the live count of every instruction follow without a serial walk; and the set of vregs whose occupancy
 // changes inside the block.  Last, offsets inside the chunk.
-template <int N>
+// WIDE: some piece of the launch has more than WIDE_OPERANDS operands, which would meet each other in pairs; it is
+// taken instruction by instruction (count_wide).
+template <int N, bool WIDE>
 __global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMany<N> a)
 {
     LIVE_ARGS;
@@ -356,7 +424,16 @@ __global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMan
         for (uint32_t w = lane; w < q.Wv; w += 32) cnt += __popc(end[w]);
         cnt = __reduce_add_sync(0xffffffffu, cnt);
         __syncwarp();
-        for (uint32_t r = 0; r < po.n; r += 32) {
+        const bool wide = WIDE && po.n > WIDE_OPERANDS;
+        if constexpr (WIDE) if (wide) {  // the bitsets: in shared memory if they fit, else in the rows of the piece's sets, used up by now
+            extern __shared__ uint32_t sm[];
+            uint32_t *live = q.wide_smem ? sm + (size_t)warp * 2 * q.Wv : q.piece_use + (size_t)p * q.Wv;
+            uint32_t *reads = q.wide_smem ? live + q.Wv : q.piece_def + (size_t)p * q.Wv;
+            for (uint32_t w = lane; w < q.Wv; w += 32) { live[w] = end[w]; reads[w] = 0; }
+            __syncwarp();
+            count_wide(q, po, live, reads, touch, s_d[warp], s_ev[warp]);
+        }
+        for (uint32_t r = 0; !wide && r < po.n; r += 32) {
             const uint32_t x = r == 0 ? x0 : po.get(q, r + lane), v = po_vreg(x), k = po_instr(x);
             const bool mine = r + lane < po.n, def = po_def(x);
             const uint32_t nd = __shfl_sync(0xffffffffu, po.nd, k < PIECE_INSTRS ? k : 0);
@@ -861,10 +938,12 @@ int live_attributes(vl_program *p)
     std::lock_guard<std::mutex> lock(mtx);
     if (done[p->device]) return VL_OK;
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1, false>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1, true>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_flow<1>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_fill<1>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY, false>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY, true>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_flow<LV_MANY>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_fill<LV_MANY>, at, 227 * 1024));
     done[p->device] = true;
@@ -916,6 +995,11 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         blk_c_off[b + 1] = (uint32_t)c_i0.size();
     }
     c_p_off.push_back((uint32_t)p_i0.size());
+    p->wide_pieces = false;
+    for (size_t j = 0; j < p_i0.size(); ++j) {
+        const uint32_t i1 = std::min(p_i0[j] + PIECE_INSTRS, c_i1[p_chunk[j]]);
+        p->wide_pieces = p->wide_pieces || p->h_op_off[i1] - p->h_op_off[p_i0[j]] > WIDE_OPERANDS;
+    }
     const uint32_t nC = p->nC = (uint32_t)c_i0.size();
     p->nP = (uint32_t)p_i0.size();
     // segments of k_flow: at most about 256 of them beside one per block
@@ -978,14 +1062,17 @@ static int vl_layout(vl_program *p, cudaStream_t st)
 
 // What a run's launches need besides the arguments.
 struct LiveShape {
+    bool wide = false;
     uint32_t set_warps = PC_WARPS, sets = 0, flows = 0, counts = 0, offs = 0, fills = 0;
-    size_t sets_smem = 0, flow_smem = 0, fill_smem = 0;
+    size_t sets_smem = 0, flow_smem = 0, count_smem = 0, fill_smem = 0;
     void add(const LiveShape &o)
     {
+        wide = wide || o.wide;
         set_warps = std::min(set_warps, o.set_warps);
         sets = std::max(sets, o.sets); flows = std::max(flows, o.flows); counts = std::max(counts, o.counts);
         offs = std::max(offs, o.offs); fills = std::max(fills, o.fills);
         sets_smem = std::max(sets_smem, o.sets_smem); flow_smem = std::max(flow_smem, o.flow_smem);
+        count_smem = std::max(count_smem, o.count_smem);
         fill_smem = std::max(fill_smem, o.fill_smem);
     }
 };
@@ -1070,6 +1157,10 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     sh.sets = std::max(1u, nC); sh.flows = fgrid; sh.counts = nC; sh.offs = nC + nB;
     sh.fills = (nP + LV_WARPS - 1) / LV_WARPS + nC + ((p->nS + 31) & ~31u) / LV_WARPS + nB;
     sh.sets_smem = (size_t)sh.set_warps * 2 * Wv * 4;
+    sh.wide = p->wide_pieces;
+    sh.count_smem = p->wide_pieces ? (size_t)PC_WARPS * 2 * Wv * 4 : 0;
+    q.wide_smem = sh.count_smem <= 40 * 1024;
+    if (!q.wide_smem) sh.count_smem = 0;
     sh.flow_smem = flow_smem;
     sh.fill_smem = (size_t)LV_WARPS * 2 * Wv * 4;
     return VL_OK;
@@ -1137,9 +1228,11 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
         VL_CUDA(p, launch_overlap(k_fill<N>, dim3(sh.fills, n), LV_NT, sh.fill_smem, st, true, many));
         return VL_OK;
     }
-    VL_CUDA(p, launch_overlap(k_sets<N>, dim3(sh.sets, n), sh.set_warps * 32, sh.sets_smem, st, true, many));
+    if (sh.wide) VL_CUDA(p, launch_overlap(k_sets<N, true>, dim3(sh.sets, n), sh.set_warps * 32, sh.sets_smem, st, true, many));
+    else VL_CUDA(p, launch_overlap(k_sets<N, false>, dim3(sh.sets, n), sh.set_warps * 32, sh.sets_smem, st, true, many));
     VL_CUDA(p, launch_overlap(k_flow<N>, dim3(sh.flows, n), FLOW_WARPS * 32, sh.flow_smem, st, true, many));
-    if (sh.counts) VL_CUDA(p, launch_overlap(k_count<N>, dim3(sh.counts, n), PC_NT, 0, st, true, many));
+    if (sh.counts && sh.wide) VL_CUDA(p, launch_overlap(k_count<N, true>, dim3(sh.counts, n), PC_NT, sh.count_smem, st, true, many));
+    else if (sh.counts) VL_CUDA(p, launch_overlap(k_count<N, false>, dim3(sh.counts, n), PC_NT, 0, st, true, many));
     VL_CUDA(p, launch_overlap(k_offsets<N>, dim3(sh.offs, n), OFF_NT, 0, st, true, many));
     return VL_OK;
 }

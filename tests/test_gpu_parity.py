@@ -450,3 +450,30 @@ def test_batch_with_a_program_given_several_times(B, oracle_mod, K):
             _assert_same(B.verdicts_to_numpy(o), _oracle_rows_threaded(oracle_mod, p, lv, r), f"call {call} entry {j}")
     gp.close()
     other.close()
+
+
+@pytest.mark.parametrize("V", [700, 12000])
+@pytest.mark.parametrize("n_defs,n_reads", [(1, 3), (1, 4), (1, 11), (2, 12), (40, 3), (255, 0), (3, 300), (200, 90)])
+def test_instructions_with_many_operands(B, oracle_mod, V, n_defs, n_reads):
+    """Pieces below, at and above the line from which their operands are taken instruction by instruction; repeated reads,
+    reads of what the instruction defines, dead co-definitions; bitsets that fit shared memory and ones that do not."""
+    rng = np.random.default_rng(n_defs * 1000 + n_reads)
+    some = rng.choice(V, 700, replace=False)
+    blocks = [[([int(v)], []) for v in some], [], []]
+    for b in (1, 2):
+        for i in range(37):
+            nd, nr = (n_defs, n_reads) if i % 3 else (1, 2)
+            defs = rng.choice(some, nd, replace=False)
+            reads = rng.choice(some if i % 2 else some[:40], nr)
+            if nr and nd:
+                reads[: nr // 4] = rng.choice(defs, nr // 4)
+            blocks[b].append(([int(v) for v in defs], [int(v) for v in reads]))
+    p = synth.program_from_lists(blocks, [(0, 1), (1, 1), (1, 2)], V, [1 + int(v) % 3 for v in rng.integers(0, 3, V)], 2500)
+    gp, lv = _check_liveness(B, oracle_mod, p)
+    rows = np.concatenate([_garbage_rows(p, 12, 1), np.stack([H.row_from_table(p, (np.arange(V) * 3) % 2490)] * 2)])
+    rows[-1, 800] += 5
+    want = oracle_mod.OracleProgram(p).verify(lv, rows)
+    _assert_same(_gpu_verify(B, gp, rows), want, "short jobs")
+    gp.set_option(B.VL_OPT_GROUP, 4)
+    _assert_same(_gpu_verify(B, gp, rows), want, "batched")
+    gp.close()
