@@ -127,6 +127,62 @@ __device__ __forceinline__ uint32_t bank_instr(const FParams &q, const uint16_t 
     return n;
 }
 
+// The same for instructions [i0, i1), counted by a whole block: four instructions of a thread in flight, from their records;
+// an instruction of more than four reads by a warp, a lane per read.  Returns this thread's share.
+__device__ __noinline__ uint32_t bank_instrs(const FParams &q, const uint16_t *T, uint32_t i0, uint32_t i1)
+{
+    constexpr uint32_t U = 4;
+    const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+    uint32_t n = 0;
+    for (uint32_t base = i0 + (threadIdx.x & ~31u); base < i1; base += U * blockDim.x) {  // (the same for a whole warp)
+        uint4 rec[U];
+        uint32_t rd[U][4];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) rec[u] = q.irec[min(base + lane + u * blockDim.x, q.nI - 1)];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) {
+            const uint32_t nr = (rec[u].y >> 24) & 127u, o = rec[u].w + ((rec[u].y >> 16) & 0xFFu);
+#pragma unroll
+            for (uint32_t r = 0; r < 4; ++r) rd[u][r] = q.op_vreg[nr ? o + min(r, nr - 1) : 0u];  // (missing reads repeat the last one)
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) {
+            const uint32_t i = base + lane + u * blockDim.x, nr = i < i1 ? (rec[u].y >> 24) & 127u : 0u;
+            uint32_t x[4], m[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) { x[a] = T[rd[u][a]]; m[a] = x[a] % q.B; }
+            if (nr <= 4) {
+#pragma unroll
+                for (int a = 1; a < 4; ++a) {
+                    bool value = false, bank = false;
+#pragma unroll
+                    for (int b = 0; b < a; ++b) { value |= x[b] == x[a]; bank |= m[b] == m[a]; }
+                    n += nr > 1 && !value && bank;
+                }
+            }
+            for (uint32_t todo = __ballot_sync(0xffffffffu, nr > 4); todo; todo &= todo - 1) {
+                const uint32_t j = base + (__ffs(todo) - 1) + u * blockDim.x;
+                const uint32_t u0 = q.op_off[j] + q.ndefs[j], k = q.op_off[j + 1] - u0;
+                for (uint32_t a0 = 0; a0 < k; a0 += 32) {
+                    const bool mine = a0 + lane < k;
+                    const uint32_t ta = mine ? T[q.op_vreg[u0 + a0 + lane]] : 0x10000u + lane, ma = mine ? ta % q.B : ta;
+                    bool value = __match_any_sync(0xffffffffu, ta) & below, bank = __match_any_sync(0xffffffffu, ma) & below;
+                    for (uint32_t b0 = 0; b0 < a0; b0 += 32) {
+                        const uint32_t tb = T[q.op_vreg[u0 + b0 + lane]], mb = tb % q.B;
+#pragma unroll 8
+                        for (uint32_t b = 0; b < 32; ++b) {
+                            value |= __shfl_sync(0xffffffffu, tb, b) == ta;
+                            bank |= __shfl_sync(0xffffffffu, mb, b) == ma;
+                        }
+                    }
+                    n += mine && !value && bank;
+                }
+            }
+        }
+    }
+    return n;
+}
+
 // Sources (up to four reads, vreg ids; repeats of a vreg do not count) that hold the register of an earlier source.
 __device__ __forceinline__ uint32_t duplicates(const uint32_t (&rd)[4], const uint16_t *T)
 {
@@ -374,7 +430,7 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
                 if (i == 0xFFFFFFFFu) continue;
                 const uint32_t n = rec.y & 0xFFFFu, nd = (rec.y >> 16) & 0xFFu, p0 = rec.x >> 2, p1 = n ? (rec.x + n - 1) >> 2 : p0;
                 uint32_t n_dup = 0;
-                for (uint32_t a = rec.w + nd + lane; a < q.op_off[i + 1]; a += 32) n_dup += duplicate_of(q, T, rec.w + nd, a);
+                for (uint32_t a = rec.w + nd + lane; q.bank_fast && a < q.op_off[i + 1]; a += 32) n_dup += duplicate_of(q, T, rec.w + nd, a);
                 n_dup = __reduce_add_sync(0xffffffffu, n_dup);
                 if (lane == 0 && n_dup) dups += n_dup - ((thcol >> b) & 1u ? member_duplicates(q, T, b, i) : 0u);
                 for (uint32_t d = 0; d < nd; ++d) {
@@ -429,7 +485,7 @@ __device__ __forceinline__ void exact_counts(const FParams &q, uint16_t *T, uint
                 i_nx2 = next_instr(b_nx2);
                 rec_nx2 = fetch_rec(i_nx2);
                 const uint32_t n = rec.y & 0xFFFFu, nd = i != 0xFFFFFFFFu ? (rec.y >> 16) & 0xFFu : 0u;
-                if (LISTED && i != 0xFFFFFFFFu) {
+                if (LISTED && i != 0xFFFFFFFFu && q.bank_fast) {  // (else the tally is made anew)
                     const uint32_t nr = (rec.y >> 24) & 127u;
                     uint32_t n_dup = 0;
                     if (nr <= 4) {  // (missing reads repeat the last one)
@@ -973,14 +1029,18 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
         if (ROWS || q.bank_fast) {
             if (tid == 0) M->bank = (part == 0 ? cs[CS_BANK] : 0u) - (ROWS ? 0u : M->dups);
         } else {  // the general tally: the whole table, this part's instructions
-            for (uint32_t v = tid; v < q.V; v += EXACT_NT) {
-                const uint32_t pos = q.first_occ[v];
-                T[v] = pos != 0xFFFFFFFFu ? row[pos] : (uint16_t)0;
+            for (uint32_t v0 = tid; v0 < q.V; v0 += 8 * EXACT_NT) {
+                uint32_t pos[8], t[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) pos[u] = q.first_occ[min(v0 + u * EXACT_NT, q.V - 1)];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) t[u] = row[pos[u] != 0xFFFFFFFFu ? pos[u] : 0u];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (v0 + u * EXACT_NT < q.V) T[v0 + u * EXACT_NT] = pos[u] != 0xFFFFFFFFu ? (uint16_t)t[u] : (uint16_t)0;
             }
             __syncthreads();
-            uint32_t n = 0;
-            const uint32_t i1 = (uint32_t)((uint64_t)q.nI * (part + 1) / parts);
-            for (uint32_t i = (uint32_t)((uint64_t)q.nI * part / parts) + tid; i < i1; i += EXACT_NT) n += bank_instr(q, T, i);
+            uint32_t n = bank_instrs(q, T, (uint32_t)((uint64_t)q.nI * part / parts), (uint32_t)((uint64_t)q.nI * (part + 1) / parts));
             n = __reduce_add_sync(0xffffffffu, n);
             if (lane == 0 && n) atomicAdd(&M->bank, n);
         }
@@ -1063,8 +1123,9 @@ FParams fused_params(const vl_program *p, bool dict)
 // its collisions in lists as long, which the batched kernels spread over the multiprocessors.  3,500 instructions with 500
 // vregs live everywhere, rows that collide everywhere: 1 row 101 us against 410, 100 rows 320 against 416, 148 rows 424
 // against 418, 300 rows 690 against 1,211; 24,300 instructions with 300 such vregs: 1 row 0.56 ms against 13, 127 rows 29.8
-// against 13, 148 rows 34.7 against 13.  (The line, 32,768 entries: 860 instructions with 200 vregs, 22,000 entries, take 60
-// us here and 65 there, 1,620 with 300, 60,000 entries, 115 and 74.  Programs whose values live shortly have below 10,000.)
+// against 13, 148 rows 34.7 against 13.  (The line, 49,152 entries: one row of 860 instructions with 200 vregs, 22,000 entries,
+// takes 60 us here and 65 there, of 1,620 with 300, 60,000 entries, 115 and 74; of 800 with 600 of which 200 read 60 vregs each,
+// 37,000 entries and no fast bank tally, 192 and 423.  Programs whose values live shortly have below 10,000.)
 #define FUSED_FEW_ROWS 128u
 // 100 rows that collide everywhere, a warp per instruction against a thread: lists of 2,330 entries on average 5,916 us against
 // 8,602, of 1,013 1,441 against 1,261, of 557 640 against 454.

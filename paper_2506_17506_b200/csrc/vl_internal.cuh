@@ -264,7 +264,7 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
 bool vl_fused_wanted(vl_program *p, uint64_t K);
 // Entries of the short chunks (vreg and short chunk at whose beginning it is occupied) from which a program counts as one
 // that occupies many.
-#define FUSED_MANY_ENTRIES 32768u  // (measured at vl_fused_wanted)
+#define FUSED_MANY_ENTRIES 49152u  // (measured at vl_fused_wanted)
 bool vl_verify_takes(const vl_program *p);  // whether the verify path takes the program (vl_verify.cu)
 bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,

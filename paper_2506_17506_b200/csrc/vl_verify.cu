@@ -1128,7 +1128,7 @@ __device__ __forceinline__ void finish_candidate(uint64_t k, uint32_t nC, uint32
     const uint32_t *cs = cstate + k * 8;
     const uint32_t walk = __ldcg(cs + CS_WALK), thcol = __ldcg(cs + CS_THCOL);
     if (list_all || (walk | thcol)) {
-        uint32_t chunks = list_all ? nC / 4 : (thcol ? nC / 8 : 0u);  // (the general bank tally; the sources in the through-set)
+        uint32_t chunks = list_all ? nC / 8 : (thcol ? nC / 8 : 0u);  // (the general bank tally; the sources in the through-set)
         if (walk & WALK_FULL) chunks += nC;
         else if (walk)
             for (uint32_t w = 0; w < AW; ++w) chunks += __popc(__ldcg(anom + k * AW + w));

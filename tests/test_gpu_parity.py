@@ -477,3 +477,23 @@ def test_instructions_with_many_operands(B, oracle_mod, V, n_defs, n_reads):
     gp.set_option(B.VL_OPT_GROUP, 4)
     _assert_same(_gpu_verify(B, gp, rows), want, "batched")
     gp.close()
+
+
+@pytest.mark.parametrize("n_banks", [3, 5, 64, 100000])
+@pytest.mark.parametrize("chunk", [160, 8])
+def test_general_bank_tally(B, oracle_mod, n_banks, chunk):
+    """Banks that have no fast tally, in the batched kernels: 0 to 130 reads per instruction (a thread, then a warp takes one),
+    vregs read twice, sources on one register, one and several items per candidate."""
+    rng = np.random.default_rng(n_banks)
+    V = 300
+    n_reads = [0, 1, 2, 3, 4, 5, 8, 31, 32, 33, 63, 64, 65, 96, 97, 130] * 12
+    blocks = [[([v], []) for v in range(V)] + [([int(rng.integers(V))], [int(x) for x in rng.integers(0, [V, 9][i % 2], n)]) for i, n in enumerate(n_reads)]]
+    p = synth.program_from_lists(blocks, [], V, [1] * V, 400, n_banks)
+    gp = B.Program(p)
+    gp.set_option(B.VL_OPT_CHUNK_INSTRS, chunk)
+    gp.set_option(B.VL_OPT_GROUP, 8)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    rows = np.concatenate([_garbage_rows(p, 18, 1), np.stack([H.row_from_table(p, np.arange(V) + k) for k in range(3)])])
+    _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows))
+    gp.close()

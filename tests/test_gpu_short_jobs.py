@@ -205,7 +205,7 @@ def _sm_count():
     return torch.cuda.get_device_properties(0).multi_processor_count
 
 
-@pytest.mark.parametrize("per_block,V,K", [(10, 200, 127), (40, 300, 1), (40, 300, 127), (40, 300, 128), (40, 300, "sms"), (40, 300, "sms+1")])
+@pytest.mark.parametrize("per_block,V,K", [(10, 200, 127), (60, 300, 1), (60, 300, 127), (60, 300, 128), (60, 300, "sms"), (60, 300, "sms+1")])
 def test_programs_that_occupy_many_vregs(B, oracle_mod, per_block, V, K):
     """Fewer and more entries of the short chunks than the line between the kernels, at the edges of its row counts."""
     K = {"sms": _sm_count(), "sms+1": _sm_count() + 1}.get(K, K)
