@@ -386,8 +386,10 @@ uint64_t vl_kernel_launches(void);
 /*
  * Device time of the verify kernels since the last call (or since VL_OPT_KERNEL_TIMING was set), summed over
  * the passes recorded (at most 4096): ms[0] table kernel (first occurrences, Consistency, Realizability, bank
- * tally), ms[1] occupancy walk (Safety), ms[2] verdict kernel, ms[3] exact counts (a short job's one kernel: in ms[0]).  ms is HOST memory for
- * 4 floats; *passes (HOST, may be NULL) receives the number of passes summed.  Kernels of different passes
+ * tally), ms[1] occupancy walk (Safety), ms[2] verdict kernel, ms[3] exact counts.  A short job is one pass: its one kernel
+ * is in ms[0], the exact counts it may hand over in ms[3]; short jobs of several programs that share a launch of
+ * vl_verify_batch have the time of the whole launch each.  ms is HOST memory for 4 floats; *passes (HOST, may be NULL)
+ * receives the number of passes summed.  Kernels of different passes
  * may run side by side (VL_OPT_LANES), so the four sums can add up to more than the duration of the calls.
  * Waits for the last recorded event, then forgets the events.  Without the option everything is 0.  Errors: INVALID_ARG, CUDA.
  */

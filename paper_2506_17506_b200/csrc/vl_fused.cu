@@ -1207,6 +1207,15 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         const int rc = vl_live_join(p, from, st);
         if (rc != VL_OK) return rc;
     }
+    // timing events: a job's one kernel counts as the table kernel, what it hands over as the exact counts; every handle of a
+    // shared launch has the whole launch
+    auto mark = [&](int times) {
+        for (uint32_t j = 0; j < n; ++j) {
+            if (!progs[j]->ktime || std::find(progs, progs + j, progs[j]) != progs + j) continue;
+            for (int t = 0; t < times; ++t) kt_mark(progs[j], st);
+        }
+    };
+    mark(1);
     if (n > 1) {
         VL_CUDA(p0, launch_overlap(k_fused<256, 3, VL_FUSED_MANY, false>, dim3((uint32_t)rows, n), 256, smem, st, true, many));
     } else {
@@ -1219,12 +1228,16 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
             if (rc != VL_OK) return rc;
             VL_CUDA(p0, pl.bpm == 3 ? launch_overlap(k_fused<256, 3, 1, true>, grid, 256, smem, st, true, one)
                                     : launch_overlap(k_fused<256, 2, 1, true>, grid, 256, smem, st, true, one));
-            return vl_exact_run(p0, ex, d_cand[0], pitch[0], d_out[0], st, dict, true);
+            mark(3);
+            const int re = vl_exact_run(p0, ex, d_cand[0], pitch[0], d_out[0], st, dict, true);
+            mark(1);
+            return re;
         }
         if (pl.threads == 512) VL_CUDA(p0, launch_overlap(k_fused<512, 1, 1, false>, grid, 512, smem, st, true, one));
         else if (pl.bpm == 3) VL_CUDA(p0, launch_overlap(k_fused<256, 3, 1, false>, grid, 256, smem, st, true, one));
         else VL_CUDA(p0, launch_overlap(k_fused<256, 2, 1, false>, grid, 256, smem, st, true, one));
     }
+    mark(4);
     return VL_OK;
 }
 

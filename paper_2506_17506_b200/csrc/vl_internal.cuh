@@ -317,6 +317,8 @@ uint64_t vl_exact_scratch(vl_program *p);
 bool vl_exact_takes_rows(vl_program *p, uint64_t rows);  // whether k_exact can count for that many rows of k_fused
 int vl_exact_run(vl_program *p, const VlExactArgs &ex, const uint16_t *d_cand, uint64_t pitch, vl_verdict *d_out, cudaStream_t st,
                  bool dict, bool overlap);
+// Records the next timing event of the handle on `st` (no-op unless kernel timing is switched on).
+void kt_mark(vl_program *p, cudaStream_t st);
 int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t pitch, vl_verdict *d_out,
                    cudaStream_t st, int slot, bool dict = false);
 int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K,

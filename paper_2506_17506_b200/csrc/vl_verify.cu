@@ -1659,8 +1659,7 @@ int ensure_scratch(vl_program *p, int slot, uint64_t rows)
 }
 }  // namespace
 
-// Records the next timing event of the handle on `st` (no-op unless kernel timing is switched on).
-static void kt_mark(vl_program *p, cudaStream_t st)
+void kt_mark(vl_program *p, cudaStream_t st)
 {
     if (!p->ktime || p->kt_used >= 5 * 4096) return;
     if (p->kt_used == p->kt_ev.size()) {
@@ -1865,10 +1864,7 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
                    cudaStream_t st, int slot, bool dict)
 {
     if (vl_fused_wanted(p, K)) {
-        kt_mark(p, st);
-        const int rf = vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, st, dict, slot);
-        for (int j = 0; j < 4; ++j) kt_mark(p, st);
-        return rf;
+        return vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, st, dict, slot);
     }
     PassPlan pp{};
     int rc = plan_passes(p, K, &pp);

@@ -247,3 +247,37 @@ def test_long_lists(B, oracle_mod, with_through, n_banks):
     rows[1, p.n_operands // 2] += 1
     _assert_same(_gpu_verify(B, gp, rows), op.verify(op.liveness(), rows))
     gp.close()
+
+
+@pytest.mark.parametrize("K", [20, 300, 700])
+def test_kernel_times_of_short_jobs(B, K):
+    """Every call records a pass of every handle that asks for it: alone, handed over, in a launch that programs share, on
+    lanes, by the batched kernels."""
+    import torch
+    wl = synth.workload(2)
+    big = synth.build_program(wl.shapes[0], wl.seeds[0])
+    small = synth.build_program(synth.shape_gemm(), 1)
+    progs = [big, small, small]
+    gps = [B.Program(p) for p in progs]
+    B.vl_liveness_batch(gps)
+    rows = [_to_dev(synth.candidate_rows(p, K, 0.3, 5)[0]) for p in progs]
+    for gp in gps[:2]:
+        gp.set_option(B.VL_OPT_KERNEL_TIMING, 1)
+    for call in range(2):
+        B.vl_verify_batch(gps, rows)
+        torch.cuda.synchronize()
+        for gp, n in zip(gps, (1, 1, 0)):
+            ms, passes = gp.vl_kernel_times()
+            assert passes == n and all(x >= 0 for x in ms) and (ms[0] > 0) == (n > 0)
+    B.vl_verify_batch([gps[1], gps[1]], [rows[1], rows[1]])     # a handle given twice in one launch, or in two
+    torch.cuda.synchronize()
+    ms, passes = gps[1].vl_kernel_times()
+    assert passes in (1, 2) and 0 < sum(ms) < 100
+    gps[0].vl_verify(rows[0])
+    torch.cuda.synchronize()
+    ms, passes = gps[0].vl_kernel_times()
+    assert passes == 1 and ms[0] > 0
+    if K == 300:                                                # 8,000 instructions: k_fused, then k_exact
+        assert ms[1] < ms[0] and ms[2] < ms[0] and ms[3] > 0.004
+    for gp in gps:
+        gp.close()
