@@ -1688,9 +1688,11 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
     Plan pl{};
     const uint32_t groups[3] = {4, 2, 1};
     if (p->group_opt == 0 || p->group_opt == 8) {
-        // (hardware rules, and no more blocks than multiprocessors: the sweep over the rules takes 512 threads; 98 blocks
-        // 51 -> 44 us.  Without rules 256 are the better choice even then, 83 us against 88 for a call of 125 blocks: a
-        // block leaves room for the first ones of the walk)
+        // (hardware rules, and no more blocks than multiprocessors: the sweep over the rules takes 512 threads.  Programs of
+        // 8,000 to 11,317 instructions, three of them, the whole call with 256 and 512 threads: 63 blocks 116, 144, 132 us and
+        // 107, 132, 126; 98 blocks 106, 127, 115 and 116, 120, 117; 125 blocks 116, 131, 130 and 122, 116, 117; 148 blocks 126,
+        // 126, 131 and 117, 123, 122; 188 blocks 133, 143, 141 and 145, 150, 152.  Without rules neither wins up to 148
+        // blocks: 104, 127, 120 and 102, 124, 118 at 63, 96, 110, 106 and 111, 111, 110 at 98, and 256 leave room for the walk)
         const bool alone = p->d_vcons && (K + 7) / 8 <= (uint64_t)vl_sm_count(p);
         if (!alone || p->threads_opt) pl = make_plan8(p, p->threads_opt ? p->threads_opt : 256, SM_BYTES / 2 - 1024);
         if (!pl.ok) pl = make_plan8(p, p->threads_opt ? p->threads_opt : 512, SM_BYTES);
@@ -1699,7 +1701,10 @@ int plan_passes(vl_program *p, uint64_t K, PassPlan *pp)
     for (uint32_t G : groups) {
         if (pl.ok) break;
         if (p->group_opt && G != p->group_opt) continue;
-        if (p->threads_opt != 256) pl = make_plan(p, G, 512, SM_BYTES);
+        // (where the caller asks for fewer candidates than fit: two blocks of 256 threads, if a multiprocessor holds them.
+        // 3,000 rows of 12,000 instructions, two candidates 238 us against 257 with 512 threads, one 327 against 370)
+        pl = make_plan(p, G, p->threads_opt ? p->threads_opt : 256, SM_BYTES / 2 - 1024);
+        if (!pl.ok && p->threads_opt != 256) pl = make_plan(p, G, 512, SM_BYTES);
         if (!pl.ok && p->threads_opt != 512) pl = make_plan(p, G, 256, SM_BYTES);
     }
     if (!pl.ok) return VL_ERR_UNSUPPORTED;
