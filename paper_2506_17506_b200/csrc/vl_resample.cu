@@ -118,8 +118,10 @@ __global__ void __launch_bounds__(256) k_resample_summary(const RsSumParams q)
     if (tid == 0) q.summary->n_cases = q.n;
 }
 
-// One block, up to a few thousand verdicts of one test case: its record goes straight to pinned host memory, then the
-// sequence number that the host polls for (a kernel less, a copy less and no stream wait in the early-exit loop).
+// One block, the verdicts of a batch: its record goes straight to pinned host memory, then the sequence number that the host
+// polls for (a kernel less, a copy less and no stream wait in the early-exit loop).  One block reads 5 verdicts per ns: 13 us
+// in a loop of 109 for 4,096 rows of 64 instructions, 22 of 1,263 for 65,536, 78 of 7,403 for 400,000; the statistics kernels
+// of many blocks, with their copy and wait, take 27, 29 and 46.
 __global__ void __launch_bounds__(RS_THREADS) k_batch_record(const uint4 *out, uint32_t K, unsigned long long *record,
                                                              unsigned long long seq)
 {

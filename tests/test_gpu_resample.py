@@ -172,3 +172,25 @@ def test_loop_of_a_new_handle_does_not_read_the_record_of_a_destroyed_one(B, ora
         assert B.verdicts_to_numpy(out).tobytes() == op.verify(lv, r).tobytes()
     for gp in new:
         gp.close()
+
+
+@pytest.mark.parametrize("K,batch_rows", [(513, 513), (20000, 8192), (20000, 10**7)])
+def test_loop_with_large_batches(B, oracle_mod, K, batch_rows):
+    """Batches of more rows than the record's block has threads; the passing row first, last, nowhere."""
+    wl = synth.workload(0)
+    p = synth.build_program(wl.shapes[0], wl.seeds[0])
+    rows, faults = synth.candidate_rows(p, 100, 0.5, wl.seeds[0])
+    good, bad = rows[faults[:, 0] == 0][0], rows[faults[:, 0] != 0]
+    gp = B.Program(p)
+    gp.vl_liveness()
+    for at in (K - 1, 0, 8192, None):
+        r = np.ascontiguousarray(bad[np.arange(K) % len(bad)])
+        if at is not None and at < K:
+            r[at] = good
+        else:
+            at = K
+        out, done, first = gp.vl_verify_until_pass(_to_dev(r), batch_rows)
+        assert first == at and done == min(K, (at // batch_rows + 1) * batch_rows)
+        flags = B.verdicts_to_numpy(out)["flags"]
+        assert (np.flatnonzero(flags == 1).tolist() == ([at] if at < K else [])) and not flags[done:].any() and flags[:done].all()
+    gp.close()
