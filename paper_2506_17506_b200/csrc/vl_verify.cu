@@ -1904,6 +1904,36 @@ struct FusedGroup {
 };
 }  // namespace
 
+namespace {
+// How the short jobs of several programs run: in shared launches, in a launch each, or by the batched kernels.
+enum Together { SHARED, SINGLE, BATCHED };
+
+// The rows of all of them decide, not those of one.  Estimates in microseconds, from 2 to 96 programs of 2,000 to 26,000
+// instructions with 20 to 148 rows each, 15 % failing: a shared launch takes rounds of three rows per multiprocessor and is as
+// long as its longest row at least, launches of their own one row per multiprocessor and a launch each, the batched kernels
+// four launches per program over the lanes.  Measured / estimated, shared, single, batched: 96 x 2,000 x 148 rows 470/550,
+// 913/1,227, 1,004/1,828; 8 x 8,000 x 50 121/128, 91/109, 201/222; 8 x 20,000 x 148 366/371, 306/307, 259/262; 48 x 20,000 x 100
+// 860/908, 977/1,199, 1,035/1,107; 48 x 26,000 x 148 1,522/1,571, 1,752/2,003, 1,307/1,276; 2 x 14,000 x 100 175/169, 86/74, 140/113.
+Together together(uint32_t nprog, vl_program *const *progs, const uint64_t *K, const std::vector<uint8_t> &shares)
+{
+    double n = 0, rows = 0, work = 0, longest = 0;
+    for (uint32_t j = 0; j < nprog; ++j) {
+        if (!shares[j]) continue;
+        const double a = progs[j]->nI / 1000.0;
+        n += 1;
+        rows += (double)K[j];
+        work += a * (double)K[j];
+        longest = std::max(longest, a);
+    }
+    if (n < 2) return SINGLE;
+    const double sms = vl_sm_count(progs[0]), a = work / rows;
+    const double shared = 35 + 8 * longest + rows / (3 * sms) * (10 + 2.8 * a);
+    const double single = 35 + 4 * n + rows / sms * (6 + 1.2 * a);
+    const double batched = 75 + 17.7 * n + 0.0019 * work;
+    return shared <= single && shared <= batched ? SHARED : (single <= batched ? SINGLE : BATCHED);
+}
+}  // namespace
+
 // Passes of one or several programs spread round-robin over the device's lane streams, so that
 // the table kernel of one pass (bound by the row stream) runs beside the walk of another (bound by
 // instruction issue).  Pass j of a program uses working set j mod lanes and runs on lane
@@ -1924,7 +1954,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
         FusedGroup g;
         for (uint32_t j = 0; j < nprog; ++j) {
             if (K[j] == 0) continue;
-            if (nprog > 1 && vl_fused_shares(progs[j], K[j])) {
+            if (jobs > 1 && nprog > 1 && vl_fused_shares(progs[j], K[j])) {
                 if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j]) && (rc = g.run(st, st, dict)) != VL_OK) return rc;
                 continue;
             }
@@ -1939,19 +1969,20 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     const uint64_t call = ++calls;
     uint64_t job = 0;
     // short jobs of different programs share launches (64 programs of one call: 2 launches instead of 64)
-    std::vector<uint8_t> shared(nprog, 0);
+    std::vector<uint8_t> shares(nprog, 0);  // may share a launch
+    for (uint32_t j = 0; j < nprog && nprog > 1; ++j) shares[j] = K[j] != 0 && vl_fused_shares(progs[j], K[j]);
     FusedGroup g;
-    for (uint32_t j = 0; j < nprog && nprog > 1 && rc == VL_OK; ++j) {
-        if (K[j] == 0 || !vl_fused_shares(progs[j], K[j])) continue;
-        shared[j] = 1;
+    const Together how = nprog > 1 ? together(nprog, progs, K, shares) : SINGLE;
+    for (uint32_t j = 0; j < nprog && how == SHARED && rc == VL_OK; ++j) {
+        if (!shares[j]) continue;
         if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j])) rc = g.run(st, lane[job++ % L], dict);
     }
     if (rc == VL_OK && g.n) rc = g.run(st, lane[job++ % L], dict);
     for (uint32_t j = 0; j < nprog && rc == VL_OK; ++j) {
         if (K[j] == 0) continue;
         vl_program *p = progs[j];
-        if (shared[j]) continue;
-        if (vl_fused_wanted(p, K[j])) {
+        if (how == SHARED && shares[j]) continue;
+        if (!(how == BATCHED && shares[j]) && vl_fused_wanted(p, K[j])) {
             rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, st, lane[job % L], dict, (int)(job % L));
             ++job;
             continue;

@@ -281,3 +281,28 @@ def test_kernel_times_of_short_jobs(B, K):
         assert ms[1] < ms[0] and ms[2] < ms[0] and ms[3] > 0.004
     for gp in gps:
         gp.close()
+
+
+@pytest.mark.parametrize("shape,n,K", [("gemm", 9, 20), ("attention", 2, 50), ("nested", 8, "sms"), ("mixed", 12, 60)])
+def test_short_jobs_of_several_programs(B, oracle_mod, shape, n, K):
+    """Jobs that share a launch (many of small programs), take one each (few of larger ones), or go to the batched kernels
+    (many rows of large programs); small and large ones together, some without rows."""
+    K = _sm_count() if K == "sms" else K
+    shapes = {"gemm": [synth.shape_gemm()], "attention": [synth.shape_attention()], "nested": [synth.shape_stress(20000, 6000)],
+              "mixed": [synth.shape_tiny(), synth.shape_gemm(), synth.shape_attention()]}[shape]
+    cases = []
+    for j, s in enumerate(shapes):
+        p = synth.build_program(s, j)
+        rows = synth.candidate_rows(p, K, 0.3, 60 + j)[0]
+        op = oracle_mod.OracleProgram(p)
+        cases.append((p, rows, op.verify(op.liveness(), rows)))
+    use = [cases[j % len(cases)] for j in range(n)]
+    gps = [B.Program(p) for p, _, _ in use]
+    devs = [_to_dev(rows[: 0 if j == n // 2 and n > 2 else K]) for j, (_, rows, _) in enumerate(use)]
+    for call in range(2):
+        B.vl_liveness_batch(gps)
+        outs = B.vl_verify_batch(gps, devs)
+        for j, (o, (_, _, want)) in enumerate(zip(outs, use)):
+            _assert_same(B.verdicts_to_numpy(o), want[: o.shape[0]], f"call {call} program {j}")
+    for gp in gps:
+        gp.close()
