@@ -228,7 +228,7 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
         p->nD8 = std::max(8u, (p->nD + 7) / 8 * 8);
         p->nDT = (p->nD8 + 4095u) / 4096u * 4096u + 4096u;
         std::vector<uint16_t> v16((size_t)p->nD8 + 8, (uint16_t)p->V);
-        std::vector<uint64_t> slot((size_t)p->nD8 / 8, 0);
+        std::vector<uint8_t> f8((size_t)p->nD8 / 8, 0);
         std::vector<uint4> off((size_t)p->nDT / 4, make_uint4(p->V * 16u, p->V * 16u, p->V * 16u, p->V * 16u));
         std::vector<uint8_t> f4((size_t)p->nDT / 4, 0);
         dict_instr.resize(p->nD8, 0);
@@ -240,13 +240,13 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
                 uint32_t *w = &off[e2 / 4].x;
                 w[e2 % 4] = v * 16u;
                 if (is_first[e2]) first_entry[v] = e2;
-                if (is_first[e2]) { slot[e2 / 8] |= 1ull << (e2 % 8); f4[e2 / 4] |= (uint8_t)(1u << (e2 % 4)); }
+                if (is_first[e2]) { f8[e2 / 8] |= (uint8_t)(1u << (e2 % 8)); f4[e2 / 4] |= (uint8_t)(1u << (e2 % 4)); }
             } else {
-                slot[e2 / 8] |= 1ull << (e2 % 8);  // padding column: writes the spare table entry, never compared
+                f8[e2 / 8] |= (uint8_t)(1u << (e2 % 8));  // padding column: writes the spare table entry, never compared
             }
         }
         up.add(&p->d_dict_vreg16, v16.data(), v16.size());
-        up.add(&p->d_dict_slotmeta, slot.data(), slot.size());
+        up.add(&p->d_dict_first8, f8.data(), f8.size());
         up.add(&p->d_dict_opoff, off.data(), off.size());
         up.add(&p->d_dict_first4, f4.data(), f4.size());
         up.add(&p->d_dict_first_occ, first_entry.data(), first_entry.size());

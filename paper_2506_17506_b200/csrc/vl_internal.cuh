@@ -115,20 +115,19 @@ struct vl_program {
 
     // tables consumed by the verify kernels
     uint16_t *d_vreg16 = nullptr;           // [nOp8 + 8] vreg id per operand (padding operands: id V)
-    uint64_t *d_slotmeta = nullptr;         // [nOp8 / 8] per 8 operands: first-occurrence bits, bank compare masks
+    uint8_t *d_first8 = nullptr;            // [nOp8 / 8] per 8 operands: first-occurrence bits
     // the same tables for rows in dictionary form (one column per (block, vreg of the block)); made once,
     // when the handle is created
     uint32_t nD = 0, nD8 = 0, nDT = 0;  // entries; rounded up to 8 (at least 8); to whole tiles plus one
     std::vector<uint32_t> h_dict_off, h_dict_vreg;
     uint16_t *d_dict_vreg16 = nullptr;
-    uint64_t *d_dict_slotmeta = nullptr;
+    uint8_t *d_dict_first8 = nullptr;
     uint4 *d_dict_opoff = nullptr;
     uint8_t *d_dict_first4 = nullptr;
     uint32_t *d_dict_first_occ = nullptr; // [V] first entry of the vreg, 0xFFFFFFFF if none
     uint32_t *d_dict_instr = nullptr;     // [nD8] first instruction of the entry's block that touches its vreg
     uint4 *d_opoff = nullptr;               // [nOpT / 4] per 4 operands: byte offsets of their vregs' 16-byte table entries
     uint8_t *d_first4 = nullptr;            // [nOpT / 4] per 4 operands: first-occurrence bits
-    uint8_t *d_opmeta = nullptr;            // [nO] scratch of the first run
     uint8_t *d_opflags = nullptr;           // [nO]
     uint32_t *d_first_occ = nullptr;        // [V] first operand that names v, 0xFFFFFFFF if none
     uint32_t *d_first_def_instr = nullptr;  // [V] lowest instruction defining v, 0xFFFFFFFF if none

@@ -630,8 +630,7 @@ __global__ void __launch_bounds__(OFF_NT) k_offsets(const __grid_constant__ Live
     }
 }
 
-// Per instruction: vreg id per operand (16 bit), first occurrence / first definition of every
-// vreg, and the bank-compare distances of every read.
+// First occurrence and first definition of every vreg.
 __global__ void k_first_occ(uint32_t nI, const uint32_t *__restrict__ op_off, const uint8_t *__restrict__ ndefs,
                             const uint32_t *__restrict__ op_vreg, uint32_t *first_occ, uint32_t *first_def_instr)
 {
@@ -653,60 +652,24 @@ __global__ void k_vreg_info(uint32_t V, const uint8_t *__restrict__ width, const
                (first_def_instr[v] != 0xFFFFFFFFu ? VINFO_DEFINED : 0u);
 }
 
-__global__ void k_operand_meta(uint32_t nI, const uint32_t *__restrict__ op_off, const uint8_t *__restrict__ ndefs,
-                               const uint32_t *__restrict__ op_vreg, const uint32_t *__restrict__ first_occ,
-                               const uint8_t *__restrict__ opflags, uint16_t *vreg16, uint8_t *opmeta,
-                               uint32_t *status)
-{
-    const uint32_t i = blockIdx.x * NT + threadIdx.x;
-    if (i >= nI) return;
-    const uint32_t o0 = op_off[i], o1 = op_off[i + 1], nd = ndefs[i];
-    for (uint32_t o = o0; o < o1; ++o) {
-        const uint32_t v = op_vreg[o];
-        uint8_t m = (first_occ[v] == o) ? 1 : 0;
-        if (o >= o0 + nd && !(opflags[o] & OPF_DUP)) {
-            const uint32_t u = o - (o0 + nd);  // reads of this instruction before this one
-            if (u >= 1) m |= 2;
-            if (u >= 2) m |= 4;
-            if (u >= 3) m |= 8;
-        }
-        vreg16[o] = (uint16_t)v;
-        opmeta[o] = m;
-    }
-}
-
-// Per 8 operands: bits 0..7 first occurrence; for d = 1..3 a 16-bit field at 8 + 16 (d-1) with
-// bit 2 j set when operand j compares its bank with the operand d places before it.
-// Also the operand metadata of the eight-candidate table kernel, per four operands: the byte offsets
-// of the vregs' 16-byte table entries and a nibble of first-occurrence bits; there, operands beyond
-// n_operands (the arrays are padded to whole tiles) name the spare entry V and are never a first
+// Vreg id per operand (16 bit), a byte of first-occurrence bits per 8 operands, and the operand metadata of the eight-candidate
+// table kernel, per four operands: the byte offsets of the vregs' 16-byte table entries and a nibble of first-occurrence bits;
+// there, operands beyond n_operands (the arrays are padded to whole tiles) name the spare entry V and are never a first
 // occurrence.  One thread per 8 operands of the padded arrays.
-__global__ void k_pack_slots(uint32_t nO, uint32_t nOp8, uint32_t n_slots_padded, uint32_t V,
-                             const uint8_t *__restrict__ opmeta, uint16_t *vreg16, uint64_t *slotmeta, uint4 *opoff,
-                             uint8_t *first4)
+__global__ void k_operand_tables(uint32_t nO, uint32_t nOp8, uint32_t n_padded, uint32_t V, const uint32_t *__restrict__ op_vreg,
+                                 const uint32_t *__restrict__ first_occ, uint16_t *vreg16, uint8_t *first8, uint4 *opoff, uint8_t *first4)
 {
     const uint32_t s = blockIdx.x * NT + threadIdx.x;
-    if (s >= n_slots_padded) return;
-    uint64_t m = 0;
-    uint32_t off[8], f = 0;
+    if (s >= n_padded) return;
+    uint32_t off[8], f = 0, padding = 0;
     for (uint32_t j = 0; j < 8; ++j) {
-        const uint32_t o = s * 8 + j;
-        off[j] = V * 16u;
-        if (o >= nO) {
-            if (o < nOp8) {
-                vreg16[o] = (uint16_t)V;  // padding operand: writes the spare table entry, never compared
-                m |= 1ull << j;
-            }
-            continue;
-        }
-        off[j] = (uint32_t)vreg16[o] * 16u;
-        const uint8_t x = opmeta[o];
-        if (x & 1) { m |= 1ull << j; f |= 1u << j; }
-        if (x & 2) m |= 1ull << (8 + 2 * j);
-        if (x & 4) m |= 1ull << (24 + 2 * j);
-        if (x & 8) m |= 1ull << (40 + 2 * j);
+        const uint32_t o = s * 8 + j, v = o < nO ? op_vreg[o] : V;
+        off[j] = v * 16u;
+        if (o < nO) f |= (first_occ[v] == o ? 1u : 0u) << j;
+        else padding |= 1u << j;  // a padding operand writes the spare table entry and is never compared
+        if (o < nOp8) vreg16[o] = (uint16_t)v;
     }
-    if (s < nOp8 / 8) slotmeta[s] = m;
+    if (s < nOp8 / 8) first8[s] = (uint8_t)(f | padding);
     opoff[2 * s] = make_uint4(off[0], off[1], off[2], off[3]);
     opoff[2 * s + 1] = make_uint4(off[4], off[5], off[6], off[7]);
     first4[2 * s] = (uint8_t)(f & 15u);
@@ -972,7 +935,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     VL_CUDA(p, cudaDeviceSynchronize());  // earlier work (on any stream) may still read the old layout
     p->layout_arena.reset();
     p->tables_built = false;
-    p->d_vreg16 = nullptr; p->d_slotmeta = nullptr; p->d_opoff = nullptr; p->d_first4 = nullptr;
+    p->d_vreg16 = nullptr; p->d_first8 = nullptr; p->d_opoff = nullptr; p->d_first4 = nullptr;
     p->d_first_def_instr = nullptr; p->d_vinfo = nullptr; p->d_first_occ = nullptr;
     std::vector<uint32_t> c_i0, c_i1, c_blk, blk_c_off(nB + 1, 0), p_i0, p_chunk, c_p_off, seg_c0, blk_seg_off(nB + 1, 0);
     for (uint32_t b = 0; b < nB; ++b) {
@@ -1096,7 +1059,7 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
         LAYOUT(&p->d_first_def_instr, (size_t)V);
         LAYOUT(&p->d_first_occ, (size_t)V);
         LAYOUT(&p->d_vreg16, (size_t)p->nOp8 + 8);
-        LAYOUT(&p->d_slotmeta, (size_t)p->nOp8 / 8);
+        LAYOUT(&p->d_first8, (size_t)p->nOp8 / 8);
         LAYOUT(&p->d_first4, (size_t)p->nOpT / 4);
         LAYOUT(&p->d_vinfo, (size_t)V);
         LAYOUT(&p->d_opoff, (size_t)p->nOpT / 4);
@@ -1144,7 +1107,6 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
         flow_smem = 0;
     }
     if (!p->tables_built) {
-        KEEP(&p->d_opmeta, (size_t)nO);
         VL_CUDA(p, cudaMemsetAsync(p->d_first_occ, 0xFF, std::max<size_t>(V, 1) * 4, st));
         VL_CUDA(p, cudaMemsetAsync(p->d_first_def_instr, 0xFF, std::max<size_t>(V, 1) * 4, st));
     }
@@ -1203,10 +1165,8 @@ static int live_tables(vl_program *p, cudaStream_t st)
     LAUNCH(k_first_occ, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
            p->d_first_def_instr);
     LAUNCH(k_vreg_info, (V + NT - 1) / NT, NT, 0, st, V, p->d_width, p->d_first_occ, p->d_first_def_instr, p->d_vinfo);
-    LAUNCH(k_operand_meta, (nI + NT - 1) / NT, NT, 0, st, nI, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_first_occ,
-           p->d_opflags, p->d_vreg16, p->d_opmeta, p->d_status);
-    LAUNCH(k_pack_slots, (p->nOpT / 8 + NT - 1) / NT, NT, 0, st, p->nO, p->nOp8, p->nOpT / 8, V, p->d_opmeta, p->d_vreg16,
-           p->d_slotmeta, p->d_opoff, p->d_first4);
+    LAUNCH(k_operand_tables, (p->nOpT / 8 + NT - 1) / NT, NT, 0, st, p->nO, p->nOp8, p->nOpT / 8, V, p->d_op_vreg, p->d_first_occ,
+           p->d_vreg16, p->d_first8, p->d_opoff, p->d_first4);
     VL_CUDA(p, cudaGetLastError());
     p->tables_built = true;
     return VL_OK;

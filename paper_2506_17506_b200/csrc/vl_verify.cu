@@ -36,7 +36,7 @@ struct TParams {
     uint32_t nI, V, nO, nOp8, P, Bmask, ntiles;
     int bank_fast;
     const uint16_t *vreg16;
-    const uint64_t *slotmeta;
+    const uint8_t *first8;
     const uint32_t *vinfo, *first_def_instr, *op_off;
     const uint2 *bank_list;
     uint32_t bank_seg[4];  // entries with n = 2, 3, 4 distinct sources: [seg[n-2], seg[n-1])
@@ -145,8 +145,6 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *tm, ui
         "l"(tm), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy)
         : "memory");
 }
-// L2 policy for data that is read once: first in line for eviction, so that it does not push out what
-// other kernels are about to read again.
 // Tiled bulk store of one box from shared memory (elements outside the tensor are not written); completion is
 // tracked by the issuing thread's bulk async-groups.
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap *tm, uint32_t x, uint32_t y, uint32_t z, const void *src)
@@ -156,17 +154,13 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *tm, uint32_t x, 
                  : "memory");
 }
 
+// L2 policy for data that is read once: first in line for eviction, so that it does not push out what
+// other kernels are about to read again.
 __device__ __forceinline__ unsigned long long l2_policy_evict_first()
 {
     unsigned long long policy;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
     return policy;
-}
-// Asks for one box of the tensor to be brought into L2.
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *tm, uint32_t x, uint32_t y, uint32_t z)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(x), "r"(y), "r"(z)
-                 : "memory");
 }
 
 // ------------------------------------------------------------- packed table access
@@ -373,7 +367,7 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
         const uint32_t o = t * TILE + tid * 8;
         if (t < q.ntiles && o < q.nOp8) {
             v4 = *reinterpret_cast<const uint4 *>(q.vreg16 + o);
-            first = (uint32_t)q.slotmeta[o >> 3] & 0xFFu;
+            first = q.first8[o >> 3];
         } else {
             v4 = make_uint4(0, 0, 0, 0);
             first = 0;
@@ -1767,7 +1761,7 @@ int run_pass(vl_program *p, const PassPlan &pp, const uint16_t *d_cand, uint64_t
     tq.nI = p->nI; tq.V = p->V; tq.nO = nO; tq.nOp8 = nOp8; tq.P = p->P; tq.Bmask = p->B - 1;
     tq.ntiles = (nOp8 + pl.NT * 8 - 1) / (pl.NT * 8);
     tq.bank_fast = p->bank_fast;
-    tq.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16; tq.slotmeta = dict ? p->d_dict_slotmeta : p->d_slotmeta;
+    tq.vreg16 = dict ? p->d_dict_vreg16 : p->d_vreg16; tq.first8 = dict ? p->d_dict_first8 : p->d_first8;
     tq.vinfo = p->d_vinfo;
     tq.entry_instr = dict ? p->d_dict_instr : nullptr;
     tq.first_def_instr = p->d_first_def_instr; tq.op_off = p->d_op_off;
