@@ -209,6 +209,7 @@ extern "C" int vl_diagnose(vl_program *p, const uint16_t *d_row, uint64_t cap, v
 }
 
 // 32 registers -> 32 bytes.  What bounds it is the store of the bytes (4 MB for 8,000 instructions and 512 registers).
+#if defined(__x86_64__)
 __attribute__((target("avx2"))) static void expand_avx2(const uint32_t *words, uint64_t n_rows, uint32_t W, uint32_t P, uint8_t *out)
 {
     typedef char v32 __attribute__((vector_size(32), aligned(1), may_alias));
@@ -229,14 +230,18 @@ __attribute__((target("avx2"))) static void expand_avx2(const uint32_t *words, u
     }
 }
 
+#endif
+
 extern "C" int vl_expand_masks(const uint32_t *words, uint64_t n_rows, uint32_t P, uint8_t *out)
 {
     if (!P || (n_rows && (!words || !out))) return VL_ERR_INVALID_ARG;
     const uint32_t W = (P + 31) / 32;
+#if defined(__x86_64__)
     if (__builtin_cpu_supports("avx2")) {
         expand_avx2(words, n_rows, W, P, out);
         return VL_OK;
     }
+#endif
     for (uint64_t i = 0; i < n_rows; ++i)
         for (uint32_t r = 0; r < P; ++r) out[i * P + r] = (uint8_t)((words[i * W + (r >> 5)] >> (r & 31)) & 1u);
     return VL_OK;
