@@ -204,16 +204,23 @@ def run_stub(args):
     return 0
 
 
+def kernels_hash():
+    """Hash of the source of the verify kernels."""
+    import hashlib
+    h = hashlib.sha256()
+    for f in ("vl_verify.cu", "vl_fused.cu", "vl_internal.cuh"):
+        h.update(open(os.path.join(ROOT, "paper_2506_17506_b200", "csrc", f), "rb").read())
+    return h.hexdigest()
+
+
 def measured_traffic(kernel_names):
     """DRAM bytes (read + write) per candidate of each verify kernel, from the profiler capture recorded in
     `profiles/dram_traffic_stress.txt`, or None when the kernels' source has changed since (the record
-    carries a hash of vl_verify.cu): a figure must not outlive the kernel it was taken from."""
-    import hashlib
+    carries a hash of it): a figure must not outlive the kernel it was taken from."""
     rec = os.path.join(ROOT, "profiles", "dram_traffic_stress.txt")
-    src = os.path.join(ROOT, "paper_2506_17506_b200", "csrc", "vl_verify.cu")
     try:
         fields = dict(line.split(":", 1) for line in open(rec).read().splitlines() if ":" in line and not line.startswith("#"))
-        if fields["vl_verify.cu sha256"].strip() != hashlib.sha256(open(src, "rb").read()).hexdigest():
+        if fields["kernels sha256"].strip() != kernels_hash():
             return None
         rows = float(fields["rows"])
         return {n: float(fields[n + " dram bytes"]) / rows for n in kernel_names if n + " dram bytes" in fields}

@@ -118,10 +118,11 @@ int vl_program_set_option(vl_program *prog, int option, uint32_t value);
  * is enqueued on an internal stream of the device, behind everything `cuda_stream` (a cudaStream_t, may be
  * NULL) holds at the call; `cuda_stream` itself is NOT made to wait for it.  A shorter program's run is
  * enqueued on `cuda_stream`.  Every call of this library that reads the
- * results waits for the run where it needs them: vl_verify* on the device (its table kernel, which
+ * results waits for the run where it needs them, whatever stream it is given: vl_verify*, vl_diagnose and
+ * vl_occupied_masks on the device (the table kernel of vl_verify, which
  * reads the candidates and the program's operand tables only, runs beside the liveness kernels;
- * the kernels after it wait), vl_liveness_result, vl_verify_host, vl_diagnose and
- * vl_occupied_masks on the host.  A caller whose own kernels read the result arrays calls
+ * the kernels after it wait; on a stream that is being captured the host waits), vl_liveness_result and
+ * vl_verify_host on the host.  A caller whose own kernels read the result arrays calls
  * vl_liveness_result after every run (it returns when the run has finished).
  * The first run of a handle (and the first after the chunk size changed) waits for the device
  * before returning, because list lengths and the status word are read back; it is the run that
@@ -138,7 +139,8 @@ int vl_liveness(vl_program *prog, void *cuda_stream);
  * runs are spread over internal streams that fork from and join back into `cuda_stream` (unlike
  * a single vl_liveness, `cuda_stream` waits for them), so that the short kernels of different
  * programs run side by side.  `progs` is HOST memory.
- * Stops at the first error and returns it.  Errors: as vl_liveness, INVALID_ARG.
+ * A handle given twice runs once.  The first error is returned: the programs in front of it have their results, those behind
+ * it keep what an earlier run left them, or stay without results.  Errors: as vl_liveness, INVALID_ARG.
  */
 int vl_liveness_batch(uint32_t n, vl_program *const *progs, void *cuda_stream);
 
@@ -165,7 +167,7 @@ int vl_liveness_result(const vl_program *prog, const uint32_t **blk_live_in, con
  * VL_OPT_LANES = 1 every kernel is enqueued on `cuda_stream` itself.
  * Host work of a call: the handle is modified (it owns the working memory of its calls).  The first
  * call on a handle, and a later one that needs larger working sets (more rows per pass, another
- * chunk size, more internal streams in use), allocates them with cudaMalloc and clears them, which
+ * chunk size, more internal streams in use, few rows after many or many after few: those are different kernels), allocates them with cudaMalloc and clears them, which
  * waits for the device: make one call of the intended size before timing or capturing.  A call that
  * fits the working sets allocates nothing and does not wait for the device, with one exception: the
  * first vl_verify* after a vl_liveness that returned early (see there) waits for that run's status
@@ -179,7 +181,7 @@ int vl_liveness_result(const vl_program *prog, const uint32_t **blk_live_in, con
  * defined by it.  Bank tally per Section 2 with B banks.
  * UNSUPPORTED: P + widest vreg > 32768; the occupancy masks of one warp of the walk,
  * (P + widest vreg + 31) / 32 words for each of 64 candidates, do not fit the shared memory of an SM
- * (P up to about 28,000 fits); or the table of one candidate, 2 (n_vregs + 1) bytes, does not.
+ * (P up to about 28,000 fits); or the table of one candidate and its bank nibbles, 4 (n_vregs + 1) bytes, do not.
  * Errors: INVALID_ARG, LIVENESS_NOT_RUN, UNSUPPORTED, CUDA.
  */
 int vl_verify(vl_program *prog, const uint16_t *d_cand, uint64_t K, uint64_t pitch_elems,
@@ -214,7 +216,7 @@ int vl_verify_dict(vl_program *prog, const uint16_t *d_dict, uint64_t K, uint64_
 /*
  * The same check for n independent programs in one call (all on the device of the
  * first program): program j checks K[j] rows of d_cand[j] into d_out[j].  The arrays of
- * pointers and sizes are HOST memory.  Stream-ordered, no synchronisation.
+ * pointers and sizes are HOST memory.  Stream-ordered, no synchronisation.  A handle may be given several times.
  */
 int vl_verify_batch(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand,
                     const uint64_t *K, const uint64_t *pitch_elems, vl_verdict *const *d_out,
@@ -297,7 +299,7 @@ int vl_resample_stats(int device, uint32_t n, const vl_verdict *const *d_out, co
  * batch_rows, in order, and stops after the first batch that holds a passing row.  *rows_checked
  * (HOST) receives the number of rows checked, a multiple of batch_rows or K; *first_pass (HOST) the
  * row of the first passing candidate, K if none passed.  Verdicts of the rows checked are in d_out
- * (16-byte aligned); those of later rows are not written.  The call waits for the stream after every
+ * (16-byte aligned); those of later rows are not written.  The call waits for the verdicts of every
  * batch (the caller needs the answer to stop sampling); the first call takes one record of
  * pinned host memory.  Errors: as vl_verify.
  */

@@ -252,7 +252,7 @@ def test_batch_call(B, oracle_mod):
         _assert_same(B.verdicts_to_numpy(o), w, f"batch member {j}")
     for gp, p in zip(gps, progs):
         _check_liveness_result(B, oracle_mod, gp, p)
-    # liveness of all members in one call, several times (the later runs are replayed recordings):
+    # liveness of all members in one call, several times (the later runs return at once):
     # same liveness results, same verdicts
     for _ in range(4):
         B.vl_liveness_batch(gps)
@@ -337,8 +337,8 @@ def test_bounded_device_wait_runs_out(B, oracle_mod):
 
 
 def test_repeated_liveness_runs(B, oracle_mod):
-    """Later liveness runs of a handle return without waiting for the GPU and are replayed from a
-    recording: the results stay those of the first run, a changed chunk size starts over, and the
+    """Later liveness runs of a handle return without waiting for the GPU, with the lengths
+    of the first: the results stay those of the first run, a changed chunk size starts over, and the
     verdicts computed behind an unsettled run are right."""
     wl = synth.workload(1)
     p = synth.build_program(wl.shapes[0], wl.seeds[0])

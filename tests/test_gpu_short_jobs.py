@@ -35,11 +35,15 @@ def test_random_programs(B, oracle_mod, P, chunk):
 
 
 @pytest.mark.parametrize("chunk", [160, 8])
-@pytest.mark.parametrize("K", [1, 148, 149, 297])
-def test_row_counts_and_many_short_chunks(B, oracle_mod, K, chunk):
-    """Attention-shaped program with one row per multiprocessor, two, and too many for the path; and with more short
-    chunks (1,000) than a thread block has threads."""
-    wl = synth.workload(2)
+@pytest.mark.parametrize("shape", ["gemm", "attention"])
+@pytest.mark.parametrize("per_sm,more", [(0, 1), (1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1), (5, 0)])
+def test_row_counts_and_many_short_chunks(B, oracle_mod, per_sm, more, shape, chunk):
+    """One, two and three rows per multiprocessor and one row more, for a program of 2,000 instructions (whose rows count their
+    own collisions, in several rounds beyond three) and one of 8,000 (which hands them over from the second row per
+    multiprocessor on, and takes the batched kernels beyond three); and with more short chunks (1,000) than a thread block
+    has threads."""
+    K = per_sm * _sm_count() + more
+    wl = synth.workload({"gemm": 1, "attention": 2}[shape])
     p = synth.build_program(wl.shapes[0], wl.seeds[0])
     rows, _ = synth.candidate_rows(p, K, 0.5, 77)
     rows[: K // 10] = _garbage_rows(p, K, 3)[: K // 10]

@@ -177,3 +177,34 @@ def test_a_later_batch_of_other_handles_is_not_waited_for(B, oracle_mod):
     for gp in mine[1:] + theirs:
         assert B.verdicts_to_numpy(gp.vl_verify(dev)).tobytes() == op.verify(op.liveness(), rows).tobytes()
         gp.close()
+
+
+@pytest.mark.parametrize("kind", ["short", "long"])
+@pytest.mark.parametrize("same_stream", [False, True])
+def test_capture_behind_a_run_in_flight(B, oracle_mod, kind, same_stream):
+    """A call that is captured while a liveness run is in flight: the host waits for the run, the graph can be launched."""
+    import torch
+    p = _program(kind)
+    gp = B.Program(p)
+    rows = _garbage_rows(p, 30, 8)
+    dev = _to_dev(rows)
+    out = torch.zeros((len(rows), 4), dtype=torch.int32, device="cuda")
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    gp.vl_liveness(s1)
+    gp.vl_verify(dev, out, s1)
+    torch.cuda.synchronize()
+    out.zero_()
+    torch.cuda.synchronize()
+    s = s1 if same_stream else s2
+    gp.vl_liveness(s1)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):
+        gp.vl_verify(dev, out, s)
+    op = oracle_mod.OracleProgram(p)
+    want = op.verify(op.liveness(), rows)
+    for _ in range(2):
+        out.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert B.verdicts_to_numpy(out).tobytes() == want.tobytes()
+    gp.close()
