@@ -121,7 +121,7 @@ int vl_program_set_option(vl_program *prog, int option, uint32_t value);
  * results waits for the run where it needs them, whatever stream it is given: vl_verify*, vl_diagnose and
  * vl_occupied_masks on the device (the table kernel of vl_verify, which
  * reads the candidates and the program's operand tables only, runs beside the liveness kernels;
- * the kernels after it wait; on a stream that is being captured the host waits), vl_liveness_result and
+ * the kernels after it wait; on a stream that is being captured, in relaxed mode, the host waits), vl_liveness_result and
  * vl_verify_host on the host.  A caller whose own kernels read the result arrays calls
  * vl_liveness_result after every run (it returns when the run has finished).
  * The first run of a handle (and the first after the chunk size changed) waits for the device

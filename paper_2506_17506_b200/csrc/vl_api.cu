@@ -453,12 +453,13 @@ extern "C" int vl_liveness(vl_program *p, void *stream)
 int vl_live_join(vl_program *p, cudaStream_t from, cudaStream_t st)
 {
     if (!p->live_pending) return VL_OK;
+    // a capture can neither wait for what is not part of it nor be asked for its stream's id
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    VL_CUDA(p, cudaStreamIsCapturing(st, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return vl_live_settle(p);
     unsigned long long id = 0;
     VL_CUDA(p, cudaStreamGetId(from, &id));
     if (id == p->live_stream) return VL_OK;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    VL_CUDA(p, cudaStreamIsCapturing(st, &cs));
-    if (cs != cudaStreamCaptureStatusNone) return vl_live_settle(p);  // (a capture cannot wait for what is not part of it)
     VL_CUDA(p, cudaStreamWaitEvent(st, p->live_done->ev, 0));
     return VL_OK;
 }
