@@ -166,6 +166,8 @@ extern "C" int vl_program_create(const vl_program_desc *d, int device, vl_progra
     for (uint32_t v = 0; v < p->V; ++v) p->wmax = std::max<uint32_t>(p->wmax, d->vreg_width[v]);
     p->h_blk_off.assign(d->block_instr_off, d->block_instr_off + p->nB + 1);
     p->h_op_off.assign(d->instr_op_off, d->instr_op_off + p->nI + 1);
+    p->h_succ_off.assign(d->succ_off, d->succ_off + p->nB + 1);
+    if (p->nE) p->h_succ.assign(d->succ, d->succ + p->nE);
 
     Upload up;
     up.add(&p->d_blk_off, d->block_instr_off, (size_t)p->nB + 1);

@@ -94,9 +94,10 @@ struct vl_program {
     // pieces of one chunk; segments: runs of chunks of one block
     uint32_t nC = 0, nP = 0, nS = 0, nSeg = 0;
     uint32_t short_len = 1;  // instructions of the longest short chunk
-    bool wide_pieces = false;  // some piece has many operands (WIDE_OPERANDS, vl_liveness.cu)
+    uint32_t share_pieces = 0, share_ops = 0;  // pieces and operands of the largest share of a thread block of k_small
+    bool wide_pieces = false;  // some piece is an instruction of many operands (PIECE_OPERANDS, vl_liveness.cu)
     uint32_t layout_chunk_instrs = 0;  // chunk size the device copies of the layout were made for (0: none)
-    std::vector<uint32_t> h_blk_off, h_op_off;
+    std::vector<uint32_t> h_blk_off, h_op_off, h_succ_off, h_succ;
     // list lengths of the last liveness run with this layout: the next run allocates from them
     bool sizes_known = false;
     unsigned long long known[6] = {0, 0, 0, 0, 0, 0};  // list entries, walk events, through-set entries, short-list entries, short-chunk events and entries
@@ -106,8 +107,9 @@ struct vl_program {
     uint32_t *d_blk_off = nullptr, *d_succ_off = nullptr, *d_succ = nullptr, *d_op_off = nullptr, *d_op_vreg = nullptr;
     uint8_t *d_ndefs = nullptr, *d_width = nullptr;
     uint32_t *d_chunk_i0 = nullptr, *d_chunk_i1 = nullptr, *d_chunk_blk = nullptr, *d_blk_chunk_off = nullptr;
-    uint32_t *d_piece_i0 = nullptr, *d_piece_chunk = nullptr, *d_chunk_piece_off = nullptr;
+    uint32_t *d_piece_i0 = nullptr, *d_piece_o0 = nullptr, *d_op_word = nullptr, *d_piece_chunk = nullptr, *d_chunk_piece_off = nullptr;
     uint32_t *d_seg_c0 = nullptr, *d_blk_seg_off = nullptr, *d_short_p0 = nullptr, *d_chunk_short_off = nullptr, *d_short_blk = nullptr, *d_short_i0 = nullptr, *d_blk_short_off = nullptr, *d_short_chunk = nullptr;
+    uint4 *d_share = nullptr;
 
     // liveness results
     uint32_t *d_blk_in = nullptr, *d_blk_out = nullptr, *d_lo_off = nullptr, *d_lo = nullptr;

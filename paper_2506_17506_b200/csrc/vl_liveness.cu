@@ -2,7 +2,7 @@
 //
 // Every block is cut into chunks (the unit of the verify walk), every chunk into pieces of at most
 // PIECE_INSTRS instructions (the unit of the instruction-level work here), and runs of pieces of one chunk
-// form short chunks (the unit of the one-candidate walk).  A run is five launches:
+// form short chunks (the unit of the one-candidate walk).  A run of a longer program is five launches:
 //   k_sets     read/write bitsets of every piece, composed to its chunk's (one thread block per chunk)
 //   k_flow     per 32 words of the bitsets: block sets, fixed point over the blocks, live sets at the
 //              chunk boundaries (bitset words are independent of each other)
@@ -11,39 +11,78 @@
 //   k_offsets  through-sets, entry counts; the last thread block makes every offset and leaves the totals
 //              and the status word in pinned host memory
 //   k_fill     live-after lists in CSR form, walk events, through-set lists, side by side in one grid
+// and of a program of up to LIVE_SMALL_INSTRS instructions two: k_small (the first four by one cluster) and k_fill.
 // What bounds a run is the chain of launches and of L2 round trips inside them, not the bytes (34 MB of
-// lists for 32,000 instructions).  The 17 launches (a recorded graph) that did the same before spent most of
-// their time on launch latency and on one-thread loops over an instruction's operands; here the lanes of a
-// warp take the operands of a piece, and a kernel's blocks start while the kernel before it drains.
-// Liveness + vl_verify of 100 rows: 98 -> 65 us for 64 instructions, 122 -> 96 us for 2,000.
+// lists for 32,000 instructions): the lanes of a warp take the operands of a piece, and a kernel's blocks start while the
+// kernel before it drains.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "vl_internal.cuh"
 
 #define NT 128  // threads per block of the operand-table kernels
-#define PIECE_INSTRS 8
+#define PIECE_INSTRS 8         // instructions of a piece, at most
 #define PC_WARPS 20            // warps per block of k_sets and k_count: the pieces of a chunk of the default size at once
 #define PC_NT (PC_WARPS * 32)
-#define WIDE_OPERANDS 96       // operands of a piece from which k_count takes it instruction by instruction: 200
-                               // instructions of 60 reads 172 us for the run against 976, 100 of 100 definitions 202 against 2,133
+#define PIECE_OPERANDS 32      // and its operands, unless it is a single instruction: one per lane
 #define LV_WARPS 8             // warps per block of k_fill
 #define LV_NT (LV_WARPS * 32)
+#define FILL_WARP_WORDS (32 + 1024 + 256)  // shared memory of a warp of k_fill behind its two bitsets
 #define FLOW_WARPS 16          // warps per block of k_flow
 #define OFF_NT 256             // threads per block of k_offsets
 #define SEG_CHUNKS 8           // chunks that a warp of k_flow composes in one go (longer in very long programs)
 #define SHORT_CHUNKS 512       // short chunks per program aimed at: the threads of one block of the one-candidate walk
 
-// Everything the five kernels of a run read and write.
+#define SMALL_NT 512
+#define SMALL_WARPS (SMALL_NT / 32)
+#define SMALL_BLOCKS 8         // thread blocks of a cluster (the portable size)
+#define SMALL_ONE_PIECES 32    // pieces up to which one thread block takes the program
+#define SMALL_SMEM (160 * 1024)   // shared memory of a thread block, at most
+#define LIVE_SMALL_INSTRS 4096    // instructions of a program, at most
+
+// Where the parts of a block's shared memory begin in k_small, in words, and how much there is.  (Made on the host: the kernel
+// reads them as constants; computed there, from seven numbers, they cost more instructions than the work between them.)
+struct SmallSmem {
+    uint16_t clo, pi, po, pc, xs, fl, pu, pd, cu, cd, bu, bd, bi, bo, bt, lo, ev, plo, pev, cev, cent, sent, sev, thn, rd;
+    uint16_t tab, tab_words, blk_chunk, chunk_piece, chunk_blk, chunk_short, short_piece, short_chunk, blk_off, succ_off, succ;  // layout tables
+    // bytes; pieces, ops: of the largest share
+    uint32_t init(uint32_t nB, uint32_t nE, uint32_t nC, uint32_t nS, uint32_t Wv, uint32_t pieces, uint32_t ops)
+    {
+        uint64_t at = 0;
+        auto take = [&](uint64_t n) { const uint64_t x = at; at += (n + 1) & ~1ull; return (uint16_t)x; };
+        clo = take(2 * nC);                                          // list entries per chunk (64 bit)
+        tab = take(0);
+        // (side by side, as vl_layout has them)
+        auto table = [&](uint64_t n) { const uint64_t x = at; at += (n + 4) & ~3ull; return (uint16_t)x; };
+        blk_chunk = table(nB + 1); chunk_piece = table(nC + 1); chunk_blk = table(nC); chunk_short = table(nC + 1); short_piece = table(nS);
+        short_chunk = table(nS); blk_off = table(nB + 1); succ_off = table(nB + 1); succ = table(nE);
+        tab_words = (uint16_t)(at - tab);
+        pi = take(pieces + 1); po = take(pieces + 1); pc = take(pieces);  // first instructions and operands of the share's pieces, their chunks
+        xs = take(ops); fl = take((ops + 3) / 4);                    // operands and their flags (a byte each)
+        const uint64_t PW = (uint64_t)pieces * Wv, CW = (uint64_t)nC * Wv, BW = (uint64_t)nB * Wv;
+        pu = take(PW); pd = take(PW);                                // sets of the share's pieces; pu: then live after the piece
+        cu = take(CW); cd = take(CW);                                // sets of every chunk; cu: then live before the chunk
+        bu = take(BW); bd = take(BW); bi = take(BW); bo = take(BW); bt = take(BW);  // of every block; bt: touched
+        lo = take(pieces * PIECE_INSTRS); ev = take(pieces * PIECE_INSTRS);  // per instruction: entries and events before it in its piece
+        plo = take(pieces); pev = take(pieces);                      // of the pieces; then before them in their chunk
+        cev = take(nC); cent = take(nC); sent = take(nS); sev = take(nS); thn = take(nB);
+        rd = take((uint64_t)SMALL_WARPS * Wv);                       // a set per warp, for pieces of more than 32 operands
+        return at > SMALL_SMEM / 4 ? 0xFFFFFFFFu : (uint32_t)at * 4;
+    }
+};
+
+// Everything the kernels of a run read and write.
 struct LiveArgs {
     uint32_t nB, nI, V, nE, Wv, nC, nP, nS, nSeg;
     int use_th, wide_smem;
     // program and layout
     const uint32_t *op_off, *op_vreg, *succ_off, *succ, *blk_off;
     const uint8_t *ndefs, *width;
-    const uint32_t *chunk_i0, *chunk_i1, *chunk_blk, *blk_chunk_off, *piece_i0, *piece_chunk, *chunk_piece_off;
+    const uint32_t *chunk_i0, *chunk_i1, *chunk_blk, *blk_chunk_off, *piece_i0, *piece_o0, *op_word, *piece_chunk, *chunk_piece_off;
     const uint32_t *seg_c0, *blk_seg_off;         // segments of k_flow: runs of chunks of one block
     const uint32_t *short_p0, *chunk_short_off;   // short chunks: first piece of each; short chunks of every chunk
     // working sets
@@ -54,6 +93,9 @@ struct LiveArgs {
     uint32_t *centry_cnt, *short_ent, *short_ev;  // entry events per chunk, per short chunk; other events per short chunk
     uint32_t *flow_scratch;                       // k_flow's working set when it does not fit shared memory
     uint32_t *counters;                           // [0] blocks of k_offsets that have finished
+    const uint4 *share;                           // k_small: shares of the thread blocks, tables for shared memory
+    const uint32_t *small_tab;
+    SmallSmem small;
     // results
     uint32_t *blk_in, *blk_out, *lo_off, *lo, *ls, *ls_adj, *blk_th, *th_cnt, *th_off, *th, *cev_off, *sev_off, *sev, *sen_off, *sen;
     uint8_t *opflags;
@@ -107,40 +149,61 @@ __device__ T block_excl_scan(T x, T *s_scan, T *total)
     return s_scan[w] + inc - x;
 }
 
-// The operands of a piece, one per lane and round of 32: vreg (16 bits), instruction inside the piece
-// (4 bits at 16), definition (bit 20).  Lanes beyond the piece hold 0xFFFFFFFF.
-struct PieceOps {
-    uint32_t ob, n, off;  // first operand, operands; lane k <= instructions of the piece: operand offset of instruction k
-    uint32_t nd, ni;      // lane k: definitions of instruction k; instructions
-    __device__ __forceinline__ void init(const LiveArgs &q, uint32_t p, uint32_t c, uint32_t lane)
+// An operand of a piece as a word: vreg (16 bits), instruction inside the piece (4 bits at 16), and how it meets the piece's
+// other operands, which the layout of the program fixes (k_operand_words; found anew in every run, by shuffles or matches of
+// a warp's lanes, it took k_sets and k_count half of their time).  In a piece that is a single instruction of more than
+// PIECE_OPERANDS operands only OW_DEF and OW_EXPOSED are set.
+enum : uint32_t {
+    OW_DEF = 1u << 20,      // definition
+    OW_DUP = 1u << 21,      // read: an earlier read of the instruction has the vreg
+    OW_OTHER = 1u << 22,    // the instruction's other side (reads / writes) has the vreg
+    OW_EXPOSED = 1u << 23,  // read: no earlier instruction of the piece writes the vreg
+    OW_LATER = 1u << 24,    // a later instruction of the piece touches the vreg ...
+    OW_READ = 1u << 25,     // ... and the first such reads it
+    OW_MANY = 1u << 26      // the instruction has several definitions
+};
+struct Piece {
+    uint32_t i0, ni, o0, n;  // first instruction, instructions; first operand, operands
+    __device__ __forceinline__ void init(const LiveArgs &q, uint32_t p)
     {
-        const uint32_t i0 = q.piece_i0[p], i1 = min(i0 + PIECE_INSTRS, q.chunk_i1[c]);
-        ni = i1 - i0;
-        off = lane <= ni ? q.op_off[i0 + lane] : 0xFFFFFFFFu;
-        nd = lane < ni ? q.ndefs[i0 + lane] : 0u;
-        ob = __shfl_sync(0xffffffffu, off, 0);
-        n = __shfl_sync(0xffffffffu, off, ni) - ob;
+        i0 = q.piece_i0[p];
+        o0 = q.piece_o0[p];
+        ni = q.piece_i0[p + 1] - i0;
+        n = q.piece_o0[p + 1] - o0;
     }
-    __device__ __forceinline__ uint32_t get(const LiveArgs &q, uint32_t j) const  // (every lane of the warp)
-    {
-        const uint32_t o = ob + j;
-        uint32_t k = 0, first = ob, nd_k = __shfl_sync(0xffffffffu, nd, 0);
-        for (uint32_t u = 1; u < ni; ++u) {
-            const uint32_t f = __shfl_sync(0xffffffffu, off, u), d = __shfl_sync(0xffffffffu, nd, u);
-            if (f <= o) { k = u; first = f; nd_k = d; }
-        }
-        return j < n ? (q.op_vreg[o] | (k << 16) | (o - first < nd_k ? 1u << 20 : 0u)) : 0xFFFFFFFFu;
-    }
+    // operand j of the piece, 0 beyond it
+    __device__ __forceinline__ uint32_t get(const LiveArgs &q, uint32_t j) const { return j < n ? q.op_word[o0 + j] : 0u; }
 };
 __device__ __forceinline__ uint32_t po_vreg(uint32_t x) { return x & 0xFFFFu; }
 __device__ __forceinline__ uint32_t po_instr(uint32_t x) { return (x >> 16) & 15u; }
-__device__ __forceinline__ bool po_def(uint32_t x) { return (x >> 20) & 1u; }
+__device__ __forceinline__ bool po_def(uint32_t x) { return x & OW_DEF; }
+__device__ __forceinline__ uint32_t low_bits(uint32_t n) { return n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u; }
+
+// Lanes whose operand belongs to the same instruction (every lane of the warp; 4 ballots at 26 cycles each, a match
+// instruction takes 380 cycles alone and 1,080 beside 15 other warps).
+__device__ __forceinline__ uint32_t same_instr(uint32_t x, bool mine)
+{
+    uint32_t same = __ballot_sync(0xffffffffu, mine);
+#pragma unroll
+    for (int j = 16; j < 19; ++j) {
+        const uint32_t bit = __ballot_sync(0xffffffffu, (x >> j) & 1u);
+        same &= (x >> j) & 1u ? bit : ~bit;
+    }
+    return same;
+}
 
 // ============================================================================ k_sets
-// One thread block per chunk.  use = vregs read before any write inside the piece (the chunk), def = vregs
-// written.  A lane holds an operand and meets the piece's other operands by shuffles; WIDE (some piece of the launch has
-// many operands): a piece of more than 32 is taken instruction by instruction.
-template <int N, bool WIDE>
+// One thread block per chunk.  use = vregs read before any write inside the piece (the chunk), def = vregs written.
+// Read and write sets of one piece, into empty bitsets of shared memory (a warp; x: its first 32 operands, one per lane).
+__device__ __forceinline__ void piece_sets(const LiveArgs &q, const Piece &po, uint32_t x, uint32_t lane, uint32_t *s_use, uint32_t *s_def)
+{
+    for (uint32_t j = lane; j < po.n; j += 32) {
+        const uint32_t y = j == lane ? x : po.get(q, j);
+        if (y & (OW_DEF | OW_EXPOSED)) atomicOr(&(po_def(y) ? s_def : s_use)[po_vreg(y) >> 5], 1u << (y & 31));
+    }
+}
+
+template <int N>
 __global__ void __launch_bounds__(PC_NT) k_sets(const __grid_constant__ LiveMany<N> a)
 {
     LIVE_ARGS;
@@ -156,39 +219,12 @@ __global__ void __launch_bounds__(PC_NT) k_sets(const __grid_constant__ LiveMany
     uint32_t *s_use = sm + (size_t)warp * 2 * q.Wv, *s_def = s_use + q.Wv;
     const uint32_t p0 = q.chunk_piece_off[c], p1 = q.chunk_piece_off[c + 1];
     for (uint32_t p = p0 + warp; p < p1; p += blockDim.x / 32) {
+        Piece po;
+        po.init(q, p);
+        const uint32_t x = po.get(q, lane);
         for (uint32_t w = lane; w < 2 * q.Wv; w += 32) s_use[w] = 0;
-        PieceOps po;
-        po.init(q, p, c, lane);
         __syncwarp();
-        if (WIDE && po.n > 32) {
-            for (uint32_t k = 0; k < po.ni; ++k) {
-                const uint32_t o0 = __shfl_sync(0xffffffffu, po.off, k), o1 = __shfl_sync(0xffffffffu, po.off, k + 1);
-                const uint32_t r0 = o0 + __shfl_sync(0xffffffffu, po.nd, k);
-                for (uint32_t o = r0 + lane; o < o1; o += 32) {
-                    const uint32_t v = q.op_vreg[o];
-                    if (!bit_get(s_def, v)) atomicOr(&s_use[v >> 5], 1u << (v & 31));
-                }
-                __syncwarp();
-                for (uint32_t o = o0 + lane; o < r0; o += 32) atomicOr(&s_def[q.op_vreg[o] >> 5], 1u << (q.op_vreg[o] & 31));
-                __syncwarp();
-            }
-        }
-        for (uint32_t r = 0; !(WIDE && po.n > 32) && r < po.n; r += 32) {
-            const uint32_t x = po.get(q, r + lane);
-            bool written = false;  // an earlier instruction of the piece writes this operand's vreg
-            for (uint32_t j0 = 0; j0 <= r; j0 += 32) {
-                const uint32_t y = j0 == r ? x : po.get(q, j0 + lane);
-#pragma unroll 8
-                for (uint32_t j = 0; j < 32; ++j) {
-                    const uint32_t z = __shfl_sync(0xffffffffu, y, j);
-                    written |= po_def(z) && po_vreg(z) == po_vreg(x) && po_instr(z) < po_instr(x);
-                }
-            }
-            if (r + lane < po.n) {
-                uint32_t *s = po_def(x) ? s_def : s_use;
-                if (po_def(x) || !written) atomicOr(&s[po_vreg(x) >> 5], 1u << (x & 31));
-            }
-        }
+        piece_sets(q, po, x, lane, s_use, s_def);
         __syncwarp();
         for (uint32_t w = lane; w < q.Wv; w += 32) {
             q.piece_use[(size_t)p * q.Wv + w] = s_use[w];
@@ -315,65 +351,100 @@ __global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const __grid_constant_
     }
 }
 
-// The operands of a wide piece (see k_count), instruction by instruction from the last: live (the vregs live after the
-// instruction) and reads (those it reads; empty between instructions) are bitsets of this warp's own.
-__device__ __noinline__ void count_wide(const LiveArgs &q, const PieceOps &po, volatile uint32_t *live, volatile uint32_t *reads,
-                                        uint32_t *touch, int *s_d, uint32_t *s_ev)
+// An operand's flags, and the walk events that it makes.  many: the instruction has several definitions; lv: its vreg is live
+// after the instruction; dup: an earlier read of the instruction has the vreg; other: the instruction's other side
+// (reads / writes) has it.
+__device__ __forceinline__ uint32_t operand_events(bool many, bool def, bool lv, bool dup, bool other, uint32_t *flags)
 {
-    const uint32_t lane = threadIdx.x & 31;
-    auto has = [](volatile uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; };
-    auto word = [](volatile uint32_t *s, uint32_t v) { return const_cast<uint32_t *>(s) + (v >> 5); };
-    auto event = [&](uint32_t v, uint32_t k, uint32_t n) {
+    if (!def) {
+        const bool kill = !dup && !lv;  // a read of a vreg that stays live releases nothing
+        *flags = (kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0);
+        return kill ? 1u : 0u;
+    }
+    const bool elide = other && lv, post = !lv && many;
+    *flags = OPF_DEF | (elide ? OPF_ELIDE : 0) | ((lv || many) ? OPF_SET : 0) | (post ? OPF_POST : 0) | (lv ? 0 : OPF_DEAD);
+    return elide ? 0u : 1u + (post ? 1u : 0u);
+}
+
+// The operands of a piece of at most 32, one per lane: flags, touched vregs, and per instruction the events (s_ev) and what it
+// adds to the live count going backwards (s_d).  An operand's vreg is live after its instruction iff the next instruction of
+// the piece that touches it reads it, or, if none does, iff it is live after the piece (end).  touched: what this lane's word
+// of touch is known to hold.
+__device__ __forceinline__ void count_narrow(const Piece &po, uint32_t x, const uint32_t *end, uint8_t *opflags, uint32_t *touch,
+                                             uint32_t touched, int *s_d, uint32_t *s_ev)
+{
+    const uint32_t lane = threadIdx.x & 31, v = po_vreg(x);
+    const bool mine = lane < po.n, def = po_def(x);
+    if (lane < PIECE_INSTRS) { s_d[lane] = 0; s_ev[lane] = 0; }
+    bool up = false, down = false;
+    uint32_t evs = 0;
+    if (mine) {
+        const bool lv = x & OW_LATER ? (x & OW_READ) != 0 : (end[v >> 5] >> (v & 31)) & 1u;
+        const bool dup = x & OW_DUP, other = x & OW_OTHER;
+        uint32_t flags;
+        evs = operand_events(x & OW_MANY, def, lv, dup, other, &flags);
+        opflags[lane] = (uint8_t)flags;
+        // a read: live before the instruction, but not among what is live behind it and not written by it
+        up = !def && !dup && !(lv && !other);
+        down = def && lv;
+        if (evs && !((touched >> (v & 31)) & 1u)) atomicOr(&touch[v >> 5], 1u << (v & 31));
+    }
+    const uint32_t here = same_instr(x, mine);
+    const uint32_t ups = __ballot_sync(0xffffffffu, up), downs = __ballot_sync(0xffffffffu, down);
+    const uint32_t ev1 = __ballot_sync(0xffffffffu, evs != 0), ev2 = __ballot_sync(0xffffffffu, evs > 1);
+    __syncwarp();
+    if (mine && lane == __ffs(here) - 1) {
+        s_d[po_instr(x)] = (int)__popc(ups & here) - (int)__popc(downs & here);
+        s_ev[po_instr(x)] = __popc(ev1 & here) + __popc(ev2 & here);
+    }
+}
+
+// The same for a piece that is a single instruction with more operands.  reads: an empty bitset of this warp's own.
+// (200 instructions of 60 reads 172 us for the run, all operands met in pairs 976; 100 of 100 definitions 202 and 2,133)
+template <bool GLOBAL>  // touch lies in global memory
+__device__ __noinline__ void count_wide(const LiveArgs &q, const Piece &po, const uint32_t *end, volatile uint32_t *reads,
+                                        uint8_t *opflags, uint32_t *touch, uint32_t *s_ev)
+{
+    const uint32_t lane = threadIdx.x & 31, nd = q.ndefs[po.i0], r0 = po.o0 + nd, o1 = po.o0 + po.n;
+    auto has = [](const volatile uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; };
+    uint32_t n_ev = 0;
+    auto event = [&](uint32_t v, uint32_t n) {
         const uint32_t bit = 1u << (v & 31);
-        atomicAdd(&s_ev[k], n);
-        if (!(__ldcg(&touch[v >> 5]) & bit)) atomicOr(&touch[v >> 5], bit);
+        n_ev += n;
+        if (n && (!GLOBAL || !(__ldcg(&touch[v >> 5]) & bit))) atomicOr(&touch[v >> 5], bit);
     };
-    for (uint32_t k = po.ni; k-- > 0;) {
-        const uint32_t o0 = __shfl_sync(0xffffffffu, po.off, k), o1 = __shfl_sync(0xffffffffu, po.off, k + 1);
-        const uint32_t nd = __shfl_sync(0xffffffffu, po.nd, k), r0 = o0 + nd;
-        for (uint32_t o = r0; o < o1; o += 32) {  // which reads are the first of their vreg
-            const bool mine = o + lane < o1;
-            const uint32_t v = mine ? q.op_vreg[o + lane] : 0x10000u + lane;
-            const uint32_t same = __match_any_sync(0xffffffffu, v);
-            const bool dup = mine && ((same & ((1u << lane) - 1u)) || has(reads, v));
-            __syncwarp();
-            if (mine) {
-                if (!dup) atomicOr(word(reads, v), 1u << (v & 31));
-                const bool kill = !dup && !has(live, v);
-                q.opflags[o + lane] = (uint8_t)((kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0));
-                if (kill) event(v, k, 1);
-            }
-            __syncwarp();
-        }
-        for (uint32_t o = o0 + lane; o < r0; o += 32) {
-            const uint32_t v = q.op_vreg[o];
-            const bool lv = has(live, v), elide = has(reads, v) && lv, post = !lv && nd > 1;
-            q.opflags[o] = (uint8_t)(OPF_DEF | (elide ? OPF_ELIDE : 0) | ((lv || nd > 1) ? OPF_SET : 0) | (post ? OPF_POST : 0) | (lv ? 0 : OPF_DEAD));
-            if (!elide) event(v, k, 1 + (post ? 1 : 0));
-            if (lv) {  // (an instruction defines a vreg once)
-                atomicSub(&s_d[k], 1);
-                atomicAnd(word(live, v), ~(1u << (v & 31)));
-            }
-        }
+    for (uint32_t o = r0; o < o1; o += 32) {  // which reads are the first of their vreg
+        const bool mine = o + lane < o1;
+        const uint32_t v = mine ? q.op_vreg[o + lane] : 0x10000u + lane;
+        const uint32_t same = __match_any_sync(0xffffffffu, v);
+        const bool dup = mine && ((same & low_bits(lane)) || has(reads, v));
         __syncwarp();
-        for (uint32_t o = r0 + lane; o < o1; o += 32) {
-            const uint32_t v = q.op_vreg[o], bit = 1u << (v & 31);
-            if (!(atomicOr(word(live, v), bit) & bit)) atomicAdd(&s_d[k], 1);
-            atomicAnd(word(reads, v), ~bit);
+        if (mine) {
+            uint32_t flags;
+            if (!dup) atomicOr(const_cast<uint32_t *>(reads) + (v >> 5), 1u << (v & 31));
+            event(v, operand_events(nd > 1, false, has(end, v), dup, false, &flags));
+            opflags[o - po.o0 + lane] = (uint8_t)flags;
         }
         __syncwarp();
     }
+    for (uint32_t o = po.o0 + lane; o < r0; o += 32) {
+        const uint32_t v = q.op_vreg[o];
+        uint32_t flags;
+        event(v, operand_events(nd > 1, true, has(end, v), false, has(reads, v), &flags));
+        opflags[o - po.o0] = (uint8_t)flags;
+    }
+    __syncwarp();
+    for (uint32_t o = r0 + lane; o < o1; o += 32) reads[q.op_vreg[o] >> 5] = 0;
+    n_ev = __reduce_add_sync(0xffffffffu, n_ev);
+    if (lane == 0) s_ev[0] = n_ev;
 }
 
 // ============================================================================ k_count
 // One thread block per chunk.  First the live set after the last instruction of every piece (one thread per
-// bitset word, backwards over the chunk's pieces).  Then one warp per piece, one lane per operand: an operand's
-// vreg is live after its instruction iff the next instruction of the piece that touches it reads it, or, if
-// none does, iff it is live after the piece.  From that the operand flags, the walk events and the change of
-// the live count of every instruction follow without a serial walk; and the set of vregs whose occupancy
-// changes inside the block.  Last, offsets inside the chunk.
-// WIDE: some piece of the launch has more than WIDE_OPERANDS operands, which would meet each other in pairs; it is
-// taken instruction by instruction (count_wide).
+// bitset word, backwards over the chunk's pieces).  Then one warp per piece, one lane per operand (count_narrow): the operand
+// flags, the walk events and the change of the live count of every instruction follow without a serial walk; and the set of
+// vregs whose occupancy changes inside the block.  Last, offsets inside the chunk.  WIDE: some piece of the launch has more
+// than PIECE_OPERANDS operands.
 template <int N, bool WIDE>
 __global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMany<N> a)
 {
@@ -385,11 +456,11 @@ __global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMan
     const uint32_t p0 = q.chunk_piece_off[c], p1 = q.chunk_piece_off[c + 1];
     const uint32_t blk = q.chunk_blk[c];
     uint32_t *touch = q.blk_touch + (size_t)blk * q.Wv;
-    PieceOps po;
-    uint32_t x0 = 0xFFFFFFFFu;  // the first 32 operands of the warp's (first) piece: all of them, as a rule
+    Piece po;
+    uint32_t x = 0;  // the operands of the warp's (first) piece
     if (p0 + warp < p1) {
-        po.init(q, p0 + warp, c, lane);
-        x0 = po.get(q, lane);
+        po.init(q, p0 + warp);
+        x = po.get(q, lane);
     }
     pdl_go();
     pdl_wait();
@@ -416,77 +487,29 @@ __global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMan
     for (uint32_t p = p0 + warp; p < p1; p += PC_WARPS) {
         const uint32_t *end = q.piece_end + (size_t)p * q.Wv;
         if (p != p0 + warp) {
-            po.init(q, p, c, lane);
-            x0 = po.get(q, lane);
+            po.init(q, p);
+            x = po.get(q, lane);
         }
-        if (lane < PIECE_INSTRS) { s_ev[warp][lane] = 0; s_d[warp][lane] = 0; }
+        const uint32_t touched = lane < po.n ? __ldcg(&touch[po_vreg(x) >> 5]) : 0u;
         uint32_t cnt = 0;
         for (uint32_t w = lane; w < q.Wv; w += 32) cnt += __popc(end[w]);
         cnt = __reduce_add_sync(0xffffffffu, cnt);
-        __syncwarp();
-        const bool wide = WIDE && po.n > WIDE_OPERANDS;
-        if constexpr (WIDE) if (wide) {  // the bitsets: in shared memory if they fit, else in the rows of the piece's sets, used up by now
+        if (!WIDE || po.n <= PIECE_OPERANDS) {
+            count_narrow(po, x, end, q.opflags + po.o0, touch, touched, s_d[warp], s_ev[warp]);
+        } else {  // the set of reads: in shared memory if it fits, else in the row of the piece's own sets, used up by now
             extern __shared__ uint32_t sm[];
-            uint32_t *live = q.wide_smem ? sm + (size_t)warp * 2 * q.Wv : q.piece_use + (size_t)p * q.Wv;
-            uint32_t *reads = q.wide_smem ? live + q.Wv : q.piece_def + (size_t)p * q.Wv;
-            for (uint32_t w = lane; w < q.Wv; w += 32) { live[w] = end[w]; reads[w] = 0; }
+            uint32_t *reads = q.wide_smem ? sm + (size_t)warp * q.Wv : q.piece_def + (size_t)p * q.Wv;
+            for (uint32_t w = lane; w < q.Wv; w += 32) reads[w] = 0;
             __syncwarp();
-            count_wide(q, po, live, reads, touch, s_d[warp], s_ev[warp]);
-        }
-        for (uint32_t r = 0; !wide && r < po.n; r += 32) {
-            const uint32_t x = r == 0 ? x0 : po.get(q, r + lane), v = po_vreg(x), k = po_instr(x);
-            const bool mine = r + lane < po.n, def = po_def(x);
-            const uint32_t nd = __shfl_sync(0xffffffffu, po.nd, k < PIECE_INSTRS ? k : 0);
-            const uint32_t touched = mine ? __ldcg(&touch[v >> 5]) : 0u;
-            const uint32_t live_end = mine ? (end[v >> 5] >> (v & 31)) & 1u : 0u;
-            uint32_t next = 0xFFFFFFFFu;  // next touch: instruction * 2 + (1 if it only writes)
-            bool dup = false, other = false;  // an earlier read of the instruction has the vreg; its other side (reads / writes) has it
-            for (uint32_t j0 = 0; j0 < po.n; j0 += 32) {
-                const uint32_t y = j0 == r ? x : po.get(q, j0 + lane);
-                const uint32_t nj = (min(32u, po.n - j0) + 7u) & ~7u;  // (lanes beyond the piece hold no vreg)
-                for (uint32_t j8 = 0; j8 < nj; j8 += 8)
-#pragma unroll
-                    for (uint32_t u = 0; u < 8; ++u) {
-                        const uint32_t z = __shfl_sync(0xffffffffu, y, j8 + u);
-                        const bool same = po_vreg(z) == v, later = (z & 0xF0000u) > (x & 0xF0000u);
-                        const bool here = same && po_instr(z) == k;
-                        if (same && later) next = min(next, po_instr(z) * 2 + (po_def(z) ? 1u : 0u));
-                        other |= here && po_def(z) != def;
-                        dup |= here && po_def(z) == def && j0 + j8 + u < r + lane;
-                    }
-            }
-            if (mine) {
-                const bool lv = next == 0xFFFFFFFFu ? live_end != 0 : (next & 1u) == 0;
-                uint32_t flags, evs = 0;
-                if (!def) {
-                    const bool kill = !dup && !lv;  // a read of a vreg that stays live releases nothing
-                    flags = (kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0);
-                    if (kill) evs = 1;
-                    // live before the instruction, but not among what is live behind it and not written by it
-                    if (!dup && !(lv && !other)) atomicAdd(&s_d[warp][k], 1);
-                } else {
-                    const bool elide = other && lv, post = !lv && nd > 1;
-                    flags = OPF_DEF | (elide ? OPF_ELIDE : 0) | ((lv || nd > 1) ? OPF_SET : 0) | (post ? OPF_POST : 0) |
-                            (lv ? 0 : OPF_DEAD);
-                    if (!elide) evs = 1 + (post ? 1 : 0);
-                    if (lv) atomicSub(&s_d[warp][k], 1);
-                }
-                q.opflags[po.ob + r + lane] = (uint8_t)flags;
-                if (evs) {
-                    atomicAdd(&s_ev[warp][k], evs);
-                    const uint32_t bit = 1u << (v & 31);
-                    if (!(touched & bit)) atomicOr(&touch[v >> 5], bit);
-                }
-            }
+            count_wide<true>(q, po, end, reads, q.opflags + po.o0, touch, s_ev[warp]);
         }
         __syncwarp();
         // live after instruction k = live after the piece + what the later instructions add going backwards
         if (lane < po.ni) {
-            const uint32_t i = q.piece_i0[p] + lane;
             int live = (int)cnt;
             for (uint32_t u = lane + 1; u < po.ni; ++u) live += s_d[warp][u];
-            q.lo_rel[i] = (uint32_t)live;
-            q.ev_rel[i] = s_ev[warp][lane];
+            q.lo_rel[po.i0 + lane] = (uint32_t)live;
+            q.ev_rel[po.i0 + lane] = s_ev[warp][lane];
         }
         __syncwarp();
     }
@@ -506,65 +529,28 @@ __global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMan
     if (tid == 0) { q.chunk_lo[c] = lo_sum; q.chunk_ev[c] = ev_sum; }
 }
 
-// The live set before piece p of chunk c (p0 = the chunk's first piece), one word, without the block's through-set.
-__device__ __forceinline__ uint32_t entry_word(const LiveArgs &q, uint32_t c, uint32_t p, uint32_t p0, uint32_t b, uint32_t w)
+// The live set before piece p of chunk c (p0 = the chunk's first piece), one word.
+__device__ __forceinline__ uint32_t live_before(const LiveArgs &q, uint32_t c, uint32_t p, uint32_t p0, uint32_t w)
 {
-    const uint32_t x = p == p0 ? q.chunk_entry[(size_t)c * q.Wv + w] : q.piece_end[(size_t)(p - 1) * q.Wv + w];
-    const uint32_t th = q.use_th ? q.blk_in[(size_t)b * q.Wv + w] & ~q.blk_touch[(size_t)b * q.Wv + w] : 0u;
-    return x & ~th;
+    return p == p0 ? q.chunk_entry[(size_t)c * q.Wv + w] : q.piece_end[(size_t)(p - 1) * q.Wv + w];
+}
+// The through-set of block b, one word, from what touched its vregs.
+__device__ __forceinline__ uint32_t through_word(const LiveArgs &q, uint32_t b, uint32_t w)
+{
+    return q.use_th ? q.blk_in[(size_t)b * q.Wv + w] & ~q.blk_touch[(size_t)b * q.Wv + w] : 0u;
 }
 
-// ============================================================================ k_offsets
-// Thread blocks [0, nC): entry events of a chunk and events of its short chunks; [nC, nC + nB): the through-set
-// of a block (live on entry and never touched by an event inside it).  The block that finishes last makes the
-// offsets: list entries per chunk, walk events per chunk (padded to groups of 8), through-sets per block, steps
-// per 32 short chunks; and writes the totals and the status word to pinned host memory.
-template <int N>
-__global__ void __launch_bounds__(OFF_NT) k_offsets(const __grid_constant__ LiveMany<N> a)
+// The offsets of everything, from what the chunks, blocks and short chunks hold, by the first LV_TOTALS warps of a block: a
+// warp per total, the scans side by side; a lane takes up to 8 consecutive values at a time, whose loads are in flight
+// together.  GLOBAL: they lie in global memory and other blocks have written them (loads past the L1 cache).
+template <bool GLOBAL>
+__device__ __forceinline__ void live_offsets(const LiveArgs &q, unsigned long long *s_tot, const unsigned long long *chunk_lo,
+                                             const uint32_t *centry_cnt, const uint32_t *chunk_ev, const uint32_t *th_cnt,
+                                             const uint32_t *blk_off, const uint32_t *short_ev, const uint32_t *short_ent)
 {
-    LIVE_ARGS;
-    __shared__ uint32_t s_scan[34];
-    __shared__ unsigned long long s_tot[LV_TOTALS];
-    __shared__ uint32_t s_last;
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (blockIdx.x >= q.nC + q.nB) return;
-    pdl_go();
-    pdl_wait();
-    if (blockIdx.x < q.nC) {
-        const uint32_t c = blockIdx.x, b = q.chunk_blk[c], p0 = q.chunk_piece_off[c];
-        const uint32_t s1 = q.chunk_short_off[c + 1];
-        for (uint32_t s = q.chunk_short_off[c] + warp; s < s1; s += OFF_NT / 32) {
-            const uint32_t p = q.short_p0[s];
-            uint32_t cnt = 0;
-            for (uint32_t w = lane; w < q.Wv; w += 32) cnt += __popc(entry_word(q, c, p, p0, b, w));
-            cnt = __reduce_add_sync(0xffffffffu, cnt);
-            if (lane == 0) {
-                if (p == p0) q.centry_cnt[c] = cnt;
-                const uint32_t ev1 = s + 1 < s1 ? q.ev_rel[q.piece_i0[q.short_p0[s + 1]]] : q.chunk_ev[c];
-                q.short_ent[s] = cnt;
-                q.short_ev[s] = ev1 - q.ev_rel[q.piece_i0[p]];
-            }
-        }
-    } else {
-        const uint32_t b = blockIdx.x - q.nC;
-        uint32_t cnt = 0, total;
-        for (uint32_t w = tid; w < q.Wv; w += OFF_NT) {
-            const uint32_t t = q.use_th ? q.blk_in[(size_t)b * q.Wv + w] & ~q.blk_touch[(size_t)b * q.Wv + w] : 0u;
-            q.blk_th[(size_t)b * q.Wv + w] = t;
-            cnt += __popc(t);
-        }
-        block_excl_scan(cnt, s_scan, &total);
-        if (tid == 0) q.th_cnt[b] = total;
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) s_last = atomicAdd(&q.counters[0], 1u) == q.nC + q.nB - 1 ? 1u : 0u;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // A warp per total, the scans side by side; a lane takes up to 8 consecutive values at a time, whose loads are in
-    // flight together.  Exclusive offsets of n values into dst[0..n) (null: none), dst[n] = total, clipped to
-    // 32 bits; the total is returned.
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto load = [](const auto *p) { return GLOBAL ? __ldcg(p) : *p; };
+    // Exclusive offsets of n values into dst[0..n) (null: none), dst[n] = total, clipped to 32 bits; the total is returned.
     auto offsets = [&](uint32_t n, uint32_t *dst, auto value, auto store) -> unsigned long long {
         unsigned long long carry = 0;
         for (uint32_t j0 = 0; j0 < n; j0 += 256) {
@@ -594,40 +580,405 @@ __global__ void __launch_bounds__(OFF_NT) k_offsets(const __grid_constant__ Live
     auto into = [](uint32_t *dst) { return [dst](uint32_t j, uint32_t at) { dst[j] = at; }; };
     unsigned long long tot = 0;
     if (warp == LV_TOT_LO) {
-        tot = offsets(q.nC, q.chunk_lo0, [&](uint32_t c) { return __ldcg(q.chunk_lo + c); }, into(q.chunk_lo0));
+        tot = offsets(q.nC, q.chunk_lo0, [&](uint32_t c) { return load(chunk_lo + c); }, into(q.chunk_lo0));
         if (lane == 0) q.lo_off[q.nI] = tot > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)tot;
     } else if (warp == LV_TOT_EV) {
         tot = offsets(q.nC, q.cev_off, [&](uint32_t c) -> unsigned long long {
-            return (__ldcg(q.centry_cnt + c) + __ldcg(q.chunk_ev + c) + 7u) / 8u * 8u;
+            return (load(centry_cnt + c) + load(chunk_ev + c) + 7u) / 8u * 8u;
         }, into(q.cev_off));
     } else if (warp == LV_TOT_TH) {
-        tot = offsets(q.nB, q.th_off, [&](uint32_t b) -> unsigned long long { return __ldcg(q.th_cnt + b); }, into(q.th_off));
+        tot = offsets(q.nB, q.th_off, [&](uint32_t b) -> unsigned long long { return load(th_cnt + b); }, into(q.th_off));
     } else if (warp == LV_TOT_LS) {
         // short lists (see vl_program): what the through-sets take off the lists of the blocks before b
         tot = offsets(q.nB, nullptr, [&](uint32_t b) -> unsigned long long {
-            return (unsigned long long)(q.blk_off[b + 1] - q.blk_off[b]) * __ldcg(q.th_cnt + b);
-        }, [&](uint32_t b, uint32_t pre) { q.ls_adj[b] = pre - q.blk_off[b] * __ldcg(q.th_cnt + b); });
+            return (unsigned long long)(blk_off[b + 1] - blk_off[b]) * load(th_cnt + b);
+        }, [&](uint32_t b, uint32_t pre) { q.ls_adj[b] = pre - blk_off[b] * load(th_cnt + b); });
     } else if (warp == LV_TOT_SEV) {  // a group of 32 short chunks per round: its longest
+#pragma unroll 4
         for (uint32_t g = 0; g * 32 < q.nS; ++g) {
-            const uint32_t m = __reduce_max_sync(0xffffffffu, g * 32 + lane < q.nS ? __ldcg(q.short_ev + g * 32 + lane) : 0u);
+            const uint32_t m = __reduce_max_sync(0xffffffffu, g * 32 + lane < q.nS ? load(short_ev + g * 32 + lane) : 0u);
             if (lane == 0) q.sev_off[g] = (uint32_t)tot;
             tot += m;
         }
         if (lane == 0) q.sev_off[(q.nS + 31) / 32] = (uint32_t)tot;
         tot *= 32;
     } else if (warp == LV_TOT_SEN) {
-        tot = offsets(q.nS, q.sen_off, [&](uint32_t s) -> unsigned long long { return __ldcg(q.short_ent + s); }, into(q.sen_off));
+        tot = offsets(q.nS, q.sen_off, [&](uint32_t s) -> unsigned long long { return load(short_ent + s); }, into(q.sen_off));
     }
     if (warp < LV_TOTALS && lane == 0) s_tot[warp] = tot;
+}
+// The totals and the status word to the host (one thread).
+__device__ __forceinline__ void live_totals(const LiveArgs &q, unsigned long long *s_tot, uint32_t st)
+{
+    s_tot[LV_TOT_LS] = s_tot[LV_TOT_LO] - s_tot[LV_TOT_LS];
+    if (s_tot[LV_TOT_LO] > 0xFFFFFFF0ull) st |= ST_SIZE_OVERFLOW;
+    q.host_out[0] = st;
+    unsigned long long *h = reinterpret_cast<unsigned long long *>(q.host_out + 2);
+    for (int j = 0; j < LV_TOTALS; ++j) h[j] = s_tot[j];
+}
+
+// ============================================================================ k_offsets
+// Thread blocks [0, nC): entry events of a chunk and events of its short chunks; [nC, nC + nB): the through-set
+// of a block (live on entry and never touched by an event inside it).  The block that finishes last makes the
+// offsets: list entries per chunk, walk events per chunk (padded to groups of 8), through-sets per block, steps
+// per 32 short chunks; and writes the totals and the status word to pinned host memory.
+template <int N>
+__global__ void __launch_bounds__(OFF_NT) k_offsets(const __grid_constant__ LiveMany<N> a)
+{
+    LIVE_ARGS;
+    __shared__ uint32_t s_scan[34];
+    __shared__ unsigned long long s_tot[LV_TOTALS];
+    __shared__ uint32_t s_last;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (blockIdx.x >= q.nC + q.nB) return;
+    pdl_go();
+    pdl_wait();
+    if (blockIdx.x < q.nC) {
+        const uint32_t c = blockIdx.x, b = q.chunk_blk[c], p0 = q.chunk_piece_off[c];
+        const uint32_t s1 = q.chunk_short_off[c + 1];
+        for (uint32_t s = q.chunk_short_off[c] + warp; s < s1; s += OFF_NT / 32) {
+            const uint32_t p = q.short_p0[s];
+            uint32_t cnt = 0;
+            for (uint32_t w = lane; w < q.Wv; w += 32) cnt += __popc(live_before(q, c, p, p0, w) & ~through_word(q, b, w));
+            cnt = __reduce_add_sync(0xffffffffu, cnt);
+            if (lane == 0) {
+                if (p == p0) q.centry_cnt[c] = cnt;
+                const uint32_t ev1 = s + 1 < s1 ? q.ev_rel[q.piece_i0[q.short_p0[s + 1]]] : q.chunk_ev[c];
+                q.short_ent[s] = cnt;
+                q.short_ev[s] = ev1 - q.ev_rel[q.piece_i0[p]];
+            }
+        }
+    } else {
+        const uint32_t b = blockIdx.x - q.nC;
+        uint32_t cnt = 0, total;
+        for (uint32_t w = tid; w < q.Wv; w += OFF_NT) {
+            const uint32_t t = through_word(q, b, w);
+            q.blk_th[(size_t)b * q.Wv + w] = t;
+            cnt += __popc(t);
+        }
+        block_excl_scan(cnt, s_scan, &total);
+        if (tid == 0) q.th_cnt[b] = total;
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&q.counters[0], 1u) == q.nC + q.nB - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    live_offsets<true>(q, s_tot, q.chunk_lo, q.centry_cnt, q.chunk_ev, q.th_cnt, q.blk_off, q.short_ev, q.short_ent);
+    __syncthreads();
+    if (tid == 0) live_totals(q, s_tot, __ldcg(q.status));
+}
+
+// ============================================================================ k_small
+// k_sets, k_flow, k_count and k_offsets of a program of up to LIVE_SMALL_INSTRS instructions in one launch: a cluster of C
+// thread blocks, each with a share of the chunks whose sets stay in its shared memory from phase to phase.  What bounds such
+// a run is not work but the chain of launches and L2 round trips: 100 rows of 2,000 instructions, liveness included, 54 us
+// with the four kernels, 37 with this one; of 64 instructions 38 and 28.  What the blocks need of each other (chunk sets,
+// touched vregs, counts) they store into each other's shared memory, behind three cluster barriers; the fixed point over the
+// blocks is cheap enough for every thread block to do all of it, which saves a barrier.  One block does the last scans.
+
+// Composes the sets of units [j0, j1) (rows of Wv words, one word), going forwards: read before written, written.  Eight
+// loads in flight.
+__device__ __forceinline__ void compose_sets(const uint32_t *use, const uint32_t *def, uint32_t j0, uint32_t j1, uint32_t Wv, uint32_t &u, uint32_t &d)
+{
+    u = d = 0;
+#pragma unroll 1
+    for (; j0 < j1; j0 += 8) {
+        uint32_t x[8], y[8];
+#pragma unroll
+        for (uint32_t t = 0; t < 8; ++t) {
+            const uint32_t at = min(j0 + t, j1 - 1) * Wv;  // (once more the last one: no harm)
+            x[t] = use[at];
+            y[t] = def[at];
+        }
+#pragma unroll
+        for (uint32_t t = 0; t < 8; ++t) { u |= x[t] & ~d; d |= y[t]; }
+    }
+}
+// Live sets of units [j0, j1) going backwards from `live`: use becomes what is live after the unit, or (BEFORE) before it.
+template <bool BEFORE>
+__device__ __forceinline__ void live_sets(uint32_t *use, const uint32_t *def, uint32_t j0, uint32_t j1, uint32_t Wv, uint32_t live)
+{
+#pragma unroll 1
+    for (; j1 > j0; j1 -= min(j1 - j0, 8u)) {
+        uint32_t x[8], y[8];
+#pragma unroll
+        for (uint32_t t = 0; t < 8; ++t) {
+            const uint32_t at = (j1 - 1 - min(t, j1 - j0 - 1)) * Wv;
+            x[t] = use[at];
+            y[t] = def[at];
+        }
+#pragma unroll
+        for (uint32_t t = 0; t < 8; ++t) {
+            if (t >= j1 - j0) break;
+            if (!BEFORE) use[(j1 - 1 - t) * Wv] = live;
+            live = x[t] | (live & ~y[t]);
+            if (BEFORE) use[(j1 - 1 - t) * Wv] = live;
+        }
+    }
+}
+
+template <int N, int C>
+__global__ void __launch_bounds__(SMALL_NT, 2) k_small(const __grid_constant__ LiveMany<N> a)
+{
+    LIVE_ARGS;
+    extern __shared__ __align__(16) uint32_t sm[];
+    __shared__ uint32_t s_ev[SMALL_WARPS][PIECE_INSTRS];
+    __shared__ int s_d[SMALL_WARPS][PIECE_INSTRS];
+    __shared__ uint32_t s_st;
+    __shared__ unsigned long long s_tot[LV_TOTALS];
+    namespace cg = cooperative_groups;
+    const uint32_t rank = C == 1 ? 0u : blockIdx.x;  // (a grid of C blocks per program, clusters of C)
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Wv = q.Wv;
+    const uint4 *share = q.share + (C == 1 ? SMALL_BLOCKS + 1 : 0);  // first chunk, piece, instruction, operand
+    const uint4 s0 = share[rank], s1 = share[rank + 1];
+    const SmallSmem &L = q.small;
+    uint32_t *pu = sm + L.pu, *pd = sm + L.pd, *cu = sm + L.cu, *cd = sm + L.cd, *bu = sm + L.bu, *bd = sm + L.bd, *bi = sm + L.bi,
+             *bo = sm + L.bo, *bt = sm + L.bt, *piece_chunk = sm + L.pc;
+    const uint32_t *blk_chunk = sm + L.blk_chunk, *chunk_piece = sm + L.chunk_piece, *chunk_blk = sm + L.chunk_blk,
+                   *chunk_short = sm + L.chunk_short, *short_piece = sm + L.short_piece, *short_chunk = sm + L.short_chunk,
+                   *s_so = sm + L.succ_off, *s_su = sm + L.succ;
+    uint8_t *s_fl = reinterpret_cast<uint8_t *>(sm + L.fl);
+    unsigned long long *s_clo = reinterpret_cast<unsigned long long *>(sm + L.clo);
+    auto sync = [&] {
+        if (C == 1) __syncthreads();
+        else cg::this_cluster().sync();
+    };
+    // p of this block as block r of the cluster has it
+    auto of = [&](auto *p, uint32_t r) { return C == 1 ? p : cg::this_cluster().map_shared_rank(p, r); };
+
+    // ---- what the phases read of the program and its layout comes to shared memory, in two L2 round trips with the shares
+    for (uint32_t i = tid; i < L.tab_words; i += SMALL_NT) sm[L.tab + i] = q.small_tab[i];
+    const uint32_t c0 = s0.x, c1 = s1.x, p0 = s0.y, np = s1.y - s0.y, o_first = s0.w, n_ops = s1.w - s0.w;
+    for (uint32_t i = tid; i <= np; i += SMALL_NT) {
+        sm[L.pi + i] = q.piece_i0[p0 + i];
+        sm[L.po + i] = q.piece_o0[p0 + i];
+        if (i < np) piece_chunk[i] = q.piece_chunk[p0 + i];
+    }
+    for (uint32_t i = tid; i < n_ops; i += SMALL_NT) sm[L.xs + i] = q.op_word[o_first + i];
+    for (uint32_t i = tid; i < np * Wv; i += SMALL_NT) pu[i] = pd[i] = 0;
+    for (uint32_t i = tid; i < q.nB * Wv; i += SMALL_NT) bt[i] = bi[i] = 0;
+    if (tid == 0) s_st = 0;
+    __syncthreads();
+    auto piece = [&](uint32_t j) {
+        Piece x;
+        x.i0 = sm[L.pi + j];
+        x.ni = sm[L.pi + j + 1] - x.i0;
+        x.o0 = sm[L.po + j];
+        x.n = sm[L.po + j + 1] - x.o0;
+        return x;
+    };
+    auto operand = [&](const Piece &x) { return lane < x.n ? sm[L.xs + x.o0 - o_first + lane] : 0u; };
+    // ---- read and write sets of the pieces
+    for (uint32_t j = warp; j < np; j += SMALL_WARPS) {
+        const Piece x = piece(j);
+        piece_sets(q, x, operand(x), lane, pu + j * Wv, pd + j * Wv);
+    }
+    sync();  // (every block has begun: its shared memory may be written to)
+    // ---- the chunks', to every block
+    for (uint32_t i = tid; i < (c1 - c0) * Wv; i += SMALL_NT) {
+        const uint32_t c = c0 + i / Wv, w = i % Wv;
+        uint32_t u, d;
+        compose_sets(pu + w, pd + w, chunk_piece[c] - p0, chunk_piece[c + 1] - p0, Wv, u, d);
+        for (uint32_t r = 0; r < C; ++r) {
+            of(cu, r)[c * Wv + w] = u;
+            of(cd, r)[c * Wv + w] = d;
+        }
+    }
+    sync();
+    // ---- block sets, fixed point, live sets at the chunk boundaries (every block: all of them)
+    for (uint32_t i = tid; i < q.nB * Wv; i += SMALL_NT) {
+        const uint32_t b = i / Wv, w = i % Wv;
+        compose_sets(cu + w, cd + w, blk_chunk[b], blk_chunk[b + 1], Wv, bu[i], bd[i]);
+    }
+    __syncthreads();
+    if (warp * 32 < Wv) {  // a warp per 32 words (and more of them where there are more words than lanes)
+        uint32_t st = 0;
+        for (uint32_t w0 = warp * 32; w0 < Wv; w0 += SMALL_NT) {
+            const uint32_t w = min(w0 + lane, Wv - 1);  // (lanes past the last word do it once more)
+            bool changed = true;
+            for (uint32_t sweep = 0; sweep < q.nB + 2 && __any_sync(0xffffffffu, changed); ++sweep) {
+                changed = false;
+                uint32_t e = s_so[q.nB];
+                for (uint32_t b = q.nB; b-- > 0;) {
+                    const uint32_t u = bu[b * Wv + w], d = bd[b * Wv + w], was = bi[b * Wv + w], e0 = s_so[b];
+                    uint32_t o = 0;
+                    while (e > e0) o |= bi[s_su[--e] * Wv + w];
+                    const uint32_t i = u | (o & ~d);
+                    changed |= i != was;
+                    bi[b * Wv + w] = i;
+                    bo[b * Wv + w] = o;
+                }
+            }
+            if (changed) st |= ST_NO_CONVERGE;
+            if (bi[w] != 0) st |= ST_NOT_STRICT;  // block 0 is the entry
+        }
+        st = __reduce_or_sync(0xffffffffu, st);
+        if (st && lane == 0) atomicOr(&s_st, st);
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < q.nB * Wv; i += SMALL_NT) {
+        const uint32_t b = i / Wv, w = i % Wv;
+        live_sets<true>(cu + w, cd + w, blk_chunk[b], blk_chunk[b + 1], Wv, bo[i]);
+    }
+    __syncthreads();
+    // ---- live sets behind the pieces of the share
+    for (uint32_t i = tid; i < (c1 - c0) * Wv; i += SMALL_NT) {
+        const uint32_t c = c0 + i / Wv, w = i % Wv, b = chunk_blk[c];
+        const uint32_t live = c + 1 < blk_chunk[b + 1] ? cu[(c + 1) * Wv + w] : bo[b * Wv + w];
+        live_sets<false>(pu + w, pd + w, chunk_piece[c] - p0, chunk_piece[c + 1] - p0, Wv, live);
+    }
+    __syncthreads();
+    // ---- operand flags, touched vregs, events and live counts (see k_count); offsets inside the pieces
+    for (uint32_t j = warp; j < np; j += SMALL_WARPS) {
+        const uint32_t *end = pu + j * Wv;
+        uint32_t *touch = bt + chunk_blk[piece_chunk[j]] * Wv;
+        const Piece x = piece(j);
+        uint32_t cnt = 0;
+        for (uint32_t w = lane; w < Wv; w += 32) cnt += __popc(end[w]);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (x.n <= PIECE_OPERANDS) {
+            count_narrow(x, operand(x), end, s_fl + x.o0 - o_first, touch, 0u, s_d[warp], s_ev[warp]);
+        } else {
+            uint32_t *reads = sm + L.rd + warp * Wv;
+            for (uint32_t w = lane; w < Wv; w += 32) reads[w] = 0;
+            __syncwarp();
+            count_wide<false>(q, x, end, reads, s_fl + x.o0 - o_first, touch, s_ev[warp]);
+        }
+        __syncwarp();
+        // live after instruction k = live after the piece + what the later instructions add going backwards
+        const bool mine = lane < x.ni;
+        int later = mine && lane + 1 < x.ni ? s_d[warp][lane + 1] : 0;
+#pragma unroll
+        for (int d = 1; d < PIECE_INSTRS; d <<= 1) later += __shfl_down_sync(0xffffffffu, later, d);  // (zeros beyond the piece)
+        const uint32_t lo = mine ? (uint32_t)((int)cnt + later) : 0u, ev = mine ? s_ev[warp][lane] : 0u;
+        uint32_t lo_i = lo, ev_i = ev;
+#pragma unroll
+        for (int d = 1; d < PIECE_INSTRS; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, lo_i, d), z = __shfl_up_sync(0xffffffffu, ev_i, d);
+            if (lane >= (uint32_t)d) { lo_i += y; ev_i += z; }
+        }
+        if (mine) { sm[L.lo + j * PIECE_INSTRS + lane] = lo_i - lo; sm[L.ev + j * PIECE_INSTRS + lane] = ev_i - ev; }
+        if (lane == PIECE_INSTRS - 1) { sm[L.plo + j] = lo_i; sm[L.pev + j] = ev_i; }
+        __syncwarp();
+    }
+    __syncthreads();
+    // ---- touched vregs to every block; offsets inside the chunks (a warp per chunk, a lane per piece), events of the short chunks
+    if (C > 1)
+        for (uint32_t i = tid; i < q.nB * Wv; i += SMALL_NT) {
+            const uint32_t t = bt[i];  // (bits that other blocks have stored meanwhile go round once more: no harm)
+            if (t)
+                for (uint32_t r = 0; r < C; ++r)
+                    if (r != rank) atomicOr(of(bt, r) + i, t);
+        }
+    uint32_t *cev = of(sm + L.cev, 0), *cent = of(sm + L.cent, 0), *sent = of(sm + L.sent, 0), *sev = of(sm + L.sev, 0);
+    unsigned long long *clo = of(s_clo, 0);
+    for (uint32_t c = c0 + warp; c < c1; c += SMALL_WARPS) {
+        const uint32_t first = chunk_piece[c] - p0, last = chunk_piece[c + 1] - p0;
+        unsigned long long lo_sum = 0;
+        uint32_t ev_sum = 0;
+        for (uint32_t j0 = first; j0 < last; j0 += 32) {
+            const uint32_t j = j0 + lane;
+            const uint32_t x = j < last ? sm[L.plo + j] : 0u, y = j < last ? sm[L.pev + j] : 0u;
+            uint32_t xi = x, yi = y;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t xo = __shfl_up_sync(0xffffffffu, xi, d), yo = __shfl_up_sync(0xffffffffu, yi, d);
+                if (lane >= (uint32_t)d) { xi += xo; yi += yo; }
+            }
+            if (j < last) { sm[L.plo + j] = (uint32_t)lo_sum + xi - x; sm[L.pev + j] = ev_sum + yi - y; }
+            lo_sum += __shfl_sync(0xffffffffu, xi, 31);
+            ev_sum += __shfl_sync(0xffffffffu, yi, 31);
+        }
+        __syncwarp();
+        if (lane == 0) { clo[c] = lo_sum; cev[c] = ev_sum; sm[L.cev + c] = ev_sum; }
+        const uint32_t s_hi = chunk_short[c + 1];
+        for (uint32_t s = chunk_short[c] + lane; s < s_hi; s += 32) {
+            const uint32_t e0 = sm[L.pev + short_piece[s] - p0], e1 = s + 1 < s_hi ? sm[L.pev + short_piece[s + 1] - p0] : ev_sum;
+            sev[s] = sm[L.sev + s] = e1 - e0;
+        }
+    }
+    sync();
+    // ---- through-sets (every block: all of them), what is occupied when chunks and short chunks of the share begin
+    for (uint32_t i = tid; i < q.nB * Wv; i += SMALL_NT) bu[i] = q.use_th ? bi[i] & ~bt[i] : 0u;
+    __syncthreads();
+    for (uint32_t s = chunk_short[c0] + warp; s < chunk_short[c1]; s += SMALL_WARPS) {
+        const uint32_t p = short_piece[s], c = short_chunk[s];
+        const bool first = p == chunk_piece[c];
+        const uint32_t *live = first ? cu + c * Wv : pu + (p - 1 - p0) * Wv, *t = bu + chunk_blk[c] * Wv;
+        uint32_t cnt = 0;
+        for (uint32_t w = lane; w < Wv; w += 32) cnt += __popc(live[w] & ~t[w]);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) {
+            sent[s] = cnt;
+            if (first) cent[c] = sm[L.cent + c] = cnt;
+        }
+    }
+    if (rank == 0)
+        for (uint32_t b = warp; b < q.nB; b += SMALL_WARPS) {
+            uint32_t cnt = 0;
+            for (uint32_t w = lane; w < Wv; w += 32) cnt += __popc(bu[b * Wv + w]);
+            cnt = __reduce_add_sync(0xffffffffu, cnt);
+            if (lane == 0) sm[L.thn + b] = cnt;
+        }
+    sync();
+    // ---- everything to global memory (stores in front of a cluster barrier would be waited for there); the offsets
+    pdl_go();
+    pdl_wait();  // an earlier call's kernels may still read what is written from here on
+    if (rank == 0) {
+        live_offsets<false>(q, s_tot, s_clo, sm + L.cent, sm + L.cev, sm + L.thn, sm + L.blk_off, sm + L.sev, sm + L.sent);
+        for (uint32_t i = tid; i < q.nB * Wv; i += SMALL_NT) { q.blk_in[i] = bi[i]; q.blk_out[i] = bo[i]; q.blk_th[i] = bu[i]; }
+        for (uint32_t b = tid; b < q.nB; b += SMALL_NT) { q.el_count[b] = 0; q.th_cnt[b] = sm[L.thn + b]; }
+    }
+    for (uint32_t i = tid; i < n_ops; i += SMALL_NT) q.opflags[o_first + i] = s_fl[i];
+    for (uint32_t i = tid; i < np * Wv; i += SMALL_NT) q.piece_end[(size_t)p0 * Wv + i] = pu[i];
+    for (uint32_t i = tid; i < (c1 - c0) * Wv; i += SMALL_NT) q.chunk_entry[(size_t)c0 * Wv + i] = cu[c0 * Wv + i];
+    for (uint32_t c = c0 + tid; c < c1; c += SMALL_NT) { q.chunk_ev[c] = sm[L.cev + c]; q.centry_cnt[c] = sm[L.cent + c]; }
+    for (uint32_t s = chunk_short[c0] + tid; s < chunk_short[c1]; s += SMALL_NT) q.short_ev[s] = sm[L.sev + s];
+    for (uint32_t i = tid; i < np * PIECE_INSTRS; i += SMALL_NT) {
+        const uint32_t j = i / PIECE_INSTRS, k = sm[L.pi + j] + i % PIECE_INSTRS;
+        if (k >= sm[L.pi + j + 1]) continue;
+        q.lo_rel[k] = sm[L.plo + j] + sm[L.lo + i];
+        q.ev_rel[k] = sm[L.pev + j] + sm[L.ev + i];
+    }
+    if (rank) return;
     __syncthreads();
     if (tid == 0) {
-        s_tot[LV_TOT_LS] = s_tot[LV_TOT_LO] - s_tot[LV_TOT_LS];
-        uint32_t st = __ldcg(q.status);
-        if (s_tot[LV_TOT_LO] > 0xFFFFFFF0ull) st |= ST_SIZE_OVERFLOW;
-        q.host_out[0] = st;
-        unsigned long long *h = reinterpret_cast<unsigned long long *>(q.host_out + 2);
-        for (int j = 0; j < LV_TOTALS; ++j) h[j] = s_tot[j];
+        const uint32_t st = s_st;
+        *q.status = st;
+        live_totals(q, s_tot, st);
     }
+}
+
+// The operand words of a layout's pieces (see Piece), a warp per piece.
+__global__ void __launch_bounds__(NT) k_operand_words(uint32_t nP, const uint32_t *__restrict__ piece_i0, const uint32_t *__restrict__ op_off,
+                                                      const uint8_t *__restrict__ ndefs, const uint32_t *__restrict__ op_vreg, uint32_t *op_word)
+{
+    const uint32_t p = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (p >= nP) return;
+    const uint32_t i0 = piece_i0[p], i1 = piece_i0[p + 1], o0 = op_off[i0], n = op_off[i1] - o0;
+    if (n > PIECE_OPERANDS) {  // a single instruction: it reads before it writes
+        for (uint32_t j = lane; j < n; j += 32) op_word[o0 + j] = op_vreg[o0 + j] | (j < ndefs[i0] ? OW_DEF : OW_EXPOSED);
+        return;
+    }
+    const bool mine = lane < n;
+    uint32_t x = 0;
+    if (mine) {
+        uint32_t i = i0;
+        while (op_off[i + 1] <= o0 + lane) ++i;
+        x = op_vreg[o0 + lane] | ((i - i0) << 16) | (o0 + lane - op_off[i] < ndefs[i] ? OW_DEF : 0u) | (ndefs[i] > 1 ? OW_MANY : 0u);
+    }
+    const uint32_t here = same_instr(x, mine), same = __match_any_sync(0xffffffffu, mine ? po_vreg(x) : 0x10000u + lane);
+    const uint32_t defs = __ballot_sync(0xffffffffu, mine && po_def(x));
+    const uint32_t before = mine ? low_bits(__ffs(here) - 1) : 0u, later = mine ? same & ~(before | here) : 0u;
+    const uint32_t here_next = __shfl_sync(0xffffffffu, here, later ? __ffs(later) - 1 : 0);
+    if (!mine) return;
+    if (!po_def(x) && (same & here & ~defs & low_bits(lane))) x |= OW_DUP;
+    if (same & here & (po_def(x) ? ~defs : defs)) x |= OW_OTHER;
+    if (!po_def(x) && !(same & before & defs)) x |= OW_EXPOSED;
+    if (later) x |= OW_LATER | (same & here_next & ~defs ? OW_READ : 0u);
+    op_word[o0 + lane] = x;
 }
 
 // First occurrence and first definition of every vreg.
@@ -752,74 +1103,126 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
     pdl_go();
     const uint32_t n_list = (q.nP + LV_WARPS - 1) / LV_WARPS, n_short = ((q.nS + 31) & ~31u) / LV_WARPS;
     if (role < n_list) {
-        // Backward walk of one piece.  Two lists per instruction: the vregs live after it, ascending, and the same
-        // without the block's through-set (every instruction of the block has all of that in its live-after set, so
-        // the short list of instruction i starts at lo_off[i] - ls_adj[b] - i * th_cnt[b]).  Every non-empty word
-        // of the live set is broadcast and each lane whose bit is set writes its id at the rank of that bit.
+        // Two lists per instruction: the vregs live after it, ascending, and the same without the block's through-set (every
+        // instruction of the block has all of that in its live-after set, so the short list of instruction i starts at
+        // lo_off[i] - ls_adj[b] - i * th_cnt[b]).  The lists of a piece's eight instructions differ by what the piece
+        // touches: its members (live after the piece, or an operand) are found once, each with a mask of the
+        // instructions it is live after, and a ballot per instruction gives 32 members their places in its two lists.
+        // (Walking the bitset word by word for every instruction, 48 programs of 2,500 instructions took 67.5 us, 52.6
+        // now; one of 32,000 73 and 52.)
         const uint32_t p = role * LV_WARPS + warp;
         const bool mine = p < q.nP;
         const uint32_t c = mine ? q.piece_chunk[p] : 0u, b = mine ? q.chunk_blk[c] : 0u;
-        PieceOps po;
-        uint32_t x0 = 0xFFFFFFFFu;  // the first 32 operands (all of them, as a rule)
+        Piece po{};
+        uint32_t x0 = 0;  // the first 32 operands (all of them, as a rule)
+        uint32_t o_k = 0, nd_k = 0, n_reads = 0;  // lane k: first operand, definitions and reads of instruction k
         if (mine) {
-            po.init(q, p, c, lane);
+            po.init(q, p);
             x0 = po.get(q, lane);
+            if (lane < po.ni) {
+                o_k = q.op_off[po.i0 + lane];
+                nd_k = q.ndefs[po.i0 + lane];
+                n_reads = q.op_off[po.i0 + lane + 1] - o_k - nd_k;
+            }
         }
+        uint32_t v0 = q.V;  // and its first defined vreg
+        if (nd_k) v0 = q.op_vreg[o_k];
         pdl_wait();
         if (!mine) return;
+        uint32_t *s_end = sm + (size_t)warp * (2 * q.Wv + FILL_WARP_WORDS), *s_u = s_end + q.Wv, *s_rank = s_u + q.Wv, *s_mem = s_rank + 32;
+        uint8_t *s_flag = reinterpret_cast<uint8_t *>(s_mem + 1024);
+        const uint32_t *th = q.blk_th + (size_t)b * q.Wv;
         const uint32_t ls_sub = q.ls_adj[b], ls_mul = q.th_cnt[b];
-        uint32_t *s_live = sm + (size_t)warp * 2 * q.Wv, *s_th = s_live + q.Wv;
-        for (uint32_t w = lane; w < q.Wv; w += 32) {
-            s_live[w] = q.piece_end[(size_t)p * q.Wv + w];
-            s_th[w] = q.blk_th[(size_t)b * q.Wv + w];
-        }
-        const uint32_t i0 = q.piece_i0[p];
+        const uint32_t i0 = po.i0;
         uint32_t my_lo = 0;
-        if (lane < po.ni) {
-            my_lo = q.chunk_lo0[c] + q.lo_rel[i0 + lane];
-            q.lo_off[i0 + lane] = my_lo;
-        }
-        uint32_t v0 = q.V, my_n = 0;  // lane k: first defined vreg of instruction k, length of its short list
-        if (lane < po.ni && po.nd) v0 = q.op_vreg[po.off];
+        if (lane < po.ni) my_lo = q.chunk_lo0[c] + q.lo_rel[i0 + lane];
+        const uint32_t th0 = nd_k ? (th[v0 >> 5] >> (v0 & 31)) & 1u : 0u;  // whether that vreg is in the through-set
+        for (uint32_t w = lane; w < q.Wv; w += 32) s_end[w] = s_u[w] = q.piece_end[(size_t)p * q.Wv + w];
+        if (lane < po.ni) q.lo_off[i0 + lane] = my_lo;
         __syncwarp();
-        const uint32_t rounds = (q.Wv + 31) / 32, below = (1u << lane) - 1u;
-        for (uint32_t k = po.ni; k-- > 0;) {
-            const uint32_t i = i0 + k;
-            uint32_t at = __shfl_sync(0xffffffffu, my_lo, k), at_s = at - ls_sub - i * ls_mul;
-            for (uint32_t r = 0; r < rounds; ++r) {
-                const uint32_t w = r * 32 + lane;
-                const uint32_t mine = w < q.Wv ? s_live[w] : 0u;
-                const uint32_t mine_th = w < q.Wv ? s_th[w] : 0u;
-                uint32_t nz = __ballot_sync(0xffffffffu, mine != 0);
-                while (nz) {
-                    const uint32_t src = __ffs(nz) - 1;
-                    nz &= nz - 1;
-                    const uint32_t x = __shfl_sync(0xffffffffu, mine, src);
-                    const uint32_t y = x & ~__shfl_sync(0xffffffffu, mine_th, src);
-                    const uint32_t id = (r * 32 + src) * 32 + lane;
-                    if ((x >> lane) & 1u) q.lo[at + __popc(x & below)] = id;
-                    if ((y >> lane) & 1u) q.ls[at_s + __popc(y & below)] = id;
-                    at += __popc(x);
-                    at_s += __popc(y);
+        for (uint32_t r = 0; r < po.n; r += 32) {
+            const uint32_t x = r == 0 ? x0 : po.get(q, r + lane);
+            if (r + lane < po.n) atomicOr(&s_u[po_vreg(x) >> 5], 1u << (x & 31));
+        }
+        __syncwarp();
+        uint32_t at[PIECE_INSTRS], as[PIECE_INSTRS];  // where the lists of instruction k go on
+#pragma unroll
+        for (uint32_t k = 0; k < PIECE_INSTRS; ++k) {
+            at[k] = __shfl_sync(0xffffffffu, my_lo, k);
+            as[k] = at[k] - ls_sub - (i0 + k) * ls_mul;
+        }
+        const uint32_t below = low_bits(lane), is_instr = 0xFFu & ~low_bits(PIECE_INSTRS - po.ni);  // bit 7 - k: instruction k
+        for (uint32_t w0 = 0; w0 < q.Wv; w0 += 32) {  // (at most 1,024 members at a time)
+            const uint32_t w = w0 + lane;
+            const uint32_t u = w < q.Wv ? s_u[w] : 0u, e = w < q.Wv ? s_end[w] : 0u, t = w < q.Wv ? th[w] : 0u;
+            if (!__any_sync(0xffffffffu, u != 0)) continue;
+            const uint32_t n_own = __popc(u);
+            uint32_t inc = n_own;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= (uint32_t)d) inc += y;
+            }
+            const uint32_t rank0 = inc - n_own, n_mem = __shfl_sync(0xffffffffu, inc, 31);
+            s_rank[lane] = rank0;
+            // every lane lists its own word, or the warp word by word, whichever is shorter
+            uint32_t words = __ballot_sync(0xffffffffu, u != 0);
+            if (__reduce_max_sync(0xffffffffu, n_own) <= 2 * __popc(words)) {
+                uint32_t rest = u, rank = rank0;
+                for (; rest; rest &= rest - 1, ++rank) {
+                    const uint32_t j = __ffs(rest) - 1;
+                    s_mem[rank] = w * 32 + j;
+                    s_flag[rank] = (uint8_t)(((e >> j) & 1u) | (((t >> j) & 1u) << 1));
+                }
+            } else {
+                for (; words; words &= words - 1) {
+                    const uint32_t src = __ffs(words) - 1;
+                    const uint32_t us = __shfl_sync(0xffffffffu, u, src), es = __shfl_sync(0xffffffffu, e, src);
+                    const uint32_t ts = __shfl_sync(0xffffffffu, t, src), rank = __shfl_sync(0xffffffffu, rank0, src) + __popc(us & below);
+                    if ((us >> lane) & 1u) {
+                        s_mem[rank] = (w0 + src) * 32 + lane;
+                        s_flag[rank] = (uint8_t)(((es >> lane) & 1u) | (((ts >> lane) & 1u) << 1));
+                    }
                 }
             }
-            if (lane == k) my_n = at - my_lo - ls_mul;
             __syncwarp();
-            for (uint32_t r = 0; r < po.n; r += 32) {  // live before the instruction: without its definitions ...
-                const uint32_t x = r == 0 ? x0 : po.get(q, r + lane);
-                if (r + lane < po.n && po_instr(x) == k && po_def(x)) atomicAnd(&s_live[po_vreg(x) >> 5], ~(1u << (x & 31)));
+            for (uint32_t r = 0; r < po.n; r += 32) {  // bits 16 + 7 - k, 24 + 7 - k: instruction k reads, defines the member
+                const uint32_t x = r == 0 ? x0 : po.get(q, r + lane), v = po_vreg(x);
+                if (r + lane < po.n && v >> 10 == w0 >> 5)
+                    atomicOr(&s_mem[s_rank[(v >> 5) & 31] + __popc(s_u[v >> 5] & low_bits(v & 31))],
+                             1u << ((po_def(x) ? 31u : 23u) - po_instr(x)));
             }
             __syncwarp();
-            for (uint32_t r = 0; r < po.n; r += 32) {  // ... with its reads
-                const uint32_t x = r == 0 ? x0 : po.get(q, r + lane);
-                if (r + lane < po.n && po_instr(x) == k && !po_def(x)) atomicOr(&s_live[po_vreg(x) >> 5], 1u << (x & 31));
+            for (uint32_t m0 = 0; m0 < n_mem; m0 += 32) {
+                const bool ok = m0 + lane < n_mem;
+                const uint32_t x = ok ? s_mem[m0 + lane] : 0u, flag = ok ? s_flag[m0 + lane] : 0u;
+                // live after instruction k iff the next instruction that touches the member reads it (in the piece's last
+                // stretch: iff it is live after the piece).  That is a carry that a read generates and a definition stops,
+                // from the last instruction to the first: an addition.
+                const uint32_t rd = (x >> 16) & 0xFFu, pass = (~(x >> 24) & 0xFFu) | rd;
+                const uint32_t mask = ok ? (rd ^ pass ^ (rd + pass + (flag & 1u))) & is_instr : 0u;
+                const uint32_t short_lanes = ~__ballot_sync(0xffffffffu, flag & 2u);
+#pragma unroll
+                for (uint32_t k = 0; k < PIECE_INSTRS; ++k) {
+                    const bool live = (mask >> (PIECE_INSTRS - 1 - k)) & 1u;
+                    const uint32_t b_lo = __ballot_sync(0xffffffffu, live), b_ls = b_lo & short_lanes;
+                    if (live) {
+                        q.lo[at[k] + __popc(b_lo & below)] = x & 0xFFFFu;
+                        if (!(flag & 2u)) q.ls[as[k] + __popc(b_ls & below)] = x & 0xFFFFu;
+                    }
+                    at[k] += __popc(b_lo);
+                    as[k] += __popc(b_ls);
+                }
             }
             __syncwarp();
         }
-        const uint32_t n_reads = __shfl_down_sync(0xffffffffu, po.off, 1) - po.off - po.nd;
+        uint32_t my_n = 0;  // lane k: length of the short list of instruction k
+#pragma unroll
+        for (uint32_t k = 0; k < PIECE_INSTRS; ++k)
+            if (lane == k) my_n = at[k] - my_lo - ls_mul;
         if (lane < po.ni)
             q.irec[i0 + lane] = make_uint4(my_lo - ls_sub - (i0 + lane) * ls_mul,
-                                           my_n | (po.nd << 16) | (min(n_reads, 127u) << 24) | (po.nd && bit_get(s_th, v0) ? 0x80000000u : 0u), v0, po.off);
+                                           my_n | (nd_k << 16) | (min(n_reads, 127u) << 24) | (th0 << 31), v0, o_k);
         return;
     }
     pdl_wait();
@@ -829,7 +1232,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
         const size_t base = q.cev_off[c];
         const uint32_t n_entry = q.centry_cnt[c], n_ev = n_entry + q.chunk_ev[c];
         if (warp == 0)
-            warp_bits(q.Wv, lane, [&](uint32_t w) { return entry_word(q, c, p0, p0, b, w); },
+            warp_bits(q.Wv, lane, [&](uint32_t w) { return live_before(q, c, p0, p0, w) & ~q.blk_th[(size_t)b * q.Wv + w]; },
                       [&](uint32_t rank, uint32_t v) { put_event(q.ev, base + rank, v, q.width[v], true, true); });
         const uint32_t i1 = q.chunk_i1[c];
         for (uint32_t i = q.chunk_i0[c] + (tid + LV_NT - 32) % LV_NT; i < i1; i += LV_NT) {
@@ -859,7 +1262,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
         if (s < q.nS) {
             const uint32_t p = q.short_p0[s], c = q.piece_chunk[p], b = q.chunk_blk[c], p0 = q.chunk_piece_off[c];
             const uint32_t ent0 = q.sen_off[s];
-            warp_bits(q.Wv, lane, [&](uint32_t w) { return entry_word(q, c, p, p0, b, w); },
+            warp_bits(q.Wv, lane, [&](uint32_t w) { return live_before(q, c, p, p0, w) & ~q.blk_th[(size_t)b * q.Wv + w]; },
                       [&](uint32_t rank, uint32_t v) { q.sen[ent0 + rank] = v | (s << 16); });
             const uint32_t i0 = q.piece_i0[p];
             const uint32_t i1 = s + 1 < q.chunk_short_off[c + 1] ? q.piece_i0[q.short_p0[s + 1]] : q.chunk_i1[c];
@@ -901,14 +1304,15 @@ int live_attributes(vl_program *p)
     std::lock_guard<std::mutex> lock(mtx);
     if (done[p->device]) return VL_OK;
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1, false>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1, true>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_flow<1>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_fill<1>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY, false>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY, true>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_flow<LV_MANY>, at, 227 * 1024));
     VL_CUDA(p, cudaFuncSetAttribute(k_fill<LV_MANY>, at, 227 * 1024));
+    VL_CUDA(p, cudaFuncSetAttribute(k_small<1, 1>, at, SMALL_SMEM));
+    VL_CUDA(p, cudaFuncSetAttribute(k_small<1, SMALL_BLOCKS>, at, SMALL_SMEM));
+    VL_CUDA(p, cudaFuncSetAttribute(k_small<LV_MANY, SMALL_BLOCKS>, at, SMALL_SMEM));
     done[p->device] = true;
     return VL_OK;
 }
@@ -937,7 +1341,7 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     p->tables_built = false;
     p->d_vreg16 = nullptr; p->d_first8 = nullptr; p->d_opoff = nullptr; p->d_first4 = nullptr;
     p->d_first_def_instr = nullptr; p->d_vinfo = nullptr; p->d_first_occ = nullptr;
-    std::vector<uint32_t> c_i0, c_i1, c_blk, blk_c_off(nB + 1, 0), p_i0, p_chunk, c_p_off, seg_c0, blk_seg_off(nB + 1, 0);
+    std::vector<uint32_t> c_i0, c_i1, c_blk, blk_c_off(nB + 1, 0), p_i0, p_o0, p_chunk, c_p_off, seg_c0, blk_seg_off(nB + 1, 0);
     for (uint32_t b = 0; b < nB; ++b) {
         const uint64_t s = p->h_blk_off[b], n = p->h_blk_off[b + 1] - s;
         uint64_t nc = (n + p->chunk_instrs - 1) / p->chunk_instrs;
@@ -947,7 +1351,8 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         for (uint64_t j = 0; j < nc; ++j) {
             const uint32_t i0 = (uint32_t)(s + j * n / nc), i1 = (uint32_t)(s + (j + 1) * n / nc);
             c_p_off.push_back((uint32_t)p_i0.size());
-            for (uint32_t q0 = i0; q0 < i1; q0 += PIECE_INSTRS) {
+            for (uint32_t q0 = i0, q1; q0 < i1; q0 = q1) {
+                for (q1 = q0 + 1; q1 < i1 && q1 < q0 + PIECE_INSTRS && p->h_op_off[q1 + 1] - p->h_op_off[q0] <= PIECE_OPERANDS;) ++q1;
                 p_i0.push_back(q0);
                 p_chunk.push_back((uint32_t)c_i0.size());
             }
@@ -958,13 +1363,12 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         blk_c_off[b + 1] = (uint32_t)c_i0.size();
     }
     c_p_off.push_back((uint32_t)p_i0.size());
+    p_i0.push_back(p->nI);
+    for (uint32_t i : p_i0) p_o0.push_back(p->h_op_off[i]);
     p->wide_pieces = false;
-    for (size_t j = 0; j < p_i0.size(); ++j) {
-        const uint32_t i1 = std::min(p_i0[j] + PIECE_INSTRS, c_i1[p_chunk[j]]);
-        p->wide_pieces = p->wide_pieces || p->h_op_off[i1] - p->h_op_off[p_i0[j]] > WIDE_OPERANDS;
-    }
+    for (size_t j = 0; j + 1 < p_o0.size(); ++j) p->wide_pieces = p->wide_pieces || p_o0[j + 1] - p_o0[j] > PIECE_OPERANDS;
     const uint32_t nC = p->nC = (uint32_t)c_i0.size();
-    p->nP = (uint32_t)p_i0.size();
+    p->nP = (uint32_t)p_chunk.size();
     // segments of k_flow: at most about 256 of them beside one per block
     const uint32_t seg = std::max<uint32_t>(SEG_CHUNKS, (nC + 255) / 256);
     for (uint32_t b = 0; b < nB; ++b) {
@@ -996,20 +1400,39 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     for (uint32_t b = 0; b <= nB; ++b) b_s_off.push_back(c_s_off[blk_c_off[b]]);
     p->short_len = 1;
     for (uint32_t j = 0; j < p->nS; ++j) p->short_len = std::max(p->short_len, s_i0[j + 1] - s_i0[j]);
+    // shares of the thread blocks of k_small: whole chunks, about equally many pieces; then that of a single one
+    std::vector<uint32_t> share, share_c0(SMALL_BLOCKS + 1, nC);
+    p->share_pieces = p->share_ops = 0;
+    for (uint32_t r = 0; r < SMALL_BLOCKS; ++r) {
+        const uint32_t want = (uint32_t)((uint64_t)p->nP * r / SMALL_BLOCKS);
+        share_c0[r] = (uint32_t)(std::lower_bound(c_p_off.begin(), c_p_off.end(), want) - c_p_off.begin());
+    }
+    share_c0.push_back(0);
+    share_c0.push_back(nC);
+    for (uint32_t c : share_c0)
+        for (uint32_t x : {c, c_p_off[c], p_i0[c_p_off[c]], p_o0[c_p_off[c]]}) share.push_back(x);
+    for (uint32_t r = 0; r < SMALL_BLOCKS; ++r) {
+        p->share_pieces = std::max(p->share_pieces, share[4 * r + 5] - share[4 * r + 1]);
+        p->share_ops = std::max(p->share_ops, share[4 * r + 7] - share[4 * r + 3]);
+    }
     std::vector<uint32_t> all;
     struct Part { uint32_t **dst; const std::vector<uint32_t> *v; };
-    const Part parts[] = {{&p->d_chunk_i0, &c_i0}, {&p->d_chunk_i1, &c_i1}, {&p->d_chunk_blk, &c_blk},
-                          {&p->d_blk_chunk_off, &blk_c_off}, {&p->d_piece_i0, &p_i0}, {&p->d_piece_chunk, &p_chunk},
-                          {&p->d_chunk_piece_off, &c_p_off}, {&p->d_seg_c0, &seg_c0}, {&p->d_blk_seg_off, &blk_seg_off},
-                          {&p->d_short_p0, &s_p0}, {&p->d_chunk_short_off, &c_s_off}, {&p->d_short_blk, &s_blk},
-                          {&p->d_short_i0, &s_i0},
-                          {&p->d_blk_short_off, &b_s_off}, {&p->d_short_chunk, &s_chunk}};
+    uint32_t *d_share = nullptr, *none = nullptr;
+    const Part parts[] = {{&d_share, &share},
+                          // (side by side, see SmallSmem)
+                          {&p->d_blk_chunk_off, &blk_c_off}, {&p->d_chunk_piece_off, &c_p_off}, {&p->d_chunk_blk, &c_blk},
+                          {&p->d_chunk_short_off, &c_s_off}, {&p->d_short_p0, &s_p0}, {&p->d_short_chunk, &s_chunk}, {&none, &p->h_blk_off},
+                          {&none, &p->h_succ_off}, {&none, &p->h_succ},
+                          {&p->d_chunk_i0, &c_i0}, {&p->d_chunk_i1, &c_i1}, {&p->d_piece_i0, &p_i0}, {&p->d_piece_o0, &p_o0},
+                          {&p->d_piece_chunk, &p_chunk}, {&p->d_seg_c0, &seg_c0}, {&p->d_blk_seg_off, &blk_seg_off}, {&p->d_short_blk, &s_blk},
+                          {&p->d_short_i0, &s_i0}, {&p->d_blk_short_off, &b_s_off}};
     for (const Part &x : parts) {
         all.insert(all.end(), x.v->begin(), x.v->end());
         all.resize((all.size() + 4) & ~(size_t)3);  // (at least one word behind every array)
     }
     uint32_t *dev = nullptr;
     p->layout_arena.hint = all.size() * 4 + (size_t)p->V * 12 + (size_t)p->nOp8 * 3 + (size_t)p->nOpT * 5 + 16384;
+    if (p->nO <= 65536) p->layout_arena.hint += (size_t)p->nO * 4;  // (else the operand words have a slab of their own)
     LAYOUT(&dev, all.size());
     VL_CUDA(p, cudaMemcpy(dev, all.data(), all.size() * 4, cudaMemcpyHostToDevice));
     size_t at = 0;
@@ -1017,6 +1440,11 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         *x.dst = dev + at;
         at = (at + x.v->size() + 4) & ~(size_t)3;
     }
+    p->d_share = reinterpret_cast<uint4 *>(d_share);
+    LAYOUT(&p->d_op_word, (size_t)p->nO);
+    LAUNCH(k_operand_words, (p->nP + NT / 32 - 1) / (NT / 32), NT, 0, st, p->nP, p->d_piece_i0, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_op_word);
+    VL_CUDA(p, cudaGetLastError());
+    VL_CUDA(p, cudaStreamSynchronize(st));  // (the first kernels of a run read the layout before they wait for the stream)
     const uint32_t Wp = (p->P + p->wmax + 31) / 32 + 1;
     p->use_th = (nB <= 32 && (uint64_t)nB * VL_MAX_GROUP * Wp * 4 <= 24 * 1024) ? 1 : 0;
     p->layout_chunk_instrs = p->chunk_instrs;
@@ -1025,12 +1453,14 @@ static int vl_layout(vl_program *p, cudaStream_t st)
 
 // What a run's launches need besides the arguments.
 struct LiveShape {
-    bool wide = false;
+    bool wide = false, small = false;  // small: k_small takes the program
+    size_t small_smem = 0;
     uint32_t set_warps = PC_WARPS, sets = 0, flows = 0, counts = 0, offs = 0, fills = 0;
     size_t sets_smem = 0, flow_smem = 0, count_smem = 0, fill_smem = 0;
     void add(const LiveShape &o)
     {
         wide = wide || o.wide;
+        small_smem = std::max(small_smem, o.small_smem);
         set_warps = std::min(set_warps, o.set_warps);
         sets = std::max(sets, o.sets); flows = std::max(flows, o.flows); counts = std::max(counts, o.counts);
         offs = std::max(offs, o.offs); fills = std::max(fills, o.fills);
@@ -1081,7 +1511,7 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg; q.succ_off = p->d_succ_off; q.succ = p->d_succ; q.blk_off = p->d_blk_off;
     q.ndefs = p->d_ndefs; q.width = p->d_width;
     q.chunk_i0 = p->d_chunk_i0; q.chunk_i1 = p->d_chunk_i1; q.chunk_blk = p->d_chunk_blk; q.blk_chunk_off = p->d_blk_chunk_off;
-    q.piece_i0 = p->d_piece_i0; q.piece_chunk = p->d_piece_chunk; q.chunk_piece_off = p->d_chunk_piece_off;
+    q.piece_i0 = p->d_piece_i0; q.piece_o0 = p->d_piece_o0; q.op_word = p->d_op_word; q.piece_chunk = p->d_piece_chunk; q.chunk_piece_off = p->d_chunk_piece_off;
     q.seg_c0 = p->d_seg_c0; q.blk_seg_off = p->d_blk_seg_off; q.short_p0 = p->d_short_p0; q.chunk_short_off = p->d_chunk_short_off;
     KEEP(&q.piece_use, (size_t)nP * Wv);
     KEEP(&q.piece_def, (size_t)nP * Wv);
@@ -1120,11 +1550,14 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     sh.fills = (nP + LV_WARPS - 1) / LV_WARPS + nC + ((p->nS + 31) & ~31u) / LV_WARPS + nB;
     sh.sets_smem = (size_t)sh.set_warps * 2 * Wv * 4;
     sh.wide = p->wide_pieces;
-    sh.count_smem = p->wide_pieces ? (size_t)PC_WARPS * 2 * Wv * 4 : 0;
+    sh.count_smem = p->wide_pieces ? (size_t)PC_WARPS * Wv * 4 : 0;
     q.wide_smem = sh.count_smem <= 40 * 1024;
     if (!q.wide_smem) sh.count_smem = 0;
     sh.flow_smem = flow_smem;
-    sh.fill_smem = (size_t)LV_WARPS * 2 * Wv * 4;
+    q.share = p->d_share; q.small_tab = p->d_blk_chunk_off;
+    sh.small_smem = q.small.init(nB, p->nE, nC, p->nS, Wv, p->share_pieces, p->share_ops);
+    sh.small = nI <= LIVE_SMALL_INSTRS && nC && sh.small_smem <= SMALL_SMEM;
+    sh.fill_smem = (size_t)LV_WARPS * (2 * Wv + FILL_WARP_WORDS) * 4;
     return VL_OK;
 }
 
@@ -1172,28 +1605,67 @@ static int live_tables(vl_program *p, cudaStream_t st)
     return VL_OK;
 }
 
-// The first four kernels of the runs of n <= N programs, or the last one.
+// k_small for the runs of n <= N programs, C thread blocks each.
+template <int N, int C>
+static int launch_small(vl_program *p, const LiveMany<N> &many, uint32_t n, size_t smem, cudaStream_t st)
+{
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = C; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(C, n); cfg.blockDim = SMALL_NT; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = at; cfg.numAttrs = C > 1 ? 2 : 1;
+    g_vl_launches.fetch_add(1);
+    VL_CUDA(p, cudaLaunchKernelEx(&cfg, k_small<N, C>, many));
+    return VL_OK;
+}
+
+// The kernels of the runs of n <= N programs up to the list lengths, or the last one.
 template <int N>
 static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *args, const LiveShape *shapes, bool fill,
                        cudaStream_t st)
 {
     vl_program *p = progs[0];
-    LiveShape sh;
     LiveMany<N> many;
-    for (uint32_t j = 0; j < n; ++j) {
-        sh.add(shapes[j]);
-        many.p[j] = args[j];
-    }
     if (fill) {
+        LiveShape sh;
+        for (uint32_t j = 0; j < n; ++j) {
+            sh.add(shapes[j]);
+            many.p[j] = args[j];
+        }
         VL_CUDA(p, launch_overlap(k_fill<N>, dim3(sh.fills, n), LV_NT, sh.fill_smem, st, true, many));
         return VL_OK;
     }
-    if (sh.wide) VL_CUDA(p, launch_overlap(k_sets<N, true>, dim3(sh.sets, n), sh.set_warps * 32, sh.sets_smem, st, true, many));
-    else VL_CUDA(p, launch_overlap(k_sets<N, false>, dim3(sh.sets, n), sh.set_warps * 32, sh.sets_smem, st, true, many));
-    VL_CUDA(p, launch_overlap(k_flow<N>, dim3(sh.flows, n), FLOW_WARPS * 32, sh.flow_smem, st, true, many));
-    if (sh.counts && sh.wide) VL_CUDA(p, launch_overlap(k_count<N, true>, dim3(sh.counts, n), PC_NT, sh.count_smem, st, true, many));
-    else if (sh.counts) VL_CUDA(p, launch_overlap(k_count<N, false>, dim3(sh.counts, n), PC_NT, 0, st, true, many));
-    VL_CUDA(p, launch_overlap(k_offsets<N>, dim3(sh.offs, n), OFF_NT, 0, st, true, many));
+    for (const bool small : {true, false}) {
+        LiveShape sh;
+        uint32_t m = 0;
+        for (uint32_t j = 0; j < n; ++j) {
+            if (shapes[j].small != small) continue;
+            sh.add(shapes[j]);
+            many.p[m++] = args[j];
+        }
+        if (!m) continue;
+        if (small) {
+            SmallSmem one;
+            const uint32_t one_smem = one.init(p->nB, p->nE, p->nC, p->nS, p->Wv, p->nP, p->nO);
+            int rc;
+            if (N == 1 && p->nP <= SMALL_ONE_PIECES && one_smem <= SMALL_SMEM) {
+                many.p[0].small = one;
+                rc = launch_small<N, N == 1 ? 1 : SMALL_BLOCKS>(p, many, m, one_smem, st);
+            } else {
+                rc = launch_small<N, SMALL_BLOCKS>(p, many, m, sh.small_smem, st);
+            }
+            if (rc != VL_OK) return rc;
+            continue;
+        }
+        VL_CUDA(p, launch_overlap(k_sets<N>, dim3(sh.sets, m), sh.set_warps * 32, sh.sets_smem, st, true, many));
+        VL_CUDA(p, launch_overlap(k_flow<N>, dim3(sh.flows, m), FLOW_WARPS * 32, sh.flow_smem, st, true, many));
+        if (sh.counts && sh.wide) VL_CUDA(p, launch_overlap(k_count<N, true>, dim3(sh.counts, m), PC_NT, sh.count_smem, st, true, many));
+        else if (sh.counts) VL_CUDA(p, launch_overlap(k_count<N, false>, dim3(sh.counts, m), PC_NT, 0, st, true, many));
+        VL_CUDA(p, launch_overlap(k_offsets<N>, dim3(sh.offs, m), OFF_NT, 0, st, true, many));
+    }
     return VL_OK;
 }
 
