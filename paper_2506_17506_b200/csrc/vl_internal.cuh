@@ -16,10 +16,14 @@ enum : uint8_t {
     OPF_DUP = 4,    // read: same vreg read earlier by this instruction
     OPF_ELIDE = 8,  // definition of a vreg the instruction also reads and that stays live:
                     //   occupancy unchanged, no walk event
-    OPF_SET = 16,   // definition: becomes occupied (live after, or several defs in the instruction)
-    OPF_POST = 32,  // definition: dead, released again after the instruction's definitions
-    OPF_DEAD = 64   // definition: vreg not live after the instruction
+    OPF_DEAD = 64   // definition: vreg not live after the instruction: released again behind the instruction's definitions
 };
+
+// ---- a walk event of k_eight: byte offset of the vreg's 16-byte table entry (bits 4 to 17), whether it tests, and the mask of
+// its width, at most 8 registers, that it toggles (0: no event)
+#define EV8_OFFSET 0x3FFF0u
+#define EV8_TEST 1u
+#define EV8_MASK_SHIFT 24
 
 enum : uint32_t { VINFO_OCCURS = 1u << 8, VINFO_DEFINED = 1u << 9 };
 
@@ -149,6 +153,7 @@ struct vl_program {
     uint4 *d_el = nullptr;
     uint32_t *d_el_count = nullptr;
     uint32_t *d_cev_off = nullptr;  // [nC+1] first walk event of each chunk (every chunk padded to 8 events)
+    uint32_t *d_ev8 = nullptr;      // walk events of k_eight, at the same places; null if it does not take the program
     uint4 *d_ev = nullptr;          // walk events, 112 bytes per group of 8, chunk after chunk
     // events of the short chunks, 4 bytes each, 32 short chunks side by side: steps [sev_off[g], sev_off[g + 1]) of
     // group g, [step][32]; and what is occupied when short chunk s begins, vreg | s << 16, [sen_off[s], sen_off[s + 1])
@@ -201,7 +206,7 @@ struct vl_program {
         uint32_t *thm = nullptr;       // [groups][n_blocks][mask words][2][32] through-set masks
         uint64_t rows = 0, aw = 0, vregs = 0, chunks = 0;
     } vs[VL_LANES + 2];              // one per lane, then one per staging buffer of vl_verify_host
-    VScratch fs[VL_LANES + 2];       // the same for what k_fused hands to k_exact: cstate, anom and racc only
+    VScratch fs[VL_LANES + 2];       // the same for what k_fused and k_eight hand to k_exact: cstate, anom and racc only
     uint32_t sub_batch = 5120;       // candidates per pass of the verify kernels
     uint32_t lanes_opt = 3;          // lanes in use (1 = everything in order on the caller's stream)
     uint64_t lane_call = 0, lane_base = 0;  // the last vl_verify* call that spread passes over lanes, the lane of its first
@@ -267,6 +272,14 @@ bool vl_fused_wanted(vl_program *p, uint64_t K);
 // that occupies many.
 #define FUSED_MANY_ENTRIES 49152u  // (measured at vl_fused_wanted)
 bool vl_verify_takes(const vl_program *p);  // whether the verify path takes the program (vl_verify.cu)
+// The one-kernel verify path with eight candidates per thread block (vl_eight.cu): whether it takes a program at all, whether
+// it is the one for a job of K rows, whether the job may share a launch, and one launch for n <= VL_EIGHT_MANY jobs.
+#define VL_EIGHT_MANY 48
+bool vl_eight_takes(const vl_program *p);
+bool vl_eight_wanted(vl_program *p, uint64_t K);
+bool vl_eight_shares(vl_program *p, uint64_t K);
+int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
+                 vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot);  // slot: working set, -1: none
 bool vl_fused_shares(vl_program *p, uint64_t K);
 int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
                  vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot);  // slot: working set, -1: none
@@ -310,9 +323,11 @@ struct VlExactArgs {
     const uint32_t *short_chunk, *chunk_short_off;  // [nS] chunk of every short chunk, [nC + 1] first short chunk of every chunk
     uint32_t *racc;               // [rows][4] overlaps, complement of the lowest instruction, bank tally, parts done; all 0
     uint32_t AW, nC, fine_items;      // fine_items: up to that many fine items are taken
-    uint32_t rows;                // k_fused's rows, each of which left the number of its items (and an exact bank tally) in cstate; 0: listed in work
+    uint32_t rows;                // rows of k_fused or k_eight, each of which left the number of its items in cstate; 0: listed in work
+    uint32_t exact_bank;          // and an exact bank tally (k_fused)
     unsigned char *scratch;       // vl_exact_scratch bytes, null if 0
 };
+int vl_hand_scratch(vl_program *p, int slot, uint64_t rows, VlExactArgs *ex);  // what k_fused or k_eight share with k_exact
 uint32_t vl_exact_blocks(vl_program *p);  // thread blocks of k_exact: one item each at a time
 uint64_t vl_exact_scratch(vl_program *p);
 bool vl_exact_takes_rows(vl_program *p, uint64_t rows);  // whether k_exact can count for that many rows of k_fused

@@ -97,7 +97,7 @@ struct LiveArgs {
     const uint32_t *small_tab;
     SmallSmem small;
     // results
-    uint32_t *blk_in, *blk_out, *lo_off, *lo, *ls, *ls_adj, *blk_th, *th_cnt, *th_off, *th, *cev_off, *sev_off, *sev, *sen_off, *sen;
+    uint32_t *blk_in, *blk_out, *lo_off, *lo, *ls, *ls_adj, *blk_th, *th_cnt, *th_off, *th, *cev_off, *ev8, *sev_off, *sev, *sen_off, *sen;
     uint8_t *opflags;
     uint4 *ev, *el, *irec;
     uint32_t *el_count, *status;
@@ -159,8 +159,7 @@ enum : uint32_t {
     OW_OTHER = 1u << 22,    // the instruction's other side (reads / writes) has the vreg
     OW_EXPOSED = 1u << 23,  // read: no earlier instruction of the piece writes the vreg
     OW_LATER = 1u << 24,    // a later instruction of the piece touches the vreg ...
-    OW_READ = 1u << 25,     // ... and the first such reads it
-    OW_MANY = 1u << 26      // the instruction has several definitions
+    OW_READ = 1u << 25      // ... and the first such reads it
 };
 struct Piece {
     uint32_t i0, ni, o0, n;  // first instruction, instructions; first operand, operands
@@ -351,19 +350,18 @@ __global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const __grid_constant_
     }
 }
 
-// An operand's flags, and the walk events that it makes.  many: the instruction has several definitions; lv: its vreg is live
-// after the instruction; dup: an earlier read of the instruction has the vreg; other: the instruction's other side
-// (reads / writes) has it.
-__device__ __forceinline__ uint32_t operand_events(bool many, bool def, bool lv, bool dup, bool other, uint32_t *flags)
+// An operand's flags, and the walk events that it makes.  lv: its vreg is live after the instruction; dup: an earlier read of
+// the instruction has the vreg; other: the instruction's other side (reads / writes) has it.
+__device__ __forceinline__ uint32_t operand_events(bool def, bool lv, bool dup, bool other, uint32_t *flags)
 {
     if (!def) {
         const bool kill = !dup && !lv;  // a read of a vreg that stays live releases nothing
         *flags = (kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0);
         return kill ? 1u : 0u;
     }
-    const bool elide = other && lv, post = !lv && many;
-    *flags = OPF_DEF | (elide ? OPF_ELIDE : 0) | ((lv || many) ? OPF_SET : 0) | (post ? OPF_POST : 0) | (lv ? 0 : OPF_DEAD);
-    return elide ? 0u : 1u + (post ? 1u : 0u);
+    const bool elide = other && lv;
+    *flags = OPF_DEF | (elide ? OPF_ELIDE : 0) | (lv ? 0 : OPF_DEAD);
+    return elide ? 0u : (lv ? 1u : 2u);  // (a dead definition occupies and releases)
 }
 
 // The operands of a piece of at most 32, one per lane: flags, touched vregs, and per instruction the events (s_ev) and what it
@@ -382,7 +380,7 @@ __device__ __forceinline__ void count_narrow(const Piece &po, uint32_t x, const 
         const bool lv = x & OW_LATER ? (x & OW_READ) != 0 : (end[v >> 5] >> (v & 31)) & 1u;
         const bool dup = x & OW_DUP, other = x & OW_OTHER;
         uint32_t flags;
-        evs = operand_events(x & OW_MANY, def, lv, dup, other, &flags);
+        evs = operand_events(def, lv, dup, other, &flags);
         opflags[lane] = (uint8_t)flags;
         // a read: live before the instruction, but not among what is live behind it and not written by it
         up = !def && !dup && !(lv && !other);
@@ -422,7 +420,7 @@ __device__ __noinline__ void count_wide(const LiveArgs &q, const Piece &po, cons
         if (mine) {
             uint32_t flags;
             if (!dup) atomicOr(const_cast<uint32_t *>(reads) + (v >> 5), 1u << (v & 31));
-            event(v, operand_events(nd > 1, false, has(end, v), dup, false, &flags));
+            event(v, operand_events(false, has(end, v), dup, false, &flags));
             opflags[o - po.o0 + lane] = (uint8_t)flags;
         }
         __syncwarp();
@@ -430,7 +428,7 @@ __device__ __noinline__ void count_wide(const LiveArgs &q, const Piece &po, cons
     for (uint32_t o = po.o0 + lane; o < r0; o += 32) {
         const uint32_t v = q.op_vreg[o];
         uint32_t flags;
-        event(v, operand_events(nd > 1, true, has(end, v), false, has(reads, v), &flags));
+        event(v, operand_events(true, has(end, v), false, has(reads, v), &flags));
         opflags[o - po.o0] = (uint8_t)flags;
     }
     __syncwarp();
@@ -967,7 +965,7 @@ __global__ void __launch_bounds__(NT) k_operand_words(uint32_t nP, const uint32_
     if (mine) {
         uint32_t i = i0;
         while (op_off[i + 1] <= o0 + lane) ++i;
-        x = op_vreg[o0 + lane] | ((i - i0) << 16) | (o0 + lane - op_off[i] < ndefs[i] ? OW_DEF : 0u) | (ndefs[i] > 1 ? OW_MANY : 0u);
+        x = op_vreg[o0 + lane] | ((i - i0) << 16) | (o0 + lane - op_off[i] < ndefs[i] ? OW_DEF : 0u);
     }
     const uint32_t here = same_instr(x, mine), same = __match_any_sync(0xffffffffu, mine ? po_vreg(x) : 0x10000u + lane);
     const uint32_t defs = __ballot_sync(0xffffffffu, mine && po_def(x));
@@ -1033,15 +1031,17 @@ __global__ void k_operand_tables(uint32_t nO, uint32_t nOp8, uint32_t n_padded, 
 // (likewise), wl[8] (16 bit: 32 - width; the range straddles a 32-bit word iff
 // (register & 31) > wl).  Ranges wider than 32 registers carry wl = 0x8000 | width and
 // toggle, test as 0/1 flags.  A no-op names the spare vreg V with empty masks.
-__device__ __forceinline__ void put_event(uint4 *ev, size_t idx, uint32_t v, uint32_t w, bool test, bool toggle)
+// And once more in 4 bytes for k_eight, where it takes the program: EV8_* (vl_internal.cuh).
+__device__ __forceinline__ void put_event(const LiveArgs &q, size_t idx, uint32_t v, uint32_t w, bool test, bool toggle)
 {
-    unsigned char *g = reinterpret_cast<unsigned char *>(ev) + (idx >> 3) * 112;
+    unsigned char *g = reinterpret_cast<unsigned char *>(q.ev) + (idx >> 3) * 112;
     const uint32_t slot = (uint32_t)(idx & 7);
     const uint32_t wm = w > 32 ? 1u : (w == 32 ? 0xFFFFFFFFu : ((1u << w) - 1u));
     reinterpret_cast<uint32_t *>(g)[slot] = v * 128u;
     reinterpret_cast<uint32_t *>(g + 32)[slot] = toggle ? wm : 0u;
     reinterpret_cast<uint32_t *>(g + 64)[slot] = test ? wm : 0u;
     reinterpret_cast<uint16_t *>(g + 96)[slot] = (uint16_t)(w > 32 ? (0x8000u | w) : (32u - w));
+    if (q.ev8) q.ev8[idx] = v * 16u | (test ? EV8_TEST : 0u) | (toggle ? wm << EV8_MASK_SHIFT : 0u);
 }
 
 // ============================================================================ k_fill
@@ -1075,22 +1075,23 @@ __device__ __forceinline__ uint32_t warp_bits(uint32_t Wv, uint32_t lane, W word
 }
 
 // The walk events of instruction i in order: the releases of dying reads, the definitions, the releases of dead
-// co-definitions: put(index, vreg, test, toggle).  skip(operand) is called for definitions without an event.
+// definitions: put(index, vreg, test), all of them toggle.  skip(operand) is called for definitions without an event.
 template <class F, class G>
 __device__ __forceinline__ void instr_events(const LiveArgs &q, uint32_t i, F put, G skip)
 {
     const uint32_t o0 = q.op_off[i], o1 = q.op_off[i + 1], nd = q.ndefs[i];
-    uint32_t e = 0;
+    uint32_t e = 0, dead = 0;
     for (uint32_t o = o0 + nd; o < o1; ++o)
-        if (q.opflags[o] & OPF_KILL) put(e++, q.op_vreg[o], false, true);
+        if (q.opflags[o] & OPF_KILL) put(e++, q.op_vreg[o], false);
     for (uint32_t o = o0; o < o0 + nd; ++o) {
         const uint32_t f = q.opflags[o];
         if (f & OPF_ELIDE) skip(o);
-        else put(e++, q.op_vreg[o], true, (f & OPF_SET) != 0);
+        else put(e++, q.op_vreg[o], true);
+        dead |= f & OPF_DEAD;
     }
-    if (nd > 1)
+    if (dead)
         for (uint32_t o = o0; o < o0 + nd; ++o)
-            if ((q.opflags[o] & OPF_POST) && !(q.opflags[o] & OPF_ELIDE)) put(e++, q.op_vreg[o], false, true);
+            if (q.opflags[o] & OPF_DEAD) put(e++, q.op_vreg[o], false);
 }
 
 template <int N>
@@ -1233,11 +1234,11 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
         const uint32_t n_entry = q.centry_cnt[c], n_ev = n_entry + q.chunk_ev[c];
         if (warp == 0)
             warp_bits(q.Wv, lane, [&](uint32_t w) { return live_before(q, c, p0, p0, w) & ~q.blk_th[(size_t)b * q.Wv + w]; },
-                      [&](uint32_t rank, uint32_t v) { put_event(q.ev, base + rank, v, q.width[v], true, true); });
+                      [&](uint32_t rank, uint32_t v) { put_event(q, base + rank, v, q.width[v], true, true); });
         const uint32_t i1 = q.chunk_i1[c];
         for (uint32_t i = q.chunk_i0[c] + (tid + LV_NT - 32) % LV_NT; i < i1; i += LV_NT) {
             const size_t at = base + n_entry + q.ev_rel[i];
-            instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) { put_event(q.ev, at + e, v, q.width[v], test, toggle); },
+            instr_events(q, i, [&](uint32_t e, uint32_t v, bool test) { put_event(q, at + e, v, q.width[v], test, true); },
                          [&](uint32_t o) {  // listed (in any order) for the exact counts of through-set collisions
                              uint32_t s = q.chunk_short_off[c];
                              while (s + 1 < q.chunk_short_off[c + 1] && q.piece_i0[q.short_p0[s + 1]] <= i) ++s;
@@ -1247,12 +1248,12 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
         }
         // no-ops up to a whole group, and two no-op groups behind the last chunk (the walk reads ahead)
         const uint32_t n_pad = (8u - (n_ev & 7u)) % 8u + (c == q.nC - 1 ? 16u : 0u);
-        if (tid < n_pad) put_event(q.ev, base + n_ev + tid, q.V, 1u, false, false);
+        if (tid < n_pad) put_event(q, base + n_ev + tid, q.V, 1u, false, false);
         return;
     }
     role -= q.nC;
     if (role < n_short) {
-        // Events of a short chunk, 4 bytes each: vreg | width << 16 | test << 24 | toggle << 25; 32 short chunks side
+        // Events of a short chunk, 4 bytes each: vreg | width << 16 | test << 24; 32 short chunks side
         // by side, step by step, padded with zeros to the longest of the 32.  What is occupied on entry (and not
         // through the whole block) is a list of its own, vreg | short chunk << 16: those need no order.
         const uint32_t s = role * LV_WARPS + warp;
@@ -1269,8 +1270,8 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
             const uint32_t ev0 = q.ev_rel[i0];
             for (uint32_t i = i0 + lane; i < i1; i += 32) {
                 const uint32_t at = q.ev_rel[i] - ev0;
-                instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) {
-                    dst[(size_t)(at + e) * 32] = v | ((uint32_t)q.width[v] << 16) | (test ? 1u << 24 : 0u) | (toggle ? 1u << 25 : 0u);
+                instr_events(q, i, [&](uint32_t e, uint32_t v, bool test) {
+                    dst[(size_t)(at + e) * 32] = v | ((uint32_t)q.width[v] << 16) | (test ? 1u << 24 : 0u);
                 }, [](uint32_t) {});
             }
             n = q.short_ev[s];
@@ -1578,14 +1579,15 @@ static int live_lengths(vl_program *p, LiveArgs &q)
     }
     p->lo_len = p->known[LV_TOT_LO];
     p->live_arena.hint = 4 * (p->known[LV_TOT_LO] + p->known[LV_TOT_LS] + p->known[LV_TOT_TH] + p->known[LV_TOT_SEV] + p->known[LV_TOT_SEN]) +
-                         14 * p->known[LV_TOT_EV] + 8 * 512;
+                         18 * p->known[LV_TOT_EV] + 9 * 512;
     KEEP(&p->d_lo, (size_t)p->lo_len);
     KEEP(&p->d_ls, (size_t)p->known[LV_TOT_LS]);
     KEEP(&p->d_ev, (size_t)(p->known[LV_TOT_EV] / 8 + 2) * 7);  // two no-op groups behind the last chunk
+    if (vl_eight_takes(p)) KEEP(&p->d_ev8, (size_t)p->known[LV_TOT_EV] + 16);
     KEEP(&p->d_th, (size_t)p->known[LV_TOT_TH]);
     KEEP(&p->d_sev, (size_t)p->known[LV_TOT_SEV]);
     KEEP(&p->d_sen, (size_t)p->known[LV_TOT_SEN]);
-    q.lo = p->d_lo; q.ls = p->d_ls; q.ev = p->d_ev; q.th = p->d_th; q.sev = p->d_sev; q.sen = p->d_sen;
+    q.lo = p->d_lo; q.ls = p->d_ls; q.ev = p->d_ev; q.ev8 = p->d_ev8; q.th = p->d_th; q.sev = p->d_sev; q.sen = p->d_sen;
     return VL_OK;
 }
 

@@ -16,7 +16,8 @@
 //            has no overlap.  The thread block that ends a group of 64 candidates writes the verdicts
 //            of its clean candidates and lists the others for k_exact
 //            (vl_fused.cu), which counts their overlaps from the per-instruction live-after lists.
-// Jobs of up to a few hundred rows take one kernel instead (k_fused, vl_fused.cu).
+// Jobs of up to a few hundred rows take one kernel instead (k_fused, vl_fused.cu), jobs of up to a few thousand another (k_eight,
+// vl_eight.cu).
 #include <cuda.h>
 
 #include <algorithm>
@@ -24,7 +25,7 @@
 #include <mutex>
 #include <type_traits>
 
-#include "vl_internal.cuh"
+#include "vl_ptx.cuh"
 
 #define MAX_STAGES 4
 #define TGW 64  // candidates side by side per vreg in the tables handed from the table kernel to the walk
@@ -101,67 +102,6 @@ struct WParams {
     uint32_t *grp_done, *work;
     vl_verdict *out;
 };
-
-// ------------------------------------------------------------------ PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ uint32_t mbar_try_wait(unsigned long long *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok;
-}
-// Bulk async copy global -> this block's shared memory, completion counted on `bar`.
-// dst, src 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, unsigned long long *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-// Tiled copy of one box of a 3-D tensor (coordinates innermost first) into this block's shared memory,
-// completion counted on `bar` with the full size of the box (elements outside the tensor arrive as
-// zeros).  dst 128-byte aligned; the innermost coordinate times the element size a multiple of 16.
-__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *tm, uint32_t x, uint32_t y, uint32_t z,
-                                            unsigned long long *bar, unsigned long long policy)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(
-            smem_u32(dst)),
-        "l"(tm), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy)
-        : "memory");
-}
-// Tiled bulk store of one box from shared memory (elements outside the tensor are not written); completion is
-// tracked by the issuing thread's bulk async-groups.
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap *tm, uint32_t x, uint32_t y, uint32_t z, const void *src)
-{
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                 ::"l"(tm), "r"(x), "r"(y), "r"(z), "r"(smem_u32(src))
-                 : "memory");
-}
-
-// L2 policy for data that is read once: first in line for eviction, so that it does not push out what
-// other kernels are about to read again.
-__device__ __forceinline__ unsigned long long l2_policy_evict_first()
-{
-    unsigned long long policy;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-    return policy;
-}
 
 // ------------------------------------------------------------- packed table access
 // In shared memory T holds, per vreg, the G candidates' registers side by side (16 bits each).
@@ -569,36 +509,6 @@ __global__ void __launch_bounds__(NT) k_tables(const TParams q)
 // transposes them with byte permutes, stores first occurrences, and compares the occurrences of the
 // tile before (whose first occurrences a barrier has already ordered) while the current tile's loads
 // are in flight: one barrier per tile, no dependent wait behind it.
-__device__ __forceinline__ uint32_t pk8_get(const uint4 &x, int g)
-{
-    const uint32_t w = (g >> 1) == 0 ? x.x : ((g >> 1) == 1 ? x.y : ((g >> 1) == 2 ? x.z : x.w));
-    return (g & 1) ? (w >> 16) : (w & 0xFFFFu);
-}
-
-template <int NT>
-__device__ __noinline__ void rules_sweep8(const uint4 *vcons, const uint16_t *rs_prefix, const uint32_t *vinfo,
-                                          const uint32_t *first_def_instr, uint32_t V, uint32_t P, const uint4 *T,
-                                          TMisc *M)
-{
-    for (uint32_t v = threadIdx.x; v < V; v += NT) {
-        const uint32_t vi = vinfo[v];
-        if (!(vi & VINFO_DEFINED)) continue;
-        const uint4 vc = vcons[v];
-        const uint32_t clo = vc.x & 0xFFFFu, chi = vc.x >> 16, al = vc.y, recip = vc.z, w = vi & 0xFFu;
-        const uint4 tt = T[v];
-#pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const uint32_t tv = pk8_get(tt, g);
-            bool bad = (al > 1 && tv != __umulhi(tv, recip) * al) || tv < clo || tv + w > chi;
-            if (!bad && rs_prefix) bad = rs_prefix[min(tv + w, P)] != rs_prefix[min(tv, P)];
-            if (bad) {
-                atomicOr(&M->flags[g], (uint32_t)VL_OUT_OF_RANGE);
-                atomicMin(&M->minR[g], first_def_instr[v]);
-            }
-        }
-    }
-}
-
 template <int NT>
 __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const __grid_constant__ CUtensorMap tm,
                                                           const __grid_constant__ CUtensorMap tmg)
@@ -874,7 +784,7 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
     // matter.)  Bound by instruction issue; as two sweeps, with a shift per candidate for the nibbles, it took 16.5 k
     // cycles per block on 10,000 vregs, now 10.
     // (From here on the producer warp only keeps the block's barriers company.)
-    if (q.vcons && tid < NT) rules_sweep8<NT>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, M);
+    if (q.vcons && tid < NT) rules_sweep8<NT>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, M->flags, M->minR);
     if (tid < NT) {
         uint32_t mk = 0, mk2 = 0, mk3 = 0, mk4 = 0;
         const uint32_t bm = q.Bmask * 0x10001u;
@@ -1865,6 +1775,7 @@ int vl_verify_impl(vl_program *p, const uint16_t *d_cand, uint64_t K, uint64_t p
     if (vl_fused_wanted(p, K)) {
         return vl_fused_run(1, &p, &d_cand, &K, &pitch, &d_out, st, st, dict, slot);
     }
+    if (vl_eight_wanted(p, K)) return vl_eight_run(1, &p, &d_cand, &K, &pitch, &d_out, st, st, dict, slot);
     PassPlan pp{};
     int rc = plan_passes(p, K, &pp);
     if (rc != VL_OK) return rc;
@@ -1889,18 +1800,18 @@ struct FusedGroup {
         progs[n] = p; cand[n] = c; K[n] = k; pitch[n] = pt; out[n] = o;
         return ++n == VL_FUSED_MANY;
     }
-    int run(cudaStream_t from, cudaStream_t st, bool dict)
+    int run(cudaStream_t from, cudaStream_t st, bool dict, bool eight = false)
     {
         const uint32_t m = n;
         n = 0;
-        return vl_fused_run(m, progs, cand, K, pitch, out, from, st, dict, -1);
+        return eight ? vl_eight_run(m, progs, cand, K, pitch, out, from, st, dict, -1) : vl_fused_run(m, progs, cand, K, pitch, out, from, st, dict, -1);
     }
 };
 }  // namespace
 
 namespace {
-// How the short jobs of several programs run: in shared launches, in a launch each, or by the batched kernels.
-enum Together { SHARED, SINGLE, BATCHED };
+// How the short jobs of several programs run: in shared launches (of k_fused, of k_eight), in a launch each, or by the batched kernels.
+enum Together { SHARED, SINGLE, BATCHED, EIGHT };
 
 // The rows of all of them decide, not those of one.  Estimates in microseconds, from 2 to 96 programs of 2,000 to 26,000
 // instructions with 20 to 148 rows each, 15 % failing: a shared launch takes rounds of three rows per multiprocessor and is as
@@ -1908,9 +1819,14 @@ enum Together { SHARED, SINGLE, BATCHED };
 // four launches per program over the lanes.  Measured / estimated, shared, single, batched: 96 x 2,000 x 148 rows 470/550,
 // 913/1,227, 1,004/1,828; 8 x 8,000 x 50 121/128, 91/109, 201/222; 8 x 20,000 x 148 366/371, 306/307, 259/262; 48 x 20,000 x 100
 // 860/908, 977/1,199, 1,035/1,107; 48 x 26,000 x 148 1,522/1,571, 1,752/2,003, 1,307/1,276; 2 x 14,000 x 100 175/169, 86/74, 140/113.
+// The kernel with eight candidates per block (EIGHT, if it takes every one of the jobs) takes rounds of two blocks per
+// multiprocessor.  In EIGHT / in the best of the others, us: 96 programs of 2,000 instructions with 148 rows 207 / 536, 48 of 4,000 with
+// 128 163 / 343, 16 of 4,000 with 100 73 / 103, 16 of 2,000 with 100 49 / 70, 8 of 8,000 with 100 100 / 91, 4 of 2,000 with 100 45 / 35,
+// 64 of 2,000 with 8 90 / 83.
 Together together(uint32_t nprog, vl_program *const *progs, const uint64_t *K, const std::vector<uint8_t> &shares)
 {
-    double n = 0, rows = 0, work = 0, longest = 0;
+    double n = 0, rows = 0, work = 0, longest = 0, blocks = 0;
+    bool eights = true;
     for (uint32_t j = 0; j < nprog; ++j) {
         if (!shares[j]) continue;
         const double a = progs[j]->nI / 1000.0;
@@ -1918,12 +1834,16 @@ Together together(uint32_t nprog, vl_program *const *progs, const uint64_t *K, c
         rows += (double)K[j];
         work += a * (double)K[j];
         longest = std::max(longest, a);
+        blocks += (double)((K[j] + 7) / 8);
+        eights = eights && vl_eight_shares(progs[j], K[j]);
     }
     if (n < 2) return SINGLE;
     const double sms = vl_sm_count(progs[0]), a = work / rows;
     const double shared = 35 + 8 * longest + rows / (3 * sms) * (10 + 2.8 * a);
     const double single = 35 + 4 * n + rows / sms * (6 + 1.2 * a);
     const double batched = 75 + 17.7 * n + 0.0019 * work;
+    const double eight = 40 + 12 * longest + blocks / (2 * sms) * (10 + 12.3 * a);
+    if (eights && eight <= shared && eight <= single && eight <= batched) return EIGHT;
     return shared <= single && shared <= batched ? SHARED : (single <= batched ? SINGLE : BATCHED);
 }
 }  // namespace
@@ -1944,6 +1864,8 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     const uint32_t L = p0->lanes_opt == 1 ? 1u : (nprog > 1 ? (uint32_t)VL_LANES : std::min<uint32_t>(VL_LANES, p0->lanes_opt));
     uint64_t jobs = 0;
     for (uint32_t j = 0; j < nprog; ++j) jobs += (K[j] + progs[j]->sub_batch - 1) / progs[j]->sub_batch;
+    // one launch, however many the rows
+    if (nprog == 1 && !vl_fused_wanted(p0, K[0]) && vl_eight_wanted(p0, K[0])) return vl_eight_run(1, progs, d_cand, K, pitch, d_out, st, st, dict, 0);
     if (L == 1 || jobs <= 1) {
         FusedGroup g;
         for (uint32_t j = 0; j < nprog; ++j) {
@@ -1967,15 +1889,15 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     for (uint32_t j = 0; j < nprog && nprog > 1; ++j) shares[j] = K[j] != 0 && vl_fused_shares(progs[j], K[j]);
     FusedGroup g;
     const Together how = nprog > 1 ? together(nprog, progs, K, shares) : SINGLE;
-    for (uint32_t j = 0; j < nprog && how == SHARED && rc == VL_OK; ++j) {
+    for (uint32_t j = 0; j < nprog && (how == SHARED || how == EIGHT) && rc == VL_OK; ++j) {
         if (!shares[j]) continue;
-        if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j])) rc = g.run(st, lane[job++ % L], dict);
+        if (g.add(progs[j], d_cand[j], K[j], pitch[j], d_out[j])) rc = g.run(st, lane[job++ % L], dict, how == EIGHT);
     }
-    if (rc == VL_OK && g.n) rc = g.run(st, lane[job++ % L], dict);
+    if (rc == VL_OK && g.n) rc = g.run(st, lane[job++ % L], dict, how == EIGHT);
     for (uint32_t j = 0; j < nprog && rc == VL_OK; ++j) {
         if (K[j] == 0) continue;
         vl_program *p = progs[j];
-        if (how == SHARED && shares[j]) continue;
+        if ((how == SHARED || how == EIGHT) && shares[j]) continue;
         if (!(how == BATCHED && shares[j]) && vl_fused_wanted(p, K[j])) {
             rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, st, lane[job % L], dict, (int)(job % L));
             ++job;

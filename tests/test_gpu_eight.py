@@ -1,0 +1,92 @@
+"""The verify path with eight candidates per thread block: at the edges of what it takes (rows, tiles, widths, register files)
+and on both sides of its rules, against the CPU oracle, every verdict field, exact."""
+import numpy as np
+import pytest
+
+from paper_2506_17506_b200 import synth
+from tests import helpers as H
+from tests.test_gpu_parity import _assert_same, _garbage_rows, _gpu_verify, _to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2506_17506_b200 import binding
+    return binding
+
+
+def _member(n_instrs, seed):
+    shape = synth.Shape("loop", [n_instrs // 4, n_instrs - n_instrs // 4], [(0, 1), (1, 1)], [(1, 1)], [],
+                        n_vregs=n_instrs * 2 // 5, widths={1: 0.7, 2: 0.2, 4: 0.1}, P=200)
+    return synth.build_program(shape, seed)
+
+
+def _rows(p, K, seed):
+    """Valid rows, rows with one fault, and garbage: many collisions, registers outside the file."""
+    rows, _ = synth.candidate_rows(p, K, 0.4, seed)
+    rows[5: K: 29] = _garbage_rows(p, K, seed)[5: K: 29]
+    return rows
+
+
+# rows: 512 threads, 256 threads, counts handed over or made by the block itself, a block with a single row; columns: whole tiles,
+# one more, few
+@pytest.mark.parametrize("n_instrs,K", [(2000, 889), (2000, 1500), (2000, 2001), (2001, 1184), (2003, 1185), (1500, 3001), (4000, 800)])
+def test_row_counts(B, oracle_mod, n_instrs, K):
+    p = _member(n_instrs, n_instrs + K)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    rows = _rows(p, K, K)
+    want = op.verify(lv, rows)
+    for _ in range(2):
+        _assert_same(_gpu_verify(B, gp, rows), want, f"{n_instrs} instructions, {K} rows")
+    drows = synth.dict_rows(p, rows)
+    got = B.verdicts_to_numpy(gp.vl_verify_dict(_to_dev(drows)))
+    _assert_same(got, op.verify_dict(lv, drows), "dictionary rows")
+    gp.close()
+
+
+# register files that end inside and at a mask word, widths at 8 (taken) and 9 (not), banks, more blocks than through-sets serve
+@pytest.mark.parametrize("P,widths,banks,max_blocks", [(32, (1, 2, 4), 4, 4), (33, (1, 3, 8), 2, 6), (64, (1, 9), 4, 4),
+                                                       (500, (1, 2, 4, 8), 1, 8), (2000, (8,), 4, 40), (64, (1, 2), 3, 4)])
+def test_random_programs(B, oracle_mod, P, widths, banks, max_blocks):
+    for seed in range(3):
+        p = H.random_program(8800 + seed, max_instrs=1800, max_vregs=300, max_blocks=max_blocks, P=P, widths=widths, B=banks)
+        gp = B.Program(p)
+        gp.vl_liveness()
+        op = oracle_mod.OracleProgram(p)
+        if seed == 1:
+            rules = dict(vreg_align=np.where(p.vreg_width > 1, 2, 1), reserved=[p.P - 1])
+            op.set_constraints(**rules)
+            gp.set_constraints(P=p.P, **rules)
+        K = 3000
+        rows = np.tile(_garbage_rows(p, 300, seed), (10, 1))
+        want = np.tile(op.verify(op.liveness(), rows[:300]), 10)
+        _assert_same(_gpu_verify(B, gp, rows[:K]), want, f"P {P} seed {seed}")
+        gp.close()
+
+
+def test_several_programs(B, oracle_mod):
+    """Jobs of several programs in one call, enough of them for the kernel to take them together; one that it does not take."""
+    import torch
+    progs = [_member(900 + 331 * j, j) for j in range(9)]
+    Ks = [100, 131, 8, 1, 97, 200, 148, 120, 90]
+    gps = [B.Program(p) for p in progs]
+    B.vl_liveness_batch(gps)
+    rows = [_rows(p, K, K) for p, K in zip(progs, Ks)]
+    wants = []
+    for p, r in zip(progs, rows):
+        op = oracle_mod.OracleProgram(p)
+        wants.append(op.verify(op.liveness(), r))
+    for reps in (1, 4):
+        outs = B.vl_verify_batch(gps * reps, [_to_dev(r) for r in rows] * reps)
+        torch.cuda.synchronize()
+        for o, w in zip(outs, wants * reps):
+            _assert_same(B.verdicts_to_numpy(o), w)
+    for gp in gps:
+        gp.close()
