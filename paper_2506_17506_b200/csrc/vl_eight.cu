@@ -12,7 +12,7 @@
 // A vreg at or beyond P takes part in step 4 as if it sat at P: two of them live together then collide, so that a chunk is
 // never missed, and step 5 compares the true registers.
 #include <algorithm>
-#include <mutex>
+#include <type_traits>
 
 #include "vl_exact.cuh"
 #include "vl_ptx.cuh"
@@ -82,12 +82,12 @@ __device__ __noinline__ uint32_t apply_far(const uint32_t *ev, uint32_t entry, u
         const uint32_t w = ev[u], pos = lds_u16(entry + (w & EV8_OFFSET)) & 0x7FFFu;
         const unsigned long long m = (unsigned long long)(w >> EV8_MASK_SHIFT) << (pos & 31);
         uint32_t *a = occ + (pos >> 5) * NT;
-        const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32), o0 = a[0];
-        a[0] = o0 ^ lo;
+        const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32), o0 = a[0], tog = w & EV8_HOLD ? 0u : 0xFFFFFFFFu;
+        a[0] = o0 ^ (lo & tog);
         uint32_t hit = o0 & lo;
         if (hi) {
             const uint32_t o1 = a[NT];
-            a[NT] = o1 ^ hi;
+            a[NT] = o1 ^ (hi & tog);
             hit |= o1 & hi;
         }
         if (w & EV8_TEST) viol |= hit;
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     m[u] = __funnelshift_l(0u, w[u] >> EV8_MASK_SHIFT, t[u]);
-                    t[u] = atom_xor(occ_addr + (t[u] & 0x7FE0u) * (NT / 8), m[u]);
+                    t[u] = atom_xor(occ_addr + (t[u] & 0x7FE0u) * (NT / 8), w[u] & EV8_HOLD ? 0u : m[u]);
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
@@ -669,8 +669,10 @@ EPlan eight_plan(vl_program *p, uint64_t K)
 }
 
 template <int NT, int N, bool HAND>
-cudaError_t launch_eight(const EMany<N> &many, dim3 grid, uint32_t smem, cudaStream_t st)
+cudaError_t launch_eight(int device, const EMany<N> &many, dim3 grid, uint32_t smem, cudaStream_t st)
 {
+    const cudaError_t e = allow_smem<k_eight<NT, N, HAND>, 227 * 1024>(device);
+    if (e != cudaSuccess) return e;
     return launch_overlap(k_eight<NT, N, HAND>, grid, NT + 32, smem, st, true, many);
 }
 }  // namespace
@@ -702,20 +704,6 @@ int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
                  vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot)
 {
     vl_program *p0 = progs[0];
-    static std::mutex mtx;
-    static bool done[64];
-    if (p0->device >= 0 && p0->device < 64) {
-        std::lock_guard<std::mutex> lock(mtx);
-        if (!done[p0->device]) {
-            const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-            VL_CUDA(p0, cudaFuncSetAttribute(k_eight<512, 1, true>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_eight<256, 1, true>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_eight<512, 1, false>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_eight<256, 1, false>, at, 227 * 1024));
-            VL_CUDA(p0, cudaFuncSetAttribute(k_eight<256, VL_EIGHT_MANY, false>, at, 227 * 1024));
-            done[p0->device] = true;
-        }
-    }
     uint64_t rows = 0;
     uint32_t smem = 0, NT = 256;
     EMany<VL_EIGHT_MANY> many;
@@ -756,7 +744,7 @@ int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
     mark(1);
     const uint32_t blocks = (uint32_t)((rows + 7) / 8);
     if (n > 1) {
-        VL_CUDA(p0, (launch_eight<256, VL_EIGHT_MANY, false>(many, dim3(blocks, n), smem, st)));
+        VL_CUDA(p0, (launch_eight<256, VL_EIGHT_MANY, false>(p0->device, many, dim3(blocks, n), smem, st)));
     } else {
         EMany<1> one;
         one.p[0] = many.p[0];
@@ -765,15 +753,15 @@ int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
             const int rc = vl_hand_scratch(p0, slot, rows, &ex);
             if (rc != VL_OK) return rc;
             ex.exact_bank = 0;
-            if (NT == 512) VL_CUDA(p0, (launch_eight<512, 1, true>(one, dim3(blocks), smem, st)));
-            else VL_CUDA(p0, (launch_eight<256, 1, true>(one, dim3(blocks), smem, st)));
+            if (NT == 512) VL_CUDA(p0, (launch_eight<512, 1, true>(p0->device, one, dim3(blocks), smem, st)));
+            else VL_CUDA(p0, (launch_eight<256, 1, true>(p0->device, one, dim3(blocks), smem, st)));
             mark(3);
             const int re = vl_exact_run(p0, ex, d_cand[0], pitch[0], d_out[0], st, dict, true);
             mark(1);
             return re;
         }
-        if (NT == 512) VL_CUDA(p0, (launch_eight<512, 1, false>(one, dim3(blocks), smem, st)));
-        else VL_CUDA(p0, (launch_eight<256, 1, false>(one, dim3(blocks), smem, st)));
+        if (NT == 512) VL_CUDA(p0, (launch_eight<512, 1, false>(p0->device, one, dim3(blocks), smem, st)));
+        else VL_CUDA(p0, (launch_eight<256, 1, false>(p0->device, one, dim3(blocks), smem, st)));
     }
     mark(4);
     return VL_OK;

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
 #pragma unroll
                 for (int u = 0; u < EU; ++u) {
                     const uint32_t w = (x[u] >> 16) & 0xFFu, m = w ? (0xFFFFFFFFu >> (32 - w)) << (t[u] & 31) : 0u;
-                    old[u] = atomicXor(&occ[(t[u] >> 5) * NTHR + tid], m);
+                    old[u] = atomicXor(&occ[(t[u] >> 5) * NTHR + tid], (x[u] >> 25) & 1u ? m : 0u);
                     t[u] = (x[u] >> 24) & 1u ? m : 0u;
                 }
 #pragma unroll
@@ -285,12 +285,12 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
 #pragma unroll
                     for (int j = 1; j < EU; ++j)
                         if (j == u) { xu = x[j]; pos = t[j]; }
-                    const uint32_t test = 0u - ((xu >> 24) & 1u);
+                    const uint32_t tog = 0u - ((xu >> 25) & 1u), test = 0u - ((xu >> 24) & 1u);
                     uint32_t left = (xu >> 16) & 0xFFu;
                     while (left) {
                         const uint32_t s2 = pos & 31, n = min(left, 32 - s2);
                         const uint32_t m = (0xFFFFFFFFu >> (32 - n)) << s2;
-                        viol |= atomicXor(&occ[(pos >> 5) * NTHR + tid], m) & m & test;
+                        viol |= atomicXor(&occ[(pos >> 5) * NTHR + tid], m & tog) & m & test;
                         pos += n;
                         left -= n;
                     }

@@ -16,13 +16,16 @@ enum : uint8_t {
     OPF_DUP = 4,    // read: same vreg read earlier by this instruction
     OPF_ELIDE = 8,  // definition of a vreg the instruction also reads and that stays live:
                     //   occupancy unchanged, no walk event
-    OPF_DEAD = 64   // definition: vreg not live after the instruction: released again behind the instruction's definitions
+    OPF_SET = 16,   // definition: becomes occupied (live after, or several defs in the instruction)
+    OPF_POST = 32,  // definition: dead, released again after the instruction's definitions
+    OPF_DEAD = 64   // definition: vreg not live after the instruction
 };
 
-// ---- a walk event of k_eight: byte offset of the vreg's 16-byte table entry (bits 4 to 17), whether it tests, and the mask of
-// its width, at most 8 registers, that it toggles (0: no event)
+// ---- a walk event of k_eight: byte offset of the vreg's 16-byte table entry (bits 4 to 17), whether it tests, whether it leaves
+// the occupancy as it is, and the mask of its width, at most 8 registers (0: no event)
 #define EV8_OFFSET 0x3FFF0u
 #define EV8_TEST 1u
+#define EV8_HOLD 2u
 #define EV8_MASK_SHIFT 24
 
 enum : uint32_t { VINFO_OCCURS = 1u << 8, VINFO_DEFINED = 1u << 9 };
@@ -252,6 +255,18 @@ static inline cudaError_t launch_overlap(void (*kernel)(P...), dim3 grid, uint32
     cfg.attrs = &at; cfg.numAttrs = overlap ? 1 : 0;
     g_vl_launches.fetch_add(1);
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Lets a kernel use that many bytes of dynamic shared memory: asked for once per device, in front of its first launch (asking
+// makes the driver load a kernel, also one that the process never uses).
+template <auto kernel, int bytes>
+static inline cudaError_t allow_smem(int device)
+{
+    static std::atomic<bool> done[64];
+    if (device >= 0 && device < 64 && done[device].load()) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && device >= 0 && device < 64) done[device].store(true);
+    return e;
 }
 
 #define VL_CUDA(prog, call)                     \

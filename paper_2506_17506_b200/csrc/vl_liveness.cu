@@ -159,7 +159,8 @@ enum : uint32_t {
     OW_OTHER = 1u << 22,    // the instruction's other side (reads / writes) has the vreg
     OW_EXPOSED = 1u << 23,  // read: no earlier instruction of the piece writes the vreg
     OW_LATER = 1u << 24,    // a later instruction of the piece touches the vreg ...
-    OW_READ = 1u << 25      // ... and the first such reads it
+    OW_READ = 1u << 25,     // ... and the first such reads it
+    OW_MANY = 1u << 26      // the instruction has several definitions
 };
 struct Piece {
     uint32_t i0, ni, o0, n;  // first instruction, instructions; first operand, operands
@@ -350,18 +351,19 @@ __global__ void __launch_bounds__(FLOW_WARPS * 32) k_flow(const __grid_constant_
     }
 }
 
-// An operand's flags, and the walk events that it makes.  lv: its vreg is live after the instruction; dup: an earlier read of
-// the instruction has the vreg; other: the instruction's other side (reads / writes) has it.
-__device__ __forceinline__ uint32_t operand_events(bool def, bool lv, bool dup, bool other, uint32_t *flags)
+// An operand's flags, and the walk events that it makes.  many: the instruction has several definitions; lv: its vreg is live
+// after the instruction; dup: an earlier read of the instruction has the vreg; other: the instruction's other side
+// (reads / writes) has it.
+__device__ __forceinline__ uint32_t operand_events(bool many, bool def, bool lv, bool dup, bool other, uint32_t *flags)
 {
     if (!def) {
         const bool kill = !dup && !lv;  // a read of a vreg that stays live releases nothing
         *flags = (kill ? OPF_KILL : 0) | (dup ? OPF_DUP : 0);
         return kill ? 1u : 0u;
     }
-    const bool elide = other && lv;
-    *flags = OPF_DEF | (elide ? OPF_ELIDE : 0) | (lv ? 0 : OPF_DEAD);
-    return elide ? 0u : (lv ? 1u : 2u);  // (a dead definition occupies and releases)
+    const bool elide = other && lv, post = !lv && many;
+    *flags = OPF_DEF | (elide ? OPF_ELIDE : 0) | ((lv || many) ? OPF_SET : 0) | (post ? OPF_POST : 0) | (lv ? 0 : OPF_DEAD);
+    return elide ? 0u : 1u + (post ? 1u : 0u);
 }
 
 // The operands of a piece of at most 32, one per lane: flags, touched vregs, and per instruction the events (s_ev) and what it
@@ -380,7 +382,7 @@ __device__ __forceinline__ void count_narrow(const Piece &po, uint32_t x, const 
         const bool lv = x & OW_LATER ? (x & OW_READ) != 0 : (end[v >> 5] >> (v & 31)) & 1u;
         const bool dup = x & OW_DUP, other = x & OW_OTHER;
         uint32_t flags;
-        evs = operand_events(def, lv, dup, other, &flags);
+        evs = operand_events(x & OW_MANY, def, lv, dup, other, &flags);
         opflags[lane] = (uint8_t)flags;
         // a read: live before the instruction, but not among what is live behind it and not written by it
         up = !def && !dup && !(lv && !other);
@@ -420,7 +422,7 @@ __device__ __noinline__ void count_wide(const LiveArgs &q, const Piece &po, cons
         if (mine) {
             uint32_t flags;
             if (!dup) atomicOr(const_cast<uint32_t *>(reads) + (v >> 5), 1u << (v & 31));
-            event(v, operand_events(false, has(end, v), dup, false, &flags));
+            event(v, operand_events(nd > 1, false, has(end, v), dup, false, &flags));
             opflags[o - po.o0 + lane] = (uint8_t)flags;
         }
         __syncwarp();
@@ -428,7 +430,7 @@ __device__ __noinline__ void count_wide(const LiveArgs &q, const Piece &po, cons
     for (uint32_t o = po.o0 + lane; o < r0; o += 32) {
         const uint32_t v = q.op_vreg[o];
         uint32_t flags;
-        event(v, operand_events(true, has(end, v), false, has(reads, v), &flags));
+        event(v, operand_events(nd > 1, true, has(end, v), false, has(reads, v), &flags));
         opflags[o - po.o0] = (uint8_t)flags;
     }
     __syncwarp();
@@ -965,7 +967,7 @@ __global__ void __launch_bounds__(NT) k_operand_words(uint32_t nP, const uint32_
     if (mine) {
         uint32_t i = i0;
         while (op_off[i + 1] <= o0 + lane) ++i;
-        x = op_vreg[o0 + lane] | ((i - i0) << 16) | (o0 + lane - op_off[i] < ndefs[i] ? OW_DEF : 0u);
+        x = op_vreg[o0 + lane] | ((i - i0) << 16) | (o0 + lane - op_off[i] < ndefs[i] ? OW_DEF : 0u) | (ndefs[i] > 1 ? OW_MANY : 0u);
     }
     const uint32_t here = same_instr(x, mine), same = __match_any_sync(0xffffffffu, mine ? po_vreg(x) : 0x10000u + lane);
     const uint32_t defs = __ballot_sync(0xffffffffu, mine && po_def(x));
@@ -1041,7 +1043,7 @@ __device__ __forceinline__ void put_event(const LiveArgs &q, size_t idx, uint32_
     reinterpret_cast<uint32_t *>(g + 32)[slot] = toggle ? wm : 0u;
     reinterpret_cast<uint32_t *>(g + 64)[slot] = test ? wm : 0u;
     reinterpret_cast<uint16_t *>(g + 96)[slot] = (uint16_t)(w > 32 ? (0x8000u | w) : (32u - w));
-    if (q.ev8) q.ev8[idx] = v * 16u | (test ? EV8_TEST : 0u) | (toggle ? wm << EV8_MASK_SHIFT : 0u);
+    if (q.ev8) q.ev8[idx] = v * 16u | (test ? EV8_TEST : 0u) | (toggle ? 0u : EV8_HOLD) | (test || toggle ? wm << EV8_MASK_SHIFT : 0u);
 }
 
 // ============================================================================ k_fill
@@ -1075,23 +1077,22 @@ __device__ __forceinline__ uint32_t warp_bits(uint32_t Wv, uint32_t lane, W word
 }
 
 // The walk events of instruction i in order: the releases of dying reads, the definitions, the releases of dead
-// definitions: put(index, vreg, test), all of them toggle.  skip(operand) is called for definitions without an event.
+// co-definitions: put(index, vreg, test, toggle).  skip(operand) is called for definitions without an event.
 template <class F, class G>
 __device__ __forceinline__ void instr_events(const LiveArgs &q, uint32_t i, F put, G skip)
 {
     const uint32_t o0 = q.op_off[i], o1 = q.op_off[i + 1], nd = q.ndefs[i];
-    uint32_t e = 0, dead = 0;
+    uint32_t e = 0;
     for (uint32_t o = o0 + nd; o < o1; ++o)
-        if (q.opflags[o] & OPF_KILL) put(e++, q.op_vreg[o], false);
+        if (q.opflags[o] & OPF_KILL) put(e++, q.op_vreg[o], false, true);
     for (uint32_t o = o0; o < o0 + nd; ++o) {
         const uint32_t f = q.opflags[o];
         if (f & OPF_ELIDE) skip(o);
-        else put(e++, q.op_vreg[o], true);
-        dead |= f & OPF_DEAD;
+        else put(e++, q.op_vreg[o], true, (f & OPF_SET) != 0);
     }
-    if (dead)
+    if (nd > 1)
         for (uint32_t o = o0; o < o0 + nd; ++o)
-            if (q.opflags[o] & OPF_DEAD) put(e++, q.op_vreg[o], false);
+            if ((q.opflags[o] & OPF_POST) && !(q.opflags[o] & OPF_ELIDE)) put(e++, q.op_vreg[o], false, true);
 }
 
 template <int N>
@@ -1238,7 +1239,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
         const uint32_t i1 = q.chunk_i1[c];
         for (uint32_t i = q.chunk_i0[c] + (tid + LV_NT - 32) % LV_NT; i < i1; i += LV_NT) {
             const size_t at = base + n_entry + q.ev_rel[i];
-            instr_events(q, i, [&](uint32_t e, uint32_t v, bool test) { put_event(q, at + e, v, q.width[v], test, true); },
+            instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) { put_event(q, at + e, v, q.width[v], test, toggle); },
                          [&](uint32_t o) {  // listed (in any order) for the exact counts of through-set collisions
                              uint32_t s = q.chunk_short_off[c];
                              while (s + 1 < q.chunk_short_off[c + 1] && q.piece_i0[q.short_p0[s + 1]] <= i) ++s;
@@ -1253,7 +1254,7 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
     }
     role -= q.nC;
     if (role < n_short) {
-        // Events of a short chunk, 4 bytes each: vreg | width << 16 | test << 24; 32 short chunks side
+        // Events of a short chunk, 4 bytes each: vreg | width << 16 | test << 24 | toggle << 25; 32 short chunks side
         // by side, step by step, padded with zeros to the longest of the 32.  What is occupied on entry (and not
         // through the whole block) is a list of its own, vreg | short chunk << 16: those need no order.
         const uint32_t s = role * LV_WARPS + warp;
@@ -1270,8 +1271,8 @@ __global__ void __launch_bounds__(LV_NT) k_fill(const __grid_constant__ LiveMany
             const uint32_t ev0 = q.ev_rel[i0];
             for (uint32_t i = i0 + lane; i < i1; i += 32) {
                 const uint32_t at = q.ev_rel[i] - ev0;
-                instr_events(q, i, [&](uint32_t e, uint32_t v, bool test) {
-                    dst[(size_t)(at + e) * 32] = v | ((uint32_t)q.width[v] << 16) | (test ? 1u << 24 : 0u);
+                instr_events(q, i, [&](uint32_t e, uint32_t v, bool test, bool toggle) {
+                    dst[(size_t)(at + e) * 32] = v | ((uint32_t)q.width[v] << 16) | (test ? 1u << 24 : 0u) | (toggle ? 1u << 25 : 0u);
                 }, [](uint32_t) {});
             }
             n = q.short_ev[s];
@@ -1296,27 +1297,6 @@ cudaError_t pool_get(VlArena &arena, T **out, size_t n)
     return arena.alloc((void **)out, std::max<size_t>(n, 1) * sizeof(T) + 64);
 }
 
-// once per device: the kernels with a bitset or two per warp may use the whole shared memory of an SM
-int live_attributes(vl_program *p)
-{
-    static std::mutex mtx;
-    static bool done[64];
-    if (p->device < 0 || p->device >= 64) return VL_OK;
-    std::lock_guard<std::mutex> lock(mtx);
-    if (done[p->device]) return VL_OK;
-    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<1>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_flow<1>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_fill<1>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_sets<LV_MANY>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_flow<LV_MANY>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_fill<LV_MANY>, at, 227 * 1024));
-    VL_CUDA(p, cudaFuncSetAttribute(k_small<1, 1>, at, SMALL_SMEM));
-    VL_CUDA(p, cudaFuncSetAttribute(k_small<1, SMALL_BLOCKS>, at, SMALL_SMEM));
-    VL_CUDA(p, cudaFuncSetAttribute(k_small<LV_MANY, SMALL_BLOCKS>, at, SMALL_SMEM));
-    done[p->device] = true;
-    return VL_OK;
-}
 }  // namespace
 #define KEEP(out, n) VL_CUDA(p, pool_get(p->live_arena, out, n))
 #define LAYOUT(out, n) VL_CUDA(p, pool_get(p->layout_arena, out, n))
@@ -1619,6 +1599,7 @@ static int launch_small(vl_program *p, const LiveMany<N> &many, uint32_t n, size
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(C, n); cfg.blockDim = SMALL_NT; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cfg.attrs = at; cfg.numAttrs = C > 1 ? 2 : 1;
+    VL_CUDA(p, (allow_smem<k_small<N, C>, SMALL_SMEM>(p->device)));
     g_vl_launches.fetch_add(1);
     VL_CUDA(p, cudaLaunchKernelEx(&cfg, k_small<N, C>, many));
     return VL_OK;
@@ -1637,6 +1618,7 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
             sh.add(shapes[j]);
             many.p[j] = args[j];
         }
+        VL_CUDA(p, (allow_smem<k_fill<N>, 227 * 1024>(p->device)));
         VL_CUDA(p, launch_overlap(k_fill<N>, dim3(sh.fills, n), LV_NT, sh.fill_smem, st, true, many));
         return VL_OK;
     }
@@ -1662,7 +1644,9 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
             if (rc != VL_OK) return rc;
             continue;
         }
+        VL_CUDA(p, (allow_smem<k_sets<N>, 227 * 1024>(p->device)));
         VL_CUDA(p, launch_overlap(k_sets<N>, dim3(sh.sets, m), sh.set_warps * 32, sh.sets_smem, st, true, many));
+        VL_CUDA(p, (allow_smem<k_flow<N>, 227 * 1024>(p->device)));
         VL_CUDA(p, launch_overlap(k_flow<N>, dim3(sh.flows, m), FLOW_WARPS * 32, sh.flow_smem, st, true, many));
         if (sh.counts && sh.wide) VL_CUDA(p, launch_overlap(k_count<N, true>, dim3(sh.counts, m), PC_NT, sh.count_smem, st, true, many));
         else if (sh.counts) VL_CUDA(p, launch_overlap(k_count<N, false>, dim3(sh.counts, m), PC_NT, 0, st, true, many));
@@ -1681,8 +1665,7 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
     std::vector<LiveShape> shapes(n);
     std::vector<uint8_t> had_run(n);
     bool lengths_known = true;
-    int rc = n ? live_attributes(progs[0]) : VL_OK, err = VL_OK;
-    if (rc != VL_OK) return rc;
+    int rc = VL_OK, err = VL_OK;
     const uint32_t per = n == 1 ? 1 : LV_MANY;
     auto stream_of = [&](uint32_t j) { return (j / per) % n_streams; };
     for (uint32_t j = 0; j < n; ++j) {
