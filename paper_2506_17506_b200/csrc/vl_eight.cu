@@ -95,7 +95,8 @@ __device__ __noinline__ uint32_t apply_far(const uint32_t *ev, uint32_t entry, u
     return viol;
 }
 
-// NT consumer threads and a producer warp.  HAND: candidates with a collision are left to k_exact, which spreads their counts over
+// NT consumer threads and a producer warp; 256 threads leave room for two blocks per multiprocessor (three, with 72 registers and
+// a ring of three stages: 6,400 rows of 64 programs 355 us with liveness, 334 with two).  HAND: candidates with a collision are left to k_exact, which spreads their counts over
 // all multiprocessors.
 template <int NT, int N, bool HAND>
 __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __grid_constant__ EMany<N> a)
@@ -286,8 +287,8 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
     // ---- 2. one sweep over the vregs (see k_tables8)
     load_blocks(q, &M->f);
     for (uint32_t j = tid; q.use_th && j < q.nB * q.Wp * G; j += NT) s_th[j] = 0;
-    if (q.vcons) rules_sweep8<NT>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, M->flags, M->minR);
-    if (q.vcons) bar_all<NT, E_BAR>();  // (the sweep below changes table entries)
+    // (the sweep below changes table entries)
+    if (q.vcons) rules_sweep8<NT, E_BAR>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, Hb, M->flags, M->minR);
     {
         uint32_t mk = 0;
         const uint32_t bm = (q.B - 1) * 0x10001u;

@@ -73,28 +73,53 @@ __device__ __forceinline__ uint32_t pk8_get(const uint4 &x, int g)
     return (g & 1) ? (w >> 16) : (w & 0xFFFFu);
 }
 
-template <int NT>
+// Hardware rules on where the tuples may sit (alignment, registers of the vreg's class, reserved registers) for the eight
+// candidates of a block, by its NT consumer threads, which meet on barrier BAR.  bits: room for P + 63 bits, the reserved
+// registers.  All eight are checked without a branch and only a violation is looked at: with a branch per candidate and two loads
+// behind it (a prefix count of the reserved registers in global memory) the sweep took 18.4 k cycles of a block with 3,301
+// vregs, now 13.4 (777 rows of 11,317 instructions 89.5 us, 85.8).
+template <int NT, int BAR>
 __device__ __noinline__ void rules_sweep8(const uint4 *vcons, const uint16_t *rs_prefix, const uint32_t *vinfo,
                                           const uint32_t *first_def_instr, uint32_t V, uint32_t P, const uint4 *T,
-                                          uint32_t *flags, uint32_t *minR)
+                                          uint32_t *bits, uint32_t *flags, uint32_t *minR)
 {
-    for (uint32_t v = threadIdx.x; v < V; v += NT) {
-        const uint32_t vi = vinfo[v];
+    const uint32_t tid = threadIdx.x, n_words = (P + 63) / 32;
+    for (uint32_t r = tid; r < n_words * 32; r += NT) {
+        const uint32_t word = __ballot_sync(0xffffffffu, rs_prefix && r < P && rs_prefix[r + 1] != rs_prefix[r]);
+        if ((tid & 31) == 0) bits[r >> 5] = word;
+    }
+    asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
+    uint4 vc_next = tid < V ? vcons[tid] : make_uint4(0, 0, 0, 0);
+    uint32_t vi_next = tid < V ? vinfo[tid] : 0u;
+    for (uint32_t v = tid; v < V; v += NT) {
+        const uint4 vc = vc_next;
+        const uint32_t vi = vi_next;
+        if (v + NT < V) { vc_next = vcons[v + NT]; vi_next = vinfo[v + NT]; }
         if (!(vi & VINFO_DEFINED)) continue;
-        const uint4 vc = vcons[v];
         const uint32_t clo = vc.x & 0xFFFFu, chi = vc.x >> 16, al = vc.y, recip = vc.z, w = vi & 0xFFu;
         const uint4 tt = T[v];
+        uint32_t bad = 0;
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
-            const uint32_t tv = pk8_get(tt, g);
-            bool bad = (al > 1 && tv != __umulhi(tv, recip) * al) || tv < clo || tv + w > chi;
-            if (!bad && rs_prefix) bad = rs_prefix[min(tv + w, P)] != rs_prefix[min(tv, P)];
-            if (bad) {
-                atomicOr(&flags[g], (uint32_t)VL_OUT_OF_RANGE);
-                atomicMin(&minR[g], first_def_instr[v]);
-            }
+            const uint32_t tv = pk8_get(tt, g), at = min(tv, P), end = min(tv + w, P);
+            // reserved registers in [at, end): up to 32 of the range lie in two words, what is wider is walked below
+            const uint32_t hold = __funnelshift_r(bits[at >> 5], bits[(at >> 5) + 1], at);
+            const uint32_t mask = end - at < 32 ? (1u << (end - at)) - 1u : 0xFFFFFFFFu;
+            const bool b = (al > 1 && tv != __umulhi(tv, recip) * al) || tv < clo || tv + w > chi || (hold & mask);
+            bad |= (b ? 1u : 0u) << g;
+        }
+        if (w > 32) {
+#pragma unroll
+            for (int g = 0; g < 8; ++g)
+                for (uint32_t r = min(pk8_get(tt, g), P) + 32; r < min(pk8_get(tt, g) + w, P); ++r) bad |= ((bits[r >> 5] >> (r & 31)) & 1u) << g;
+        }
+        for (; bad; bad &= bad - 1) {
+            const uint32_t g = __ffs(bad) - 1;
+            atomicOr(&flags[g], (uint32_t)VL_OUT_OF_RANGE);
+            atomicMin(&minR[g], first_def_instr[v]);
         }
     }
+    asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");  // (bits may be overwritten)
 }
 
 }  // namespace

@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
     // matter.)  Bound by instruction issue; as two sweeps, with a shift per candidate for the nibbles, it took 16.5 k
     // cycles per block on 10,000 vregs, now 10.
     // (From here on the producer warp only keeps the block's barriers company.)
-    if (q.vcons && tid < NT) rules_sweep8<NT>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, M->flags, M->minR);
+    if (q.vcons && tid < NT) rules_sweep8<NT, 2>(q.vcons, q.rs_prefix, q.vinfo, q.first_def_instr, q.V, q.P, T, Hb, M->flags, M->minR);
     if (tid < NT) {
         uint32_t mk = 0, mk2 = 0, mk3 = 0, mk4 = 0;
         const uint32_t bm = q.Bmask * 0x10001u;
