@@ -164,7 +164,8 @@ int vl_liveness_result(const vl_program *prog, const uint32_t **blk_live_in, con
  * A call with more than one pass (VL_OPT_SUB_BATCH; the passes of a call are made equally long)
  * spreads its passes over internal streams of the device (VL_OPT_LANES) that fork from and join
  * back into `cuda_stream`, so that kernels of different passes run side by side; with
- * VL_OPT_LANES = 1 every kernel is enqueued on `cuda_stream` itself.
+ * VL_OPT_LANES = 1 every kernel is enqueued on `cuda_stream` itself.  Jobs of up to a few thousand rows, depending on the
+ * program, are checked by one or two kernels on `cuda_stream`, whatever these two options say.
  * Host work of a call: the handle is modified (it owns the working memory of its calls).  The first
  * call on a handle, and a later one that needs larger working sets (more rows per pass, another
  * chunk size, more internal streams in use, few rows after many or many after few: those are different kernels), allocates them with cudaMalloc and clears them, which
@@ -388,7 +389,7 @@ uint64_t vl_kernel_launches(void);
 /*
  * Device time of the verify kernels since the last call (or since VL_OPT_KERNEL_TIMING was set), summed over
  * the passes recorded (at most 4096): ms[0] table kernel (first occurrences, Consistency, Realizability, bank
- * tally), ms[1] occupancy walk (Safety), ms[2] verdict kernel, ms[3] exact counts.  A short job is one pass: its one kernel
+ * tally), ms[1] occupancy walk (Safety), ms[2] verdict kernel, ms[3] exact counts.  A job that one kernel checks is one pass: that kernel
  * is in ms[0], the exact counts it may hand over in ms[3]; short jobs of several programs that share a launch of
  * vl_verify_batch have the time of the whole launch each.  ms is HOST memory for 4 floats; *passes (HOST, may be NULL)
  * receives the number of passes summed.  Kernels of different passes
