@@ -58,9 +58,10 @@ enum {
                                 many microseconds apart (0..200, default 12), so that not all of them stream, then all of them
                                 sweep, in step; only for calls of at least two waves */
     VL_OPT_TEST_WAIT = 7     /* test hook for the bounded device waits: 1 = the table kernel (8 candidates per
-                                block) waits for its first tile on a barrier that nothing completes, with a short
-                                poll limit, so that the wait runs out: the call still returns, its verdicts are
-                                garbage and vl_verify_status reports VL_ERR_DEVICE_WAIT.  0 = normal (default) */
+                                block), or the one kernel that checks a job of up to a few thousand rows, waits for its
+                                first tile on a barrier that nothing completes, with a short poll limit, so that the wait
+                                runs out: the call still returns, its verdicts are garbage and vl_verify_status reports
+                                VL_ERR_DEVICE_WAIT.  0 = normal (default) */
 };
 
 /*

@@ -31,6 +31,7 @@ struct ESmem {
 struct EMisc {
     unsigned long long bar[E_STAGES], empty[E_STAGES];  // a stage is full; every consumer warp has read it
     unsigned long long stored[2];                       // every consumer warp has stored its first occurrences of a tile (by tile parity)
+    unsigned long long never;                           // test hook: nothing completes it
     uint32_t flags[8], minop[8], minR[8], bank[8], nout[8], thcol[8];
     uint32_t pairs[8], mind[8];
     uint32_t any, marks, abort_flag, next;
@@ -41,6 +42,7 @@ struct EParams {
     FParams f;
     ESmem sm;
     uint32_t nOp8, ntiles, nC, CW, bank_total, pf;
+    uint32_t test_wait;  // test hook: the consumers wait on a barrier that nothing completes, with a short limit
     const uint4 *opoff;
     const uint8_t *first4;
     const uint32_t *ev8, *cev_off, *chunk_blk, *short_chunk;
@@ -126,6 +128,7 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
         for (uint32_t s = 0; s < E_STAGES; ++s) { mbar_init(&M->bar[s], 1); mbar_init(&M->empty[s], WARPS); }
         mbar_init(&M->stored[0], WARPS);
         mbar_init(&M->stored[1], WARPS);
+        mbar_init(&M->never, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         T[q.V] = make_uint4(0, 0, 0, 0);  // the spare entry: what padding columns are compared with
     }
@@ -135,9 +138,8 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
     pdl_wait();  // (the rows, and what liveness computed)
 
     auto wait_bar = [&](unsigned long long *bar, uint32_t parity) {
-        // Bounded.  When it runs out the block raises the status bit and carries on with short waits (its results are
-        // garbage, every index still in bounds); the producer issues no further copies and, before the block returns,
-        // waits again for the copies it did issue.
+        // Bounded.  When it runs out the block raises the status bit and carries on with short waits to the end of the
+        // streaming phase, where it leaves; the producer issues no further copies.
         if (mbar_try_wait(bar, parity)) return;
         uint32_t spins = 0;
         const uint32_t limit = *(volatile uint32_t *)&M->abort_flag ? 64u : (1u << 20);
@@ -166,7 +168,9 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
             if (++stage == e.sm.NS) { stage = 0; parity ^= 1; }
         }
         __syncwarp();
-        if (lane == 0 && *(volatile uint32_t *)&M->abort_flag)  // give the copies that were issued their time
+        // No thread block goes away while a copy into its shared memory is on its way: not even if a consumer's wait runs out
+        // after the last copy has been issued.
+        if (lane == 0)
             for (uint32_t s = 0; s < e.sm.NS && s < issued; ++s) {
                 const uint32_t t_last = s + (issued - 1 - s) / e.sm.NS * e.sm.NS;  // the last tile issued into stage s
                 uint32_t spins = 0;
@@ -267,6 +271,12 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
         for (int j = 0; j < 4; ++j) pcB[j] = make_uint4(0, 0, 0, 0);
         offB = make_uint4(spare_off, spare_off, spare_off, spare_off);  // "the tile before tile 0": zeros against the spare entry
         const std::integral_constant<bool, false> more{};
+        if (e.test_wait) {  // test hook: this wait runs out
+            uint32_t spins = 0;
+            while (!mbar_try_wait(&M->never, 0)) {
+                if (++spins > (1u << 16)) { M->abort_flag = 1; atomicOr(e.status, ST_DEVICE_WAIT); break; }
+            }
+        }
         uint32_t t = 0;
         for (; t + 2 <= last; t += 2) {
             step(t, pcA, offA, pcB, offB, more);
@@ -283,6 +293,16 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
         compare(pcA, offA, last * TILE + tid * 4);
     }
     bar_all<NT, E_BAR>();
+    // A wait ran out: copies that are still on their way may land in what takes the ring's place from here on (lists of
+    // instructions among it), and the table may hold anything.  The rows get a record that is no verdict.  (If a wait of the
+    // producer runs out, so does one of every consumer, for the tile that is never issued: all threads see the same flag.)
+    if (M->abort_flag) {
+        if (tid < G && k0 + tid < q.K) {
+            if (HAND) q.ex.cstate[(k0 + tid) * 8 + CS_ITEMS] = 0;
+            q.out[k0 + tid] = vl_verdict{0u, -1, 0u, 0u};
+        }
+        return;
+    }
 
     // ---- 2. one sweep over the vregs (see k_tables8)
     load_blocks(q, &M->f);
@@ -691,7 +711,7 @@ bool vl_eight_takes(const vl_program *p) { return p->V < 16384 && p->wmax <= 8 &
 #define EIGHT_INSTR_ROWS 24000000ull
 bool vl_eight_wanted(vl_program *p, uint64_t K)
 {
-    if (p->group_opt || p->threads_opt || p->test_wait) return false;  // the caller asks for the batched kernels
+    if (p->group_opt || p->threads_opt) return false;  // the caller asks for the batched kernels
     if (!p->d_ev8 || !p->bank_fast || p->nS > 65535u || !vl_verify_takes(p)) return false;
     if (p->known[VL_KNOWN_SEN] >= FUSED_MANY_ENTRIES || p->known[VL_KNOWN_LS] >= (uint64_t)EXACT_LONG * p->nI) return false;
     if (K > 8ull * vl_sm_count(p) && K * p->nI > EIGHT_INSTR_ROWS) return false;
@@ -729,7 +749,7 @@ int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
         e.bank_total = 2 * (p->bank_seg[1] - p->bank_seg[0]) + 3 * (p->bank_seg[2] - p->bank_seg[1]) + 4 * (p->bank_seg[3] - p->bank_seg[2]);
         e.opoff = dict ? p->d_dict_opoff : p->d_opoff; e.first4 = dict ? p->d_dict_first4 : p->d_first4;
         e.ev8 = p->d_ev8; e.cev_off = p->d_cev_off; e.chunk_blk = p->d_chunk_blk; e.short_chunk = p->d_short_chunk;
-        e.status = p->d_status + 1;
+        e.status = p->d_status + 1; e.test_wait = p->test_wait;
         smem = std::max(smem, pl.sm.total);
         rows = std::max(rows, K[j]);
         const int rc = vl_live_join(p, from, st);

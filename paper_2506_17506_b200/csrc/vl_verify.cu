@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
     auto wait_bar = [&](unsigned long long *bar, uint32_t parity) {
         // Bounded wait.  When it runs out the block raises the status bit and carries on with short
         // waits (its results are garbage, every index still in bounds); the producer issues no
-        // further copies and, before the block returns, waits again for the copies it did issue.
+        // further copies.
         if (mbar_try_wait(bar, parity)) return;
         uint32_t spins = 0;
         const uint32_t limit = *(volatile uint32_t *)&M->abort_flag ? 64u : (1u << 20);
@@ -615,9 +615,8 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
                 }
                 if (++stage == q.NS) { stage = 0; parity ^= 1; }
             }
-            if (*(volatile uint32_t *)&M->abort_flag) {
-                // a wait ran out: give the copies that were issued their time before the block (and its
-                // shared memory) goes away
+            {   // no block goes away while a copy into its shared memory is on its way: not even if a consumer's wait runs out
+                // after the last copy has been issued
                 for (uint32_t s = 0; s < q.NS; ++s) {
                     if (issued <= s) continue;
                     uint32_t t_last = s + (issued - 1 - s) / q.NS * q.NS;  // the last tile issued into stage s

@@ -90,3 +90,30 @@ def test_several_programs(B, oracle_mod):
             _assert_same(B.verdicts_to_numpy(o), w)
     for gp in gps:
         gp.close()
+
+
+# counts handed over (512 and 256 threads), made by the block itself
+@pytest.mark.parametrize("K", [40, 1500, 2500])
+def test_bounded_wait_runs_out(B, oracle_mod, K):
+    """The wait of the consumers for their first tile runs out (test hook): the call returns, no verdict passes, the status says so,
+    and the next call is exact again."""
+    import torch
+    p = _member(2000, K)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    rows = _rows(p, K, K)
+    want = op.verify(op.liveness(), rows)
+    _assert_same(_gpu_verify(B, gp, rows), want, "before")
+    gp.set_option(B.VL_OPT_TEST_WAIT, 1)
+    out = gp.vl_verify(_to_dev(rows))
+    torch.cuda.synchronize()
+    with pytest.raises(B.VlError) as e:
+        gp.vl_verify_status()
+    assert e.value.code == B.VL_ERR_DEVICE_WAIT
+    got = B.verdicts_to_numpy(out)
+    assert np.all(got["flags"] == 0) and np.all(got["first_violation_instr"] == -1), "a row of a block that gave up has a verdict"
+    gp.set_option(B.VL_OPT_TEST_WAIT, 0)
+    for _ in range(2):
+        _assert_same(_gpu_verify(B, gp, rows), want, "after the wait ran out")
+    gp.close()
