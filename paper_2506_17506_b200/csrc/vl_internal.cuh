@@ -52,6 +52,7 @@ struct VlArena {
     struct Slab { char *ptr; size_t size; };
     std::vector<Slab> slabs;
     size_t cur = 0, off = 0;
+    size_t kept_cur = 0, kept_off = 0;  // what lies in front of this place outlives reset()
     size_t hint = 0;  // what the next slab should hold (a slab costs 20 us up to 64 KB, 330 us from 1 MB on, however large)
     cudaError_t alloc(void **out, size_t bytes)
     {
@@ -72,12 +73,14 @@ struct VlArena {
         off = bytes;
         return cudaSuccess;
     }
-    void reset() { cur = 0; off = 0; }
+    void keep() { kept_cur = cur; kept_off = off; }
+    void reset() { cur = kept_cur; off = kept_off; }
+    void clear() { kept_cur = kept_off = 0; reset(); }
     void release()
     {
         for (auto &s : slabs) cudaFree(s.ptr);
         slabs.clear();
-        reset();
+        clear();
     }
 };
 
@@ -103,6 +106,7 @@ struct vl_program {
     uint32_t short_len = 1;  // instructions of the longest short chunk
     uint32_t share_pieces = 0, share_ops = 0;  // pieces and operands of the largest share of a thread block of k_small
     bool wide_pieces = false;  // some piece is an instruction of many operands (PIECE_OPERANDS, vl_liveness.cu)
+    bool words_new = false;  // the kernel that makes the operand words has been launched since the last run
     uint32_t layout_chunk_instrs = 0;  // chunk size the device copies of the layout were made for (0: none)
     std::vector<uint32_t> h_blk_off, h_op_off, h_succ_off, h_succ;
     // list lengths of the last liveness run with this layout: the next run allocates from them

@@ -1309,6 +1309,13 @@ cudaError_t pool_get(VlArena &arena, T **out, size_t n)
         }                                                       \
     } while (0)
 
+// About the memory of a run that does not depend on the list lengths (live_begin).
+static size_t live_bytes(const vl_program *p)
+{
+    return 4 * ((size_t)3 * p->nP + 4 * (size_t)p->nC + 5 * (size_t)p->nB) * p->Wv + (size_t)p->nI * 28 + (size_t)p->nO * 18 +
+           (size_t)p->nC * 40 + (size_t)p->nS * 16 + (size_t)p->nB * 24 + 40 * 512;
+}
+
 // Chunks, pieces, short chunks and segments depend on the program and on the chunk size only: they are laid
 // out (and uploaded, in one copy) when the chunk size changes, not on every call.
 static int vl_layout(vl_program *p, cudaStream_t st)
@@ -1413,7 +1420,6 @@ static int vl_layout(vl_program *p, cudaStream_t st)
     }
     uint32_t *dev = nullptr;
     p->layout_arena.hint = all.size() * 4 + (size_t)p->V * 12 + (size_t)p->nOp8 * 3 + (size_t)p->nOpT * 5 + 16384;
-    if (p->nO <= 65536) p->layout_arena.hint += (size_t)p->nO * 4;  // (else the operand words have a slab of their own)
     LAYOUT(&dev, all.size());
     VL_CUDA(p, cudaMemcpy(dev, all.data(), all.size() * 4, cudaMemcpyHostToDevice));
     size_t at = 0;
@@ -1422,10 +1428,16 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         at = (at + x.v->size() + 4) & ~(size_t)3;
     }
     p->d_share = reinterpret_cast<uint4 *>(d_share);
-    LAYOUT(&p->d_op_word, (size_t)p->nO);
+    // (in the slab of the runs' memory: beside the layout's tables they would take a program of 32,000 instructions one
+    // device allocation more, 300 us of the first run's 1,200)
+    vl_free_liveness(p);
+    p->live_arena.clear();
+    p->live_arena.hint = live_bytes(p) + (size_t)p->nO * 4 + 512;
+    KEEP(&p->d_op_word, (size_t)p->nO);
+    p->live_arena.keep();
     LAUNCH(k_operand_words, (p->nP + NT / 32 - 1) / (NT / 32), NT, 0, st, p->nP, p->d_piece_i0, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_op_word);
     VL_CUDA(p, cudaGetLastError());
-    VL_CUDA(p, cudaStreamSynchronize(st));  // (the first kernels of a run read the layout before they wait for the stream)
+    p->words_new = true;
     const uint32_t Wp = (p->P + p->wmax + 31) / 32 + 1;
     p->use_th = (nB <= 32 && (uint64_t)nB * VL_MAX_GROUP * Wp * 4 <= 24 * 1024) ? 1 : 0;
     p->layout_chunk_instrs = p->chunk_instrs;
@@ -1457,9 +1469,7 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     vl_free_liveness(p);
     const uint32_t nB = p->nB, nI = p->nI, V = p->V, nO = p->nO, Wv = p->Wv, nC = p->nC, nP = p->nP;
 
-    // about what follows, in one slab
-    p->live_arena.hint = 4 * ((size_t)3 * nP + 4 * (size_t)nC + 5 * (size_t)nB) * Wv + (size_t)nI * 28 + (size_t)nO * 18 +
-                         (size_t)nC * 40 + (size_t)p->nS * 16 + (size_t)nB * 24 + 40 * 512;
+    p->live_arena.hint = live_bytes(p);  // what follows, in one slab
     // ---- results and tables that do not depend on the list lengths
     KEEP(&p->d_blk_in, (size_t)2 * nB * Wv);  // live-in rows, then live-out rows
     p->d_blk_out = p->d_blk_in + (size_t)nB * Wv;
@@ -1589,11 +1599,11 @@ static int live_tables(vl_program *p, cudaStream_t st)
 
 // k_small for the runs of n <= N programs, C thread blocks each.
 template <int N, int C>
-static int launch_small(vl_program *p, const LiveMany<N> &many, uint32_t n, size_t smem, cudaStream_t st)
+static int launch_small(vl_program *p, const LiveMany<N> &many, uint32_t n, size_t smem, cudaStream_t st, bool overlap)
 {
     cudaLaunchAttribute at[2] = {};
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = C; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
@@ -1625,8 +1635,13 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
     for (const bool small : {true, false}) {
         LiveShape sh;
         uint32_t m = 0;
+        // The first kernel of a run reads the operand words before it waits for the stream: behind the kernel that makes them it
+        // starts when that one has ended.  (A wait of the host in between: 82.3 us for the first run of 64 instructions, 79.4
+        // without operand words.)
+        bool overlap = true;
         for (uint32_t j = 0; j < n; ++j) {
             if (shapes[j].small != small) continue;
+            overlap = overlap && !progs[j]->words_new;
             sh.add(shapes[j]);
             many.p[m++] = args[j];
         }
@@ -1637,15 +1652,15 @@ static int live_launch(vl_program *const *progs, uint32_t n, const LiveArgs *arg
             int rc;
             if (N == 1 && p->nP <= SMALL_ONE_PIECES && one_smem <= SMALL_SMEM) {
                 many.p[0].small = one;
-                rc = launch_small<N, N == 1 ? 1 : SMALL_BLOCKS>(p, many, m, one_smem, st);
+                rc = launch_small<N, N == 1 ? 1 : SMALL_BLOCKS>(p, many, m, one_smem, st, overlap);
             } else {
-                rc = launch_small<N, SMALL_BLOCKS>(p, many, m, sh.small_smem, st);
+                rc = launch_small<N, SMALL_BLOCKS>(p, many, m, sh.small_smem, st, overlap);
             }
             if (rc != VL_OK) return rc;
             continue;
         }
         VL_CUDA(p, (allow_smem<k_sets<N>, 227 * 1024>(p->device)));
-        VL_CUDA(p, launch_overlap(k_sets<N>, dim3(sh.sets, m), sh.set_warps * 32, sh.sets_smem, st, true, many));
+        VL_CUDA(p, launch_overlap(k_sets<N>, dim3(sh.sets, m), sh.set_warps * 32, sh.sets_smem, st, overlap, many));
         VL_CUDA(p, (allow_smem<k_flow<N>, 227 * 1024>(p->device)));
         VL_CUDA(p, launch_overlap(k_flow<N>, dim3(sh.flows, m), FLOW_WARPS * 32, sh.flow_smem, st, true, many));
         if (sh.counts && sh.wide) VL_CUDA(p, launch_overlap(k_count<N, true>, dim3(sh.counts, m), PC_NT, sh.count_smem, st, true, many));
@@ -1689,6 +1704,7 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
         return VL_OK;
     };
     if ((rc = launch(false)) != VL_OK) return rc;
+    for (uint32_t j = 0; j < n; ++j) progs[j]->words_new = false;
     if (!lengths_known)
         for (uint32_t s = 0; s < n_streams; ++s) VL_CUDA(progs[0], cudaStreamSynchronize(streams[s]));
     std::vector<vl_program *> run;  // the programs that the last kernel is launched for
