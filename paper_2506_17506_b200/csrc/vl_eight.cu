@@ -67,6 +67,13 @@ __device__ __forceinline__ uint32_t atom_xor(uint32_t addr, uint32_t v)
     asm volatile("atom.shared.xor.b32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
     return old;
 }
+// The same where v is not 0; else 0.
+__device__ __forceinline__ uint32_t atom_xor_some(uint32_t addr, uint32_t v, uint32_t some)
+{
+    uint32_t old = 0;
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %3, 0;\n @p atom.shared.xor.b32 %0, [%1], %2;\n}\n" : "+r"(old) : "r"(addr), "r"(v), "r"(some) : "memory");
+    return old;
+}
 __device__ __forceinline__ uint32_t lds_u16(uint32_t addr)
 {
     uint16_t v;
@@ -74,25 +81,36 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t addr)
     return v;
 }
 
-// Eight events at ev for one candidate (see the walk in k_eight), ranges of any position, word by word: the occupied bits that
-// tests found.
+// Eight events at ev for one candidate (see the walk in k_eight), some of whose ranges reach into the next word: an atomic more,
+// in the order of the events.  The occupied bits that tests found.  A function of its own: in the walk's loop it slowed the other
+// events down.  (Rows of which no tuple is aligned, with a load, a change and a store for each word one after the other / with
+// atomics, us: 2,000 instructions, 1,600 rows 42.1 / 35.6; 8,000, 1,184 rows 72.1 / 62.2; 24,000, 600 rows 143 / 124.)
 template <int NT>
-__device__ __noinline__ uint32_t apply_far(const uint32_t *ev, uint32_t entry, uint32_t *occ)
+__device__ __noinline__ uint32_t apply_far(const uint32_t *ev, uint32_t entry, uint32_t occ_addr)
 {
     uint32_t viol = 0;
-    for (uint32_t u = 0; u < 8; ++u) {
-        const uint32_t w = ev[u], pos = lds_u16(entry + (w & EV8_OFFSET)) & 0x7FFFu;
-        const unsigned long long m = (unsigned long long)(w >> EV8_MASK_SHIFT) << (pos & 31);
-        uint32_t *a = occ + (pos >> 5) * NT;
-        const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32), o0 = a[0], tog = w & EV8_HOLD ? 0u : 0xFFFFFFFFu;
-        a[0] = o0 ^ (lo & tog);
-        uint32_t hit = o0 & lo;
-        if (hi) {
-            const uint32_t o1 = a[NT];
-            a[NT] = o1 ^ (hi & tog);
-            hit |= o1 & hi;
+    uint32_t w[8], t[8];
+    {
+        const uint4 a = reinterpret_cast<const uint4 *>(ev)[0], b = reinterpret_cast<const uint4 *>(ev)[1];
+        w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = lds_u16(entry + (w[u] & EV8_OFFSET));
+#pragma unroll
+    for (int h = 0; h < 8; h += 4) {
+        uint32_t lo[4], hi[4], old_hi[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t x = w[h + u], mask = x >> EV8_MASK_SHIFT, keep = x & EV8_HOLD ? 0u : 0xFFFFFFFFu;
+            const uint32_t at = occ_addr + (t[h + u] & 0x7FE0u) * (NT / 8);
+            lo[u] = __funnelshift_l(0u, mask, t[h + u]);
+            hi[u] = __funnelshift_l(mask, 0u, t[h + u]);
+            t[h + u] = atom_xor(at, lo[u] & keep);
+            old_hi[u] = atom_xor_some(at + NT * 4, hi[u] & keep, hi[u]);
         }
-        if (w & EV8_TEST) viol |= hit;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (w[h + u] & EV8_TEST) viol |= (t[h + u] & lo[u]) | (old_hi[u] & hi[u]);
     }
     return viol;
 }
@@ -512,27 +530,31 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
             // Eight events at a time; the next eight are on their way, and the line after those of the next (a line holds 32 events
             // of a chunk) is asked for.  Toggling returns the old word: occupied and released are both a toggle as long as no
             // collision has been seen (after one, the chunk is counted exactly anyway).
+            auto events = [&](auto marked) {
 #pragma unroll 1
-            for (uint32_t i = 0; i < n_max; i += 8) {
-                const uint32_t w[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-                if (e0 + i + 64 < e1) asm volatile("prefetch.global.L1 [%0];" ::"l"(e.ev8 + e0 + i + 64));
-                fetch(e0 + i + 8);
-                uint32_t t[8], m[8];
+                for (uint32_t i = 0; i < n_max; i += 8) {
+                    const uint32_t w[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+                    if (e0 + i + 64 < e1) asm volatile("prefetch.global.L1 [%0];" ::"l"(e.ev8 + e0 + i + 64));
+                    fetch(e0 + i + 8);
+                    uint32_t t[8], m[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) t[u] = *reinterpret_cast<const uint16_t *>(smem + ((w[u] & EV8_OFFSET) | g2));
-                if (check && __any_sync(0xffffffffu, (t[0] | t[1] | t[2] | t[3] | t[4] | t[5] | t[6] | t[7]) & 0x8000u)) {
-                    viol |= apply_far<NT>(e.ev8 + (e0 + i < e1 ? e0 + i : none), smem_base + g2, occ);
-                    continue;
+                    for (int u = 0; u < 8; ++u) t[u] = *reinterpret_cast<const uint16_t *>(smem + ((w[u] & EV8_OFFSET) | g2));
+                    if (decltype(marked)::value && __any_sync(0xffffffffu, (t[0] | t[1] | t[2] | t[3] | t[4] | t[5] | t[6] | t[7]) & 0x8000u)) {
+                        viol |= apply_far<NT>(e.ev8 + (e0 + i < e1 ? e0 + i : none), smem_base + g2, occ_addr);
+                        continue;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        m[u] = __funnelshift_l(0u, w[u] >> EV8_MASK_SHIFT, t[u]);
+                        t[u] = atom_xor(occ_addr + (t[u] & 0x7FE0u) * (NT / 8), w[u] & EV8_HOLD ? 0u : m[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (w[u] & EV8_TEST) viol |= t[u] & m[u];
                 }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    m[u] = __funnelshift_l(0u, w[u] >> EV8_MASK_SHIFT, t[u]);
-                    t[u] = atom_xor(occ_addr + (t[u] & 0x7FE0u) * (NT / 8), w[u] & EV8_HOLD ? 0u : m[u]);
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (w[u] & EV8_TEST) viol |= t[u] & m[u];
-            }
+            };
+            if (check) events(std::integral_constant<bool, true>{});
+            else events(std::integral_constant<bool, false>{});
             if (viol) {
                 atomicOr(&s_coll[g_own * e.CW + (c >> 5)], 1u << (c & 31));
                 atomicOr(&M->any, 1u << g_own);
@@ -610,18 +632,21 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
         }
         if (HAND && (((M->any >> g) & 1u) | M->thcol[g])) {
             const uint64_t k = k0 + g;
-            uint32_t chunks = lane == 0 && M->thcol[g] ? e.nC / 8 : 0u;  // (the sources in the through-set)
+            uint32_t chunks = 0;
             for (uint32_t w = lane; w < e.CW; w += 32) {
                 const uint32_t bits = s_coll[g * e.CW + w];
                 q.ex.anom[k * e.CW + w] = bits;
                 chunks += __popc(bits);
             }
             chunks = __reduce_add_sync(0xffffffffu, chunks);
+            const bool full = chunks == e.nC;  // (with every chunk counted in full, nothing is left of the through-sets)
+            const uint32_t thcol = full ? 0u : M->thcol[g];
+            if (thcol) chunks += e.nC / 8;  // (the sources in the through-set)
             if (lane < 4) q.ex.racc[k * 4 + lane] = 0;
             if (lane == 0) {
                 uint32_t *cs = q.ex.cstate + k * 8;
                 cs[CS_FLAGS] = M->flags[g]; cs[CS_FIRST] = first; cs[CS_BANK] = e.bank_total - M->bank[g];
-                cs[CS_WALK] = (M->any >> g) & 1u ? WALK_ANOM : 0u; cs[CS_THCOL] = M->thcol[g];
+                cs[CS_WALK] = ((M->any >> g) & 1u ? WALK_ANOM : 0u) | (full ? WALK_FULL : 0u); cs[CS_THCOL] = thcol;
                 cs[CS_ITEMS] = exact_parts(chunks, EXACT_PART_CHUNKS) | exact_parts(chunks, EXACT_FINE_CHUNKS) << 16;
             }
             return;

@@ -117,3 +117,44 @@ def test_bounded_wait_runs_out(B, oracle_mod, K):
     for _ in range(2):
         _assert_same(_gpu_verify(B, gp, rows), want, "after the wait ran out")
     gp.close()
+
+
+# counts handed over (few rows; many rows of a long program, up to the most), made by the block itself; candidates in fine items, in
+# coarse ones, one item each
+@pytest.mark.parametrize("n_instrs,K,launches", [(2399, 2000, 2), (2399, 2001, 1), (2400, 2001, 1), (2400, 8192, 1), (2400, 8193, 1), (4100, 700, 2)])
+@pytest.mark.parametrize("noise", [0.004, 0.2, 1.0])
+def test_rows_that_collide_everywhere(B, oracle_mod, n_instrs, K, launches, noise):
+    """Rows of random registers (every chunk collides, vregs outside the file, tuples across mask words) among valid ones."""
+    p = _member(n_instrs, 7)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    some = _rows(p, 100, 3)
+    some[50:] = _garbage_rows(p, 50, 4)
+    verdicts = op.verify(op.liveness(), some)
+    rng = np.random.default_rng(K)
+    pick = np.where(rng.random(K) < noise, rng.integers(50, 100, K), rng.integers(0, 50, K))
+    dev = _to_dev(some[pick])
+    out = gp.vl_verify(dev)
+    before = B.vl_kernel_launches()
+    gp.vl_verify(dev, out)
+    assert B.vl_kernel_launches() - before == launches, "another path has checked the rows"
+    _assert_same(B.verdicts_to_numpy(out), verdicts[pick], f"{K} rows")
+    gp.close()
+
+
+@pytest.mark.parametrize("K", [600, 1500])
+def test_tuples_across_mask_words(B, oracle_mod, K):
+    """Valid rows whose tuples sit anywhere: ranges that reach into the next word of the occupancy masks, in every block."""
+    import copy
+    p = copy.copy(_member(3000, 5))
+    rows, _ = synth.candidate_rows(p, K, 0.2, 9)
+    rows += 3
+    p.P += 8
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    want = op.verify(op.liveness(), rows)
+    assert (want["flags"] == B.VL_PASS).mean() > 0.7
+    _assert_same(_gpu_verify(B, gp, rows), want)
+    gp.close()
