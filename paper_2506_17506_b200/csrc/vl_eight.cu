@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
     // producer runs out, so does one of every consumer, for the tile that is never issued: all threads see the same flag.)
     if (M->abort_flag) {
         if (tid < G && k0 + tid < q.K) {
-            if (HAND) q.ex.cstate[(k0 + tid) * 8 + CS_ITEMS] = 0;
+            if (HAND) q.ex.items[k0 + tid] = 0;
             q.out[k0 + tid] = vl_verdict{0u, -1, 0u, 0u};
         }
         return;
@@ -647,12 +647,12 @@ __global__ void __launch_bounds__(NT + 32, NT == 256 ? 2 : 1) k_eight(const __gr
                 uint32_t *cs = q.ex.cstate + k * 8;
                 cs[CS_FLAGS] = M->flags[g]; cs[CS_FIRST] = first; cs[CS_BANK] = e.bank_total - M->bank[g];
                 cs[CS_WALK] = ((M->any >> g) & 1u ? WALK_ANOM : 0u) | (full ? WALK_FULL : 0u); cs[CS_THCOL] = thcol;
-                cs[CS_ITEMS] = exact_parts(chunks, EXACT_PART_CHUNKS) | exact_parts(chunks, EXACT_FINE_CHUNKS) << 16;
+                q.ex.items[k] = exact_parts(chunks, EXACT_PART_CHUNKS) | exact_parts(chunks, EXACT_FINE_CHUNKS) << 16;
             }
             return;
         }
         if (lane == 0) {
-            if (HAND) q.ex.cstate[(k0 + g) * 8 + CS_ITEMS] = 0;
+            if (HAND) q.ex.items[k0 + g] = 0;
             const uint32_t flags = M->flags[g] | (M->pairs[g] ? (uint32_t)VL_INTERFERENCE : 0u);
             vl_verdict vd;
             vd.flags = flags ? flags : (uint32_t)VL_PASS;
@@ -746,6 +746,9 @@ bool vl_eight_wanted(vl_program *p, uint64_t K)
 // Whether a job may share a launch with jobs of other programs: blocks of 256 threads, two per multiprocessor.
 bool vl_eight_shares(vl_program *p, uint64_t K) { return vl_eight_wanted(p, K) && eight_smem(p, 256, E_HALF).total; }
 
+#define EIGHT_HAND_ROWS 2000u
+#define EIGHT_HAND_INSTRS 2400u
+
 int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
                  vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot)
 {
@@ -794,7 +797,7 @@ int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
     } else {
         EMany<1> one;
         one.p[0] = many.p[0];
-        if (slot >= 0 && vl_exact_takes_rows(p0, rows)) {
+        if (slot >= 0 && vl_exact_takes_rows(p0, rows) && (rows <= EIGHT_HAND_ROWS || p0->nI >= EIGHT_HAND_INSTRS)) {
             VlExactArgs &ex = one.p[0].f.ex;
             const int rc = vl_hand_scratch(p0, slot, rows, &ex);
             if (rc != VL_OK) return rc;

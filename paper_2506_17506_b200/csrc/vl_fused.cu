@@ -18,8 +18,9 @@
 #include "vl_exact.cuh"
 
 #define EXACT_NT 256
+#define EXACT_ROUNDS 2
 #define EXACT_SMEM (224u * 1024)  // shared memory of a block of k_exact, at most
-#define EXACT_ROWS 2000           // rows that k_fused leaves counts of, at most: their items fit 16 bits
+#define EXACT_ROWS 8192           // rows that k_fused and k_eight leave counts of, at most: each block adds up their items
 
 namespace {
 
@@ -349,10 +350,10 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
                 uint32_t *cs = q.ex.cstate + k * 8;
                 cs[CS_FLAGS] = M->flags; cs[CS_FIRST] = first; cs[CS_BANK] = M->bank;
                 cs[CS_WALK] = M->any ? WALK_ANOM : 0u; cs[CS_THCOL] = M->thcol;
-                cs[CS_ITEMS] = exact_parts(chunks, EXACT_PART_CHUNKS) | exact_parts(chunks, EXACT_FINE_CHUNKS) << 16;
+                q.ex.items[k] = exact_parts(chunks, EXACT_PART_CHUNKS) | exact_parts(chunks, EXACT_FINE_CHUNKS) << 16;
             }
         } else if (lane == 0) {
-            if (HAND) q.ex.cstate[k * 8 + CS_ITEMS] = 0;
+            if (HAND) q.ex.items[k] = 0;
             const uint32_t flags = M->flags | (M->pairs ? (uint32_t)VL_INTERFERENCE : 0u);
             vl_verdict vd;
             vd.flags = flags ? flags : (uint32_t)VL_PASS;
@@ -388,33 +389,48 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
     const uint32_t *items = nullptr;
     uint32_t *first = reinterpret_cast<uint32_t *>(base + q.sm.total);  // ROWS: [rows + 1] first item of every row
     if (ROWS) {
-        __shared__ uint32_t s_sum[EXACT_NT / 32];
-        const uint32_t per = (q.ex.rows + EXACT_NT - 1) / EXACT_NT, k0 = tid * per, k1 = min(k0 + per, q.ex.rows);
-        uint32_t n = 0;  // of this thread's rows, coarse | fine << 16 (at most EXACT_ROWS rows: neither half overflows)
-        for (uint32_t k = k0; k < k1; ++k) {
-            const uint32_t x = q.ex.cstate[(size_t)k * 8 + CS_ITEMS];
-            first[k] = x;
-            n += x;
+        using u64 = unsigned long long;
+        __shared__ u64 s_sum[EXACT_NT / 32];
+        constexpr uint32_t U = 8;
+        bool any = false;
+        for (uint32_t k0 = tid; k0 < q.ex.rows; k0 += U * EXACT_NT) {
+            uint32_t x[U];
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) x[u] = q.ex.items[min(k0 + u * EXACT_NT, q.ex.rows - 1)];
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) {
+                if (k0 + u * EXACT_NT < q.ex.rows) first[k0 + u * EXACT_NT] = x[u];
+                any |= x[u] != 0;
+            }
         }
-        uint32_t inc = n;
+        if (!__syncthreads_or(any)) return;
+        // (an odd number of rows per thread: their places begin in different banks)
+        const uint32_t per = (q.ex.rows + EXACT_NT - 1) / EXACT_NT | 1u, k0 = tid * per, k1 = min(k0 + per, q.ex.rows);
+        // of this thread's rows: coarse items, fine items << 20, rows with any << 40
+        auto fields = [](uint32_t x) { return (u64)(x & 0xFFFFu) | (u64)(x >> 16) << 20 | (u64)(x ? 1u : 0u) << 40; };
+        u64 n = 0;
+        for (uint32_t k = k0; k < k1; ++k) n += fields(first[k]);
+        u64 inc = n;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+            const u64 y = __shfl_up_sync(0xffffffffu, inc, d);
             if (lane >= (uint32_t)d) inc += y;
         }
         if (lane == 31) s_sum[tid >> 5] = inc;
         __syncthreads();
-        uint32_t before = inc - n, all = 0;
+        u64 before = inc - n, all = 0;
 #pragma unroll
         for (uint32_t w = 0; w < EXACT_NT / 32; ++w) {
             if (w < tid >> 5) before += s_sum[w];
             all += s_sum[w];
         }
-        const uint32_t shift = all >> 16 <= q.ex.fine_items ? 16u : 0u;
-        n_items = (all >> shift) & 0xFFFFu;
-        uint32_t at = (before >> shift) & 0xFFFFu;
+        // Fine items if each has a thread block; a row each where the rows alone keep every block busy for several rounds (an
+        // item fetches its part of the row anew); else coarse ones.
+        const uint32_t shift = ((all >> 20) & 0xFFFFFu) <= q.ex.fine_items ? 20u : ((uint32_t)(all >> 40) >= EXACT_ROUNDS * gridDim.x ? 40u : 0u);
+        n_items = (uint32_t)(all >> shift) & 0xFFFFFu;
+        uint32_t at = (uint32_t)(before >> shift) & 0xFFFFFu;
         for (uint32_t k = k0; k < k1; ++k) {
-            const uint32_t x = (first[k] >> shift) & 0xFFFFu;
+            const uint32_t x = (uint32_t)(fields(first[k]) >> shift) & 0xFFFFFu;
             first[k] = at;
             at += x;
         }
@@ -580,11 +596,11 @@ int vl_hand_scratch(vl_program *p, int slot, uint64_t rows, VlExactArgs *ex)
         VL_CUDA(p, cudaFree(v.block));
         v = vl_program::VScratch{};
         rows = std::max<uint64_t>(rows, 3ull * vl_sm_count(p));
-        VL_CUDA(p, cudaMalloc(&v.block, rows * (8 + 4 + aw) * 4));
-        v.cstate = static_cast<uint32_t *>(v.block); v.racc = v.cstate + rows * 8; v.anom = v.racc + rows * 4;
+        VL_CUDA(p, cudaMalloc(&v.block, rows * (8 + 4 + 1 + aw) * 4));
+        v.cstate = static_cast<uint32_t *>(v.block); v.racc = v.cstate + rows * 8; v.work = v.racc + rows * 4; v.anom = v.work + rows;
         v.rows = rows; v.aw = aw;
     }
-    ex->cstate = v.cstate; ex->racc = v.racc; ex->anom = v.anom;
+    ex->cstate = v.cstate; ex->racc = v.racc; ex->items = v.work; ex->anom = v.anom;
     ex->AW = (uint32_t)aw; ex->nC = p->nC;
     ex->short_chunk = p->d_short_chunk; ex->chunk_short_off = p->d_chunk_short_off;
     ex->fine_items = std::min<uint32_t>(vl_exact_blocks(p), EXACT_FINE_ITEMS);

@@ -213,7 +213,7 @@ struct vl_program {
         uint32_t *thm = nullptr;       // [groups][n_blocks][mask words][2][32] through-set masks
         uint64_t rows = 0, aw = 0, vregs = 0, chunks = 0;
     } vs[VL_LANES + 2];              // one per lane, then one per staging buffer of vl_verify_host
-    VScratch fs[VL_LANES + 2];       // the same for what k_fused and k_eight hand to k_exact: cstate, anom and racc only
+    VScratch fs[VL_LANES + 2];       // the same for what k_fused and k_eight hand to k_exact: cstate, anom, racc and (in work) the rows' items
     uint32_t sub_batch = 5120;       // candidates per pass of the verify kernels
     uint32_t lanes_opt = 3;          // lanes in use (1 = everything in order on the caller's stream)
     uint64_t lane_call = 0, lane_base = 0;  // the last vl_verify* call that spread passes over lanes, the lane of its first
@@ -315,8 +315,8 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
 #define EXACT_FINE_CHUNKS 2
 #define EXACT_FINE_ITEMS 512
 #define EXACT_LONG 1024      // entries of an instruction's short list, on average, from which a warp counts them together
-// per-candidate state between the kernels (8 words); CS_ITEMS: what k_fused leaves for k_exact, coarse | fine items << 16
-enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_ITEMS = 3, CS_WALK = 6, CS_THCOL = 7 };
+// per-candidate state between the kernels (8 words)
+enum { CS_FLAGS = 0, CS_FIRST = 1, CS_BANK = 2, CS_WALK = 6, CS_THCOL = 7 };
 enum : uint32_t { WALK_ANOM = 1u, WALK_FULL = 2u };
 // Items of a candidate with that many chunks to count.
 __device__ __forceinline__ uint32_t exact_parts(uint32_t chunks, uint32_t per_item, uint32_t most = EXACT_MAX_PARTS)
@@ -342,7 +342,8 @@ struct VlExactArgs {
     const uint32_t *short_chunk, *chunk_short_off;  // [nS] chunk of every short chunk, [nC + 1] first short chunk of every chunk
     uint32_t *racc;               // [rows][4] overlaps, complement of the lowest instruction, bank tally, parts done; all 0
     uint32_t AW, nC, fine_items;      // fine_items: up to that many fine items are taken
-    uint32_t rows;                // rows of k_fused or k_eight, each of which left the number of its items in cstate; 0: listed in work
+    uint32_t rows;                // rows of k_fused or k_eight; 0: the candidates are listed in work
+    uint32_t *items;              // [rows] a row's items, coarse | fine << 16
     uint32_t exact_bank;          // and an exact bank tally (k_fused)
     unsigned char *scratch;       // vl_exact_scratch bytes, null if 0
 };

@@ -121,7 +121,7 @@ def test_bounded_wait_runs_out(B, oracle_mod, K):
 
 # counts handed over (few rows; many rows of a long program, up to the most), made by the block itself; candidates in fine items, in
 # coarse ones, one item each
-@pytest.mark.parametrize("n_instrs,K,launches", [(2399, 2000, 2), (2399, 2001, 1), (2400, 2001, 1), (2400, 8192, 1), (2400, 8193, 1), (4100, 700, 2)])
+@pytest.mark.parametrize("n_instrs,K,launches", [(2399, 2000, 2), (2399, 2001, 1), (2400, 2001, 2), (2400, 8192, 2), (2400, 8193, 1), (4100, 700, 2)])
 @pytest.mark.parametrize("noise", [0.004, 0.2, 1.0])
 def test_rows_that_collide_everywhere(B, oracle_mod, n_instrs, K, launches, noise):
     """Rows of random registers (every chunk collides, vregs outside the file, tuples across mask words) among valid ones."""
