@@ -728,24 +728,37 @@ cudaError_t launch_eight(int device, const EMany<N> &many, dim3 grid, uint32_t s
 bool vl_eight_takes(const vl_program *p) { return p->V < 16384 && p->wmax <= 8 && p->P + p->wmax <= 32768u && p->nC > 0; }
 
 // Up to one block per multiprocessor it wins over the batched kernels for every program it takes, beyond that up to about 24
-// million instructions times rows: the batched kernels look an event up for 64 rows at a time.  This kernel / the batched ones,
-// us, 10 % of the rows failing: 2,000 instructions, 1,184 rows 37 / 57, 2,368 rows 44 / 96, 4,000 rows 61 / 99; 8,000 instructions,
-// 600 rows 61 / 82, 1,184 rows 66 / 92, 2,368 rows 119 / 152, 4,000 rows 170 / 168; 11,317 instructions, 1,600 rows 99 / 115,
-// 2,368 rows 158 / 160, 4,000 rows 281 / 189; 32,000 instructions, 1,184 rows 138 / 172, 1,600 rows 233 / 233; 64 and 1,000
-// instructions, 10,000 rows 53 / 98 and 101 / 124.
+// million instructions times rows and 16,000 instructions: the batched kernels look an event up for 64 rows at a time.  This
+// kernel / the batched ones, us, 10 % of the rows failing: 2,000 instructions, 1,184 rows 37 / 49, 2,368 rows 42 / 100, 4,736 rows
+// 70 / 103, 12,000 rows 146 / 151; 8,000 instructions, 600 rows 62 / 83, 1,184 rows 66 / 92, 2,368 rows 90 / 152, 3,000 rows
+// 142 / 164; 11,900 instructions, 1,600 rows 102 / 115, 2,001 rows 103 / 114; 14,500 instructions, 1,420 rows 116 / 115, 1,550 rows 116 / 119;
+// 18,000 instructions, 1,330 rows 150 / 139; 32,000 instructions, 1,184 rows 133 / 158; 64 and 1,000 instructions, 10,000
+// rows 53 / 87 and 103 / 126, 375,000 and 24,000 rows 1,550 / 1,969 and 215 / 230.  With 40 % failing: 8,000 instructions, 1,600
+// rows 122 / 138, 3,000 rows 177 / 198.
+// Little more than one block per multiprocessor leaves most of them with one block of 256 threads: up to 1 1/6 of them the
+// line lies at 11,000 instructions.  1,190 rows, none failing and 10 %: 10,000 instructions 69 / 72 and 97 / 103, 13,000 85 / 76 and
+// 103 / 99, 16,000 101 / 86 and 120 / 109.
 #define EIGHT_INSTR_ROWS 24000000ull
+#define EIGHT_MOST_INSTRS 16000u
+#define EIGHT_EDGE_INSTRS 11000u
 bool vl_eight_wanted(vl_program *p, uint64_t K)
 {
     if (p->group_opt || p->threads_opt) return false;  // the caller asks for the batched kernels
     if (!p->d_ev8 || !p->bank_fast || p->nS > 65535u || !vl_verify_takes(p)) return false;
     if (p->known[VL_KNOWN_SEN] >= FUSED_MANY_ENTRIES || p->known[VL_KNOWN_LS] >= (uint64_t)EXACT_LONG * p->nI) return false;
-    if (K > 8ull * vl_sm_count(p) && K * p->nI > EIGHT_INSTR_ROWS) return false;
+    const uint64_t wave = 8ull * vl_sm_count(p);
+    if (K > wave && (K * p->nI > EIGHT_INSTR_ROWS || p->nI > (6 * K < 7 * wave ? EIGHT_EDGE_INSTRS : EIGHT_MOST_INSTRS))) return false;
     return eight_plan(p, K).NT != 0;
 }
 
 // Whether a job may share a launch with jobs of other programs: blocks of 256 threads, two per multiprocessor.
 bool vl_eight_shares(vl_program *p, uint64_t K) { return vl_eight_wanted(p, K) && eight_smem(p, 256, E_HALF).total; }
 
+// A job of one program leaves the counts of its rows that collide to k_exact: a row that fails would keep its block busy for longer
+// than all the rest takes.  Of more than 2,000 rows of a short program enough blocks are left to go on meanwhile, and k_exact
+// costs 4 to 7 us.  Counted by the block / handed over, us, none failing, 10 % and 40 %: 1,000 instructions, 2,368 rows
+// 19 / 24, 35 / 38, 49 / 50; 2,000 instructions 24 / 26, 42 / 42, 65 / 55; 3,000 instructions 31 / 33, 62 / 49, 81 / 67; 8,000
+// instructions 62 / 69, 119 / 92, 230 / 123.
 #define EIGHT_HAND_ROWS 2000u
 #define EIGHT_HAND_INSTRS 2400u
 

@@ -158,3 +158,25 @@ def test_tuples_across_mask_words(B, oracle_mod, K):
     assert (want["flags"] == B.VL_PASS).mean() > 0.7
     _assert_same(_gpu_verify(B, gp, rows), want)
     gp.close()
+
+
+@pytest.mark.parametrize("n_instrs,K,launches", [(11200, 1184, 2), (11200, 1190, 4), (11200, 1381, 4), (11200, 1382, 2), (10900, 1190, 2), (16100, 1430, 4), (16100, 1184, 2)])
+def test_route(B, oracle_mod, n_instrs, K, launches):
+    """On both sides of the lines beyond one block per multiprocessor (148 of them)."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the lines lie elsewhere")
+    p = _member(n_instrs, 7)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    some = _rows(p, 60, 3)
+    verdicts = op.verify(op.liveness(), some)
+    pick = np.arange(K) % 60
+    dev = _to_dev(some[pick])
+    out = gp.vl_verify(dev)
+    before = B.vl_kernel_launches()
+    gp.vl_verify(dev, out)
+    assert B.vl_kernel_launches() - before == launches, "another path has checked the rows"
+    _assert_same(B.verdicts_to_numpy(out), verdicts[pick], f"{K} rows")
+    gp.close()
