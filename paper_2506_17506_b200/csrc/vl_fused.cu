@@ -564,7 +564,7 @@ FPlan fused_plan(vl_program *p, uint64_t K)
 // 8,602, of 1,013 1,441 against 1,261, of 557 640 against 454.
 static bool long_lists(const vl_program *p) { return p->known[VL_KNOWN_LS] >= (uint64_t)EXACT_LONG * p->nI; }
 
-bool vl_fused_wanted(vl_program *p, uint64_t K)
+bool vl_fused_wanted(vl_program *p, uint64_t K, bool alone)
 {
     if (p->group_opt || p->threads_opt || p->test_wait) return false;  // the caller asks for the batched kernels
     if (!vl_verify_takes(p)) return false;                             // (refused, however few the rows)
@@ -576,7 +576,7 @@ bool vl_fused_wanted(vl_program *p, uint64_t K)
     // Where k_eight takes the job it wins sooner: 1,000 instructions, 1,184 rows 32 us against 34 there, 1,600 rows 40 against 34;
     // 2,000 instructions, 600 rows 29 against 36, 1,000 rows 47 against 38; 4,000 instructions, 400 rows 36 against 40, 600 rows 61
     // against 39.
-    return rounds <= 1 || rounds * (6000 + 7ull * p->nI) <= (vl_eight_wanted(p, K) ? 42000u : 72000u);
+    return rounds <= 1 || rounds * (6000 + 7ull * p->nI) <= (alone && vl_eight_wanted(p, K) ? 42000u : 72000u);
 }
 
 // Programs of at least that many instructions whose rows share multiprocessors hand the exact counts to k_exact: a row that
@@ -681,7 +681,7 @@ int vl_fused_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
 // share a multiprocessor whatever the others need.
 bool vl_fused_shares(vl_program *p, uint64_t K)
 {
-    return vl_fused_wanted(p, K) && fused_smem(p, 256).total <= 48 * 1024;
+    return vl_fused_wanted(p, K, false) && fused_smem(p, 256).total <= 48 * 1024;
 }
 
 // Shared memory of a block of k_exact; beyond what a multiprocessor has, its arrays take global memory.

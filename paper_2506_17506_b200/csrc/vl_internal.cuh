@@ -286,7 +286,7 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
 // The one-kernel verify path of short jobs (vl_fused.cu): whether a job of K rows takes it, whether it may share a
 // launch with other programs' jobs, and one launch for n <= VL_FUSED_MANY jobs.
 #define VL_FUSED_MANY 48
-bool vl_fused_wanted(vl_program *p, uint64_t K);
+bool vl_fused_wanted(vl_program *p, uint64_t K, bool alone = true);  // alone: k_eight would take the job instead
 // Entries of the short chunks (vreg and short chunk at whose beginning it is occupied) from which a program counts as one
 // that occupies many.
 #define FUSED_MANY_ENTRIES 49152u  // (measured at vl_fused_wanted)

@@ -1822,9 +1822,13 @@ enum Together { SHARED, SINGLE, BATCHED, EIGHT };
 // multiprocessor.  In EIGHT / in the best of the others, us: 96 programs of 2,000 instructions with 148 rows 207 / 536, 48 of 4,000 with
 // 128 163 / 343, 16 of 4,000 with 100 73 / 103, 16 of 2,000 with 100 49 / 70, 8 of 8,000 with 100 100 / 91, 4 of 2,000 with 100 45 / 35,
 // 64 of 2,000 with 8 90 / 83.
+// Programs all with more rows than a round of k_fused takes (444) have estimates of their own for EIGHT and the batched kernels, whose
+// launches then cost less than their work.  Measured / estimated, EIGHT, batched: 4 x 300 x 3,000 rows 96/76, 104/91; 8 x 1,000 x 1,500
+// 135/112, 131/131; 8 x 2,000 x 900 108/112, 118/131; 32 x 2,000 x 900 349/341, 437/387; 8 x 4,000 x 450 110/117, 103/125; 8 x 4,000 x
+// 800 152/166, 137/160; 16 x 4,000 x 600 205/222, 228/235.
 Together together(uint32_t nprog, vl_program *const *progs, const uint64_t *K, const std::vector<uint8_t> &shares)
 {
-    double n = 0, rows = 0, work = 0, longest = 0, blocks = 0;
+    double n = 0, rows = 0, work = 0, longest = 0, blocks = 0, fewest = 1e30;
     bool eights = true;
     for (uint32_t j = 0; j < nprog; ++j) {
         if (!shares[j]) continue;
@@ -1833,6 +1837,7 @@ Together together(uint32_t nprog, vl_program *const *progs, const uint64_t *K, c
         rows += (double)K[j];
         work += a * (double)K[j];
         longest = std::max(longest, a);
+        fewest = std::min(fewest, (double)K[j]);
         blocks += (double)((K[j] + 7) / 8);
         eights = eights && vl_eight_shares(progs[j], K[j]);
     }
@@ -1841,6 +1846,8 @@ Together together(uint32_t nprog, vl_program *const *progs, const uint64_t *K, c
     const double shared = 35 + 8 * longest + rows / (3 * sms) * (10 + 2.8 * a);
     const double single = 35 + 4 * n + rows / sms * (6 + 1.2 * a);
     const double batched = 75 + 17.7 * n + 0.0019 * work;
+    const bool many = fewest > 3 * sms;
+    if (many && eights) return 20 + 8 * longest + blocks / (2 * sms) * (8 + 8.5 * a) <= 45 + 4.5 * n + 0.0015 * rows + 0.0027 * work ? EIGHT : BATCHED;
     const double eight = 40 + 12 * longest + blocks / (2 * sms) * (10 + 12.3 * a);
     if (eights && eight <= shared && eight <= single && eight <= batched) return EIGHT;
     return shared <= single && shared <= batched ? SHARED : (single <= batched ? SINGLE : BATCHED);
@@ -1897,7 +1904,7 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
         if (K[j] == 0) continue;
         vl_program *p = progs[j];
         if ((how == SHARED || how == EIGHT) && shares[j]) continue;
-        if (!(how == BATCHED && shares[j]) && vl_fused_wanted(p, K[j])) {
+        if (!(how == BATCHED && shares[j]) && vl_fused_wanted(p, K[j], false)) {
             rc = vl_fused_run(1, &p, d_cand + j, K + j, pitch + j, d_out + j, st, lane[job % L], dict, (int)(job % L));
             ++job;
             continue;

@@ -71,14 +71,42 @@ def test_random_programs(B, oracle_mod, P, widths, banks, max_blocks):
         gp.close()
 
 
+@pytest.mark.parametrize("n,n_instrs,K,launches", [(4, 2000, 900, 1), (9, 4000, 600, 1), (4, 300, 3000, 1), (8, 4000, 800, 32)])
+def test_programs_of_many_rows(B, oracle_mod, n, n_instrs, K, launches):
+    """Jobs that k_eight would take alone and that k_fused could: they share a launch of one or the other, or run batched (the last)."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the lines lie elsewhere")
+    progs = [_member(n_instrs, 60 + j) for j in range(n)]
+    gps = [B.Program(p) for p in progs]
+    B.vl_liveness_batch(gps)
+    pick = np.arange(K) % 50
+    devs, wants = [], []
+    for j, p in enumerate(progs):
+        op = oracle_mod.OracleProgram(p)
+        some = _rows(p, 50, j)
+        wants.append(op.verify(op.liveness(), some)[pick])
+        devs.append(_to_dev(some[pick]))
+    B.vl_verify_batch(gps, devs)
+    before = B.vl_kernel_launches()
+    outs = B.vl_verify_batch(gps, devs)
+    torch.cuda.synchronize()
+    assert B.vl_kernel_launches() - before == launches
+    for o, w in zip(outs, wants):
+        _assert_same(B.verdicts_to_numpy(o), w)
+    for gp in gps:
+        gp.close()
+
+
 def test_several_programs(B, oracle_mod):
     """Jobs of several programs in one call, enough of them for the kernel to take them together; one that it does not take."""
     import torch
     progs = [_member(900 + 331 * j, j) for j in range(9)]
-    Ks = [100, 131, 8, 1, 97, 200, 148, 120, 90]
+    progs.append(H.random_program(8900, max_instrs=900, max_vregs=200, P=64, widths=(1, 9)))
+    Ks = [100, 131, 8, 1, 97, 200, 148, 120, 90, 110]
     gps = [B.Program(p) for p in progs]
     B.vl_liveness_batch(gps)
-    rows = [_rows(p, K, K) for p, K in zip(progs, Ks)]
+    rows = [_rows(p, K, K) if p.gen else _garbage_rows(p, K, K) for p, K in zip(progs, Ks)]
     wants = []
     for p, r in zip(progs, rows):
         op = oracle_mod.OracleProgram(p)
