@@ -28,7 +28,7 @@
 #define PIECE_INSTRS 8         // instructions of a piece, at most
 #define PC_WARPS 20            // warps per block of k_sets and k_count: the pieces of a chunk of the default size at once
 #define PC_NT (PC_WARPS * 32)
-#define PIECE_OPERANDS 32      // and its operands, unless it is a single instruction: one per lane
+#define PIECE_OPERANDS 32      // and its operands, one per lane, unless its instructions have many (vl_layout)
 #define LV_WARPS 8             // warps per block of k_fill
 #define LV_NT (LV_WARPS * 32)
 #define FILL_WARP_WORDS (32 + 1024 + 256)  // shared memory of a warp of k_fill behind its two bitsets
@@ -151,8 +151,8 @@ __device__ T block_excl_scan(T x, T *s_scan, T *total)
 
 // An operand of a piece as a word: vreg (16 bits), instruction inside the piece (4 bits at 16), and how it meets the piece's
 // other operands, which the layout of the program fixes (k_operand_words; found anew in every run, by shuffles or matches of
-// a warp's lanes, it took k_sets and k_count half of their time).  In a piece that is a single instruction of more than
-// PIECE_OPERANDS operands only OW_DEF and OW_EXPOSED are set.
+// a warp's lanes, it took k_sets and k_count half of their time).  In a piece of more than PIECE_OPERANDS operands only OW_DEF
+// and OW_EXPOSED are set.
 enum : uint32_t {
     OW_DEF = 1u << 20,      // definition
     OW_DUP = 1u << 21,      // read: an earlier read of the instruction has the vreg
@@ -399,44 +399,67 @@ __device__ __forceinline__ void count_narrow(const Piece &po, uint32_t x, const 
     }
 }
 
-// The same for a piece that is a single instruction with more operands.  reads: an empty bitset of this warp's own.
+// The same for a piece with more operands: instruction by instruction, from the last to the first.  reads: an empty bitset of
+// this warp's own; live: one for the live set (null: the piece is a single instruction).
 // (200 instructions of 60 reads 172 us for the run, all operands met in pairs 976; 100 of 100 definitions 202 and 2,133)
 template <bool GLOBAL>  // touch lies in global memory
 __device__ __noinline__ void count_wide(const LiveArgs &q, const Piece &po, const uint32_t *end, volatile uint32_t *reads,
-                                        uint8_t *opflags, uint32_t *touch, uint32_t *s_ev)
+                                        volatile uint32_t *live, uint8_t *opflags, uint32_t *touch, int *s_d, uint32_t *s_ev)
 {
-    const uint32_t lane = threadIdx.x & 31, nd = q.ndefs[po.i0], r0 = po.o0 + nd, o1 = po.o0 + po.n;
+    const uint32_t lane = threadIdx.x & 31;
     auto has = [](const volatile uint32_t *s, uint32_t v) { return (s[v >> 5] >> (v & 31)) & 1u; };
-    uint32_t n_ev = 0;
-    auto event = [&](uint32_t v, uint32_t n) {
-        const uint32_t bit = 1u << (v & 31);
-        n_ev += n;
-        if (n && (!GLOBAL || !(__ldcg(&touch[v >> 5]) & bit))) atomicOr(&touch[v >> 5], bit);
-    };
-    for (uint32_t o = r0; o < o1; o += 32) {  // which reads are the first of their vreg
-        const bool mine = o + lane < o1;
-        const uint32_t v = mine ? q.op_vreg[o + lane] : 0x10000u + lane;
-        const uint32_t same = __match_any_sync(0xffffffffu, v);
-        const bool dup = mine && ((same & low_bits(lane)) || has(reads, v));
+    if (live) {
+        for (uint32_t w = lane; w < q.Wv; w += 32) live[w] = end[w];
         __syncwarp();
-        if (mine) {
+    }
+    const volatile uint32_t *after = live ? live : end;
+    for (uint32_t k = po.ni; k-- > 0;) {
+        const uint32_t o0 = q.op_off[po.i0 + k], nd = q.ndefs[po.i0 + k], r0 = o0 + nd, o1 = q.op_off[po.i0 + k + 1];
+        uint32_t n_ev = 0;
+        auto event = [&](uint32_t v, uint32_t n) {
+            const uint32_t bit = 1u << (v & 31);
+            n_ev += n;
+            if (n && (!GLOBAL || !(__ldcg(&touch[v >> 5]) & bit))) atomicOr(&touch[v >> 5], bit);
+        };
+        for (uint32_t o = r0; o < o1; o += 32) {  // which reads are the first of their vreg
+            const bool mine = o + lane < o1;
+            const uint32_t v = mine ? q.op_vreg[o + lane] : 0x10000u + lane;
+            const uint32_t same = __match_any_sync(0xffffffffu, v);
+            const bool dup = mine && ((same & low_bits(lane)) || has(reads, v));
+            __syncwarp();
+            if (mine) {
+                uint32_t flags;
+                if (!dup) atomicOr(const_cast<uint32_t *>(reads) + (v >> 5), 1u << (v & 31));
+                event(v, operand_events(nd > 1, false, has(after, v), dup, false, &flags));
+                opflags[o - po.o0 + lane] = (uint8_t)flags;
+            }
+            __syncwarp();
+        }
+        for (uint32_t o = o0 + lane; o < r0; o += 32) {
+            const uint32_t v = q.op_vreg[o];
             uint32_t flags;
-            if (!dup) atomicOr(const_cast<uint32_t *>(reads) + (v >> 5), 1u << (v & 31));
-            event(v, operand_events(nd > 1, false, has(end, v), dup, false, &flags));
-            opflags[o - po.o0 + lane] = (uint8_t)flags;
+            event(v, operand_events(nd > 1, true, has(after, v), false, has(reads, v), &flags));
+            opflags[o - po.o0] = (uint8_t)flags;
         }
         __syncwarp();
+        int change = 0;  // of the live count, going backwards
+        if (live) {
+            for (uint32_t o = o0 + lane; o < r0; o += 32) {
+                const uint32_t v = q.op_vreg[o];
+                if (has(live, v)) { --change; atomicAnd(const_cast<uint32_t *>(live) + (v >> 5), ~(1u << (v & 31))); }
+            }
+            __syncwarp();
+            for (uint32_t o = r0 + lane; o < o1; o += 32) {
+                const uint32_t v = q.op_vreg[o], bit = 1u << (v & 31);
+                if (!(atomicOr(const_cast<uint32_t *>(live) + (v >> 5), bit) & bit)) ++change;
+            }
+        }
+        for (uint32_t o = r0 + lane; o < o1; o += 32) reads[q.op_vreg[o] >> 5] = 0;
+        n_ev = __reduce_add_sync(0xffffffffu, n_ev);
+        change = __reduce_add_sync(0xffffffffu, change);
+        if (lane == 0) { s_ev[k] = n_ev; s_d[k] = change; }
+        __syncwarp();
     }
-    for (uint32_t o = po.o0 + lane; o < r0; o += 32) {
-        const uint32_t v = q.op_vreg[o];
-        uint32_t flags;
-        event(v, operand_events(nd > 1, true, has(end, v), false, has(reads, v), &flags));
-        opflags[o - po.o0] = (uint8_t)flags;
-    }
-    __syncwarp();
-    for (uint32_t o = r0 + lane; o < o1; o += 32) reads[q.op_vreg[o] >> 5] = 0;
-    n_ev = __reduce_add_sync(0xffffffffu, n_ev);
-    if (lane == 0) s_ev[0] = n_ev;
 }
 
 // ============================================================================ k_count
@@ -496,12 +519,13 @@ __global__ void __launch_bounds__(PC_NT) k_count(const __grid_constant__ LiveMan
         cnt = __reduce_add_sync(0xffffffffu, cnt);
         if (!WIDE || po.n <= PIECE_OPERANDS) {
             count_narrow(po, x, end, q.opflags + po.o0, touch, touched, s_d[warp], s_ev[warp]);
-        } else {  // the set of reads: in shared memory if it fits, else in the row of the piece's own sets, used up by now
+        } else {  // the sets of reads and of what is live: in shared memory if they fit, else in the rows of the piece's own sets, used up by now
             extern __shared__ uint32_t sm[];
-            uint32_t *reads = q.wide_smem ? sm + (size_t)warp * q.Wv : q.piece_def + (size_t)p * q.Wv;
+            uint32_t *reads = q.wide_smem ? sm + (size_t)warp * 2 * q.Wv : q.piece_def + (size_t)p * q.Wv;
+            uint32_t *live = q.wide_smem ? reads + q.Wv : q.piece_use + (size_t)p * q.Wv;
             for (uint32_t w = lane; w < q.Wv; w += 32) reads[w] = 0;
             __syncwarp();
-            count_wide<true>(q, po, end, reads, q.opflags + po.o0, touch, s_ev[warp]);
+            count_wide<true>(q, po, end, reads, po.ni > 1 ? live : nullptr, q.opflags + po.o0, touch, s_d[warp], s_ev[warp]);
         }
         __syncwarp();
         // live after instruction k = live after the piece + what the later instructions add going backwards
@@ -844,7 +868,7 @@ __global__ void __launch_bounds__(SMALL_NT, 2) k_small(const __grid_constant__ L
             uint32_t *reads = sm + L.rd + warp * Wv;
             for (uint32_t w = lane; w < Wv; w += 32) reads[w] = 0;
             __syncwarp();
-            count_wide<false>(q, x, end, reads, s_fl + x.o0 - o_first, touch, s_ev[warp]);
+            count_wide<false>(q, x, end, reads, nullptr, s_fl + x.o0 - o_first, touch, s_d[warp], s_ev[warp]);
         }
         __syncwarp();
         // live after instruction k = live after the piece + what the later instructions add going backwards
@@ -958,8 +982,15 @@ __global__ void __launch_bounds__(NT) k_operand_words(uint32_t nP, const uint32_
     const uint32_t p = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (p >= nP) return;
     const uint32_t i0 = piece_i0[p], i1 = piece_i0[p + 1], o0 = op_off[i0], n = op_off[i1] - o0;
-    if (n > PIECE_OPERANDS) {  // a single instruction: it reads before it writes
-        for (uint32_t j = lane; j < n; j += 32) op_word[o0 + j] = op_vreg[o0 + j] | (j < ndefs[i0] ? OW_DEF : OW_EXPOSED);
+    if (n > PIECE_OPERANDS) {
+        for (uint32_t j = lane, i = i0; j < n; j += 32) {
+            while (op_off[i + 1] <= o0 + j) ++i;
+            const uint32_t v = op_vreg[o0 + j];
+            bool fresh = true;  // no earlier instruction of the piece writes the vreg
+            for (uint32_t h = i0; h < i; ++h)
+                for (uint32_t d = 0; d < ndefs[h]; ++d) fresh = fresh && op_vreg[op_off[h] + d] != v;
+            op_word[o0 + j] = v | ((i - i0) << 16) | (o0 + j - op_off[i] < ndefs[i] ? OW_DEF : (fresh ? OW_EXPOSED : 0u));
+        }
         return;
     }
     const bool mine = lane < n;
@@ -1339,8 +1370,14 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         for (uint64_t j = 0; j < nc; ++j) {
             const uint32_t i0 = (uint32_t)(s + j * n / nc), i1 = (uint32_t)(s + (j + 1) * n / nc);
             c_p_off.push_back((uint32_t)p_i0.size());
+            // Instructions of more operands than half a piece's would each be a piece, with three sets of all vregs: in a long
+            // program they share one, whose operands are taken instruction by instruction.  (32,000 instructions of 24
+            // operands each, 500 and 10,666 vregs, a run of theirs: 221 us and 1,663, so 155 and 1,087)
+            auto many = [&](uint32_t i) { return p->nI > LIVE_SMALL_INSTRS && p->h_op_off[i + 1] - p->h_op_off[i] > PIECE_OPERANDS / 2; };
             for (uint32_t q0 = i0, q1; q0 < i1; q0 = q1) {
-                for (q1 = q0 + 1; q1 < i1 && q1 < q0 + PIECE_INSTRS && p->h_op_off[q1 + 1] - p->h_op_off[q0] <= PIECE_OPERANDS;) ++q1;
+                for (q1 = q0 + 1; q1 < i1 && q1 < q0 + PIECE_INSTRS && many(q0) && many(q1);) ++q1;
+                if (q1 == q0 + 1)
+                    while (q1 < i1 && q1 < q0 + PIECE_INSTRS && p->h_op_off[q1 + 1] - p->h_op_off[q0] <= PIECE_OPERANDS) ++q1;
                 p_i0.push_back(q0);
                 p_chunk.push_back((uint32_t)c_i0.size());
             }
@@ -1541,7 +1578,7 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     sh.fills = (nP + LV_WARPS - 1) / LV_WARPS + nC + ((p->nS + 31) & ~31u) / LV_WARPS + nB;
     sh.sets_smem = (size_t)sh.set_warps * 2 * Wv * 4;
     sh.wide = p->wide_pieces;
-    sh.count_smem = p->wide_pieces ? (size_t)PC_WARPS * Wv * 4 : 0;
+    sh.count_smem = p->wide_pieces ? (size_t)PC_WARPS * 2 * Wv * 4 : 0;
     q.wide_smem = sh.count_smem <= 40 * 1024;
     if (!q.wide_smem) sh.count_smem = 0;
     sh.flow_smem = flow_smem;

@@ -35,9 +35,11 @@ def _program(n_instrs, n_blocks, n_vregs, max_reads, seed):
 
 
 # instructions around 32 pieces (one block or a cluster) and around 4,096 (a cluster or the separate kernels); instructions of so
-# many operands that a piece holds one, or is one; more than 32 and more than 1,024 vregs; many blocks, few chunks, long chunks
+# many operands that a piece holds one, or is one; more than 32 and more than 1,024 vregs; many blocks, few chunks, long chunks;
+# long programs whose instructions of many operands share pieces, with bitsets that fit shared memory and ones that do not
 CASES = [(256, 1, 5, 3, 160), (257, 2, 40, 3, 160), (250, 3, 70, 40, 160), (1000, 7, 1100, 6, 160), (4096, 5, 300, 3, 160),
-         (4097, 5, 300, 3, 160), (2000, 40, 200, 4, 160), (2000, 3, 200, 4, 8), (3000, 2, 100, 3, 65536), (300, 2, 2100, 100, 24)]
+         (4097, 5, 300, 3, 160), (2000, 40, 200, 4, 160), (2000, 3, 200, 4, 8), (3000, 2, 100, 3, 65536), (300, 2, 2100, 100, 24),
+         (4200, 5, 300, 40, 160), (4300, 2, 40, 90, 24), (6000, 3, 9000, 60, 160)]
 
 
 @pytest.mark.parametrize("n_instrs,n_blocks,n_vregs,max_reads,chunk", CASES)
