@@ -74,16 +74,16 @@ __device__ __forceinline__ uint32_t pk8_get(const uint4 &x, int g)
 }
 
 // Hardware rules on where the tuples may sit (alignment, registers of the vreg's class, reserved registers) for the eight
-// candidates of a block, by its NT consumer threads, which meet on barrier BAR.  bits: room for P + 63 bits, the reserved
+// candidates of a block, by its NT consumer threads, which meet on barrier BAR.  bits: room for P + 64 bits, the reserved
 // registers.  All eight are checked without a branch and only a violation is looked at: with a branch per candidate and two loads
 // behind it (a prefix count of the reserved registers in global memory) the sweep took 18.4 k cycles of a block with 3,301
-// vregs, now 13.4 (777 rows of 11,317 instructions 89.5 us, 85.8).
+// vregs, now 13.4 (777 rows of 11,317 instructions 93.0 us, 91.2; 4,096 of 32,000 618, 576).
 template <int NT, int BAR>
 __device__ __noinline__ void rules_sweep8(const uint4 *vcons, const uint16_t *rs_prefix, const uint32_t *vinfo,
                                           const uint32_t *first_def_instr, uint32_t V, uint32_t P, const uint4 *T,
                                           uint32_t *bits, uint32_t *flags, uint32_t *minR)
 {
-    const uint32_t tid = threadIdx.x, n_words = (P + 63) / 32;
+    const uint32_t tid = threadIdx.x, n_words = P / 32 + 2;  // (a range that begins at P looks at the word after it)
     for (uint32_t r = tid; r < n_words * 32; r += NT) {
         const uint32_t word = __ballot_sync(0xffffffffu, rs_prefix && r < P && rs_prefix[r + 1] != rs_prefix[r]);
         if ((tid & 31) == 0) bits[r >> 5] = word;

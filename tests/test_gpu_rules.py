@@ -64,6 +64,31 @@ def test_random_small_programs_with_rules(B, oracle_mod, seed):
     gp.close()
 
 
+@pytest.mark.parametrize("P", [256, 479, 512])
+def test_rules_on_wide_tuples(B, oracle_mod, P):
+    """Reserved registers under tuples of up to 200 registers, in files that end with a mask word and inside one: in every kernel."""
+    rng = np.random.default_rng(P)
+    for seed in range(3):
+        p = H.random_program(6100 + seed, max_instrs=60, max_vregs=20, P=P, widths=(1, 31, 32, 33, 64, 65, 200))
+        gp = B.Program(p)
+        gp.vl_liveness()
+        op = oracle_mod.OracleProgram(p)
+        lv = op.liveness()
+        rows = np.concatenate([_garbage_rows(p, 40, seed), np.stack([H.row_from_table(p, rng.choice([0, 1, 30, P - 200], p.n_vregs)) for _ in range(20)])])
+        plain = op.verify(lv, rows)
+        changed = 0
+        for reserved in ([P - 1], [33], [0, 64, 100, P - 32], list(range(P - 70, P - 66))):
+            op.set_constraints(reserved=reserved)
+            gp.set_constraints(P=p.P, reserved=reserved)
+            want = op.verify(lv, rows)
+            changed += int((want != plain).sum())
+            for G in (0, 1, 2, 4, 8):
+                gp.set_option(B.VL_OPT_GROUP, G)
+                _assert_same(_gpu_verify(B, gp, rows), want, f"seed {seed} reserved {reserved} G {G}")
+        assert changed > 20, "the rules change next to nothing"
+        gp.close()
+
+
 def test_gemm_workload_with_rules(B, oracle_mod):
     """The GEMM-shaped workload: its valid rows keep every tuple on a multiple of its width, so
     alignment = width changes nothing for them; reserved registers and classes fail the rows that
