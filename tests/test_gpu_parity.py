@@ -204,7 +204,7 @@ def test_register_file_too_large_is_refused(B):
 
 @pytest.mark.parametrize("lanes,sub", [(1, 64), (2, 32), (3, 96), (4, 32), (8, 32), (4, 4096)])
 def test_passes_over_lanes(B, oracle_mod, lanes, sub):
-    """Many passes spread over the internal streams give the records of a single pass."""
+    """Many passes spread over the internal streams (the batched kernels) give the records of a single pass, and of one kernel."""
     wl = synth.workload(1)
     p = synth.build_program(wl.shapes[0], wl.seeds[0])
     gp, lv = _check_liveness(B, oracle_mod, p)
@@ -213,8 +213,9 @@ def test_passes_over_lanes(B, oracle_mod, lanes, sub):
     want = oracle_mod.OracleProgram(p).verify(lv, rows)
     gp.set_option(B.VL_OPT_LANES, lanes)
     gp.set_option(B.VL_OPT_SUB_BATCH, sub)
-    for _ in range(2):                                               # working sets reused by the next call
-        _assert_same(_gpu_verify(B, gp, rows), want, f"lanes {lanes} sub {sub}")
+    for group in (0, 0, 8, 8):                                       # working sets reused by the next call
+        gp.set_option(B.VL_OPT_GROUP, group)
+        _assert_same(_gpu_verify(B, gp, rows), want, f"lanes {lanes} sub {sub} group {group}")
     gp.close()
 
 
@@ -307,7 +308,9 @@ def test_recount_work_list_full(B, oracle_mod):
         if chunk:
             gp.set_option(B.VL_OPT_CHUNK_INSTRS, chunk)
             gp.vl_liveness()
-        _assert_same(_gpu_verify(B, gp, rows), want, f"sub {sub} chunk {chunk}")
+        for group in (0, 8):
+            gp.set_option(B.VL_OPT_GROUP, group)
+            _assert_same(_gpu_verify(B, gp, rows), want, f"sub {sub} chunk {chunk} group {group}")
     gp.close()
 
 
@@ -370,15 +373,18 @@ def test_determinism(B):
     gp.close()
 
 
-def test_liveness_and_verify_on_different_streams(B, oracle_mod):
+@pytest.mark.parametrize("group", [0, 8])
+def test_liveness_and_verify_on_different_streams(B, oracle_mod, group):
     """vl_liveness runs on an internal stream and holds no caller stream; vl_verify waits for it on the
     device where it reads its results.  Liveness on one stream, verify on another, no synchronisation
-    in between, new rows every step, several passes per call: every verdict must be right."""
+    in between, new rows every step: every verdict must be right.  One kernel that waits in front of the rows (0), and
+    (8) several passes over the internal streams, whose table kernels run beside the liveness run."""
     import torch
     wl = synth.workload(2)
     p = synth.build_program(wl.shapes[0], wl.seeds[0])
     gp, lv = _check_liveness(B, oracle_mod, p)
     gp.set_option(B.VL_OPT_SUB_BATCH, 128)
+    gp.set_option(B.VL_OPT_GROUP, group)
     orc = oracle_mod.OracleProgram(p)
     s_live, s_ver = torch.cuda.Stream(), torch.cuda.Stream()
     outs, wants = [], []
