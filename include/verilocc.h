@@ -58,7 +58,7 @@ enum {
                                 many microseconds apart (0..200, default 12), so that not all of them stream, then all of them
                                 sweep, in step; only for calls of at least two waves */
     VL_OPT_TEST_WAIT = 7     /* test hook for the bounded device waits: 1 = the table kernel (8 candidates per
-                                block), or the one kernel that checks a job of up to a few thousand rows, waits for its
+                                block), or the one kernel that checks a job of some hundred rows and more, waits for its
                                 first tile on a barrier that nothing completes, with a short poll limit, so that the wait
                                 runs out: the call still returns, its verdicts are garbage and vl_verify_status reports
                                 VL_ERR_DEVICE_WAIT.  0 = normal (default) */
@@ -165,8 +165,10 @@ int vl_liveness_result(const vl_program *prog, const uint32_t **blk_live_in, con
  * A call with more than one pass (VL_OPT_SUB_BATCH; the passes of a call are made equally long)
  * spreads its passes over internal streams of the device (VL_OPT_LANES) that fork from and join
  * back into `cuda_stream`, so that kernels of different passes run side by side; with
- * VL_OPT_LANES = 1 every kernel is enqueued on `cuda_stream` itself.  Jobs of up to a few thousand rows, depending on the
- * program, are checked by one or two kernels on `cuda_stream`, whatever these two options say.
+ * VL_OPT_LANES = 1 every kernel is enqueued on `cuda_stream` itself.  Jobs of up to about 24 million instructions times
+ * rows (1,000 to 2,000 rows of a program of more than 8,000 instructions, some hundred thousand of one of 64) are checked by one or
+ * two kernels, whatever these two options say.  Calls on one handle share its working memory: order a call on another stream
+ * behind the earlier ones.
  * Host work of a call: the handle is modified (it owns the working memory of its calls).  The first
  * call on a handle, and a later one that needs larger working sets (more rows per pass, another
  * chunk size, more internal streams in use, few rows after many or many after few: those are different kernels), allocates them with cudaMalloc and clears them, which

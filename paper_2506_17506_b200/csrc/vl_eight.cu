@@ -756,11 +756,17 @@ bool vl_eight_shares(vl_program *p, uint64_t K) { return vl_eight_wanted(p, K) &
 
 // A job of one program leaves the counts of its rows that collide to k_exact: a row that fails would keep its block busy for longer
 // than all the rest takes.  Of more than 2,000 rows of a short program enough blocks are left to go on meanwhile, and k_exact
-// costs 4 to 7 us.  Counted by the block / handed over, us, none failing, 10 % and 40 %: 1,000 instructions, 2,368 rows
+// costs 4 to 7 us, and more the more rows there are to look through.  Counted by the block / handed over, us, none failing, 10 % and 40 %: 1,000 instructions, 2,368 rows
 // 19 / 24, 35 / 38, 49 / 50; 2,000 instructions 24 / 26, 42 / 42, 65 / 55; 3,000 instructions 31 / 33, 62 / 49, 81 / 67; 8,000
-// instructions 62 / 69, 119 / 92, 230 / 123.
+// instructions 62 / 62, 119 / 87, 230 / 118; 3,000 instructions, 4,736 rows 59 / 58, 92 / 82, 126 / 122, 8,000 rows 101 / 105,
+// 136 / 140, 186 / 189.
 #define EIGHT_HAND_ROWS 2000u
 #define EIGHT_HAND_INSTRS 2400u
+
+bool vl_eight_hands(vl_program *p, uint64_t rows)
+{
+    return vl_exact_takes_rows(p, rows) && (rows <= EIGHT_HAND_ROWS || (p->nI >= EIGHT_HAND_INSTRS && rows <= 2ull * p->nI));
+}
 
 int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
                  vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot)
@@ -810,7 +816,7 @@ int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_
     } else {
         EMany<1> one;
         one.p[0] = many.p[0];
-        if (slot >= 0 && vl_exact_takes_rows(p0, rows) && (rows <= EIGHT_HAND_ROWS || p0->nI >= EIGHT_HAND_INSTRS)) {
+        if (slot >= 0 && vl_eight_hands(p0, rows)) {
             VlExactArgs &ex = one.p[0].f.ex;
             const int rc = vl_hand_scratch(p0, slot, rows, &ex);
             if (rc != VL_OK) return rc;

@@ -297,6 +297,7 @@ bool vl_verify_takes(const vl_program *p);  // whether the verify path takes the
 bool vl_eight_takes(const vl_program *p);
 bool vl_eight_wanted(vl_program *p, uint64_t K);
 bool vl_eight_shares(vl_program *p, uint64_t K);
+bool vl_eight_hands(vl_program *p, uint64_t rows);  // whether a job of its own leaves counts to k_exact, in a working set
 int vl_eight_run(uint32_t n, vl_program *const *progs, const uint16_t *const *d_cand, const uint64_t *K, const uint64_t *pitch,
                  vl_verdict *const *d_out, cudaStream_t from, cudaStream_t st, bool dict, int slot);  // slot: working set, -1: none
 bool vl_fused_shares(vl_program *p, uint64_t K);

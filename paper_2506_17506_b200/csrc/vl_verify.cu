@@ -16,8 +16,8 @@
 //            has no overlap.  The thread block that ends a group of 64 candidates writes the verdicts
 //            of its clean candidates and lists the others for k_exact
 //            (vl_fused.cu), which counts their overlaps from the per-instruction live-after lists.
-// Jobs of up to a few hundred rows take one kernel instead (k_fused, vl_fused.cu), jobs of up to a few thousand another (k_eight,
-// vl_eight.cu).
+// Jobs of up to a few hundred rows take one kernel instead (k_fused, vl_fused.cu), jobs of up to a few million instructions times
+// rows another (k_eight, vl_eight.cu).
 #include <cuda.h>
 
 #include <algorithm>
@@ -1870,8 +1870,18 @@ int vl_verify_lanes(uint32_t nprog, vl_program *const *progs, const uint16_t *co
     const uint32_t L = p0->lanes_opt == 1 ? 1u : (nprog > 1 ? (uint32_t)VL_LANES : std::min<uint32_t>(VL_LANES, p0->lanes_opt));
     uint64_t jobs = 0;
     for (uint32_t j = 0; j < nprog; ++j) jobs += (K[j] + progs[j]->sub_batch - 1) / progs[j]->sub_batch;
-    // one launch, however many the rows
-    if (nprog == 1 && !vl_fused_wanted(p0, K[0]) && vl_eight_wanted(p0, K[0])) return vl_eight_run(1, progs, d_cand, K, pitch, d_out, st, st, dict, 0);
+    // One launch, however many the rows.  (What is more than a pass elsewhere keeps its working set to an internal stream here too,
+    // so that such calls on two streams do not meet in it.)
+    if (nprog == 1 && !vl_fused_wanted(p0, K[0]) && vl_eight_wanted(p0, K[0])) {
+        if (L == 1 || jobs <= 1 || !vl_eight_hands(p0, K[0])) return vl_eight_run(1, progs, d_cand, K, pitch, d_out, st, st, dict, 0);
+        VL_CUDA(p0, cudaEventRecord(p0->ev_fork, st));
+        VL_CUDA(p0, cudaStreamWaitEvent(lane[0], p0->ev_fork, 0));
+        rc = vl_eight_run(1, progs, d_cand, K, pitch, d_out, st, lane[0], dict, 0);
+        cudaError_t e = cudaEventRecord(p0->ev_join[0], lane[0]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, p0->ev_join[0], 0);
+        if (e != cudaSuccess && rc == VL_OK) { p0->last_cuda_error = (int)e; rc = VL_ERR_CUDA; }
+        return rc;
+    }
     if (L == 1 || jobs <= 1) {
         FusedGroup g;
         for (uint32_t j = 0; j < nprog; ++j) {

@@ -32,10 +32,17 @@ def _rows(p, K, seed):
     return rows
 
 
-# rows: 512 threads, 256 threads, counts handed over or made by the block itself, a block with a single row; columns: whole tiles,
-# one more, few
-@pytest.mark.parametrize("n_instrs,K", [(2000, 889), (2000, 1500), (2000, 2001), (2001, 1184), (2003, 1185), (1500, 3001), (4000, 800)])
-def test_row_counts(B, oracle_mod, n_instrs, K):
+def _launches(B, call):
+    before = B.vl_kernel_launches()
+    call()
+    return B.vl_kernel_launches() - before
+
+
+# rows: 512 threads, 256 threads, counts handed over or made by the block itself (one launch less), a block with a single row;
+# columns: whole tiles, one more, few
+@pytest.mark.parametrize("n_instrs,K,launches", [(2000, 889, 2), (2000, 1500, 2), (2000, 2001, 1), (2001, 1184, 2), (2003, 1185, 2), (1500, 3001, 1),
+                                                 (4000, 800, 2)])
+def test_row_counts(B, oracle_mod, n_instrs, K, launches):
     p = _member(n_instrs, n_instrs + K)
     gp = B.Program(p)
     gp.vl_liveness()
@@ -48,6 +55,38 @@ def test_row_counts(B, oracle_mod, n_instrs, K):
     drows = synth.dict_rows(p, rows)
     got = B.verdicts_to_numpy(gp.vl_verify_dict(_to_dev(drows)))
     _assert_same(got, op.verify_dict(lv, drows), "dictionary rows")
+    dev, ddev = _to_dev(rows), _to_dev(drows)
+    assert _launches(B, lambda: gp.vl_verify(dev)) == launches, "another path has checked the rows"
+    assert _launches(B, lambda: gp.vl_verify_dict(ddev)) == launches, "another path has checked the dictionary rows"
+    gp.close()
+
+
+# the largest tables: a multiprocessor each, 512 threads and 256; one that does not fit
+@pytest.mark.parametrize("V,launches", [(10200, 2), (11400, 2), (12500, 3)])
+def test_many_vregs(B, oracle_mod, V, launches):
+    """A chain: every instruction defines a vreg of its own and reads some of the last ones."""
+    rng = np.random.default_rng(V)
+    ins = [([v], [int(u) for u in v - rng.integers(1, 9, int(rng.integers(0, 4))) if u >= 0]) for v in range(V)]
+    cut = V // 3
+    p = synth.program_from_lists([ins[:cut], ins[cut:]], [(0, 1)], V, [1, 2] * (V // 2), 64)
+    table = np.arange(V) * 2 % 64
+    some = np.stack([H.row_from_table(p, (table + 2 * k) % 64) for k in range(20)])
+    for k in range(8):                       # an overlap, a vreg outside the file, an occurrence that differs
+        t = (table + 2 * k) % 64
+        v = int(rng.integers(20, V))
+        t[v] = (t[v - 3], 64 + k)[k % 2]
+        some[k] = H.row_from_table(p, t)
+    some[8, p.n_operands - 1] += 2
+    some[9:11, : p.n_operands] = rng.integers(0, 70, (2, p.n_operands))
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    verdicts = op.verify(op.liveness(), some)
+    assert (verdicts["flags"] == B.VL_PASS).any()
+    pick = np.arange(500) % 20
+    dev = _to_dev(some[pick])
+    _assert_same(B.verdicts_to_numpy(gp.vl_verify(dev)), verdicts[pick])
+    assert _launches(B, lambda: gp.vl_verify(dev)) == launches, "another path has checked the rows"
     gp.close()
 
 
@@ -149,7 +188,7 @@ def test_bounded_wait_runs_out(B, oracle_mod, K):
 
 # counts handed over (few rows; many rows of a long program, up to the most), made by the block itself; candidates in fine items, in
 # coarse ones, one item each
-@pytest.mark.parametrize("n_instrs,K,launches", [(2399, 2000, 2), (2399, 2001, 1), (2400, 2001, 2), (2400, 8192, 2), (2400, 8193, 1), (4100, 700, 2)])
+@pytest.mark.parametrize("n_instrs,K,launches", [(2399, 2000, 2), (2399, 2001, 1), (2400, 2001, 2), (2400, 4800, 2), (2400, 4801, 1), (3500, 6800, 2), (4100, 700, 2)])
 @pytest.mark.parametrize("noise", [0.004, 0.2, 1.0])
 def test_rows_that_collide_everywhere(B, oracle_mod, n_instrs, K, launches, noise):
     """Rows of random registers (every chunk collides, vregs outside the file, tuples across mask words) among valid ones."""

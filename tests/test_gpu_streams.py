@@ -208,3 +208,32 @@ def test_capture_behind_a_run_in_flight(B, oracle_mod, kind, same_stream):
         torch.cuda.synchronize()
         assert B.verdicts_to_numpy(out).tobytes() == want.tobytes()
     gp.close()
+
+
+def test_many_rows_on_two_streams(B, oracle_mod):
+    """Calls of more rows than a pass holds, on two streams, without anything between them: they do not meet in the handle's
+    working set."""
+    import torch
+    shape = synth.Shape("line", [3100], [], [], [], n_vregs=1000, widths={1: 0.7, 2: 0.2, 4: 0.1}, P=128)
+    p = synth.build_program(shape, 3)
+    gp = B.Program(p)
+    gp.vl_liveness()
+    op = oracle_mod.OracleProgram(p)
+    lv = op.liveness()
+    K = 6000
+    some = [_garbage_rows(p, 60, 70 + j) for j in range(2)]
+    for s in some:
+        s[:30] = synth.candidate_rows(p, 30, 0.3, 4)[0]
+    picks = [np.random.default_rng(j).integers(0, 60, K) for j in range(2)]
+    devs = [_to_dev(s[pick]) for s, pick in zip(some, picks)]
+    wants = [op.verify(lv, s)[pick] for s, pick in zip(some, picks)]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    outs = [torch.zeros((K, 4), dtype=torch.int32, device="cuda") for _ in range(8)]
+    gp.vl_verify(devs[0], outs[0])
+    torch.cuda.synchronize()
+    for j in range(8):
+        gp.vl_verify(devs[j % 2], outs[j], streams[j % 2])
+    torch.cuda.synchronize()
+    for j in range(8):
+        assert B.verdicts_to_numpy(outs[j]).tobytes() == wants[j % 2].tobytes(), f"call {j}"
+    gp.close()
