@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "vl_internal.cuh"
 
 namespace {
@@ -71,6 +73,174 @@ __device__ __forceinline__ uint32_t pk8_get(const uint4 &x, int g)
 {
     const uint32_t w = (g >> 1) == 0 ? x.x : ((g >> 1) == 1 ? x.y : ((g >> 1) == 2 ? x.z : x.w));
     return (g & 1) ? (w >> 16) : (w & 0xFFFFu);
+}
+
+// The warp has read its part of a stage, or has stored its first occurrences of a tile.
+__device__ __forceinline__ void warp_arrive(unsigned long long *bar)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// A thread's four columns of a tile, as eight rows have them, to "eight candidates side by side per column".
+__device__ __forceinline__ void transpose8(const uint2 (&r)[8], uint4 (&pc)[4])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
+        uint32_t w[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            w[m] = (j < 2) ? __byte_perm(r[2 * m].x, r[2 * m + 1].x, sel) : __byte_perm(r[2 * m].y, r[2 * m + 1].y, sel);
+        pc[j] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+// Those that are first occurrences (bits of first) to their table entries, off bytes into the table.
+__device__ __forceinline__ void store_first8(unsigned char *table, const uint4 (&pc)[4], const uint4 &off, uint32_t first)
+{
+    const uint32_t of[4] = {off.x, off.y, off.z, off.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if ((first >> j) & 1) *reinterpret_cast<uint4 *>(table + of[j]) = pc[j];
+}
+// Every occurrence against the table (a first occurrence trivially matches; padding columns were zeroed and name the all-zero
+// spare entry); o_base: the first one's column.
+__device__ __forceinline__ void compare8(const unsigned char *table, const uint4 (&pc)[4], const uint4 &off, uint32_t o_base, uint32_t *flags,
+                                         uint32_t *minop)
+{
+    const uint32_t of[4] = {off.x, off.y, off.z, off.w};
+    uint4 x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = *reinterpret_cast<const uint4 *>(table + of[j]);
+    uint32_t acc = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc |= (x[j].x ^ pc[j].x) | (x[j].y ^ pc[j].y) | (x[j].z ^ pc[j].z) | (x[j].w ^ pc[j].w);
+    if (acc) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t d[4] = {x[j].x ^ pc[j].x, x[j].y ^ pc[j].y, x[j].z ^ pc[j].z, x[j].w ^ pc[j].w};
+#pragma unroll
+            for (int g = 0; g < 8; ++g)
+                if ((g & 1) ? (d[g >> 1] >> 16) : (d[g >> 1] & 0xFFFFu)) {
+                    atomicOr(&flags[g], (uint32_t)VL_INCONSISTENT);
+                    atomicMin(&minop[g], o_base + j);
+                }
+        }
+    }
+}
+
+// The one-hot bank nibbles of the eight candidates of a table entry (byte j: candidate j low, candidate j + 4 high): a byte
+// permute looks up 1 << bank for four of them at a time.  bm: the number of banks less 1, in both halves.
+__device__ __forceinline__ uint32_t bank_nibbles8(const uint32_t (&x)[4], uint32_t bm)
+{
+    uint32_t h[2];
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+        const uint32_t w = (x[2 * m] & bm) | ((x[2 * m + 1] & bm) << 8);
+        h[m] = __byte_perm(0x08040201u, 0u, w | (w >> 12));
+    }
+    return h[0] | (h[1] << 4);
+}
+// 0 if all eight ranges of width w lie inside the file: with c = 0x7FFF - (P - width) added to an entry below 2^15, bit 15 of the
+// sum is set iff entry + width > P; entries at or above 2^15 are outside any file these kernels accept.
+__device__ __forceinline__ uint32_t outside8(const uint32_t (&x)[4], uint32_t w, uint32_t P)
+{
+    if (w > P) return 1u;
+    const uint32_t c2 = (0x7FFFu - (P - w)) * 0x10001u;
+    return (((x[0] + c2) | x[0]) | ((x[1] + c2) | x[1]) | ((x[2] + c2) | x[2]) | ((x[3] + c2) | x[3])) & 0x80008000u;
+}
+// Two registers with bit 15 := ((register & 31) + width > 32): the range reaches into the next word of an occupancy mask.
+// 0x7FDF = 0x8000 - 33
+__device__ __forceinline__ uint32_t straddle_mark(uint32_t x, uint32_t w)
+{
+    return (x & 0x7FFF7FFFu) | (((x & 0x001F001Fu) + w * 0x10001u + 0x7FDF7FDFu) & 0x80008000u);
+}
+
+// Bank tally of the eight candidates over the instructions with 2..4 distinct sources, by NT threads: the banks an instruction
+// touches are the bits of the OR of its sources' nibbles, counted with carry-save adders and added to bank.
+template <int NT>
+__device__ __forceinline__ void bank_tally8(const uint32_t *Hb, const uint2 *list, const uint32_t (&seg)[4], uint32_t *bank)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    auto csa = [](uint32_t &h, uint32_t &l, uint32_t a, uint32_t b, uint32_t c) {
+        const uint32_t u = a ^ b;
+        h = (a & b) | (u & c);
+        l = u ^ c;
+    };
+    // population count of each of the 8 nibbles, as byte fields: even nibbles and odd nibbles
+    auto nib_even = [](uint32_t y) -> uint32_t { return y & 0x0F0F0F0Fu; };
+    auto nib_odd = [](uint32_t y) -> uint32_t { return (y >> 4) & 0x0F0F0F0Fu; };
+    auto nib_counts = [](uint32_t x) -> uint32_t {
+        const uint32_t y = x - ((x >> 1) & 0x55555555u);
+        return (y & 0x33333333u) + ((y >> 2) & 0x33333333u);
+    };
+    uint32_t ones = 0, twos = 0, fours = 0, acc_e = 0, acc_o = 0, rounds = 0;
+    uint32_t sum[8];
+#pragma unroll
+    for (int g = 0; g < 8; ++g) sum[g] = 0;
+    auto flush = [&](uint32_t weight) {
+#pragma unroll
+        for (int g = 0; g < 8; ++g) sum[g] += weight * (((g >= 4 ? acc_o : acc_e) >> (8 * (g & 3))) & 0xFFu);
+        acc_e = 0; acc_o = 0;
+    };
+    // one segment of the list per number of sources: as many lookups as an entry has sources (with four for every
+    // entry the shared-memory pipe took 12.4 k cycles per block on 31,000 entries, now 9)
+    auto segment = [&](auto sources, uint32_t e_lo, uint32_t e_hi) {
+        constexpr int S = decltype(sources)::value;
+        uint2 ids_next[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) ids_next[u] = e_lo + tid + u * NT < e_hi ? list[e_lo + tid + u * NT] : make_uint2(0, 0);
+        for (uint32_t e0 = e_lo + tid; e0 < e_hi; e0 += 8 * NT) {
+            uint2 ids[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                ids[u] = ids_next[u];
+                const uint32_t en = e0 + 8 * NT + u * NT;
+                ids_next[u] = en < e_hi ? list[en] : make_uint2(0, 0);
+            }
+            uint32_t x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                uint32_t o = Hb[ids[u].x & 0xFFFFu] | Hb[ids[u].x >> 16];
+                if (S > 2) o |= Hb[ids[u].y & 0xFFFFu];
+                if (S > 3) o |= Hb[ids[u].y >> 16];
+                x[u] = e0 + u * NT < e_hi ? o : 0u;
+            }
+            uint32_t ta, tb, fa, fb, eights;
+            csa(ta, ones, ones, x[0], x[1]);
+            csa(tb, ones, ones, x[2], x[3]);
+            csa(fa, twos, twos, ta, tb);
+            csa(ta, ones, ones, x[4], x[5]);
+            csa(tb, ones, ones, x[6], x[7]);
+            csa(fb, twos, twos, ta, tb);
+            csa(eights, fours, fours, fa, fb);
+            const uint32_t c8 = nib_counts(eights);
+            acc_e += nib_even(c8);
+            acc_o += nib_odd(c8);
+            if (++rounds == 32) {  // the byte fields hold at most 4 per round
+                flush(8u);
+                rounds = 0;
+            }
+        }
+    };
+    segment(std::integral_constant<int, 2>{}, seg[0], seg[1]);
+    segment(std::integral_constant<int, 3>{}, seg[1], seg[2]);
+    segment(std::integral_constant<int, 4>{}, seg[2], seg[3]);
+    flush(8u);
+    uint32_t c = nib_counts(fours);
+    acc_e = nib_even(c); acc_o = nib_odd(c);
+    flush(4u);
+    c = nib_counts(twos);
+    acc_e = nib_even(c); acc_o = nib_odd(c);
+    flush(2u);
+    c = nib_counts(ones);
+    acc_e = nib_even(c); acc_o = nib_odd(c);
+    flush(1u);
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+        const uint32_t x = __reduce_add_sync(0xffffffffu, sum[g]);
+        if (lane == 0 && x) atomicAdd(&bank[g], x);
+    }
 }
 
 // Hardware rules on where the tuples may sit (alignment, registers of the vreg's class, reserved registers) for the eight

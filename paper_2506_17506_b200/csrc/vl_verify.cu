@@ -637,52 +637,7 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
         const uint32_t spare_off = q.V * 16u;
         const uint4 *opoff = q.opoff + tid;
         const uint8_t *first4 = q.first4 + tid;
-        // every occurrence of a tile against the table (a first occurrence trivially matches; padding
-        // operands were zeroed and name the all-zero spare entry)
-        auto compare = [&](const uint4 (&pc)[4], const uint4 &off, uint32_t o_base) {
-            const uint32_t of[4] = {off.x, off.y, off.z, off.w};
-            uint4 x[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) x[j] = *reinterpret_cast<const uint4 *>(smem + of[j]);
-            uint32_t acc = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                acc |= (x[j].x ^ pc[j].x) | (x[j].y ^ pc[j].y) | (x[j].z ^ pc[j].z) | (x[j].w ^ pc[j].w);
-            if (acc) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t d[4] = {x[j].x ^ pc[j].x, x[j].y ^ pc[j].y, x[j].z ^ pc[j].z, x[j].w ^ pc[j].w};
-#pragma unroll
-                    for (int g = 0; g < G; ++g)
-                        if ((g & 1) ? (d[g >> 1] >> 16) : (d[g >> 1] & 0xFFFFu)) {
-                            atomicOr(&M->flags[g], (uint32_t)VL_INCONSISTENT);
-                            atomicMin(&M->minop[g], o_base + j);
-                        }
-                }
-            }
-        };
-        auto transpose = [&](const uint2 (&r)[G], uint4 (&pc)[4]) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
-                uint32_t w[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m)
-                    w[m] = (j < 2) ? __byte_perm(r[2 * m].x, r[2 * m + 1].x, sel) : __byte_perm(r[2 * m].y, r[2 * m + 1].y, sel);
-                pc[j] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        };
-        auto store_first = [&](const uint4 (&pc)[4], const uint4 &off, uint32_t first) {
-            const uint32_t of[4] = {off.x, off.y, off.z, off.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if ((first >> j) & 1) *reinterpret_cast<uint4 *>(smem + of[j]) = pc[j];
-        };
-        // the warp has read its part of a stage / has stored its first occurrences of a tile
-        auto warp_arrive = [&](unsigned long long *bar) {
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-        };
+        auto compare = [&](const uint4 (&pc)[4], const uint4 &off, uint32_t o_base) { compare8(smem, pc, off, o_base, M->flags, M->minop); };
         uint32_t stage = 0, parity = 0;
         const uint32_t last = q.ntiles - 1;
         // thread i asks for line i % (ROW_BYTES / 128) of row i / (ROW_BYTES / 128) of a tile
@@ -711,9 +666,9 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
             const unsigned char *src = region + (size_t)stage * STAGE_BYTES + tid * 8;
 #pragma unroll
             for (int g = 0; g < G; ++g) r[g] = *reinterpret_cast<const uint2 *>(src + g * ROW_BYTES);
-            transpose(r, pc);
+            transpose8(r, pc);
             warp_arrive(&M->empty[stage]);
-            store_first(pc, off, first);
+            store_first8(smem, pc, off, first);
             warp_arrive(&M->stored[t & 1]);
             if (t) wait_bar(&M->stored[(t - 1) & 1], ((t - 1) >> 1) & 1u);
             compare(ppc, poff, (t - 1) * TILE + tid * 4);
@@ -762,11 +717,11 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
 #pragma unroll
                 for (int g = 0; g < G; ++g) r[g] = *reinterpret_cast<const uint2 *>(src + g * ROW_BYTES);
             }
-            transpose(r, pcA);
+            transpose8(r, pcA);
 #pragma unroll
             for (int j = 0; j < 4; ++j)  // operands beyond n_operands compare as zero against the spare entry
                 if (o_base + j >= q.nO) pcA[j] = make_uint4(0, 0, 0, 0);
-            store_first(pcA, offA, first);
+            store_first8(smem, pcA, offA, first);
             warp_arrive(&M->stored[last & 1]);
             if (last) wait_bar(&M->stored[(last - 1) & 1], ((last - 1) >> 1) & 1u);
             compare(pcB, offB, (last - 1) * TILE + tid * 4);
@@ -804,25 +759,9 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
                 if (v >= q.V) break;
                 const uint4 tt = T[v];
                 const uint32_t x[4] = {tt.x, tt.y, tt.z, tt.w};
-                if (q.bank_fast) {  // a byte permute looks up 1 << bank for four candidates at a time
-                    uint32_t h[2];
-#pragma unroll
-                    for (int m = 0; m < 2; ++m) {
-                        const uint32_t w = (x[2 * m] & bm) | ((x[2 * m + 1] & bm) << 8);
-                        h[m] = __byte_perm(0x08040201u, 0u, w | (w >> 12));
-                    }
-                    Hb[v] = h[0] | (h[1] << 4);
-                }
+                if (q.bank_fast) Hb[v] = bank_nibbles8(x, bm);
                 if (!(vi & VINFO_OCCURS)) continue;
-                // quick test for "all eight inside the file": with c = 0x7FFF - (P - width) added to an
-                // entry below 2^15, bit 15 of the sum is set iff entry + width > P; entries at or above
-                // 2^15 are outside any file this kernel accepts.  The exact test runs only if a bit shows.
-                const uint32_t w = vi & 0xFFu;
-                uint32_t f = 1;
-                if (w <= q.P) {
-                    const uint32_t c2 = (0x7FFFu - (q.P - w)) * 0x10001u;
-                    f = (((x[0] + c2) | x[0]) | ((x[1] + c2) | x[1]) | ((x[2] + c2) | x[2]) | ((x[3] + c2) | x[3])) & 0x80008000u;
-                }
+                const uint32_t w = vi & 0xFFu, f = outside8(x, w, q.P);
                 if (f) {
 #pragma unroll
                     for (int g = 0; g < G; ++g) {
@@ -836,12 +775,10 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
                         }
                     }
                 }
-                // bit 15 := ((register & 31) + width > 32), per 16-bit entry; 0x7FDF = 0x8000 - 33
-                const uint32_t wc = w * 0x10001u + 0x7FDF7FDFu;
                 uint32_t o[4], diff = 0;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    o[m] = (x[m] & 0x7FFF7FFFu) | (((x[m] & 0x001F001Fu) + wc) & 0x80008000u);
+                    o[m] = straddle_mark(x[m], w);
                     diff |= o[m] ^ x[m];
                 }
                 if (diff) T[v] = make_uint4(o[0], o[1], o[2], o[3]);
@@ -883,89 +820,8 @@ __global__ void __launch_bounds__(NT + 32, 1) k_tables8(const TParams q, const _
         }
     }
 
-    // ---- bank tally over the instructions with 2..4 distinct sources (see k_tables): the banks an
-    // instruction touches are the bits of the OR of its sources' nibbles, counted with carry-save adders
-    if (q.bank_fast && tid < NT) {
-        auto csa = [](uint32_t &h, uint32_t &l, uint32_t a, uint32_t b, uint32_t c) {
-            const uint32_t u = a ^ b;
-            h = (a & b) | (u & c);
-            l = u ^ c;
-        };
-        // population count of each of the 8 nibbles, as byte fields: even nibbles and odd nibbles
-        auto nib_even = [](uint32_t y) -> uint32_t { return y & 0x0F0F0F0Fu; };
-        auto nib_odd = [](uint32_t y) -> uint32_t { return (y >> 4) & 0x0F0F0F0Fu; };
-        auto nib_counts = [](uint32_t x) -> uint32_t {
-            const uint32_t y = x - ((x >> 1) & 0x55555555u);
-            return (y & 0x33333333u) + ((y >> 2) & 0x33333333u);
-        };
-        uint32_t ones = 0, twos = 0, fours = 0, acc_e = 0, acc_o = 0, rounds = 0;
-        uint32_t sum[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) sum[g] = 0;
-        auto flush = [&](uint32_t weight) {
-#pragma unroll
-            for (int g = 0; g < G; ++g) sum[g] += weight * (((g >= 4 ? acc_o : acc_e) >> (8 * (g & 3))) & 0xFFu);
-            acc_e = 0; acc_o = 0;
-        };
-        // one segment of the list per number of sources: as many lookups as an entry has sources (with four for every
-        // entry the shared-memory pipe took 12.4 k cycles per block on 31,000 entries, now 9)
-        auto segment = [&](auto sources, uint32_t e_lo, uint32_t e_hi) {
-            constexpr int N = decltype(sources)::value;
-            uint2 ids_next[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) ids_next[u] = e_lo + tid + u * NT < e_hi ? q.bank_list[e_lo + tid + u * NT] : make_uint2(0, 0);
-            for (uint32_t e0 = e_lo + tid; e0 < e_hi; e0 += 8 * NT) {
-                uint2 ids[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    ids[u] = ids_next[u];
-                    const uint32_t en = e0 + 8 * NT + u * NT;
-                    ids_next[u] = en < e_hi ? q.bank_list[en] : make_uint2(0, 0);
-                }
-                uint32_t x[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    uint32_t o = Hb[ids[u].x & 0xFFFFu] | Hb[ids[u].x >> 16];
-                    if (N > 2) o |= Hb[ids[u].y & 0xFFFFu];
-                    if (N > 3) o |= Hb[ids[u].y >> 16];
-                    x[u] = e0 + u * NT < e_hi ? o : 0u;
-                }
-                uint32_t ta, tb, fa, fb, eights;
-                csa(ta, ones, ones, x[0], x[1]);
-                csa(tb, ones, ones, x[2], x[3]);
-                csa(fa, twos, twos, ta, tb);
-                csa(ta, ones, ones, x[4], x[5]);
-                csa(tb, ones, ones, x[6], x[7]);
-                csa(fb, twos, twos, ta, tb);
-                csa(eights, fours, fours, fa, fb);
-                const uint32_t c8 = nib_counts(eights);
-                acc_e += nib_even(c8);
-                acc_o += nib_odd(c8);
-                if (++rounds == 32) {  // the byte fields hold at most 4 per round
-                    flush(8u);
-                    rounds = 0;
-                }
-            }
-        };
-        segment(std::integral_constant<int, 2>{}, q.bank_seg[0], q.bank_seg[1]);
-        segment(std::integral_constant<int, 3>{}, q.bank_seg[1], q.bank_seg[2]);
-        segment(std::integral_constant<int, 4>{}, q.bank_seg[2], q.bank_seg[3]);
-        flush(8u);
-        uint32_t c = nib_counts(fours);
-        acc_e = nib_even(c); acc_o = nib_odd(c);
-        flush(4u);
-        c = nib_counts(twos);
-        acc_e = nib_even(c); acc_o = nib_odd(c);
-        flush(2u);
-        c = nib_counts(ones);
-        acc_e = nib_even(c); acc_o = nib_odd(c);
-        flush(1u);
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const uint32_t x = __reduce_add_sync(0xffffffffu, sum[g]);
-            if (lane == 0 && x) atomicAdd(&M->bank[g], x);
-        }
-    }
+    // ---- bank tally over the instructions with 2..4 distinct sources
+    if (q.bank_fast && tid < NT) bank_tally8<NT>(Hb, q.bank_list, q.bank_seg, M->bank);
     __syncthreads();
 
     // ------------------------------------------------- hand-over to the walk (see k_tables)
