@@ -208,7 +208,7 @@ def kernels_hash():
     """Hash of the source of the verify kernels."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("vl_verify.cu", "vl_fused.cu", "vl_internal.cuh", "vl_exact.cuh", "vl_ptx.cuh"):
+    for f in ("vl_verify.cu", "vl_fused.cu", "vl_eight.cu", "vl_internal.cuh", "vl_exact.cuh", "vl_ptx.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2506_17506_b200", "csrc", f), "rb").read())
     return h.hexdigest()
 

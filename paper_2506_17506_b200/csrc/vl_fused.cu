@@ -18,7 +18,11 @@
 #include "vl_exact.cuh"
 
 #define EXACT_NT 256
-#define EXACT_ROUNDS 2
+// Coarse items of k_fused's and k_eight's rows: more than four rounds of the blocks become three.  Four / three rounds, us: 8,000
+// instructions, 1,184 rows, half of them noise 611 / 526, 32,000 instructions, 749 rows, a tenth 560 / 504; all items, three
+// rounds: 24,000 instructions, 999 rows with one fault each 184 / 195, half of them noise 2,464 / 1,416.
+#define EXACT_ROUNDS 3
+#define EXACT_MOST_ROUNDS 4
 #define EXACT_SMEM (224u * 1024)  // shared memory of a block of k_exact, at most
 #define EXACT_ROWS 8192           // rows that k_fused and k_eight leave counts of, at most: each block adds up their items
 
@@ -406,31 +410,46 @@ __global__ void __launch_bounds__(EXACT_NT, 2) k_exact(const __grid_constant__ F
         if (!__syncthreads_or(any)) return;
         // (an odd number of rows per thread: their places begin in different banks)
         const uint32_t per = (q.ex.rows + EXACT_NT - 1) / EXACT_NT | 1u, k0 = tid * per, k1 = min(k0 + per, q.ex.rows);
-        // of this thread's rows: coarse items, fine items << 20, rows with any << 40
-        auto fields = [](uint32_t x) { return (u64)(x & 0xFFFFu) | (u64)(x >> 16) << 20 | (u64)(x ? 1u : 0u) << 40; };
-        u64 n = 0;
-        for (uint32_t k = k0; k < k1; ++k) n += fields(first[k]);
-        u64 inc = n;
+        auto scan = [&](u64 n, u64 &all) {  // of the threads in front of this one; of all
+            u64 inc = n;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const u64 y = __shfl_up_sync(0xffffffffu, inc, d);
-            if (lane >= (uint32_t)d) inc += y;
-        }
-        if (lane == 31) s_sum[tid >> 5] = inc;
-        __syncthreads();
-        u64 before = inc - n, all = 0;
+            for (int d = 1; d < 32; d <<= 1) {
+                const u64 y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= (uint32_t)d) inc += y;
+            }
+            __syncthreads();
+            if (lane == 31) s_sum[tid >> 5] = inc;
+            __syncthreads();
+            u64 before = inc - n;
+            all = 0;
 #pragma unroll
-        for (uint32_t w = 0; w < EXACT_NT / 32; ++w) {
-            if (w < tid >> 5) before += s_sum[w];
-            all += s_sum[w];
+            for (uint32_t w = 0; w < EXACT_NT / 32; ++w) {
+                if (w < tid >> 5) before += s_sum[w];
+                all += s_sum[w];
+            }
+            return before;
+        };
+        u64 n = 0, all;  // coarse items, fine items << 32
+        for (uint32_t k = k0; k < k1; ++k) n += (first[k] & 0xFFFFu) | (u64)(first[k] >> 16) << 32;
+        u64 before = scan(n, all);
+        // Fine items if each has a thread block; else coarse ones, and no more of them than a few rounds of the blocks take: an item
+        // fetches its part of the row anew (15 to 20 us) and counts it.
+        const uint32_t coarse = (uint32_t)all, most = EXACT_ROUNDS * gridDim.x;
+        const bool fine = (uint32_t)(all >> 32) <= q.ex.fine_items, fewer = !fine && coarse > EXACT_MOST_ROUNDS * gridDim.x;
+        auto of_row = [&](uint32_t x) {
+            if (fine) return x >> 16;
+            x &= 0xFFFFu;
+            return fewer && x ? max(1u, x * most / coarse) : x;
+        };
+        if (fewer) {
+            n = 0;
+            for (uint32_t k = k0; k < k1; ++k) n += of_row(first[k]);
+            before = scan(n, all);
         }
-        // Fine items if each has a thread block; a row each where the rows alone keep every block busy for several rounds (an
-        // item fetches its part of the row anew); else coarse ones.
-        const uint32_t shift = ((all >> 20) & 0xFFFFFu) <= q.ex.fine_items ? 20u : ((uint32_t)(all >> 40) >= EXACT_ROUNDS * gridDim.x ? 40u : 0u);
-        n_items = (uint32_t)(all >> shift) & 0xFFFFFu;
-        uint32_t at = (uint32_t)(before >> shift) & 0xFFFFFu;
+        n_items = (uint32_t)(fine ? all >> 32 : all);
+        uint32_t at = (uint32_t)(fine ? before >> 32 : before);
         for (uint32_t k = k0; k < k1; ++k) {
-            const uint32_t x = (uint32_t)(fields(first[k]) >> shift) & 0xFFFFFu;
+            const uint32_t x = of_row(first[k]);
             first[k] = at;
             at += x;
         }
