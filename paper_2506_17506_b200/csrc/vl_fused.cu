@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(NTHR, BPM) k_fused(const __grid_constant__ FMa
 // file, or the program has no fast bank tally), listed in work as items of one or several parts per candidate; a thread
 // block takes an item.  Consistency and Realizability are in cstate; a chunk of the walk that collided marks all of its
 // short chunks.  GLOBAL: the block's arrays lie in a slice of global memory (programs that do not fit a multiprocessor).
-// ROWS: the candidates are the rows of k_fused, which left the number of items of each in cstate; every block adds them up
+// ROWS: the candidates are the rows of k_fused or k_eight, which left the number of items of each; every block adds them up
 // for itself (a list with its counts would have to be cleared in front of every call: 3.3 us of 26 for 200 rows of 8,000
 // instructions by a memset; reset by the last block, it is left as it is by a call whose second launch fails).
 template <bool GLOBAL, bool ROWS, bool LONG>
