@@ -1727,7 +1727,13 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
         err = vl_layout(p, streams[stream_of(j)]);
         if (err == VL_OK && !p->h_live && !(p->h_live = (uint32_t *)vl_pinned_get())) err = VL_ERR_CUDA;
         if (err == VL_OK) err = live_begin(p, args[j], shapes[j], streams[stream_of(j)]);
-        if (err != VL_OK) { n = j; break; }  // (those behind it are untouched)
+        if (err != VL_OK) {
+            // (its next run may be on another stream than the kernel that makes its operand words)
+            if (p->words_new) cudaStreamSynchronize(streams[stream_of(j)]);
+            p->words_new = false;
+            n = j;  // (those behind it are untouched)
+            break;
+        }
         lengths_known = lengths_known && p->sizes_known;
     }
     auto launch = [&](bool fill) -> int {
@@ -1740,8 +1746,12 @@ int vl_liveness_impl(vl_program *const *progs, uint32_t n, const cudaStream_t *s
         }
         return VL_OK;
     };
-    if ((rc = launch(false)) != VL_OK) return rc;
-    for (uint32_t j = 0; j < n; ++j) progs[j]->words_new = false;
+    rc = launch(false);
+    for (uint32_t j = 0; j < n; ++j) {
+        if (rc != VL_OK && progs[j]->words_new) cudaStreamSynchronize(streams[stream_of(j)]);
+        progs[j]->words_new = false;
+    }
+    if (rc != VL_OK) return rc;
     if (!lengths_known)
         for (uint32_t s = 0; s < n_streams; ++s) VL_CUDA(progs[0], cudaStreamSynchronize(streams[s]));
     std::vector<vl_program *> run;  // the programs that the last kernel is launched for
