@@ -1340,10 +1340,11 @@ cudaError_t pool_get(VlArena &arena, T **out, size_t n)
         }                                                       \
     } while (0)
 
-// About the memory of a run that does not depend on the list lengths (live_begin).
-static size_t live_bytes(const vl_program *p)
+// About the memory of a run that does not depend on the list lengths (live_begin); small: k_small takes the program.
+static size_t live_bytes(const vl_program *p, bool small)
 {
-    return 4 * ((size_t)3 * p->nP + 4 * (size_t)p->nC + 5 * (size_t)p->nB) * p->Wv + (size_t)p->nI * 28 + (size_t)p->nO * 18 +
+    const size_t sets = small ? (size_t)p->nP + p->nC + 4 * (size_t)p->nB : 3 * (size_t)p->nP + 4 * (size_t)p->nC + 5 * (size_t)p->nB;
+    return 4 * sets * p->Wv + (size_t)p->nI * 28 + (size_t)p->nO * 18 +
            (size_t)p->nC * 40 + (size_t)p->nS * 16 + (size_t)p->nB * 24 + 40 * 512;
 }
 
@@ -1456,7 +1457,11 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         all.resize((all.size() + 4) & ~(size_t)3);  // (at least one word behind every array)
     }
     uint32_t *dev = nullptr;
-    p->layout_arena.hint = all.size() * 4 + (size_t)p->V * 12 + (size_t)p->nOp8 * 3 + (size_t)p->nOpT * 5 + 16384;
+    // The operand words lie beside the tables; those of a long program in the slab of the runs' memory: they would take a program
+    // of 32,000 instructions one device allocation more, 300 us of the first run's 1,200.  (There for every program: a run of a
+    // short one, its memory untouched for a while, 1 % slower.)
+    const bool beside = p->nO <= 65536;
+    p->layout_arena.hint = all.size() * 4 + (size_t)p->V * 12 + (beside ? (size_t)p->nO * 4 : 0) + (size_t)p->nOp8 * 3 + (size_t)p->nOpT * 5 + 16384;
     LAYOUT(&dev, all.size());
     VL_CUDA(p, cudaMemcpy(dev, all.data(), all.size() * 4, cudaMemcpyHostToDevice));
     size_t at = 0;
@@ -1465,12 +1470,14 @@ static int vl_layout(vl_program *p, cudaStream_t st)
         at = (at + x.v->size() + 4) & ~(size_t)3;
     }
     p->d_share = reinterpret_cast<uint4 *>(d_share);
-    // (in the slab of the runs' memory: beside the layout's tables they would take a program of 32,000 instructions one
-    // device allocation more, 300 us of the first run's 1,200)
     vl_free_liveness(p);
     p->live_arena.clear();
-    p->live_arena.hint = live_bytes(p) + (size_t)p->nO * 4 + 512;
-    KEEP(&p->d_op_word, (size_t)p->nO);
+    if (beside) {
+        LAYOUT(&p->d_op_word, (size_t)p->nO);
+    } else {
+        p->live_arena.hint = live_bytes(p, false) + (size_t)p->nO * 4 + 512;
+        KEEP(&p->d_op_word, (size_t)p->nO);
+    }
     p->live_arena.keep();
     LAUNCH(k_operand_words, (p->nP + NT / 32 - 1) / (NT / 32), NT, 0, st, p->nP, p->d_piece_i0, p->d_op_off, p->d_ndefs, p->d_op_vreg, p->d_op_word);
     VL_CUDA(p, cudaGetLastError());
@@ -1506,7 +1513,10 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     vl_free_liveness(p);
     const uint32_t nB = p->nB, nI = p->nI, V = p->V, nO = p->nO, Wv = p->Wv, nC = p->nC, nP = p->nP;
 
-    p->live_arena.hint = live_bytes(p);  // what follows, in one slab
+    q = LiveArgs{};
+    sh.small_smem = q.small.init(nB, p->nE, nC, p->nS, Wv, p->share_pieces, p->share_ops);
+    sh.small = nI <= LIVE_SMALL_INSTRS && nC && sh.small_smem <= SMALL_SMEM;
+    p->live_arena.hint = live_bytes(p, sh.small);  // what follows, in one slab
     // ---- results and tables that do not depend on the list lengths
     KEEP(&p->d_blk_in, (size_t)2 * nB * Wv);  // live-in rows, then live-out rows
     p->d_blk_out = p->d_blk_in + (size_t)nB * Wv;
@@ -1533,7 +1543,6 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     KEEP(&p->d_sen_off, (size_t)p->nS + 1);
     KEEP(&p->d_irec, (size_t)nI);
 
-    q = LiveArgs{};
     q.nB = nB; q.nI = nI; q.V = V; q.nE = p->nE; q.Wv = Wv; q.nC = nC; q.nP = nP; q.nS = p->nS; q.nSeg = p->nSeg;
     q.use_th = p->use_th;
     q.op_off = p->d_op_off; q.op_vreg = p->d_op_vreg; q.succ_off = p->d_succ_off; q.succ = p->d_succ; q.blk_off = p->d_blk_off;
@@ -1541,26 +1550,28 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     q.chunk_i0 = p->d_chunk_i0; q.chunk_i1 = p->d_chunk_i1; q.chunk_blk = p->d_chunk_blk; q.blk_chunk_off = p->d_blk_chunk_off;
     q.piece_i0 = p->d_piece_i0; q.piece_o0 = p->d_piece_o0; q.op_word = p->d_op_word; q.piece_chunk = p->d_piece_chunk; q.chunk_piece_off = p->d_chunk_piece_off;
     q.seg_c0 = p->d_seg_c0; q.blk_seg_off = p->d_blk_seg_off; q.short_p0 = p->d_short_p0; q.chunk_short_off = p->d_chunk_short_off;
-    KEEP(&q.piece_use, (size_t)nP * Wv);
-    KEEP(&q.piece_def, (size_t)nP * Wv);
+    if (!sh.small) {  // (k_small keeps these in shared memory)
+        KEEP(&q.piece_use, (size_t)nP * Wv);
+        KEEP(&q.piece_def, (size_t)nP * Wv);
+        KEEP(&q.chunk_use, (size_t)nC * Wv);
+        KEEP(&q.chunk_def, (size_t)nC * Wv);
+        KEEP(&q.chunk_end, (size_t)nC * Wv);
+        KEEP(&q.blk_touch, (size_t)nB * Wv);
+        KEEP(&q.chunk_lo, (size_t)nC);
+        KEEP(&q.short_ent, (size_t)p->nS);
+        KEEP(&q.counters, 1);
+    }
     KEEP(&q.piece_end, (size_t)nP * Wv);
-    KEEP(&q.chunk_use, (size_t)nC * Wv);
-    KEEP(&q.chunk_def, (size_t)nC * Wv);
-    KEEP(&q.chunk_end, (size_t)nC * Wv);
     KEEP(&q.chunk_entry, (size_t)nC * Wv);
-    KEEP(&q.blk_touch, (size_t)nB * Wv);
     KEEP(&q.lo_rel, (size_t)nI);
     KEEP(&q.ev_rel, (size_t)nI);
-    KEEP(&q.chunk_lo, (size_t)nC);
     KEEP(&q.chunk_ev, (size_t)nC);
     KEEP(&q.chunk_lo0, (size_t)nC + 1);
     KEEP(&q.centry_cnt, (size_t)nC);
-    KEEP(&q.short_ent, (size_t)p->nS);
     KEEP(&q.short_ev, (size_t)p->nS);
-    KEEP(&q.counters, 1);
     const uint32_t fgrid = (Wv + 31) / 32;
     size_t flow_smem = (((size_t)4 * nB + 2 * (size_t)p->nSeg) * 32 + nB + 1 + p->nE) * 4;
-    if (flow_smem > 200 * 1024) {
+    if (flow_smem > 200 * 1024 && !sh.small) {
         KEEP(&q.flow_scratch, flow_smem / 4 * fgrid);
         flow_smem = 0;
     }
@@ -1583,8 +1594,6 @@ static int live_begin(vl_program *p, LiveArgs &q, LiveShape &sh, cudaStream_t st
     if (!q.wide_smem) sh.count_smem = 0;
     sh.flow_smem = flow_smem;
     q.share = p->d_share; q.small_tab = p->d_blk_chunk_off;
-    sh.small_smem = q.small.init(nB, p->nE, nC, p->nS, Wv, p->share_pieces, p->share_ops);
-    sh.small = nI <= LIVE_SMALL_INSTRS && nC && sh.small_smem <= SMALL_SMEM;
     sh.fill_smem = (size_t)LV_WARPS * (2 * Wv + FILL_WARP_WORDS) * 4;
     return VL_OK;
 }
